@@ -21,7 +21,7 @@ struct LayerPlan {
     bool tc;
     bool planes;
     int splits;
-    size_t hdr, Abar, Alo, Bbar, W0, W1, W2, W3, f32buf, xs, gs, gAbar, gBbar, scan, part, dot, total;
+    size_t hdr, Abar, Alo, W0, W1, W2, W3, f32buf, xs, gs, gAbar, gg, scan, part, dot, total;
     size_t u3, gy3, x3, s3, acc;   // plane path: planes of u, gy, x, s and the fp32 result of a projection
 };
 
@@ -55,7 +55,6 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true) {
     p.hdr = take(off, sizeof(WsHeader));
     p.Abar = take(off, (size_t)s.P * 8);
     p.Alo = take(off, (size_t)s.P * 8);
-    p.Bbar = take(off, PH * 8);
     if (p.tc) {
         p.W0 = take(off, 4 * PH * 2);   // hi/lo stacked Bbar operand  [4P, H] bf16
         p.W1 = take(off, 4 * PH * 2);   // hi/lo stacked conj(C) operand [4P, H] bf16
@@ -82,7 +81,7 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true) {
         }
     }
     p.gAbar = take(off, (size_t)s.P * 8);
-    p.gBbar = take(off, PH * 8);
+    p.gg = take(off, (size_t)gamma_part_rows(s.H) * s.P * 8);
     p.scan = take(off, scan_scratch_bytes(s.B, s.T, s.P, 2));
     p.part = take(off, (size_t)2 * p.splits * 2 * PH * 4);   // split-K partials of gBbar, then those of dC
     {   // dD: partial column sums of gy * u, from the stand-alone kernel or from the epilogue of the du projection
@@ -136,8 +135,8 @@ SSM_API int ssm_discretize(const ssm_shape* shape, const ssm_c64* Lambda, const 
     if (!Lambda || !Delta || !Bc || !Abar || !Bbar) return SSM_ERR_NULL;
     if (misaligned(Lambda) || misaligned(Delta) || misaligned(Bc) || misaligned(Abar) || misaligned(Bbar))
         return SSM_ERR_ALIGN;
-    launch_discretize(shape->H, shape->P, (const float2*)Lambda, Delta, (const float2*)Bc, (float2*)Abar, nullptr,
-                      (float2*)Bbar, (cudaStream_t)stream);
+    launch_discretize(shape->H, shape->P, (const float2*)Lambda, Delta, (const float2*)Bc, (float2*)Abar, (float2*)Bbar,
+                      (cudaStream_t)stream);
     SSM_RETURN_IF_CUDA_ERROR();
     return SSM_OK;
 }
@@ -220,29 +219,20 @@ SSM_API int ssm_layer_plan_string(const ssm_shape* shape, char* buf, size_t len)
     return SSM_OK;
 }
 
-// Discretised parameters and packed projection operands into the workspace.
+// Discretised parameters and packed projection operands into the workspace; clears the status word of `hdr` if given.
 static void layer_prepare(const ssm_shape& s, const LayerPlan& p, const ssm_c64* Lambda, const float* Delta,
-                          const ssm_c64* Bc, const ssm_c64* Cc, void* ws, cudaStream_t st) {
+                          const ssm_c64* Bc, const ssm_c64* Cc, void* ws, WsHeader* hdr, cudaStream_t st) {
     StageTimer tm("discretize_pack", st);
-    if (p.tc) {
-        // one kernel (the kernels that scan in the epilogue of a projection want their own column order)
-        const int group = tc_gemm_scan_group(s.B, s.T, s.H, s.P);
-        launch_discretize_pack_tc(s.H, s.P, group, group, (const float2*)Lambda, Delta,
-                                  (const float2*)Bc, (const float2*)Cc, at<float2>(ws, p.Abar), at<float2>(ws, p.Alo),
-                                  at<float2>(ws, p.Bbar), at<void>(ws, p.W0), at<void>(ws, p.W1), at<void>(ws, p.W2),
-                                  at<void>(ws, p.W3), st);
-        return;
-    }
-    if (p.planes) {
-        launch_discretize_pack_planes(s.H, s.P, (const float2*)Lambda, Delta, (const float2*)Bc, (const float2*)Cc,
-                                      at<float2>(ws, p.Abar), at<float2>(ws, p.Alo), at<float2>(ws, p.Bbar),
-                                      at<void>(ws, p.W0), at<void>(ws, p.W1), at<void>(ws, p.W2), at<void>(ws, p.W3), st);
-        return;
-    }
-    launch_discretize(s.H, s.P, (const float2*)Lambda, Delta, (const float2*)Bc, at<float2>(ws, p.Abar),
-                      at<float2>(ws, p.Alo), at<float2>(ws, p.Bbar), st);
-    launch_pack_operands(s.H, s.P, false, at<float2>(ws, p.Bbar), (const float2*)Cc, at<void>(ws, p.W0),
-                         at<void>(ws, p.W3), at<void>(ws, p.W2), at<void>(ws, p.W1), st);
+    const float2 *L = (const float2*)Lambda, *B = (const float2*)Bc, *C = (const float2*)Cc;
+    float2 *Abar = at<float2>(ws, p.Abar), *Alo = at<float2>(ws, p.Alo);
+    void *W0 = at<void>(ws, p.W0), *W1 = at<void>(ws, p.W1), *W2 = at<void>(ws, p.W2), *W3 = at<void>(ws, p.W3);
+    if (p.tc)   // (the kernels that scan in the epilogue of a projection want their own column order)
+        launch_discretize_pack_tc(s.H, s.P, tc_gemm_scan_group(s.B, s.T, s.H, s.P), L, Delta, B, C, Abar, Alo, W0, W1, W2, W3,
+                                  hdr, st);
+    else if (p.planes)
+        launch_discretize_pack_planes(s.H, s.P, L, Delta, B, C, Abar, Alo, W0, W1, W2, W3, hdr, st);
+    else
+        launch_discretize_pack_f32(s.H, s.P, L, Delta, B, C, Abar, Alo, W0, W1, W2, W3, hdr, st);
 }
 
 // Launch sequence of one layer's forward pass from a prepared workspace.  `hdr` receives the
@@ -355,8 +345,8 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
 static int layer_fwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo& io, const ssm_c64* Lambda,
                           const float* Delta, const ssm_c64* Bc, const ssm_c64* Cc, const float* D, const void* u,
                           const uint8_t* done, const ssm_c64* x0, void* y, ssm_c64* xT, void* ws, WsHeader* hdr,
-                          cudaStream_t st) {
-    layer_prepare(s, p, Lambda, Delta, Bc, Cc, ws, st);
+                          bool clear_hdr, cudaStream_t st) {
+    layer_prepare(s, p, Lambda, Delta, Bc, Cc, ws, clear_hdr ? hdr : nullptr, st);
     return layer_fwd_run(s, p, io, D, u, done, x0, y, xT, ws, hdr, st);
 }
 
@@ -373,8 +363,7 @@ SSM_API int ssm_layer_fwd(const ssm_shape* shape, const ssm_c64* Lambda, const f
     if (int rc = check_ws(ws, ws_bytes, p.total)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     WsHeader* hdr = at<WsHeader>(ws, p.hdr);
-    if (cudaMemsetAsync(ws, 0, sizeof(WsHeader), st) != cudaSuccess) return SSM_ERR_CUDA;
-    return layer_fwd_impl(s, p, layer_io(s), Lambda, Delta, Bc, Cc, D, u, done, x0, y, xT, ws, hdr, st);
+    return layer_fwd_impl(s, p, layer_io(s), Lambda, Delta, Bc, Cc, D, u, done, x0, y, xT, ws, hdr, true, st);
 }
 
 // Single-step mode: the layer's forward launch sequence for T = 1 from operands prepared once.
@@ -398,8 +387,7 @@ SSM_API int ssm_step_prepare(const ssm_shape* shape, const ssm_c64* Lambda, cons
     const LayerPlan p = plan_layer(s);
     if (int rc = check_ws(ws, ws_bytes, p.total)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    if (cudaMemsetAsync(ws, 0, sizeof(WsHeader), st) != cudaSuccess) return SSM_ERR_CUDA;
-    layer_prepare(s, p, Lambda, Delta, Bc, Cc, ws, st);
+    layer_prepare(s, p, Lambda, Delta, Bc, Cc, ws, at<WsHeader>(ws, p.hdr), st);
     SSM_RETURN_IF_CUDA_ERROR();
     return SSM_OK;
 }
@@ -714,9 +702,10 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
             int groups = launch_dot_columns_partial(io.gy_bf16, gy, io.u_bf16, u, BT, s.H, tmp, st);
             dD_part = launch_reduce_rows(tmp, groups, s.H, tmp + (size_t)groups * s.H, kMaxPartialRows, &dD_rows, st);
         }
-        launch_splitk_reduce2(part, part_c, p.splits, s.H, P2, at<float2>(ws, p.gBbar), (float2*)dC, st);
-        launch_layer_finalize(s.H, s.P, (const float2*)Lambda, Delta, (const float2*)Bc, gA_part, gA_rows,
-                              at<float2>(ws, p.gBbar), (float2*)dLambda, dDelta, (float2*)dB, dD_part, dD_rows, dD, st);
+        launch_reduce_weight_grads(s.H, s.P, p.splits, part, part_c, (const float2*)Lambda, Delta, (const float2*)Bc,
+                                   (float2*)dB, (float2*)dC, at<float2>(ws, p.gg), st);
+        launch_layer_finalize(s.H, s.P, (const float2*)Lambda, Delta, gA_part, gA_rows, at<float2>(ws, p.gg),
+                              (float2*)dLambda, dDelta, dD_part, dD_rows, dD, st);
     }
     SSM_RETURN_IF_CUDA_ERROR();
     return SSM_OK;
@@ -821,7 +810,6 @@ SSM_API int ssm_stack_fwd(const ssm_shape* shape, int n_layers, const ssm_stack_
     const int BT = s.B * s.T;
     const size_t stat = align_up((size_t)BT * 4, 256);
     WsHeader* hdr = at<WsHeader>(ws, sp.hdr);
-    if (cudaMemsetAsync(ws, 0, sizeof(WsHeader), st) != cudaSuccess) return SSM_ERR_CUDA;
     const void* in = u;
     for (int l = 0; l < n_layers; ++l) {
         const ssm_stack_params& q = params[l];
@@ -830,7 +818,7 @@ SSM_API int ssm_stack_fwd(const ssm_shape* shape, int n_layers, const ssm_stack_
         float* v = at<float>(ws, sp.vs + sp.act * l);
         void* o = last ? out : at<void>(ws, sp.acts + sp.act * l);
         const LayerIo io{first && bf16, false, false, false};
-        if (int rc = layer_fwd_impl(ls, lp, io, q.Lambda, q.Delta, q.Bc, q.Cc, q.D, in, done, nullptr, v, nullptr, lws, hdr, st))
+        if (int rc = layer_fwd_impl(ls, lp, io, q.Lambda, q.Delta, q.Bc, q.Cc, q.D, in, done, nullptr, v, nullptr, lws, hdr, first, st))
             return rc;
         StageTimer tm("stack_gelu_ln_fwd", st);
         launch_stack_fwd(first && bf16, last && bf16, BT, s.H, in, v, q.ln_weight, q.ln_bias, o,

@@ -33,15 +33,12 @@ __device__ __forceinline__ ZohTerms zoh_terms(float2 lam, float dt) {
 
 // One block per state p: Abar[p], Bbar[p, :] = gamma_p * B[p, :].
 __global__ void discretize_kernel(int H, const float2* __restrict__ Lambda, const float* __restrict__ Delta,
-                                  const float2* __restrict__ Bc, float2* __restrict__ Abar,
-                                  float2* __restrict__ Abar_lo, float2* __restrict__ Bbar) {
+                                  const float2* __restrict__ Bc, float2* __restrict__ Abar, float2* __restrict__ Bbar) {
     __shared__ float2 gamma_s;
     const int p = blockIdx.x;
     if (threadIdx.x == 0) {
         ZohTerms z = zoh_terms(Lambda[p], Delta[p]);
-        const float2 ah = make_float2((float)z.ar, (float)z.ai);
-        Abar[p] = ah;
-        if (Abar_lo) Abar_lo[p] = make_float2((float)(z.ar - (double)ah.x), (float)(z.ai - (double)ah.y));
+        Abar[p] = make_float2((float)z.ar, (float)z.ai);
         gamma_s = make_float2((float)z.gr, (float)z.gi);
     }
     __syncthreads();
@@ -49,41 +46,31 @@ __global__ void discretize_kernel(int H, const float2* __restrict__ Lambda, cons
     for (int h = threadIdx.x; h < H; h += blockDim.x) Bbar[(size_t)p * H + h] = cmul(g, Bc[(size_t)p * H + h]);
 }
 
-// Adjoint.  One block per state p.  gAbar arrives as gA_rows rows of partial sums ([gA_rows, P], summed here
-// in a fixed order; one row = the finished gradient).  Blocks past the P states (if any) finish dD the same
-// way: dD[h] = sum of the dD_rows rows of dD_part ([dD_rows, H]).
+// Adjoint of the discretisation for one state: from gAbar and g_gamma (= sum_h conj(B) gBbar).
+__device__ __forceinline__ void zoh_adjoint(const ZohTerms& z, float2 lam, float dt, double gar, double gai, double ggr,
+                                            double ggi, float2& dLambda, float& dDelta) {
+    const double lr = lam.x, li = lam.y, d = dt;
+    // dgamma/dLambda = (Delta Abar - gamma) / Lambda     (= (Delta Abar Lambda - (Abar-1)) / Lambda^2)
+    const double nr = d * z.ar - z.gr, ni = d * z.ai - z.gi;
+    const double n = lr * lr + li * li;
+    const double qr = (nr * lr + ni * li) / n, qi = (ni * lr - nr * li) / n;
+    // dLambda = conj(Delta Abar) gAbar + conj(dgamma/dLambda) g_gamma
+    const double outr = d * (z.ar * gar + z.ai * gai) + (qr * ggr + qi * ggi);
+    const double outi = d * (z.ar * gai - z.ai * gar) + (qr * ggi - qi * ggr);
+    dLambda = make_float2((float)outr, (float)outi);
+    // dDelta = Re(conj(Lambda Abar) gAbar) + Re(conj(Abar) g_gamma)
+    const double lar = lr * z.ar - li * z.ai, lai = lr * z.ai + li * z.ar;
+    dDelta = (float)((lar * gar + lai * gai) + (z.ar * ggr + z.ai * ggi));
+}
+
+// ssm_discretize_bwd: one block per state p.
 __global__ void discretize_bwd_kernel(int H, int P, const float2* __restrict__ Lambda, const float* __restrict__ Delta,
-                                      const float2* __restrict__ Bc, const float2* __restrict__ gAbar, int gA_rows,
+                                      const float2* __restrict__ Bc, const float2* __restrict__ gAbar,
                                       const float2* __restrict__ gBbar, float2* __restrict__ dLambda,
-                                      float* __restrict__ dDelta, float2* __restrict__ dB,
-                                      const float* __restrict__ dD_part, int dD_rows, float* __restrict__ dD) {
+                                      float* __restrict__ dDelta, float2* __restrict__ dB) {
     __shared__ float2 gamma_s;
     __shared__ float red[2][32];
-    __shared__ double redA[2][32];
-    if ((int)blockIdx.x >= P) {   // columns of dD
-        const int h = ((int)blockIdx.x - P) * blockDim.x + threadIdx.x;
-        if (h < H) {
-            float acc = 0.f;
-            for (int r = 0; r < dD_rows; ++r) acc += dD_part[(size_t)r * H + h];
-            dD[h] = acc;
-        }
-        return;
-    }
     const int p = blockIdx.x;
-    double gar_t = 0.0, gai_t = 0.0;   // this thread's rows of the partial sums of gAbar[p]
-    for (int r = threadIdx.x; r < gA_rows; r += blockDim.x) {
-        const float2 v = gAbar[(size_t)r * P + p];
-        gar_t += (double)v.x;
-        gai_t += (double)v.y;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        gar_t += __shfl_xor_sync(0xffffffffu, gar_t, o);
-        gai_t += __shfl_xor_sync(0xffffffffu, gai_t, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        redA[0][threadIdx.x >> 5] = gar_t;
-        redA[1][threadIdx.x >> 5] = gai_t;
-    }
     const float2 lam = Lambda[p];
     const float dt = Delta[p];
     ZohTerms z = {};
@@ -117,110 +104,22 @@ __global__ void discretize_bwd_kernel(int H, int P, const float2* __restrict__ L
             ggr += red[0][w];
             ggi += red[1][w];
         }
-        const double lr = lam.x, li = lam.y, d = dt;
-        double gar = 0.0, gai = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            gar += redA[0][w];
-            gai += redA[1][w];
-        }
-        // dgamma/dLambda = (Delta Abar - gamma) / Lambda     (= (Delta Abar Lambda - (Abar-1)) / Lambda^2)
-        const double nr = d * z.ar - z.gr, ni = d * z.ai - z.gi;
-        const double n = lr * lr + li * li;
-        const double qr = (nr * lr + ni * li) / n, qi = (ni * lr - nr * li) / n;
-        // dLambda = conj(Delta Abar) gAbar + conj(dgamma/dLambda) g_gamma
-        double outr = d * (z.ar * gar + z.ai * gai) + (qr * ggr + qi * ggi);
-        double outi = d * (z.ar * gai - z.ai * gar) + (qr * ggi - qi * ggr);
-        dLambda[p] = make_float2((float)outr, (float)outi);
-        // dDelta = Re(conj(Lambda Abar) gAbar) + Re(conj(Abar) g_gamma)
-        const double lar = lr * z.ar - li * z.ai, lai = lr * z.ai + li * z.ar;
-        dDelta[p] = (float)((lar * gar + lai * gai) + (z.ar * ggr + z.ai * ggi));
+        zoh_adjoint(z, lam, dt, gAbar[p].x, gAbar[p].y, ggr, ggi, dLambda[p], dDelta[p]);
     }
 }
 
-// Real GEMM operands from the complex parameters (W = float or bf16):
-//   Bp[2p+c, h] = Bq[h, 2p+c] = c ? Im Bbar[p,h] : Re Bbar[p,h]
-//   Cp[h, 2p+c] = Cq[2p+c, h] = c ? -Im C[h,p]   : Re C[h,p]
-template <typename W>
-__global__ void pack_operands_kernel(int H, int P, const float2* __restrict__ Bbar, const float2* __restrict__ Cc,
-                                     W* __restrict__ Bp, W* __restrict__ Bq, W* __restrict__ Cp,
-                                     W* __restrict__ Cq) {
-    const size_t n = (size_t)P * H;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        {   // i indexes Bbar[p, h]
-            const int p = (int)(i / H), h = (int)(i % H);
-            const float2 v = Bbar[i];
-            Bp[(size_t)(2 * p) * H + h] = from_f32<W>(v.x);
-            Bp[(size_t)(2 * p + 1) * H + h] = from_f32<W>(v.y);
-            Bq[(size_t)h * 2 * P + 2 * p] = from_f32<W>(v.x);
-            Bq[(size_t)h * 2 * P + 2 * p + 1] = from_f32<W>(v.y);
-        }
-        {   // i indexes C[h, p]
-            const int h = (int)(i / P), p = (int)(i % P);
-            const float2 v = Cc[i];
-            Cp[(size_t)h * 2 * P + 2 * p] = from_f32<W>(v.x);
-            Cp[(size_t)h * 2 * P + 2 * p + 1] = from_f32<W>(-v.y);
-            Cq[(size_t)(2 * p) * H + h] = from_f32<W>(v.x);
-            Cq[(size_t)(2 * p + 1) * H + h] = from_f32<W>(-v.y);
-        }
-    }
-}
-
-// Operands of the tensor-core path.  A weight w is carried as hi = bf16(w), lo = bf16(w - hi)
-// in the two projections that feed the states (Bu and g_x), so that the states see ~16
-// mantissa bits of the parameters.  Logical row n of the [2P, H] operand goes to rows
-// (n/128)*256 + n%128 (hi) and (n/128)*256 + 128 + n%128 (lo) of the stacked [4P, H] matrix.
-// `stack`: rows per hi (and per lo) block, 128 for the plain projections, twice the states per chain otherwise.
-__device__ __forceinline__ void store_split(__nv_bfloat16* W, int H, int n, int h, float w, int stack = 128) {
+// hi = bf16(w) and lo = bf16(w - hi) into row n of the hi block and of the lo block of a stacked operand of
+// 2^stack_log2 rows per block.
+__device__ __forceinline__ void store_split(__nv_bfloat16* W, int H, int n, int h, float w, int stack_log2) {
     const __nv_bfloat16 hi = __float2bfloat16_rn(w);
     const __nv_bfloat16 lo = __float2bfloat16_rn(w - __bfloat162float(hi));
-    const size_t r = (size_t)(n / stack) * (2 * stack) + (n % stack);
+    const int stack = 1 << stack_log2;
+    const size_t r = (size_t)(((n >> stack_log2) << (stack_log2 + 1)) + (n & (stack - 1)));
     W[r * H + h] = hi;
     W[(r + stack) * H + h] = lo;
 }
 
-// Discretisation and operand packing of the tensor-core path in one kernel: block p computes Abar_p and
-// gamma_p (double precision, one thread), then the row p of Bbar with its packed forms and the packed forms
-// of column p of C.
-__global__ void __launch_bounds__(128)
-discretize_pack_tc_kernel(int H, int P, int group_B, int group_C, const float2* __restrict__ Lambda,
-                          const float* __restrict__ Delta, const float2* __restrict__ Bc, const float2* __restrict__ Cc,
-                          float2* __restrict__ Abar, float2* __restrict__ Abar_lo, float2* __restrict__ Bbar,
-                          __nv_bfloat16* __restrict__ WsB, __nv_bfloat16* __restrict__ WsC,
-                          __nv_bfloat16* __restrict__ Cp, __nv_bfloat16* __restrict__ Bq) {
-    __shared__ float2 gamma_s;
-    const int p = blockIdx.x;
-    if (threadIdx.x == 0) {
-        ZohTerms z = zoh_terms(Lambda[p], Delta[p]);
-        const float2 ah = make_float2((float)z.ar, (float)z.ai);
-        Abar[p] = ah;
-        if (Abar_lo) Abar_lo[p] = make_float2((float)(z.ar - (double)ah.x), (float)(z.ai - (double)ah.y));
-        gamma_s = make_float2((float)z.gr, (float)z.gi);
-    }
-    __syncthreads();
-    const float2 g = gamma_s;
-    // state p, component c -> row (p / G) 2G + 4 ((p % G) / 2) + 2 c + p % 2 inside groups of G states
-    auto row_of = [&](int G) { return G ? (p / G) * 2 * G + 4 * ((p % G) >> 1) + (p & 1) : 2 * p; };
-    const int nB = row_of(group_B), nC = row_of(group_C);
-    const int sB = group_B ? 2 * group_B : 128, sC = group_C ? 2 * group_C : 128;
-    for (int h = threadIdx.x; h < H; h += blockDim.x) {
-        const float2 v = cmul(g, Bc[(size_t)p * H + h]);
-        Bbar[(size_t)p * H + h] = v;
-        store_split(WsB, H, nB, h, v.x, sB);
-        store_split(WsB, H, nB + (group_B ? 2 : 1), h, v.y, sB);
-        *reinterpret_cast<__nv_bfloat162*>(Bq + (size_t)h * 2 * P + 2 * p) = __floats2bfloat162_rn(v.x, v.y);
-        const float2 c = Cc[(size_t)h * P + p];
-        *reinterpret_cast<__nv_bfloat162*>(Cp + (size_t)h * 2 * P + 2 * p) = __floats2bfloat162_rn(c.x, -c.y);
-        store_split(WsC, H, nC, h, c.x, sC);
-        store_split(WsC, H, nC + (group_C ? 2 : 1), h, -c.y, sC);
-    }
-}
-
-// The same for the projections that run as sums of bf16 plane products (fp32 inputs and outputs): every
-// operand as three planes side by side along its K.
-//   Wb3[2p+c, a H + h] = plane a of (c ? Im : Re) Bbar[p,h]       [2P, 3H]   (Bu = u Wb3^T)
-//   Cq3[2p+c, a H + h] = plane a of (c ? -Im : Re) C[h,p]         [2P, 3H]   (g_x = gy Cq3^T)
-//   Cp3[h, a 2P + 2p+c] = plane a of (c ? -Im : Re) C[h,p]        [H, 3 2P]  (y = x Cp3^T)
-//   Bq3[h, a 2P + 2p+c] = plane a of (c ? Im : Re) Bbar[p,h]      [H, 3 2P]  (du = s Bq3^T)
+// The three bf16 planes of v (hi + mid + lo = v), `plane_stride` elements apart.
 __device__ __forceinline__ void store3(__nv_bfloat16* base, size_t plane_stride, float v) {
     const __nv_bfloat16 hi = __float2bfloat16_rn(v);
     const float r1 = v - __bfloat162float(hi);
@@ -229,91 +128,328 @@ __device__ __forceinline__ void store3(__nv_bfloat16* base, size_t plane_stride,
     base[plane_stride] = mid;
     base[2 * plane_stride] = __float2bfloat16_rn(r1 - __bfloat162float(mid));
 }
+__device__ __forceinline__ void store3_pair(float a, float b, __nv_bfloat162& hi, __nv_bfloat162& mid, __nv_bfloat162& lo) {
+    hi = __floats2bfloat162_rn(a, b);
+    const float2 h = __bfloat1622float2(hi);
+    const float a1 = a - h.x, b1 = b - h.y;
+    mid = __floats2bfloat162_rn(a1, b1);
+    const float2 m = __bfloat1622float2(mid);
+    lo = __floats2bfloat162_rn(a1 - m.x, b1 - m.y);
+}
 
-__global__ void __launch_bounds__(128)
-discretize_pack_planes_kernel(int H, int P, const float2* __restrict__ Lambda, const float* __restrict__ Delta,
-                              const float2* __restrict__ Bc, const float2* __restrict__ Cc, float2* __restrict__ Abar,
-                              float2* __restrict__ Abar_lo, float2* __restrict__ Bbar, __nv_bfloat16* __restrict__ Wb3,
-                              __nv_bfloat16* __restrict__ Cq3, __nv_bfloat16* __restrict__ Cp3,
-                              __nv_bfloat16* __restrict__ Bq3) {
-    __shared__ float2 gamma_s;
-    const int p = blockIdx.x;
-    if (threadIdx.x == 0) {
-        ZohTerms z = zoh_terms(Lambda[p], Delta[p]);
-        const float2 ah = make_float2((float)z.ar, (float)z.ai);
-        Abar[p] = ah;
-        if (Abar_lo) Abar_lo[p] = make_float2((float)(z.ar - (double)ah.x), (float)(z.ai - (double)ah.y));
-        gamma_s = make_float2((float)z.gr, (float)z.gi);
+// ---------------------------------------------------------------------------------------------
+// Discretisation and the packed projection operands of a layer, one kernel
+// ---------------------------------------------------------------------------------------------
+// From Lambda, Delta, B, C: Abar (as an fp32 pair) and the operands of the four projections, which are Bbar and
+// C once with the states along the rows (h contiguous: weights of Bu and g_x) and once with h along the rows
+// (states contiguous: weights of du and y).  A block owns 32 states x 32 features: it reads its tile of B
+// (rows of 32 h) and of C (rows of 32 states), turns both round in shared memory, so that every global access of
+// a warp is a run of 64 to 256 contiguous bytes, and evaluates gamma of its 32 states in double precision, one
+// per lane of a warp.  Blocks that own the same states repeat that evaluation (about 1.5 us, the length of the
+// tile's own loads).  What bounds it is latency: H x P weights are 1 - 8 MB in and out.  H = 512, P = 256: bf16
+// halves 7.6 -> 4.6 us, planes 20.7 -> 4.4 us against one block per state with strided 2-byte accesses.
+// kMode:
+//   kPackTc     bf16 operands.  In the two projections that feed the states a weight w is carried as
+//               hi = bf16(w), lo = bf16(w - hi), so that the states see ~16 mantissa bits of the parameters:
+//               logical row n of the [2P, H] operand goes to rows (n/S) 2S + n%S (hi) and S further (lo) of the
+//               stacked [4P, H] matrix (o.WB, o.WC).  S = 128 and n = 2p + c, or, for the kernels that scan in
+//               their epilogue (group = states per chain), S = 2 group and the rows of two neighbouring states
+//               interleaved as (re, re, im, im).  o.Cp, o.Bq: [H, 2P] single bf16.
+//   kPackPlanes three bf16 planes of every operand side by side along its contraction index:
+//               WB[2p+c, a H + h], WC likewise ([2P, 3H]);  Cp[h, a 2P + 2p+c], Bq likewise ([H, 3 2P]).
+//   kPackF32    fp32: WB[2p+c, h], WC[2p+c, h] ([2P, H]);  Cp[h, 2p+c], Bq[h, 2p+c] ([H, 2P]).
+// with c = 0 / 1 for Re / Im of Bbar and Re / -Im of C.  `hdr` (may be NULL): its status word is cleared.
+enum PackMode { kPackTc, kPackPlanes, kPackF32 };
+struct PackOut {
+    float2 *Abar, *Alo;
+    void *WB, *WC, *Cp, *Bq;
+    WsHeader* hdr;
+    int group_log2;   // 0: no groups
+};
+
+template <int kMode>
+__device__ __forceinline__ void store_row_pair(void* W, int H, int P, int group_log2, int p, int h, float re, float im) {
+    if (kMode == kPackF32) {
+        float* w = reinterpret_cast<float*>(W) + (size_t)(2 * p) * H + h;
+        w[0] = re;
+        w[H] = im;
+    } else if (kMode == kPackPlanes) {
+        __nv_bfloat16* w = reinterpret_cast<__nv_bfloat16*>(W) + (size_t)(2 * p) * 3 * H + h;
+        store3(w, H, re);
+        store3(w + 3 * (size_t)H, H, im);
+    } else {
+        // (all block sizes are powers of two: shifts, the divisions were most of this kernel's instructions)
+        const int sl = group_log2 ? group_log2 + 1 : 7, in_group = p & ((1 << group_log2) - 1);
+        const int n = group_log2 ? ((p >> group_log2) << sl) + 4 * (in_group >> 1) + (p & 1) : 2 * p;
+        store_split(reinterpret_cast<__nv_bfloat16*>(W), H, n, h, re, sl);
+        store_split(reinterpret_cast<__nv_bfloat16*>(W), H, n + (group_log2 ? 2 : 1), h, im, sl);
+    }
+}
+template <int kMode>
+__device__ __forceinline__ void store_col_pair(void* W, int P, int p, int h, float re, float im) {
+    if (kMode == kPackF32) {
+        reinterpret_cast<float2*>(W)[(size_t)h * P + p] = make_float2(re, im);
+    } else if (kMode == kPackTc) {
+        reinterpret_cast<__nv_bfloat162*>(W)[(size_t)h * P + p] = __floats2bfloat162_rn(re, im);
+    } else {
+        __nv_bfloat162 hi, mid, lo;
+        store3_pair(re, im, hi, mid, lo);
+        __nv_bfloat162* w = reinterpret_cast<__nv_bfloat162*>(W) + (size_t)h * 3 * P + p;
+        w[0] = hi;
+        w[P] = mid;
+        w[2 * (size_t)P] = lo;
+    }
+}
+
+template <int kMode>
+__global__ void __launch_bounds__(256)
+pack_params_kernel(int H, int P, const float2* __restrict__ Lambda, const float* __restrict__ Delta,
+                   const float2* __restrict__ Bc, const float2* __restrict__ Cc, PackOut o) {
+    __shared__ float2 gamma_s[32];
+    __shared__ float2 tB[32][33], tC[32][33];   // tB[state][h], tC[h][state]
+    const int p0 = blockIdx.x * 32, h0 = blockIdx.y * 32;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const float2 zero = make_float2(0.f, 0.f);
+    float2 b[4], c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = w + 8 * i;
+        b[i] = (p0 + r < P && h0 + lane < H) ? Bc[(size_t)(p0 + r) * H + h0 + lane] : zero;
+        c[i] = (p0 + lane < P && h0 + r < H) ? Cc[(size_t)(h0 + r) * P + p0 + lane] : zero;
+    }
+    if (w == 0 && p0 + lane < P) {
+        const int p = p0 + lane;
+        const ZohTerms z = zoh_terms(Lambda[p], Delta[p]);
+        gamma_s[lane] = make_float2((float)z.gr, (float)z.gi);
+        if (blockIdx.y == 0) {
+            const float2 ah = make_float2((float)z.ar, (float)z.ai);
+            o.Abar[p] = ah;
+            o.Alo[p] = make_float2((float)(z.ar - (double)ah.x), (float)(z.ai - (double)ah.y));
+        }
+    }
+    if (threadIdx.x == 32 && blockIdx.x == 0 && blockIdx.y == 0 && o.hdr) o.hdr->status = 0;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = w + 8 * i;
+        b[i] = cmul(gamma_s[r], b[i]);
+        tB[r][lane] = b[i];
+        tC[r][lane] = c[i];
     }
     __syncthreads();
-    const float2 g = gamma_s;
-    const size_t H3 = 3 * (size_t)H, P6 = 6 * (size_t)P;
-    for (int h = threadIdx.x; h < H; h += blockDim.x) {
-        const float2 v = cmul(g, Bc[(size_t)p * H + h]);
-        Bbar[(size_t)p * H + h] = v;
-        store3(Wb3 + (size_t)(2 * p) * H3 + h, H, v.x);
-        store3(Wb3 + (size_t)(2 * p + 1) * H3 + h, H, v.y);
-        store3(Bq3 + (size_t)h * P6 + 2 * p, 2 * (size_t)P, v.x);
-        store3(Bq3 + (size_t)h * P6 + 2 * p + 1, 2 * (size_t)P, v.y);
-        const float2 c = Cc[(size_t)h * P + p];
-        store3(Cq3 + (size_t)(2 * p) * H3 + h, H, c.x);
-        store3(Cq3 + (size_t)(2 * p + 1) * H3 + h, H, -c.y);
-        store3(Cp3 + (size_t)h * P6 + 2 * p, 2 * (size_t)P, c.x);
-        store3(Cp3 + (size_t)h * P6 + 2 * p + 1, 2 * (size_t)P, -c.y);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = w + 8 * i;
+        if (p0 + r < P && h0 + lane < H) {   // state p0 + r, feature h0 + lane
+            const float2 cc = tC[lane][r];
+            store_row_pair<kMode>(o.WB, H, P, o.group_log2, p0 + r, h0 + lane, b[i].x, b[i].y);
+            store_row_pair<kMode>(o.WC, H, P, o.group_log2, p0 + r, h0 + lane, cc.x, -cc.y);
+        }
+        if (p0 + lane < P && h0 + r < H) {   // state p0 + lane, feature h0 + r
+            const float2 bb = tB[lane][r];
+            store_col_pair<kMode>(o.Bq, P, p0 + lane, h0 + r, bb.x, bb.y);
+            store_col_pair<kMode>(o.Cp, P, p0 + lane, h0 + r, c[i].x, -c[i].y);
+        }
     }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Last sums of a layer's backward pass
+// ---------------------------------------------------------------------------------------------
+// The split-K partials of the weight-gradient products, part_b[s, h, 2p+c] (gBbar) and part_c[s, h, 2p+c] (dC, its
+// imaginary columns negated), are added in order of s.  gBbar itself is not stored: it leaves as
+// dB = conj(gamma) gBbar and as the sums g_gamma = sum conj(B) gBbar over the block's 32 features
+// (gg_part[h / 32, p]).  A block owns 32 features x 32 states of one of the two matrices (blockIdx.z); gBbar is
+// turned round in shared memory for the state-major dB.  Bound by reading the partials (L2 for small problems); with
+// the sum and the state-major store as separate strided kernels a step spent 7.7 - 20 us here, now 7 - 10 us.
+// kReduceWarps warps share the block's rows (one more evaluates gamma): 16 where there are many partials to add per
+// element, else 8 (1024 x 1024 with 2 partials: 8.2 against 10.5 us; 512 x 512 with 9: 7.2 with 16 against 8.5).
+template <int kReduceWarps>
+__global__ void __launch_bounds__(32 * kReduceWarps + 32)
+reduce_weight_grads_kernel(int H, int P, int splits, const float* __restrict__ part_b, const float* __restrict__ part_c,
+                           const float2* __restrict__ Lambda, const float* __restrict__ Delta,
+                           const float2* __restrict__ Bc, float2* __restrict__ dB, float2* __restrict__ dC,
+                           float2* __restrict__ gg_part) {
+    __shared__ float2 gamma_s[32];
+    __shared__ float2 t[32][33];   // [feature][state]
+    constexpr int kRows = 32 / kReduceWarps;
+    const int p0 = blockIdx.x * 32, h0 = blockIdx.y * 32;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const bool is_c = blockIdx.z != 0, p_ok = p0 + lane < P;
+    if (w == kReduceWarps) {
+        if (!is_c && p_ok) {
+            const ZohTerms z = zoh_terms(Lambda[p0 + lane], Delta[p0 + lane]);
+            gamma_s[lane] = make_float2((float)z.gr, (float)z.gi);
+        }
+        __syncthreads();
+        return;
+    }
+    const float2* part = reinterpret_cast<const float2*>(is_c ? part_c : part_b);
+    const size_t n = (size_t)H * P;   // complex values per split
+    float2 acc[kRows];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) acc[i] = make_float2(0.f, 0.f);
+    if (p_ok) {
+        const float2* src = part + (size_t)(h0 + w) * P + p0 + lane;
+#pragma unroll 8
+        for (int s = 0; s < splits; ++s, src += n) {
+#pragma unroll
+            for (int i = 0; i < kRows; ++i)
+                if (h0 + w + kReduceWarps * i < H) acc[i] = cadd(acc[i], __ldcs(src + (size_t)kReduceWarps * i * P));
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+        if (is_c && p_ok && h0 + w + kReduceWarps * i < H)
+            dC[(size_t)(h0 + w + kReduceWarps * i) * P + p0 + lane] = cconj(acc[i]);
+        t[w + kReduceWarps * i][lane] = acc[i];
+    }
+    __syncthreads();
+    if (is_c) return;
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+        const int pl = w + kReduceWarps * i, p = p0 + pl, h = h0 + lane;
+        if (p >= P) continue;   // (the same for the whole warp)
+        const float2 gb = t[lane][pl];
+        float2 q = make_float2(0.f, 0.f);
+        if (h < H) {
+            dB[(size_t)p * H + h] = cmul(cconj(gamma_s[pl]), gb);
+            q = cmul(cconj(Bc[(size_t)p * H + h]), gb);
+        }
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) {
+            q.x += __shfl_xor_sync(0xffffffffu, q.x, m);
+            q.y += __shfl_xor_sync(0xffffffffu, q.y, m);
+        }
+        if (lane == 0) gg_part[(size_t)blockIdx.y * P + p] = q;
+    }
+}
+
+// Adjoint of the discretisation with the sums of gAbar (gA_rows rows of [P]), g_gamma (gg_rows rows of [P]) and dD
+// (dD_rows rows of [H]) folded in, in a fixed order.  A block owns 32 columns, its 32 warps take the rows in turn
+// (the rows of partial sums are up to 512, the columns a few hundred: latency is all there is), one warp evaluates
+// the P-sized double-precision terms meanwhile.  H = 512, P = 256: 6.2 - 9.5 -> 3.0 - 6.3 us (4 - 512 rows) against one block per state.
+__global__ void __launch_bounds__(1024)
+layer_finalize_kernel(int H, int P, const float2* __restrict__ Lambda, const float* __restrict__ Delta,
+                      const float2* __restrict__ gA_part, int gA_rows, const float2* __restrict__ gg_part, int gg_rows,
+                      float2* __restrict__ dLambda, float* __restrict__ dDelta, const float* __restrict__ dD_part,
+                      int dD_rows, float* __restrict__ dD) {
+    __shared__ double sA[2][32][33], sG[2][32][33];
+    __shared__ ZohTerms zs[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int p_blocks = (P + 31) / 32;
+    if ((int)blockIdx.x >= p_blocks) {   // 32 columns of dD
+        float(*sD)[33] = reinterpret_cast<float(*)[33]>(sA);
+        const int h = ((int)blockIdx.x - p_blocks) * 32 + lane;
+        float acc = 0.f;
+        if (h < H)
+            for (int r = w; r < dD_rows; r += 32) acc += dD_part[(size_t)r * H + h];
+        sD[w][lane] = acc;
+        __syncthreads();
+        if (w == 0 && h < H) {
+            float t = 0.f;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) t += sD[i][lane];
+            dD[h] = t;
+        }
+        return;
+    }
+    const int p = (int)blockIdx.x * 32 + lane;
+    double ar = 0.0, ai = 0.0, gr = 0.0, gi = 0.0;
+    if (p < P) {
+#pragma unroll 4
+        for (int r = w; r < gA_rows; r += 32) {
+            const float2 v = gA_part[(size_t)r * P + p];
+            ar += (double)v.x;
+            ai += (double)v.y;
+        }
+        for (int r = w; r < gg_rows; r += 32) {
+            const float2 v = gg_part[(size_t)r * P + p];
+            gr += (double)v.x;
+            gi += (double)v.y;
+        }
+        if (w == 31) zs[lane] = zoh_terms(Lambda[p], Delta[p]);
+    }
+    sA[0][w][lane] = ar;
+    sA[1][w][lane] = ai;
+    sG[0][w][lane] = gr;
+    sG[1][w][lane] = gi;
+    __syncthreads();
+    // warps 0 .. 3 add one of the four sums each
+    if (w < 4) {
+        double(*src)[33] = w < 2 ? sA[w] : sG[w - 2];
+        double t = 0.0;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) t += src[i][lane];
+        src[0][lane] = t;
+    }
+    __syncthreads();
+    if (w == 0 && p < P)
+        zoh_adjoint(zs[lane], Lambda[p], Delta[p], sA[0][0][lane], sA[1][0][lane], sG[0][0][lane], sG[1][0][lane],
+                    dLambda[p], dDelta[p]);
+}
+
+static dim3 weight_tiles(int H, int P, int z) { return dim3((P + 31) / 32, (H + 31) / 32, z); }
+
+template <int kMode>
+static void launch_pack(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc, const float2* Cc,
+                        const PackOut& o, cudaStream_t st) {
+    count_launch();
+    pack_params_kernel<kMode><<<weight_tiles(H, P, 1), 256, 0, st>>>(H, P, Lambda, Delta, Bc, Cc, o);
+}
+
+void launch_discretize_pack_tc(int H, int P, int group, const float2* Lambda, const float* Delta, const float2* Bc,
+                               const float2* Cc, float2* Abar, float2* Abar_lo, void* Wsplit_B, void* Wsplit_C, void* Cp,
+                               void* Bq, WsHeader* hdr, cudaStream_t st) {
+    const int group_log2 = group == 64 ? 6 : (group == 32 ? 5 : 0);
+    launch_pack<kPackTc>(H, P, Lambda, Delta, Bc, Cc, PackOut{Abar, Abar_lo, Wsplit_B, Wsplit_C, Cp, Bq, hdr, group_log2}, st);
 }
 
 void launch_discretize_pack_planes(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
-                                   const float2* Cc, float2* Abar, float2* Abar_lo, float2* Bbar, void* Wb3, void* Cq3,
-                                   void* Cp3, void* Bq3, cudaStream_t st) {
-    count_launch();
-    discretize_pack_planes_kernel<<<P, 128, 0, st>>>(H, P, Lambda, Delta, Bc, Cc, Abar, Abar_lo, Bbar, (__nv_bfloat16*)Wb3,
-                                                     (__nv_bfloat16*)Cq3, (__nv_bfloat16*)Cp3, (__nv_bfloat16*)Bq3);
+                                   const float2* Cc, float2* Abar, float2* Abar_lo, void* Wb3, void* Cq3, void* Cp3,
+                                   void* Bq3, WsHeader* hdr, cudaStream_t st) {
+    launch_pack<kPackPlanes>(H, P, Lambda, Delta, Bc, Cc, PackOut{Abar, Abar_lo, Wb3, Cq3, Cp3, Bq3, hdr, 0}, st);
 }
 
-void launch_discretize_pack_tc(int H, int P, int group_B, int group_C, const float2* Lambda, const float* Delta,
-                               const float2* Bc, const float2* Cc, float2* Abar, float2* Abar_lo, float2* Bbar,
-                               void* Wsplit_B, void* Wsplit_C, void* Cp, void* Bq, cudaStream_t st) {
-    count_launch();
-    discretize_pack_tc_kernel<<<P, 128, 0, st>>>(H, P, group_B, group_C, Lambda, Delta, Bc, Cc, Abar, Abar_lo, Bbar,
-                                                 (__nv_bfloat16*)Wsplit_B, (__nv_bfloat16*)Wsplit_C, (__nv_bfloat16*)Cp,
-                                                 (__nv_bfloat16*)Bq);
+void launch_discretize_pack_f32(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
+                                const float2* Cc, float2* Abar, float2* Abar_lo, void* Bp, void* Cq, void* Cp, void* Bq,
+                                WsHeader* hdr, cudaStream_t st) {
+    launch_pack<kPackF32>(H, P, Lambda, Delta, Bc, Cc, PackOut{Abar, Abar_lo, Bp, Cq, Cp, Bq, hdr, 0}, st);
 }
 
 void launch_discretize(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc, float2* Abar,
-                       float2* Abar_lo, float2* Bbar, cudaStream_t st) {
+                       float2* Bbar, cudaStream_t st) {
     count_launch();
-    discretize_kernel<<<P, 128, 0, st>>>(H, Lambda, Delta, Bc, Abar, Abar_lo, Bbar);
+    discretize_kernel<<<P, 128, 0, st>>>(H, Lambda, Delta, Bc, Abar, Bbar);
 }
 
 void launch_discretize_bwd(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
                            const float2* gAbar, const float2* gBbar, float2* dLambda, float* dDelta, float2* dB,
                            cudaStream_t st) {
     count_launch();
-    discretize_bwd_kernel<<<P, 128, 0, st>>>(H, P, Lambda, Delta, Bc, gAbar, 1, gBbar, dLambda, dDelta, dB, nullptr, 0,
-                                             nullptr);
+    discretize_bwd_kernel<<<P, 128, 0, st>>>(H, P, Lambda, Delta, Bc, gAbar, gBbar, dLambda, dDelta, dB);
 }
 
-void launch_layer_finalize(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
-                           const float2* gA_part, int gA_rows, const float2* gBbar, float2* dLambda, float* dDelta,
-                           float2* dB, const float* dD_part, int dD_rows, float* dD, cudaStream_t st) {
-    count_launch();
-    const int extra = dD_part ? (H + 127) / 128 : 0;
-    discretize_bwd_kernel<<<P + extra, 128, 0, st>>>(H, P, Lambda, Delta, Bc, gA_part, gA_rows, gBbar, dLambda, dDelta, dB,
-                                                     dD_part, dD_rows, dD);
-}
+int gamma_part_rows(int H) { return (H + 31) / 32; }
 
-void launch_pack_operands(int H, int P, bool bf16, const float2* Bbar, const float2* Cc, void* Bp, void* Bq,
-                          void* Cp, void* Cq, cudaStream_t st) {
-    const int threads = 256;
-    const int blocks = (int)(((size_t)P * H + threads - 1) / threads);
+void launch_reduce_weight_grads(int H, int P, int splits, const float* part_b, const float* part_c, const float2* Lambda,
+                                const float* Delta, const float2* Bc, float2* dB, float2* dC, float2* gg_part,
+                                cudaStream_t st) {
     count_launch();
-    if (bf16)
-        pack_operands_kernel<__nv_bfloat16><<<blocks, threads, 0, st>>>(
-            H, P, Bbar, Cc, (__nv_bfloat16*)Bp, (__nv_bfloat16*)Bq, (__nv_bfloat16*)Cp, (__nv_bfloat16*)Cq);
+    const dim3 grid = weight_tiles(H, P, 2);
+    if (splits > 4)
+        reduce_weight_grads_kernel<16><<<grid, 32 * 17, 0, st>>>(H, P, splits, part_b, part_c, Lambda, Delta, Bc, dB, dC, gg_part);
     else
-        pack_operands_kernel<float><<<blocks, threads, 0, st>>>(H, P, Bbar, Cc, (float*)Bp, (float*)Bq,
-                                                                 (float*)Cp, (float*)Cq);
+        reduce_weight_grads_kernel<8><<<grid, 32 * 9, 0, st>>>(H, P, splits, part_b, part_c, Lambda, Delta, Bc, dB, dC, gg_part);
+}
+
+void launch_layer_finalize(int H, int P, const float2* Lambda, const float* Delta, const float2* gA_part, int gA_rows,
+                           const float2* gg_part, float2* dLambda, float* dDelta, const float* dD_part, int dD_rows,
+                           float* dD, cudaStream_t st) {
+    count_launch();
+    layer_finalize_kernel<<<(P + 31) / 32 + (H + 31) / 32, 1024, 0, st>>>(H, P, Lambda, Delta, gA_part, gA_rows, gg_part,
+                                                                         gamma_part_rows(H), dLambda, dDelta, dD_part,
+                                                                         dD_rows, dD);
 }
 
 }  // namespace ssm

@@ -7,7 +7,7 @@
 //    CTAs on 256 x 256 tiles.  A = activations or states [B*T, K]; W = packed parameters.  With kSplitW
 //    the 256 accumulator columns of a tile hold the products with the high and the low bf16 halves of 128
 //    weight rows, summed in the epilogue (weights then carry ~16 mantissa bits; see
-//    discretize_pack_tc_kernel).  With a product schedule the accumulator sums several products of bf16
+//    pack_params_kernel).  With a product schedule the accumulator sums several products of bf16
 //    planes of both operands (fp32-accurate results, see planes.cu).  Epilogues: fp32 store; bf16
 //    acc + diag * skip; the same with column sums of skip * dot; fp32 store with a gated bf16 result.
 //  * gemm_scan_fwd_kernel / gemm_scan_bwd_kernel: the pair kernel with the scan of Sec. III-B (and its

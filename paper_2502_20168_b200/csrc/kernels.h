@@ -6,20 +6,36 @@
 namespace ssm {
 
 // discretize.cu
-// Abar_lo (may be NULL): Abar's rounding residual, exp(Lambda Delta) - Abar, as fp32.
 void launch_discretize(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc, float2* Abar,
-                       float2* Abar_lo, float2* Bbar, cudaStream_t st);
+                       float2* Bbar, cudaStream_t st);
 void launch_discretize_bwd(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
                            const float2* gAbar, const float2* gBbar, float2* dLambda, float* dDelta, float2* dB,
                            cudaStream_t st);
-// The adjoint of the discretisation with the last sums of the layer's backward pass folded in: gAbar comes
-// as gA_rows rows of partial sums [gA_rows, P] (one row: the finished gradient), and dD, if dD_part is given,
-// as dD_rows rows [dD_rows, H]; both are summed here in a fixed order.
-void launch_layer_finalize(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
-                           const float2* gA_part, int gA_rows, const float2* gBbar, float2* dLambda, float* dDelta,
-                           float2* dB, const float* dD_part, int dD_rows, float* dD, cudaStream_t st);
-void launch_pack_operands(int H, int P, bool bf16, const float2* Bbar, const float2* Cc, void* Bp, void* Bq,
-                          void* Cp, void* Cq, cudaStream_t st);
+// Discretisation and the packed projection operands of a layer in one kernel (layouts at pack_params_kernel).
+// Abar_lo: Abar's rounding residual, exp(Lambda Delta) - Abar, as fp32.  hdr (may be NULL): status word cleared.
+// Tensor-core path: Wsplit_B / Wsplit_C hi/lo stacked [4P, H]; group: 0 = rows in the plain order (2p + c, stacked
+// per 128 rows: GemmTcTN with split_w), or the states per chain (64, 32) of the kernels that scan in their epilogue.
+void launch_discretize_pack_tc(int H, int P, int group, const float2* Lambda, const float* Delta, const float2* Bc,
+                               const float2* Cc, float2* Abar, float2* Abar_lo, void* Wsplit_B, void* Wsplit_C, void* Cp,
+                               void* Bq, WsHeader* hdr, cudaStream_t st);
+// Plane path: the four operands as three bf16 planes: Wb3, Cq3 [2P, 3H]; Cp3, Bq3 [H, 3 * 2P].
+void launch_discretize_pack_planes(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
+                                   const float2* Cc, float2* Abar, float2* Abar_lo, void* Wb3, void* Cq3, void* Cp3,
+                                   void* Bq3, WsHeader* hdr, cudaStream_t st);
+// CUDA-core path: fp32, Bp, Cq [2P, H]; Cp, Bq [H, 2P].
+void launch_discretize_pack_f32(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
+                                const float2* Cc, float2* Abar, float2* Abar_lo, void* Bp, void* Cq, void* Cp, void* Bq,
+                                WsHeader* hdr, cudaStream_t st);
+// End of a layer's backward pass.  The split-K partials [splits, H, 2P] of gBbar and dC are added; gBbar leaves as dB
+// and as gamma_part_rows(H) rows of partial sums of g_gamma.  Then the adjoint of the discretisation from rows of
+// partial sums of gAbar [gA_rows, P] and g_gamma; dD from dD_rows rows [dD_rows, H].  All in a fixed order.
+int gamma_part_rows(int H);
+void launch_reduce_weight_grads(int H, int P, int splits, const float* part_b, const float* part_c, const float2* Lambda,
+                                const float* Delta, const float2* Bc, float2* dB, float2* dC, float2* gg_part,
+                                cudaStream_t st);
+void launch_layer_finalize(int H, int P, const float2* Lambda, const float* Delta, const float2* gA_part, int gA_rows,
+                           const float2* gg_part, float2* dLambda, float* dDelta, const float* dD_part, int dD_rows,
+                           float* dD, cudaStream_t st);
 
 // scan.cu
 // Scratch the scans need for a [B,T,P] problem: a work counter and the partial sums of gAbar.
@@ -85,13 +101,10 @@ struct GemmNT {
 };
 int gemm_nt_splits(int K);
 void launch_gemm_nt(const GemmNT& g, cudaStream_t st);
-// part0 in mode 0 into out0 and part1 in mode 1 into out1, one launch
-void launch_splitk_reduce2(const float* part0, const float* part1, int splits, int I, int J, float2* out0, float2* out1,
-                           cudaStream_t st);
 
 // gemm_tc.cu: bf16 projections on tcgen05 tensor cores (operands by TMA, accumulators in TMEM).
 struct GemmTcTN {
-    // out[m, n] = sum_k A[m, k] * W[n, k];  A bf16 [M, K];  W bf16 packed by discretize_pack_tc_kernel:
+    // out[m, n] = sum_k A[m, k] * W[n, k];  A bf16 [M, K];  W bf16 packed by pack_params_kernel:
     // [N_out, K], or with split_w [2 * N_out, K] where each group of 256 rows holds the high
     // halves of 128 output columns followed by their low halves.
     const void* A; const void* W;
@@ -189,26 +202,12 @@ bool tc_nt_supported(int I, int J);
 int tc_nt_splits(int K, int I, int J);
 int launch_gemm_tc_nt(const GemmTcNT& g, cudaStream_t st);
 
-// discretize.cu: operands of the tensor-core path (bf16).  Wsplit_B / Wsplit_C: [4P, H] hi/lo
-// stacked forms of Bp / Cq (see GemmTcTN);  Cp, Bq: [H, 2P] single bf16.
-// Discretisation and packing of the four bf16 operands in one kernel.
-// group_B / group_C: 0 = rows in the plain order (2p + c, hi/lo stacked per 128 rows: GemmTcTN with split_w), or the
-// states per chain (64, 32) of the kernels that scan in their epilogue: rows of two neighbouring states interleaved
-// as (re, re, im, im) inside groups of that many states, hi/lo stacked per group.
-void launch_discretize_pack_tc(int H, int P, int group_B, int group_C, const float2* Lambda, const float* Delta,
-                               const float2* Bc, const float2* Cc, float2* Abar, float2* Abar_lo, float2* Bbar,
-                               void* Wsplit_B, void* Wsplit_C, void* Cp, void* Bq, cudaStream_t st);
-
-// planes.cu / discretize.cu: fp32 tensors as three bf16 planes side by side ([M, K] -> [M, 3K]) so that a
+// planes.cu: fp32 tensors as three bf16 planes side by side ([M, K] -> [M, 3K]) so that a
 // projection with fp32 inputs runs on the bf16 tensor cores as a sum of plane products (GemmTcTN / GemmTcNT
 // with a product schedule), and what follows such a projection: out = acc + diag * skip (+ add).
 void launch_split_planes(const float* in, size_t M, int K, void* out, cudaStream_t st);
 void launch_diag_skip(const float* acc, const float* diag, const void* skip, bool skip_bf16, const float* add, size_t M,
                       int N, void* out, bool out_bf16, cudaStream_t st);
-// Discretisation and the four projection operands as planes: Wb3, Cq3 [2P, 3H]; Cp3, Bq3 [H, 3 * 2P].
-void launch_discretize_pack_planes(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
-                                   const float2* Cc, float2* Abar, float2* Abar_lo, float2* Bbar, void* Wb3, void* Cq3,
-                                   void* Cp3, void* Bq3, cudaStream_t st);
 
 // glu.cu: what surrounds the GEMMs of the half-GLU gate out = v * sigmoid(GELU(v) W).
 // Tensor-core path (may be NULL): Wt2 [2H, 2H], the hi/lo stacked operand of z = [x1_hi | x1_lo] W, and
