@@ -85,7 +85,7 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true) {
     p.scan = take(off, scan_scratch_bytes(s.B, s.T, s.P, 2));
     p.part = take(off, (size_t)2 * p.splits * 2 * PH * 4);   // split-K partials of gBbar, then those of dC
     {   // dD: partial column sums of gy * u, from the stand-alone kernel or from the epilogue of the du projection
-        const size_t rows = (size_t)tc_tn_dot_max_rows();
+        const size_t rows = (size_t)tc_tn_dot_max_rows((int)BT, s.H);
         const size_t fused = rows * s.H + colsum_tmp_floats((int)rows, s.H);
         p.dot = take(off, std::max(dot_columns_tmp_floats((int)BT, s.H), fused) * 4);
     }
@@ -304,8 +304,9 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
                                  at<char>(ws, p.scan), st);
             if (rc) return rc;
         }
-        {   // y = x Cp^T + D u: planes of x, six products, then the skip term
+        {   // y = x Cp^T + D u: planes of x, six products, the skip term in the epilogue or after it
             StageTimer tm("gemm_y", st);
+            const bool small = tc_tn_small(BT, s.H, false);
             launch_split_planes(at<float>(ws, p.xs), (size_t)BT, P2, at<void>(ws, p.x3), st);
             GemmTcTN g{at<void>(ws, p.x3), at<void>(ws, p.W2), BT, s.H, P2, false, true, at<void>(ws, p.acc), nullptr,
                        nullptr, hdr};
@@ -314,8 +315,11 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
             g.planes_w = 3;
             g.prod_a = kProd6A;
             g.prod_w = kProd6B;
+            if (small) {
+                g.store_f32 = !io.y_bf16, g.out = y, g.diag = D, g.skip = u, g.skip_bf16 = io.u_bf16;
+            }
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
-            launch_diag_skip(at<float>(ws, p.acc), D, u, io.u_bf16, nullptr, (size_t)BT, s.H, y, io.y_bf16, st);
+            if (!small) launch_diag_skip(at<float>(ws, p.acc), D, u, io.u_bf16, nullptr, (size_t)BT, s.H, y, io.y_bf16, st);
         }
     } else {
         {
@@ -454,7 +458,6 @@ SSM_API int ssm_glu_fwd(const ssm_shape* shape, const float* W, const void* v, v
     const int M = s.B * s.T;
     const size_t n = (size_t)M * s.H;
     WsHeader* hdr = at<WsHeader>(ws, p.hdr);
-    const bool fused_gate = p.tc && tc_tn_gate_supported(M, s.H, 2 * s.H);
     if (cudaMemsetAsync(ws, 0, sizeof(WsHeader), st) != cudaSuccess) return SSM_ERR_CUDA;
     {
         StageTimer tm("glu_pack_gelu", st);
@@ -466,19 +469,23 @@ SSM_API int ssm_glu_fwd(const ssm_shape* shape, const float* W, const void* v, v
         StageTimer tm("glu_gemm_z", st);
         if (p.tc) {
             // both planes of x1 along K: a single bf16 rounding of x1 here costs 2e-2 on dW
-            GemmTcTN g{at<void>(ws, p.x1), at<void>(ws, p.Wt), M, s.H, 2 * s.H, true, true, at<void>(ws, p.z), nullptr, nullptr, hdr};
-            if (fused_gate) {   // out = v * sigmoid(z) leaves from the same epilogue
-                g.skip = v;
-                g.gate_out = out;
+            // out = v * sigmoid(z) leaves from the same epilogue
+            GemmTcTN g{at<void>(ws, p.x1), at<void>(ws, p.Wt), M, s.H, 2 * s.H, true, true, at<void>(ws, p.z), nullptr, v, hdr};
+            g.gate_out = out;
+            if (tc_tn_small(M, s.H, true)) {   // the same three products as a schedule: lo hi, hi lo, hi hi
+                g.K = s.H, g.split_w = false, g.w_plane_rows = 128, g.w_pitch = 2 * s.H;
+                g.n_products = 3, g.planes_a = 2, g.planes_w = 2, g.prod_a = 0x001u, g.prod_w = 0x010u;
+                if (int rc = launch_gemm_tc_tn_small(g, st)) return rc;
+            } else if (int rc = launch_gemm_tc_tn(g, st)) {
+                return rc;
             }
-            if (int rc = launch_gemm_tc_tn(g, st)) return rc;
         } else {
             GemmTN g{at<void>(ws, p.x1), false, s.H, at<void>(ws, p.Wt), false, s.H, M, s.H, s.H, Epi::StoreF32,
                      at<void>(ws, p.z), false, nullptr, nullptr, false, nullptr};
             launch_gemm_tn(g, st);
         }
     }
-    if (!fused_gate) {
+    if (!p.tc) {
         StageTimer tm("glu_out", st);
         launch_glu_out(bf16, n, v, at<float>(ws, p.z), out, st);
     }
@@ -629,8 +636,9 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
                                  at<char>(ws, p.scan), st, &gA_part, &gA_rows);
             if (rc) return rc;
         }
-        {   // du = s Bq^T + D gy (+ the residual branch's gradient)
+        {   // du = s Bq^T + D gy (+ the residual branch's gradient); where the epilogue does that, dD's sums as well
             StageTimer tm("gemm_du", st);
+            const bool small = tc_tn_small(BT, s.H, false);
             launch_split_planes(at<float>(ws, p.gs), (size_t)BT, P2, at<void>(ws, p.s3), st);
             GemmTcTN g{at<void>(ws, p.s3), at<void>(ws, p.W3), BT, s.H, P2, false, true, at<void>(ws, p.acc), nullptr,
                        nullptr, hdr};
@@ -639,8 +647,13 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
             g.planes_w = 3;
             g.prod_a = kProd6A;
             g.prod_w = kProd6B;
+            if (small) {
+                g.store_f32 = !io.du_bf16, g.out = du, g.diag = D, g.skip = gy, g.skip_bf16 = gyb, g.add = du_add;
+                g.dot = u, g.dot_bf16 = ub, g.dot_part = at<float>(ws, p.dot), g.dot_rows = &dD_rows;
+                dD_part = g.dot_part;
+            }
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
-            launch_diag_skip(at<float>(ws, p.acc), D, gy, gyb, du_add, (size_t)BT, s.H, du, io.du_bf16, st);
+            if (!small) launch_diag_skip(at<float>(ws, p.acc), D, gy, gyb, du_add, (size_t)BT, s.H, du, io.du_bf16, st);
         }
         {   // gBbar = s^T u
             StageTimer tm("gemm_gBbar", st);

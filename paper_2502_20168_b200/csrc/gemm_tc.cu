@@ -2,9 +2,9 @@
 // bf16 projections on the 5th-generation tensor cores (tcgen05.mma, accumulators in tensor
 // memory, operands staged in shared memory by TMA).  The kernels:
 //
-//  * gemm_tc_tn_kernel / gemm_tc_tn_pair_kernel: out[m, n] = sum_k A[m, k] * W[n, k]  (both operands
-//    K-contiguous).  Persistent; one CTA per SM walking 128 x 256 accumulator tiles, or clusters of two
-//    CTAs on 256 x 256 tiles.  A = activations or states [B*T, K]; W = packed parameters.  With kSplitW
+//  * gemm_tc_tn_pair_kernel: out[m, n] = sum_k A[m, k] * W[n, k]  (both operands K-contiguous).  Persistent
+//    clusters of two CTAs walking 256 x 256 accumulator tiles (problems with fewer tiles than CTA pairs:
+//    gemm_tc_small.cu).  A = activations or states [B*T, K]; W = packed parameters.  With kSplitW
 //    the 256 accumulator columns of a tile hold the products with the high and the low bf16 halves of 128
 //    weight rows, summed in the epilogue (weights then carry ~16 mantissa bits; see
 //    pack_params_kernel).  With a product schedule the accumulator sums several products of bf16
@@ -26,18 +26,14 @@
 #include <utility>
 
 #include "kernels.h"
-#include "tma.cuh"
+#include "tcgen05.cuh"
 
 namespace ssm {
 namespace tc {
 using namespace tma;
 
-constexpr int BM = 128;   // accumulator rows per tile = TMEM lanes
 constexpr int BN = 256;   // accumulator columns per tile
-constexpr int BK = 64;    // bf16 elements per shared-memory row: 128 bytes, one swizzle span
-constexpr int UK = 16;    // K extent of one tcgen05.mma of kind::f16
 constexpr int kStages = 4;      // shared-memory stages of the NT kernel (and size of the barrier arrays)
-constexpr int kTnStages = 3;    // the TN kernel gives one stage up for its epilogue buffers
 constexpr int kABytes = BM * BK * 2;
 constexpr int kBBytes = BN * BK * 2;
 constexpr int kStageBytes = kABytes + kBBytes;
@@ -58,158 +54,7 @@ __host__ __device__ constexpr int tn_diag_bytes(int epi) {
     return epi == 1 ? kMaxDiag * 4 : (epi == 3 ? kDotMaxN * 4 + kTnEpiWarps * (kDotMaxN / 2) * 4 : 0);
 }
 __host__ __device__ constexpr int tn_staging_bytes(int epi) { return epi == 2 ? kStagingBytes + kStagingBytes / 2 : kStagingBytes; }
-constexpr size_t tn_smem_bytes(int epi) {
-    return (size_t)kTnStages * kStageBytes + tn_staging_bytes(epi) + tn_skip_bytes(epi) + tn_diag_bytes(epi) +
-           1024 /*alignment slack*/ + 256 /*barriers*/;
-}
 constexpr size_t kNtSmemBytes = (size_t)kStages * kStageBytes + 1024 + 256;
-
-// ---------------------------------------------------------------------------------------------
-// PTX wrappers
-// ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t cols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(cols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// Arrives on the mbarrier once every MMA issued so far by this thread has completed.
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-// ---- CTA pairs (cta_group::2): one MMA spans the tensor cores and tensor memory of two CTAs
-// of a cluster; each CTA holds its 128 rows of A and its half of the B rows in shared memory at
-// the same offsets.  Allocation and release of tensor memory are issued by one warp of each CTA.
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-}
-// Address of the same shared-memory location in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// For data handed from one CTA of the cluster to the other through shared memory: the sender stores into the
-// peer's memory and arrives (release, cluster scope) on the peer's barrier, the receiver waits with acquire.
-__device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait_acquire_cluster(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait_acquire_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-    for (uint32_t i = 0; i < kSpinLimit; ++i) {
-        if (mbar_try_wait_acquire_cluster(bar, parity)) return true;
-        if ((i & 255u) == 255u && *abort_flag) return false;
-    }
-    *abort_flag = 1;
-    return false;
-}
-__device__ __forceinline__ void st_cluster_f4(uint32_t cluster_addr, float4 v) {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
-                 : "memory");
-}
-__device__ __forceinline__ void tmem_alloc_pair(uint32_t dst_smem, uint32_t cols) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(cols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t cols) {
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
-}
-// Asks L2 to fetch a contiguous range (a multiple of 16 bytes from a 16-byte aligned address).
-__device__ __forceinline__ void l2_prefetch_bulk(const void* ptr, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(ptr), "r"(bytes) : "memory");
-}
-// Tile load whose completion is counted on a barrier of either CTA of the pair (cluster address).
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar_cluster, int c0, int c1) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-        ::"r"(dst), "l"(map), "r"(bar_cluster), "r"(c0), "r"(c1)
-        : "memory");
-}
-__device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// Arrives on the barrier at this offset in both CTAs once every MMA issued so far has completed.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(bar), "h"((uint16_t)3) : "memory");
-}
-
-// 32 lanes x 32 consecutive 32-bit columns: thread i of the warp gets lane (base lane + i).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// Shared-memory matrix descriptors (128-byte swizzle).  Fields: start address >> 4 in bits
-// [0,14), leading byte offset >> 4 in [16,30), stride byte offset >> 4 in [32,46), descriptor
-// version 1 in [46,48), swizzle mode 2 (128 B) in [61,64).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-// K-major tile: rows of 128 bytes, groups of 8 rows 1024 bytes apart (leading offset unused).
-__device__ __forceinline__ uint64_t smem_desc_kmajor(uint32_t addr) { return smem_desc(addr, 16, 1024); }
-// MN-major tile made of [BK rows][64 elements] blocks: 64-element blocks 8192 bytes apart,
-// groups of 8 k-rows 1024 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc_mnmajor(uint32_t addr) { return smem_desc(addr, BK * 128, 1024); }
-
-// Instruction descriptor: D = f32 (bits [4,6) = 1), A = B = bf16 (bits [7,10), [10,13) = 1),
-// operand majors in bits 15 / 16 (0 = K), N >> 3 in [17,23), M >> 4 in [24,29).
-__host__ __device__ constexpr uint32_t instr_desc(int m, int n, int a_mn, int b_mn) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
-           ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
 
 struct Smem {
     uint8_t* tiles;       // 1024-byte aligned
@@ -539,104 +384,14 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
     return true;
 }
 
-// kEpi 0: store fp32;  kEpi 1: out = bf16(acc + diag[n] * skip[m, n]).
-// kSplitW: columns [0,128) and [128,256) of the accumulator tile are the hi and lo weight
-// halves of the same 128 output columns.
-template <int kEpi, bool kSplitW>
-__global__ void __launch_bounds__(kTnThreads, 1)
-gemm_tc_tn_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
-                  const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ CUtensorMap tmSkip,
-                  const __grid_constant__ CUtensorMap tmGate, TnParams p) {
-    extern __shared__ uint8_t smem_raw[];
-    const Smem s = carve_smem(smem_raw, kTnStages, tn_staging_bytes(kEpi), tn_diag_bytes(kEpi), kStageBytes, tn_skip_bytes(kEpi));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (kEpi == 1)   // (zero where the last tile reaches past the output's columns)
-        for (int i = threadIdx.x; i < p.n_tiles * BN; i += kTnThreads) s.diag[i] = i < p.ldo ? p.diag[i] : 0.f;
-    const uint32_t tmem_base = prologue(s, warp, lane, 32 * kTnEpiWarps);
-    const int m_tiles = (p.M + BM - 1) / BM;
-    const int total = m_tiles * p.n_tiles;
-    constexpr int kOutCols = kSplitW ? BN / 2 : BN;
-
-    if (warp == 0) {
-        if (lane == 0) {
-            prefetch_tmap(&tmA);
-            prefetch_tmap(&tmW);
-            int stage = 0;
-            uint32_t phase = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
-                const int m0 = (tile / p.n_tiles) * BM, n0 = (tile % p.n_tiles) * BN;
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!(ok = mbar_wait(s.empty(stage), phase ^ 1u, s.abort_flag))) break;
-                    mbar_expect_tx(s.full(stage), kStageBytes);
-                    const uint32_t a_dst = smem_u32(s.tiles + (size_t)stage * kStageBytes);
-                    tma_load_2d(a_dst, &tmA, s.full(stage), p.a_col(kb), m0);
-                    tma_load_2d(a_dst + kABytes, &tmW, s.full(stage), p.w_col(kb), n0);
-                    if (++stage == kTnStages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
-                }
-            }
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = instr_desc(BM, BN, 0, 0);
-            int stage = 0, acc = 0;
-            uint32_t phase = 0, acc_phase = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
-                if (!(ok = mbar_wait(s.tmem_empty(acc), acc_phase ^ 1u, s.abort_flag))) break;
-                tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!(ok = mbar_wait(s.full(stage), phase, s.abort_flag))) break;
-                    tc_fence_after();
-                    const uint32_t a_addr = smem_u32(s.tiles + (size_t)stage * kStageBytes);
-                    const uint64_t adesc = smem_desc_kmajor(a_addr);
-                    const uint64_t bdesc = smem_desc_kmajor(a_addr + kABytes);
-#pragma unroll
-                    for (int k = 0; k < BK / UK; ++k) {
-                        // 16 bf16 = 32 bytes further along the 128-byte row: +2 in the address field
-                        umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
-                                  (uint32_t)((kb | k) != 0));
-                    }
-                    umma_commit(s.empty(stage));
-                    if (++stage == kTnStages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
-                }
-                if (!ok) break;
-                umma_commit(s.tmem_full(acc));
-                if ((acc ^= 1) == 0) acc_phase ^= 1u;
-            }
-        }
-    } else {
-        int acc = 0;
-        uint32_t acc_phase = 0, skip_phase = 0;
-        bool ok = true;
-        for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
-            const int m0 = (tile / p.n_tiles) * BM, n_out0 = (tile % p.n_tiles) * kOutCols;
-            if (!(ok = tn_drain_tile<kEpi, kSplitW>(s, p, &tmOut, &tmSkip, &tmGate, warp, lane, m0, n_out0, acc, acc_phase, tmem_base,
-                                                    skip_phase)))
-                break;
-            tc_fence_before();
-            mbar_arrive(s.tmem_empty(acc));
-            if ((acc ^= 1) == 0) acc_phase ^= 1u;
-        }
-        if (lane == 0) tma_store_wait_all();
-    }
-    epilogue_exit(s, warp, tmem_base, p.hdr);
-}
-
 // ---------------------------------------------------------------------------------------------
 // TN kernel on CTA pairs
 // ---------------------------------------------------------------------------------------------
-// Same product, same epilogue, but a cluster of two CTAs works on a 256 x 256 accumulator tile:
+// kEpi: see tn_drain_tile.  kSplitW: columns [0,128) and [128,256) of the accumulator tile are the hi and lo weight
+// halves of the same 128 output columns.  A cluster of two CTAs works on a 256 x 256 accumulator tile:
 // CTA r holds rows m0 + 128 r .. of A and rows n0 + 128 r .. of the W tile, so every CTA brings
 // in 32 KB per k-block instead of 48 KB for the same number of tensor-core cycles (operand
-// delivery into the SM, not the tensor pipe, bounds the single-CTA kernel).  The leader (CTA 0)
+// delivery into the SM, not the tensor pipe, bounds a single-CTA kernel).  The leader (CTA 0)
 // issues the MMAs; its `full` barriers count the bytes of both CTAs' loads; its commits arrive
 // on the `empty` / `tmem_full` barriers of both CTAs; both CTAs' epilogue warps arrive on the
 // leader's `tmem_empty` barriers.
@@ -2109,21 +1864,6 @@ gemm_tc_nt_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 // ---------------------------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------------------------
-// Row-major bf16 matrix [rows, cols] (cols contiguous), boxes of box_cols x box_rows, 128-byte swizzle.
-static bool make_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols,
-                     uint32_t box_rows, bool f32 = false, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B,
-                     uint64_t pitch_elems = 0) {
-    PFN_cuTensorMapEncodeTiled fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {cols, rows};
-    cuuint64_t strides[1] = {(pitch_elems ? pitch_elems : cols) * (f32 ? 4u : 2u)};   // rows may be wider than the view
-    cuuint32_t box[2] = {box_cols, box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    return fn(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 static int sm_count() { return device_sm_count(); }
 
 // How many clusters of two CTAs of `kernel` the current device runs at the same time (cached per
@@ -2175,25 +1915,31 @@ bool tc_tn_supported(int M, int N_out, int K, bool split_w) {
 
 static int pair_tiles_of(int M, int n_tiles) { return ((M + 2 * tc::BM - 1) / (2 * tc::BM)) * n_tiles; }
 
-// The bf16 epilogue can also sum skip * dot over the rows (one partial row per CTA) where the pair kernel
-// runs and the output is at most kDotMaxN wide.
-bool tc_tn_dot_supported(int M, int N_out, int K) {
-    return tc_tn_supported(M, N_out, K, false) && N_out <= tc::kDotMaxN && pair_tiles_of(M, (N_out + tc::BN - 1) / tc::BN) >= tc::sm_count() / 2;
+// Too few 256-row tiles to give every CTA pair one.
+bool tc_tn_small(int M, int N_out, bool split_w) {
+    const int out_cols = split_w ? tc::BN / 2 : tc::BN;
+    return pair_tiles_of(M, (N_out + out_cols - 1) / out_cols) < tc::sm_count() / 2;
 }
-int tc_tn_dot_max_rows() { return 2 * tc::sm_count(); }
 
-bool tc_tn_gate_supported(int M, int N_out, int K) {
-    return tc_tn_supported(M, N_out, K, true) && pair_tiles_of(M, N_out / (tc::BN / 2)) >= tc::sm_count() / 2;
+// The bf16 epilogue can also sum skip * dot over the rows (one partial row per CTA); the pair kernel does for outputs
+// of at most kDotMaxN columns.
+bool tc_tn_dot_supported(int M, int N_out, int K) {
+    return tc_tn_supported(M, N_out, K, false) && (tc_tn_small(M, N_out, false) || N_out <= tc::kDotMaxN);
+}
+int tc_tn_dot_max_rows(int M, int N_out) {
+    return tc_tn_small(M, N_out, false) ? tc_tn_small_max_dot_rows(M) : 2 * tc::sm_count();
 }
 
 int launch_gemm_tc_tn(const GemmTcTN& g, cudaStream_t st) {
     using namespace tc;
+    if (tc_tn_small(g.M, g.N_out, g.split_w)) return launch_gemm_tc_tn_small(g, st);
+    if (g.a_f32 || g.add || g.w_plane_rows) return SSM_ERR_SHAPE;
     const int out_cols = g.split_w ? BN / 2 : BN;
     const int n_tiles = (g.N_out + out_cols - 1) / out_cols;
     const int epi = g.gate_out ? 2 : (g.store_f32 ? 0 : (g.dot ? 3 : 1));
     if ((epi == 1 || epi == 3) && (g.split_w || !g.diag || !g.skip)) return SSM_ERR_SHAPE;
     if (epi == 3 && (!g.dot_part || !g.dot_rows || !tc_tn_dot_supported(g.M, g.N_out, g.K))) return SSM_ERR_SHAPE;
-    if (epi == 2 && (!g.split_w || !g.store_f32 || !g.skip || !tc_tn_gate_supported(g.M, g.N_out, g.K))) return SSM_ERR_SHAPE;
+    if (epi == 2 && (!g.split_w || !g.store_f32 || !g.skip)) return SSM_ERR_SHAPE;
     CUtensorMap ma, mw, mo, ms, mg;
     // with a product schedule the operands are planes_a / planes_w bf16 planes of K columns each, side by side
     const int n_prod = g.n_products > 0 ? g.n_products : 1;
@@ -2216,47 +1962,30 @@ int launch_gemm_tc_tn(const GemmTcTN& g, cudaStream_t st) {
         return SSM_ERR_CUDA;   // (the dot operand travels in the map slot of the gated result)
     TnParams p{g.M, n_tiles, n_prod * (g.K / BK), g.N_out, g.diag, g.hdr, (const char*)g.A, (int)a_cols * 2, g.dot_part,
                g.n_products > 0 ? g.K / BK : 0, g.prod_a, g.prod_w};
-    const int m_tiles = (g.M + BM - 1) / BM;
     const int pair_tiles = pair_tiles_of(g.M, n_tiles);
     // rows of the packed weight matrix that exist (tiles may reach past them: those rows read as zero)
     const uint64_t w_rows = g.split_w ? (uint64_t)2 * g.N_out : (uint64_t)g.N_out;
     bool ok = true;
-    if (pair_tiles >= sm_count() / 2) {   // enough 256-row tiles to give every CTA pair one
-        if (!make_map(&mw, g.W, w_rows, w_cols, BK, BN / 2)) return SSM_ERR_CUDA;
-        count_launch();
-        // The kernel is persistent: its grid is the number of CTA pairs the device can hold at once
-        // (not every SM has a partner that a cluster may use).
-#define SSM_LAUNCH_PAIR(EPI, SPLIT)                                                                        \
-    do {                                                                                                   \
-        auto kern = gemm_tc_tn_pair_kernel<EPI, SPLIT>;                                                    \
-        constexpr size_t smem = pair_smem_bytes(EPI);                                                      \
-        ok = set_smem(kern, smem);                                                                         \
-        const int pairs = ok ? resident_pairs(reinterpret_cast<const void*>(kern), smem) : 0;              \
-        ok = ok && pairs > 0;                                                                              \
-        if (ok) kern<<<2 * min(pairs, pair_tiles), kTnThreads, smem, st>>>(ma, mw, mo, ms, mg, p);         \
-        if (ok && g.dot_rows) *g.dot_rows = 2 * min(pairs, pair_tiles);                                    \
-    } while (0)
-        if (epi == 3) SSM_LAUNCH_PAIR(3, false);
-        else if (epi == 2) SSM_LAUNCH_PAIR(2, true);
-        else if (epi == 1) SSM_LAUNCH_PAIR(1, false);
-        else if (g.split_w) SSM_LAUNCH_PAIR(0, true);
-        else SSM_LAUNCH_PAIR(0, false);
-#undef SSM_LAUNCH_PAIR
-        return ok ? SSM_OK : SSM_ERR_CUDA;
-    }
-    if (!make_map(&mw, g.W, w_rows, w_cols, BK, BN)) return SSM_ERR_CUDA;
-    const int grid = min(sm_count(), m_tiles * n_tiles);
+    if (!make_map(&mw, g.W, w_rows, w_cols, BK, BN / 2)) return SSM_ERR_CUDA;
     count_launch();
-#define SSM_LAUNCH_TN(EPI, SPLIT)                                                                          \
-    do {                                                                                                   \
-        auto kern = gemm_tc_tn_kernel<EPI, SPLIT>;                                                         \
-        ok = set_smem(kern, tn_smem_bytes(EPI));                                                           \
-        if (ok) kern<<<grid, kTnThreads, tn_smem_bytes(EPI), st>>>(ma, mw, mo, ms, mg, p);                 \
-    } while (0)
-    if (epi == 1) SSM_LAUNCH_TN(1, false);
-    else if (g.split_w) SSM_LAUNCH_TN(0, true);
-    else SSM_LAUNCH_TN(0, false);
-#undef SSM_LAUNCH_TN
+    // The kernel is persistent: its grid is the number of CTA pairs the device can hold at once
+    // (not every SM has a partner that a cluster may use).
+#define SSM_LAUNCH_PAIR(EPI, SPLIT)                                                                        \
+do {                                                                                                   \
+    auto kern = gemm_tc_tn_pair_kernel<EPI, SPLIT>;                                                    \
+    constexpr size_t smem = pair_smem_bytes(EPI);                                                      \
+    ok = set_smem(kern, smem);                                                                         \
+    const int pairs = ok ? resident_pairs(reinterpret_cast<const void*>(kern), smem) : 0;              \
+    ok = ok && pairs > 0;                                                                              \
+    if (ok) kern<<<2 * min(pairs, pair_tiles), kTnThreads, smem, st>>>(ma, mw, mo, ms, mg, p);         \
+    if (ok && g.dot_rows) *g.dot_rows = 2 * min(pairs, pair_tiles);                                    \
+} while (0)
+    if (epi == 3) SSM_LAUNCH_PAIR(3, false);
+    else if (epi == 2) SSM_LAUNCH_PAIR(2, true);
+    else if (epi == 1) SSM_LAUNCH_PAIR(1, false);
+    else if (g.split_w) SSM_LAUNCH_PAIR(0, true);
+    else SSM_LAUNCH_PAIR(0, false);
+#undef SSM_LAUNCH_PAIR
     return ok ? SSM_OK : SSM_ERR_CUDA;
 }
 

@@ -1,0 +1,502 @@
+// Tensor-core projections for problems of few tiles: training batches of a few thousand rows, single steps, and
+// the layers of a stack.
+//
+// The kernels of gemm_tc.cu walk 128 x 256 or 256 x 256 accumulator tiles, which is what a machine full of tiles
+// wants; 1024 rows x 512 columns are 16 such tiles, so 132 of 148 SMs idled and the time was the serial chain of
+// one tile's k-blocks (15 - 25 us with the six plane products of fp32 operands).  Here
+//  * a tile is 128 rows x 64, 128 or 256 columns, and a cluster of 1, 2 or 4 CTAs shares one tile, each taking a
+//    part of the contraction; the parts are added through distributed shared memory in the order of the ranks, so
+//    results repeat bit for bit and no partial sum goes through memory;
+//  * a k-block brings every plane of both operands into shared memory once and all products of the schedule are
+//    issued from it (the other kernels load a pair of planes per product: 12 tiles instead of 6);
+//  * an fp32 A operand needs no planes in memory: the warps that later run the epilogue read it, split it into its
+//    three bf16 planes and write them to the operand stages themselves;
+//  * the accumulator tile is staged in shared memory (over the operand stages, which are free by then) and read
+//    back by rows, so that the epilogue's operands and results are plain coalesced accesses in any type.
+#include <algorithm>
+
+#include "kernels.h"
+#include "tcgen05.cuh"
+
+namespace ssm {
+namespace tc {
+
+// Epilogue warps: 8, or 16 for tiles of 256 columns, whose CTAs are never shared (a CTA of 18 warps takes about
+// 1 us longer to start than one of 10, which small tiles would notice).
+__host__ __device__ constexpr int sm_epi_warps(int bn) { return bn == 256 ? 16 : 8; }
+__host__ __device__ constexpr int sm_threads(int bn) { return 64 + 32 * sm_epi_warps(bn); }
+constexpr int kSmMaxStages = 6;
+constexpr int kSmATile = BM * BK * 2;            // one plane of the A tile of a k-block
+constexpr size_t kSmSmemMax = 218 * 1024;        // of the 227 KB a CTA can have (the rest: static shared memory)
+
+struct SmallTnArgs {
+    int M, N;                  // rows; output columns
+    int n_tiles, cluster;      // tiles along N; CTAs per tile
+    int k_blocks;              // per product
+    int stages, stage_bytes;
+    int planes_a, planes_w, n_prod;
+    uint32_t prod_a, prod_w;   // product j: plane (prod_a >> 4 j) & 15 of A, (prod_w >> 4 j) & 15 of W
+    int a_plane, w_plane_cols, w_plane_rows, w_stacked;   // where the planes lie (w_stacked: hi / lo blocks of 128 rows)
+    const float* a_f32;        // A as fp32 [M, K] (planes made here), or NULL: bf16 planes by TMA
+    int K;
+    // epilogue
+    void* out;
+    const float* diag;
+    const void* skip;
+    const void* dot;
+    const float* add;
+    float* dot_part;
+    __nv_bfloat16* gate_out;
+    bool out_bf16, skip_bf16, dot_bf16;
+    WsHeader* hdr;
+};
+
+// Epilogues: fp32 result; out = acc + diag * skip (+ add) with, if asked for, the column sums of skip * dot over the
+// rows of this CTA; fp32 result and out2 = skip * sigmoid(acc) in bf16.
+enum SmallEpi { kSmStore, kSmDiag, kSmGate };
+
+// Four neighbouring values of an epilogue operand as loaded; decoded when they are used, so that many can be in
+// flight.  kBf16: the operands are known to be bf16 (half the registers), else the flag says.
+template <bool kBf16> struct Raw4;
+template <> struct Raw4<true> {
+    uint2 r;
+    __device__ __forceinline__ void load(const void* p, bool, size_t i) {
+        r = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(p) + i);
+    }
+    __device__ __forceinline__ float4 get(bool) const {
+        return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
+                           __uint_as_float(r.y & 0xffff0000u));
+    }
+};
+template <> struct Raw4<false> {
+    uint4 r;
+    __device__ __forceinline__ void load(const void* p, bool bf16, size_t i) {
+        if (bf16) {
+            const uint2 t = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(p) + i);
+            r.x = t.x, r.y = t.y;
+        } else {
+            r = *reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(p) + i);
+        }
+    }
+    __device__ __forceinline__ float4 get(bool bf16) const {
+        if (bf16) return Raw4<true>{make_uint2(r.x, r.y)}.get(true);
+        return make_float4(__uint_as_float(r.x), __uint_as_float(r.y), __uint_as_float(r.z), __uint_as_float(r.w));
+    }
+};
+__device__ __forceinline__ uint2 pack4_bf16(float4 v) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+    return make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+}
+__device__ __forceinline__ void store4_io(void* p, bool bf16, size_t i, float4 v) {
+    if (!bf16) *reinterpret_cast<float4*>(reinterpret_cast<float*>(p) + i) = v;
+    else *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p) + i) = pack4_bf16(v);
+}
+
+// Eight fp32 values -> the 16-byte chunks of their three bf16 planes (hi + mid + lo = value).
+__device__ __forceinline__ void split8(const float4 a, const float4 b, uint4& hi, uint4& mid, uint4& lo) {
+    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    uint32_t* h = &hi.x;
+    uint32_t* m = &mid.x;
+    uint32_t* l = &lo.x;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+        const float2 pf = __bfloat1622float2(p);
+        const float r0 = v[2 * i] - pf.x, r1 = v[2 * i + 1] - pf.y;
+        const __nv_bfloat162 q = __floats2bfloat162_rn(r0, r1);
+        const float2 qf = __bfloat1622float2(q);
+        const __nv_bfloat162 t = __floats2bfloat162_rn(r0 - qf.x, r1 - qf.y);
+        h[i] = *reinterpret_cast<const uint32_t*>(&p);
+        m[i] = *reinterpret_cast<const uint32_t*>(&q);
+        l[i] = *reinterpret_cast<const uint32_t*>(&t);
+    }
+}
+
+struct SmallBars {
+    uint64_t full[kSmMaxStages], empty[kSmMaxStages], done;
+    uint32_t tmem;
+    int abort_flag;
+};
+
+template <int kBN, int kEpi, bool kSplitA, bool kBf16>
+__global__ void __launch_bounds__(sm_threads(kBN), 1)
+gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, SmallTnArgs p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ SmallBars bars;
+    uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    constexpr int kSmEpiWarps = sm_epi_warps(kBN);
+    constexpr int kWTile = kBN * BK * 2;
+    constexpr int kPitch = kBN + 4;   // staging: floats per row; 16 bytes of padding keep both directions free of bank conflicts
+    volatile int* abort_flag = &bars.abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)cluster_ctarank(), tile = (int)blockIdx.x / p.cluster;
+    const int m0 = (tile / p.n_tiles) * BM, n0 = (tile % p.n_tiles) * kBN;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < p.stages; ++i) {
+            mbar_init(smem_u32(&bars.full[i]), kSplitA ? 1 + kSmEpiWarps : 1);
+            mbar_init(smem_u32(&bars.empty[i]), 1);
+        }
+        mbar_init(smem_u32(&bars.done), 1);
+        bars.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+    if (warp == 1) tmem_alloc(smem_u32(&bars.tmem), kBN);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = bars.tmem;
+    grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
+    grid_dep_launch();
+    const int kb0 = p.k_blocks * rank / p.cluster, kb1 = p.k_blocks * (rank + 1) / p.cluster;
+    const uint32_t a_bytes = (uint32_t)p.planes_a * kSmATile;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            if (!kSplitA) prefetch_tmap(&tmA);
+            prefetch_tmap(&tmW);
+            const uint32_t bytes = (uint32_t)p.planes_w * kWTile + (kSplitA ? 0u : a_bytes);
+            const int wrow = p.w_stacked ? (n0 / 128) * 256 + n0 % 128 : n0;
+            int stage = 0;
+            uint32_t phase = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
+                const uint32_t full = smem_u32(&bars.full[stage]);
+                const uint32_t dst = smem_u32(tiles) + (uint32_t)stage * (uint32_t)p.stage_bytes;
+                mbar_expect_tx(full, bytes);
+                if (!kSplitA)
+                    for (int a = 0; a < p.planes_a; ++a) tma_load_2d(dst + a * kSmATile, &tmA, full, a * p.a_plane + kb * BK, m0);
+                for (int w = 0; w < p.planes_w; ++w)
+                    tma_load_2d(dst + a_bytes + w * kWTile, &tmW, full, w * p.w_plane_cols + kb * BK, wrow + w * p.w_plane_rows);
+                if (++stage == p.stages) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = instr_desc(BM, kBN, 0, 0);
+            int stage = 0;
+            uint32_t phase = 0, accumulate = 0;
+            bool ok = true;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!(ok = mbar_wait(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
+                tc_fence_after();
+                const uint32_t base = smem_u32(tiles) + (uint32_t)stage * (uint32_t)p.stage_bytes;
+                for (int j = 0; j < p.n_prod; ++j) {
+                    const uint64_t ad = smem_desc_kmajor(base + ((p.prod_a >> (4 * j)) & 15u) * kSmATile);
+                    const uint64_t wd = smem_desc_kmajor(base + a_bytes + ((p.prod_w >> (4 * j)) & 15u) * kWTile);
+#pragma unroll
+                    for (int k = 0; k < BK / UK; ++k) {
+                        umma_bf16(tmem_base, ad + (uint64_t)(2 * k), wd + (uint64_t)(2 * k), idesc, accumulate);
+                        accumulate = 1;
+                    }
+                }
+                umma_commit(smem_u32(&bars.empty[stage]));
+                if (++stage == p.stages) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
+            }
+            if (ok) umma_commit(smem_u32(&bars.done));
+        }
+    } else {
+        if (kSplitA) {
+            const int te = threadIdx.x - 64;
+            // A: 128 rows x 8 chunks of 8 values per k-block, two chunks per thread; 8 threads read a row's 256
+            // bytes, the next k-block's values are on their way while this one is split and stored
+            const int c8 = te & 7, r0 = te >> 3;
+            constexpr int kC = 1024 / (32 * kSmEpiWarps), kStep = 4 * kSmEpiWarps;   // chunks per thread, rows between them
+            float4 va[kC], vb[kC];
+            auto fetch = [&](int kb) {
+#pragma unroll
+                for (int i = 0; i < kC; ++i) {
+                    const int m = m0 + r0 + kStep * i;
+                    va[i] = vb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (m < p.M) {
+                        const float4* src = reinterpret_cast<const float4*>(p.a_f32 + (size_t)m * p.K + kb * BK + 8 * c8);
+                        va[i] = src[0];
+                        vb[i] = src[1];
+                    }
+                }
+            };
+            if (kb0 < kb1) fetch(kb0);
+            int stage = 0;
+            uint32_t phase = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
+                uint8_t* dst = tiles + (size_t)stage * p.stage_bytes;
+#pragma unroll
+                for (int i = 0; i < kC; ++i) {
+                    const int r = r0 + kStep * i;
+                    uint4 hi, mid, lo;
+                    split8(va[i], vb[i], hi, mid, lo);
+                    uint8_t* q = dst + r * 128 + ((c8 ^ (r & 7)) << 4);   // the 128-byte swizzle of a K-major tile
+                    *reinterpret_cast<uint4*>(q) = hi;
+                    *reinterpret_cast<uint4*>(q + kSmATile) = mid;
+                    *reinterpret_cast<uint4*>(q + 2 * kSmATile) = lo;
+                }
+                if (kb + 1 < kb1) fetch(kb + 1);
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bars.full[stage]));
+                if (++stage == p.stages) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
+            }
+        }
+    }
+
+    // Epilogue: CTA `rank` finishes rows [rank, rank + 1) * 128 / cluster of the tile; a thread keeps its 4 columns and
+    // takes every kRowGroups-th row, kU rows at a time.
+    constexpr int kC4 = kBN / 4, kRowGroups = 32 * kSmEpiWarps / kC4, kU = kBN == 256 && !kBf16 ? 4 : 8;
+    const int te = (int)threadIdx.x - 64, c4 = te % kC4, rg = te / kC4;
+    const int rows = BM / p.cluster, row_base = rank * rows;
+    const int n = n0 + 4 * c4;
+    Raw4<kBf16> sk[kU], dt[kU];
+    // the epilogue's operands come from far: the first rows are asked for while the MMAs run
+    auto fetch_operands = [&](int r0) {
+#pragma unroll
+        for (int i = 0; i < kU; ++i) {
+            const int r = r0 + i * kRowGroups, m = m0 + row_base + r;
+            if (kEpi != kSmStore && r < rows && m < p.M && n < p.N) {
+                const size_t e = (size_t)m * p.N + n;
+                sk[i].load(p.skip, p.skip_bf16, e);
+                if (kEpi == kSmDiag && p.dot) dt[i].load(p.dot, p.dot_bf16, e);
+            }
+        }
+    };
+    if (warp >= 2) {
+        fetch_operands(rg);
+        if (mbar_wait(smem_u32(&bars.done), 0, abort_flag)) {
+            // this CTA's part of the tile -> shared memory (every operand stage has been read: the MMAs are done)
+            tc_fence_after();
+            const int q = warp & 3, grp = (warp - 2) >> 2;   // TMEM lane quarter; every fourth slab of 32 columns
+            float* row = reinterpret_cast<float*>(tiles) + (size_t)(q * 32 + lane) * kPitch;
+            const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
+#pragma unroll 1
+            for (int c = grp * 32; c < kBN; c += 32 * (kSmEpiWarps / 4)) {
+                uint32_t r[32];
+                tmem_ld32(t_row + (uint32_t)c, r);
+                tmem_ld_wait();
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    *reinterpret_cast<float4*>(row + c + 4 * j) =
+                        make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]), __uint_as_float(r[4 * j + 2]),
+                                    __uint_as_float(r[4 * j + 3]));
+            }
+            tc_fence_before();
+        }
+    }
+    __syncwarp();
+    if (p.cluster > 1) cluster_sync_all();   // the parts of all CTAs of the cluster are in place
+    else __syncthreads();
+    if (warp >= 2 && !*abort_flag) {
+        const bool n_ok = n < p.N;
+        float4 dg = make_float4(0.f, 0.f, 0.f, 0.f), dsum = dg;
+        if (kEpi == kSmDiag && n_ok) dg = *reinterpret_cast<const float4*>(p.diag + n);
+        for (int r0 = rg; r0 < rows; r0 += kU * kRowGroups) {
+            if (r0 != rg) fetch_operands(r0);
+#pragma unroll
+            for (int i0 = 0; i0 < kU; i0 += 4) {
+                const int r1 = r0 + i0 * kRowGroups;
+                if (r1 >= rows) break;
+                const float* own = reinterpret_cast<const float*>(tiles) + (size_t)(row_base + r1) * kPitch + 4 * c4;
+                float4 v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = r1 + i * kRowGroups, m = m0 + row_base + r;
+                    v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (kEpi == kSmDiag && p.add && r < rows && m < p.M && n_ok)
+                        v[i] = *reinterpret_cast<const float4*>(p.add + (size_t)m * p.N + n);
+                }
+                for (int q = 0; q < p.cluster; ++q) {
+                    const uint32_t a = map_to_cta(smem_u32(own), (uint32_t)q);
+                    float4 t[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (r1 + i * kRowGroups < rows)
+                            t[i] = p.cluster == 1 ? *reinterpret_cast<const float4*>(own + (size_t)i * kRowGroups * kPitch)
+                                                  : ld_cluster_f4(a + (uint32_t)i * (kRowGroups * kPitch * 4u));
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (r1 + i * kRowGroups < rows) v[i].x += t[i].x, v[i].y += t[i].y, v[i].z += t[i].z, v[i].w += t[i].w;
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = r1 + i * kRowGroups, m = m0 + row_base + r;
+                    if (r >= rows || m >= p.M || !n_ok) continue;
+                    const size_t e = (size_t)m * p.N + n;
+                    if (kEpi == kSmStore) {
+                        *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + e) = v[i];
+                    } else if (kEpi == kSmDiag) {
+                        const float4 s4 = sk[i0 + i].get(p.skip_bf16);
+                        v[i].x = fmaf(dg.x, s4.x, v[i].x);
+                        v[i].y = fmaf(dg.y, s4.y, v[i].y);
+                        v[i].z = fmaf(dg.z, s4.z, v[i].z);
+                        v[i].w = fmaf(dg.w, s4.w, v[i].w);
+                        store4_io(p.out, p.out_bf16, e, v[i]);
+                        if (p.dot) {
+                            const float4 d4 = dt[i0 + i].get(p.dot_bf16);
+                            dsum.x = fmaf(s4.x, d4.x, dsum.x);
+                            dsum.y = fmaf(s4.y, d4.y, dsum.y);
+                            dsum.z = fmaf(s4.z, d4.z, dsum.z);
+                            dsum.w = fmaf(s4.w, d4.w, dsum.w);
+                        }
+                    } else {
+                        const float4 s4 = sk[i0 + i].get(true);
+                        *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + e) = v[i];
+                        *reinterpret_cast<uint2*>(p.gate_out + e) =
+                            pack4_bf16(make_float4(s4.x / (1.f + __expf(-v[i].x)), s4.y / (1.f + __expf(-v[i].y)),
+                                                   s4.z / (1.f + __expf(-v[i].z)), s4.w / (1.f + __expf(-v[i].w))));
+                    }
+                }
+            }
+        }
+        if (kEpi == kSmDiag && p.dot) {
+            // column sums over this CTA's rows: the row groups added in a fixed order, one row of dot_part per CTA
+            __shared__ float4 red[32 * kSmEpiWarps];
+            red[te] = dsum;
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kSmEpiWarps) : "memory");
+            if (rg == 0 && n_ok) {
+                float4 t = red[c4];
+#pragma unroll
+                for (int g = 1; g < kRowGroups; ++g) {
+                    const float4 u = red[g * kC4 + c4];
+                    t.x += u.x, t.y += u.y, t.z += u.z, t.w += u.w;
+                }
+                *reinterpret_cast<float4*>(p.dot_part + (size_t)((tile / p.n_tiles) * p.cluster + rank) * p.N + n) = t;
+            }
+        }
+    }
+    // nobody leaves (or frees tensor memory) while another CTA may still read its part
+    tc_fence_before();
+    __syncwarp();
+    if (p.cluster > 1) cluster_sync_all();
+    else __syncthreads();
+    tc_fence_after();
+    if (warp == 1) tmem_dealloc(tmem_base, kBN);
+    if (threadIdx.x == 0 && *abort_flag && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
+}
+
+// ---------------------------------------------------------------------------------------------
+// Host side
+// ---------------------------------------------------------------------------------------------
+namespace {
+
+struct SmallShape {
+    int bn, cluster, stages;
+};
+
+size_t stage_bytes_of(int bn, int planes_a, int planes_w) { return (size_t)planes_a * kSmATile + (size_t)planes_w * bn * BK * 2; }
+
+// Tile width and cluster size: the pair with the shortest estimated time.  The estimate is a fit, in microseconds, to
+// timings of all pairs on twenty shapes from 16 x 256 x 256 to 4096 x 1024 x 1024, back to back (within 10 % of the
+// measured time, and the pair it picks within 8 % of the fastest): a wave of CTAs takes a fixed part that grows with
+// the tile (start, first loads, epilogue), its k-blocks at 48 bytes of operands per cycle and SM (L2), 0.95 us where
+// fp32 operands are split on the way, and the exchange between the CTAs of a cluster.
+SmallShape pick_small(int M, int N, int k_blocks, int planes_a, int planes_w, bool split_a, bool w_stacked) {
+    SmallShape best{0, 0, 0};
+    double best_t = 0.0;
+    const int m_tiles = (M + BM - 1) / BM, sms = device_sm_count();
+    for (int bn = 64; bn <= (w_stacked ? 128 : 256); bn *= 2) {
+        const size_t sb = stage_bytes_of(bn, planes_a, planes_w);
+        const int stages = std::min<int>(kSmMaxStages, (int)((kSmSmemMax - 1024) / sb));
+        if (stages < 2) continue;
+        const int tiles = m_tiles * ((N + bn - 1) / bn);
+        for (int c = 1; c <= 4 && c <= k_blocks; c *= 2) {
+            const int slots = c == 1 ? sms : (c == 2 ? sms - 4 : sms - 16);   // clusters must fit a GPC
+            const int waves = (tiles * c + slots - 1) / slots;
+            const double per_kb = std::max((double)sb / 91000.0, split_a ? 0.95 : 0.0);
+            const double exchange = c == 1 ? 0.0 : bn * c / 256.0;
+            const double t = waves * (4.6 + bn * 0.0115 + exchange + ((k_blocks + c - 1) / c) * per_kb);
+            if (best.bn == 0 || t < best_t) {
+                best_t = t;
+                best = {bn, c, stages};
+            }
+        }
+    }
+    return best;
+}
+
+template <int kBN, int kEpi, bool kSplitA, bool kBf16>
+int launch_small(const CUtensorMap& ma, const CUtensorMap& mw, const SmallTnArgs& p, int grid, size_t smem, cudaStream_t st) {
+    auto kern = gemm_tc_tn_small_kernel<kBN, kEpi, kSplitA, kBf16>;
+    if (!set_max_dynamic_smem(reinterpret_cast<const void*>(kern), kSmSmemMax)) return SSM_ERR_CUDA;
+    count_launch();
+    return launch_dep_cluster(kern, (unsigned)p.cluster, grid, sm_threads(kBN), smem, st, ma, mw, p) ? SSM_OK : SSM_ERR_CUDA;
+}
+
+}  // namespace
+}  // namespace tc
+
+int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st) {
+    using namespace tc;
+    const int epi = g.gate_out ? kSmGate : (g.store_f32 && !g.diag ? kSmStore : kSmDiag);
+    if (g.K % BK != 0 || g.N_out % 64 != 0 || g.n_products > 8) return SSM_ERR_SHAPE;
+    if (epi == kSmDiag && (!g.diag || !g.skip)) return SSM_ERR_SHAPE;
+    if (epi == kSmGate && (!g.skip || !g.skip_bf16)) return SSM_ERR_SHAPE;
+    SmallTnArgs p{};
+    p.M = g.M;
+    p.N = g.N_out;
+    p.K = g.K;
+    p.k_blocks = g.K / BK;
+    if (g.split_w) {          // hi / lo blocks of 128 weight rows; lo product first
+        p.planes_a = 1, p.planes_w = 2, p.n_prod = 2;
+        p.prod_a = 0x00u, p.prod_w = 0x01u;
+        p.w_plane_rows = 128, p.w_stacked = 1;
+    } else if (g.n_products > 0) {
+        p.planes_a = g.planes_a, p.planes_w = g.planes_w, p.n_prod = g.n_products;
+        p.prod_a = g.prod_a, p.prod_w = g.prod_w;
+        p.w_plane_cols = g.w_plane_rows ? 0 : g.K;
+        p.w_plane_rows = g.w_plane_rows;
+        p.w_stacked = g.w_plane_rows ? 1 : 0;
+    } else {
+        p.planes_a = p.planes_w = p.n_prod = 1;
+    }
+    p.a_plane = g.K;
+    p.a_f32 = g.a_f32 ? reinterpret_cast<const float*>(g.A) : nullptr;
+    if (g.a_f32 && p.planes_a != 3) return SSM_ERR_SHAPE;
+    p.out = g.out, p.diag = g.diag, p.skip = g.skip, p.dot = g.dot, p.add = g.add;
+    p.dot_part = g.dot_part, p.gate_out = reinterpret_cast<__nv_bfloat16*>(g.gate_out);
+    p.out_bf16 = !g.store_f32, p.skip_bf16 = g.skip_bf16, p.dot_bf16 = g.dot_bf16;
+    p.hdr = g.hdr;
+    const SmallShape s = pick_small(g.M, g.N_out, p.k_blocks, p.planes_a, p.planes_w, g.a_f32, p.w_stacked != 0);
+    if (s.bn == 0) return SSM_ERR_SHAPE;
+    p.cluster = s.cluster;
+    p.stages = s.stages;
+    p.stage_bytes = (int)stage_bytes_of(s.bn, p.planes_a, p.planes_w);
+    p.n_tiles = (g.N_out + s.bn - 1) / s.bn;
+    const size_t smem = std::max((size_t)p.stages * p.stage_bytes, (size_t)BM * (s.bn + 4) * 4) + 1024;
+    const int m_tiles = (g.M + BM - 1) / BM, grid = m_tiles * p.n_tiles * p.cluster;
+    if (g.dot_rows) *g.dot_rows = m_tiles * p.cluster;
+    CUtensorMap ma, mw;
+    const uint64_t w_rows = (uint64_t)g.N_out * (p.w_stacked ? p.planes_w : 1);
+    const uint64_t w_cols = (uint64_t)g.K * (p.w_stacked ? 1 : p.planes_w);
+    if (!make_map(&mw, g.W, w_rows, w_cols, BK, (uint32_t)s.bn, false, CU_TENSOR_MAP_SWIZZLE_128B, (uint64_t)g.w_pitch))
+        return SSM_ERR_CUDA;
+    ma = mw;   // unused when A is split here
+    if (!g.a_f32 && !make_map(&ma, g.A, (uint64_t)g.M, (uint64_t)g.K * p.planes_a, BK, BM)) return SSM_ERR_CUDA;
+    const bool io_bf16 = g.skip_bf16 && (!g.dot || g.dot_bf16);
+#define SSM_SMALL(EPI, SPLIT, BF)                                                             \
+    do {                                                                                      \
+        if (s.bn == 64) return launch_small<64, EPI, SPLIT, BF>(ma, mw, p, grid, smem, st);   \
+        if (s.bn == 128) return launch_small<128, EPI, SPLIT, BF>(ma, mw, p, grid, smem, st); \
+        return launch_small<256, EPI, SPLIT, BF>(ma, mw, p, grid, smem, st);                  \
+    } while (0)
+    if (epi == kSmGate) SSM_SMALL(kSmGate, false, true);
+    if (epi == kSmStore && g.a_f32) SSM_SMALL(kSmStore, true, true);
+    if (epi == kSmStore) SSM_SMALL(kSmStore, false, true);
+    if (g.a_f32) SSM_SMALL(kSmDiag, true, false);
+    if (io_bf16) SSM_SMALL(kSmDiag, false, true);
+    SSM_SMALL(kSmDiag, false, false);
+#undef SSM_SMALL
+}
+
+// One partial row of column sums per CTA along M.
+int tc_tn_small_max_dot_rows(int M) { return 4 * ((M + tc::BM - 1) / tc::BM); }
+
+}  // namespace ssm

@@ -114,8 +114,8 @@ struct GemmTcTN {
     void* out;
     const float* diag; const void* skip;   // bf16 result: out = acc + diag[n] * skip[m, n]
     WsHeader* hdr;
-    // Gate (with store_f32, split_w and skip): besides the fp32 result also gate_out[m, n] =
-    // bf16(skip[m, n] * sigmoid(acc)).  Only where tc_tn_gate_supported says so.
+    // Gate (with store_f32 and skip; split_w or a product schedule): besides the fp32 result also gate_out[m, n] =
+    // bf16(skip[m, n] * sigmoid(acc)).
     void* gate_out = nullptr;
     // Column sums (with the bf16 epilogue, where tc_tn_dot_supported says so): dot_part[c, n] = sum over the
     // rows m that CTA c drained of skip[m, n] * dot[m, n]; *dot_rows receives the number of rows c written
@@ -128,12 +128,21 @@ struct GemmTcTN {
     // product j multiplies plane (prod_a >> 4 j) & 15 of A by plane (prod_w >> 4 j) & 15 of W.  fp32 result only.
     int n_products = 0, planes_a = 1, planes_w = 1;
     uint32_t prod_a = 0, prod_w = 0;
+    // Only where tc_tn_small says so (the kernel for problems of few tiles):
+    bool a_f32 = false;                  // A is fp32 [M, K]; its three planes are made on the way to the tensor cores
+    bool skip_bf16 = true, dot_bf16 = true;   // types of skip and dot; with diag and store_f32 the result is fp32
+    const float* add = nullptr;          // fp32 [M, N_out], added to acc + diag * skip
+    int w_plane_rows = 0;                // planes of W this many rows apart in blocks of 128 rows (as with split_w) ...
+    int w_pitch = 0;                     // ... and its row pitch in elements, if it is not K
 };
 bool tc_tn_supported(int M, int N_out, int K, bool split_w);
+// Whether a projection has too few 256 x 256 tiles for the kernels on CTA pairs and takes the one of gemm_tc_small.cu.
+bool tc_tn_small(int M, int N_out, bool split_w);
+int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st);
+int tc_tn_small_max_dot_rows(int M);
 int tc_max_n();   // widest output of the tensor-core projections
 bool tc_tn_dot_supported(int M, int N_out, int K);
-int tc_tn_dot_max_rows();
-bool tc_tn_gate_supported(int M, int N_out, int K);
+int tc_tn_dot_max_rows(int M, int N_out);
 int launch_gemm_tc_tn(const GemmTcTN& g, cudaStream_t st);
 
 // Input projection and forward scan fused (gemm_tc.cu): x = scan(u Bbar^T) written as the two bf16

@@ -1,0 +1,27 @@
+"""Projections of few tiles (csrc/gemm_tc_small.cu) at the edges of their tiles: one row, one row more or less than a
+128-row tile, output widths that leave the last 64-, 128- or 256-column tile partly empty, a contraction of one or
+two k-blocks (clusters of at most as many CTAs), and the widest outputs."""
+import pytest
+
+from paper_2502_20168_b200 import inputs as I
+from tests.test_gpu_half_glu import _run as run_gate
+from tests.test_gpu_layer_parity import run
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,T,H,P", [(1, 1, 128, 64), (127, 1, 128, 64), (1, 129, 640, 64), (9, 57, 384, 320),
+                                     (3, 43, 1152, 128), (60, 65, 384, 64), (31, 125, 768, 256)])
+def test_bf16_edges(B, T, H, P):
+    run(I.Workload("few", B=B, T=T, H=H, P=P, io_dtype="bf16", p_done=0.02, seed=B + H), with_x0=True, with_gxT=True)
+
+
+@pytest.mark.parametrize("B,T,H,P", [(1, 1, 256, 128), (1, 127, 256, 128), (43, 3, 512, 128), (5, 205, 256, 384),
+                                     (2, 64, 1024, 256), (37, 111, 256, 128)])
+def test_fp32_edges(B, T, H, P):
+    run(I.Workload("few32", B=B, T=T, H=H, P=P, io_dtype="f32", p_done=0.02, seed=B + H), with_x0=True, with_gxT=True)
+
+
+@pytest.mark.parametrize("rows,H", [(1, 128), (129, 256), (1000, 384)])
+def test_gate_edges_bf16(rows, H):
+    run_gate(I.Workload("few_gate", B=1, T=rows, H=H, P=8, io_dtype="bf16", seed=rows + H))
