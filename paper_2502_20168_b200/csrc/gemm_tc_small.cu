@@ -142,7 +142,11 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncwarp();
-    if (warp == 1) tmem_alloc(smem_u32(&bars.tmem), kBN);
+    // Several products: the last one (hi hi) has an accumulator of its own, the small ones share a second, and the two
+    // are added once.  (In one accumulator every small term would be rounded at the magnitude of the sum: measured 2 - 3 x
+    // the error on the gradients of small fp32 layers.)
+    const uint32_t tmem_cols = p.n_prod > 1 ? 2 * kBN : kBN;
+    if (warp == 1) tmem_alloc(smem_u32(&bars.tmem), tmem_cols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -179,19 +183,21 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         if (lane == 0) {
             constexpr uint32_t idesc = instr_desc(BM, kBN, 0, 0);
             int stage = 0;
-            uint32_t phase = 0, accumulate = 0;
+            uint32_t phase = 0;
             bool ok = true;
             for (int kb = kb0; kb < kb1; ++kb) {
                 if (!(ok = mbar_wait(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
                 tc_fence_after();
                 const uint32_t base = smem_u32(tiles) + (uint32_t)stage * (uint32_t)p.stage_bytes;
                 for (int j = 0; j < p.n_prod; ++j) {
+                    const bool small = j < p.n_prod - 1;
+                    const uint32_t d_tmem = tmem_base + (small ? (uint32_t)kBN : 0u);
+                    const bool first = kb == kb0 && (j == 0 || !small);
                     const uint64_t ad = smem_desc_kmajor(base + ((p.prod_a >> (4 * j)) & 15u) * kSmATile);
                     const uint64_t wd = smem_desc_kmajor(base + a_bytes + ((p.prod_w >> (4 * j)) & 15u) * kWTile);
 #pragma unroll
                     for (int k = 0; k < BK / UK; ++k) {
-                        umma_bf16(tmem_base, ad + (uint64_t)(2 * k), wd + (uint64_t)(2 * k), idesc, accumulate);
-                        accumulate = 1;
+                        umma_bf16(d_tmem, ad + (uint64_t)(2 * k), wd + (uint64_t)(2 * k), idesc, (uint32_t)!(first && k == 0));
                     }
                 }
                 umma_commit(smem_u32(&bars.empty[stage]));
@@ -281,7 +287,15 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             for (int c = grp * 32; c < kBN; c += 32 * (kSmEpiWarps / 4)) {
                 uint32_t r[32];
                 tmem_ld32(t_row + (uint32_t)c, r);
-                tmem_ld_wait();
+                if (p.n_prod > 1) {
+                    uint32_t r2[32];
+                    tmem_ld32(t_row + (uint32_t)(kBN + c), r2);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
+                } else {
+                    tmem_ld_wait();
+                }
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
                     *reinterpret_cast<float4*>(row + c + 4 * j) =
@@ -378,7 +392,7 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     if (p.cluster > 1) cluster_sync_all();
     else __syncthreads();
     tc_fence_after();
-    if (warp == 1) tmem_dealloc(tmem_base, kBN);
+    if (warp == 1) tmem_dealloc(tmem_base, tmem_cols);
     if (threadIdx.x == 0 && *abort_flag && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
 }
 
