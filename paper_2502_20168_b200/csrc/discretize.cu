@@ -32,8 +32,10 @@ __device__ __forceinline__ ZohTerms zoh_terms(float2 lam, float dt) {
 }
 
 // One block per state p: Abar[p], Bbar[p, :] = gamma_p * B[p, :].
-__global__ void discretize_kernel(int H, const float2* __restrict__ Lambda, const float* __restrict__ Delta,
-                                  const float2* __restrict__ Bc, float2* __restrict__ Abar, float2* __restrict__ Bbar) {
+__global__ void discretize_kernel(int H, const float2* Lambda, const float* Delta,
+                                  const float2* Bc, float2* Abar, float2* Bbar) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ float2 gamma_s;
     const int p = blockIdx.x;
     if (threadIdx.x == 0) {
@@ -64,10 +66,12 @@ __device__ __forceinline__ void zoh_adjoint(const ZohTerms& z, float2 lam, float
 }
 
 // ssm_discretize_bwd: one block per state p.
-__global__ void discretize_bwd_kernel(int H, int P, const float2* __restrict__ Lambda, const float* __restrict__ Delta,
-                                      const float2* __restrict__ Bc, const float2* __restrict__ gAbar,
-                                      const float2* __restrict__ gBbar, float2* __restrict__ dLambda,
-                                      float* __restrict__ dDelta, float2* __restrict__ dB) {
+__global__ void discretize_bwd_kernel(int H, int P, const float2* Lambda, const float* Delta,
+                                      const float2* Bc, const float2* gAbar,
+                                      const float2* gBbar, float2* dLambda,
+                                      float* dDelta, float2* dB) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ float2 gamma_s;
     __shared__ float red[2][32];
     const int p = blockIdx.x;
@@ -203,8 +207,10 @@ __device__ __forceinline__ void store_col_pair(void* W, int P, int p, int h, flo
 
 template <int kMode>
 __global__ void __launch_bounds__(256)
-pack_params_kernel(int H, int P, const float2* __restrict__ Lambda, const float* __restrict__ Delta,
-                   const float2* __restrict__ Bc, const float2* __restrict__ Cc, PackOut o) {
+pack_params_kernel(int H, int P, const float2* Lambda, const float* Delta,
+                   const float2* Bc, const float2* Cc, PackOut o) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ float2 gamma_s[32];
     __shared__ float2 tB[32][33], tC[32][33];   // tB[state][h], tC[h][state]
     const int p0 = blockIdx.x * 32, h0 = blockIdx.y * 32;
@@ -266,10 +272,12 @@ pack_params_kernel(int H, int P, const float2* __restrict__ Lambda, const float*
 // element, else 8 (1024 x 1024 with 2 partials: 8.2 against 10.5 us; 512 x 512 with 9: 7.2 with 16 against 8.5).
 template <int kReduceWarps>
 __global__ void __launch_bounds__(32 * kReduceWarps + 32)
-reduce_weight_grads_kernel(int H, int P, int splits, const float* __restrict__ part_b, const float* __restrict__ part_c,
-                           const float2* __restrict__ Lambda, const float* __restrict__ Delta,
-                           const float2* __restrict__ Bc, float2* __restrict__ dB, float2* __restrict__ dC,
-                           float2* __restrict__ gg_part) {
+reduce_weight_grads_kernel(int H, int P, int splits, const float* part_b, const float* part_c,
+                           const float2* Lambda, const float* Delta,
+                           const float2* Bc, float2* dB, float2* dC,
+                           float2* gg_part) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ float2 gamma_s[32];
     __shared__ float2 t[32][33];   // [feature][state]
     constexpr int kRows = 32 / kReduceWarps;
@@ -295,7 +303,7 @@ reduce_weight_grads_kernel(int H, int P, int splits, const float* __restrict__ p
         for (int s = 0; s < splits; ++s, src += n) {
 #pragma unroll
             for (int i = 0; i < kRows; ++i)
-                if (h0 + w + kReduceWarps * i < H) acc[i] = cadd(acc[i], __ldcs(src + (size_t)kReduceWarps * i * P));
+                if (h0 + w + kReduceWarps * i < H) acc[i] = cadd(acc[i], ld_stream(src + (size_t)kReduceWarps * i * P));
         }
     }
 #pragma unroll
@@ -330,10 +338,12 @@ reduce_weight_grads_kernel(int H, int P, int splits, const float* __restrict__ p
 // (the rows of partial sums are up to 512, the columns a few hundred: latency is all there is), one warp evaluates
 // the P-sized double-precision terms meanwhile.  H = 512, P = 256: 6.2 - 9.5 -> 3.0 - 6.3 us (4 - 512 rows) against one block per state.
 __global__ void __launch_bounds__(1024)
-layer_finalize_kernel(int H, int P, const float2* __restrict__ Lambda, const float* __restrict__ Delta,
-                      const float2* __restrict__ gA_part, int gA_rows, const float2* __restrict__ gg_part, int gg_rows,
-                      float2* __restrict__ dLambda, float* __restrict__ dDelta, const float* __restrict__ dD_part,
-                      int dD_rows, float* __restrict__ dD) {
+layer_finalize_kernel(int H, int P, const float2* Lambda, const float* Delta,
+                      const float2* gA_part, int gA_rows, const float2* gg_part, int gg_rows,
+                      float2* dLambda, float* dDelta, const float* dD_part,
+                      int dD_rows, float* dD) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ double sA[2][32][33], sG[2][32][33];
     __shared__ ZohTerms zs[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -395,7 +405,7 @@ template <int kMode>
 static void launch_pack(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc, const float2* Cc,
                         const PackOut& o, cudaStream_t st) {
     count_launch();
-    pack_params_kernel<kMode><<<weight_tiles(H, P, 1), 256, 0, st>>>(H, P, Lambda, Delta, Bc, Cc, o);
+    launch_dep(pack_params_kernel<kMode>, weight_tiles(H, P, 1), 256, 0, st, H, P, Lambda, Delta, Bc, Cc, o);
 }
 
 void launch_discretize_pack_tc(int H, int P, int group, const float2* Lambda, const float* Delta, const float2* Bc,
@@ -420,14 +430,14 @@ void launch_discretize_pack_f32(int H, int P, const float2* Lambda, const float*
 void launch_discretize(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc, float2* Abar,
                        float2* Bbar, cudaStream_t st) {
     count_launch();
-    discretize_kernel<<<P, 128, 0, st>>>(H, Lambda, Delta, Bc, Abar, Bbar);
+    launch_dep(discretize_kernel, P, 128, 0, st, H, Lambda, Delta, Bc, Abar, Bbar);
 }
 
 void launch_discretize_bwd(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
                            const float2* gAbar, const float2* gBbar, float2* dLambda, float* dDelta, float2* dB,
                            cudaStream_t st) {
     count_launch();
-    discretize_bwd_kernel<<<P, 128, 0, st>>>(H, P, Lambda, Delta, Bc, gAbar, gBbar, dLambda, dDelta, dB);
+    launch_dep(discretize_bwd_kernel, P, 128, 0, st, H, P, Lambda, Delta, Bc, gAbar, gBbar, dLambda, dDelta, dB);
 }
 
 int gamma_part_rows(int H) { return (H + 31) / 32; }
@@ -438,16 +448,16 @@ void launch_reduce_weight_grads(int H, int P, int splits, const float* part_b, c
     count_launch();
     const dim3 grid = weight_tiles(H, P, 2);
     if (splits > 4)
-        reduce_weight_grads_kernel<16><<<grid, 32 * 17, 0, st>>>(H, P, splits, part_b, part_c, Lambda, Delta, Bc, dB, dC, gg_part);
+        launch_dep(reduce_weight_grads_kernel<16>, grid, 32 * 17, 0, st, H, P, splits, part_b, part_c, Lambda, Delta, Bc, dB, dC, gg_part);
     else
-        reduce_weight_grads_kernel<8><<<grid, 32 * 9, 0, st>>>(H, P, splits, part_b, part_c, Lambda, Delta, Bc, dB, dC, gg_part);
+        launch_dep(reduce_weight_grads_kernel<8>, grid, 32 * 9, 0, st, H, P, splits, part_b, part_c, Lambda, Delta, Bc, dB, dC, gg_part);
 }
 
 void launch_layer_finalize(int H, int P, const float2* Lambda, const float* Delta, const float2* gA_part, int gA_rows,
                            const float2* gg_part, float2* dLambda, float* dDelta, const float* dD_part, int dD_rows,
                            float* dD, cudaStream_t st) {
     count_launch();
-    layer_finalize_kernel<<<(P + 31) / 32 + (H + 31) / 32, 1024, 0, st>>>(H, P, Lambda, Delta, gA_part, gA_rows, gg_part,
+    launch_dep(layer_finalize_kernel, (P + 31) / 32 + (H + 31) / 32, 1024, 0, st, H, P, Lambda, Delta, gA_part, gA_rows, gg_part,
                                                                          gamma_part_rows(H), dLambda, dDelta, dD_part,
                                                                          dD_rows, dD);
 }

@@ -35,8 +35,10 @@ struct EpiArgs {
 // TO: type of out; TS: type of the skip operand; the addend, where there is one, is fp32.
 template <typename TA, typename TB, typename TO, typename TS, bool kAddDiag>
 __global__ void __launch_bounds__(kGemmThreads)
-gemm_tn_kernel(const TA* __restrict__ A, int lda, const TB* __restrict__ Bm, int ldb, int M, int N, int K,
+gemm_tn_kernel(const TA* A, int lda, const TB* Bm, int ldb, int M, int N, int K,
                EpiArgs e) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ __align__(16) float As[TK][TM + 4];
     __shared__ __align__(16) float Bs[TK][TN + 4];
     const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;   // rows along x: grid.y is limited to 65535
@@ -96,15 +98,15 @@ static void dispatch_tn(const GemmTN& g, cudaStream_t st) {
     const TB* Bm = (const TB*)g.Bm;
     using bf = __nv_bfloat16;
     if (g.epi == Epi::StoreF32)
-        gemm_tn_kernel<TA, TB, float, float, false><<<grid, kGemmThreads, 0, st>>>(A, g.lda, Bm, g.ldb, g.M, g.N, g.K, e);
+        launch_dep(gemm_tn_kernel<TA, TB, float, float, false>, grid, kGemmThreads, 0, st, A, g.lda, Bm, g.ldb, g.M, g.N, g.K, e);
     else if (g.out_bf16 && g.skip_bf16)
-        gemm_tn_kernel<TA, TB, bf, bf, true><<<grid, kGemmThreads, 0, st>>>(A, g.lda, Bm, g.ldb, g.M, g.N, g.K, e);
+        launch_dep(gemm_tn_kernel<TA, TB, bf, bf, true>, grid, kGemmThreads, 0, st, A, g.lda, Bm, g.ldb, g.M, g.N, g.K, e);
     else if (g.out_bf16)
-        gemm_tn_kernel<TA, TB, bf, float, true><<<grid, kGemmThreads, 0, st>>>(A, g.lda, Bm, g.ldb, g.M, g.N, g.K, e);
+        launch_dep(gemm_tn_kernel<TA, TB, bf, float, true>, grid, kGemmThreads, 0, st, A, g.lda, Bm, g.ldb, g.M, g.N, g.K, e);
     else if (g.skip_bf16)
-        gemm_tn_kernel<TA, TB, float, bf, true><<<grid, kGemmThreads, 0, st>>>(A, g.lda, Bm, g.ldb, g.M, g.N, g.K, e);
+        launch_dep(gemm_tn_kernel<TA, TB, float, bf, true>, grid, kGemmThreads, 0, st, A, g.lda, Bm, g.ldb, g.M, g.N, g.K, e);
     else
-        gemm_tn_kernel<TA, TB, float, float, true><<<grid, kGemmThreads, 0, st>>>(A, g.lda, Bm, g.ldb, g.M, g.N, g.K, e);
+        launch_dep(gemm_tn_kernel<TA, TB, float, float, true>, grid, kGemmThreads, 0, st, A, g.lda, Bm, g.ldb, g.M, g.N, g.K, e);
 }
 
 void launch_gemm_tn(const GemmTN& g, cudaStream_t st) {
@@ -117,8 +119,10 @@ void launch_gemm_tn(const GemmTN& g, cudaStream_t st) {
 // part[s,i,j] = sum_{k in slice s} A[k,i] Bm[k,j]; both operands contiguous in i / j.
 template <typename TA, typename TB>
 __global__ void __launch_bounds__(kGemmThreads)
-gemm_nt_kernel(const TA* __restrict__ A, int I, const TB* __restrict__ Bm, int J, int K, int k_per_split,
-               float* __restrict__ part) {
+gemm_nt_kernel(const TA* A, int I, const TB* Bm, int J, int K, int k_per_split,
+               float* part) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ __align__(16) float As[TK][TM + 4];
     __shared__ __align__(16) float Bs[TK][TN + 4];
     const int i0 = blockIdx.y * TM, j0 = blockIdx.x * TN;
@@ -173,13 +177,13 @@ void launch_gemm_nt(const GemmNT& g, cudaStream_t st) {
     dim3 grid((g.J + TN - 1) / TN, (g.I + TM - 1) / TM, g.splits);
     count_launch();
     if (g.a_bf16 && g.b_bf16)
-        gemm_nt_kernel<__nv_bfloat16, __nv_bfloat16><<<grid, kGemmThreads, 0, st>>>((const __nv_bfloat16*)g.A, g.I, (const __nv_bfloat16*)g.Bm, g.J, g.K, kps, g.part);
+        launch_dep(gemm_nt_kernel<__nv_bfloat16, __nv_bfloat16>, grid, kGemmThreads, 0, st, (const __nv_bfloat16*)g.A, g.I, (const __nv_bfloat16*)g.Bm, g.J, g.K, kps, g.part);
     else if (g.a_bf16)
-        gemm_nt_kernel<__nv_bfloat16, float><<<grid, kGemmThreads, 0, st>>>((const __nv_bfloat16*)g.A, g.I, (const float*)g.Bm, g.J, g.K, kps, g.part);
+        launch_dep(gemm_nt_kernel<__nv_bfloat16, float>, grid, kGemmThreads, 0, st, (const __nv_bfloat16*)g.A, g.I, (const float*)g.Bm, g.J, g.K, kps, g.part);
     else if (g.b_bf16)
-        gemm_nt_kernel<float, __nv_bfloat16><<<grid, kGemmThreads, 0, st>>>((const float*)g.A, g.I, (const __nv_bfloat16*)g.Bm, g.J, g.K, kps, g.part);
+        launch_dep(gemm_nt_kernel<float, __nv_bfloat16>, grid, kGemmThreads, 0, st, (const float*)g.A, g.I, (const __nv_bfloat16*)g.Bm, g.J, g.K, kps, g.part);
     else
-        gemm_nt_kernel<float, float><<<grid, kGemmThreads, 0, st>>>((const float*)g.A, g.I, (const float*)g.Bm, g.J, g.K, kps, g.part);
+        launch_dep(gemm_nt_kernel<float, float>, grid, kGemmThreads, 0, st, (const float*)g.A, g.I, (const float*)g.Bm, g.J, g.K, kps, g.part);
 }
 
 }  // namespace ssm

@@ -418,10 +418,6 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                               tn_skip_bytes(kEpi));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
-    if (kEpi == 1 || kEpi == 3)   // (zero where the last tile reaches past the output's columns)
-        for (int i = threadIdx.x; i < p.n_tiles * BN; i += kTnThreads) s.diag[i] = i < p.ldo ? p.diag[i] : 0.f;
-    if (kEpi == 3)   // the epilogue warps' column sums start at zero
-        for (int i = threadIdx.x; i < kTnEpiWarps * (kDotMaxN / 2); i += kTnThreads) s.diag[kDotMaxN + i] = 0.f;
     // barriers and tensor memory (both CTAs), then the whole pair meets
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) {
@@ -443,6 +439,13 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = *s.tmem_slot_ptr;
+    grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
+    grid_dep_launch();
+    if (kEpi == 1 || kEpi == 3)   // (zero where the last tile reaches past the output's columns)
+        for (int i = threadIdx.x; i < p.n_tiles * BN; i += kTnThreads) s.diag[i] = i < p.ldo ? p.diag[i] : 0.f;
+    if (kEpi == 3)   // the epilogue warps' column sums start at zero
+        for (int i = threadIdx.x; i < kTnEpiWarps * (kDotMaxN / 2); i += kTnThreads) s.diag[kDotMaxN + i] = 0.f;
+    if (kEpi == 1 || kEpi == 3) __syncthreads();
 
     const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     const int m_pairs = (p.M + 2 * BM - 1) / (2 * BM);
@@ -700,6 +703,8 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = *s.tmem_slot_ptr;
+    grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
+    grid_dep_launch();
 
     const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     const int M = p.B * p.T;
@@ -1146,6 +1151,8 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = *s.tmem_slot_ptr;
+    grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
+    grid_dep_launch();
 
     const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     const int M = p.B * p.T;
@@ -1615,6 +1622,8 @@ gemm_tc_nt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     const Smem s = carve_smem(smem_raw, kStages, 0, 0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t tmem_base = prologue(s, warp, lane, 128);
+    grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
+    grid_dep_launch();
     const int tile = blockIdx.x, split = blockIdx.y;
     constexpr int kOutCols = kMulti ? BN : BN / 2;   // (not kMulti) accumulator columns [0,128): hi plane, [128,256): lo plane
     const int i0 = (tile / p.j_tiles) * BM, j0 = (tile % p.j_tiles) * kOutCols;
@@ -1763,6 +1772,8 @@ gemm_tc_nt_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = *s.tmem_slot_ptr;
+    grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
+    grid_dep_launch();
 
     const int tile = blockIdx.x >> 1, split = blockIdx.y;
     constexpr int kOutCols = BN / 2;
@@ -1977,7 +1988,7 @@ do {                                                                            
     ok = set_smem(kern, smem);                                                                         \
     const int pairs = ok ? resident_pairs(reinterpret_cast<const void*>(kern), smem) : 0;              \
     ok = ok && pairs > 0;                                                                              \
-    if (ok) kern<<<2 * min(pairs, pair_tiles), kTnThreads, smem, st>>>(ma, mw, mo, ms, mg, p);         \
+    if (ok) launch_dep(kern, 2 * min(pairs, pair_tiles), kTnThreads, smem, st, ma, mw, mo, ms, mg, p);         \
     if (ok && g.dot_rows) *g.dot_rows = 2 * min(pairs, pair_tiles);                                    \
 } while (0)
     if (epi == 3) SSM_LAUNCH_PAIR(3, false);
@@ -2074,7 +2085,7 @@ static int launch_gemm_scan_fwd_s(const GemmScanFwd& g, cudaStream_t st) {
     if (!set_smem(kern, Cfg::kSmemBytes)) return SSM_ERR_CUDA;
     const int pairs = resident_pairs(reinterpret_cast<const void*>(kern), Cfg::kSmemBytes, Cfg::kThreads);
     if (pairs <= 0) return SSM_ERR_CUDA;
-    kern<<<2 * min(pairs, p.nchains), Cfg::kThreads, Cfg::kSmemBytes, st>>>(ma, mw, mx, p);
+    launch_dep(kern, 2 * min(pairs, p.nchains), Cfg::kThreads, Cfg::kSmemBytes, st, ma, mw, mx, p);
     return SSM_OK;
 }
 
@@ -2113,7 +2124,7 @@ static int launch_gemm_scan_bwd_s(const GemmScanBwd& g, cudaStream_t st) {
     if (!set_smem(kern, Cfg::kSmemBytes)) return SSM_ERR_CUDA;
     const int pairs = resident_pairs(reinterpret_cast<const void*>(kern), Cfg::kSmemBytes, Cfg::kThreads);
     if (pairs <= 0) return SSM_ERR_CUDA;
-    kern<<<2 * min(pairs, p.nchains), Cfg::kThreads, Cfg::kSmemBytes, st>>>(ma, mw, mx, ms, p);
+    launch_dep(kern, 2 * min(pairs, p.nchains), Cfg::kThreads, Cfg::kSmemBytes, st, ma, mw, mx, ms, p);
     return SSM_OK;
 }
 
@@ -2153,7 +2164,7 @@ int launch_gemm_tc_nt(const GemmTcNT& g, cudaStream_t st) {
         dim3 grid((g.I / BM) * j_tiles, g.splits);
         count_launch();
         const bool ok = set_smem(gemm_tc_nt_kernel<true>, kNtSmemBytes);
-        gemm_tc_nt_kernel<true><<<grid, kThreads, kNtSmemBytes, st>>>(ma, mbh, mbh, p);
+        launch_dep(gemm_tc_nt_kernel<true>, grid, kThreads, kNtSmemBytes, st, ma, mbh, mbh, p);
         return ok ? SSM_OK : SSM_ERR_CUDA;
     }
     if (!make_map(&ma, g.A, (uint64_t)g.K, (uint64_t)g.I, 64, BK, false, CU_TENSOR_MAP_SWIZZLE_128B, (uint64_t)g.lda))
@@ -2166,13 +2177,13 @@ int launch_gemm_tc_nt(const GemmTcNT& g, cudaStream_t st) {
         dim3 grid(2 * (g.I / (2 * BM)) * j_tiles, g.splits);
         count_launch();
         const bool ok = set_smem(gemm_tc_nt_pair_kernel, kNtPairSmemBytes);
-        gemm_tc_nt_pair_kernel<<<grid, kThreads, kNtPairSmemBytes, st>>>(ma, mbh, mbl, p);
+        launch_dep(gemm_tc_nt_pair_kernel, grid, kThreads, kNtPairSmemBytes, st, ma, mbh, mbl, p);
         return ok ? SSM_OK : SSM_ERR_CUDA;
     }
     dim3 grid((g.I / BM) * j_tiles, g.splits);
     count_launch();
     const bool ok = set_smem(gemm_tc_nt_kernel<false>, kNtSmemBytes);
-    gemm_tc_nt_kernel<false><<<grid, kThreads, kNtSmemBytes, st>>>(ma, mbh, mbl, p);
+    launch_dep(gemm_tc_nt_kernel<false>, grid, kThreads, kNtSmemBytes, st, ma, mbh, mbl, p);
     return ok ? SSM_OK : SSM_ERR_CUDA;
 }
 

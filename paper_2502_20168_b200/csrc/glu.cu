@@ -26,8 +26,10 @@ inline int blocks_for(size_t n) {
 //        reduction index k < H -> W[k, j] (hi, lo rows), k >= H -> W[k - H, j] (hi rows only;
 //        the product of two low halves is dropped);  [2H rows, 2H columns].
 //   Wn:  for g_x1 = gz W^T: output column i, reduction index j;  [2H rows, H columns].
-__global__ void glu_pack_kernel(int H, const float* __restrict__ W, __nv_bfloat16* __restrict__ Wt2,
-                                __nv_bfloat16* __restrict__ Wn_split, float* __restrict__ Wt_f32) {
+__global__ void glu_pack_kernel(int H, const float* W, __nv_bfloat16* Wt2,
+                                __nv_bfloat16* Wn_split, float* Wt_f32) {
+    grid_dep_wait();
+    grid_dep_launch();
     const size_t n = (size_t)H * H;
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
         const int i = (int)(e / H), j = (int)(e % H);
@@ -55,11 +57,11 @@ struct F8 {
 };
 template <typename T> __device__ __forceinline__ F8 load8(const T* p);
 template <> __device__ __forceinline__ F8 load8<float>(const float* p) {
-    const float4 a = __ldcs(reinterpret_cast<const float4*>(p)), b = __ldcs(reinterpret_cast<const float4*>(p) + 1);
+    const float4 a = ld_stream(reinterpret_cast<const float4*>(p)), b = ld_stream(reinterpret_cast<const float4*>(p) + 1);
     return F8{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
 }
 template <> __device__ __forceinline__ F8 load8<__nv_bfloat16>(const __nv_bfloat16* p) {
-    const uint4 r = __ldcs(reinterpret_cast<const uint4*>(p));
+    const uint4 r = ld_stream(reinterpret_cast<const uint4*>(p));
     const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&r);
     F8 o;
 #pragma unroll
@@ -104,7 +106,9 @@ __device__ __forceinline__ void store8_planes(__nv_bfloat16* p, size_t plane, co
 // halves (bf16(x1 - hi)) in [H, 2H): one operand for the gate's GEMM with both planes along K, two
 // column blocks for the weight-gradient products.  A single bf16 rounding of x1 is not enough there.
 template <typename IO, bool kPlanes>
-__global__ void glu_gelu_kernel(size_t n, int H, const IO* __restrict__ v, void* __restrict__ x1) {
+__global__ void glu_gelu_kernel(size_t n, int H, const IO* v, void* x1) {
+    grid_dep_wait();
+    grid_dep_launch();
     for (size_t e = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 8; e < n; e += (size_t)gridDim.x * blockDim.x * 8) {
         F8 a = load8<IO>(v + e);
 #pragma unroll
@@ -119,7 +123,9 @@ __global__ void glu_gelu_kernel(size_t n, int H, const IO* __restrict__ v, void*
 }
 
 template <typename IO>
-__global__ void glu_out_kernel(size_t n, const IO* __restrict__ v, const float* __restrict__ z, IO* __restrict__ out) {
+__global__ void glu_out_kernel(size_t n, const IO* v, const float* z, IO* out) {
+    grid_dep_wait();
+    grid_dep_launch();
     for (size_t e = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 8; e < n; e += (size_t)gridDim.x * blockDim.x * 8) {
         const F8 a = load8<IO>(v + e), zz = load8<float>(z + e);
         F8 o;
@@ -131,8 +137,10 @@ __global__ void glu_out_kernel(size_t n, const IO* __restrict__ v, const float* 
 
 // gz = gout * v * s (1 - s), s = sigmoid(z): fp32, or two bf16 planes hi / lo `plane` elements apart
 template <typename IO, bool kPlanes>
-__global__ void glu_gz_kernel(size_t n, const IO* __restrict__ v, const IO* __restrict__ gout,
-                              const float* __restrict__ z, void* __restrict__ gz, size_t plane) {
+__global__ void glu_gz_kernel(size_t n, const IO* v, const IO* gout,
+                              const float* z, void* gz, size_t plane) {
+    grid_dep_wait();
+    grid_dep_launch();
     for (size_t e = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 8; e < n; e += (size_t)gridDim.x * blockDim.x * 8) {
         const F8 a = load8<IO>(v + e), g = load8<IO>(gout + e), zz = load8<float>(z + e);
         F8 o;
@@ -147,8 +155,10 @@ __global__ void glu_gz_kernel(size_t n, const IO* __restrict__ v, const IO* __re
 }
 
 template <typename IO>
-__global__ void glu_gv_kernel(size_t n, const IO* __restrict__ v, const IO* __restrict__ gout,
-                              const float* __restrict__ z, const float* __restrict__ gx1, IO* __restrict__ gv) {
+__global__ void glu_gv_kernel(size_t n, const IO* v, const IO* gout,
+                              const float* z, const float* gx1, IO* gv) {
+    grid_dep_wait();
+    grid_dep_launch();
     for (size_t e = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 8; e < n; e += (size_t)gridDim.x * blockDim.x * 8) {
         const F8 a = load8<IO>(v + e), g = load8<IO>(gout + e), zz = load8<float>(z + e), x = load8<float>(gx1 + e);
         F8 o;
@@ -158,7 +168,9 @@ __global__ void glu_gv_kernel(size_t n, const IO* __restrict__ v, const IO* __re
     }
 }
 
-__global__ void glu_reduce_kernel(const float* __restrict__ part, int splits, size_t n, float* __restrict__ out) {
+__global__ void glu_reduce_kernel(const float* part, int splits, size_t n, float* out) {
+    grid_dep_wait();
+    grid_dep_launch();
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
         float acc = 0.f;
         for (int s = 0; s < splits; ++s) acc += part[(size_t)s * n + e];
@@ -170,7 +182,7 @@ __global__ void glu_reduce_kernel(const float* __restrict__ part, int splits, si
 
 void launch_glu_pack(int H, const float* W, void* Wt2, void* Wn_split, float* Wt_f32, cudaStream_t st) {
     count_launch();
-    glu_pack_kernel<<<blocks_for((size_t)H * H), kThreads, 0, st>>>(H, W, (__nv_bfloat16*)Wt2,
+    launch_dep(glu_pack_kernel, blocks_for((size_t)H * H), kThreads, 0, st, H, W, (__nv_bfloat16*)Wt2,
                                                                     (__nv_bfloat16*)Wn_split, Wt_f32);
 }
 
@@ -178,18 +190,18 @@ void launch_glu_gelu(bool io_bf16, bool planes, size_t n, int H, const void* v, 
     count_launch();
     const int b = blocks_for(n / 8);
     if (io_bf16 && planes)
-        glu_gelu_kernel<__nv_bfloat16, true><<<b, kThreads, 0, st>>>(n, H, (const __nv_bfloat16*)v, x1);
+        launch_dep(glu_gelu_kernel<__nv_bfloat16, true>, b, kThreads, 0, st, n, H, (const __nv_bfloat16*)v, x1);
     else if (io_bf16)
-        glu_gelu_kernel<__nv_bfloat16, false><<<b, kThreads, 0, st>>>(n, H, (const __nv_bfloat16*)v, x1);
+        launch_dep(glu_gelu_kernel<__nv_bfloat16, false>, b, kThreads, 0, st, n, H, (const __nv_bfloat16*)v, x1);
     else
-        glu_gelu_kernel<float, false><<<b, kThreads, 0, st>>>(n, H, (const float*)v, x1);
+        launch_dep(glu_gelu_kernel<float, false>, b, kThreads, 0, st, n, H, (const float*)v, x1);
 }
 
 void launch_glu_out(bool io_bf16, size_t n, const void* v, const float* z, void* out, cudaStream_t st) {
     count_launch();
     const int b = blocks_for(n / 8);
-    if (io_bf16) glu_out_kernel<<<b, kThreads, 0, st>>>(n, (const __nv_bfloat16*)v, z, (__nv_bfloat16*)out);
-    else glu_out_kernel<<<b, kThreads, 0, st>>>(n, (const float*)v, z, (float*)out);
+    if (io_bf16) launch_dep(glu_out_kernel<__nv_bfloat16>, b, kThreads, 0, st, n, (const __nv_bfloat16*)v, z, (__nv_bfloat16*)out);
+    else launch_dep(glu_out_kernel<float>, b, kThreads, 0, st, n, (const float*)v, z, (float*)out);
 }
 
 void launch_glu_gz(bool io_bf16, bool planes, size_t n, const void* v, const void* gout, const float* z, void* gz,
@@ -197,11 +209,11 @@ void launch_glu_gz(bool io_bf16, bool planes, size_t n, const void* v, const voi
     count_launch();
     const int b = blocks_for(n / 8);
     if (io_bf16 && planes)
-        glu_gz_kernel<__nv_bfloat16, true><<<b, kThreads, 0, st>>>(n, (const __nv_bfloat16*)v, (const __nv_bfloat16*)gout, z, gz, n);
+        launch_dep(glu_gz_kernel<__nv_bfloat16, true>, b, kThreads, 0, st, n, (const __nv_bfloat16*)v, (const __nv_bfloat16*)gout, z, gz, n);
     else if (io_bf16)
-        glu_gz_kernel<__nv_bfloat16, false><<<b, kThreads, 0, st>>>(n, (const __nv_bfloat16*)v, (const __nv_bfloat16*)gout, z, gz, n);
+        launch_dep(glu_gz_kernel<__nv_bfloat16, false>, b, kThreads, 0, st, n, (const __nv_bfloat16*)v, (const __nv_bfloat16*)gout, z, gz, n);
     else
-        glu_gz_kernel<float, false><<<b, kThreads, 0, st>>>(n, (const float*)v, (const float*)gout, z, gz, n);
+        launch_dep(glu_gz_kernel<float, false>, b, kThreads, 0, st, n, (const float*)v, (const float*)gout, z, gz, n);
 }
 
 void launch_glu_gv(bool io_bf16, size_t n, const void* v, const void* gout, const float* z, const float* gx1, void* gv,
@@ -209,14 +221,14 @@ void launch_glu_gv(bool io_bf16, size_t n, const void* v, const void* gout, cons
     count_launch();
     const int b = blocks_for(n / 8);
     if (io_bf16)
-        glu_gv_kernel<<<b, kThreads, 0, st>>>(n, (const __nv_bfloat16*)v, (const __nv_bfloat16*)gout, z, gx1, (__nv_bfloat16*)gv);
+        launch_dep(glu_gv_kernel<__nv_bfloat16>, b, kThreads, 0, st, n, (const __nv_bfloat16*)v, (const __nv_bfloat16*)gout, z, gx1, (__nv_bfloat16*)gv);
     else
-        glu_gv_kernel<<<b, kThreads, 0, st>>>(n, (const float*)v, (const float*)gout, z, gx1, (float*)gv);
+        launch_dep(glu_gv_kernel<float>, b, kThreads, 0, st, n, (const float*)v, (const float*)gout, z, gx1, (float*)gv);
 }
 
 void launch_glu_reduce(const float* part, int splits, size_t n, float* out, cudaStream_t st) {
     count_launch();
-    glu_reduce_kernel<<<blocks_for(n), kThreads, 0, st>>>(part, splits, n, out);
+    launch_dep(glu_reduce_kernel, blocks_for(n), kThreads, 0, st, part, splits, n, out);
 }
 
 }  // namespace ssm

@@ -20,7 +20,9 @@ __device__ __forceinline__ void split3(float v, __nv_bfloat16& hi, __nv_bfloat16
 
 // in [M, K] fp32 -> out [M, 3K] bf16 (planes side by side).  One thread per 4 neighbouring elements.
 __global__ void __launch_bounds__(256)
-split_planes_kernel(const float* __restrict__ in, size_t M, int K, __nv_bfloat16* __restrict__ out) {
+split_planes_kernel(const float* in, size_t M, int K, __nv_bfloat16* out) {
+    grid_dep_wait();
+    grid_dep_launch();
     const size_t quads = M * (size_t)(K / 4);
     for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < quads; q += (size_t)gridDim.x * blockDim.x) {
         const size_t m = q / (K / 4);
@@ -41,15 +43,17 @@ void launch_split_planes(const float* in, size_t M, int K, void* out, cudaStream
     const size_t quads = M * (size_t)(K / 4);
     const int blocks = (int)std::min<size_t>((quads + 255) / 256, 148 * 16);
     count_launch();
-    split_planes_kernel<<<blocks, 256, 0, st>>>(in, M, K, (__nv_bfloat16*)out);
+    launch_dep(split_planes_kernel, blocks, 256, 0, st, in, M, K, (__nv_bfloat16*)out);
 }
 
 // out[m, n] = acc[m, n] + diag[n] * skip[m, n] (+ add[m, n]): what follows a projection whose fp32 result
 // came out of the tensor cores without an epilogue.  TS / TO: types of skip and out; add is fp32 or NULL.
 template <typename TS, typename TO>
 __global__ void __launch_bounds__(256)
-diag_skip_kernel(const float* __restrict__ acc, const float* __restrict__ diag, const TS* __restrict__ skip,
-                 const float* __restrict__ add, size_t M, int N, TO* __restrict__ out) {
+diag_skip_kernel(const float* acc, const float* diag, const TS* skip,
+                 const float* add, size_t M, int N, TO* out) {
+    grid_dep_wait();
+    grid_dep_launch();
     const size_t n = M * (size_t)N;
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
         float v = fmaf(diag[e % N], to_f32<TS>(skip[e]), acc[e]);
@@ -65,13 +69,13 @@ void launch_diag_skip(const float* acc, const float* diag, const void* skip, boo
     const int blocks = (int)std::min<size_t>((n + 255) / 256, 148 * 16);
     count_launch();
     if (skip_bf16 && out_bf16)
-        diag_skip_kernel<bf, bf><<<blocks, 256, 0, st>>>(acc, diag, (const bf*)skip, add, M, N, (bf*)out);
+        launch_dep(diag_skip_kernel<bf, bf>, blocks, 256, 0, st, acc, diag, (const bf*)skip, add, M, N, (bf*)out);
     else if (skip_bf16)
-        diag_skip_kernel<bf, float><<<blocks, 256, 0, st>>>(acc, diag, (const bf*)skip, add, M, N, (float*)out);
+        launch_dep(diag_skip_kernel<bf, float>, blocks, 256, 0, st, acc, diag, (const bf*)skip, add, M, N, (float*)out);
     else if (out_bf16)
-        diag_skip_kernel<float, bf><<<blocks, 256, 0, st>>>(acc, diag, (const float*)skip, add, M, N, (bf*)out);
+        launch_dep(diag_skip_kernel<float, bf>, blocks, 256, 0, st, acc, diag, (const float*)skip, add, M, N, (bf*)out);
     else
-        diag_skip_kernel<float, float><<<blocks, 256, 0, st>>>(acc, diag, (const float*)skip, add, M, N, (float*)out);
+        launch_dep(diag_skip_kernel<float, float>, blocks, 256, 0, st, acc, diag, (const float*)skip, add, M, N, (float*)out);
 }
 
 }  // namespace ssm

@@ -7,8 +7,10 @@ constexpr int kRowsPerBlock = 64;
 
 // block = 32 columns x 8 row lanes; grid.x = row groups (the dimension that grows with B*T), grid.y = ceil(C/32).
 // out[g, c] = sum of in[r, c] for r in group g.
-__global__ void colsum_kernel(const float* __restrict__ in, int R, int C, int rows_per_group,
-                              float* __restrict__ out) {
+__global__ void colsum_kernel(const float* in, int R, int C, int rows_per_group,
+                              float* out) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ float sm[8][33];
     const int c = blockIdx.y * 32 + threadIdx.x;
     const int r0 = blockIdx.x * rows_per_group;
@@ -33,13 +35,13 @@ void launch_colsum(const float* in, int R, int C, float* out, float* tmp, cudaSt
     const int gx = (C + 31) / 32;
     if (R <= kRowsPerBlock * 2) {
         count_launch();
-        colsum_kernel<<<dim3(1, gx), blk, 0, st>>>(in, R, C, R, out);
+        launch_dep(colsum_kernel, dim3(1, gx), blk, 0, st, in, R, C, R, out);
         return;
     }
     const int groups = (R + kRowsPerBlock - 1) / kRowsPerBlock;
     count_launch(2);
-    colsum_kernel<<<dim3(groups, gx), blk, 0, st>>>(in, R, C, kRowsPerBlock, tmp);
-    colsum_kernel<<<dim3(1, gx), blk, 0, st>>>(tmp, groups, C, groups, out);
+    launch_dep(colsum_kernel, dim3(groups, gx), blk, 0, st, in, R, C, kRowsPerBlock, tmp);
+    launch_dep(colsum_kernel, dim3(1, gx), blk, 0, st, tmp, groups, C, groups, out);
 }
 
 // Brings a [R, C] array of partial sums down to at most `limit` rows by summing groups of kRowsPerBlock rows
@@ -53,7 +55,7 @@ const float* launch_reduce_rows(float* in, int R, int C, float* tmp, int limit, 
     while (R > limit) {
         const int groups = (R + kRowsPerBlock - 1) / kRowsPerBlock;
         count_launch();
-        colsum_kernel<<<dim3(groups, gx), blk, 0, st>>>(cur, R, C, kRowsPerBlock, other);
+        launch_dep(colsum_kernel, dim3(groups, gx), blk, 0, st, cur, R, C, kRowsPerBlock, other);
         float* t = cur;
         cur = other;
         other = t;
@@ -70,12 +72,12 @@ template <typename T>
 __device__ __forceinline__ void load_quad(const T* p, float (&v)[4]);
 template <>
 __device__ __forceinline__ void load_quad<float>(const float* p, float (&v)[4]) {
-    const float4 t = __ldcs(reinterpret_cast<const float4*>(p));
+    const float4 t = ld_stream(reinterpret_cast<const float4*>(p));
     v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
 }
 template <>
 __device__ __forceinline__ void load_quad<__nv_bfloat16>(const __nv_bfloat16* p, float (&v)[4]) {
-    const uint2 t = __ldcs(reinterpret_cast<const uint2*>(p));
+    const uint2 t = ld_stream(reinterpret_cast<const uint2*>(p));
     const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&t.x));
     const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&t.y));
     v[0] = lo.x; v[1] = lo.y; v[2] = hi.x; v[3] = hi.y;
@@ -83,7 +85,9 @@ __device__ __forceinline__ void load_quad<__nv_bfloat16>(const __nv_bfloat16* p,
 
 template <typename TA, typename TB>
 __global__ void __launch_bounds__(256)
-dot_columns_kernel(const TA* __restrict__ a, const TB* __restrict__ b, int M, int C, float* __restrict__ part) {
+dot_columns_kernel(const TA* a, const TB* b, int M, int C, float* part) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ float4 sm[8][33];
     const int c = (blockIdx.y * 32 + threadIdx.x) * 4;
     const int r0 = blockIdx.x * kDotRows;
@@ -127,13 +131,13 @@ int launch_dot_columns_partial(bool a_bf16, const void* a, bool b_bf16, const vo
     dim3 blk(32, 8), grid(g, (C + 127) / 128);
     count_launch();
     if (a_bf16 && b_bf16)
-        dot_columns_kernel<bf, bf><<<grid, blk, 0, st>>>((const bf*)a, (const bf*)b, M, C, tmp);
+        launch_dep(dot_columns_kernel<bf, bf>, grid, blk, 0, st, (const bf*)a, (const bf*)b, M, C, tmp);
     else if (a_bf16)
-        dot_columns_kernel<bf, float><<<grid, blk, 0, st>>>((const bf*)a, (const float*)b, M, C, tmp);
+        launch_dep(dot_columns_kernel<bf, float>, grid, blk, 0, st, (const bf*)a, (const float*)b, M, C, tmp);
     else if (b_bf16)
-        dot_columns_kernel<float, bf><<<grid, blk, 0, st>>>((const float*)a, (const bf*)b, M, C, tmp);
+        launch_dep(dot_columns_kernel<float, bf>, grid, blk, 0, st, (const float*)a, (const bf*)b, M, C, tmp);
     else
-        dot_columns_kernel<float, float><<<grid, blk, 0, st>>>((const float*)a, (const float*)b, M, C, tmp);
+        launch_dep(dot_columns_kernel<float, float>, grid, blk, 0, st, (const float*)a, (const float*)b, M, C, tmp);
     return g;
 }
 

@@ -34,7 +34,7 @@ __device__ __forceinline__ C2 c2_zero() { return C2{make_float2(0.f, 0.f), make_
 template <typename ST> struct StateIO;
 template <> struct StateIO<float4> {
     static __device__ __forceinline__ C2 load(const float4* p, size_t) {
-        const float4 v = __ldcs(p);
+        const float4 v = ld_stream(p);
         return C2{make_float2(v.x, v.y), make_float2(v.z, v.w)};
     }
     static __device__ __forceinline__ void store(float4* p, const C2& v, size_t) {
@@ -54,7 +54,7 @@ __device__ __forceinline__ uint2 pack_bf16x4(const C2& v) {
 }
 template <> struct StateIO<uint2> {
     static __device__ __forceinline__ C2 load(const uint2* p, size_t plane) {
-        const C2 h = unpack_bf16x4(__ldcs(p)), l = unpack_bf16x4(__ldcs(p + plane));
+        const C2 h = unpack_bf16x4(ld_stream(p)), l = unpack_bf16x4(ld_stream(p + plane));
         return C2{cadd(h.a, l.a), cadd(h.b, l.b)};
     }
     static __device__ __forceinline__ void store(uint2* p, const C2& v, size_t plane) {
@@ -74,10 +74,12 @@ __device__ __forceinline__ float4 c2_pack(const C2& v) { return make_float4(v.a.
 // grid: ceil(B * P/2 / kSeqThreads); thread -> (b, pair of states).  x may alias Bu.
 template <typename XT>
 __global__ void __launch_bounds__(kSeqThreads)
-scan_fwd_seq_kernel(int B, int T, int P2, const float4* __restrict__ Abar, const float4* __restrict__ Alo,
+scan_fwd_seq_kernel(int B, int T, int P2, const float4* Abar, const float4* Alo,
                     const float4* Bu,
-                    const uint8_t* __restrict__ done, const float4* __restrict__ x0, XT* x,
-                    float4* __restrict__ xT) {
+                    const uint8_t* done, const float4* x0, XT* x,
+                    float4* xT) {
+    grid_dep_wait();
+    grid_dep_launch();
     const int idx = blockIdx.x * kSeqThreads + threadIdx.x;
     if (idx >= B * P2) return;
     const int b = idx / P2, pp = idx - b * P2;
@@ -117,15 +119,15 @@ scan_fwd_seq_kernel(int B, int T, int P2, const float4* __restrict__ Abar, const
 template <typename XS> struct Raw1;
 template <> struct Raw1<float2> {
     float2 v;
-    __device__ __forceinline__ void load(const float2* p, size_t) { v = __ldcs(p); }
+    __device__ __forceinline__ void load(const float2* p, size_t) { v = ld_stream(p); }
     __device__ __forceinline__ float2 get() const { return v; }
     static __device__ __forceinline__ void store(float2* p, float2 s, size_t) { *p = s; }
 };
 template <> struct Raw1<uint32_t> {
     uint32_t hi, lo;
     __device__ __forceinline__ void load(const uint32_t* p, size_t plane) {
-        hi = __ldcs(p);
-        lo = __ldcs(p + plane);
+        hi = ld_stream(p);
+        lo = ld_stream(p + plane);
     }
     __device__ __forceinline__ float2 get() const {
         const float2 h = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hi));
@@ -151,10 +153,12 @@ template <> struct Raw1<uint32_t> {
 constexpr int kUnroll1 = 8;
 template <typename XS>
 __global__ void __launch_bounds__(kSeqThreads)
-scan_bwd_seq1_kernel(int B, int T, int P, const float2* __restrict__ Abar, const float2* __restrict__ Alo,
-                     const uint8_t* __restrict__ done, const float2* __restrict__ x0, const XS* __restrict__ x,
-                     const float2* gx, const float2* __restrict__ gxT, XS* gBu, float2* __restrict__ gA_part,
-                     float2* __restrict__ gx0) {
+scan_bwd_seq1_kernel(int B, int T, int P, const float2* Abar, const float2* Alo,
+                     const uint8_t* done, const float2* x0, const XS* x,
+                     const float2* gx, const float2* gxT, XS* gBu, float2* gA_part,
+                     float2* gx0) {
+    grid_dep_wait();
+    grid_dep_launch();
     const int idx = blockIdx.x * kSeqThreads + threadIdx.x;
     if (idx >= B * P) return;
     const int b = idx / P, p = idx - b * P;
@@ -181,7 +185,7 @@ scan_bwd_seq1_kernel(int B, int T, int P, const float2* __restrict__ Abar, const
         q.flags = 0u;
 #pragma unroll
         for (int i = 0; i < kUnroll1; ++i) {
-            q.v[i] = __ldcs(gp - (ptrdiff_t)i * P);
+            q.v[i] = ld_stream(gp - (ptrdiff_t)i * P);
             q.xr[i].load(xp - (ptrdiff_t)i * P, plane);
             if (dn && dn[t0 - i] != 0) q.flags |= 1u << i;
         }
@@ -222,7 +226,7 @@ scan_bwd_seq1_kernel(int B, int T, int P, const float2* __restrict__ Abar, const
         }
     }
     for (; t >= 0; --t) {
-        const float2 v = __ldcs(gp);
+        const float2 v = ld_stream(gp);
         float2 xprev = xinit;
         if (t > 0) {
             Raw1<XS> r;
@@ -246,9 +250,11 @@ scan_bwd_seq1_kernel(int B, int T, int P, const float2* __restrict__ Abar, const
 // a thread reads its entry before it writes it).
 template <typename XT>
 __global__ void __launch_bounds__(256)
-scan_fwd_step_kernel(int B, int P2, const float4* __restrict__ Abar, const float4* __restrict__ Alo,
-                     const float4* Bu /* may be the array x is written to */, const uint8_t* __restrict__ done,
+scan_fwd_step_kernel(int B, int P2, const float4* Abar, const float4* Alo,
+                     const float4* Bu /* may be the array x is written to */, const uint8_t* done,
                      const float4* x0, XT* x, float4* xT) {
+    grid_dep_wait();
+    grid_dep_launch();
     const int idx = blockIdx.x * 256 + threadIdx.x;
     if (idx >= B * P2) return;
     const int b = idx / P2, pp = idx - b * P2;
@@ -311,11 +317,11 @@ int launch_scan_fwd(int B, int T, int P, const float2* Abar, const float2* Alo, 
         const int n = B * (P / 2);
         count_launch();
         if (x_bf16)
-            scan_fwd_step_kernel<uint2><<<(n + 255) / 256, 256, 0, st>>>(B, P / 2, (const float4*)Abar, (const float4*)Alo,
+            launch_dep(scan_fwd_step_kernel<uint2>, (n + 255) / 256, 256, 0, st, B, P / 2, (const float4*)Abar, (const float4*)Alo,
                                                                          (const float4*)Bu, done, (const float4*)x0,
                                                                          (uint2*)x, (float4*)xT);
         else
-            scan_fwd_step_kernel<float4><<<(n + 255) / 256, 256, 0, st>>>(B, P / 2, (const float4*)Abar, (const float4*)Alo,
+            launch_dep(scan_fwd_step_kernel<float4>, (n + 255) / 256, 256, 0, st, B, P / 2, (const float4*)Abar, (const float4*)Alo,
                                                                           (const float4*)Bu, done, (const float4*)x0,
                                                                           (float4*)x, (float4*)xT);
         return SSM_OK;
@@ -327,10 +333,10 @@ int launch_scan_fwd(int B, int T, int P, const float2* Abar, const float2* Alo, 
     const int blocks = (int)(((size_t)B * P2 + kSeqThreads - 1) / kSeqThreads);
     count_launch();
     if (x_bf16)
-        scan_fwd_seq_kernel<uint2><<<blocks, kSeqThreads, 0, st>>>(B, T, P2, (const float4*)Abar, (const float4*)Alo, (const float4*)Bu,
+        launch_dep(scan_fwd_seq_kernel<uint2>, blocks, kSeqThreads, 0, st, B, T, P2, (const float4*)Abar, (const float4*)Alo, (const float4*)Bu,
                                                                    done, (const float4*)x0, (uint2*)x, (float4*)xT);
     else
-        scan_fwd_seq_kernel<float4><<<blocks, kSeqThreads, 0, st>>>(B, T, P2, (const float4*)Abar, (const float4*)Alo, (const float4*)Bu,
+        launch_dep(scan_fwd_seq_kernel<float4>, blocks, kSeqThreads, 0, st, B, T, P2, (const float4*)Abar, (const float4*)Alo, (const float4*)Bu,
                                                                     done, (const float4*)x0, (float4*)x, (float4*)xT);
     return SSM_OK;
 }
@@ -352,10 +358,10 @@ int launch_scan_bwd(int B, int T, int P, const float2* Abar, const float2* Alo, 
         count_launch();
         const int blocks1 = (int)(((size_t)B * P + kSeqThreads - 1) / kSeqThreads);
         if (x_bf16)
-            scan_bwd_seq1_kernel<uint32_t><<<blocks1, kSeqThreads, 0, st>>>(
+            launch_dep(scan_bwd_seq1_kernel<uint32_t>, blocks1, kSeqThreads, 0, st, 
                 B, T, P, Abar, Alo, done, x0, (const uint32_t*)x, gx, gxT, (uint32_t*)gBu, (float2*)part, gx0);
         else
-            scan_bwd_seq1_kernel<float2><<<blocks1, kSeqThreads, 0, st>>>(
+            launch_dep(scan_bwd_seq1_kernel<float2>, blocks1, kSeqThreads, 0, st, 
                 B, T, P, Abar, Alo, done, x0, (const float2*)x, gx, gxT, (float2*)gBu, (float2*)part, gx0);
     }
     if (gA_part && gA_rows)

@@ -189,8 +189,8 @@ __device__ __forceinline__ void producer(const Args& k, Shared& sm, uint8_t* sta
 template <int G, typename XS, bool kPair>
 __global__ void __launch_bounds__(kThreads, 2)
 scan_fwd_stream_kernel(Args k, const __grid_constant__ CUtensorMap tm_in, const __grid_constant__ CUtensorMap tm_o0,
-                       const __grid_constant__ CUtensorMap tm_o1, const float2* __restrict__ x0,
-                       float2* __restrict__ xT) {
+                       const __grid_constant__ CUtensorMap tm_o1, const float2* x0,
+                       float2* xT) {
     constexpr int r = kFwdRows, slices = kConsumers / G, R = slices * r;
     constexpr uint32_t stage_bytes = (uint32_t)R * G * 8;
     extern __shared__ uint8_t stream_raw[];
@@ -198,6 +198,8 @@ scan_fwd_stream_kernel(Args k, const __grid_constant__ CUtensorMap tm_in, const 
     uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(stream_raw) + 127) & ~(uintptr_t)127);
     const int tid = threadIdx.x;
     init_shared(sm);
+    grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
+    grid_dep_launch();
     if (tid >= kConsumers) {
         producer<false>(k, sm, stages, stage_bytes, &tm_in, nullptr, nullptr, stage_bytes, 0, 0);
         return;
@@ -336,8 +338,8 @@ template <int G, typename XS, bool kPair, int kRowsPerThread>
 __global__ void __launch_bounds__(kThreads, 2)
 scan_bwd_stream_kernel(Args k, const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_x0,
                        const __grid_constant__ CUtensorMap tm_x1, const __grid_constant__ CUtensorMap tm_o0,
-                       const __grid_constant__ CUtensorMap tm_o1, const float2* __restrict__ x0,
-                       const float2* __restrict__ gxT, float2* __restrict__ gA_part, float2* __restrict__ gx0) {
+                       const __grid_constant__ CUtensorMap tm_o1, const float2* x0,
+                       const float2* gxT, float2* gA_part, float2* gx0) {
     constexpr int r = kRowsPerThread, slices = kConsumers / G, R = slices * r;
     constexpr uint32_t tile_bytes = (uint32_t)R * G * 8, stage_bytes = 2 * tile_bytes;
     extern __shared__ uint8_t stream_raw[];
@@ -345,6 +347,8 @@ scan_bwd_stream_kernel(Args k, const __grid_constant__ CUtensorMap tm_g, const _
     uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(stream_raw) + 127) & ~(uintptr_t)127);
     const int tid = threadIdx.x;
     init_shared(sm);
+    grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
+    grid_dep_launch();
     if (tid >= kConsumers) {
         if (sizeof(XS) == 4)
             producer<true>(k, sm, stages, stage_bytes, &tm_g, &tm_x0, &tm_x1, tile_bytes, tile_bytes / 2, tile_bytes / 2);
@@ -607,7 +611,7 @@ int launch_scan_fwd_stream(int B, int T, int P, const float2* Abar, const float2
     do {                                                                                \
         auto kern = scan_fwd_stream_kernel<GG, XS, PAIR>;                               \
         if (!set_smem(kern, smem)) return SSM_ERR_CUDA;                                 \
-        kern<<<grid, kThreads, smem, st>>>(k, mi, o0, o1, x0, xT);                      \
+        launch_dep(kern, grid, kThreads, smem, st, k, mi, o0, o1, x0, xT);                      \
     } while (0)
 #define SSM_LAUNCH(XS, PAIR)                                                            \
     do {                                                                                \
@@ -653,11 +657,11 @@ int launch_scan_bwd_stream(int B, int T, int P, const float2* Abar, const float2
         if (tall) {                                                                                \
             auto kern = scan_bwd_stream_kernel<GG, XS, PAIR, kBwdRowsLong>;                        \
             if (!set_smem(kern, smem)) return SSM_ERR_CUDA;                                        \
-            kern<<<grid, kThreads, smem, st>>>(k, mg, x0m, x1m, o0, o1, x0, gxT, part, gx0);       \
+            launch_dep(kern, grid, kThreads, smem, st, k, mg, x0m, x1m, o0, o1, x0, gxT, part, gx0);       \
         } else {                                                                                   \
             auto kern = scan_bwd_stream_kernel<GG, XS, PAIR, kBwdRows>;                            \
             if (!set_smem(kern, smem)) return SSM_ERR_CUDA;                                        \
-            kern<<<grid, kThreads, smem, st>>>(k, mg, x0m, x1m, o0, o1, x0, gxT, part, gx0);       \
+            launch_dep(kern, grid, kThreads, smem, st, k, mg, x0m, x1m, o0, o1, x0, gxT, part, gx0);       \
         }                                                                                          \
     } while (0)
 #define SSM_LAUNCH(XS, PAIR)                                                                       \

@@ -30,9 +30,11 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 // TI: type of the layer input u; TO: type of out.
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(kRowThreads)
-stack_fwd_kernel(int H, const TI* __restrict__ u, const float* __restrict__ v, const float* __restrict__ w,
-                 const float* __restrict__ b, TO* __restrict__ out, float* __restrict__ mu_out,
-                 float* __restrict__ rstd_out) {
+stack_fwd_kernel(int H, const TI* u, const float* v, const float* w,
+                 const float* b, TO* out, float* mu_out,
+                 float* rstd_out) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ float red[kRowThreads / 32];
     const size_t row = blockIdx.x;
     const TI* ur = u + row * H;
@@ -60,9 +62,11 @@ stack_fwd_kernel(int H, const TI* __restrict__ u, const float* __restrict__ v, c
 // backward takes).  TG: type of the incoming gradient g; TI: type of the layer input u.
 template <typename TG, typename TI>
 __global__ void __launch_bounds__(kRowThreads)
-stack_bwd_kernel(int H, const TG* __restrict__ g, const TI* __restrict__ u, const float* __restrict__ v,
-                 const float* __restrict__ w, const float* __restrict__ mu_in, const float* __restrict__ rstd_in,
-                 float* __restrict__ gz_out, float* __restrict__ gv) {
+stack_bwd_kernel(int H, const TG* g, const TI* u, const float* v,
+                 const float* w, const float* mu_in, const float* rstd_in,
+                 float* gz_out, float* gv) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ float red[kRowThreads / 32];
     const size_t row = blockIdx.x;
     const TG* gr = g + row * H;
@@ -91,9 +95,11 @@ stack_bwd_kernel(int H, const TG* __restrict__ g, const TI* __restrict__ u, cons
 constexpr int kLnGradRows = 64;
 template <typename TG, typename TI>
 __global__ void __launch_bounds__(256)
-ln_param_grad_kernel(int M, int H, const TG* __restrict__ g, const TI* __restrict__ u, const float* __restrict__ v,
-                     const float* __restrict__ mu_in, const float* __restrict__ rstd_in,
-                     float* __restrict__ part_w, float* __restrict__ part_b) {
+ln_param_grad_kernel(int M, int H, const TG* g, const TI* u, const float* v,
+                     const float* mu_in, const float* rstd_in,
+                     float* part_w, float* part_b) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ float sw[8][33], sb[8][33];
     const int h = blockIdx.y * 32 + threadIdx.x;
     const int r0 = blockIdx.x * kLnGradRows, r1 = min(M, r0 + kLnGradRows);   // row groups along x (no 65535 limit)
@@ -133,21 +139,21 @@ void launch_stack_fwd(bool u_bf16, bool out_bf16, int M, int H, const void* u, c
     using bf = __nv_bfloat16;
     count_launch();
     if (u_bf16 && out_bf16)
-        stack_fwd_kernel<bf, bf><<<M, kRowThreads, 0, st>>>(H, (const bf*)u, v, w, b, (bf*)out, mu, rstd);
+        launch_dep(stack_fwd_kernel<bf, bf>, M, kRowThreads, 0, st, H, (const bf*)u, v, w, b, (bf*)out, mu, rstd);
     else if (u_bf16)
-        stack_fwd_kernel<bf, float><<<M, kRowThreads, 0, st>>>(H, (const bf*)u, v, w, b, (float*)out, mu, rstd);
+        launch_dep(stack_fwd_kernel<bf, float>, M, kRowThreads, 0, st, H, (const bf*)u, v, w, b, (float*)out, mu, rstd);
     else if (out_bf16)
-        stack_fwd_kernel<float, bf><<<M, kRowThreads, 0, st>>>(H, (const float*)u, v, w, b, (bf*)out, mu, rstd);
+        launch_dep(stack_fwd_kernel<float, bf>, M, kRowThreads, 0, st, H, (const float*)u, v, w, b, (bf*)out, mu, rstd);
     else
-        stack_fwd_kernel<float, float><<<M, kRowThreads, 0, st>>>(H, (const float*)u, v, w, b, (float*)out, mu, rstd);
+        launch_dep(stack_fwd_kernel<float, float>, M, kRowThreads, 0, st, H, (const float*)u, v, w, b, (float*)out, mu, rstd);
 }
 
 template <typename TG, typename TI>
 static void stack_bwd_launch(int M, int H, const void* g, const void* u, const float* v, const float* w, const float* mu,
                              const float* rstd, float* gz, float* gv, float* part_w, float* part_b, cudaStream_t st) {
     dim3 blk(32, 8), grid(ln_groups(M), (H + 31) / 32);
-    stack_bwd_kernel<TG, TI><<<M, kRowThreads, 0, st>>>(H, (const TG*)g, (const TI*)u, v, w, mu, rstd, gz, gv);
-    ln_param_grad_kernel<TG, TI><<<grid, blk, 0, st>>>(M, H, (const TG*)g, (const TI*)u, v, mu, rstd, part_w, part_b);
+    launch_dep(stack_bwd_kernel<TG, TI>, M, kRowThreads, 0, st, H, (const TG*)g, (const TI*)u, v, w, mu, rstd, gz, gv);
+    launch_dep(ln_param_grad_kernel<TG, TI>, grid, blk, 0, st, M, H, (const TG*)g, (const TI*)u, v, mu, rstd, part_w, part_b);
 }
 
 void launch_stack_bwd(bool g_bf16, bool u_bf16, int M, int H, const void* g, const void* u, const float* v,
