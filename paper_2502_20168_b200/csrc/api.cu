@@ -406,6 +406,16 @@ SSM_API int ssm_step(const ssm_shape* shape, const float* D, const void* u, cons
     const LayerPlan p = plan_layer(s);
     if (int rc = check_ws(ws, ws_bytes, p.total)) return rc;
     // each (trajectory, state) is read as x0 and written as xT by the same thread, so x_next may be x_prev
+    const bool few = use_step_small(s.B, s.H, s.P);
+    if ((p.tc || p.planes) && (few || use_step_kernel(s.H, s.P, p.planes))) {
+        StageTimer tm("step", (cudaStream_t)stream);
+        const StepCall g{s.B, s.H, s.P, p.planes, at<void>(ws, p.W0), at<void>(ws, p.W2), at<float2>(ws, p.Abar), at<float2>(ws, p.Alo),
+                         D, u, done, (const float2*)x_prev, (float2*)x_next, at<void>(ws, p.xs), y, at<WsHeader>(ws, p.hdr)};
+        const int rc = few ? launch_step_small(g, (cudaStream_t)stream) : launch_step(g, (cudaStream_t)stream);
+        if (rc) return rc;
+        SSM_RETURN_IF_CUDA_ERROR();
+        return SSM_OK;
+    }
     return layer_fwd_run(s, p, layer_io(s), D, u, done, x_prev, y, x_next, ws, at<WsHeader>(ws, p.hdr),
                          (cudaStream_t)stream);
 }

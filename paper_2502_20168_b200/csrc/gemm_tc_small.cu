@@ -16,7 +16,7 @@
 #include <algorithm>
 
 #include "kernels.h"
-#include "tcgen05.cuh"
+#include "small_tile.cuh"
 
 namespace ssm {
 namespace tc {
@@ -26,7 +26,6 @@ namespace tc {
 __host__ __device__ constexpr int sm_epi_warps(int bn) { return bn == 256 ? 16 : 8; }
 __host__ __device__ constexpr int sm_threads(int bn) { return 64 + 32 * sm_epi_warps(bn); }
 constexpr int kSmMaxStages = 6;
-constexpr int kSmATile = BM * BK * 2;            // one plane of the A tile of a k-block
 constexpr size_t kSmSmemMax = 218 * 1024;        // of the 227 KB a CTA can have (the rest: static shared memory)
 
 struct SmallTnArgs {
@@ -54,63 +53,6 @@ struct SmallTnArgs {
 // Epilogues: fp32 result; out = acc + diag * skip (+ add) with, if asked for, the column sums of skip * dot over the
 // rows of this CTA; fp32 result and out2 = skip * sigmoid(acc) in bf16.
 enum SmallEpi { kSmStore, kSmDiag, kSmGate };
-
-// Four neighbouring values of an epilogue operand as loaded; decoded when they are used, so that many can be in
-// flight.  kBf16: the operands are known to be bf16 (half the registers), else the flag says.
-template <bool kBf16> struct Raw4;
-template <> struct Raw4<true> {
-    uint2 r;
-    __device__ __forceinline__ void load(const void* p, bool, size_t i) {
-        r = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(p) + i);
-    }
-    __device__ __forceinline__ float4 get(bool) const {
-        return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
-                           __uint_as_float(r.y & 0xffff0000u));
-    }
-};
-template <> struct Raw4<false> {
-    uint4 r;
-    __device__ __forceinline__ void load(const void* p, bool bf16, size_t i) {
-        if (bf16) {
-            const uint2 t = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(p) + i);
-            r.x = t.x, r.y = t.y;
-        } else {
-            r = *reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(p) + i);
-        }
-    }
-    __device__ __forceinline__ float4 get(bool bf16) const {
-        if (bf16) return Raw4<true>{make_uint2(r.x, r.y)}.get(true);
-        return make_float4(__uint_as_float(r.x), __uint_as_float(r.y), __uint_as_float(r.z), __uint_as_float(r.w));
-    }
-};
-__device__ __forceinline__ uint2 pack4_bf16(float4 v) {
-    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-    return make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
-}
-__device__ __forceinline__ void store4_io(void* p, bool bf16, size_t i, float4 v) {
-    if (!bf16) *reinterpret_cast<float4*>(reinterpret_cast<float*>(p) + i) = v;
-    else *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p) + i) = pack4_bf16(v);
-}
-
-// Eight fp32 values -> the 16-byte chunks of their three bf16 planes (hi + mid + lo = value).
-__device__ __forceinline__ void split8(const float4 a, const float4 b, uint4& hi, uint4& mid, uint4& lo) {
-    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    uint32_t* h = &hi.x;
-    uint32_t* m = &mid.x;
-    uint32_t* l = &lo.x;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-        const float2 pf = __bfloat1622float2(p);
-        const float r0 = v[2 * i] - pf.x, r1 = v[2 * i + 1] - pf.y;
-        const __nv_bfloat162 q = __floats2bfloat162_rn(r0, r1);
-        const float2 qf = __bfloat1622float2(q);
-        const __nv_bfloat162 t = __floats2bfloat162_rn(r0 - qf.x, r1 - qf.y);
-        h[i] = *reinterpret_cast<const uint32_t*>(&p);
-        m[i] = *reinterpret_cast<const uint32_t*>(&q);
-        l[i] = *reinterpret_cast<const uint32_t*>(&t);
-    }
-}
 
 struct SmallBars {
     uint64_t full[kSmMaxStages], empty[kSmMaxStages], done;
@@ -211,40 +153,14 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     } else {
         if (kSplitA) {
             const int te = threadIdx.x - 64;
-            // A: 128 rows x 8 chunks of 8 values per k-block, two chunks per thread; 8 threads read a row's 256
-            // bytes, the next k-block's values are on their way while this one is split and stored
-            const int c8 = te & 7, r0 = te >> 3;
-            constexpr int kC = 1024 / (32 * kSmEpiWarps), kStep = 4 * kSmEpiWarps;   // chunks per thread, rows between them
-            float4 va[kC], vb[kC];
-            auto fetch = [&](int kb) {
-#pragma unroll
-                for (int i = 0; i < kC; ++i) {
-                    const int m = m0 + r0 + kStep * i;
-                    va[i] = vb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (m < p.M) {
-                        const float4* src = reinterpret_cast<const float4*>(p.a_f32 + (size_t)m * p.K + kb * BK + 8 * c8);
-                        va[i] = src[0];
-                        vb[i] = src[1];
-                    }
-                }
-            };
-            if (kb0 < kb1) fetch(kb0);
+            SplitA<32 * kSmEpiWarps> sp;   // the next k-block's values are on their way while this one is split and stored
+            if (kb0 < kb1) sp.fetch(p.a_f32, p.K, p.M, m0, kb0, te);
             int stage = 0;
             uint32_t phase = 0;
             for (int kb = kb0; kb < kb1; ++kb) {
                 if (!mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
-                uint8_t* dst = tiles + (size_t)stage * p.stage_bytes;
-#pragma unroll
-                for (int i = 0; i < kC; ++i) {
-                    const int r = r0 + kStep * i;
-                    uint4 hi, mid, lo;
-                    split8(va[i], vb[i], hi, mid, lo);
-                    uint8_t* q = dst + r * 128 + ((c8 ^ (r & 7)) << 4);   // the 128-byte swizzle of a K-major tile
-                    *reinterpret_cast<uint4*>(q) = hi;
-                    *reinterpret_cast<uint4*>(q + kSmATile) = mid;
-                    *reinterpret_cast<uint4*>(q + 2 * kSmATile) = lo;
-                }
-                if (kb + 1 < kb1) fetch(kb + 1);
+                sp.store(tiles + (size_t)stage * p.stage_bytes, p.M, m0, te);
+                if (kb + 1 < kb1) sp.fetch(p.a_f32, p.K, p.M, m0, kb + 1, te);
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bars.full[stage]));

@@ -145,6 +145,28 @@ bool tc_tn_dot_supported(int M, int N_out, int K);
 int tc_tn_dot_max_rows(int M, int N_out);
 int launch_gemm_tc_tn(const GemmTcTN& g, cudaStream_t st);
 
+// One step for B trajectories in one kernel (gemm_tc_step.cu), from the operands of the tensor-core path (f32 = false:
+// Wb hi/lo stacked [4P, H] in the plain order, Wc [H, 2P]) or of the plane path (f32: Wb [2P, 3H], Wc [H, 6P]).
+struct StepCall {
+    int B, H, P;
+    bool f32;
+    const void *Wb, *Wc;
+    const float2 *Abar, *Alo;
+    const float* D;
+    const void* u;             // [B, H] io
+    const uint8_t* done;       // [B] or NULL
+    const float2* x_prev;      // [B, P]
+    float2* x_next;            // [B, P]; may be x_prev
+    void* x_bf16;              // scratch [B, 2P] bf16 (f32: unused)
+    void* y;                   // [B, H] io
+    WsHeader* hdr;
+};
+bool use_step_kernel(int H, int P, bool f32);
+int launch_step(const StepCall& g, cudaStream_t st);
+// The same for a few trajectories, on the CUDA cores (step_small.cu).
+bool use_step_small(int B, int H, int P);
+int launch_step_small(const StepCall& g, cudaStream_t st);
+
 // Input projection and forward scan fused (gemm_tc.cu): x = scan(u Bbar^T) written as the two bf16
 // planes of x; Bu never reaches memory.  T must be a multiple of 128 and there must be enough
 // (sequence, 64 states) chains for every pair of CTAs (tc_gemm_scan_fwd_supported).

@@ -1,0 +1,18 @@
+"""The kernels of single-step mode at the edges of their dispatch: the CUDA-core pair (few trajectories, rows off its
+groups of 8), the cluster kernel (one row more than a 128-row tile, widths that leave the last column tile of a cluster
+empty or partly filled, more state columns than features and the other way round), and fp32 wider than it takes."""
+import pytest
+
+from paper_2502_20168_b200 import inputs as I
+from tests.test_gpu_step_mode import _rollout
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("io,B,H,P", [("f32", 1, 256, 128), ("f32", 13, 512, 128), ("bf16", 3, 128, 64), ("bf16", 29, 384, 448),
+                                      ("bf16", 129, 512, 256), ("bf16", 300, 384, 64), ("bf16", 2100, 128, 192),
+                                      ("bf16", 257, 640, 320), ("f32", 129, 256, 128), ("f32", 1100, 256, 128),
+                                      ("f32", 130, 512, 128)])
+def test_rollout(io, B, H, P, in_place):
+    _rollout(I.Workload("step_k", B=B, T=1, H=H, P=P, io_dtype=io, p_done=0.1, seed=B + H), 3, in_place)
