@@ -51,7 +51,7 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true) {
     p.tc = allow_tc && s.io_dtype == SSM_BF16 && tc_tn_supported((int)BT, P2, s.H, true) &&
            tc_tn_supported((int)BT, s.H, P2, false) && tc_nt_supported(s.H, P2);
     p.planes = !p.tc && s.io_dtype == SSM_F32 && planes_supported(s);
-    p.splits = p.tc ? tc_nt_splits((int)BT, s.H, P2) : (p.planes ? tc_nt_multi_splits((int)BT, s.H, P2) : gemm_nt_splits((int)BT));
+    p.splits = p.tc ? tc_nt_splits((int)BT, s.H, P2) : (p.planes ? tc_nt_planes_splits((int)BT, s.H, P2) : gemm_nt_splits((int)BT));
     p.hdr = take(off, sizeof(WsHeader));
     p.Abar = take(off, (size_t)s.P * 8);
     p.Alo = take(off, (size_t)s.P * 8);
@@ -236,7 +236,7 @@ static void layer_prepare(const ssm_shape& s, const LayerPlan& p, const ssm_c64*
 }
 
 // Launch sequence of one layer's forward pass from a prepared workspace.  `hdr` receives the
-// status of bounded waits.
+// status of bounded waits.  keep_planes: a backward pass will follow (fp32 layers leave the planes of u and x for it).
 // Storage types of the tensors a layer reads and writes.  For the entry points of a single layer all
 // of them are shape->io_dtype; inside a stack only the stack's own input and outputs are.
 struct LayerIo {
@@ -250,7 +250,7 @@ static LayerIo layer_io(const ssm_shape& s) {
 
 static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& io, const float* D, const void* u,
                          const uint8_t* done, const ssm_c64* x0, void* y, ssm_c64* xT, void* ws, WsHeader* hdr,
-                         cudaStream_t st) {
+                         bool keep_planes, cudaStream_t st) {
     const int BT = s.B * s.T, P2 = 2 * s.P;
     if (p.tc && !(io.u_bf16 && io.y_bf16)) return SSM_ERR_DTYPE;   // the tensor-core path reads and writes bf16
     int rc = SSM_OK;
@@ -287,14 +287,16 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
     } else if (p.planes) {
         {   // Bu = u Bbar^T as a sum of plane products (u: three planes of an fp32 input, or the bf16 input itself)
             StageTimer tm("gemm_Bu", st);
-            if (!io.u_bf16) launch_split_planes((const float*)u, (size_t)BT, s.H, at<void>(ws, p.u3), st);
-            GemmTcTN g{io.u_bf16 ? u : at<void>(ws, p.u3), at<void>(ws, p.W0), BT, P2, s.H, false, true, at<void>(ws, p.xs),
+            const bool split_here = !io.u_bf16 && tc_tn_small(BT, P2, false);
+            if (!io.u_bf16 && !split_here) launch_split_planes((const float*)u, (size_t)BT, s.H, at<void>(ws, p.u3), st);
+            GemmTcTN g{io.u_bf16 || split_here ? u : at<void>(ws, p.u3), at<void>(ws, p.W0), BT, P2, s.H, false, true, at<void>(ws, p.xs),
                        nullptr, nullptr, hdr};
             g.n_products = io.u_bf16 ? 3 : 6;
             g.planes_a = io.u_bf16 ? 1 : 3;
             g.planes_w = 3;
             g.prod_a = io.u_bf16 ? kProd3A : kProd6A;
             g.prod_w = io.u_bf16 ? kProd3B : kProd6B;
+            if (split_here) g.a_f32 = true, g.a_planes_out = keep_planes ? at<void>(ws, p.u3) : nullptr;
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
         }
         {
@@ -307,8 +309,8 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
         {   // y = x Cp^T + D u: planes of x, six products, the skip term in the epilogue or after it
             StageTimer tm("gemm_y", st);
             const bool small = tc_tn_small(BT, s.H, false);
-            launch_split_planes(at<float>(ws, p.xs), (size_t)BT, P2, at<void>(ws, p.x3), st);
-            GemmTcTN g{at<void>(ws, p.x3), at<void>(ws, p.W2), BT, s.H, P2, false, true, at<void>(ws, p.acc), nullptr,
+            if (!small) launch_split_planes(at<float>(ws, p.xs), (size_t)BT, P2, at<void>(ws, p.x3), st);
+            GemmTcTN g{small ? at<void>(ws, p.xs) : at<void>(ws, p.x3), at<void>(ws, p.W2), BT, s.H, P2, false, true, at<void>(ws, p.acc), nullptr,
                        nullptr, hdr};
             g.n_products = 6;
             g.planes_a = 3;
@@ -317,6 +319,7 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
             g.prod_w = kProd6B;
             if (small) {
                 g.store_f32 = !io.y_bf16, g.out = y, g.diag = D, g.skip = u, g.skip_bf16 = io.u_bf16;
+                g.a_f32 = true, g.a_planes_out = keep_planes ? at<void>(ws, p.x3) : nullptr;
             }
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
             if (!small) launch_diag_skip(at<float>(ws, p.acc), D, u, io.u_bf16, nullptr, (size_t)BT, s.H, y, io.y_bf16, st);
@@ -351,7 +354,7 @@ static int layer_fwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
                           const uint8_t* done, const ssm_c64* x0, void* y, ssm_c64* xT, void* ws, WsHeader* hdr,
                           bool clear_hdr, cudaStream_t st) {
     layer_prepare(s, p, Lambda, Delta, Bc, Cc, ws, clear_hdr ? hdr : nullptr, st);
-    return layer_fwd_run(s, p, io, D, u, done, x0, y, xT, ws, hdr, st);
+    return layer_fwd_run(s, p, io, D, u, done, x0, y, xT, ws, hdr, true, st);
 }
 
 SSM_API int ssm_layer_fwd(const ssm_shape* shape, const ssm_c64* Lambda, const float* Delta, const ssm_c64* Bc,
@@ -416,7 +419,7 @@ SSM_API int ssm_step(const ssm_shape* shape, const float* D, const void* u, cons
         SSM_RETURN_IF_CUDA_ERROR();
         return SSM_OK;
     }
-    return layer_fwd_run(s, p, layer_io(s), D, u, done, x_prev, y, x_next, ws, at<WsHeader>(ws, p.hdr),
+    return layer_fwd_run(s, p, layer_io(s), D, u, done, x_prev, y, x_next, ws, at<WsHeader>(ws, p.hdr), false,
                          (cudaStream_t)stream);
 }
 
@@ -628,14 +631,16 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
         const bool gyb = io.gy_bf16, ub = io.u_bf16;
         {   // g_x = gy conj(C)
             StageTimer tm("gemm_gx", st);
-            if (!gyb) launch_split_planes((const float*)gy, (size_t)BT, s.H, at<void>(ws, p.gy3), st);
-            GemmTcTN g{gyb ? gy : at<void>(ws, p.gy3), at<void>(ws, p.W1), BT, P2, s.H, false, true, at<void>(ws, p.gs),
+            const bool split_here = !gyb && tc_tn_small(BT, P2, false);
+            if (!gyb && !split_here) launch_split_planes((const float*)gy, (size_t)BT, s.H, at<void>(ws, p.gy3), st);
+            GemmTcTN g{gyb || split_here ? gy : at<void>(ws, p.gy3), at<void>(ws, p.W1), BT, P2, s.H, false, true, at<void>(ws, p.gs),
                        nullptr, nullptr, hdr};
             g.n_products = gyb ? 3 : 6;
             g.planes_a = gyb ? 1 : 3;
             g.planes_w = 3;
             g.prod_a = gyb ? kProd3A : kProd6A;
             g.prod_w = gyb ? kProd3B : kProd6B;
+            if (split_here) g.a_f32 = true, g.a_planes_out = at<void>(ws, p.gy3);
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
         }
         {
@@ -649,8 +654,8 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
         {   // du = s Bq^T + D gy (+ the residual branch's gradient); where the epilogue does that, dD's sums as well
             StageTimer tm("gemm_du", st);
             const bool small = tc_tn_small(BT, s.H, false);
-            launch_split_planes(at<float>(ws, p.gs), (size_t)BT, P2, at<void>(ws, p.s3), st);
-            GemmTcTN g{at<void>(ws, p.s3), at<void>(ws, p.W3), BT, s.H, P2, false, true, at<void>(ws, p.acc), nullptr,
+            if (!small) launch_split_planes(at<float>(ws, p.gs), (size_t)BT, P2, at<void>(ws, p.s3), st);
+            GemmTcTN g{small ? at<void>(ws, p.gs) : at<void>(ws, p.s3), at<void>(ws, p.W3), BT, s.H, P2, false, true, at<void>(ws, p.acc), nullptr,
                        nullptr, hdr};
             g.n_products = 6;
             g.planes_a = 3;
@@ -661,29 +666,20 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
                 g.store_f32 = !io.du_bf16, g.out = du, g.diag = D, g.skip = gy, g.skip_bf16 = gyb, g.add = du_add;
                 g.dot = u, g.dot_bf16 = ub, g.dot_part = at<float>(ws, p.dot), g.dot_rows = &dD_rows;
                 dD_part = g.dot_part;
+                g.a_f32 = true, g.a_planes_out = at<void>(ws, p.s3);
             }
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
             if (!small) launch_diag_skip(at<float>(ws, p.acc), D, gy, gyb, du_add, (size_t)BT, s.H, du, io.du_bf16, st);
         }
-        {   // gBbar = s^T u
-            StageTimer tm("gemm_gBbar", st);
-            GemmTcNT g{ub ? u : at<void>(ws, p.u3), s.H, at<void>(ws, p.s3), nullptr, P2, BT, p.splits, part, hdr};
-            g.n_products = ub ? 3 : 6;
-            g.planes_a = ub ? 1 : 3;
-            g.planes_b = 3;
-            g.prod_a = ub ? kProd3A : kProd6A;
-            g.prod_b = ub ? kProd3B : kProd6B;
-            if ((rc = launch_gemm_tc_nt(g, st))) return rc;
-        }
-        {   // dC = gy^T conj(x)
-            StageTimer tm("gemm_gC", st);
-            GemmTcNT g{gyb ? gy : at<void>(ws, p.gy3), s.H, at<void>(ws, p.x3), nullptr, P2, BT, p.splits, part_c, hdr};
-            g.n_products = gyb ? 3 : 6;
-            g.planes_a = gyb ? 1 : 3;
-            g.planes_b = 3;
-            g.prod_a = gyb ? kProd3A : kProd6A;
-            g.prod_b = gyb ? kProd3B : kProd6B;
-            if ((rc = launch_gemm_tc_nt(g, st))) return rc;
+        {   // gBbar = s^T u and dC = gy^T conj(x)
+            StageTimer tm("gemm_gBbar_gC", st);
+            const GemmTcNtPlanes g{
+                BT, s.H, P2, p.splits,
+                {{ub ? u : at<void>(ws, p.u3), at<void>(ws, p.s3), ub ? 1 : 3, 3, ub ? 3 : 6, ub ? kProd3A : kProd6A, ub ? kProd3B : kProd6B, part},
+                 {gyb ? gy : at<void>(ws, p.gy3), at<void>(ws, p.x3), gyb ? 1 : 3, 3, gyb ? 3 : 6, gyb ? kProd3A : kProd6A,
+                  gyb ? kProd3B : kProd6B, part_c}},
+                hdr};
+            if ((rc = launch_gemm_tc_nt_planes(g, st))) return rc;
         }
     } else {
         {

@@ -1606,15 +1606,9 @@ struct NtParams {
     int blocks_per_split;  // k-blocks (of BK rows) per slice
     float* part;        // [splits, I, J]
     WsHeader* hdr;
-    // kMulti: n_prod products of bf16 planes in one accumulator; product j takes plane (pa >> 4 j) & 15 of A
-    // (columns [a I, (a + 1) I) of its matrix) and plane (pb >> 4 j) & 15 of Bm (columns [b J, (b + 1) J)).
-    int n_prod;
-    uint32_t pa, pb;
 };
 
-// kMulti = false: the 256 accumulator columns are 128 output columns times the two planes (hi, lo) of Bm, added
-// in the epilogue.  kMulti = true: 256 output columns, every product of the schedule accumulated in place.
-template <bool kMulti>
+// The 256 accumulator columns are 128 output columns times the two planes (hi, lo) of Bm, added in the epilogue.
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_nt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBhi,
                   const __grid_constant__ CUtensorMap tmBlo, NtParams p) {
@@ -1625,7 +1619,7 @@ gemm_tc_nt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
     grid_dep_launch();
     const int tile = blockIdx.x, split = blockIdx.y;
-    constexpr int kOutCols = kMulti ? BN : BN / 2;   // (not kMulti) accumulator columns [0,128): hi plane, [128,256): lo plane
+    constexpr int kOutCols = BN / 2;   // accumulator columns [0,128): hi plane, [128,256): lo plane
     const int i0 = (tile / p.j_tiles) * BM, j0 = (tile % p.j_tiles) * kOutCols;
     const int total_blocks = (p.K + BK - 1) / BK;
     const int kb0 = split * p.blocks_per_split;
@@ -1639,26 +1633,17 @@ gemm_tc_nt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             prefetch_tmap(&tmBlo);
             int stage = 0;
             uint32_t phase = 0;
-            for (int kq = 0; kq < (kMulti ? p.n_prod : 1) * nkb; ++kq) {
+            for (int kb = 0; kb < nkb; ++kb) {
                 if (!mbar_wait(s.empty(stage), phase ^ 1u, s.abort_flag)) break;
                 mbar_expect_tx(s.full(stage), kStageBytes);
                 const uint32_t a_dst = smem_u32(s.tiles + (size_t)stage * kStageBytes);
-                const int j = kq / max(nkb, 1), kb = kq - j * nkb;   // product of the schedule, k-block of the slice
                 const int row = (kb0 + kb) * BK;
-                const int ia = kMulti ? (int)((p.pa >> (4 * j)) & 15u) * p.I + i0 : i0;
-                const int jb = kMulti ? (int)((p.pb >> (4 * j)) & 15u) * p.J + j0 : j0;
 #pragma unroll
-                for (int h = 0; h < BM / 64; ++h) tma_load_2d(a_dst + h * (BK * 128), &tmA, s.full(stage), ia + 64 * h, row);
-                if (kMulti) {
+                for (int h = 0; h < BM / 64; ++h) tma_load_2d(a_dst + h * (BK * 128), &tmA, s.full(stage), i0 + 64 * h, row);
 #pragma unroll
-                    for (int h = 0; h < BN / 64; ++h)
-                        tma_load_2d(a_dst + kABytes + h * (BK * 128), &tmBhi, s.full(stage), jb + 64 * h, row);
-                } else {
-#pragma unroll
-                    for (int h = 0; h < BN / 128; ++h) {
-                        tma_load_2d(a_dst + kABytes + h * (BK * 128), &tmBhi, s.full(stage), j0 + 64 * h, row);
-                        tma_load_2d(a_dst + kABytes + (BN / 128 + h) * (BK * 128), &tmBlo, s.full(stage), j0 + 64 * h, row);
-                    }
+                for (int h = 0; h < BN / 128; ++h) {
+                    tma_load_2d(a_dst + kABytes + h * (BK * 128), &tmBhi, s.full(stage), j0 + 64 * h, row);
+                    tma_load_2d(a_dst + kABytes + (BN / 128 + h) * (BK * 128), &tmBlo, s.full(stage), j0 + 64 * h, row);
                 }
                 if (++stage == kStages) {
                     stage = 0;
@@ -1672,7 +1657,7 @@ gemm_tc_nt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
-            for (int kb = 0; kb < (kMulti ? p.n_prod : 1) * nkb; ++kb) {
+            for (int kb = 0; kb < nkb; ++kb) {
                 if (!(ok = mbar_wait(s.full(stage), phase, s.abort_flag))) break;
                 tc_fence_after();
                 const uint32_t a_addr = smem_u32(s.tiles + (size_t)stage * kStageBytes);
@@ -1712,12 +1697,10 @@ gemm_tc_nt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     tmem_ld_wait();
 #pragma unroll
                     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-                    if (!kMulti) {
-                        tmem_ld32(t_row + (uint32_t)(kOutCols + c), r);
-                        tmem_ld_wait();
+                    tmem_ld32(t_row + (uint32_t)(kOutCols + c), r);
+                    tmem_ld_wait();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) v[i] += __uint_as_float(r[i]);
-                    }
+                    for (int i = 0; i < 32; ++i) v[i] += __uint_as_float(r[i]);
                 } else {
 #pragma unroll
                     for (int i = 0; i < 32; ++i) v[i] = 0.f;
@@ -2155,24 +2138,12 @@ int launch_gemm_tc_nt(const GemmTcNT& g, cudaStream_t st) {
     CUtensorMap ma, mbh, mbl;
     const int blocks = (g.K + BK - 1) / BK;
     const int bps = (blocks + g.splits - 1) / g.splits;
-    if (g.n_products > 0) {   // planes side by side: A [K, planes_a * I], Bm [K, planes_b * J]
-        if (g.n_products > 8 || g.J % BN != 0) return SSM_ERR_SHAPE;
-        if (!make_map(&ma, g.A, (uint64_t)g.K, (uint64_t)g.I * g.planes_a, 64, BK)) return SSM_ERR_CUDA;
-        if (!make_map(&mbh, g.Bm_hi, (uint64_t)g.K, (uint64_t)g.J * g.planes_b, 64, BK)) return SSM_ERR_CUDA;
-        const int j_tiles = g.J / BN;
-        NtParams p{g.K, g.J, g.I, j_tiles, bps, g.part, g.hdr, g.n_products, g.prod_a, g.prod_b};
-        dim3 grid((g.I / BM) * j_tiles, g.splits);
-        count_launch();
-        const bool ok = set_smem(gemm_tc_nt_kernel<true>, kNtSmemBytes);
-        launch_dep(gemm_tc_nt_kernel<true>, grid, kThreads, kNtSmemBytes, st, ma, mbh, mbh, p);
-        return ok ? SSM_OK : SSM_ERR_CUDA;
-    }
     if (!make_map(&ma, g.A, (uint64_t)g.K, (uint64_t)g.I, 64, BK, false, CU_TENSOR_MAP_SWIZZLE_128B, (uint64_t)g.lda))
         return SSM_ERR_CUDA;
     if (!make_map(&mbh, g.Bm_hi, (uint64_t)g.K, (uint64_t)g.J, 64, BK)) return SSM_ERR_CUDA;
     if (!make_map(&mbl, g.Bm_lo, (uint64_t)g.K, (uint64_t)g.J, 64, BK)) return SSM_ERR_CUDA;
     const int j_tiles = g.J / (BN / 2);
-    NtParams p{g.K, g.J, g.I, j_tiles, bps, g.part, g.hdr, 0, 0u, 0u};
+    NtParams p{g.K, g.J, g.I, j_tiles, bps, g.part, g.hdr};
     if (SSM_NT_PAIRS && g.I % (2 * BM) == 0) {   // 256 x 256 tiles on CTA pairs
         dim3 grid(2 * (g.I / (2 * BM)) * j_tiles, g.splits);
         count_launch();
@@ -2182,20 +2153,9 @@ int launch_gemm_tc_nt(const GemmTcNT& g, cudaStream_t st) {
     }
     dim3 grid((g.I / BM) * j_tiles, g.splits);
     count_launch();
-    const bool ok = set_smem(gemm_tc_nt_kernel<false>, kNtSmemBytes);
-    launch_dep(gemm_tc_nt_kernel<false>, grid, kThreads, kNtSmemBytes, st, ma, mbh, mbl, p);
+    const bool ok = set_smem(gemm_tc_nt_kernel, kNtSmemBytes);
+    launch_dep(gemm_tc_nt_kernel, grid, kThreads, kNtSmemBytes, st, ma, mbh, mbl, p);
     return ok ? SSM_OK : SSM_ERR_CUDA;
-}
-
-// Split-K factor of the product-schedule variant (tiles of 128 x 256 outputs).
-int tc_nt_multi_splits(int K, int I, int J) {
-    const int tiles = (I / tc::BM) * (J / tc::BN);
-    const int blocks = (K + tc::BK - 1) / tc::BK;
-    int s = tc::sm_count() / (tiles > 0 ? tiles : 1);
-    if (s < 1) s = 1;
-    if (s > blocks) s = blocks;
-    if (s > 64) s = 64;
-    return s;
 }
 
 }  // namespace ssm

@@ -1,0 +1,215 @@
+// Weight gradients of fp32 layers: both products of a backward pass (gBbar = s^T u and dC = gy^T conj(x)) as sums of
+// products of bf16 planes, in one launch.
+//   part[s, i, j] = sum over the rows m of slice s of A[m, i] B[m, j],  A [K, I], B [K, J] as bf16 planes
+// Both operands are contiguous in the output index (MN-major tiles of [64 rows][64 columns]).  One CTA per 128 x 128
+// tile, slice of the rows and product: a k-block brings every plane of both operands in once (96 KB) and all six
+// products are issued from it; the kernel this replaces loaded a pair of planes per product (288 KB for a tile of
+// twice the size) and took one launch per product.  The last product (hi hi) has an accumulator of its own (see
+// gemm_tc_small.cu).  The tensor core truncates at every addition, so the error of a sum grows with the length of its
+// chain: after kNpSegment k-blocks the epilogue warps take the tile out of tensor memory and add it to their registers
+// while the next segment runs in the other half of tensor memory (64000 rows: dB 1.6e-5 off without).  Bound by operand delivery (96 KB per 1536 tensor-core cycles) on large problems, by the fixed
+// part of a launch on small ones.
+#include <algorithm>
+
+#include "kernels.h"
+#include "tcgen05.cuh"
+
+namespace ssm {
+namespace tc {
+
+constexpr int kNpTile = 128 * BK * 2;    // one plane of an operand tile of a k-block
+constexpr int kNpMaxStages = 4;
+constexpr int kNpSegment = 4;            // k-blocks per segment: 256 rows, 16 chained additions
+constexpr int kNpThreads = 64 + 256;     // producer, MMA, eight epilogue warps
+constexpr size_t kNpSmemMax = 220 * 1024;
+
+struct NtPlanesArgs {
+    int K, I, J, j_tiles, blocks_per_split;
+    int stages, stage_bytes;
+    int planes_a[2], planes_b[2], n_prod[2];
+    uint32_t pa[2], pb[2];
+    float* part[2];
+    WsHeader* hdr;
+};
+
+struct NtPlanesBars {
+    uint64_t full[kNpMaxStages], empty[kNpMaxStages], done[2], free[2];
+    uint32_t tmem;
+    int abort_flag;
+};
+
+__global__ void __launch_bounds__(kNpThreads, 1)
+gemm_tc_nt_planes_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
+                         const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1, NtPlanesArgs p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ NtPlanesBars bars;
+    uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    volatile int* abort_flag = &bars.abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, z = blockIdx.z;
+    const int i0 = ((int)blockIdx.x / p.j_tiles) * 128, j0 = ((int)blockIdx.x % p.j_tiles) * 128;
+    const int total = (p.K + BK - 1) / BK;
+    const int kb0 = (int)blockIdx.y * p.blocks_per_split, kb1 = min(total, kb0 + p.blocks_per_split);
+    const int planes_a = p.planes_a[z], planes_b = p.planes_b[z];
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < p.stages; ++i) {
+            mbar_init(smem_u32(&bars.full[i]), 1);
+            mbar_init(smem_u32(&bars.empty[i]), 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(smem_u32(&bars.done[i]), 1);
+            mbar_init(smem_u32(&bars.free[i]), 8);
+        }
+        bars.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        prefetch_tmap(z ? &tmA1 : &tmA0);
+        prefetch_tmap(z ? &tmB1 : &tmB0);
+    }
+    __syncwarp();
+    if (warp == 1) tmem_alloc(smem_u32(&bars.tmem), 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = bars.tmem;
+    grid_dep_wait();
+    grid_dep_launch();
+
+    if (warp == 0) {
+        if (lane == 0) {
+            const CUtensorMap *ta = z ? &tmA1 : &tmA0, *tb = z ? &tmB1 : &tmB0;
+            const uint32_t bytes = (uint32_t)(planes_a + planes_b) * kNpTile;
+            int stage = 0;
+            uint32_t phase = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
+                const uint32_t full = smem_u32(&bars.full[stage]);
+                uint32_t dst = smem_u32(tiles) + (uint32_t)stage * (uint32_t)p.stage_bytes;
+                mbar_expect_tx(full, bytes);
+                for (int q = 0; q < planes_a; ++q, dst += kNpTile) {
+                    tma_load_2d(dst, ta, full, q * p.I + i0, kb * BK);
+                    tma_load_2d(dst + kNpTile / 2, ta, full, q * p.I + i0 + 64, kb * BK);
+                }
+                for (int q = 0; q < planes_b; ++q, dst += kNpTile) {
+                    tma_load_2d(dst, tb, full, q * p.J + j0, kb * BK);
+                    tma_load_2d(dst + kNpTile / 2, tb, full, q * p.J + j0 + 64, kb * BK);
+                }
+                if (++stage == p.stages) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0 && kb0 < kb1) {
+            constexpr uint32_t idesc = instr_desc(128, 128, 1, 1);
+            const int n_prod = p.n_prod[z];
+            const uint32_t pa = p.pa[z], pb = p.pb[z];
+            int stage = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                const int seg = (kb - kb0) / kNpSegment, buf = seg & 1;
+                const bool seg_first = (kb - kb0) % kNpSegment == 0;
+                if (seg_first && seg >= 2) {   // the epilogue has taken segment seg - 2 out of this half of tensor memory
+                    if (!(ok = mbar_wait(smem_u32(&bars.free[buf]), (uint32_t)((seg >> 1) - 1) & 1u, abort_flag))) break;
+                    tc_fence_after();
+                }
+                if (!(ok = mbar_wait(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
+                tc_fence_after();
+                const uint32_t base = smem_u32(tiles) + (uint32_t)stage * (uint32_t)p.stage_bytes;
+                for (int j = 0; j < n_prod; ++j) {
+                    const bool small = j < n_prod - 1;
+                    const uint32_t d_tmem = tmem_base + 256u * (uint32_t)buf + (small ? 128u : 0u);
+                    const bool first = seg_first && (j == 0 || !small);
+                    const uint64_t ad = smem_desc_mnmajor(base + ((pa >> (4 * j)) & 15u) * kNpTile);
+                    const uint64_t bd = smem_desc_mnmajor(base + ((uint32_t)planes_a + ((pb >> (4 * j)) & 15u)) * kNpTile);
+#pragma unroll
+                    for (int k = 0; k < BK / UK; ++k)   // 16 rows of 128 bytes further: +128 in the address field
+                        umma_bf16(d_tmem, ad + (uint64_t)(128 * k), bd + (uint64_t)(128 * k), idesc, (uint32_t)!(first && k == 0));
+                }
+                umma_commit(smem_u32(&bars.empty[stage]));
+                if (kb + 1 == kb1 || (kb + 1 - kb0) % kNpSegment == 0) umma_commit(smem_u32(&bars.done[buf]));
+                if (++stage == p.stages) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
+            }
+        }
+    } else {
+        const int q = warp & 3, half = (warp - 2) >> 2;
+        const int row = i0 + q * 32 + lane;
+        float* dst = p.part[z] + ((size_t)blockIdx.y * p.I + row) * p.J + j0 + 64 * half;
+        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + 64u * (uint32_t)half;
+        float sum[64];
+#pragma unroll
+        for (int j = 0; j < 64; ++j) sum[j] = 0.f;
+        const int segs = (max(0, kb1 - kb0) + kNpSegment - 1) / kNpSegment;
+        bool ok = true;
+        for (int seg = 0; seg < segs; ++seg) {
+            const int buf = seg & 1;
+            if (!(ok = mbar_wait(smem_u32(&bars.done[buf]), (uint32_t)(seg >> 1) & 1u, abort_flag))) break;
+            tc_fence_after();
+#pragma unroll
+            for (int c = 0; c < 64; c += 32) {
+                uint32_t v[32], w[32];
+                tmem_ld32(t_row + 256u * (uint32_t)buf + (uint32_t)c, v);
+                tmem_ld32(t_row + 256u * (uint32_t)buf + 128u + (uint32_t)c, w);
+                tmem_ld_wait();
+#pragma unroll
+                for (int j = 0; j < 32; ++j) sum[c + j] += __uint_as_float(v[j]) + __uint_as_float(w[j]);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bars.free[buf]));
+        }
+        if (ok)
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                *reinterpret_cast<float4*>(dst + 4 * j) = make_float4(sum[4 * j], sum[4 * j + 1], sum[4 * j + 2], sum[4 * j + 3]);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 1) tmem_dealloc(tmem_base, 512);
+    if (threadIdx.x == 0 && *abort_flag && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
+}
+
+}  // namespace tc
+
+// Slices of the rows: as many as leave every SM at most one CTA of the launch.
+int tc_nt_planes_splits(int K, int I, int J) {
+    const int units = 2 * (I / 128) * (J / 128), blocks = (K + tc::BK - 1) / tc::BK;
+    return std::max(1, std::min(std::min(blocks, 64), device_sm_count() / std::max(units, 1)));
+}
+
+int launch_gemm_tc_nt_planes(const GemmTcNtPlanes& g, cudaStream_t st) {
+    using namespace tc;
+    if (g.I % 128 != 0 || g.J % 128 != 0) return SSM_ERR_SHAPE;
+    NtPlanesArgs p{};
+    p.K = g.K, p.I = g.I, p.J = g.J, p.j_tiles = g.J / 128, p.hdr = g.hdr;
+    const int blocks = (g.K + BK - 1) / BK;
+    p.blocks_per_split = (blocks + g.splits - 1) / g.splits;
+    CUtensorMap ma[2], mb[2];
+    int planes = 0;
+    for (int z = 0; z < 2; ++z) {
+        const GemmTcNtPlanes::Product& q = g.product[z];
+        if (q.n_products < 2 || q.n_products > 8) return SSM_ERR_SHAPE;
+        p.planes_a[z] = q.planes_a, p.planes_b[z] = q.planes_b, p.n_prod[z] = q.n_products;
+        p.pa[z] = q.prod_a, p.pb[z] = q.prod_b, p.part[z] = q.part;
+        planes = std::max(planes, q.planes_a + q.planes_b);
+        if (!make_map(&ma[z], q.A, (uint64_t)g.K, (uint64_t)g.I * q.planes_a, 64, BK)) return SSM_ERR_CUDA;
+        if (!make_map(&mb[z], q.B, (uint64_t)g.K, (uint64_t)g.J * q.planes_b, 64, BK)) return SSM_ERR_CUDA;
+    }
+    p.stage_bytes = planes * kNpTile;
+    p.stages = std::min<int>(kNpMaxStages, (int)((kNpSmemMax - 1024) / p.stage_bytes));
+    if (p.stages < 2) return SSM_ERR_SHAPE;
+    if (!set_max_dynamic_smem(reinterpret_cast<const void*>(gemm_tc_nt_planes_kernel), kNpSmemMax)) return SSM_ERR_CUDA;
+    count_launch();
+    const dim3 grid((unsigned)((g.I / 128) * p.j_tiles), (unsigned)g.splits, 2);
+    return launch_dep(gemm_tc_nt_planes_kernel, grid, kNpThreads, (size_t)p.stages * p.stage_bytes + 1024, st, ma[0], mb[0], ma[1],
+                      mb[1], p)
+               ? SSM_OK
+               : SSM_ERR_CUDA;
+}
+
+}  // namespace ssm

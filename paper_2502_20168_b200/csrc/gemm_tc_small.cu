@@ -37,6 +37,7 @@ struct SmallTnArgs {
     uint32_t prod_a, prod_w;   // product j: plane (prod_a >> 4 j) & 15 of A, (prod_w >> 4 j) & 15 of W
     int a_plane, w_plane_cols, w_plane_rows, w_stacked;   // where the planes lie (w_stacked: hi / lo blocks of 128 rows)
     const float* a_f32;        // A as fp32 [M, K] (planes made here), or NULL: bf16 planes by TMA
+    __nv_bfloat16* a_planes;   // or NULL: the planes made here also go to memory (by the CTAs of the first column tile)
     int K;
     // epilogue
     void* out;
@@ -159,7 +160,7 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             uint32_t phase = 0;
             for (int kb = kb0; kb < kb1; ++kb) {
                 if (!mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
-                sp.store(tiles + (size_t)stage * p.stage_bytes, p.M, m0, te);
+                sp.store(tiles + (size_t)stage * p.stage_bytes, p.M, m0, te, n0 == 0 ? p.a_planes : nullptr, p.K, kb);
                 if (kb + 1 < kb1) sp.fetch(p.a_f32, p.K, p.M, m0, kb + 1, te);
                 fence_async_smem();
                 __syncwarp();
@@ -389,6 +390,7 @@ int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st) {
     }
     p.a_plane = g.K;
     p.a_f32 = g.a_f32 ? reinterpret_cast<const float*>(g.A) : nullptr;
+    p.a_planes = reinterpret_cast<__nv_bfloat16*>(g.a_planes_out);
     if (g.a_f32 && p.planes_a != 3) return SSM_ERR_SHAPE;
     p.out = g.out, p.diag = g.diag, p.skip = g.skip, p.dot = g.dot, p.add = g.add;
     p.dot_part = g.dot_part, p.gate_out = reinterpret_cast<__nv_bfloat16*>(g.gate_out);

@@ -129,7 +129,8 @@ struct GemmTcTN {
     int n_products = 0, planes_a = 1, planes_w = 1;
     uint32_t prod_a = 0, prod_w = 0;
     // Only where tc_tn_small says so (the kernel for problems of few tiles):
-    bool a_f32 = false;                  // A is fp32 [M, K]; its three planes are made on the way to the tensor cores
+    bool a_f32 = false;                  // A is fp32 [M, K]; its three planes are made on the way to the tensor cores ...
+    void* a_planes_out = nullptr;        // ... and, if asked for, stored [M, 3K] for a later kernel
     bool skip_bf16 = true, dot_bf16 = true;   // types of skip and dot; with diag and store_f32 the result is fp32
     const float* add = nullptr;          // fp32 [M, N_out], added to acc + diag * skip
     int w_plane_rows = 0;                // planes of W this many rows apart in blocks of 128 rows (as with split_w) ...
@@ -223,12 +224,21 @@ struct GemmTcNT {
     float* part;
     WsHeader* hdr;
     int lda = 0;   // elements between rows of A when A is a column block of a wider matrix (0: I)
-    // Product schedule (see GemmTcTN): A = planes_a planes of I columns, Bm_hi = planes_b planes of J columns
-    // (Bm_lo unused), J a multiple of 256; splits from tc_nt_multi_splits.
-    int n_products = 0, planes_a = 1, planes_b = 1;
-    uint32_t prod_a = 0, prod_b = 0;
 };
-int tc_nt_multi_splits(int K, int I, int J);
+// Both weight-gradient products of an fp32 layer from planes (gemm_tc_nt_planes.cu): A = planes_a planes of I columns
+// side by side, B = planes_b planes of J columns; product schedules as in GemmTcTN.  I and J multiples of 128.
+struct GemmTcNtPlanes {
+    int K, I, J, splits;
+    struct Product {
+        const void *A, *B;
+        int planes_a, planes_b, n_products;
+        uint32_t prod_a, prod_b;
+        float* part;   // [splits, I, J]
+    } product[2];
+    WsHeader* hdr;
+};
+int tc_nt_planes_splits(int K, int I, int J);
+int launch_gemm_tc_nt_planes(const GemmTcNtPlanes& g, cudaStream_t st);
 bool tc_nt_supported(int I, int J);
 int tc_nt_splits(int K, int I, int J);
 int launch_gemm_tc_nt(const GemmTcNT& g, cudaStream_t st);

@@ -84,7 +84,9 @@ struct SplitA {
             }
         }
     }
-    __device__ __forceinline__ void store(uint8_t* dst, int M, int m0, int te) const {
+    // `planes` (may be NULL): the three planes also go to [M, 3K] in global memory.
+    __device__ __forceinline__ void store(uint8_t* dst, int M, int m0, int te, __nv_bfloat16* planes = nullptr, int K = 0,
+                                          int kb = 0) const {
 #pragma unroll
         for (int i = 0; i < kC; ++i) {
             const int r = (te >> 3) + kStep * i;
@@ -95,6 +97,12 @@ struct SplitA {
             *reinterpret_cast<uint4*>(q) = hi;
             *reinterpret_cast<uint4*>(q + kSmATile) = mid;
             *reinterpret_cast<uint4*>(q + 2 * kSmATile) = lo;
+            if (planes) {
+                __nv_bfloat16* g = planes + (size_t)(m0 + r) * 3 * K + kb * BK + 8 * (te & 7);
+                *reinterpret_cast<uint4*>(g) = hi;
+                *reinterpret_cast<uint4*>(g + K) = mid;
+                *reinterpret_cast<uint4*>(g + 2 * (size_t)K) = lo;
+            }
         }
     }
 };
