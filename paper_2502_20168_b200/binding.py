@@ -116,6 +116,8 @@ def _load() -> ctypes.CDLL:
 
 
 _lib = _load()
+_raw_stream = torch._C._cuda_getCurrentRawStream
+_current_device = torch.cuda.current_device
 
 
 def lib() -> ctypes.CDLL:
@@ -135,20 +137,21 @@ def make_shape(B: int, T: int, H: int, P: int, io_dtype) -> ssm_shape:
 
 
 def _ptr(t):
+    """Device pointer of a tensor as a plain int (ctypes converts it; making c_void_p objects cost as much as the rest)."""
     if t is None:
-        return c_void_p(0)
+        return None
     if isinstance(t, int):
-        return c_void_p(t)
+        return t
     if not t.is_cuda:
         raise ValueError("expected a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError("expected a contiguous tensor")
-    return c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return c_void_p(s.cuda_stream)
+    # the raw handle: torch.cuda.current_stream() builds a Stream object on every call
+    return _raw_stream(_current_device()) if stream is None else stream.cuda_stream
 
 
 def _nbytes(t) -> int:
@@ -259,7 +262,7 @@ def _struct_array(cls, dicts):
     arr = (cls * len(dicts))()
     for i, d in enumerate(dicts):
         for name, _ in cls._fields_:
-            setattr(arr[i], name, _ptr(d[name]).value)
+            setattr(arr[i], name, _ptr(d[name]))
     return arr
 
 

@@ -59,7 +59,7 @@ int launch_scan_bwd(int B, int T, int P, const float2* Abar, const float2* Alo, 
 bool scan_stream_supported(int B, int T, int P);
 int launch_scan_fwd_stream(int B, int T, int P, const float2* Abar, const float2* Alo, const float2* Bu,
                            const uint8_t* done, const float2* x0, void* x, bool x_bf16, float2* xT, WsHeader* hdr,
-                           int* ticket, cudaStream_t st);
+                           cudaStream_t st);
 int launch_scan_bwd_stream(int B, int T, int P, const float2* Abar, const float2* Alo, const uint8_t* done,
                            const float2* x0, const void* x, bool x_bf16, const float2* gx, const float2* gxT,
                            void* gBu, float2* gx0, float2* part, WsHeader* hdr, int* ticket, cudaStream_t st);

@@ -274,14 +274,8 @@ scan_fwd_step_kernel(int B, int P2, const float4* Abar, const float4* Alo,
 // =============================================================================================
 // Host side
 // =============================================================================================
-// Scratch layout: [counter of the streaming kernels (256 B)][gAbar partials: B rows of P float2]
-// [column-sum scratch].
+// Scratch layout: [work counter (256 B)][gAbar partials: B rows of P float2][column-sum scratch].
 namespace {
-
-struct ScanCounters {
-    int ticket;
-    int pad[63];
-};
 
 struct ScanPlan {
     size_t off_part, off_tmp, total;
@@ -290,7 +284,7 @@ struct ScanPlan {
 // rows_per_seq: rows of partial sums per sequence (2 for the kernel that puts both CTAs of a pair on one sequence)
 ScanPlan plan_scan(int B, int P, int rows_per_seq = 1) {
     ScanPlan s{};
-    size_t off = sizeof(ScanCounters);
+    size_t off = 256;
     s.off_part = off;
     off += align_up((size_t)rows_per_seq * B * P * 8, 256);
     s.off_tmp = off;
@@ -327,8 +321,7 @@ int launch_scan_fwd(int B, int T, int P, const float2* Abar, const float2* Alo, 
         return SSM_OK;
     }
     if (use_stream(B, T, P))
-        return launch_scan_fwd_stream(B, T, P, Abar, Alo, Bu, done, x0, x, x_bf16, xT, hdr,
-                                      &reinterpret_cast<ScanCounters*>(scratch)->ticket, st);
+        return launch_scan_fwd_stream(B, T, P, Abar, Alo, Bu, done, x0, x, x_bf16, xT, hdr, st);
     const int P2 = P / 2;
     const int blocks = (int)(((size_t)B * P2 + kSeqThreads - 1) / kSeqThreads);
     count_launch();
@@ -352,7 +345,7 @@ int launch_scan_bwd(int B, int T, int P, const float2* Abar, const float2* Alo, 
     if (x_bf16 != s_bf16) return SSM_ERR_DTYPE;
     if (use_stream(B, T, P)) {
         const int err = launch_scan_bwd_stream(B, T, P, Abar, Alo, done, x0, x, x_bf16, gx, gxT, gBu, gx0, (float2*)part,
-                                               hdr, &reinterpret_cast<ScanCounters*>(scratch)->ticket, st);
+                                               hdr, reinterpret_cast<int*>(scratch), st);
         if (err != SSM_OK) return err;
     } else {
         count_launch();

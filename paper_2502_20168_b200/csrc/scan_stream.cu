@@ -3,8 +3,8 @@
 // parallelism over time stays inside one CTA.
 //
 // A chain is one sequence b and a group of G neighbouring states (G = 16..128, chosen so that
-// there are enough chains to fill the machine).  A persistent CTA takes chains from an atomic
-// counter and walks each one from its first step to its last (the adjoint: last to first) in
+// there are enough chains to fill the machine).  A persistent CTA takes every gridDim.x-th chain (all
+// chains are equally long; the adjoint of many chains: the next one from a counter) and walks each one from its first step to its last (the adjoint: last to first) in
 // tiles of R rows x G states.  The 256 scanning threads of the CTA are `slices` = 256 / G
 // groups of G; group q owns rows [q r, (q + 1) r) of the tile (r = kRows) and one thread owns
 // one state there.  Per tile:
@@ -50,7 +50,7 @@ struct Args {
     const float2* Abar;
     const float2* Alo;   // low part of Abar as an fp32 pair, or NULL
     const uint8_t* done;
-    int* ticket;
+    int* ticket;         // counter the chains are taken from, or NULL: every gridDim.x-th
     WsHeader* hdr;
 };
 
@@ -132,7 +132,7 @@ __device__ __forceinline__ void init_shared(Shared& sm) {
     __syncthreads();
 }
 
-// Producer warp: chains from the counter; per tile the done flags and up to three TMA loads
+// Producer warp: this CTA's chains; per tile the done flags and up to three TMA loads
 // (m1 / m2, the states of the adjoint, start one row earlier).
 template <bool kBwd>
 __device__ __forceinline__ void producer(const Args& k, Shared& sm, uint8_t* stages, uint32_t stage_bytes,
@@ -140,10 +140,11 @@ __device__ __forceinline__ void producer(const Args& k, Shared& sm, uint8_t* sta
                                          uint32_t bytes0, uint32_t bytes1, uint32_t bytes2) {
     const int lane = threadIdx.x & 31;
     int s = 0, round = 0;   // stage of the next tile; how many times the ring has wrapped
-    for (;;) {
-        int chain = 0;
-        if (lane == 0) chain = atomicAdd(k.ticket, 1);
-        chain = __shfl_sync(0xffffffffu, chain, 0);
+    for (int chain = blockIdx.x;; chain += gridDim.x) {
+        if (kBwd && k.ticket) {
+            if (lane == 0) chain = atomicAdd(k.ticket, 1);
+            chain = __shfl_sync(0xffffffffu, chain, 0);
+        }
         const bool end = chain >= k.nchains;
         const int tiles = end ? 1 : k.ntiles;
         for (int j = 0; j < tiles; ++j, s = (s + 1 == k.stages) ? 0 : s + 1, round += (s == 0)) {
@@ -530,7 +531,7 @@ bool make_map3(CUtensorMap* map, const void* base, bool bf16, int B, int T, int 
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-Args make_args(int B, int T, int P, int rows, bool forward, const float2* Abar, const float2* Alo, const uint8_t* done, int* ticket,
+Args make_args(int B, int T, int P, int rows, bool forward, const float2* Abar, const float2* Alo, const uint8_t* done,
                WsHeader* hdr) {
     Args k{};
     k.B = B;
@@ -573,7 +574,6 @@ Args make_args(int B, int T, int P, int rows, bool forward, const float2* Abar, 
     k.Abar = Abar;
     k.Alo = Alo;
     k.done = done;
-    k.ticket = ticket;
     k.hdr = hdr;
     return k;
 }
@@ -594,9 +594,9 @@ bool scan_stream_supported(int B, int T, int P) {
 
 int launch_scan_fwd_stream(int B, int T, int P, const float2* Abar, const float2* Alo, const float2* Bu,
                            const uint8_t* done, const float2* x0, void* x, bool x_bf16, float2* xT, WsHeader* hdr,
-                           int* ticket, cudaStream_t st) {
+                           cudaStream_t st) {
     using namespace stream;
-    const Args k = make_args(B, T, P, kFwdRows, true, Abar, Alo, done, ticket, hdr);
+    const Args k = make_args(B, T, P, kFwdRows, true, Abar, Alo, done, hdr);
     const size_t smem = (size_t)k.stages * k.R * k.G * 8 + 128;
     const int grid = k.nchains < kCtasPerSm * sm_count() ? k.nchains : kCtasPerSm * sm_count();
     const size_t plane_bytes = (size_t)B * T * P * 4;
@@ -605,7 +605,6 @@ int launch_scan_fwd_stream(int B, int T, int P, const float2* Abar, const float2
     if (!make_map3(&o0, x, x_bf16, B, T, P, k.G, k.R)) return SSM_ERR_CUDA;
     o1 = o0;
     if (x_bf16 && !make_map3(&o1, (const char*)x + plane_bytes, true, B, T, P, k.G, k.R)) return SSM_ERR_CUDA;
-    if (cudaMemsetAsync(ticket, 0, sizeof(int), st) != cudaSuccess) return SSM_ERR_CUDA;
     count_launch();
 #define SSM_LAUNCH_G(GG, XS, PAIR)                                                      \
     do {                                                                                \
@@ -636,9 +635,17 @@ int launch_scan_bwd_stream(int B, int T, int P, const float2* Abar, const float2
                            void* gBu, float2* gx0, float2* part, WsHeader* hdr, int* ticket, cudaStream_t st) {
     using namespace stream;
     const bool tall = T >= kBwdLongT;
-    const Args k = make_args(B, T, P, tall ? kBwdRowsLong : kBwdRows, false, Abar, Alo, done, ticket, hdr);
+    Args k = make_args(B, T, P, tall ? kBwdRowsLong : kBwdRows, false, Abar, Alo, done, hdr);
     const size_t smem = (size_t)k.stages * 2 * k.R * k.G * 8 + 128;
     const int grid = k.nchains < kCtasPerSm * sm_count() ? k.nchains : kCtasPerSm * sm_count();
+    // From three rounds of chains on they are dealt out by a counter: the CTAs of the adjoint run at different speeds
+    // (256 x 1024, P = 256: 259 us, 285 with every gridDim.x-th chain; 4096 x 64: 250 / 273).  Up to two rounds the
+    // counter's memset and atomics cost more than they balance (150 x 200, P = 192: 41 / 35).  The forward scan is equal or
+    // faster without at every size (64 x 4096: 189 / 183).
+    if (k.nchains > 2 * grid) {
+        if (cudaMemsetAsync(ticket, 0, sizeof(int), st) != cudaSuccess) return SSM_ERR_CUDA;
+        k.ticket = ticket;
+    }
     const size_t plane_bytes = (size_t)B * T * P * 4;
     CUtensorMap mg, x0m, x1m, o0, o1;
     if (!make_map3(&mg, gx, false, B, T, P, k.G, k.R)) return SSM_ERR_CUDA;
@@ -650,7 +657,6 @@ int launch_scan_bwd_stream(int B, int T, int P, const float2* Abar, const float2
         if (!make_map3(&x1m, (const char*)x + plane_bytes, true, B, T, P, k.G, k.R)) return SSM_ERR_CUDA;
         if (!make_map3(&o1, (const char*)gBu + plane_bytes, true, B, T, P, k.G, k.R)) return SSM_ERR_CUDA;
     }
-    if (cudaMemsetAsync(ticket, 0, sizeof(int), st) != cudaSuccess) return SSM_ERR_CUDA;
     count_launch();
 #define SSM_LAUNCH_G(GG, XS, PAIR)                                                                 \
     do {                                                                                           \
