@@ -37,6 +37,8 @@ bool planes_supported(const ssm_shape& s) {
 constexpr uint32_t kProd6A = 0x001102u, kProd6B = 0x010120u;
 constexpr uint32_t kProd3A = 0x000u, kProd3B = 0x012u;
 
+constexpr int kMaxStackLayers = 64;
+
 size_t take(size_t& off, size_t bytes) {
     const size_t at = off;
     off = align_up(off + bytes, 256);
@@ -51,7 +53,7 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true) {
     p.tc = allow_tc && s.io_dtype == SSM_BF16 && tc_tn_supported((int)BT, P2, s.H, true) &&
            tc_tn_supported((int)BT, s.H, P2, false) && tc_nt_supported(s.H, P2);
     p.planes = !p.tc && s.io_dtype == SSM_F32 && planes_supported(s);
-    p.splits = p.tc ? tc_nt_splits((int)BT, s.H, P2) : (p.planes ? tc_nt_planes_splits((int)BT, s.H, P2) : gemm_nt_splits((int)BT));
+    p.splits = p.tc ? tc_nt_splits((int)BT, s.H, P2) : (p.planes ? tc_nt_planes_splits((int)BT, s.H, P2, 2) : gemm_nt_splits((int)BT));
     p.hdr = take(off, sizeof(WsHeader));
     p.Abar = take(off, (size_t)s.P * 8);
     p.Alo = take(off, (size_t)s.P * 8);
@@ -220,19 +222,21 @@ SSM_API int ssm_layer_plan_string(const ssm_shape* shape, char* buf, size_t len)
 }
 
 // Discretised parameters and packed projection operands into the workspace; clears the status word of `hdr` if given.
+static PackJob pack_job(const LayerPlan& p, const ssm_c64* Lambda, const float* Delta, const ssm_c64* Bc, const ssm_c64* Cc,
+                        void* ws) {
+    return {(const float2*)Lambda, Delta, (const float2*)Bc, (const float2*)Cc, at<float2>(ws, p.Abar), at<float2>(ws, p.Alo),
+            at<void>(ws, p.W0), at<void>(ws, p.W1), at<void>(ws, p.W2), at<void>(ws, p.W3)};
+}
 static void layer_prepare(const ssm_shape& s, const LayerPlan& p, const ssm_c64* Lambda, const float* Delta,
                           const ssm_c64* Bc, const ssm_c64* Cc, void* ws, WsHeader* hdr, cudaStream_t st) {
     StageTimer tm("discretize_pack", st);
-    const float2 *L = (const float2*)Lambda, *B = (const float2*)Bc, *C = (const float2*)Cc;
-    float2 *Abar = at<float2>(ws, p.Abar), *Alo = at<float2>(ws, p.Alo);
-    void *W0 = at<void>(ws, p.W0), *W1 = at<void>(ws, p.W1), *W2 = at<void>(ws, p.W2), *W3 = at<void>(ws, p.W3);
+    const PackJob job = pack_job(p, Lambda, Delta, Bc, Cc, ws);
     if (p.tc)   // (the kernels that scan in the epilogue of a projection want their own column order)
-        launch_discretize_pack_tc(s.H, s.P, tc_gemm_scan_group(s.B, s.T, s.H, s.P), L, Delta, B, C, Abar, Alo, W0, W1, W2, W3,
-                                  hdr, st);
+        launch_discretize_pack_tc(s.H, s.P, tc_gemm_scan_group(s.B, s.T, s.H, s.P), job, hdr, st);
     else if (p.planes)
-        launch_discretize_pack_planes(s.H, s.P, L, Delta, B, C, Abar, Alo, W0, W1, W2, W3, hdr, st);
+        launch_discretize_pack_planes(s.H, s.P, 1, &job, hdr, st);
     else
-        launch_discretize_pack_f32(s.H, s.P, L, Delta, B, C, Abar, Alo, W0, W1, W2, W3, hdr, st);
+        launch_discretize_pack_f32(s.H, s.P, 1, &job, hdr, st);
 }
 
 // Launch sequence of one layer's forward pass from a prepared workspace.  `hdr` receives the
@@ -352,8 +356,8 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
 static int layer_fwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo& io, const ssm_c64* Lambda,
                           const float* Delta, const ssm_c64* Bc, const ssm_c64* Cc, const float* D, const void* u,
                           const uint8_t* done, const ssm_c64* x0, void* y, ssm_c64* xT, void* ws, WsHeader* hdr,
-                          bool clear_hdr, cudaStream_t st) {
-    layer_prepare(s, p, Lambda, Delta, Bc, Cc, ws, clear_hdr ? hdr : nullptr, st);
+                          cudaStream_t st) {
+    layer_prepare(s, p, Lambda, Delta, Bc, Cc, ws, hdr, st);
     return layer_fwd_run(s, p, io, D, u, done, x0, y, xT, ws, hdr, true, st);
 }
 
@@ -370,7 +374,7 @@ SSM_API int ssm_layer_fwd(const ssm_shape* shape, const ssm_c64* Lambda, const f
     if (int rc = check_ws(ws, ws_bytes, p.total)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     WsHeader* hdr = at<WsHeader>(ws, p.hdr);
-    return layer_fwd_impl(s, p, layer_io(s), Lambda, Delta, Bc, Cc, D, u, done, x0, y, xT, ws, hdr, true, st);
+    return layer_fwd_impl(s, p, layer_io(s), Lambda, Delta, Bc, Cc, D, u, done, x0, y, xT, ws, hdr, st);
 }
 
 // Single-step mode: the layer's forward launch sequence for T = 1 from operands prepared once.
@@ -559,13 +563,20 @@ SSM_API int ssm_glu_bwd(const ssm_shape* shape, const float* W, const void* v, c
     return SSM_OK;
 }
 
-// Launch sequence of one layer's backward pass.  du_add (fp32 [B,T,H], may be NULL) is added to du
-// before it is stored (the gradient of the residual branch of a stacked model).
+// What a layer's backward pass leaves for its last kernels, which a stack runs for all its layers together.
+struct LayerTail {
+    GradTail tail;
+    GemmTcNtPlanes products[2];   // plane path: the weight-gradient products, not launched yet
+    int gA_rows;
+};
+
+// Launch sequence of one layer's backward pass, all but its last kernels (layer_bwd_tail).  du_add (fp32 [B,T,H], may
+// be NULL) is added to du before it is stored (the gradient of the residual branch of a stacked model).
 static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo& io, const ssm_c64* Lambda,
                           const float* Delta, const ssm_c64* Bc, const float* D, const void* u, const uint8_t* done,
                           const ssm_c64* x0, const void* gy, const ssm_c64* gxT, const float* du_add, void* ws,
                           WsHeader* hdr, void* du, ssm_c64* dLambda, float* dDelta, ssm_c64* dB, ssm_c64* dC, float* dD,
-                          ssm_c64* dx0, cudaStream_t st) {
+                          ssm_c64* dx0, LayerTail* left, cudaStream_t st) {
     const int BT = s.B * s.T, P2 = 2 * s.P;
     if (p.tc && !(io.u_bf16 && io.gy_bf16 && io.du_bf16)) return SSM_ERR_DTYPE;
     float* part = at<float>(ws, p.part);                       // split-K partials of gBbar ...
@@ -671,16 +682,11 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
             if (!small) launch_diag_skip(at<float>(ws, p.acc), D, gy, gyb, du_add, (size_t)BT, s.H, du, io.du_bf16, st);
         }
-        {   // gBbar = s^T u and dC = gy^T conj(x)
-            StageTimer tm("gemm_gBbar_gC", st);
-            const GemmTcNtPlanes g{
-                BT, s.H, P2, p.splits,
-                {{ub ? u : at<void>(ws, p.u3), at<void>(ws, p.s3), ub ? 1 : 3, 3, ub ? 3 : 6, ub ? kProd3A : kProd6A, ub ? kProd3B : kProd6B, part},
-                 {gyb ? gy : at<void>(ws, p.gy3), at<void>(ws, p.x3), gyb ? 1 : 3, 3, gyb ? 3 : 6, gyb ? kProd3A : kProd6A,
-                  gyb ? kProd3B : kProd6B, part_c}},
-                hdr};
-            if ((rc = launch_gemm_tc_nt_planes(g, st))) return rc;
-        }
+        // gBbar = s^T u and dC = gy^T conj(x)
+        left->products[0] = {ub ? u : at<void>(ws, p.u3), at<void>(ws, p.s3), ub ? 1 : 3, 3, ub ? 3 : 6, ub ? kProd3A : kProd6A,
+                             ub ? kProd3B : kProd6B, part};
+        left->products[1] = {gyb ? gy : at<void>(ws, p.gy3), at<void>(ws, p.x3), gyb ? 1 : 3, 3, gyb ? 3 : 6,
+                             gyb ? kProd3A : kProd6A, gyb ? kProd3B : kProd6B, part_c};
     } else {
         {
             StageTimer tm("gemm_gx", st);
@@ -713,19 +719,37 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
             launch_gemm_nt(g6, st);
         }
     }
-    {   // dD[h] = sum_m gy[m,h] u[m,h] (unless the du projection left its partial sums already), the two split-K
-        // sums, then the adjoint of the discretisation with the sums of gAbar and dD folded in
-        StageTimer tm("gD_and_discretize_bwd", st);
-        if (!dD_part) {
-            float* tmp = at<float>(ws, p.dot);
-            int groups = launch_dot_columns_partial(io.gy_bf16, gy, io.u_bf16, u, BT, s.H, tmp, st);
-            dD_part = launch_reduce_rows(tmp, groups, s.H, tmp + (size_t)groups * s.H, kMaxPartialRows, &dD_rows, st);
-        }
-        launch_reduce_weight_grads(s.H, s.P, p.splits, part, part_c, (const float2*)Lambda, Delta, (const float2*)Bc,
-                                   (float2*)dB, (float2*)dC, at<float2>(ws, p.gg), st);
-        launch_layer_finalize(s.H, s.P, (const float2*)Lambda, Delta, gA_part, gA_rows, at<float2>(ws, p.gg),
-                              (float2*)dLambda, dDelta, dD_part, dD_rows, dD, st);
+    if (!dD_part) {   // dD[h] = sum_m gy[m,h] u[m,h], unless the du projection left its partial sums already
+        StageTimer tm("dot_gy_u", st);
+        float* tmp = at<float>(ws, p.dot);
+        int groups = launch_dot_columns_partial(io.gy_bf16, gy, io.u_bf16, u, BT, s.H, tmp, st);
+        dD_part = launch_reduce_rows(tmp, groups, s.H, tmp + (size_t)groups * s.H, kMaxPartialRows, &dD_rows, st);
     }
+    left->gA_rows = gA_rows;
+    left->tail = {(const float2*)Lambda, Delta, (const float2*)Bc, part, part_c, (float2*)dB, (float2*)dC, at<float2>(ws, p.gg),
+                  gA_part, (float2*)dLambda, dDelta, {dD_part, nullptr, nullptr}, {dD_rows, 0, 0}, {dD, nullptr, nullptr}};
+    SSM_RETURN_IF_CUDA_ERROR();
+    return SSM_OK;
+}
+
+// The weight-gradient products of the plane path, the sums over split-K partials and the adjoint of the discretisation
+// (with the sums of gAbar, dD and a stack's LayerNorm parameters) of n layers of one shape.
+static int layer_bwd_tail(const ssm_shape& s, const LayerPlan& p, int n, const LayerTail* left, WsHeader* hdr, cudaStream_t st) {
+    GemmTcNtPlanes products[2 * kMaxStackLayers];
+    GradTail tails[kMaxStackLayers];
+    for (int l = 0; l < n; ++l) {
+        products[2 * l] = left[l].products[0];
+        products[2 * l + 1] = left[l].products[1];
+        tails[l] = left[l].tail;
+    }
+    int splits = p.splits;
+    if (p.planes) {
+        StageTimer tm("gemm_gBbar_gC", st);
+        splits = std::min(splits, tc_nt_planes_splits(s.B * s.T, s.H, 2 * s.P, 2 * n));
+        if (int rc = launch_gemm_tc_nt_planes(s.B * s.T, s.H, 2 * s.P, splits, 2 * n, products, hdr, st)) return rc;
+    }
+    StageTimer tm("gD_and_discretize_bwd", st);
+    launch_layer_tail(s.H, s.P, splits, n, tails, left[0].gA_rows, st);
     SSM_RETURN_IF_CUDA_ERROR();
     return SSM_OK;
 }
@@ -747,8 +771,11 @@ SSM_API int ssm_layer_bwd(const ssm_shape* shape, const ssm_c64* Lambda, const f
     if (int rc = check_ws(ws, ws_bytes, p.total)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     WsHeader* hdr = at<WsHeader>(ws, p.hdr);
-    return layer_bwd_impl(s, p, layer_io(s), Lambda, Delta, Bc, D, u, done, x0, gy, gxT, nullptr, ws, hdr, du, dLambda,
-                          dDelta, dB, dC, dD, dx0, st);
+    LayerTail left{};
+    if (int rc = layer_bwd_impl(s, p, layer_io(s), Lambda, Delta, Bc, D, u, done, x0, gy, gxT, nullptr, ws, hdr, du, dLambda,
+                                dDelta, dB, dC, dD, dx0, &left, st))
+        return rc;
+    return layer_bwd_tail(s, p, 1, &left, hdr, st);
 }
 
 // ---- stacked model -----------------------------------------------------------------------------
@@ -764,7 +791,7 @@ namespace {
 struct StackPlan {
     size_t layer_ws;   // bytes of one layer workspace
     size_t act;        // bytes of one fp32 [B,T,H] tensor
-    size_t hdr, layers, acts, vs, stats, gz, gv, g0, g1, tmp, total;
+    size_t hdr, layers, acts, vs, stats, gz, gv, g0, g1, tmp, tmp_stride, total;
 };
 
 ssm_shape stack_layer_shape(const ssm_shape& s) {
@@ -788,14 +815,15 @@ StackPlan plan_stack(const ssm_shape& s, int L) {
     p.gv = take(off, p.act);
     p.g0 = take(off, p.act);
     p.g1 = take(off, p.act);
-    p.tmp = take(off, stack_tmp_floats((int)BT, s.H) * 4);
+    p.tmp_stride = align_up(stack_tmp_floats((int)BT, s.H) * 4, 256);
+    p.tmp = take(off, p.tmp_stride * L);
     p.total = off;
     return p;
 }
 
 int check_stack_args(const ssm_shape* shape, int n_layers, const ssm_stack_params* params) {
     if (int rc = check_shape(shape)) return rc;
-    if (n_layers < 1 || n_layers > 64) return SSM_ERR_SHAPE;
+    if (n_layers < 1 || n_layers > kMaxStackLayers) return SSM_ERR_SHAPE;
     if (!params) return SSM_ERR_NULL;
     for (int l = 0; l < n_layers; ++l) {
         const ssm_stack_params& q = params[l];
@@ -810,7 +838,7 @@ int check_stack_args(const ssm_shape* shape, int n_layers, const ssm_stack_param
 }  // namespace
 
 SSM_API size_t ssm_stack_workspace_bytes(const ssm_shape* shape, int n_layers) {
-    if (check_shape(shape) != SSM_OK || n_layers < 1 || n_layers > 64) return 0;
+    if (check_shape(shape) != SSM_OK || n_layers < 1 || n_layers > kMaxStackLayers) return 0;
     return plan_stack(*shape, n_layers).total;
 }
 
@@ -829,6 +857,14 @@ SSM_API int ssm_stack_fwd(const ssm_shape* shape, int n_layers, const ssm_stack_
     const int BT = s.B * s.T;
     const size_t stat = align_up((size_t)BT * 4, 256);
     WsHeader* hdr = at<WsHeader>(ws, sp.hdr);
+    {   // the parameters of all layers in one launch
+        StageTimer tm("discretize_pack", st);
+        PackJob jobs[kMaxStackLayers];
+        for (int l = 0; l < n_layers; ++l)
+            jobs[l] = pack_job(lp, params[l].Lambda, params[l].Delta, params[l].Bc, params[l].Cc, at<void>(ws, sp.layers + sp.layer_ws * l));
+        if (lp.planes) launch_discretize_pack_planes(ls.H, ls.P, n_layers, jobs, hdr, st);
+        else launch_discretize_pack_f32(ls.H, ls.P, n_layers, jobs, hdr, st);
+    }
     const void* in = u;
     for (int l = 0; l < n_layers; ++l) {
         const ssm_stack_params& q = params[l];
@@ -837,7 +873,7 @@ SSM_API int ssm_stack_fwd(const ssm_shape* shape, int n_layers, const ssm_stack_
         float* v = at<float>(ws, sp.vs + sp.act * l);
         void* o = last ? out : at<void>(ws, sp.acts + sp.act * l);
         const LayerIo io{first && bf16, false, false, false};
-        if (int rc = layer_fwd_impl(ls, lp, io, q.Lambda, q.Delta, q.Bc, q.Cc, q.D, in, done, nullptr, v, nullptr, lws, hdr, first, st))
+        if (int rc = layer_fwd_run(ls, lp, io, q.D, in, done, nullptr, v, nullptr, lws, hdr, true, st))
             return rc;
         StageTimer tm("stack_gelu_ln_fwd", st);
         launch_stack_fwd(first && bf16, last && bf16, BT, s.H, in, v, q.ln_weight, q.ln_bias, o,
@@ -872,6 +908,7 @@ SSM_API int ssm_stack_bwd(const ssm_shape* shape, int n_layers, const ssm_stack_
     const size_t stat = align_up((size_t)BT * 4, 256);
     WsHeader* hdr = at<WsHeader>(ws, sp.hdr);
     const void* g = gout;
+    LayerTail left[kMaxStackLayers] = {};
     for (int l = n_layers - 1; l >= 0; --l) {
         const ssm_stack_params& q = params[l];
         const ssm_stack_grads& gr = grads[l];
@@ -880,20 +917,29 @@ SSM_API int ssm_stack_bwd(const ssm_shape* shape, int n_layers, const ssm_stack_
         const void* in = first ? u : at<void>(ws, sp.acts + sp.act * (l - 1));
         const float* v = at<float>(ws, sp.vs + sp.act * l);
         void* gnext = first ? du : at<void>(ws, (l & 1) ? sp.g1 : sp.g0);
+        const float *dw_part = nullptr, *db_part = nullptr;
+        int ln_rows = 0;
         {
             StageTimer tm("stack_gelu_ln_bwd", st);
             launch_stack_bwd(top && bf16, first && bf16, BT, s.H, g, in, v, q.ln_weight,
                              at<float>(ws, sp.stats + stat * (2 * l)), at<float>(ws, sp.stats + stat * (2 * l + 1)),
-                             at<float>(ws, sp.gz), at<float>(ws, sp.gv), gr.dln_weight, gr.dln_bias, at<float>(ws, sp.tmp), st);
+                             at<float>(ws, sp.gz), at<float>(ws, sp.gv), at<float>(ws, sp.tmp + sp.tmp_stride * l), &dw_part,
+                             &db_part, &ln_rows, st);
         }
         // the gradient handed down: gz (residual branch) + du of the SSM, summed in fp32 in the du epilogue
         const LayerIo io{first && bf16, false, false, first && bf16};
         if (int rc = layer_bwd_impl(ls, lp, io, q.Lambda, q.Delta, q.Bc, q.D, in, done, nullptr, at<void>(ws, sp.gv), nullptr,
                                     at<float>(ws, sp.gz), lws, hdr, gnext, gr.dLambda, gr.dDelta, gr.dB, gr.dC, gr.dD,
-                                    nullptr, st))
+                                    nullptr, &left[l], st))
             return rc;
+        GradTail& t = left[l].tail;
+        t.sum_part[1] = dw_part, t.sum_part[2] = db_part;
+        t.sum_rows[1] = t.sum_rows[2] = ln_rows;
+        t.sum_out[1] = gr.dln_weight, t.sum_out[2] = gr.dln_bias;
         g = gnext;
     }
+    // What no other layer waits for, for all layers together.
+    if (int rc = layer_bwd_tail(ls, lp, n_layers, left, hdr, st)) return rc;
     SSM_RETURN_IF_CUDA_ERROR();
     return SSM_OK;
 }

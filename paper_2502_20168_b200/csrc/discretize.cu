@@ -1,5 +1,7 @@
 // Zero-order-hold discretisation of the diagonal SSM (Sec. III-B, Eq. 3) and its adjoint,
 // plus the packing of the discretised parameters into real GEMM operands.
+#include <algorithm>
+
 #include "kernels.h"
 
 namespace ssm {
@@ -164,9 +166,11 @@ __device__ __forceinline__ void store3_pair(float a, float b, __nv_bfloat162& hi
 //   kPackF32    fp32: WB[2p+c, h], WC[2p+c, h] ([2P, H]);  Cp[h, 2p+c], Bq[h, 2p+c] ([H, 2P]).
 // with c = 0 / 1 for Re / Im of Bbar and Re / -Im of C.  `hdr` (may be NULL): its status word is cleared.
 enum PackMode { kPackTc, kPackPlanes, kPackF32 };
-struct PackOut {
-    float2 *Abar, *Alo;
-    void *WB, *WC, *Cp, *Bq;
+// A launch does the layers of a stack together (blockIdx.z), up to kN = kLayerBatch of them; a single layer's launch
+// carries the parameters of one (kN = 1).
+template <int kN>
+struct PackArgs {
+    PackJob job[kN];
     WsHeader* hdr;
     int group_log2;   // 0: no groups
 };
@@ -205,12 +209,13 @@ __device__ __forceinline__ void store_col_pair(void* W, int P, int p, int h, flo
     }
 }
 
-template <int kMode>
+template <int kMode, int kN>
 __global__ void __launch_bounds__(256)
-pack_params_kernel(int H, int P, const float2* Lambda, const float* Delta,
-                   const float2* Bc, const float2* Cc, PackOut o) {
+pack_params_kernel(int H, int P, const __grid_constant__ PackArgs<kN> o) {
     grid_dep_wait();
     grid_dep_launch();
+    const PackJob& q = o.job[blockIdx.z];
+    const float2 *Bc = q.Bc, *Cc = q.Cc;
     __shared__ float2 gamma_s[32];
     __shared__ float2 tB[32][33], tC[32][33];   // tB[state][h], tC[h][state]
     const int p0 = blockIdx.x * 32, h0 = blockIdx.y * 32;
@@ -225,15 +230,15 @@ pack_params_kernel(int H, int P, const float2* Lambda, const float* Delta,
     }
     if (w == 0 && p0 + lane < P) {
         const int p = p0 + lane;
-        const ZohTerms z = zoh_terms(Lambda[p], Delta[p]);
+        const ZohTerms z = zoh_terms(q.Lambda[p], q.Delta[p]);
         gamma_s[lane] = make_float2((float)z.gr, (float)z.gi);
         if (blockIdx.y == 0) {
             const float2 ah = make_float2((float)z.ar, (float)z.ai);
-            o.Abar[p] = ah;
-            o.Alo[p] = make_float2((float)(z.ar - (double)ah.x), (float)(z.ai - (double)ah.y));
+            q.Abar[p] = ah;
+            q.Alo[p] = make_float2((float)(z.ar - (double)ah.x), (float)(z.ai - (double)ah.y));
         }
     }
-    if (threadIdx.x == 32 && blockIdx.x == 0 && blockIdx.y == 0 && o.hdr) o.hdr->status = 0;
+    if (threadIdx.x == 32 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && o.hdr) o.hdr->status = 0;
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -248,20 +253,24 @@ pack_params_kernel(int H, int P, const float2* Lambda, const float* Delta,
         const int r = w + 8 * i;
         if (p0 + r < P && h0 + lane < H) {   // state p0 + r, feature h0 + lane
             const float2 cc = tC[lane][r];
-            store_row_pair<kMode>(o.WB, H, P, o.group_log2, p0 + r, h0 + lane, b[i].x, b[i].y);
-            store_row_pair<kMode>(o.WC, H, P, o.group_log2, p0 + r, h0 + lane, cc.x, -cc.y);
+            store_row_pair<kMode>(q.WB, H, P, o.group_log2, p0 + r, h0 + lane, b[i].x, b[i].y);
+            store_row_pair<kMode>(q.WC, H, P, o.group_log2, p0 + r, h0 + lane, cc.x, -cc.y);
         }
         if (p0 + lane < P && h0 + r < H) {   // state p0 + lane, feature h0 + r
             const float2 bb = tB[lane][r];
-            store_col_pair<kMode>(o.Bq, P, p0 + lane, h0 + r, bb.x, bb.y);
-            store_col_pair<kMode>(o.Cp, P, p0 + lane, h0 + r, c[i].x, -c[i].y);
+            store_col_pair<kMode>(q.Bq, P, p0 + lane, h0 + r, bb.x, bb.y);
+            store_col_pair<kMode>(q.Cp, P, p0 + lane, h0 + r, c[i].x, -c[i].y);
         }
     }
 }
 
 // ---------------------------------------------------------------------------------------------
-// Last sums of a layer's backward pass
+// Last sums of a layer's backward pass (the layers of a stack together)
 // ---------------------------------------------------------------------------------------------
+template <int kN>
+struct TailArgs {
+    GradTail layer[kN];
+};
 // The split-K partials of the weight-gradient products, part_b[s, h, 2p+c] (gBbar) and part_c[s, h, 2p+c] (dC, its
 // imaginary columns negated), are added in order of s.  gBbar itself is not stored: it leaves as
 // dB = conj(gamma) gBbar and as the sums g_gamma = sum conj(B) gBbar over the block's 32 features
@@ -270,29 +279,27 @@ pack_params_kernel(int H, int P, const float2* Lambda, const float* Delta,
 // the sum and the state-major store as separate strided kernels a step spent 7.7 - 20 us here, now 7 - 10 us.
 // kReduceWarps warps share the block's rows (one more evaluates gamma): 16 where there are many partials to add per
 // element, else 8 (1024 x 1024 with 2 partials: 8.2 against 10.5 us; 512 x 512 with 9: 7.2 with 16 against 8.5).
-template <int kReduceWarps>
+template <int kReduceWarps, int kN>
 __global__ void __launch_bounds__(32 * kReduceWarps + 32)
-reduce_weight_grads_kernel(int H, int P, int splits, const float* part_b, const float* part_c,
-                           const float2* Lambda, const float* Delta,
-                           const float2* Bc, float2* dB, float2* dC,
-                           float2* gg_part) {
+reduce_weight_grads_kernel(int H, int P, int splits, const __grid_constant__ TailArgs<kN> args) {
     grid_dep_wait();
     grid_dep_launch();
+    const GradTail& q = args.layer[blockIdx.z >> 1];
     __shared__ float2 gamma_s[32];
     __shared__ float2 t[32][33];   // [feature][state]
     constexpr int kRows = 32 / kReduceWarps;
     const int p0 = blockIdx.x * 32, h0 = blockIdx.y * 32;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const bool is_c = blockIdx.z != 0, p_ok = p0 + lane < P;
+    const bool is_c = (blockIdx.z & 1) != 0, p_ok = p0 + lane < P;
     if (w == kReduceWarps) {
         if (!is_c && p_ok) {
-            const ZohTerms z = zoh_terms(Lambda[p0 + lane], Delta[p0 + lane]);
+            const ZohTerms z = zoh_terms(q.Lambda[p0 + lane], q.Delta[p0 + lane]);
             gamma_s[lane] = make_float2((float)z.gr, (float)z.gi);
         }
         __syncthreads();
         return;
     }
-    const float2* part = reinterpret_cast<const float2*>(is_c ? part_c : part_b);
+    const float2* part = reinterpret_cast<const float2*>(is_c ? q.part_c : q.part_b);
     const size_t n = (size_t)H * P;   // complex values per split
     float2 acc[kRows];
 #pragma unroll
@@ -309,7 +316,7 @@ reduce_weight_grads_kernel(int H, int P, int splits, const float* part_b, const 
 #pragma unroll
     for (int i = 0; i < kRows; ++i) {
         if (is_c && p_ok && h0 + w + kReduceWarps * i < H)
-            dC[(size_t)(h0 + w + kReduceWarps * i) * P + p0 + lane] = cconj(acc[i]);
+            q.dC[(size_t)(h0 + w + kReduceWarps * i) * P + p0 + lane] = cconj(acc[i]);
         t[w + kReduceWarps * i][lane] = acc[i];
     }
     __syncthreads();
@@ -319,17 +326,17 @@ reduce_weight_grads_kernel(int H, int P, int splits, const float* part_b, const 
         const int pl = w + kReduceWarps * i, p = p0 + pl, h = h0 + lane;
         if (p >= P) continue;   // (the same for the whole warp)
         const float2 gb = t[lane][pl];
-        float2 q = make_float2(0.f, 0.f);
+        float2 gq = make_float2(0.f, 0.f);
         if (h < H) {
-            dB[(size_t)p * H + h] = cmul(cconj(gamma_s[pl]), gb);
-            q = cmul(cconj(Bc[(size_t)p * H + h]), gb);
+            q.dB[(size_t)p * H + h] = cmul(cconj(gamma_s[pl]), gb);
+            gq = cmul(cconj(q.Bc[(size_t)p * H + h]), gb);
         }
 #pragma unroll
         for (int m = 16; m > 0; m >>= 1) {
-            q.x += __shfl_xor_sync(0xffffffffu, q.x, m);
-            q.y += __shfl_xor_sync(0xffffffffu, q.y, m);
+            gq.x += __shfl_xor_sync(0xffffffffu, gq.x, m);
+            gq.y += __shfl_xor_sync(0xffffffffu, gq.y, m);
         }
-        if (lane == 0) gg_part[(size_t)blockIdx.y * P + p] = q;
+        if (lane == 0) q.gg[(size_t)blockIdx.y * P + p] = gq;
     }
 }
 
@@ -337,30 +344,33 @@ reduce_weight_grads_kernel(int H, int P, int splits, const float* part_b, const 
 // (dD_rows rows of [H]) folded in, in a fixed order.  A block owns 32 columns, its 32 warps take the rows in turn
 // (the rows of partial sums are up to 512, the columns a few hundred: latency is all there is), one warp evaluates
 // the P-sized double-precision terms meanwhile.  H = 512, P = 256: 6.2 - 9.5 -> 3.0 - 6.3 us (4 - 512 rows) against one block per state.
+template <int kN>
 __global__ void __launch_bounds__(1024)
-layer_finalize_kernel(int H, int P, const float2* Lambda, const float* Delta,
-                      const float2* gA_part, int gA_rows, const float2* gg_part, int gg_rows,
-                      float2* dLambda, float* dDelta, const float* dD_part,
-                      int dD_rows, float* dD) {
+layer_finalize_kernel(int H, int P, int gA_rows, int gg_rows, const __grid_constant__ TailArgs<kN> args) {
     grid_dep_wait();
     grid_dep_launch();
+    const GradTail& q = args.layer[blockIdx.z];
+    const float2 *Lambda = q.Lambda, *gA_part = q.gA_part, *gg_part = q.gg;
+    const float* Delta = q.Delta;
     __shared__ double sA[2][32][33], sG[2][32][33];
     __shared__ ZohTerms zs[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int p_blocks = (P + 31) / 32;
-    if ((int)blockIdx.x >= p_blocks) {   // 32 columns of dD
+    if ((int)blockIdx.x >= p_blocks) {   // 32 columns of one of the sums over row groups (dD, then a stack's dw, db)
         float(*sD)[33] = reinterpret_cast<float(*)[33]>(sA);
-        const int h = ((int)blockIdx.x - p_blocks) * 32 + lane;
+        const int h_blocks = (H + 31) / 32, blk = (int)blockIdx.x - p_blocks, which = blk / h_blocks;
+        const int h = (blk - which * h_blocks) * 32 + lane;
+        const float* part = q.sum_part[which];
         float acc = 0.f;
         if (h < H)
-            for (int r = w; r < dD_rows; r += 32) acc += dD_part[(size_t)r * H + h];
+            for (int r = w; r < q.sum_rows[which]; r += 32) acc += part[(size_t)r * H + h];
         sD[w][lane] = acc;
         __syncthreads();
         if (w == 0 && h < H) {
             float t = 0.f;
 #pragma unroll
             for (int i = 0; i < 32; ++i) t += sD[i][lane];
-            dD[h] = t;
+            q.sum_out[which][h] = t;
         }
         return;
     }
@@ -396,35 +406,35 @@ layer_finalize_kernel(int H, int P, const float2* Lambda, const float* Delta,
     __syncthreads();
     if (w == 0 && p < P)
         zoh_adjoint(zs[lane], Lambda[p], Delta[p], sA[0][0][lane], sA[1][0][lane], sG[0][0][lane], sG[1][0][lane],
-                    dLambda[p], dDelta[p]);
+                    q.dLambda[p], q.dDelta[p]);
 }
 
 static dim3 weight_tiles(int H, int P, int z) { return dim3((P + 31) / 32, (H + 31) / 32, z); }
 
-template <int kMode>
-static void launch_pack(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc, const float2* Cc,
-                        const PackOut& o, cudaStream_t st) {
+template <int kMode, int kN>
+static void launch_pack_n(int H, int P, int n, const PackJob* jobs, int group, WsHeader* hdr, cudaStream_t st) {
+    PackArgs<kN> o{};
+    std::copy(jobs, jobs + n, o.job);
+    o.hdr = hdr;
+    o.group_log2 = group == 64 ? 6 : (group == 32 ? 5 : 0);
     count_launch();
-    launch_dep(pack_params_kernel<kMode>, weight_tiles(H, P, 1), 256, 0, st, H, P, Lambda, Delta, Bc, Cc, o);
+    launch_dep(pack_params_kernel<kMode, kN>, weight_tiles(H, P, n), 256, 0, st, H, P, o);
+}
+template <int kMode>
+static void launch_pack(int H, int P, int n, const PackJob* jobs, int group, WsHeader* hdr, cudaStream_t st) {
+    if (n == 1) return launch_pack_n<kMode, 1>(H, P, 1, jobs, group, hdr, st);
+    for (int l = 0; l < n; l += kLayerBatch)
+        launch_pack_n<kMode, kLayerBatch>(H, P, std::min(kLayerBatch, n - l), jobs + l, group, l == 0 ? hdr : nullptr, st);
 }
 
-void launch_discretize_pack_tc(int H, int P, int group, const float2* Lambda, const float* Delta, const float2* Bc,
-                               const float2* Cc, float2* Abar, float2* Abar_lo, void* Wsplit_B, void* Wsplit_C, void* Cp,
-                               void* Bq, WsHeader* hdr, cudaStream_t st) {
-    const int group_log2 = group == 64 ? 6 : (group == 32 ? 5 : 0);
-    launch_pack<kPackTc>(H, P, Lambda, Delta, Bc, Cc, PackOut{Abar, Abar_lo, Wsplit_B, Wsplit_C, Cp, Bq, hdr, group_log2}, st);
+void launch_discretize_pack_tc(int H, int P, int group, const PackJob& job, WsHeader* hdr, cudaStream_t st) {
+    launch_pack<kPackTc>(H, P, 1, &job, group, hdr, st);
 }
-
-void launch_discretize_pack_planes(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
-                                   const float2* Cc, float2* Abar, float2* Abar_lo, void* Wb3, void* Cq3, void* Cp3,
-                                   void* Bq3, WsHeader* hdr, cudaStream_t st) {
-    launch_pack<kPackPlanes>(H, P, Lambda, Delta, Bc, Cc, PackOut{Abar, Abar_lo, Wb3, Cq3, Cp3, Bq3, hdr, 0}, st);
+void launch_discretize_pack_planes(int H, int P, int n, const PackJob* jobs, WsHeader* hdr, cudaStream_t st) {
+    launch_pack<kPackPlanes>(H, P, n, jobs, 0, hdr, st);
 }
-
-void launch_discretize_pack_f32(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
-                                const float2* Cc, float2* Abar, float2* Abar_lo, void* Bp, void* Cq, void* Cp, void* Bq,
-                                WsHeader* hdr, cudaStream_t st) {
-    launch_pack<kPackF32>(H, P, Lambda, Delta, Bc, Cc, PackOut{Abar, Abar_lo, Bp, Cq, Cp, Bq, hdr, 0}, st);
+void launch_discretize_pack_f32(int H, int P, int n, const PackJob* jobs, WsHeader* hdr, cudaStream_t st) {
+    launch_pack<kPackF32>(H, P, n, jobs, 0, hdr, st);
 }
 
 void launch_discretize(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc, float2* Abar,
@@ -442,24 +452,23 @@ void launch_discretize_bwd(int H, int P, const float2* Lambda, const float* Delt
 
 int gamma_part_rows(int H) { return (H + 31) / 32; }
 
-void launch_reduce_weight_grads(int H, int P, int splits, const float* part_b, const float* part_c, const float2* Lambda,
-                                const float* Delta, const float2* Bc, float2* dB, float2* dC, float2* gg_part,
-                                cudaStream_t st) {
-    count_launch();
-    const dim3 grid = weight_tiles(H, P, 2);
-    if (splits > 4)
-        launch_dep(reduce_weight_grads_kernel<16>, grid, 32 * 17, 0, st, H, P, splits, part_b, part_c, Lambda, Delta, Bc, dB, dC, gg_part);
-    else
-        launch_dep(reduce_weight_grads_kernel<8>, grid, 32 * 9, 0, st, H, P, splits, part_b, part_c, Lambda, Delta, Bc, dB, dC, gg_part);
+template <int kN>
+static void launch_tail_n(int H, int P, int splits, int n, const GradTail* tails, int gA_rows, cudaStream_t st) {
+    TailArgs<kN> args{};
+    std::copy(tails, tails + n, args.layer);
+    const int n_sums = tails[0].sum_out[2] ? 3 : 1;
+    const dim3 grid = weight_tiles(H, P, 2 * n);
+    count_launch(2);
+    if (splits > 4) launch_dep(reduce_weight_grads_kernel<16, kN>, grid, 32 * 17, 0, st, H, P, splits, args);
+    else launch_dep(reduce_weight_grads_kernel<8, kN>, grid, 32 * 9, 0, st, H, P, splits, args);
+    launch_dep(layer_finalize_kernel<kN>, dim3((P + 31) / 32 + n_sums * ((H + 31) / 32), 1, n), 1024, 0, st, H, P, gA_rows,
+               gamma_part_rows(H), args);
 }
 
-void launch_layer_finalize(int H, int P, const float2* Lambda, const float* Delta, const float2* gA_part, int gA_rows,
-                           const float2* gg_part, float2* dLambda, float* dDelta, const float* dD_part, int dD_rows,
-                           float* dD, cudaStream_t st) {
-    count_launch();
-    launch_dep(layer_finalize_kernel, (P + 31) / 32 + (H + 31) / 32, 1024, 0, st, H, P, Lambda, Delta, gA_part, gA_rows, gg_part,
-                                                                         gamma_part_rows(H), dLambda, dDelta, dD_part,
-                                                                         dD_rows, dD);
+void launch_layer_tail(int H, int P, int splits, int n, const GradTail* tails, int gA_rows, cudaStream_t st) {
+    if (n == 1) return launch_tail_n<1>(H, P, splits, 1, tails, gA_rows, st);
+    for (int l = 0; l < n; l += kLayerBatch)
+        launch_tail_n<kLayerBatch>(H, P, splits, std::min(kLayerBatch, n - l), tails + l, gA_rows, st);
 }
 
 }  // namespace ssm

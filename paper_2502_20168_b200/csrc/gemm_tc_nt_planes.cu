@@ -1,5 +1,5 @@
-// Weight gradients of fp32 layers: both products of a backward pass (gBbar = s^T u and dC = gy^T conj(x)) as sums of
-// products of bf16 planes, in one launch.
+// Weight gradients of fp32 layers: the products of a backward pass (gBbar = s^T u and dC = gy^T conj(x)) as sums of
+// products of bf16 planes, both of a layer, or all of a stack's layers, in one launch.
 //   part[s, i, j] = sum over the rows m of slice s of A[m, i] B[m, j],  A [K, I], B [K, J] as bf16 planes
 // Both operands are contiguous in the output index (MN-major tiles of [64 rows][64 columns]).  One CTA per 128 x 128
 // tile, slice of the rows and product: a k-block brings every plane of both operands in once (96 KB) and all six
@@ -26,10 +26,16 @@ constexpr size_t kNpSmemMax = 220 * 1024;
 struct NtPlanesArgs {
     int K, I, J, j_tiles, blocks_per_split;
     int stages, stage_bytes;
-    int planes_a[2], planes_b[2], n_prod[2];
-    uint32_t pa[2], pb[2];
-    float* part[2];
     WsHeader* hdr;
+    struct Product {
+        int planes_a, planes_b, n_prod;
+        uint32_t pa, pb;
+        float* part;
+    } product[2 * kLayerBatch];
+};
+template <int kN>
+struct NtPlanesMaps {   // (a single layer does not carry a batch's 8 KB of tensor maps through its launch)
+    CUtensorMap a[kN], b[kN];
 };
 
 struct NtPlanesBars {
@@ -38,18 +44,20 @@ struct NtPlanesBars {
     int abort_flag;
 };
 
+template <int kN>
 __global__ void __launch_bounds__(kNpThreads, 1)
-gemm_tc_nt_planes_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
-                         const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1, NtPlanesArgs p) {
+gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __grid_constant__ NtPlanesArgs p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ NtPlanesBars bars;
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     volatile int* abort_flag = &bars.abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, z = blockIdx.z;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const NtPlanesArgs::Product& pr = p.product[blockIdx.z];
+    const CUtensorMap *ta = &maps.a[blockIdx.z], *tb = &maps.b[blockIdx.z];
     const int i0 = ((int)blockIdx.x / p.j_tiles) * 128, j0 = ((int)blockIdx.x % p.j_tiles) * 128;
     const int total = (p.K + BK - 1) / BK;
     const int kb0 = (int)blockIdx.y * p.blocks_per_split, kb1 = min(total, kb0 + p.blocks_per_split);
-    const int planes_a = p.planes_a[z], planes_b = p.planes_b[z];
+    const int planes_a = pr.planes_a, planes_b = pr.planes_b;
     if (threadIdx.x == 0) {
         for (int i = 0; i < p.stages; ++i) {
             mbar_init(smem_u32(&bars.full[i]), 1);
@@ -62,8 +70,8 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_
         bars.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        prefetch_tmap(z ? &tmA1 : &tmA0);
-        prefetch_tmap(z ? &tmB1 : &tmB0);
+        prefetch_tmap(ta);
+        prefetch_tmap(tb);
     }
     __syncwarp();
     if (warp == 1) tmem_alloc(smem_u32(&bars.tmem), 512);
@@ -76,7 +84,6 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_
 
     if (warp == 0) {
         if (lane == 0) {
-            const CUtensorMap *ta = z ? &tmA1 : &tmA0, *tb = z ? &tmB1 : &tmB0;
             const uint32_t bytes = (uint32_t)(planes_a + planes_b) * kNpTile;
             int stage = 0;
             uint32_t phase = 0;
@@ -102,8 +109,8 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_
     } else if (warp == 1) {
         if (lane == 0 && kb0 < kb1) {
             constexpr uint32_t idesc = instr_desc(128, 128, 1, 1);
-            const int n_prod = p.n_prod[z];
-            const uint32_t pa = p.pa[z], pb = p.pb[z];
+            const int n_prod = pr.n_prod;
+            const uint32_t pa = pr.pa, pb = pr.pb;
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -138,7 +145,7 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_
     } else {
         const int q = warp & 3, half = (warp - 2) >> 2;
         const int row = i0 + q * 32 + lane;
-        float* dst = p.part[z] + ((size_t)blockIdx.y * p.I + row) * p.J + j0 + 64 * half;
+        float* dst = pr.part + ((size_t)blockIdx.y * p.I + row) * p.J + j0 + 64 * half;
         const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + 64u * (uint32_t)half;
         float sum[64];
 #pragma unroll
@@ -177,39 +184,48 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_
 }  // namespace tc
 
 // Slices of the rows: as many as leave every SM at most one CTA of the launch.
-int tc_nt_planes_splits(int K, int I, int J) {
-    const int units = 2 * (I / 128) * (J / 128), blocks = (K + tc::BK - 1) / tc::BK;
+int tc_nt_planes_splits(int K, int I, int J, int n_products) {
+    const int units = n_products * (I / 128) * (J / 128), blocks = (K + tc::BK - 1) / tc::BK;
     return std::max(1, std::min(std::min(blocks, 64), device_sm_count() / std::max(units, 1)));
 }
 
-int launch_gemm_tc_nt_planes(const GemmTcNtPlanes& g, cudaStream_t st) {
+template <int kN>
+static int launch_nt_planes(int K, int I, int J, int splits, int n, const GemmTcNtPlanes* products, WsHeader* hdr, cudaStream_t st) {
     using namespace tc;
-    if (g.I % 128 != 0 || g.J % 128 != 0) return SSM_ERR_SHAPE;
+    auto kern = gemm_tc_nt_planes_kernel<kN>;
+    if (!set_max_dynamic_smem(reinterpret_cast<const void*>(kern), kNpSmemMax)) return SSM_ERR_CUDA;
+    const int blocks = (K + BK - 1) / BK;
     NtPlanesArgs p{};
-    p.K = g.K, p.I = g.I, p.J = g.J, p.j_tiles = g.J / 128, p.hdr = g.hdr;
-    const int blocks = (g.K + BK - 1) / BK;
-    p.blocks_per_split = (blocks + g.splits - 1) / g.splits;
-    CUtensorMap ma[2], mb[2];
+    NtPlanesMaps<kN> maps{};
+    p.K = K, p.I = I, p.J = J, p.j_tiles = J / 128, p.hdr = hdr;
+    p.blocks_per_split = (blocks + splits - 1) / splits;
     int planes = 0;
-    for (int z = 0; z < 2; ++z) {
-        const GemmTcNtPlanes::Product& q = g.product[z];
+    for (int z = 0; z < n; ++z) {
+        const GemmTcNtPlanes& q = products[z];
         if (q.n_products < 2 || q.n_products > 8) return SSM_ERR_SHAPE;
-        p.planes_a[z] = q.planes_a, p.planes_b[z] = q.planes_b, p.n_prod[z] = q.n_products;
-        p.pa[z] = q.prod_a, p.pb[z] = q.prod_b, p.part[z] = q.part;
+        p.product[z] = {q.planes_a, q.planes_b, q.n_products, q.prod_a, q.prod_b, q.part};
         planes = std::max(planes, q.planes_a + q.planes_b);
-        if (!make_map(&ma[z], q.A, (uint64_t)g.K, (uint64_t)g.I * q.planes_a, 64, BK)) return SSM_ERR_CUDA;
-        if (!make_map(&mb[z], q.B, (uint64_t)g.K, (uint64_t)g.J * q.planes_b, 64, BK)) return SSM_ERR_CUDA;
+        if (!make_map(&maps.a[z], q.A, (uint64_t)K, (uint64_t)I * q.planes_a, 64, BK)) return SSM_ERR_CUDA;
+        if (!make_map(&maps.b[z], q.B, (uint64_t)K, (uint64_t)J * q.planes_b, 64, BK)) return SSM_ERR_CUDA;
     }
     p.stage_bytes = planes * kNpTile;
     p.stages = std::min<int>(kNpMaxStages, (int)((kNpSmemMax - 1024) / p.stage_bytes));
     if (p.stages < 2) return SSM_ERR_SHAPE;
-    if (!set_max_dynamic_smem(reinterpret_cast<const void*>(gemm_tc_nt_planes_kernel), kNpSmemMax)) return SSM_ERR_CUDA;
     count_launch();
-    const dim3 grid((unsigned)((g.I / 128) * p.j_tiles), (unsigned)g.splits, 2);
-    return launch_dep(gemm_tc_nt_planes_kernel, grid, kNpThreads, (size_t)p.stages * p.stage_bytes + 1024, st, ma[0], mb[0], ma[1],
-                      mb[1], p)
-               ? SSM_OK
-               : SSM_ERR_CUDA;
+    const dim3 grid((unsigned)((I / 128) * p.j_tiles), (unsigned)splits, (unsigned)n);
+    return launch_dep(kern, grid, kNpThreads, (size_t)p.stages * p.stage_bytes + 1024, st, maps, p) ? SSM_OK : SSM_ERR_CUDA;
+}
+
+int launch_gemm_tc_nt_planes(int K, int I, int J, int splits, int n_products, const GemmTcNtPlanes* products, WsHeader* hdr,
+                             cudaStream_t st) {
+    if (I % 128 != 0 || J % 128 != 0) return SSM_ERR_SHAPE;
+    for (int first = 0; first < n_products; first += 2 * kLayerBatch) {
+        const int n = std::min(2 * kLayerBatch, n_products - first);
+        const int rc = n <= 2 ? launch_nt_planes<2>(K, I, J, splits, n, products + first, hdr, st)
+                              : launch_nt_planes<2 * kLayerBatch>(K, I, J, splits, n, products + first, hdr, st);
+        if (rc) return rc;
+    }
+    return SSM_OK;
 }
 
 }  // namespace ssm

@@ -11,31 +11,35 @@ void launch_discretize(int H, int P, const float2* Lambda, const float* Delta, c
 void launch_discretize_bwd(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
                            const float2* gAbar, const float2* gBbar, float2* dLambda, float* dDelta, float2* dB,
                            cudaStream_t st);
-// Discretisation and the packed projection operands of a layer in one kernel (layouts at pack_params_kernel).
-// Abar_lo: Abar's rounding residual, exp(Lambda Delta) - Abar, as fp32.  hdr (may be NULL): status word cleared.
-// Tensor-core path: Wsplit_B / Wsplit_C hi/lo stacked [4P, H]; group: 0 = rows in the plain order (2p + c, stacked
-// per 128 rows: GemmTcTN with split_w), or the states per chain (64, 32) of the kernels that scan in their epilogue.
-void launch_discretize_pack_tc(int H, int P, int group, const float2* Lambda, const float* Delta, const float2* Bc,
-                               const float2* Cc, float2* Abar, float2* Abar_lo, void* Wsplit_B, void* Wsplit_C, void* Cp,
-                               void* Bq, WsHeader* hdr, cudaStream_t st);
-// Plane path: the four operands as three bf16 planes: Wb3, Cq3 [2P, 3H]; Cp3, Bq3 [H, 3 * 2P].
-void launch_discretize_pack_planes(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
-                                   const float2* Cc, float2* Abar, float2* Abar_lo, void* Wb3, void* Cq3, void* Cp3,
-                                   void* Bq3, WsHeader* hdr, cudaStream_t st);
-// CUDA-core path: fp32, Bp, Cq [2P, H]; Cp, Bq [H, 2P].
-void launch_discretize_pack_f32(int H, int P, const float2* Lambda, const float* Delta, const float2* Bc,
-                                const float2* Cc, float2* Abar, float2* Abar_lo, void* Bp, void* Cq, void* Cp, void* Bq,
-                                WsHeader* hdr, cudaStream_t st);
-// End of a layer's backward pass.  The split-K partials [splits, H, 2P] of gBbar and dC are added; gBbar leaves as dB
-// and as gamma_part_rows(H) rows of partial sums of g_gamma.  Then the adjoint of the discretisation from rows of
-// partial sums of gAbar [gA_rows, P] and g_gamma; dD from dD_rows rows [dD_rows, H].  All in a fixed order.
+// Discretisation and the packed projection operands of layers in one kernel (layouts at pack_params_kernel).
+// Alo: Abar's rounding residual, exp(Lambda Delta) - Abar, as fp32.  hdr (may be NULL): status word cleared.
+struct PackJob {
+    const float2* Lambda; const float* Delta; const float2 *Bc, *Cc;
+    float2 *Abar, *Alo;
+    void *WB, *WC, *Cp, *Bq;
+};
+constexpr int kLayerBatch = 16;   // layers of a stack that one launch of the parameter kernels takes
+// Tensor-core path: WB / WC hi/lo stacked [4P, H]; group: 0 = rows in the plain order (2p + c, stacked per 128 rows:
+// GemmTcTN with split_w), or the states per chain (64, 32) of the kernels that scan in their epilogue.
+void launch_discretize_pack_tc(int H, int P, int group, const PackJob& job, WsHeader* hdr, cudaStream_t st);
+// Plane path: the four operands as three bf16 planes: WB, WC [2P, 3H]; Cp, Bq [H, 3 * 2P].
+void launch_discretize_pack_planes(int H, int P, int n, const PackJob* jobs, WsHeader* hdr, cudaStream_t st);
+// CUDA-core path: fp32, WB, WC [2P, H]; Cp, Bq [H, 2P].
+void launch_discretize_pack_f32(int H, int P, int n, const PackJob* jobs, WsHeader* hdr, cudaStream_t st);
+// End of the backward pass of n layers of one shape.  The split-K partials [splits, H, 2P] of gBbar and dC are added;
+// gBbar leaves as dB and as gamma_part_rows(H) rows of partial sums of g_gamma (gg).  Then the adjoint of the
+// discretisation from rows of partial sums of gAbar [gA_rows, P] and g_gamma; sums[0] = dD and, in a stack, sums[1],
+// sums[2] (LayerNorm weight and bias) from rows of partial sums [sum_rows, H].  All in a fixed order.
+struct GradTail {
+    const float2* Lambda; const float* Delta; const float2* Bc;
+    const float *part_b, *part_c;
+    float2 *dB, *dC, *gg;
+    const float2* gA_part;
+    float2* dLambda; float* dDelta;
+    const float* sum_part[3]; int sum_rows[3]; float* sum_out[3];
+};
 int gamma_part_rows(int H);
-void launch_reduce_weight_grads(int H, int P, int splits, const float* part_b, const float* part_c, const float2* Lambda,
-                                const float* Delta, const float2* Bc, float2* dB, float2* dC, float2* gg_part,
-                                cudaStream_t st);
-void launch_layer_finalize(int H, int P, const float2* Lambda, const float* Delta, const float2* gA_part, int gA_rows,
-                           const float2* gg_part, float2* dLambda, float* dDelta, const float* dD_part, int dD_rows,
-                           float* dD, cudaStream_t st);
+void launch_layer_tail(int H, int P, int splits, int n, const GradTail* tails, int gA_rows, cudaStream_t st);
 
 // scan.cu
 // Scratch the scans need for a [B,T,P] problem: a work counter and the partial sums of gAbar.
@@ -225,20 +229,17 @@ struct GemmTcNT {
     WsHeader* hdr;
     int lda = 0;   // elements between rows of A when A is a column block of a wider matrix (0: I)
 };
-// Both weight-gradient products of an fp32 layer from planes (gemm_tc_nt_planes.cu): A = planes_a planes of I columns
-// side by side, B = planes_b planes of J columns; product schedules as in GemmTcTN.  I and J multiples of 128.
+// Weight-gradient products of fp32 layers from planes (gemm_tc_nt_planes.cu), two per layer: A = planes_a planes of I
+// columns side by side, B = planes_b planes of J columns; product schedules as in GemmTcTN.  I, J multiples of 128.
 struct GemmTcNtPlanes {
-    int K, I, J, splits;
-    struct Product {
-        const void *A, *B;
-        int planes_a, planes_b, n_products;
-        uint32_t prod_a, prod_b;
-        float* part;   // [splits, I, J]
-    } product[2];
-    WsHeader* hdr;
+    const void *A, *B;
+    int planes_a, planes_b, n_products;
+    uint32_t prod_a, prod_b;
+    float* part;   // [splits, I, J]
 };
-int tc_nt_planes_splits(int K, int I, int J);
-int launch_gemm_tc_nt_planes(const GemmTcNtPlanes& g, cudaStream_t st);
+int tc_nt_planes_splits(int K, int I, int J, int n_products);
+int launch_gemm_tc_nt_planes(int K, int I, int J, int splits, int n_products, const GemmTcNtPlanes* products, WsHeader* hdr,
+                             cudaStream_t st);
 bool tc_nt_supported(int I, int J);
 int tc_nt_splits(int K, int I, int J);
 int launch_gemm_tc_nt(const GemmTcNT& g, cudaStream_t st);
@@ -271,8 +272,9 @@ void launch_glu_reduce(const float* part, int splits, size_t n, float* out, cuda
 size_t stack_tmp_floats(int M, int H);
 void launch_stack_fwd(bool u_bf16, bool out_bf16, int M, int H, const void* u, const float* v, const float* w,
                       const float* b, void* out, float* mu, float* rstd, cudaStream_t st);
+// The sums for dw and db are left as *part_rows <= kMaxPartialRows rows of [H] each, inside tmp.
 void launch_stack_bwd(bool g_bf16, bool u_bf16, int M, int H, const void* g, const void* u, const float* v,
-                      const float* w, const float* mu, const float* rstd, float* gz, float* gv, float* dw, float* db,
-                      float* tmp, cudaStream_t st);
+                      const float* w, const float* mu, const float* rstd, float* gz, float* gv, float* tmp,
+                      const float** dw_part, const float** db_part, int* part_rows, cudaStream_t st);
 
 }  // namespace ssm
