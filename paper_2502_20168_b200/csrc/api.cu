@@ -22,7 +22,7 @@ struct LayerPlan {
     bool planes;
     int splits;
     size_t hdr, Abar, Alo, W0, W1, W2, W3, f32buf, xs, gs, gAbar, gg, scan, part, dot, total;
-    size_t u3, gy3, x3, s3, acc;   // plane path: planes of u, gy, x, s and the fp32 result of a projection
+    size_t u3, gy3, x3, s3;   // plane path: planes of u, gy, x, s for the weight gradients
 };
 
 #ifndef SSM_PLANES_MIN_ROWS
@@ -79,7 +79,6 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true) {
             p.gy3 = take(off, BT * 3 * s.H * 2);
             p.x3 = take(off, BT * 6 * s.P * 2);
             p.s3 = take(off, BT * 6 * s.P * 2);
-            p.acc = take(off, BT * s.H * 4);
         }
     }
     p.gAbar = take(off, (size_t)s.P * 8);
@@ -87,7 +86,7 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true) {
     p.scan = take(off, scan_scratch_bytes(s.B, s.T, s.P, 2));
     p.part = take(off, (size_t)2 * p.splits * 2 * PH * 4);   // split-K partials of gBbar, then those of dC
     {   // dD: partial column sums of gy * u, from the stand-alone kernel or from the epilogue of the du projection
-        const size_t rows = (size_t)tc_tn_dot_max_rows((int)BT, s.H);
+        const size_t rows = (size_t)tc_tn_dot_max_rows((int)BT);
         const size_t fused = rows * s.H + colsum_tmp_floats((int)rows, s.H);
         p.dot = take(off, std::max(dot_columns_tmp_floats((int)BT, s.H), fused) * 4);
     }
@@ -291,16 +290,14 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
     } else if (p.planes) {
         {   // Bu = u Bbar^T as a sum of plane products (u: three planes of an fp32 input, or the bf16 input itself)
             StageTimer tm("gemm_Bu", st);
-            const bool split_here = !io.u_bf16 && tc_tn_small(BT, P2, false);
-            if (!io.u_bf16 && !split_here) launch_split_planes((const float*)u, (size_t)BT, s.H, at<void>(ws, p.u3), st);
-            GemmTcTN g{io.u_bf16 || split_here ? u : at<void>(ws, p.u3), at<void>(ws, p.W0), BT, P2, s.H, false, true, at<void>(ws, p.xs),
+            GemmTcTN g{u, at<void>(ws, p.W0), BT, P2, s.H, false, true, at<void>(ws, p.xs),
                        nullptr, nullptr, hdr};
             g.n_products = io.u_bf16 ? 3 : 6;
             g.planes_a = io.u_bf16 ? 1 : 3;
             g.planes_w = 3;
             g.prod_a = io.u_bf16 ? kProd3A : kProd6A;
             g.prod_w = io.u_bf16 ? kProd3B : kProd6B;
-            if (split_here) g.a_f32 = true, g.a_planes_out = keep_planes ? at<void>(ws, p.u3) : nullptr;
+            if (!io.u_bf16) g.a_f32 = true, g.a_planes_out = keep_planes ? at<void>(ws, p.u3) : nullptr;
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
         }
         {
@@ -310,23 +307,17 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
                                  at<char>(ws, p.scan), st);
             if (rc) return rc;
         }
-        {   // y = x Cp^T + D u: planes of x, six products, the skip term in the epilogue or after it
+        {   // y = x Cp^T + D u: six products of planes, the skip term in the epilogue
             StageTimer tm("gemm_y", st);
-            const bool small = tc_tn_small(BT, s.H, false);
-            if (!small) launch_split_planes(at<float>(ws, p.xs), (size_t)BT, P2, at<void>(ws, p.x3), st);
-            GemmTcTN g{small ? at<void>(ws, p.xs) : at<void>(ws, p.x3), at<void>(ws, p.W2), BT, s.H, P2, false, true, at<void>(ws, p.acc), nullptr,
-                       nullptr, hdr};
+            GemmTcTN g{at<void>(ws, p.xs), at<void>(ws, p.W2), BT, s.H, P2, false, !io.y_bf16, y, D, u, hdr};
+            g.skip_bf16 = io.u_bf16;
             g.n_products = 6;
             g.planes_a = 3;
             g.planes_w = 3;
             g.prod_a = kProd6A;
             g.prod_w = kProd6B;
-            if (small) {
-                g.store_f32 = !io.y_bf16, g.out = y, g.diag = D, g.skip = u, g.skip_bf16 = io.u_bf16;
-                g.a_f32 = true, g.a_planes_out = keep_planes ? at<void>(ws, p.x3) : nullptr;
-            }
+            g.a_f32 = true, g.a_planes_out = keep_planes ? at<void>(ws, p.x3) : nullptr;
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
-            if (!small) launch_diag_skip(at<float>(ws, p.acc), D, u, io.u_bf16, nullptr, (size_t)BT, s.H, y, io.y_bf16, st);
         }
     } else {
         {
@@ -440,11 +431,10 @@ GluPlan plan_glu(const ssm_shape& s) {
     GluPlan p{};
     size_t off = 0;
     const size_t M = (size_t)s.B * s.T, HH = (size_t)s.H * s.H;
-    p.tc = s.io_dtype == SSM_BF16 && tc_tn_supported((int)M, s.H, 2 * s.H, true) &&
-           tc_tn_supported((int)M, s.H, s.H, true) && tc_nt_supported(s.H, s.H);
+    p.tc = s.io_dtype == SSM_BF16 && tc_tn_supported((int)M, s.H, s.H, false) && tc_nt_supported(s.H, s.H);
     p.splits = p.tc ? tc_nt_splits((int)M, s.H, s.H) : gemm_nt_splits((int)M);
     p.hdr = take(off, sizeof(WsHeader));
-    p.Wt = take(off, p.tc ? 4 * HH * 2 : HH * 4);   // tc: hi/lo stacked bf16 [2H, 2H]; else W^T fp32
+    p.Wt = take(off, HH * 4);   // W^T: bf16 planes hi | lo [H, 2H], or fp32
     p.Wn = take(off, p.tc ? 2 * HH * 2 : 0);
     p.x1 = take(off, M * s.H * 4);                  // GELU(v): fp32, or two bf16 planes
     p.z = take(off, M * s.H * 4);                   // the gate's argument
@@ -475,27 +465,21 @@ SSM_API int ssm_glu_fwd(const ssm_shape* shape, const float* W, const void* v, v
     const int M = s.B * s.T;
     const size_t n = (size_t)M * s.H;
     WsHeader* hdr = at<WsHeader>(ws, p.hdr);
-    if (cudaMemsetAsync(ws, 0, sizeof(WsHeader), st) != cudaSuccess) return SSM_ERR_CUDA;
     {
         StageTimer tm("glu_pack_gelu", st);
         launch_glu_pack(s.H, W, p.tc ? at<void>(ws, p.Wt) : nullptr, p.tc ? at<void>(ws, p.Wn) : nullptr,
-                        p.tc ? nullptr : at<float>(ws, p.Wt), st);
+                        p.tc ? nullptr : at<float>(ws, p.Wt), hdr, st);
         launch_glu_gelu(bf16, p.tc, n, s.H, v, at<void>(ws, p.x1), st);
     }
     {   // z[m, j] = sum_i x1[m, i] W[i, j]
         StageTimer tm("glu_gemm_z", st);
         if (p.tc) {
-            // both planes of x1 along K: a single bf16 rounding of x1 here costs 2e-2 on dW
-            // out = v * sigmoid(z) leaves from the same epilogue
-            GemmTcTN g{at<void>(ws, p.x1), at<void>(ws, p.Wt), M, s.H, 2 * s.H, true, true, at<void>(ws, p.z), nullptr, v, hdr};
+            // three products of the planes of x1 and W (lo hi, hi lo, hi hi; a single bf16 rounding of x1 here costs
+            // 2e-2 on dW); out = v * sigmoid(z) leaves from the same epilogue
+            GemmTcTN g{at<void>(ws, p.x1), at<void>(ws, p.Wt), M, s.H, s.H, false, true, at<void>(ws, p.z), nullptr, v, hdr};
             g.gate_out = out;
-            if (tc_tn_small(M, s.H, true)) {   // the same three products as a schedule: lo hi, hi lo, hi hi
-                g.K = s.H, g.split_w = false, g.w_plane_rows = 128, g.w_pitch = 2 * s.H;
-                g.n_products = 3, g.planes_a = 2, g.planes_w = 2, g.prod_a = 0x001u, g.prod_w = 0x010u;
-                if (int rc = launch_gemm_tc_tn_small(g, st)) return rc;
-            } else if (int rc = launch_gemm_tc_tn(g, st)) {
-                return rc;
-            }
+            g.n_products = 3, g.planes_a = 2, g.planes_w = 2, g.prod_a = 0x001u, g.prod_w = 0x010u;
+            if (int rc = launch_gemm_tc_tn(g, st)) return rc;
         } else {
             GemmTN g{at<void>(ws, p.x1), false, s.H, at<void>(ws, p.Wt), false, s.H, M, s.H, s.H, Epi::StoreF32,
                      at<void>(ws, p.z), false, nullptr, nullptr, false, nullptr};
@@ -530,7 +514,8 @@ SSM_API int ssm_glu_bwd(const ssm_shape* shape, const float* W, const void* v, c
     {   // g_x1[m, i] = sum_j gz[m, j] W[i, j]
         StageTimer tm("glu_gemm_gx1", st);
         if (p.tc) {
-            GemmTcTN g{at<void>(ws, p.gz), at<void>(ws, p.Wn), M, s.H, s.H, true, true, at<void>(ws, p.gx1), nullptr, nullptr, hdr};
+            GemmTcTN g{at<void>(ws, p.gz), at<void>(ws, p.Wn), M, s.H, s.H, false, true, at<void>(ws, p.gx1), nullptr, nullptr, hdr};
+            g.n_products = 2, g.planes_a = 1, g.planes_w = 2, g.prod_a = 0x00u, g.prod_w = 0x01u;   // gz_hi with lo, then hi
             if (int rc = launch_gemm_tc_tn(g, st)) return rc;
         } else {
             GemmTN g{at<void>(ws, p.gz), false, s.H, W, false, s.H, M, s.H, s.H, Epi::StoreF32,
@@ -541,13 +526,12 @@ SSM_API int ssm_glu_bwd(const ssm_shape* shape, const float* W, const void* v, c
     {   // dW[i, j] = sum_m x1[m, i] gz[m, j]
         StageTimer tm("glu_gemm_dW", st);
         if (p.tc) {
-            // (x1_hi + x1_lo)^T (gz_hi + gz_lo) as two products, one per plane of x1
-            GemmTcNT g{at<void>(ws, p.x1), s.H, at<void>(ws, p.gz), at<void>(ws, p.gz + n * 2), s.H, M, p.splits,
-                       at<float>(ws, p.part), hdr, 2 * s.H};
-            if (int rc = launch_gemm_tc_nt(g, st)) return rc;
-            g.A = at<void>(ws, p.x1 + (size_t)s.H * 2);   // the low halves: columns [H, 2H) of x1
-            g.part = at<float>(ws, p.part) + (size_t)p.splits * HH;
-            if (int rc = launch_gemm_tc_nt(g, st)) return rc;
+            // (x1_hi + x1_lo)^T (gz_hi + gz_lo) as two products, one per plane of x1 (column blocks of x1)
+            GemmTcNT g0{at<void>(ws, p.x1), 2 * s.H, at<void>(ws, p.gz), at<void>(ws, p.gz + n * 2), at<float>(ws, p.part)};
+            GemmTcNT g1 = g0;
+            g1.A = at<void>(ws, p.x1 + (size_t)s.H * 2);
+            g1.part = at<float>(ws, p.part) + (size_t)p.splits * HH;
+            if (int rc = launch_gemm_tc_nt2(M, s.H, s.H, p.splits, g0, g1, hdr, st)) return rc;
             launch_glu_reduce(at<float>(ws, p.part), 2 * p.splits, HH, dW, st);
         } else {
             GemmNT g{at<void>(ws, p.x1), false, s.H, at<void>(ws, p.gz), false, s.H, M, p.splits, at<float>(ws, p.part)};
@@ -561,6 +545,11 @@ SSM_API int ssm_glu_bwd(const ssm_shape* shape, const float* W, const void* v, c
     }
     SSM_RETURN_IF_CUDA_ERROR();
     return SSM_OK;
+}
+
+// dD's partial sums (rows of [H]) brought down to what the last kernel of the pass adds.
+static const float* reduce_dD(const ssm_shape& s, float* part, int* rows, cudaStream_t st) {
+    return launch_reduce_rows(part, *rows, s.H, part + (size_t)*rows * s.H, kMaxPartialRows, rows, st);
 }
 
 // What a layer's backward pass leaves for its last kernels, which a stack runs for all its layers together.
@@ -616,42 +605,28 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
             StageTimer tm("gemm_du", st);
             if (du_add) return SSM_ERR_SHAPE;   // the residual addend exists only on the CUDA-core path (stacks)
             GemmTcTN g{at<void>(ws, p.gs), at<void>(ws, p.W3), BT, s.H, P2, false, false, du, D, gy, hdr};
-            int rows = 0;
-            if (tc_tn_dot_supported(BT, s.H, P2)) {
-                g.dot = u;
-                g.dot_part = at<float>(ws, p.dot);
-                g.dot_rows = &rows;
-            }
+            if (tc_tn_dot_supported(BT, s.H)) g.dot = u, g.dot_part = at<float>(ws, p.dot), g.dot_rows = &dD_rows;
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
-            if (g.dot) {
-                dD_part = at<float>(ws, p.dot);
-                dD_rows = rows;
-            }
+            if (g.dot) dD_part = reduce_dD(s, g.dot_part, &dD_rows, st);
         }
-        {   // gBbar[p,h] = sum_m s[m,p] u[m,h]
-            StageTimer tm("gemm_gBbar", st);
-            GemmTcNT g{u, s.H, at<void>(ws, p.gs), at<void>(ws, p.gs + plane), P2, BT, p.splits, part, hdr};
-            if ((rc = launch_gemm_tc_nt(g, st))) return rc;
-        }
-        {   // dC[h,p] = sum_m gy[m,h] conj(x[m,p])
-            StageTimer tm("gemm_gC", st);
-            GemmTcNT g{gy, s.H, at<void>(ws, p.xs), at<void>(ws, p.xs + plane), P2, BT, p.splits, part_c, hdr};
-            if ((rc = launch_gemm_tc_nt(g, st))) return rc;
+        {   // gBbar[p,h] = sum_m s[m,p] u[m,h] and dC[h,p] = sum_m gy[m,h] conj(x[m,p])
+            StageTimer tm("gemm_gBbar_gC", st);
+            const GemmTcNT gB{u, s.H, at<void>(ws, p.gs), at<void>(ws, p.gs + plane), part};
+            const GemmTcNT gC{gy, s.H, at<void>(ws, p.xs), at<void>(ws, p.xs + plane), part_c};
+            if ((rc = launch_gemm_tc_nt2(BT, s.H, P2, p.splits, gB, gC, hdr, st))) return rc;
         }
     } else if (p.planes) {
         const bool gyb = io.gy_bf16, ub = io.u_bf16;
         {   // g_x = gy conj(C)
             StageTimer tm("gemm_gx", st);
-            const bool split_here = !gyb && tc_tn_small(BT, P2, false);
-            if (!gyb && !split_here) launch_split_planes((const float*)gy, (size_t)BT, s.H, at<void>(ws, p.gy3), st);
-            GemmTcTN g{gyb || split_here ? gy : at<void>(ws, p.gy3), at<void>(ws, p.W1), BT, P2, s.H, false, true, at<void>(ws, p.gs),
+            GemmTcTN g{gy, at<void>(ws, p.W1), BT, P2, s.H, false, true, at<void>(ws, p.gs),
                        nullptr, nullptr, hdr};
             g.n_products = gyb ? 3 : 6;
             g.planes_a = gyb ? 1 : 3;
             g.planes_w = 3;
             g.prod_a = gyb ? kProd3A : kProd6A;
             g.prod_w = gyb ? kProd3B : kProd6B;
-            if (split_here) g.a_f32 = true, g.a_planes_out = at<void>(ws, p.gy3);
+            if (!gyb) g.a_f32 = true, g.a_planes_out = at<void>(ws, p.gy3);
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
         }
         {
@@ -662,25 +637,19 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
                                  at<char>(ws, p.scan), st, &gA_part, &gA_rows);
             if (rc) return rc;
         }
-        {   // du = s Bq^T + D gy (+ the residual branch's gradient); where the epilogue does that, dD's sums as well
+        {   // du = s Bq^T + D gy (+ the residual branch's gradient), and dD's sums
             StageTimer tm("gemm_du", st);
-            const bool small = tc_tn_small(BT, s.H, false);
-            if (!small) launch_split_planes(at<float>(ws, p.gs), (size_t)BT, P2, at<void>(ws, p.s3), st);
-            GemmTcTN g{small ? at<void>(ws, p.gs) : at<void>(ws, p.s3), at<void>(ws, p.W3), BT, s.H, P2, false, true, at<void>(ws, p.acc), nullptr,
-                       nullptr, hdr};
+            GemmTcTN g{at<void>(ws, p.gs), at<void>(ws, p.W3), BT, s.H, P2, false, !io.du_bf16, du, D, gy, hdr};
+            g.skip_bf16 = gyb, g.add = du_add;
+            g.dot = u, g.dot_bf16 = ub, g.dot_part = at<float>(ws, p.dot), g.dot_rows = &dD_rows;
             g.n_products = 6;
             g.planes_a = 3;
             g.planes_w = 3;
             g.prod_a = kProd6A;
             g.prod_w = kProd6B;
-            if (small) {
-                g.store_f32 = !io.du_bf16, g.out = du, g.diag = D, g.skip = gy, g.skip_bf16 = gyb, g.add = du_add;
-                g.dot = u, g.dot_bf16 = ub, g.dot_part = at<float>(ws, p.dot), g.dot_rows = &dD_rows;
-                dD_part = g.dot_part;
-                g.a_f32 = true, g.a_planes_out = at<void>(ws, p.s3);
-            }
+            g.a_f32 = true, g.a_planes_out = at<void>(ws, p.s3);
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
-            if (!small) launch_diag_skip(at<float>(ws, p.acc), D, gy, gyb, du_add, (size_t)BT, s.H, du, io.du_bf16, st);
+            dD_part = reduce_dD(s, g.dot_part, &dD_rows, st);
         }
         // gBbar = s^T u and dC = gy^T conj(x)
         left->products[0] = {ub ? u : at<void>(ws, p.u3), at<void>(ws, p.s3), ub ? 1 : 3, 3, ub ? 3 : 6, ub ? kProd3A : kProd6A,

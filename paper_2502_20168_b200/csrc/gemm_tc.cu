@@ -8,7 +8,7 @@
 //    the 256 accumulator columns of a tile hold the products with the high and the low bf16 halves of 128
 //    weight rows, summed in the epilogue (weights then carry ~16 mantissa bits; see
 //    pack_params_kernel).  With a product schedule the accumulator sums several products of bf16
-//    planes of both operands (fp32-accurate results, see planes.cu).  Epilogues: fp32 store; bf16
+//    planes of both operands (fp32-accurate results, see gemm_tc_small.cu).  Epilogues: fp32 store; bf16
 //    acc + diag * skip; the same with column sums of skip * dot; fp32 store with a gated bf16 result.
 //  * gemm_scan_fwd_kernel / gemm_scan_bwd_kernel: the pair kernel with the scan of Sec. III-B (and its
 //    adjoint) in the epilogue, so that Bu and g_x never reach memory.  The CTAs of a pair take two
@@ -21,6 +21,7 @@
 // warps drain accumulators (each may read one TMEM lane quarter).  Every mbarrier wait is bounded; a wait
 // that gives up raises a CTA-wide abort flag, the status word of the workspace header is set, tensor
 // memory is released and the kernel returns.
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <utility>
@@ -247,7 +248,7 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
     if (!mbar_wait(s.tmem_full(acc), acc_phase, s.abort_flag)) return false;
     tc_fence_after();
     if (kEpi == 2) {
-        // z = acc (hi + lo columns) goes out in fp32, skip * sigmoid(z) in bf16; one staging buffer each
+        // z = acc goes out in fp32, skip * sigmoid(z) in bf16; one staging buffer each
         float4* stg = reinterpret_cast<float4*>(stg_bytes);
         uint8_t* ob = stg_bytes + 4096;
 #pragma unroll
@@ -255,7 +256,7 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
             const int c = (slab0 + sl) * 32, b = sl & 1;
             uint32_t r[32], r2[32];
             tmem_ld32(t_row + (uint32_t)c, r);
-            tmem_ld32(t_row + (uint32_t)(BN / 2 + c), r2);
+            if (kSplitW) tmem_ld32(t_row + (uint32_t)(BN / 2 + c), r2);
             if (!mbar_wait(sbar[b], (skip_phase >> b) & 1u, s.abort_flag)) return false;
             skip_phase ^= 1u << b;
             uint4 sk[4];
@@ -279,13 +280,13 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
                 __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&o[j]);
                 float z[8];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) z[e] = __uint_as_float(r[8 * j + e]) + __uint_as_float(r2[8 * j + e]);
+                for (int e = 0; e < 8; ++e) z[e] = __uint_as_float(r[8 * j + e]) + (kSplitW ? __uint_as_float(r2[8 * j + e]) : 0.f);
                 stg[lane * 8 + ((2 * j) ^ (lane & 7))] = make_float4(z[0], z[1], z[2], z[3]);
                 stg[lane * 8 + ((2 * j + 1) ^ (lane & 7))] = make_float4(z[4], z[5], z[6], z[7]);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float2 sf = __bfloat1622float2(s2[e]);
-                    o2[e] = __floats2bfloat162_rn(sf.x / (1.f + __expf(-z[2 * e])), sf.y / (1.f + __expf(-z[2 * e + 1])));
+                    o2[e] = __floats2bfloat162_rn(gate_value(sf.x, z[2 * e]), gate_value(sf.y, z[2 * e + 1]));
                 }
                 *reinterpret_cast<uint4*>(ob + lane * 64 + ((j ^ swz) << 4)) = o[j];
             }
@@ -1602,16 +1603,21 @@ struct NtParams {
     int K;              // rows of A and Bm (the reduction index)
     int J;              // columns of Bm = leading dimension of a partial
     int I;              // columns of A
-    int j_tiles;        // J / BN
+    int j_tiles;        // J / (BN / 2)
     int blocks_per_split;  // k-blocks (of BK rows) per slice
-    float* part;        // [splits, I, J]
+    int first;          // the product blockIdx.z = 0 stands for
+    float* part[2];     // [splits, I, J] each
     WsHeader* hdr;
+};
+struct NtMaps {
+    CUtensorMap a[2], hi[2], lo[2];   // per product
 };
 
 // The 256 accumulator columns are 128 output columns times the two planes (hi, lo) of Bm, added in the epilogue.
 __global__ void __launch_bounds__(kThreads, 1)
-gemm_tc_nt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBhi,
-                  const __grid_constant__ CUtensorMap tmBlo, NtParams p) {
+gemm_tc_nt_kernel(const __grid_constant__ NtMaps maps, const __grid_constant__ NtParams p) {
+    const int z = (int)blockIdx.z + p.first;
+    const CUtensorMap &tmA = maps.a[z], &tmBhi = maps.hi[z], &tmBlo = maps.lo[z];
     extern __shared__ uint8_t smem_raw[];
     const Smem s = carve_smem(smem_raw, kStages, 0, 0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1680,7 +1686,7 @@ gemm_tc_nt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     } else {
         const int q = warp & 3;
         const int row = i0 + q * 32 + lane;
-        float* dst_row = p.part + ((size_t)split * p.I + row) * p.J + j0;
+        float* dst_row = p.part[z] + ((size_t)split * p.I + row) * p.J + j0;
         bool ok = true;
         if (nkb > 0) {
             ok = mbar_wait(s.tmem_full(0), 0, s.abort_flag);
@@ -1730,8 +1736,9 @@ constexpr int kNtPairStageBytes = kABytes + kBBytes / 2;   // 32 KB
 constexpr size_t kNtPairSmemBytes = (size_t)kNtPairStages * kNtPairStageBytes + 1024 + 256;
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-gemm_tc_nt_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBhi,
-                       const __grid_constant__ CUtensorMap tmBlo, NtParams p) {
+gemm_tc_nt_pair_kernel(const __grid_constant__ NtMaps maps, const __grid_constant__ NtParams p) {
+    const int z = (int)blockIdx.z + p.first;
+    const CUtensorMap &tmA = maps.a[z], &tmBhi = maps.hi[z], &tmBlo = maps.lo[z];
     extern __shared__ uint8_t smem_raw[];
     const Smem s = carve_smem(smem_raw, kNtPairStages, 0, 0, kNtPairStageBytes, 0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1816,7 +1823,7 @@ gemm_tc_nt_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     } else {
         const int q = warp & 3;
         const int row = i0 + q * 32 + lane;
-        float* dst_row = p.part + ((size_t)split * p.I + row) * p.J + j0;
+        float* dst_row = p.part[z] + ((size_t)split * p.I + row) * p.J + j0;
         bool ok = true;
         if (nkb > 0) {
             ok = mbar_wait(s.tmem_full(0), 0, s.abort_flag);
@@ -1909,31 +1916,37 @@ bool tc_tn_supported(int M, int N_out, int K, bool split_w) {
 
 static int pair_tiles_of(int M, int n_tiles) { return ((M + 2 * tc::BM - 1) / (2 * tc::BM)) * n_tiles; }
 
-// Too few 256-row tiles to give every CTA pair one.
-bool tc_tn_small(int M, int N_out, bool split_w) {
-    const int out_cols = split_w ? tc::BN / 2 : tc::BN;
-    return pair_tiles_of(M, (N_out + out_cols - 1) / out_cols) < tc::sm_count() / 2;
+// Whether a projection has enough 256 x 256 tiles for the kernel on CTA pairs; the others take gemm_tc_small.cu.
+// us back to back, pairs / few tiles, by number of tiles:
+//   acc + diag * skip:         24 tiles 9.3 / 9.5, 32: 12.2 / 12.4, 48: 9.7 / 11.6, 64: 12.7 / 14.6
+//   the same with column sums: 32: 11.5 / 10.1, 48: 12.0 / 14.2 (the pair kernel keeps the sums of kDotMaxN columns)
+//   hi + lo weights:           32: 6.6 / 5.9 and 10.4 / 11.9, 48: 7.9 / 8.9, 128: 17.4 / 25.0
+//   two products of planes:    64: 19.8 / 17.8, 94: 20.4 / 23.5, 512: 111 / 133;  with the gate 94: 33.0 / 32.8, 512: 118 / 134
+// Six products of planes, whose planes the few-tile kernel loads once, stay there at every size.
+enum { kEpiStore = 0, kEpiDiag = 1, kEpiGate = 2, kEpiDot = 3 };
+static int epi_of(const GemmTcTN& g) { return g.gate_out ? kEpiGate : (g.store_f32 && !g.diag ? kEpiStore : (g.dot ? kEpiDot : kEpiDiag)); }
+static bool use_pairs(const GemmTcTN& g) {
+    if (g.n_products > 3 || g.a_f32 || g.add || (g.diag && g.store_f32)) return false;
+    const int out_cols = g.split_w ? tc::BN / 2 : tc::BN, tiles = pair_tiles_of(g.M, (g.N_out + out_cols - 1) / out_cols);
+    const int epi = epi_of(g);
+    if (epi == kEpiDot && g.N_out > tc::kDotMaxN) return false;
+    return tiles >= (g.n_products > 0 ? 80 : (epi == kEpiDiag ? 32 : 40));
 }
-
-// The bf16 epilogue can also sum skip * dot over the rows (one partial row per CTA); the pair kernel does for outputs
-// of at most kDotMaxN columns.
-bool tc_tn_dot_supported(int M, int N_out, int K) {
-    return tc_tn_supported(M, N_out, K, false) && (tc_tn_small(M, N_out, false) || N_out <= tc::kDotMaxN);
-}
-int tc_tn_dot_max_rows(int M, int N_out) {
-    return tc_tn_small(M, N_out, false) ? tc_tn_small_max_dot_rows(M) : 2 * tc::sm_count();
-}
+// Whether acc + diag * skip also leaves the column sums of skip * dot: not for many rows of very wide outputs, which the
+// pair kernel takes faster without than the few-tile kernel with them.
+bool tc_tn_dot_supported(int M, int N_out) { return N_out <= tc::kDotMaxN || pair_tiles_of(M, (N_out + tc::BN - 1) / tc::BN) < 32; }
+// Most rows of column sums a projection leaves.
+int tc_tn_dot_max_rows(int M) { return std::max(tc_tn_small_max_dot_rows(M), 2 * tc::sm_count()); }
 
 int launch_gemm_tc_tn(const GemmTcTN& g, cudaStream_t st) {
     using namespace tc;
-    if (tc_tn_small(g.M, g.N_out, g.split_w)) return launch_gemm_tc_tn_small(g, st);
-    if (g.a_f32 || g.add || g.w_plane_rows) return SSM_ERR_SHAPE;
+    if (!use_pairs(g)) return launch_gemm_tc_tn_small(g, st);
     const int out_cols = g.split_w ? BN / 2 : BN;
     const int n_tiles = (g.N_out + out_cols - 1) / out_cols;
-    const int epi = g.gate_out ? 2 : (g.store_f32 ? 0 : (g.dot ? 3 : 1));
+    const int epi = epi_of(g);
     if ((epi == 1 || epi == 3) && (g.split_w || !g.diag || !g.skip)) return SSM_ERR_SHAPE;
-    if (epi == 3 && (!g.dot_part || !g.dot_rows || !tc_tn_dot_supported(g.M, g.N_out, g.K))) return SSM_ERR_SHAPE;
-    if (epi == 2 && (!g.split_w || !g.store_f32 || !g.skip)) return SSM_ERR_SHAPE;
+    if (epi == 3 && (!g.dot_part || !g.dot_rows)) return SSM_ERR_SHAPE;
+    if (epi == 2 && (g.split_w || !g.store_f32 || !g.skip)) return SSM_ERR_SHAPE;
     CUtensorMap ma, mw, mo, ms, mg;
     // with a product schedule the operands are planes_a / planes_w bf16 planes of K columns each, side by side
     const int n_prod = g.n_products > 0 ? g.n_products : 1;
@@ -1975,7 +1988,7 @@ do {                                                                            
     if (ok && g.dot_rows) *g.dot_rows = 2 * min(pairs, pair_tiles);                                    \
 } while (0)
     if (epi == 3) SSM_LAUNCH_PAIR(3, false);
-    else if (epi == 2) SSM_LAUNCH_PAIR(2, true);
+    else if (epi == 2) SSM_LAUNCH_PAIR(2, false);
     else if (epi == 1) SSM_LAUNCH_PAIR(1, false);
     else if (g.split_w) SSM_LAUNCH_PAIR(0, true);
     else SSM_LAUNCH_PAIR(0, false);
@@ -2120,42 +2133,54 @@ int launch_gemm_scan_bwd(const GemmScanBwd& g, cudaStream_t st) {
 
 bool tc_nt_supported(int I, int J) { return (I % tc::BM) == 0 && (J % (tc::BN / 2)) == 0; }
 
-int tc_nt_splits(int K, int I, int J) {
-    const int tiles = (I / tc::BM) * (J / (tc::BN / 2));
+// Both products of a pair in one launch where the slices then still are short (a launch costs about 5 us of ramp and
+// drain that the next one hides only partly; 0.35 us per k-block and CTA), else one launch each with twice the slices.
+struct NtPlan {
+    bool pairs, together;
+    int splits;
+};
+static NtPlan nt_plan(int K, int I, int J) {
+    const bool pairs = I % (2 * tc::BM) == 0;
+    const int tiles = (pairs ? I / (2 * tc::BM) : I / tc::BM) * (J / (tc::BN / 2));
+    const int slots = pairs ? tc::sm_count() / 2 : tc::sm_count();
     const int blocks = (K + tc::BK - 1) / tc::BK;
-    int s = tc::sm_count() / (tiles > 0 ? tiles : 1);
-    if (s < 1) s = 1;
-    if (s > blocks) s = blocks;
-    if (s > 64) s = 64;
-    return s;
+    auto clamp = [&](int s) { return std::max(1, std::min(std::min(s, blocks), 64)); };
+    const int one = clamp(slots / tiles), two = clamp(slots / (2 * tiles));
+    auto rounds = [&](int units) { return (units + slots - 1) / slots; };
+    const double t_one = 2.0 * (rounds(tiles * one) * ((blocks + one - 1) / one) * 0.35 + 5.0);
+    const double t_two = rounds(2 * tiles * two) * ((blocks + two - 1) / two) * 0.35 + 7.0;
+    return t_two < t_one ? NtPlan{pairs, true, two} : NtPlan{pairs, false, one};
 }
+int tc_nt_splits(int K, int I, int J) { return nt_plan(K, I, J).splits; }
 
-#ifndef SSM_NT_PAIRS
-#define SSM_NT_PAIRS 1   // weight-gradient products on CTA pairs where the output has a multiple of 256 rows
-#endif
-int launch_gemm_tc_nt(const GemmTcNT& g, cudaStream_t st) {
+int launch_gemm_tc_nt2(int K, int I, int J, int splits, const GemmTcNT& g0, const GemmTcNT& g1, WsHeader* hdr, cudaStream_t st) {
     using namespace tc;
-    CUtensorMap ma, mbh, mbl;
-    const int blocks = (g.K + BK - 1) / BK;
-    const int bps = (blocks + g.splits - 1) / g.splits;
-    if (!make_map(&ma, g.A, (uint64_t)g.K, (uint64_t)g.I, 64, BK, false, CU_TENSOR_MAP_SWIZZLE_128B, (uint64_t)g.lda))
-        return SSM_ERR_CUDA;
-    if (!make_map(&mbh, g.Bm_hi, (uint64_t)g.K, (uint64_t)g.J, 64, BK)) return SSM_ERR_CUDA;
-    if (!make_map(&mbl, g.Bm_lo, (uint64_t)g.K, (uint64_t)g.J, 64, BK)) return SSM_ERR_CUDA;
-    const int j_tiles = g.J / (BN / 2);
-    NtParams p{g.K, g.J, g.I, j_tiles, bps, g.part, g.hdr};
-    if (SSM_NT_PAIRS && g.I % (2 * BM) == 0) {   // 256 x 256 tiles on CTA pairs
-        dim3 grid(2 * (g.I / (2 * BM)) * j_tiles, g.splits);
-        count_launch();
-        const bool ok = set_smem(gemm_tc_nt_pair_kernel, kNtPairSmemBytes);
-        launch_dep(gemm_tc_nt_pair_kernel, grid, kThreads, kNtPairSmemBytes, st, ma, mbh, mbl, p);
-        return ok ? SSM_OK : SSM_ERR_CUDA;
+    const NtPlan plan = nt_plan(K, I, J);
+    if (splits != plan.splits) return SSM_ERR_SHAPE;
+    NtMaps maps;
+    const GemmTcNT* g[2] = {&g0, &g1};
+    for (int z = 0; z < 2; ++z) {
+        if (!make_map(&maps.a[z], g[z]->A, (uint64_t)K, (uint64_t)I, 64, BK, false, CU_TENSOR_MAP_SWIZZLE_128B, (uint64_t)g[z]->lda))
+            return SSM_ERR_CUDA;
+        if (!make_map(&maps.hi[z], g[z]->Bm_hi, (uint64_t)K, (uint64_t)J, 64, BK)) return SSM_ERR_CUDA;
+        if (!make_map(&maps.lo[z], g[z]->Bm_lo, (uint64_t)K, (uint64_t)J, 64, BK)) return SSM_ERR_CUDA;
     }
-    dim3 grid((g.I / BM) * j_tiles, g.splits);
-    count_launch();
-    const bool ok = set_smem(gemm_tc_nt_kernel, kNtSmemBytes);
-    launch_dep(gemm_tc_nt_kernel, grid, kThreads, kNtSmemBytes, st, ma, mbh, mbl, p);
-    return ok ? SSM_OK : SSM_ERR_CUDA;
+    const int blocks = (K + BK - 1) / BK, j_tiles = J / (BN / 2);
+    NtParams p{K, J, I, j_tiles, (blocks + splits - 1) / splits, 0, {g0.part, g1.part}, hdr};
+    for (; p.first < 2; p.first += plan.together ? 2 : 1) {
+        const unsigned nz = plan.together ? 2 : 1;
+        count_launch();
+        bool ok;
+        if (plan.pairs) {   // 256 x 256 tiles on CTA pairs
+            ok = set_smem(gemm_tc_nt_pair_kernel, kNtPairSmemBytes) &&
+                 launch_dep(gemm_tc_nt_pair_kernel, dim3(2 * (I / (2 * BM)) * j_tiles, splits, nz), kThreads, kNtPairSmemBytes, st, maps, p);
+        } else {
+            ok = set_smem(gemm_tc_nt_kernel, kNtSmemBytes) &&
+                 launch_dep(gemm_tc_nt_kernel, dim3((I / BM) * j_tiles, splits, nz), kThreads, kNtSmemBytes, st, maps, p);
+        }
+        if (!ok) return SSM_ERR_CUDA;
+    }
+    return SSM_OK;
 }
 
 }  // namespace ssm

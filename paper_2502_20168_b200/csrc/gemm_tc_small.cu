@@ -281,8 +281,7 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         const float4 s4 = sk[i0 + i].get(true);
                         *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + e) = v[i];
                         *reinterpret_cast<uint2*>(p.gate_out + e) =
-                            pack4_bf16(make_float4(s4.x / (1.f + __expf(-v[i].x)), s4.y / (1.f + __expf(-v[i].y)),
-                                                   s4.z / (1.f + __expf(-v[i].z)), s4.w / (1.f + __expf(-v[i].w))));
+                            pack4_bf16(make_float4(gate_value(s4.x, v[i].x), gate_value(s4.y, v[i].y), gate_value(s4.z, v[i].z), gate_value(s4.w, v[i].w)));
                     }
                 }
             }
@@ -382,9 +381,7 @@ int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st) {
     } else if (g.n_products > 0) {
         p.planes_a = g.planes_a, p.planes_w = g.planes_w, p.n_prod = g.n_products;
         p.prod_a = g.prod_a, p.prod_w = g.prod_w;
-        p.w_plane_cols = g.w_plane_rows ? 0 : g.K;
-        p.w_plane_rows = g.w_plane_rows;
-        p.w_stacked = g.w_plane_rows ? 1 : 0;
+        p.w_plane_cols = g.K;
     } else {
         p.planes_a = p.planes_w = p.n_prod = 1;
     }
@@ -408,8 +405,7 @@ int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st) {
     CUtensorMap ma, mw;
     const uint64_t w_rows = (uint64_t)g.N_out * (p.w_stacked ? p.planes_w : 1);
     const uint64_t w_cols = (uint64_t)g.K * (p.w_stacked ? 1 : p.planes_w);
-    if (!make_map(&mw, g.W, w_rows, w_cols, BK, (uint32_t)s.bn, false, CU_TENSOR_MAP_SWIZZLE_128B, (uint64_t)g.w_pitch))
-        return SSM_ERR_CUDA;
+    if (!make_map(&mw, g.W, w_rows, w_cols, BK, (uint32_t)s.bn)) return SSM_ERR_CUDA;
     ma = mw;   // unused when A is split here
     if (!g.a_f32 && !make_map(&ma, g.A, (uint64_t)g.M, (uint64_t)g.K * p.planes_a, BK, BM)) return SSM_ERR_CUDA;
     const bool io_bf16 = g.skip_bf16 && (!g.dot || g.dot_bf16);

@@ -118,10 +118,10 @@ struct GemmTcTN {
     void* out;
     const float* diag; const void* skip;   // bf16 result: out = acc + diag[n] * skip[m, n]
     WsHeader* hdr;
-    // Gate (with store_f32 and skip; split_w or a product schedule): besides the fp32 result also gate_out[m, n] =
+    // Gate (with store_f32, skip and a product schedule): besides the fp32 result also gate_out[m, n] =
     // bf16(skip[m, n] * sigmoid(acc)).
     void* gate_out = nullptr;
-    // Column sums (with the bf16 epilogue, where tc_tn_dot_supported says so): dot_part[c, n] = sum over the
+    // Column sums (with diag and skip): dot_part[c, n] = sum over the
     // rows m that CTA c drained of skip[m, n] * dot[m, n]; *dot_rows receives the number of rows c written
     // (at most tc_tn_dot_max_rows()).  dot: bf16 [M, N_out].
     const void* dot = nullptr;
@@ -132,22 +132,18 @@ struct GemmTcTN {
     // product j multiplies plane (prod_a >> 4 j) & 15 of A by plane (prod_w >> 4 j) & 15 of W.  fp32 result only.
     int n_products = 0, planes_a = 1, planes_w = 1;
     uint32_t prod_a = 0, prod_w = 0;
-    // Only where tc_tn_small says so (the kernel for problems of few tiles):
+    // (These are left to the kernel of gemm_tc_small.cu.)
     bool a_f32 = false;                  // A is fp32 [M, K]; its three planes are made on the way to the tensor cores ...
     void* a_planes_out = nullptr;        // ... and, if asked for, stored [M, 3K] for a later kernel
     bool skip_bf16 = true, dot_bf16 = true;   // types of skip and dot; with diag and store_f32 the result is fp32
     const float* add = nullptr;          // fp32 [M, N_out], added to acc + diag * skip
-    int w_plane_rows = 0;                // planes of W this many rows apart in blocks of 128 rows (as with split_w) ...
-    int w_pitch = 0;                     // ... and its row pitch in elements, if it is not K
 };
 bool tc_tn_supported(int M, int N_out, int K, bool split_w);
-// Whether a projection has too few 256 x 256 tiles for the kernels on CTA pairs and takes the one of gemm_tc_small.cu.
-bool tc_tn_small(int M, int N_out, bool split_w);
 int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st);
 int tc_tn_small_max_dot_rows(int M);
 int tc_max_n();   // widest output of the tensor-core projections
-bool tc_tn_dot_supported(int M, int N_out, int K);
-int tc_tn_dot_max_rows(int M, int N_out);
+bool tc_tn_dot_supported(int M, int N_out);
+int tc_tn_dot_max_rows(int M);
 int launch_gemm_tc_tn(const GemmTcTN& g, cudaStream_t st);
 
 // One step for B trajectories in one kernel (gemm_tc_step.cu), from the operands of the tensor-core path (f32 = false:
@@ -219,16 +215,17 @@ int launch_gemm_scan_bwd(const GemmScanBwd& g, cudaStream_t st);
 // *gA_rows <= kMaxPartialRows rows at *gA_part_out; the caller sums those.
 int launch_gemm_scan_bwd_part(GemmScanBwd g, void* scratch, const float2** gA_part_out, int* gA_rows, cudaStream_t st);
 
+// Weight-gradient products: part[s, i, j] = sum_{m in slice s} A[m, i] * (Bm_hi[m, j] + Bm_lo[m, j]);  A bf16 [K, I]
+// with lda elements between rows, Bm_hi / Bm_lo bf16 [K, J]: the two planes of a state tensor.
 struct GemmTcNT {
-    // part[s, i, j] = sum_{m in slice s} A[m, i] * (Bm_hi[m, j] + Bm_lo[m, j]);  A bf16 [K, I],
-    // Bm_hi / Bm_lo bf16 [K, J]: the two planes of a state tensor
-    const void* A; int I;
-    const void* Bm_hi; const void* Bm_lo; int J;
-    int K; int splits;
-    float* part;
-    WsHeader* hdr;
-    int lda = 0;   // elements between rows of A when A is a column block of a wider matrix (0: I)
+    const void* A; int lda;
+    const void* Bm_hi; const void* Bm_lo;
+    float* part;   // [splits, I, J]
 };
+bool tc_nt_supported(int I, int J);
+// Slices of the rows for a pair of products of one shape.
+int tc_nt_splits(int K, int I, int J);
+int launch_gemm_tc_nt2(int K, int I, int J, int splits, const GemmTcNT& g0, const GemmTcNT& g1, WsHeader* hdr, cudaStream_t st);
 // Weight-gradient products of fp32 layers from planes (gemm_tc_nt_planes.cu), two per layer: A = planes_a planes of I
 // columns side by side, B = planes_b planes of J columns; product schedules as in GemmTcTN.  I, J multiples of 128.
 struct GemmTcNtPlanes {
@@ -240,21 +237,11 @@ struct GemmTcNtPlanes {
 int tc_nt_planes_splits(int K, int I, int J, int n_products);
 int launch_gemm_tc_nt_planes(int K, int I, int J, int splits, int n_products, const GemmTcNtPlanes* products, WsHeader* hdr,
                              cudaStream_t st);
-bool tc_nt_supported(int I, int J);
-int tc_nt_splits(int K, int I, int J);
-int launch_gemm_tc_nt(const GemmTcNT& g, cudaStream_t st);
-
-// planes.cu: fp32 tensors as three bf16 planes side by side ([M, K] -> [M, 3K]) so that a
-// projection with fp32 inputs runs on the bf16 tensor cores as a sum of plane products (GemmTcTN / GemmTcNT
-// with a product schedule), and what follows such a projection: out = acc + diag * skip (+ add).
-void launch_split_planes(const float* in, size_t M, int K, void* out, cudaStream_t st);
-void launch_diag_skip(const float* acc, const float* diag, const void* skip, bool skip_bf16, const float* add, size_t M,
-                      int N, void* out, bool out_bf16, cudaStream_t st);
 
 // glu.cu: what surrounds the GEMMs of the half-GLU gate out = v * sigmoid(GELU(v) W).
-// Tensor-core path (may be NULL): Wt2 [2H, 2H], the hi/lo stacked operand of z = [x1_hi | x1_lo] W, and
-// Wn_split [2H, H], that of g_x1 = gz W^T;  Wt_f32 (CUDA-core path, may be NULL): W transposed.
-void launch_glu_pack(int H, const float* W, void* Wt2, void* Wn_split, float* Wt_f32, cudaStream_t st);
+// Tensor-core path (may be NULL): Wz, Wn [H, 2H], hi | lo planes of W transposed (z = x1 W) and of W (g_x1 = gz W^T);
+// Wt_f32 (CUDA-core path, may be NULL): W transposed.  Clears the header's status word.
+void launch_glu_pack(int H, const float* W, void* Wz, void* Wn, float* Wt_f32, WsHeader* hdr, cudaStream_t st);
 // x1 = GELU(v); planes: bf16 [M, 2H], high halves in columns [0, H), low halves in [H, 2H); else fp32 [M, H]
 void launch_glu_gelu(bool io_bf16, bool planes, size_t n, int H, const void* v, void* x1, cudaStream_t st);
 void launch_glu_out(bool io_bf16, size_t n, const void* v, const float* z, void* out, cudaStream_t st);
