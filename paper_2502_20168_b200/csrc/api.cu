@@ -238,6 +238,25 @@ static void layer_prepare(const ssm_shape& s, const LayerPlan& p, const ssm_c64*
         launch_discretize_pack_f32(s.H, s.P, 1, &job, hdr, st);
 }
 
+// One projection of the plane path.  `g` has its fp32 or bf16 operand in A; `planes` is where the planes of an fp32
+// operand go (keep: they are wanted later, by the weight gradients).
+static int plane_projection(GemmTcTN g, bool a_bf16, void* planes, bool keep, cudaStream_t st) {
+    g.n_products = a_bf16 ? 3 : 6;
+    g.planes_a = a_bf16 ? 1 : 3;
+    g.planes_w = 3;
+    g.prod_a = a_bf16 ? kProd3A : kProd6A;
+    g.prod_w = a_bf16 ? kProd3B : kProd6B;
+    if (tc_planes_many_tiles(g.M, g.N_out)) {
+        if (!a_bf16) {
+            launch_split_planes((const float*)g.A, (size_t)g.M, g.K, planes, st);
+            g.A = planes;
+        }
+        return launch_gemm_tc_planes(g, st);
+    }
+    if (!a_bf16) g.a_f32 = true, g.a_planes_out = keep ? planes : nullptr;
+    return launch_gemm_tc_tn(g, st);
+}
+
 // Launch sequence of one layer's forward pass from a prepared workspace.  `hdr` receives the
 // status of bounded waits.  keep_planes: a backward pass will follow (fp32 layers leave the planes of u and x for it).
 // Storage types of the tensors a layer reads and writes.  For the entry points of a single layer all
@@ -290,15 +309,8 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
     } else if (p.planes) {
         {   // Bu = u Bbar^T as a sum of plane products (u: three planes of an fp32 input, or the bf16 input itself)
             StageTimer tm("gemm_Bu", st);
-            GemmTcTN g{u, at<void>(ws, p.W0), BT, P2, s.H, false, true, at<void>(ws, p.xs),
-                       nullptr, nullptr, hdr};
-            g.n_products = io.u_bf16 ? 3 : 6;
-            g.planes_a = io.u_bf16 ? 1 : 3;
-            g.planes_w = 3;
-            g.prod_a = io.u_bf16 ? kProd3A : kProd6A;
-            g.prod_w = io.u_bf16 ? kProd3B : kProd6B;
-            if (!io.u_bf16) g.a_f32 = true, g.a_planes_out = keep_planes ? at<void>(ws, p.u3) : nullptr;
-            if ((rc = launch_gemm_tc_tn(g, st))) return rc;
+            const GemmTcTN g{u, at<void>(ws, p.W0), BT, P2, s.H, false, true, at<void>(ws, p.xs), nullptr, nullptr, hdr};
+            if ((rc = plane_projection(g, io.u_bf16, at<void>(ws, p.u3), keep_planes, st))) return rc;
         }
         {
             StageTimer tm("scan_fwd", st);
@@ -311,13 +323,7 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
             StageTimer tm("gemm_y", st);
             GemmTcTN g{at<void>(ws, p.xs), at<void>(ws, p.W2), BT, s.H, P2, false, !io.y_bf16, y, D, u, hdr};
             g.skip_bf16 = io.u_bf16;
-            g.n_products = 6;
-            g.planes_a = 3;
-            g.planes_w = 3;
-            g.prod_a = kProd6A;
-            g.prod_w = kProd6B;
-            g.a_f32 = true, g.a_planes_out = keep_planes ? at<void>(ws, p.x3) : nullptr;
-            if ((rc = launch_gemm_tc_tn(g, st))) return rc;
+            if ((rc = plane_projection(g, false, at<void>(ws, p.x3), keep_planes, st))) return rc;
         }
     } else {
         {
@@ -619,15 +625,8 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
         const bool gyb = io.gy_bf16, ub = io.u_bf16;
         {   // g_x = gy conj(C)
             StageTimer tm("gemm_gx", st);
-            GemmTcTN g{gy, at<void>(ws, p.W1), BT, P2, s.H, false, true, at<void>(ws, p.gs),
-                       nullptr, nullptr, hdr};
-            g.n_products = gyb ? 3 : 6;
-            g.planes_a = gyb ? 1 : 3;
-            g.planes_w = 3;
-            g.prod_a = gyb ? kProd3A : kProd6A;
-            g.prod_w = gyb ? kProd3B : kProd6B;
-            if (!gyb) g.a_f32 = true, g.a_planes_out = at<void>(ws, p.gy3);
-            if ((rc = launch_gemm_tc_tn(g, st))) return rc;
+            const GemmTcTN g{gy, at<void>(ws, p.W1), BT, P2, s.H, false, true, at<void>(ws, p.gs), nullptr, nullptr, hdr};
+            if ((rc = plane_projection(g, gyb, at<void>(ws, p.gy3), true, st))) return rc;
         }
         {
             StageTimer tm("scan_bwd", st);
@@ -642,13 +641,7 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
             GemmTcTN g{at<void>(ws, p.gs), at<void>(ws, p.W3), BT, s.H, P2, false, !io.du_bf16, du, D, gy, hdr};
             g.skip_bf16 = gyb, g.add = du_add;
             g.dot = u, g.dot_bf16 = ub, g.dot_part = at<float>(ws, p.dot), g.dot_rows = &dD_rows;
-            g.n_products = 6;
-            g.planes_a = 3;
-            g.planes_w = 3;
-            g.prod_a = kProd6A;
-            g.prod_w = kProd6B;
-            g.a_f32 = true, g.a_planes_out = at<void>(ws, p.s3);
-            if ((rc = launch_gemm_tc_tn(g, st))) return rc;
+            if ((rc = plane_projection(g, false, at<void>(ws, p.s3), true, st))) return rc;
             dD_part = reduce_dD(s, g.dot_part, &dD_rows, st);
         }
         // gBbar = s^T u and dC = gy^T conj(x)

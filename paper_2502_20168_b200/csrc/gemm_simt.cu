@@ -23,6 +23,18 @@ __device__ __forceinline__ void load4<__nv_bfloat16>(const __nv_bfloat16* p, flo
     v[0] = __low2float(lo); v[1] = __high2float(lo); v[2] = __low2float(hi); v[3] = __high2float(hi);
 }
 
+template <typename T>
+__device__ __forceinline__ void store4(T* p, const float (&v)[4]);
+template <>
+__device__ __forceinline__ void store4<float>(float* p, const float (&v)[4]) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+template <>
+__device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* p, const float (&v)[4]) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
+    *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+}
+
 struct EpiArgs {
     void* out;
     const float* diag;
@@ -38,7 +50,6 @@ __global__ void __launch_bounds__(kGemmThreads)
 gemm_tn_kernel(const TA* A, int lda, const TB* Bm, int ldb, int M, int N, int K,
                EpiArgs e) {
     grid_dep_wait();
-    grid_dep_launch();
     __shared__ __align__(16) float As[TK][TM + 4];
     __shared__ __align__(16) float Bs[TK][TN + 4];
     const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;   // rows along x: grid.y is limited to 65535
@@ -47,16 +58,22 @@ gemm_tn_kernel(const TA* A, int lda, const TB* Bm, int ldb, int M, int N, int K,
     const int lk = (tid & 3) * 4;    // 0,4,8,12: k offset
     const int tx = tid & 15, ty = tid >> 4;  // 16 x 16 threads, 4 x 4 outputs each
     float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += TK) {
-        float va[4] = {0.f, 0.f, 0.f, 0.f}, vb[4] = {0.f, 0.f, 0.f, 0.f};
+    float va[4], vb[4];
+    auto fetch = [&](int k0) {   // the next block's operands, on their way while this one is multiplied
+#pragma unroll
+        for (int i = 0; i < 4; ++i) va[i] = vb[i] = 0.f;
         if (m0 + lr < M && k0 + lk < K) load4<TA>(A + (size_t)(m0 + lr) * lda + k0 + lk, va);
         if (n0 + lr < N && k0 + lk < K) load4<TB>(Bm + (size_t)(n0 + lr) * ldb + k0 + lk, vb);
+    };
+    fetch(0);
+    for (int k0 = 0; k0 < K; k0 += TK) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             As[lk + i][lr] = va[i];
             Bs[lk + i][lr] = vb[i];
         }
         __syncthreads();
+        if (k0 + TK < K) fetch(k0 + TK);
 #pragma unroll
         for (int k = 0; k < TK; ++k) {
             const float4 a = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
@@ -69,23 +86,32 @@ gemm_tn_kernel(const TA* A, int lda, const TB* Bm, int ldb, int M, int N, int K,
         }
         __syncthreads();
     }
-    TO* out = reinterpret_cast<TO*>(e.out);
+    // Not earlier: the next kernel's blocks would be placed while this one's fill the SMs unevenly, and with several blocks
+    // per SM that imbalance lasted (6272 x 176 x 168: 17 -> 28 us).
+    grid_dep_launch();
+    // 4 neighbouring columns at a time (N is a multiple of 8); everything is read before anything is written
+    const int n = n0 + tx * 4;
+    if (n >= N) return;
+    if (kAddDiag) {
+        const float4 dg = *reinterpret_cast<const float4*>(e.diag + n);
+        float sk[4][4], ad[4][4] = {};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int m = m0 + ty * 4 + i;
+            if (m >= M) continue;
+            load4<TS>(reinterpret_cast<const TS*>(e.skip) + (size_t)m * e.ldo + n, sk[i]);
+            if (e.add) load4<float>(reinterpret_cast<const float*>(e.add) + (size_t)m * e.ldo + n, ad[i]);
+        }
+        const float dd[4] = {dg.x, dg.y, dg.z, dg.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(dd[j], sk[i][j], acc[i][j]) + ad[i][j];
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int m = m0 + ty * 4 + i;
-        if (m >= M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + tx * 4 + j;
-            if (n >= N) continue;
-            float v = acc[i][j];
-            if (kAddDiag) {
-                const TS* skip = reinterpret_cast<const TS*>(e.skip);
-                v = fmaf(e.diag[n], to_f32<TS>(skip[(size_t)m * e.ldo + n]), v);
-                if (e.add) v += reinterpret_cast<const float*>(e.add)[(size_t)m * e.ldo + n];
-            }
-            out[(size_t)m * e.ldo + n] = from_f32<TO>(v);
-        }
+        if (m < M) store4<TO>(reinterpret_cast<TO*>(e.out) + (size_t)m * e.ldo + n, acc[i]);
     }
 }
 
@@ -122,7 +148,6 @@ __global__ void __launch_bounds__(kGemmThreads)
 gemm_nt_kernel(const TA* A, int I, const TB* Bm, int J, int K, int k_per_split,
                float* part) {
     grid_dep_wait();
-    grid_dep_launch();
     __shared__ __align__(16) float As[TK][TM + 4];
     __shared__ __align__(16) float Bs[TK][TN + 4];
     const int i0 = blockIdx.y * TM, j0 = blockIdx.x * TN;
@@ -132,15 +157,21 @@ gemm_nt_kernel(const TA* A, int I, const TB* Bm, int J, int K, int k_per_split,
     const int lc = (tid & 15) * 4;    // 0..60
     const int tx = tid & 15, ty = tid >> 4;
     float acc[4][4] = {};
-    for (int k0 = kb; k0 < ke; k0 += TK) {
-        float va[4] = {0.f, 0.f, 0.f, 0.f}, vb[4] = {0.f, 0.f, 0.f, 0.f};
+    float va[4], vb[4];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) va[i] = vb[i] = 0.f;
         if (k0 + lk < ke) {
             if (i0 + lc < I) load4<TA>(A + (size_t)(k0 + lk) * I + i0 + lc, va);
             if (j0 + lc < J) load4<TB>(Bm + (size_t)(k0 + lk) * J + j0 + lc, vb);
         }
+    };
+    fetch(kb);
+    for (int k0 = kb; k0 < ke; k0 += TK) {
         *reinterpret_cast<float4*>(&As[lk][lc]) = make_float4(va[0], va[1], va[2], va[3]);
         *reinterpret_cast<float4*>(&Bs[lk][lc]) = make_float4(vb[0], vb[1], vb[2], vb[3]);
         __syncthreads();
+        if (k0 + TK < ke) fetch(k0 + TK);
 #pragma unroll
         for (int k = 0; k < TK; ++k) {
             const float4 a = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
@@ -153,16 +184,14 @@ gemm_nt_kernel(const TA* A, int I, const TB* Bm, int J, int K, int k_per_split,
         }
         __syncthreads();
     }
+    grid_dep_launch();
     float* out = part + (size_t)blockIdx.z * I * J;
+    const int jj = j0 + tx * 4;
+    if (jj >= J) return;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int ii = i0 + ty * 4 + i;
-        if (ii >= I) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int jj = j0 + tx * 4 + j;
-            if (jj < J) out[(size_t)ii * J + jj] = acc[i][j];
-        }
+        if (ii < I) store4<float>(out + (size_t)ii * J + jj, acc[i]);
     }
 }
 

@@ -132,7 +132,7 @@ struct GemmTcTN {
     // product j multiplies plane (prod_a >> 4 j) & 15 of A by plane (prod_w >> 4 j) & 15 of W.  fp32 result only.
     int n_products = 0, planes_a = 1, planes_w = 1;
     uint32_t prod_a = 0, prod_w = 0;
-    // (These are left to the kernel of gemm_tc_small.cu.)
+    // (These are left to the kernel of gemm_tc_small.cu; skip, dot and add in any type also to gemm_tc_planes.cu.)
     bool a_f32 = false;                  // A is fp32 [M, K]; its three planes are made on the way to the tensor cores ...
     void* a_planes_out = nullptr;        // ... and, if asked for, stored [M, 3K] for a later kernel
     bool skip_bf16 = true, dot_bf16 = true;   // types of skip and dot; with diag and store_f32 the result is fp32
@@ -140,6 +140,8 @@ struct GemmTcTN {
 };
 bool tc_tn_supported(int M, int N_out, int K, bool split_w);
 int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st);
+bool tc_planes_many_tiles(int M, int N_out);
+int launch_gemm_tc_planes(const GemmTcTN& g, cudaStream_t st);   // gemm_tc_planes.cu: products of planes, many tiles
 int tc_tn_small_max_dot_rows(int M);
 int tc_max_n();   // widest output of the tensor-core projections
 bool tc_tn_dot_supported(int M, int N_out);
@@ -237,6 +239,9 @@ struct GemmTcNtPlanes {
 int tc_nt_planes_splits(int K, int I, int J, int n_products);
 int launch_gemm_tc_nt_planes(int K, int I, int J, int splits, int n_products, const GemmTcNtPlanes* products, WsHeader* hdr,
                              cudaStream_t st);
+
+// planes.cu: fp32 tensors as three bf16 planes side by side ([M, K] -> [M, 3K]).
+void launch_split_planes(const float* in, size_t M, int K, void* out, cudaStream_t st);
 
 // glu.cu: what surrounds the GEMMs of the half-GLU gate out = v * sigmoid(GELU(v) W).
 // Tensor-core path (may be NULL): Wz, Wn [H, 2H], hi | lo planes of W transposed (z = x1 W) and of W (g_x1 = gz W^T);

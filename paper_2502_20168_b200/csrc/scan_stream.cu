@@ -200,7 +200,6 @@ scan_fwd_stream_kernel(Args k, const __grid_constant__ CUtensorMap tm_in, const 
     const int tid = threadIdx.x;
     init_shared(sm);
     grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
-    grid_dep_launch();
     if (tid >= kConsumers) {
         producer<false>(k, sm, stages, stage_bytes, &tm_in, nullptr, nullptr, stage_bytes, 0, 0);
         return;
@@ -324,6 +323,7 @@ scan_fwd_stream_kernel(Args k, const __grid_constant__ CUtensorMap tm_in, const 
             tma_commit_group();
         }
     }
+    grid_dep_launch();   // (late: blocks placed beside this kernel's are placed unevenly)
     if (tid == 0) tma_store_wait_all();
 }
 
@@ -349,7 +349,6 @@ scan_bwd_stream_kernel(Args k, const __grid_constant__ CUtensorMap tm_g, const _
     const int tid = threadIdx.x;
     init_shared(sm);
     grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
-    grid_dep_launch();
     if (tid >= kConsumers) {
         if (sizeof(XS) == 4)
             producer<true>(k, sm, stages, stage_bytes, &tm_g, &tm_x0, &tm_x1, tile_bytes, tile_bytes / 2, tile_bytes / 2);
@@ -499,6 +498,7 @@ scan_bwd_stream_kernel(Args k, const __grid_constant__ CUtensorMap tm_g, const _
             gA_part[(size_t)b * k.P + p] = sum;   // every (sequence, state) belongs to exactly one chain
         }
     }
+    grid_dep_launch();   // (late: blocks placed beside this kernel's are placed unevenly)
     if (tid == 0) tma_store_wait_all();
 }
 

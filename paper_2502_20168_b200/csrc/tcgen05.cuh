@@ -135,6 +135,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         : "r"(taddr)
         : "memory");
 }
+// The same for 16 columns.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Shared-memory matrix descriptors (128-byte swizzle).  Fields: start address >> 4 in bits
@@ -151,6 +161,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes,
 }
 // K-major tile: rows of 128 bytes, groups of 8 rows 1024 bytes apart (leading offset unused).
 __device__ __forceinline__ uint64_t smem_desc_kmajor(uint32_t addr) { return smem_desc(addr, 16, 1024); }
+// K-major tile with rows of 64 bytes (64-byte swizzle, mode 4), groups of 8 rows 512 bytes apart.
+__device__ __forceinline__ uint64_t smem_desc_kmajor64(uint32_t addr) {
+    return (smem_desc(addr, 16, 512) & ~((uint64_t)7 << 61)) | ((uint64_t)4 << 61);
+}
 // MN-major tile made of [BK rows][64 elements] blocks: 64-element blocks 8192 bytes apart,
 // groups of 8 k-rows 1024 bytes apart.
 __device__ __forceinline__ uint64_t smem_desc_mnmajor(uint32_t addr) { return smem_desc(addr, BK * 128, 1024); }

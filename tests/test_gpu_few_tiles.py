@@ -31,3 +31,20 @@ def test_gate_edges_bf16(rows, H):
 def test_weight_gradients_from_planes_fp32(B, T, H, P):
     # one k-block and a row of the next; slices of several segments with a ragged end; one slice per tile
     run(I.Workload("nt32", B=B, T=T, H=H, P=P, io_dtype="f32", p_done=0.01, seed=B + T), with_gxT=True)
+
+
+@pytest.mark.parametrize("B,T,H,P", [(50, 131, 256, 128), (7, 301, 768, 384), (1, 12801, 256, 128)])
+def test_many_tiles_fp32(B, T, H, P):
+    # the persistent plane kernel: from 100 tiles on, a ragged last row of tiles, more tiles than CTAs
+    run(I.Workload("many32", B=B, T=T, H=H, P=P, io_dtype="f32", p_done=0.01, seed=B + H), with_x0=True, with_gxT=True)
+
+
+def test_many_tiles_of_a_bf16_stack():
+    # the first layer's bf16 input is one plane (three products), the last layer's output is bf16
+    from tests.test_gpu_stack_parity import run as run_stack
+    run_stack(I.Workload("many_stack", B=50, T=131, H=256, P=128, io_dtype="bf16", p_done=0.01, n_layers=2, seed=3))
+
+
+@pytest.mark.parametrize("rows,H", [(5000, 512), (10300, 640)])
+def test_gate_on_both_sides_of_the_pair_kernel_bf16(rows, H):
+    run_gate(I.Workload("gate_pair", B=1, T=rows, H=H, P=8, io_dtype="bf16", seed=rows + H))
