@@ -53,7 +53,7 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true) {
     p.tc = allow_tc && s.io_dtype == SSM_BF16 && tc_tn_supported((int)BT, P2, s.H, true) &&
            tc_tn_supported((int)BT, s.H, P2, false) && tc_nt_supported(s.H, P2);
     p.planes = !p.tc && s.io_dtype == SSM_F32 && planes_supported(s);
-    p.splits = p.tc ? tc_nt_splits((int)BT, s.H, P2) : (p.planes ? tc_nt_planes_splits((int)BT, s.H, P2, 2) : gemm_nt_splits((int)BT));
+    p.splits = p.tc ? tc_nt_splits((int)BT, s.H, P2) : (p.planes ? tc_nt_planes_splits((int)BT, s.H, P2, 2) : gemm_nt_splits((int)BT, s.H, P2));
     p.hdr = take(off, sizeof(WsHeader));
     p.Abar = take(off, (size_t)s.P * 8);
     p.Alo = take(off, (size_t)s.P * 8);
@@ -438,7 +438,7 @@ GluPlan plan_glu(const ssm_shape& s) {
     size_t off = 0;
     const size_t M = (size_t)s.B * s.T, HH = (size_t)s.H * s.H;
     p.tc = s.io_dtype == SSM_BF16 && tc_tn_supported((int)M, s.H, s.H, false) && tc_nt_supported(s.H, s.H);
-    p.splits = p.tc ? tc_nt_splits((int)M, s.H, s.H) : gemm_nt_splits((int)M);
+    p.splits = p.tc ? tc_nt_splits((int)M, s.H, s.H) : gemm_nt_splits((int)M, s.H, s.H);
     p.hdr = take(off, sizeof(WsHeader));
     p.Wt = take(off, HH * 4);   // W^T: bf16 planes hi | lo [H, 2H], or fp32
     p.Wn = take(off, p.tc ? 2 * HH * 2 : 0);
@@ -540,8 +540,8 @@ SSM_API int ssm_glu_bwd(const ssm_shape* shape, const float* W, const void* v, c
             if (int rc = launch_gemm_tc_nt2(M, s.H, s.H, p.splits, g0, g1, hdr, st)) return rc;
             launch_glu_reduce(at<float>(ws, p.part), 2 * p.splits, HH, dW, st);
         } else {
-            GemmNT g{at<void>(ws, p.x1), false, s.H, at<void>(ws, p.gz), false, s.H, M, p.splits, at<float>(ws, p.part)};
-            launch_gemm_nt(g, st);
+            const GemmNT g{at<void>(ws, p.x1), false, s.H, at<float>(ws, p.gz), s.H, M, p.splits, at<float>(ws, p.part)};
+            launch_gemm_nt(&g, 1, nullptr, st);
             launch_glu_reduce(at<float>(ws, p.part), p.splits, HH, dW, st);
         }
     }
@@ -670,15 +670,14 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
                       du, io.du_bf16, D, gy, io.gy_bf16, du_add};
             launch_gemm_tn(g4, st);
         }
-        {
-            StageTimer tm("gemm_gBbar", st);
-            GemmNT g5{u, io.u_bf16, s.H, at<void>(ws, p.gs), false, P2, BT, p.splits, part};
-            launch_gemm_nt(g5, st);
-        }
-        {
-            StageTimer tm("gemm_gC", st);
-            GemmNT g6{gy, io.gy_bf16, s.H, at<void>(ws, p.xs), false, P2, BT, p.splits, part_c};
-            launch_gemm_nt(g6, st);
+        {   // both weight gradients, and the row groups' sums of gy * u for dD
+            StageTimer tm("gemm_gBbar_gC", st);
+            const GemmNT g[2] = {{u, io.u_bf16, s.H, at<float>(ws, p.gs), P2, BT, p.splits, part},
+                                 {gy, io.gy_bf16, s.H, at<float>(ws, p.xs), P2, BT, p.splits, part_c}};
+            const SimtDot dot{gy, u, io.gy_bf16, io.u_bf16, at<float>(ws, p.dot)};
+            launch_gemm_nt(g, 2, &dot, st);
+            dD_rows = dot_groups(BT);
+            dD_part = reduce_dD(s, at<float>(ws, p.dot), &dD_rows, st);
         }
     }
     if (!dD_part) {   // dD[h] = sum_m gy[m,h] u[m,h], unless the du projection left its partial sums already

@@ -1,6 +1,8 @@
 // fp32-accumulate CUDA-core GEMMs.  They serve the fp32 workloads (whose 1e-4 tolerance a
 // single-pass reduced-precision tensor-core product cannot meet; those shapes are tiny) and
 // any shape the tensor-core path does not take.
+#include <algorithm>
+
 #include "kernels.h"
 
 namespace ssm {
@@ -142,16 +144,66 @@ void launch_gemm_tn(const GemmTN& g, cudaStream_t st) {
     else dispatch_tn<float, float>(g, st);
 }
 
-// part[s,i,j] = sum_{k in slice s} A[k,i] Bm[k,j]; both operands contiguous in i / j.
-template <typename TA, typename TB>
+// part[s,i,j] = sum_{k in slice s} A[k,i] Bm[k,j]; both operands contiguous in i / j, Bm fp32.  Up to two products of one
+// shape (blockIdx.z = product * splits + slice) and, behind them, the column dot products of a and b: a layer's weight
+// gradients and dD in one launch, which at the sizes this path is for are a few microseconds each.
+struct NtSimtArgs {
+    GemmNT g[2];
+    int n, k_per_split;
+    const void *dot_a, *dot_b;
+    bool dot_a_bf16, dot_b_bf16;
+    float* dot_part;
+    int dot_groups, dot_blocks;   // row groups; blocks the dot products take
+};
+
+__device__ __forceinline__ void load4_any(const void* p, bool bf16, size_t i, float (&v)[4]) {
+    if (bf16) load4<__nv_bfloat16>(reinterpret_cast<const __nv_bfloat16*>(p) + i, v);
+    else load4<float>(reinterpret_cast<const float*>(p) + i, v);
+}
+
 __global__ void __launch_bounds__(kGemmThreads)
-gemm_nt_kernel(const TA* A, int I, const TB* Bm, int J, int K, int k_per_split,
-               float* part) {
+gemm_nt_kernel(const __grid_constant__ NtSimtArgs q) {
     grid_dep_wait();
     __shared__ __align__(16) float As[TK][TM + 4];
     __shared__ __align__(16) float Bs[TK][TN + 4];
+    const int z = (int)blockIdx.z / q.g[0].splits;
+    if (z >= q.n) {   // dot products: block = 32 column quads x 8 row lanes, kDotRows rows
+        const int extra = (int)blockIdx.z - q.n * q.g[0].splits;
+        const int blk = (extra * (int)gridDim.y + (int)blockIdx.y) * (int)gridDim.x + (int)blockIdx.x;
+        grid_dep_launch();
+        if (blk >= q.dot_blocks) return;
+        const int C = q.g[0].I, M = q.g[0].K, grp = blk % q.dot_groups, c = (blk / q.dot_groups * 32 + (threadIdx.x & 31)) * 4;
+        const int rl = threadIdx.x >> 5, r0 = grp * kDotRows, r1 = min(M, r0 + kDotRows);
+        float4(*sm)[32] = reinterpret_cast<float4(*)[32]>(&As[0][0]);   // 8 x 32 float4 = 4 KB
+        static_assert(sizeof(As) >= 8 * 32 * sizeof(float4), "the dot products' sums fit the operand tile");
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        if (c < C) {
+#pragma unroll 4
+            for (int r = r0 + rl; r < r1; r += 8) {
+                float va[4], vb[4];
+                load4_any(q.dot_a, q.dot_a_bf16, (size_t)r * C + c, va);
+                load4_any(q.dot_b, q.dot_b_bf16, (size_t)r * C + c, vb);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[i] = fmaf(va[i], vb[i], acc[i]);
+            }
+        }
+        sm[rl][threadIdx.x & 31] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        __syncthreads();
+        if (rl == 0 && c < C) {
+            float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float4 v = sm[i][threadIdx.x];
+                t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+            }
+            *reinterpret_cast<float4*>(q.dot_part + (size_t)grp * C + c) = t;
+        }
+        return;
+    }
+    const GemmNT& g = q.g[z];
+    const int slice = (int)blockIdx.z - z * g.splits, I = g.I, J = g.J;
     const int i0 = blockIdx.y * TM, j0 = blockIdx.x * TN;
-    const int kb = blockIdx.z * k_per_split, ke = min(K, kb + k_per_split);
+    const int kb = slice * q.k_per_split, ke = min(g.K, kb + q.k_per_split);
     const int tid = threadIdx.x;
     const int lk = tid >> 4;          // 0..15
     const int lc = (tid & 15) * 4;    // 0..60
@@ -162,8 +214,8 @@ gemm_nt_kernel(const TA* A, int I, const TB* Bm, int J, int K, int k_per_split,
 #pragma unroll
         for (int i = 0; i < 4; ++i) va[i] = vb[i] = 0.f;
         if (k0 + lk < ke) {
-            if (i0 + lc < I) load4<TA>(A + (size_t)(k0 + lk) * I + i0 + lc, va);
-            if (j0 + lc < J) load4<TB>(Bm + (size_t)(k0 + lk) * J + j0 + lc, vb);
+            if (i0 + lc < I) load4_any(g.A, g.a_bf16, (size_t)(k0 + lk) * I + i0 + lc, va);
+            if (j0 + lc < J) load4<float>(g.Bm + (size_t)(k0 + lk) * J + j0 + lc, vb);
         }
     };
     fetch(kb);
@@ -185,7 +237,7 @@ gemm_nt_kernel(const TA* A, int I, const TB* Bm, int J, int K, int k_per_split,
         __syncthreads();
     }
     grid_dep_launch();
-    float* out = part + (size_t)blockIdx.z * I * J;
+    float* out = g.part + (size_t)slice * I * J;
     const int jj = j0 + tx * 4;
     if (jj >= J) return;
 #pragma unroll
@@ -195,24 +247,30 @@ gemm_nt_kernel(const TA* A, int I, const TB* Bm, int J, int K, int k_per_split,
     }
 }
 
-int gemm_nt_splits(int K) {
-    int s = (K + 511) / 512;
-    return s < 1 ? 1 : (s > 64 ? 64 : s);
+// Slices of the rows for a pair of products: about three blocks per SM, at least 64 rows each (6272 rows, 168 x 176
+// outputs: one launch of 468 blocks 38 us, two of 117 59 us).
+int gemm_nt_splits(int K, int I, int J) {
+    const int tiles = ((J + TN - 1) / TN) * ((I + TM - 1) / TM);
+    const int want = 3 * device_sm_count() / (2 * tiles), most = (K + 63) / 64;
+    return std::max(1, std::min(std::min(want, most), 64));
 }
 
-void launch_gemm_nt(const GemmNT& g, cudaStream_t st) {
-    int kps = (g.K + g.splits - 1) / g.splits;
-    kps = (kps + TK - 1) / TK * TK;
-    dim3 grid((g.J + TN - 1) / TN, (g.I + TM - 1) / TM, g.splits);
+void launch_gemm_nt(const GemmNT* g, int n, const SimtDot* dot, cudaStream_t st) {
+    NtSimtArgs q{};
+    for (int i = 0; i < n; ++i) q.g[i] = g[i];
+    q.n = n;
+    const int kps = (g->K + g->splits - 1) / g->splits;
+    q.k_per_split = (kps + TK - 1) / TK * TK;
+    dim3 grid((g->J + TN - 1) / TN, (g->I + TM - 1) / TM, n * g->splits);
+    if (dot) {
+        q.dot_a = dot->a, q.dot_b = dot->b, q.dot_a_bf16 = dot->a_bf16, q.dot_b_bf16 = dot->b_bf16, q.dot_part = dot->part;
+        q.dot_groups = dot_groups(g->K);
+        q.dot_blocks = q.dot_groups * ((g->I + 127) / 128);
+        const int per_z = (int)(grid.x * grid.y);
+        grid.z += (q.dot_blocks + per_z - 1) / per_z;
+    }
     count_launch();
-    if (g.a_bf16 && g.b_bf16)
-        launch_dep(gemm_nt_kernel<__nv_bfloat16, __nv_bfloat16>, grid, kGemmThreads, 0, st, (const __nv_bfloat16*)g.A, g.I, (const __nv_bfloat16*)g.Bm, g.J, g.K, kps, g.part);
-    else if (g.a_bf16)
-        launch_dep(gemm_nt_kernel<__nv_bfloat16, float>, grid, kGemmThreads, 0, st, (const __nv_bfloat16*)g.A, g.I, (const float*)g.Bm, g.J, g.K, kps, g.part);
-    else if (g.b_bf16)
-        launch_dep(gemm_nt_kernel<float, __nv_bfloat16>, grid, kGemmThreads, 0, st, (const float*)g.A, g.I, (const __nv_bfloat16*)g.Bm, g.J, g.K, kps, g.part);
-    else
-        launch_dep(gemm_nt_kernel<float, float>, grid, kGemmThreads, 0, st, (const float*)g.A, g.I, (const float*)g.Bm, g.J, g.K, kps, g.part);
+    launch_dep(gemm_nt_kernel, grid, kGemmThreads, 0, st, q);
 }
 
 }  // namespace ssm

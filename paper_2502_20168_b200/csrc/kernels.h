@@ -76,6 +76,8 @@ size_t colsum_tmp_floats(int R, int C);
 // colsum_tmp_floats(R, C) floats, are both overwritten); returns where the rows are, *rows_out how many.
 const float* launch_reduce_rows(float* in, int R, int C, float* tmp, int limit, int* rows_out, cudaStream_t st);
 // part[g, c] = sum over the rows m of group g of a[m,c]*b[m,c]; a and b each fp32 or bf16.
+constexpr int kDotRows = 128;
+inline int dot_groups(int M) { return (M + kDotRows - 1) / kDotRows; }
 size_t dot_columns_tmp_floats(int M, int C);
 // The group sums only: tmp[g, c] for g < the returned number of groups.
 int launch_dot_columns_partial(bool a_bf16, const void* a, bool b_bf16, const void* b, int M, int C, float* tmp,
@@ -99,12 +101,20 @@ void launch_gemm_tn(const GemmTN& g, cudaStream_t st);
 struct GemmNT {
     // part[s, i, j] = sum_{k in slice s} A[k, i] * Bm[k, j]
     const void* A; bool a_bf16; int I;
-    const void* Bm; bool b_bf16; int J;
+    const float* Bm; int J;
     int K; int splits;
     float* part;
 };
-int gemm_nt_splits(int K);
-void launch_gemm_nt(const GemmNT& g, cudaStream_t st);
+// part[g, c] = sum over the rows k of group g (kDotRows rows) of a[k, c] * b[k, c]: rides along with the products, on
+// their K and I.
+struct SimtDot {
+    const void *a, *b;
+    bool a_bf16, b_bf16;
+    float* part;   // [dot_groups(K), I]
+};
+int gemm_nt_splits(int K, int I, int J);
+// n = 1 or 2 products of one shape in one launch, and dot (may be NULL).
+void launch_gemm_nt(const GemmNT* g, int n, const SimtDot* dot, cudaStream_t st);
 
 // gemm_tc.cu: bf16 projections on tcgen05 tensor cores (operands by TMA, accumulators in TMEM).
 struct GemmTcTN {

@@ -67,7 +67,6 @@ const float* launch_reduce_rows(float* in, int R, int C, float* tmp, int limit, 
 
 // part[g, c] = sum_{m in group g} a[m, c] * b[m, c].  A thread owns 4 neighbouring columns
 // (16 bytes of fp32, 8 bytes of bf16 per load); block = 32 column quads x 8 row lanes.
-constexpr int kDotRows = 128;
 template <typename T>
 __device__ __forceinline__ void load_quad(const T* p, float (&v)[4]);
 template <>
@@ -115,8 +114,6 @@ dot_columns_kernel(const TA* a, const TB* b, int M, int C, float* part) {
         *reinterpret_cast<float4*>(part + (size_t)blockIdx.x * C + c) = t;
     }
 }
-
-static inline int dot_groups(int M) { return (M + kDotRows - 1) / kDotRows; }
 
 size_t dot_columns_tmp_floats(int M, int C) {
     const int g = dot_groups(M);
