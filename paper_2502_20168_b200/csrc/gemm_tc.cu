@@ -577,9 +577,9 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 // halves of its results into its row group's part of the tile (everybody has read the tile by
 // then), which one lane per row group hands to the TMA unit (8-byte global stores from the
 // threads themselves measured 5 % slower).
-// T is a multiple of 128, or 16, 32 or 64: then a tile holds 128 / T whole sequences, a chain is one
-// tile, and every row group that begins a sequence starts from that sequence's initial state.
-// kTPair (few long sequences, T a multiple of 256): both CTAs of a pair walk ONE sequence, CTA 0 its
+// T = 16, 32 or 64: a tile holds 128 / T whole sequences, a chain is one tile, and every row group that
+// begins a sequence starts from that sequence's initial state.
+// kTPair (few long sequences): both CTAs of a pair walk ONE sequence, CTA 0 its
 // even tiles and CTA 1 its odd ones, which gives twice the chains at the full tile size.  Every row
 // group then folds from zero; the last row group joins the groups' results into the tile's own
 // contribution, waits for the state that enters the tile (written into this CTA's shared memory by
@@ -590,7 +590,7 @@ struct FsParams {
     int B, T, P;
     int n_tiles;      // state groups: P / kS
     int k_blocks;     // H / 64
-    int tblocks;      // tiles a CTA walks per chain: T / 128, or 1; kTPair: T / 256
+    int tblocks;      // tiles a CTA walks per chain: T / 128 rounded up, or 1; kTPair: T / 256 rounded up
     int unit_rows;    // rows of a chain: T, or 128 when T < 128
     int n_units;      // chains per state group: B, or ceil(B * T / 128)
     int gps;          // row groups per sequence inside a tile: 8, or T / 16
@@ -666,7 +666,7 @@ __device__ __forceinline__ C2 cstep2(f32x2 ar, f32x2 ai, f32x2 nai, C2 x, C2 b) 
 template <int kThreadsN>
 __device__ __forceinline__ void epi_sync_n() { asm volatile("bar.sync 1, %0;" ::"n"(kThreadsN) : "memory"); }
 
-template <int kS, bool kTPair>
+template <int kS, bool kTPair, bool kRagged>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FsCfg<kS>::kThreads, 1)
 gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmWh,
                      const __grid_constant__ CUtensorMap tmX, FsParams p) {
@@ -810,7 +810,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         for (int chain = pair; chain < p.nchains && ok; chain += npairs) {
             const int n_tile = chain % p.n_tiles, b = seq_of(chain);
             const bool has_seq = b < p.n_units;
-            const bool short_seq = !kTPair && p.T < BM;        // then b counts tiles of rows, not sequences
+            const bool short_seq = !kTPair && !kRagged && p.T < BM;        // then b counts tiles of rows, not sequences
             const int g0 = sl - sl % p.gps;         // the first row group of this group's sequence in the tile
             const bool from_carry = !kTPair && sl == g0;   // (kTPair: the carried state arrives late; every group joins)
             const int pg = n_tile * kS + 2 * sp;    // the first of this thread's two states
@@ -896,7 +896,10 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 // (2) scan: this thread's two states over its R rows.  The flags of a row group are the
                 // same for the whole warp: a group without flags takes loops without the tests.
                 const int r0 = sl * R;
-                const bool grp_valid = has_seq && m0 + r0 < M;           // (short sequences: the last tile may be ragged)
+                // kRagged: rows of the tile that lie inside the sequence (the others hold rows of the next one: nothing that
+                // is kept depends on them); else the last tile of short sequences may be ragged
+                const int left = p.T - (kTPair ? 2 * tb + (int)rank : tb) * BM;
+                const bool grp_valid = has_seq && (kRagged ? r0 < left : m0 + r0 < M);
                 const int b_grp = short_seq ? (m0 + r0) / p.T : b;      // this group's sequence
                 uint32_t gflags = 0;   // bit g: row group g has a flag
                 if (p.done) {
@@ -1029,24 +1032,41 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     out[i * kPairs] = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
                     out[(R + i) * kPairs] = make_uint2(*reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1));
                 };
+                C2 xend = zero;   // kRagged: the state after the sequence's last row, in the group that holds it
+                const int iend = left - 1 - r0;
                 if (from_carry) {
 #pragma unroll
-                    for (int i = 0; i < R; ++i) emit(i, v[i]);
+                    for (int i = 0; i < R; ++i) {
+                        emit(i, v[i]);
+                        if (kRagged && i == iend) xend = v[i];
+                    }
                 } else if (mask == 0u) {
 #pragma unroll
-                    for (int i = 0; i < R; ++i) emit(i, x = cstep2(ar, ai, nai, x, v[i]));
+                    for (int i = 0; i < R; ++i) {
+                        emit(i, x = cstep2(ar, ai, nai, x, v[i]));
+                        if (kRagged && i == iend) xend = x;
+                    }
                 } else {
 #pragma unroll
                     for (int i = 0; i < R; ++i) {
                         if ((mask >> i) & 1u) x = zero;
                         emit(i, x = cstep2(ar, ai, nai, x, v[i]));
+                        if (kRagged && i == iend) xend = x;
                     }
                 }
                 fence_async_smem();
                 __syncwarp();
                 if (group_leader && grp_valid) {
-                    tma_store_3d_nocommit(&tmX, smem_u32(warp_out), n_tile * kS, m0 + r0, 0);
+                    if (kRagged) tma_store_4d_nocommit(&tmX, smem_u32(warp_out), n_tile * kS, p.T - left + r0, b, 0);   // clipped at T
+                    else tma_store_3d_nocommit(&tmX, smem_u32(warp_out), n_tile * kS, m0 + r0, 0);
                     tma_commit_group();
+                }
+                if (kRagged && p.xT && has_seq && iend >= 0 && iend < R) {
+                    float x0r, x1r, x0i, x1i;
+                    unpack2(xend.re, x0r, x1r);
+                    unpack2(xend.im, x0i, x1i);
+                    p.xT[(size_t)b * p.P + pg] = make_float2(x0r, x0i);
+                    p.xT[(size_t)b * p.P + pg + 1] = make_float2(x1r, x1i);
                 }
                 if (short_seq ? (sl - g0 == p.gps - 1) : (sl == nsl - 1)) {   // the group that ends a sequence or the tile
                     float x0r, x1r, x0i, x1i;
@@ -1054,13 +1074,13 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     unpack2(x.im, x0i, x1i);
                     // (not after the chain's last tile: by then the first group may already have set up the next chain)
                     if (kTPair) {
-                        if (rank == 1 && tb == p.tblocks - 1 && p.xT) {
+                        if (!kRagged && rank == 1 && tb == p.tblocks - 1 && p.xT) {
                             p.xT[(size_t)b * p.P + pg] = make_float2(x0r, x0i);
                             p.xT[(size_t)b * p.P + pg + 1] = make_float2(x1r, x1i);
                         }
                     } else if (!short_seq && tb < p.tblocks - 1) {
                         carry_s[sp] = make_float4(x0r, x1r, x0i, x1i);
-                    } else if (p.xT && grp_valid) {
+                    } else if (!kRagged && p.xT && grp_valid) {
                         p.xT[(size_t)b_grp * p.P + pg] = make_float2(x0r, x0i);
                         p.xT[(size_t)b_grp * p.P + pg + 1] = make_float2(x1r, x1i);
                     }
@@ -1098,7 +1118,7 @@ struct FbParams {
     int B, T, P;
     int n_tiles;      // state groups: P / kS
     int k_blocks;     // H / 64
-    int tblocks;      // tiles a CTA walks per chain: T / 128, or 1; kTPair: T / 256
+    int tblocks;      // tiles a CTA walks per chain: T / 128 rounded up, or 1; kTPair: T / 256 rounded up
     int unit_rows;    // rows of a chain: T, or 128 when T < 128 (a tile then holds 128 / T whole sequences)
     int n_units;      // chains per state group: B, or ceil(B * T / 128)
     int gps;          // row groups per sequence inside a tile: 8, or T / 16
@@ -1112,7 +1132,7 @@ struct FbParams {
     WsHeader* hdr;
 };
 
-template <int kS, bool kTPair>
+template <int kS, bool kTPair, bool kRagged>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FsCfg<kS>::kThreads, 1)
 gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmWh,
                      const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmS, FbParams p) {
@@ -1232,7 +1252,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         const int sp = te % kPairs, sl = te / kPairs;   // scan role: pair of states of the tile, group of its rows
         const bool group_leader = lane % kPairs == 0;   // the lane that talks to the TMA unit for its row group
         const int prow = q * 32 + lane;             // drain role: row of the tile
-        const bool short_seq = !kTPair && p.T < BM;            // then a chain is one tile of 128 / T whole sequences
+        const bool short_seq = !kTPair && !kRagged && p.T < BM;            // then a chain is one tile of 128 / T whole sequences
         const int g0 = sl - sl % p.gps;             // first and last row group of this group's sequence in the tile
         const int gl = g0 + p.gps - 1;
         const bool from_carry = !kTPair && sl == gl;           // the last rows come first (kTPair: the carried value arrives late; every group joins)
@@ -1352,7 +1372,8 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 epi_sync();
                 // (2) this thread's two states over its R rows, last row first
                 const int r0 = sl * R;
-                const bool grp_valid = has_seq && m0 + r0 < M;           // (short sequences: the last tile may be ragged)
+                const int left = p.T - (kTPair ? 2 * tb + (int)rank : tb) * BM;   // kRagged: rows of the tile inside the sequence
+                const bool grp_valid = has_seq && (kRagged ? r0 < left : m0 + r0 < M);   // (short sequences: the last tile may be ragged)
                 const int b_grp = short_seq ? (m0 + r0) / p.T : b;      // this group's sequence
                 uint32_t gflags = 0;   // bit g: a reset acts inside or right after row group g
                 uint32_t mask = 0u, mask0 = 0u;
@@ -1375,7 +1396,19 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     v[i].re = pack2(t.x, t.y);
                     v[i].im = pack2(t.z, t.w);
                 }
-                if (sl == gl && tb == p.tblocks - 1 && (!kTPair || rank == 1) && p.gxT && grp_valid) {   // the gradient of the final state
+                if (kRagged && left < r0 + R) {   // rows of the next sequence: nothing may come from them
+#pragma unroll
+                    for (int i = 0; i < R; ++i)
+                        if (r0 + i >= left) v[i] = zero;
+                }
+                if (kRagged && p.gxT && has_seq && left > r0 && left <= r0 + R) {   // the gradient of the final state
+                    const float2 c0 = p.gxT[(size_t)b * p.P + pg], c1 = p.gxT[(size_t)b * p.P + pg + 1];
+                    const C2 add = {pack2(c0.x, c1.x), pack2(c0.y, c1.y)};
+#pragma unroll
+                    for (int i = 0; i < R; ++i)
+                        if (r0 + i == left - 1) v[i].re = add2(v[i].re, add.re), v[i].im = add2(v[i].im, add.im);
+                }
+                if (!kRagged && sl == gl && tb == p.tblocks - 1 && (!kTPair || rank == 1) && p.gxT && grp_valid) {   // the gradient of the final state
                     const float2 c0 = p.gxT[(size_t)b_grp * p.P + pg], c1 = p.gxT[(size_t)b_grp * p.P + pg + 1];
                     float v0, v1, v2, v3;
                     unpack2(v[R - 1].re, v0, v1);
@@ -1545,7 +1578,8 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 fence_async_smem();
                 __syncwarp();
                 if (group_leader && grp_valid) {
-                    tma_store_3d_nocommit(&tmS, smem_u32(warp_buf), n_tile * kS, m0 + r0, 0);
+                    if (kRagged) tma_store_4d_nocommit(&tmS, smem_u32(warp_buf), n_tile * kS, p.T - left + r0, b, 0);   // clipped at T
+                    else tma_store_3d_nocommit(&tmS, smem_u32(warp_buf), n_tile * kS, m0 + r0, 0);
                     tma_commit_group();
                 }
                 if (sl == g0) {   // x is s of the first row of the tile (of the sequence, when it lies inside the tile)
@@ -2009,6 +2043,20 @@ static bool make_plane_map(CUtensorMap* map, const void* planes, int M, int P, i
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same planes as [2, B, T, P] words, in boxes of one sequence: rows past a sequence's end are clipped.
+static bool make_plane_map4(CUtensorMap* map, const void* planes, int B, int T, int P, int states) {
+    PFN_cuTensorMapEncodeTiled fn = tc::encode_fn();
+    if (!fn) return false;
+    const cuuint64_t row = (cuuint64_t)P * 4;
+    cuuint64_t dims[4] = {(cuuint64_t)P, (cuuint64_t)T, (cuuint64_t)B, 2};
+    cuuint64_t strides[3] = {row, row * T, row * T * B};
+    cuuint32_t box[4] = {(cuuint32_t)states, (cuuint32_t)tc::kFsRows, 1, 2};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, const_cast<void*>(planes), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Fewest (sequence, state group) chain pairs for which the kernels that scan in the epilogue of a projection
 // are taken: below it too many CTA pairs would idle while a few walk their chains tile by tile.
 #ifndef SSM_FUSED_MIN_PAIRS
@@ -2018,8 +2066,11 @@ static bool make_plane_map(CUtensorMap* map, const void* planes, int M, int P, i
 #define SSM_FUSED_NARROW_BELOW 0   // 0: chains of 32 states where chains of 64 would occupy at most half of the CTA pairs
 #endif
 
+// Sequences whose rows do not fall on tile boundaries: a sequence's last tile is then partly empty.
+static bool fs_ragged(int T) { return !(T % tc::BM == 0 || T == 16 || T == 32 || T == 64); }
+static int fs_tiles(int T) { return (T + tc::BM - 1) / tc::BM; }   // tiles of a sequence (T a multiple of BM, or ragged)
 // Chains per state group: the sequences, or, when a 128-row tile holds several whole sequences, the tiles.
-static int fs_units(int B, int T) { return T >= tc::BM ? B : (B * T + tc::BM - 1) / tc::BM; }
+static int fs_units(int B, int T) { return T >= tc::BM || fs_ragged(T) ? B : (B * T + tc::BM - 1) / tc::BM; }
 
 // How the kernels that scan in their epilogue take a problem: chains of 64 states, of 32 (few sequences: twice
 // the chains, half the tile), or not at all (group 0); and, for few long sequences, both CTAs of a pair on one
@@ -2033,33 +2084,47 @@ struct FusedMode {
     bool time_pairs;
 };
 static FusedMode fused_mode(int B, int T, int H, int P) {
-    const bool t_ok = T % tc::BM == 0 || T == 16 || T == 32 || T == 64;
-    if (!t_ok || H % tc::BK != 0 || P % 64 != 0) return {0, false};
+    if (H % tc::BK != 0 || P % 64 != 0) return {0, false};
+    const bool ragged = fs_ragged(T);
     const int pairs64 = (P / 64) * ((fs_units(B, T) + 1) / 2);
+    const int np = tc::sm_count() / 2;
     // A tile of 32 states takes about 0.8 of the time of a tile of 64 (measured), so halving the chains pays only
     // where the second half of the CTA pairs would otherwise idle: 16 x 16384 at P = 256 1.88 -> 1.78 ms per step,
     // 16 x 1024 0.242 -> 0.229; with 64 of 74 pairs busy (32 sequences) it costs 30 - 50 % in these kernels.
     // Time pairs double the chains at the full tile: 16 x 16384 1.76 -> 1.48 ms, 16 x 1024 0.228 -> 0.212.
     const int narrow_below = SSM_FUSED_NARROW_BELOW > 0 ? SSM_FUSED_NARROW_BELOW : tc::sm_count() / 4 + 1;
-    const bool tp_ok = SSM_FUSED_TIME_PAIRS && T % (2 * tc::BM) == 0;
+    const bool tp_ok = SSM_FUSED_TIME_PAIRS && (T % (2 * tc::BM) == 0 || (ragged && T > tc::BM));
+    // Rounds of chains x tiles per chain: what the kernels' time goes with.
+    const int tiles = T >= tc::BM || ragged ? fs_tiles(T) : 1, tp_tiles = (T + 2 * tc::BM - 1) / (2 * tc::BM);
+    const int steps = (pairs64 + np - 1) / np * tiles;
+    const int tp_chains = (P / 64) * B, tp_steps = (tp_chains + np - 1) / np * tp_tiles;
+    FusedMode m{0, false};
     if (pairs64 >= narrow_below) {
         // Enough chains either way.  Time pairs give twice the chains at half the length, which fills the last
         // round of chains better when there are only a few rounds (48 sequences at P = 256: 96 chains take two
         // rounds on 74 CTA pairs, 192 half-length chains three half-rounds).
-        const int np = tc::sm_count() / 2;
-        const int rounds = (pairs64 + np - 1) / np, half_rounds = (2 * pairs64 + np - 1) / np;
-        return {64, tp_ok && half_rounds < 2 * rounds};
+        m = {64, tp_ok && tp_steps < steps};
+    } else if (tp_ok && tp_chains >= SSM_FUSED_MIN_PAIRS) {
+        m = {64, true};
+    } else if (pairs64 >= SSM_FUSED_MIN_PAIRS) {
+        m = {32, false};
     }
-    if (tp_ok && (P / 64) * B >= SSM_FUSED_MIN_PAIRS) return {64, true};
-    if (pairs64 < SSM_FUSED_MIN_PAIRS) return {0, false};
-    return {32, false};
+    // A ragged length costs the empty rows of each sequence's last tile (empty = rows of its tiles / T).  us per forward and
+    // backward pass, separate / fused, at H, P = 512, 256 unless stated:
+    //   empty 1.02: 16 x 1000 165 / 136, 60 x 3000 1248 / 1020;  1.1: 9 x 2500 (H 256) 202 / 174, 30 x 1100 (256, 128) 146 / 126
+    //   1.28: 16 x 100 69.5 / 60.5, 64 x 100 99 / 85, 150 x 200 (384, 192) 198 / 191;  1.42: 700 x 90 (256, 128) 219 / 211
+    //   1.6: 100 x 80 106 / 97;  1.78: 1000 x 72 508 / 523;  1.94: 200 x 66 153 / 146;  2.6: 500 x 50 235 / 262;  3.2: 2000 x 40 561 / 786
+    // With few rounds the time is latency, which empty rows do not lengthen.
+    const int empty16 = ragged ? 16 * tc::BM * fs_tiles(T) / T : 16;
+    if (empty16 > 26 && !(empty16 <= 32 && (m.time_pairs ? tp_steps : steps) <= 8)) return {0, false};
+    return m;
 }
 int tc_gemm_scan_group(int B, int T, int H, int P) { return fused_mode(B, T, H, P).group; }
 bool tc_gemm_scan_time_pairs(int B, int T, int H, int P) { return fused_mode(B, T, H, P).time_pairs; }
 bool tc_gemm_scan_fwd_supported(int B, int T, int H, int P) { return tc_gemm_scan_group(B, T, H, P) != 0; }
 bool tc_gemm_scan_bwd_supported(int B, int T, int H, int P) { return tc_gemm_scan_group(B, T, H, P) != 0; }
 
-template <int kS, bool kTPair>
+template <int kS, bool kTPair, bool kRagged>
 static int launch_gemm_scan_fwd_s(const GemmScanFwd& g, cudaStream_t st) {
     using namespace tc;
     using Cfg = FsCfg<kS>;
@@ -2067,17 +2132,17 @@ static int launch_gemm_scan_fwd_s(const GemmScanFwd& g, cudaStream_t st) {
     CUtensorMap ma, mw, mx;
     if (!make_map(&ma, g.u, (uint64_t)M, (uint64_t)g.H, BK, BM)) return SSM_ERR_CUDA;
     if (!make_map(&mw, g.Wsplit, (uint64_t)4 * g.P, (uint64_t)g.H, BK, Cfg::kWRows)) return SSM_ERR_CUDA;
-    if (!make_plane_map(&mx, g.x_planes, M, g.P, kS)) return SSM_ERR_CUDA;
+    if (!(kRagged ? make_plane_map4(&mx, g.x_planes, g.B, g.T, g.P, kS) : make_plane_map(&mx, g.x_planes, M, g.P, kS))) return SSM_ERR_CUDA;
     const int units = fs_units(g.B, g.T), n_tiles = g.P / kS;
-    FsParams p{g.B, g.T, g.P, n_tiles, g.H / BK, g.T >= BM ? g.T / BM : 1, g.T >= BM ? g.T : BM, units,
-               g.T >= BM ? BM / kFsRows : g.T / kFsRows, n_tiles * ((units + 1) / 2),
+    FsParams p{g.B, g.T, g.P, n_tiles, g.H / BK, kRagged ? fs_tiles(g.T) : (g.T >= BM ? g.T / BM : 1),
+               kRagged || g.T >= BM ? g.T : BM, units, kRagged || g.T >= BM ? BM / kFsRows : g.T / kFsRows, n_tiles * ((units + 1) / 2),
                g.Abar, g.done, g.x0, g.xT, (uint32_t*)g.x_planes, (size_t)M * g.P, g.hdr};
     if (kTPair) {   // a chain is one sequence; each CTA has every other tile
-        p.tblocks = g.T / (2 * BM);
+        p.tblocks = (g.T + 2 * BM - 1) / (2 * BM);
         p.nchains = n_tiles * g.B;
     }
     count_launch();
-    auto kern = gemm_scan_fwd_kernel<kS, kTPair>;
+    auto kern = gemm_scan_fwd_kernel<kS, kTPair, kRagged>;
     if (!set_smem(kern, Cfg::kSmemBytes)) return SSM_ERR_CUDA;
     const int pairs = resident_pairs(reinterpret_cast<const void*>(kern), Cfg::kSmemBytes, Cfg::kThreads);
     if (pairs <= 0) return SSM_ERR_CUDA;
@@ -2085,11 +2150,16 @@ static int launch_gemm_scan_fwd_s(const GemmScanFwd& g, cudaStream_t st) {
     return SSM_OK;
 }
 
+template <bool kRagged>
+static int launch_gemm_scan_fwd_r(const GemmScanFwd& g, const FusedMode& m, cudaStream_t st) {
+    if (m.group == 64)
+        return m.time_pairs ? launch_gemm_scan_fwd_s<64, true, kRagged>(g, st) : launch_gemm_scan_fwd_s<64, false, kRagged>(g, st);
+    if (m.group == 32) return launch_gemm_scan_fwd_s<32, false, kRagged>(g, st);
+    return SSM_ERR_SHAPE;
+}
 int launch_gemm_scan_fwd(const GemmScanFwd& g, cudaStream_t st) {
     const FusedMode m = fused_mode(g.B, g.T, g.H, g.P);
-    if (m.group == 64) return m.time_pairs ? launch_gemm_scan_fwd_s<64, true>(g, st) : launch_gemm_scan_fwd_s<64, false>(g, st);
-    if (m.group == 32) return launch_gemm_scan_fwd_s<32, false>(g, st);
-    return SSM_ERR_SHAPE;
+    return fs_ragged(g.T) ? launch_gemm_scan_fwd_r<true>(g, m, st) : launch_gemm_scan_fwd_r<false>(g, m, st);
 }
 
 // Rows of gA_part that launch_gemm_scan_bwd writes: one per chain of a state group (two per sequence where both
@@ -2098,7 +2168,7 @@ int tc_gemm_scan_bwd_part_rows(int B, int T, int H, int P) {
     return fused_mode(B, T, H, P).time_pairs ? 2 * B : fs_units(B, T);
 }
 
-template <int kS, bool kTPair>
+template <int kS, bool kTPair, bool kRagged>
 static int launch_gemm_scan_bwd_s(const GemmScanBwd& g, cudaStream_t st) {
     using namespace tc;
     using Cfg = FsCfg<kS>;
@@ -2106,17 +2176,18 @@ static int launch_gemm_scan_bwd_s(const GemmScanBwd& g, cudaStream_t st) {
     CUtensorMap ma, mw, mx, ms;
     if (!make_map(&ma, g.gy, (uint64_t)M, (uint64_t)g.H, BK, BM)) return SSM_ERR_CUDA;
     if (!make_map(&mw, g.Wsplit, (uint64_t)4 * g.P, (uint64_t)g.H, BK, Cfg::kWRows)) return SSM_ERR_CUDA;
-    if (!make_plane_map(&mx, g.x_planes, M, g.P, kS) || !make_plane_map(&ms, g.s_planes, M, g.P, kS)) return SSM_ERR_CUDA;
+    if (!make_plane_map(&mx, g.x_planes, M, g.P, kS)) return SSM_ERR_CUDA;
+    if (!(kRagged ? make_plane_map4(&ms, g.s_planes, g.B, g.T, g.P, kS) : make_plane_map(&ms, g.s_planes, M, g.P, kS))) return SSM_ERR_CUDA;
     const int units = fs_units(g.B, g.T), n_tiles = g.P / kS;
-    FbParams p{g.B, g.T, g.P, n_tiles, g.H / BK, g.T >= BM ? g.T / BM : 1, g.T >= BM ? g.T : BM, units,
-               g.T >= BM ? BM / kFsRows : g.T / kFsRows, n_tiles * ((units + 1) / 2),
+    FbParams p{g.B, g.T, g.P, n_tiles, g.H / BK, kRagged ? fs_tiles(g.T) : (g.T >= BM ? g.T / BM : 1),
+               kRagged || g.T >= BM ? g.T : BM, units, kRagged || g.T >= BM ? BM / kFsRows : g.T / kFsRows, n_tiles * ((units + 1) / 2),
                g.Abar, g.done, g.x0, g.gxT, g.gA_part, g.gx0, g.hdr};
     if (kTPair) {
-        p.tblocks = g.T / (2 * BM);
+        p.tblocks = (g.T + 2 * BM - 1) / (2 * BM);
         p.nchains = n_tiles * g.B;
     }
     count_launch();
-    auto kern = gemm_scan_bwd_kernel<kS, kTPair>;
+    auto kern = gemm_scan_bwd_kernel<kS, kTPair, kRagged>;
     if (!set_smem(kern, Cfg::kSmemBytes)) return SSM_ERR_CUDA;
     const int pairs = resident_pairs(reinterpret_cast<const void*>(kern), Cfg::kSmemBytes, Cfg::kThreads);
     if (pairs <= 0) return SSM_ERR_CUDA;
@@ -2124,11 +2195,16 @@ static int launch_gemm_scan_bwd_s(const GemmScanBwd& g, cudaStream_t st) {
     return SSM_OK;
 }
 
+template <bool kRagged>
+static int launch_gemm_scan_bwd_r(const GemmScanBwd& g, const FusedMode& m, cudaStream_t st) {
+    if (m.group == 64)
+        return m.time_pairs ? launch_gemm_scan_bwd_s<64, true, kRagged>(g, st) : launch_gemm_scan_bwd_s<64, false, kRagged>(g, st);
+    if (m.group == 32) return launch_gemm_scan_bwd_s<32, false, kRagged>(g, st);
+    return SSM_ERR_SHAPE;
+}
 int launch_gemm_scan_bwd(const GemmScanBwd& g, cudaStream_t st) {
     const FusedMode m = fused_mode(g.B, g.T, g.H, g.P);
-    if (m.group == 64) return m.time_pairs ? launch_gemm_scan_bwd_s<64, true>(g, st) : launch_gemm_scan_bwd_s<64, false>(g, st);
-    if (m.group == 32) return launch_gemm_scan_bwd_s<32, false>(g, st);
-    return SSM_ERR_SHAPE;
+    return fs_ragged(g.T) ? launch_gemm_scan_bwd_r<true>(g, m, st) : launch_gemm_scan_bwd_r<false>(g, m, st);
 }
 
 bool tc_nt_supported(int I, int J) { return (I % tc::BM) == 0 && (J % (tc::BN / 2)) == 0; }

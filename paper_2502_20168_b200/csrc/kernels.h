@@ -181,8 +181,8 @@ bool use_step_small(int B, int H, int P);
 int launch_step_small(const StepCall& g, cudaStream_t st);
 
 // Input projection and forward scan fused (gemm_tc.cu): x = scan(u Bbar^T) written as the two bf16
-// planes of x; Bu never reaches memory.  T must be a multiple of 128 and there must be enough
-// (sequence, 64 states) chains for every pair of CTAs (tc_gemm_scan_fwd_supported).
+// planes of x; Bu never reaches memory.  For lengths that fill most of their 128-row tiles (or 16, 32, 64: a
+// tile then holds whole sequences) and enough (sequence, 64 states) chains (tc_gemm_scan_fwd_supported).
 struct GemmScanFwd {
     const void* u;          // bf16 [B*T, H]
     const void* Wsplit;     // hi/lo stacked Bbar operand [4P, H] (as for GemmTcTN with split_w)
@@ -204,8 +204,7 @@ int launch_gemm_scan_fwd(const GemmScanFwd& g, cudaStream_t st);
 
 // g_x projection and reverse scan fused (gemm_tc.cu): s = reverse scan(gy conj(C)) written as the two
 // bf16 planes of s, the sums s_t conj(x_{t-1}) per (sequence, state) in gA_part; g_x never reaches
-// memory.  T must be a multiple of 128, or 16, 32 or 64 (a 128-row tile then holds whole sequences), with
-// enough chains (tc_gemm_scan_bwd_supported).
+// memory.  Lengths and chains as for the forward kernel (tc_gemm_scan_bwd_supported).
 struct GemmScanBwd {
     const void* gy;         // bf16 [B*T, H]
     const void* Wsplit;     // hi/lo stacked conj(C) operand [4P, H], rows in the pair_cols order

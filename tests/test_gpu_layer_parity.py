@@ -99,6 +99,25 @@ def test_fused_projection_and_scan_shapes_bf16(B, T, H, P):
     run(I.small_variant(w, p_done=0.0))
 
 
+@pytest.mark.parametrize("B,T,H,P", [(146, 127, 256, 128), (147, 129, 256, 128), (74, 250, 128, 128), (37, 383, 256, 128), (20, 500, 256, 256),
+                                     (9, 1000, 256, 256), (74, 1137, 128, 64), (36, 120, 256, 128), (16, 257, 256, 512)])
+def test_fused_projection_and_scan_ragged_lengths_bf16(B, T, H, P):
+    # Sequences that end inside a tile (one row short of it, one row into the next, anywhere): the rows after the end
+    # belong to the next sequence and must neither be written nor contribute.  Chains of 64 and of 32 states, and both CTAs
+    # of a pair on one sequence, whose second tile may lie past the end altogether.
+    w = I.Workload("ragged", B=B, T=T, H=H, P=P, io_dtype="bf16", p_done=0.02, seed=B + T)
+
+    def flags(d):
+        d["done"][0, T - 1] = 1             # the last row of a sequence
+        d["done"][1:, 0] = 1                # the row after a sequence's last one in memory
+        d["done"][2, 0] = 0
+        d["done"][3, 0] = 0
+        d["done"][4, T // 2:] = 1           # every row of the last tile
+    run(w, with_x0=True, with_gxT=True, mutate=flags)
+    run(I.small_variant(w, p_done=0.0), with_x0=True, with_gxT=True)
+    run(I.small_variant(w, p_done=0.0))
+
+
 @pytest.mark.parametrize("io,B,T,H,P", [("f32", 3, 50, 40, 48), ("bf16", 80, 128, 256, 128), ("bf16", 5, 77, 256, 256)])
 def test_conjugate_symmetric_variant_is_the_layer_with_half_the_states_and_doubled_C(io, B, T, H, P):
     """A system whose P states come in conjugate pairs is stored as its first P/2 states and run as
