@@ -454,68 +454,72 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     constexpr int kOutCols = kSplitW ? BN / 2 : BN;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             prefetch_tmap(&tmA);
             prefetch_tmap(&tmWh);
-            const uint32_t leader_full0 = map_to_cta(s.full(0), 0);   // (the leader's barriers are 8 bytes apart there too)
-            int stage = 0;
-            uint32_t phase = 0;
-            bool ok = true;
-            // The 128 rows of A a tile needs are one contiguous range: have L2 fetch the next tile's
-            // range in one piece, so that DRAM sees long bursts instead of 128-byte row pieces.
-            auto prefetch_a = [&](int tile) {
-                if (tile >= total) return;
-                const int m0 = (tile / p.n_tiles) * (2 * BM) + (int)rank * BM;
-                const int rows = min(BM, p.M - m0);
-                if (rows > 0) l2_prefetch_bulk(p.a_base + (size_t)m0 * p.a_row_bytes, (uint32_t)rows * p.a_row_bytes);
-                // (asking L2 for the epilogue's operand rows as well made the bf16-epilogue kernels 15 - 30 % slower)
-            };
-            prefetch_a(pair);
-            for (int tile = pair; tile < total && ok; tile += npairs) {
-                const int m0 = (tile / p.n_tiles) * (2 * BM) + (int)rank * BM;
-                const int n0 = (tile % p.n_tiles) * BN + (int)rank * (BN / 2);
-                prefetch_a(tile + npairs);
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!(ok = mbar_wait(s.empty(stage), phase ^ 1u, s.abort_flag))) break;
+        }
+        const uint32_t leader_full0 = map_to_cta(s.full(0), 0);   // (the leader's barriers are 8 bytes apart there too)
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        // The 128 rows of A a tile needs are one contiguous range: have L2 fetch the next tile's
+        // range in one piece, so that DRAM sees long bursts instead of 128-byte row pieces.
+        auto prefetch_a = [&](int tile) {
+            if (tile >= total) return;
+            const int m0 = (tile / p.n_tiles) * (2 * BM) + (int)rank * BM;
+            const int rows = min(BM, p.M - m0);
+            if (rows > 0 && elect_one()) l2_prefetch_bulk(p.a_base + (size_t)m0 * p.a_row_bytes, (uint32_t)rows * p.a_row_bytes);
+            // (asking L2 for the epilogue's operand rows as well made the bf16-epilogue kernels 15 - 30 % slower)
+        };
+        prefetch_a(pair);
+        for (int tile = pair; tile < total && ok; tile += npairs) {
+            const int m0 = (tile / p.n_tiles) * (2 * BM) + (int)rank * BM;
+            const int n0 = (tile % p.n_tiles) * BN + (int)rank * (BN / 2);
+            prefetch_a(tile + npairs);
+            for (int kb = 0; kb < p.k_blocks; ++kb) {
+                if (!(ok = mbar_wait_warp(s.empty(stage), phase ^ 1u, s.abort_flag))) break;
+                if (elect_one()) {
                     if (rank == 0) mbar_expect_tx(s.full(stage), 2 * kPairStageBytes);
                     const uint32_t a_dst = smem_u32(s.tiles + (size_t)stage * kPairStageBytes);
                     tma_load_2d_pair(a_dst, &tmA, leader_full0 + 8u * stage, p.a_col(kb), m0);
                     tma_load_2d_pair(a_dst + kABytes, &tmWh, leader_full0 + 8u * stage, p.w_col(kb), n0);
-                    if (++stage == kSt) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
+                }
+                if (++stage == kSt) {
+                    stage = 0;
+                    phase ^= 1u;
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             constexpr uint32_t idesc = instr_desc(2 * BM, BN, 0, 0);
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
             bool ok = true;
             for (int tile = pair; tile < total && ok; tile += npairs) {
-                if (!(ok = mbar_wait(s.tmem_empty(acc), acc_phase ^ 1u, s.abort_flag))) break;
+                if (!(ok = mbar_wait_warp(s.tmem_empty(acc), acc_phase ^ 1u, s.abort_flag))) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
                 for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!(ok = mbar_wait(s.full(stage), phase, s.abort_flag))) break;
+                    if (!(ok = mbar_wait_warp(s.full(stage), phase, s.abort_flag))) break;
                     tc_fence_after();
                     const uint32_t a_addr = smem_u32(s.tiles + (size_t)stage * kPairStageBytes);
                     const uint64_t adesc = smem_desc_kmajor(a_addr);
                     const uint64_t bdesc = smem_desc_kmajor(a_addr + kABytes);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < BK / UK; ++k)
-                        umma_bf16_pair(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
-                                       (uint32_t)((kb | k) != 0));
-                    umma_commit_pair(s.empty(stage));
+                        for (int k = 0; k < BK / UK; ++k)
+                            umma_bf16_pair(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
+                                           (uint32_t)((kb | k) != 0));
+                        umma_commit_pair(s.empty(stage));
+                    }
                     if (++stage == kSt) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
                 if (!ok) break;
-                umma_commit_pair(s.tmem_full(acc));
+                if (elect_one()) umma_commit_pair(s.tmem_full(acc));
                 if ((acc ^= 1) == 0) acc_phase ^= 1u;
             }
         }
@@ -719,61 +723,65 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     };
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             prefetch_tmap(&tmA);
             prefetch_tmap(&tmWh);
-            int stage = 0;
-            uint32_t phase = 0;
-            bool ok = true;
-            for (int chain = pair; chain < p.nchains && ok; chain += npairs) {
-                const int n0 = (chain % p.n_tiles) * Cfg::kN + (int)rank * Cfg::kWRows;
-                for (int tb = 0; tb < p.tblocks && ok; ++tb) {
-                    const int m0 = row_of(chain, tb);
-                    // (no L2 prefetch of the next tile's rows here: with it the kernel ran 7 % slower)
-                    for (int kb = 0; kb < p.k_blocks; ++kb) {
-                        if (!(ok = mbar_wait(s.empty(stage), phase ^ 1u, s.abort_flag))) break;
-                        const uint32_t leader_full = map_to_cta(s.full(stage), 0);
+        }
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int chain = pair; chain < p.nchains && ok; chain += npairs) {
+            const int n0 = (chain % p.n_tiles) * Cfg::kN + (int)rank * Cfg::kWRows;
+            for (int tb = 0; tb < p.tblocks && ok; ++tb) {
+                const int m0 = row_of(chain, tb);
+                // (no L2 prefetch of the next tile's rows here: with it the kernel ran 7 % slower)
+                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    if (!(ok = mbar_wait_warp(s.empty(stage), phase ^ 1u, s.abort_flag))) break;
+                    const uint32_t leader_full = map_to_cta(s.full(stage), 0);
+                    if (elect_one()) {
                         if (rank == 0) mbar_expect_tx(s.full(stage), 2 * kStageB);
                         const uint32_t a_dst = smem_u32(s.tiles + (size_t)stage * kStageB);
                         tma_load_2d_pair(a_dst, &tmA, leader_full, kb * BK, m0);
                         tma_load_2d_pair(a_dst + kABytes, &tmWh, leader_full, kb * BK, n0);
-                        if (++stage == kPairStages) {
-                            stage = 0;
-                            phase ^= 1u;
-                        }
+                    }
+                    if (++stage == kPairStages) {
+                        stage = 0;
+                        phase ^= 1u;
                     }
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             constexpr uint32_t idesc = instr_desc(2 * BM, Cfg::kN, 0, 0);
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
             bool ok = true;
             for (int chain = pair; chain < p.nchains && ok; chain += npairs) {
                 for (int tb = 0; tb < p.tblocks && ok; ++tb) {
-                    if (!(ok = mbar_wait(s.tmem_empty(acc), acc_phase ^ 1u, s.abort_flag))) break;
+                    if (!(ok = mbar_wait_warp(s.tmem_empty(acc), acc_phase ^ 1u, s.abort_flag))) break;
                     tc_fence_after();
                     const uint32_t d_tmem = tmem_base + (uint32_t)(acc * Cfg::kN);
                     for (int kb = 0; kb < p.k_blocks; ++kb) {
-                        if (!(ok = mbar_wait(s.full(stage), phase, s.abort_flag))) break;
+                        if (!(ok = mbar_wait_warp(s.full(stage), phase, s.abort_flag))) break;
                         tc_fence_after();
                         const uint32_t a_addr = smem_u32(s.tiles + (size_t)stage * kStageB);
                         const uint64_t adesc = smem_desc_kmajor(a_addr);
                         const uint64_t bdesc = smem_desc_kmajor(a_addr + kABytes);
+                        if (elect_one()) {
 #pragma unroll
-                        for (int k = 0; k < BK / UK; ++k)
-                            umma_bf16_pair(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
-                                           (uint32_t)((kb | k) != 0));
-                        umma_commit_pair(s.empty(stage));
+                            for (int k = 0; k < BK / UK; ++k)
+                                umma_bf16_pair(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
+                                               (uint32_t)((kb | k) != 0));
+                            umma_commit_pair(s.empty(stage));
+                        }
                         if (++stage == kPairStages) {
                             stage = 0;
                             phase ^= 1u;
                         }
                     }
                     if (!ok) break;
-                    umma_commit_pair(s.tmem_full(acc));
+                    if (elect_one()) umma_commit_pair(s.tmem_full(acc));
                     if ((acc ^= 1) == 0) acc_phase ^= 1u;
                 }
             }
@@ -1186,60 +1194,64 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     };
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             prefetch_tmap(&tmA);
             prefetch_tmap(&tmWh);
-            int stage = 0;
-            uint32_t phase = 0;
-            bool ok = true;
-            for (int chain = pair; chain < p.nchains && ok; chain += npairs) {
-                const int n0 = (chain % p.n_tiles) * Cfg::kN + (int)rank * Cfg::kWRows;
-                for (int tb = p.tblocks - 1; tb >= 0 && ok; --tb) {
-                    const int m0 = row_of(chain, tb);
-                    for (int kb = 0; kb < p.k_blocks; ++kb) {
-                        if (!(ok = mbar_wait(s.empty(stage), phase ^ 1u, s.abort_flag))) break;
-                        const uint32_t leader_full = map_to_cta(s.full(stage), 0);
+        }
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int chain = pair; chain < p.nchains && ok; chain += npairs) {
+            const int n0 = (chain % p.n_tiles) * Cfg::kN + (int)rank * Cfg::kWRows;
+            for (int tb = p.tblocks - 1; tb >= 0 && ok; --tb) {
+                const int m0 = row_of(chain, tb);
+                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    if (!(ok = mbar_wait_warp(s.empty(stage), phase ^ 1u, s.abort_flag))) break;
+                    const uint32_t leader_full = map_to_cta(s.full(stage), 0);
+                    if (elect_one()) {
                         if (rank == 0) mbar_expect_tx(s.full(stage), 2 * kStageB);
                         const uint32_t a_dst = smem_u32(s.tiles + (size_t)stage * kStageB);
                         tma_load_2d_pair(a_dst, &tmA, leader_full, kb * BK, m0);
                         tma_load_2d_pair(a_dst + kABytes, &tmWh, leader_full, kb * BK, n0);
-                        if (++stage == kPairStages) {
-                            stage = 0;
-                            phase ^= 1u;
-                        }
+                    }
+                    if (++stage == kPairStages) {
+                        stage = 0;
+                        phase ^= 1u;
                     }
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             constexpr uint32_t idesc = instr_desc(2 * BM, Cfg::kN, 0, 0);
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
             bool ok = true;
             for (int chain = pair; chain < p.nchains && ok; chain += npairs) {
                 for (int tb = 0; tb < p.tblocks && ok; ++tb) {
-                    if (!(ok = mbar_wait(s.tmem_empty(acc), acc_phase ^ 1u, s.abort_flag))) break;
+                    if (!(ok = mbar_wait_warp(s.tmem_empty(acc), acc_phase ^ 1u, s.abort_flag))) break;
                     tc_fence_after();
                     const uint32_t d_tmem = tmem_base + (uint32_t)(acc * Cfg::kN);
                     for (int kb = 0; kb < p.k_blocks; ++kb) {
-                        if (!(ok = mbar_wait(s.full(stage), phase, s.abort_flag))) break;
+                        if (!(ok = mbar_wait_warp(s.full(stage), phase, s.abort_flag))) break;
                         tc_fence_after();
                         const uint32_t a_addr = smem_u32(s.tiles + (size_t)stage * kStageB);
                         const uint64_t adesc = smem_desc_kmajor(a_addr);
                         const uint64_t bdesc = smem_desc_kmajor(a_addr + kABytes);
+                        if (elect_one()) {
 #pragma unroll
-                        for (int k = 0; k < BK / UK; ++k)
-                            umma_bf16_pair(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
-                                           (uint32_t)((kb | k) != 0));
-                        umma_commit_pair(s.empty(stage));
+                            for (int k = 0; k < BK / UK; ++k)
+                                umma_bf16_pair(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
+                                               (uint32_t)((kb | k) != 0));
+                            umma_commit_pair(s.empty(stage));
+                        }
                         if (++stage == kPairStages) {
                             stage = 0;
                             phase ^= 1u;
                         }
                     }
                     if (!ok) break;
-                    umma_commit_pair(s.tmem_full(acc));
+                    if (elect_one()) umma_commit_pair(s.tmem_full(acc));
                     if ((acc ^= 1) == 0) acc_phase ^= 1u;
                 }
             }
@@ -1667,14 +1679,16 @@ gemm_tc_nt_kernel(const __grid_constant__ NtMaps maps, const __grid_constant__ N
     const int nkb = max(0, kb1 - kb0);
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             prefetch_tmap(&tmA);
             prefetch_tmap(&tmBhi);
             prefetch_tmap(&tmBlo);
-            int stage = 0;
-            uint32_t phase = 0;
-            for (int kb = 0; kb < nkb; ++kb) {
-                if (!mbar_wait(s.empty(stage), phase ^ 1u, s.abort_flag)) break;
+        }
+        int stage = 0;
+        uint32_t phase = 0;
+        for (int kb = 0; kb < nkb; ++kb) {
+            if (!mbar_wait_warp(s.empty(stage), phase ^ 1u, s.abort_flag)) break;
+            if (elect_one()) {
                 mbar_expect_tx(s.full(stage), kStageBytes);
                 const uint32_t a_dst = smem_u32(s.tiles + (size_t)stage * kStageBytes);
                 const int row = (kb0 + kb) * BK;
@@ -1685,37 +1699,39 @@ gemm_tc_nt_kernel(const __grid_constant__ NtMaps maps, const __grid_constant__ N
                     tma_load_2d(a_dst + kABytes + h * (BK * 128), &tmBhi, s.full(stage), j0 + 64 * h, row);
                     tma_load_2d(a_dst + kABytes + (BN / 128 + h) * (BK * 128), &tmBlo, s.full(stage), j0 + 64 * h, row);
                 }
-                if (++stage == kStages) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
+            }
+            if (++stage == kStages) {
+                stage = 0;
+                phase ^= 1u;
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && nkb > 0) {
+        if (nkb > 0) {
             constexpr uint32_t idesc = instr_desc(BM, BN, 1, 1);
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!(ok = mbar_wait(s.full(stage), phase, s.abort_flag))) break;
+                if (!(ok = mbar_wait_warp(s.full(stage), phase, s.abort_flag))) break;
                 tc_fence_after();
                 const uint32_t a_addr = smem_u32(s.tiles + (size_t)stage * kStageBytes);
                 const uint64_t adesc = smem_desc_mnmajor(a_addr);
                 const uint64_t bdesc = smem_desc_mnmajor(a_addr + kABytes);
+                if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < BK / UK; ++k) {
-                    // 16 k-rows of 128 bytes further: +2048 bytes = +128 in the address field
-                    umma_bf16(tmem_base, adesc + (uint64_t)(128 * k), bdesc + (uint64_t)(128 * k), idesc,
-                              (uint32_t)((kb | k) != 0));
+                    for (int k = 0; k < BK / UK; ++k) {
+                        // 16 k-rows of 128 bytes further: +2048 bytes = +128 in the address field
+                        umma_bf16(tmem_base, adesc + (uint64_t)(128 * k), bdesc + (uint64_t)(128 * k), idesc,
+                                  (uint32_t)((kb | k) != 0));
+                    }
+                    umma_commit(s.empty(stage));
                 }
-                umma_commit(s.empty(stage));
                 if (++stage == kStages) {
                     stage = 0;
                     phase ^= 1u;
                 }
             }
-            if (ok) umma_commit(s.tmem_full(0));
+            if (ok && elect_one()) umma_commit(s.tmem_full(0));
         }
     } else {
         const int q = warp & 3;
@@ -1807,15 +1823,17 @@ gemm_tc_nt_pair_kernel(const __grid_constant__ NtMaps maps, const __grid_constan
     const int nkb = max(0, min(total_blocks, kb0 + p.blocks_per_split) - kb0);
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             prefetch_tmap(&tmA);
             prefetch_tmap(rank == 0 ? &tmBhi : &tmBlo);
-            const CUtensorMap* tmB = rank == 0 ? &tmBhi : &tmBlo;
-            int stage = 0;
-            uint32_t phase = 0;
-            for (int kb = 0; kb < nkb; ++kb) {
-                if (!mbar_wait(rempty(stage), phase ^ 1u, s.abort_flag)) break;
-                const uint32_t leader_full = map_to_cta(rfull(stage), 0);
+        }
+        const CUtensorMap* tmB = rank == 0 ? &tmBhi : &tmBlo;
+        int stage = 0;
+        uint32_t phase = 0;
+        for (int kb = 0; kb < nkb; ++kb) {
+            if (!mbar_wait_warp(rempty(stage), phase ^ 1u, s.abort_flag)) break;
+            const uint32_t leader_full = map_to_cta(rfull(stage), 0);
+            if (elect_one()) {
                 if (rank == 0) mbar_expect_tx(rfull(stage), 2 * kNtPairStageBytes);
                 const uint32_t a_dst = smem_u32(s.tiles + (size_t)stage * kNtPairStageBytes);
                 const int row = (kb0 + kb) * BK;
@@ -1824,35 +1842,37 @@ gemm_tc_nt_pair_kernel(const __grid_constant__ NtMaps maps, const __grid_constan
 #pragma unroll
                 for (int h = 0; h < kOutCols / 64; ++h)
                     tma_load_2d_pair(a_dst + kABytes + h * (BK * 128), tmB, leader_full, j0 + 64 * h, row);
-                if (++stage == kNtPairStages) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
+            }
+            if (++stage == kNtPairStages) {
+                stage = 0;
+                phase ^= 1u;
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0 && nkb > 0) {
+        if (rank == 0 && nkb > 0) {
             constexpr uint32_t idesc = instr_desc(2 * BM, BN, 1, 1);
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!(ok = mbar_wait(rfull(stage), phase, s.abort_flag))) break;
+                if (!(ok = mbar_wait_warp(rfull(stage), phase, s.abort_flag))) break;
                 tc_fence_after();
                 const uint32_t a_addr = smem_u32(s.tiles + (size_t)stage * kNtPairStageBytes);
                 const uint64_t adesc = smem_desc_mnmajor(a_addr);
                 const uint64_t bdesc = smem_desc_mnmajor(a_addr + kABytes);
+                if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < BK / UK; ++k)
-                    umma_bf16_pair(tmem_base, adesc + (uint64_t)(128 * k), bdesc + (uint64_t)(128 * k), idesc,
-                                   (uint32_t)((kb | k) != 0));
-                umma_commit_pair(rempty(stage));
+                    for (int k = 0; k < BK / UK; ++k)
+                        umma_bf16_pair(tmem_base, adesc + (uint64_t)(128 * k), bdesc + (uint64_t)(128 * k), idesc,
+                                       (uint32_t)((kb | k) != 0));
+                    umma_commit_pair(rempty(stage));
+                }
                 if (++stage == kNtPairStages) {
                     stage = 0;
                     phase ^= 1u;
                 }
             }
-            if (ok) umma_commit_pair(s.tmem_full(0));
+            if (ok && elect_one()) umma_commit_pair(s.tmem_full(0));
         }
     } else {
         const int q = warp & 3;

@@ -83,14 +83,14 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __
     grid_dep_launch();
 
     if (warp == 0) {
-        if (lane == 0) {
-            const uint32_t bytes = (uint32_t)(planes_a + planes_b) * kNpTile;
-            int stage = 0;
-            uint32_t phase = 0;
-            for (int kb = kb0; kb < kb1; ++kb) {
-                if (!mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
-                const uint32_t full = smem_u32(&bars.full[stage]);
-                uint32_t dst = smem_u32(tiles) + (uint32_t)stage * (uint32_t)p.stage_bytes;
+        const uint32_t bytes = (uint32_t)(planes_a + planes_b) * kNpTile;
+        int stage = 0;
+        uint32_t phase = 0;
+        for (int kb = kb0; kb < kb1; ++kb) {
+            if (!mbar_wait_warp(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
+            const uint32_t full = smem_u32(&bars.full[stage]);
+            uint32_t dst = smem_u32(tiles) + (uint32_t)stage * (uint32_t)p.stage_bytes;
+            if (elect_one()) {
                 mbar_expect_tx(full, bytes);
                 for (int q = 0; q < planes_a; ++q, dst += kNpTile) {
                     tma_load_2d(dst, ta, full, q * p.I + i0, kb * BK);
@@ -100,14 +100,14 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __
                     tma_load_2d(dst, tb, full, q * p.J + j0, kb * BK);
                     tma_load_2d(dst + kNpTile / 2, tb, full, q * p.J + j0 + 64, kb * BK);
                 }
-                if (++stage == p.stages) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
+            }
+            if (++stage == p.stages) {
+                stage = 0;
+                phase ^= 1u;
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && kb0 < kb1) {
+        if (kb0 < kb1) {
             constexpr uint32_t idesc = instr_desc(128, 128, 1, 1);
             const int n_prod = pr.n_prod;
             const uint32_t pa = pr.pa, pb = pr.pb;
@@ -118,24 +118,26 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __
                 const int seg = (kb - kb0) / kNpSegment, buf = seg & 1;
                 const bool seg_first = (kb - kb0) % kNpSegment == 0;
                 if (seg_first && seg >= 2) {   // the epilogue has taken segment seg - 2 out of this half of tensor memory
-                    if (!(ok = mbar_wait(smem_u32(&bars.free[buf]), (uint32_t)((seg >> 1) - 1) & 1u, abort_flag))) break;
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars.free[buf]), (uint32_t)((seg >> 1) - 1) & 1u, abort_flag))) break;
                     tc_fence_after();
                 }
-                if (!(ok = mbar_wait(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
+                if (!(ok = mbar_wait_warp(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
                 tc_fence_after();
                 const uint32_t base = smem_u32(tiles) + (uint32_t)stage * (uint32_t)p.stage_bytes;
-                for (int j = 0; j < n_prod; ++j) {
-                    const bool small = j < n_prod - 1;
-                    const uint32_t d_tmem = tmem_base + 256u * (uint32_t)buf + (small ? 128u : 0u);
-                    const bool first = seg_first && (j == 0 || !small);
-                    const uint64_t ad = smem_desc_mnmajor(base + ((pa >> (4 * j)) & 15u) * kNpTile);
-                    const uint64_t bd = smem_desc_mnmajor(base + ((uint32_t)planes_a + ((pb >> (4 * j)) & 15u)) * kNpTile);
+                if (elect_one()) {
+                    for (int j = 0; j < n_prod; ++j) {
+                        const bool small = j < n_prod - 1;
+                        const uint32_t d_tmem = tmem_base + 256u * (uint32_t)buf + (small ? 128u : 0u);
+                        const bool first = seg_first && (j == 0 || !small);
+                        const uint64_t ad = smem_desc_mnmajor(base + ((pa >> (4 * j)) & 15u) * kNpTile);
+                        const uint64_t bd = smem_desc_mnmajor(base + ((uint32_t)planes_a + ((pb >> (4 * j)) & 15u)) * kNpTile);
 #pragma unroll
-                    for (int k = 0; k < BK / UK; ++k)   // 16 rows of 128 bytes further: +128 in the address field
-                        umma_bf16(d_tmem, ad + (uint64_t)(128 * k), bd + (uint64_t)(128 * k), idesc, (uint32_t)!(first && k == 0));
+                        for (int k = 0; k < BK / UK; ++k)   // 16 rows of 128 bytes further: +128 in the address field
+                            umma_bf16(d_tmem, ad + (uint64_t)(128 * k), bd + (uint64_t)(128 * k), idesc, (uint32_t)!(first && k == 0));
+                    }
+                    umma_commit(smem_u32(&bars.empty[stage]));
+                    if (kb + 1 == kb1 || (kb + 1 - kb0) % kNpSegment == 0) umma_commit(smem_u32(&bars.done[buf]));
                 }
-                umma_commit(smem_u32(&bars.empty[stage]));
-                if (kb + 1 == kb1 || (kb + 1 - kb0) % kNpSegment == 0) umma_commit(smem_u32(&bars.done[buf]));
                 if (++stage == p.stages) {
                     stage = 0;
                     phase ^= 1u;

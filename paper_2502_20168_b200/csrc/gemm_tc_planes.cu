@@ -81,46 +81,46 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     grid_dep_launch();
 
     if (warp == 0) {
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x) {
-                const int m0 = (tile / p.n_tiles) * BM, n0 = (tile % p.n_tiles) * kPlBN;
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!(ok = mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag))) break;
-                    const uint32_t full = smem_u32(&bars.full[stage]);
-                    const uint32_t dst = smem_u32(stages) + (uint32_t)stage * kPlStageBytes;
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x) {
+            const int m0 = (tile / p.n_tiles) * BM, n0 = (tile % p.n_tiles) * kPlBN;
+            for (int kb = 0; kb < p.k_blocks; ++kb) {
+                if (!(ok = mbar_wait_warp(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag))) break;
+                const uint32_t full = smem_u32(&bars.full[stage]);
+                const uint32_t dst = smem_u32(stages) + (uint32_t)stage * kPlStageBytes;
+                if (elect_one()) {
                     mbar_expect_tx(full, (uint32_t)(p.planes_a * kPlATile + 3 * kPlWTile));
                     for (int q = 0; q < p.planes_a; ++q) tma_load_2d(dst + q * kPlATile, &tmA, full, q * p.K + kb * kPlBK, m0);
 #pragma unroll
                     for (int q = 0; q < 3; ++q)
                         tma_load_2d(dst + 3 * kPlATile + q * kPlWTile, &tmW, full, q * p.K + kb * kPlBK, n0);
-                    if (++stage == kPlStages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
+                }
+                if (++stage == kPlStages) {
+                    stage = 0;
+                    phase ^= 1u;
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = instr_desc(BM, kPlBN, 0, 0);
-            const int n_prod = p.n_prod;
-            const uint32_t pa = p.pa, pw = p.pw;
-            int stage = 0, n = 0;
-            uint32_t phase = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x, ++n) {
-                const int buf = n & 1;
-                if (n >= 2) {   // the epilogue has taken tile n - 2 out of this half of tensor memory
-                    if (!(ok = mbar_wait(smem_u32(&bars.free[buf]), (uint32_t)((n >> 1) - 1) & 1u, abort_flag))) break;
-                    tc_fence_after();
-                }
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!(ok = mbar_wait(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
-                    tc_fence_after();
-                    const uint32_t base = smem_u32(stages) + (uint32_t)stage * kPlStageBytes;
+        constexpr uint32_t idesc = instr_desc(BM, kPlBN, 0, 0);
+        const int n_prod = p.n_prod;
+        const uint32_t pa = p.pa, pw = p.pw;
+        int stage = 0, n = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x, ++n) {
+            const int buf = n & 1;
+            if (n >= 2) {   // the epilogue has taken tile n - 2 out of this half of tensor memory
+                if (!(ok = mbar_wait_warp(smem_u32(&bars.free[buf]), (uint32_t)((n >> 1) - 1) & 1u, abort_flag))) break;
+                tc_fence_after();
+            }
+            for (int kb = 0; kb < p.k_blocks; ++kb) {
+                if (!(ok = mbar_wait_warp(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
+                tc_fence_after();
+                const uint32_t base = smem_u32(stages) + (uint32_t)stage * kPlStageBytes;
+                if (elect_one()) {
                     for (int j = 0; j < n_prod; ++j) {
                         const bool small = j < n_prod - 1;
                         const uint32_t d_tmem = tmem_base + 256u * (uint32_t)buf + (small ? 128u : 0u);
@@ -132,13 +132,13 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                                       (uint32_t)!(kb == 0 && k == 0 && (j == 0 || !small)));
                     }
                     umma_commit(smem_u32(&bars.empty[stage]));
-                    if (++stage == kPlStages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
                 }
-                if (ok) umma_commit(smem_u32(&bars.done[buf]));
+                if (++stage == kPlStages) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
             }
+            if (ok && elect_one()) umma_commit(smem_u32(&bars.done[buf]));
         }
     } else {
         // A warp drains 32 rows x 64 columns of a tile in slabs of 32 x 32.  A slab is turned round in the warp's 4 KB of

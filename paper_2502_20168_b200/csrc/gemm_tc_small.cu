@@ -61,19 +61,21 @@ struct SmallBars {
     int abort_flag;
 };
 
-template <int kBN, int kEpi, bool kSplitA, bool kBf16>
+template <int kBN, int kEpi, bool kSplitA, bool kBf16, bool kPair>
 __global__ void __launch_bounds__(sm_threads(kBN), 1)
 gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, SmallTnArgs p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ SmallBars bars;
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr int kSmEpiWarps = sm_epi_warps(kBN);
-    constexpr int kWTile = kBN * BK * 2;
+    constexpr int kWRows = kPair ? kBN / 2 : kBN;   // weight rows this CTA loads
+    constexpr int kWTile = kWRows * BK * 2;
     constexpr int kPitch = kBN + 4;   // staging: floats per row; 16 bytes of padding keep both directions free of bank conflicts
     volatile int* abort_flag = &bars.abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rank = (int)cluster_ctarank(), tile = (int)blockIdx.x / p.cluster;
-    const int m0 = (tile / p.n_tiles) * BM, n0 = (tile % p.n_tiles) * kBN;
+    const int crank = (int)cluster_ctarank(), rank = kPair ? 0 : crank, tile = (int)blockIdx.x / (kPair ? 2 : p.cluster);
+    const int m_tile = kPair ? 2 * (tile / p.n_tiles) + crank : tile / p.n_tiles;
+    const int m0 = m_tile * BM, n0 = (tile % p.n_tiles) * kBN;
     if (threadIdx.x == 0) {
         for (int i = 0; i < p.stages; ++i) {
             mbar_init(smem_u32(&bars.full[i]), kSplitA ? 1 + kSmEpiWarps : 1);
@@ -89,9 +91,13 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     // are added once.  (In one accumulator every small term would be rounded at the magnitude of the sum: measured 2 - 3 x
     // the error on the gradients of small fp32 layers.)
     const uint32_t tmem_cols = p.n_prod > 1 ? 2 * kBN : kBN;
-    if (warp == 1) tmem_alloc(smem_u32(&bars.tmem), tmem_cols);
+    if (warp == 1) {
+        if (kPair) tmem_alloc_pair(smem_u32(&bars.tmem), tmem_cols);
+        else tmem_alloc(smem_u32(&bars.tmem), tmem_cols);
+    }
     tc_fence_before();
-    __syncthreads();
+    if (kPair) cluster_sync_all();   // the other CTA's barriers are set up
+    else __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = bars.tmem;
     grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
@@ -100,56 +106,70 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     const uint32_t a_bytes = (uint32_t)p.planes_a * kSmATile;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             if (!kSplitA) prefetch_tmap(&tmA);
             prefetch_tmap(&tmW);
-            const uint32_t bytes = (uint32_t)p.planes_w * kWTile + (kSplitA ? 0u : a_bytes);
-            const int wrow = p.w_stacked ? (n0 / 128) * 256 + n0 % 128 : n0;
-            int stage = 0;
-            uint32_t phase = 0;
-            for (int kb = kb0; kb < kb1; ++kb) {
-                if (!mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
-                const uint32_t full = smem_u32(&bars.full[stage]);
+        }
+        const uint32_t bytes = (uint32_t)p.planes_w * kWTile + (kSplitA ? 0u : a_bytes);
+        const int wn = n0 + (kPair ? crank * kWRows : 0), wrow = p.w_stacked ? (wn / 128) * 256 + wn % 128 : wn;
+        int stage = 0;
+        uint32_t phase = 0;
+        for (int kb = kb0; kb < kb1; ++kb) {
+            if (!mbar_wait_warp(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
+            // (a pair counts both CTAs' loads on the barrier of CTA 0, which issues the MMAs)
+            const uint32_t full = kPair ? map_to_cta(smem_u32(&bars.full[stage]), 0) : smem_u32(&bars.full[stage]);
+            if (elect_one()) {
                 const uint32_t dst = smem_u32(tiles) + (uint32_t)stage * (uint32_t)p.stage_bytes;
-                mbar_expect_tx(full, bytes);
+                if (!kPair || crank == 0) mbar_expect_tx(smem_u32(&bars.full[stage]), kPair ? 2 * bytes : bytes);
+                auto load = [&](uint32_t to, const CUtensorMap* map, int c0, int c1) {
+                    if (kPair) tma_load_2d_pair(to, map, full, c0, c1);
+                    else tma_load_2d(to, map, full, c0, c1);
+                };
                 if (!kSplitA)
-                    for (int a = 0; a < p.planes_a; ++a) tma_load_2d(dst + a * kSmATile, &tmA, full, a * p.a_plane + kb * BK, m0);
+                    for (int a = 0; a < p.planes_a; ++a) load(dst + a * kSmATile, &tmA, a * p.a_plane + kb * BK, m0);
                 for (int w = 0; w < p.planes_w; ++w)
-                    tma_load_2d(dst + a_bytes + w * kWTile, &tmW, full, w * p.w_plane_cols + kb * BK, wrow + w * p.w_plane_rows);
-                if (++stage == p.stages) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
+                    load(dst + a_bytes + w * kWTile, &tmW, w * p.w_plane_cols + kb * BK, wrow + w * p.w_plane_rows);
+            }
+            if (++stage == p.stages) {
+                stage = 0;
+                phase ^= 1u;
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = instr_desc(BM, kBN, 0, 0);
+        if (!kPair || crank == 0) {
+            constexpr uint32_t idesc = instr_desc(kPair ? 2 * BM : BM, kBN, 0, 0);
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
             for (int kb = kb0; kb < kb1; ++kb) {
-                if (!(ok = mbar_wait(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
+                if (!(ok = mbar_wait_warp(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
                 tc_fence_after();
                 const uint32_t base = smem_u32(tiles) + (uint32_t)stage * (uint32_t)p.stage_bytes;
-                for (int j = 0; j < p.n_prod; ++j) {
-                    const bool small = j < p.n_prod - 1;
-                    const uint32_t d_tmem = tmem_base + (small ? (uint32_t)kBN : 0u);
-                    const bool first = kb == kb0 && (j == 0 || !small);
-                    const uint64_t ad = smem_desc_kmajor(base + ((p.prod_a >> (4 * j)) & 15u) * kSmATile);
-                    const uint64_t wd = smem_desc_kmajor(base + a_bytes + ((p.prod_w >> (4 * j)) & 15u) * kWTile);
+                if (elect_one()) {
+                    for (int j = 0; j < p.n_prod; ++j) {
+                        const bool small = j < p.n_prod - 1;
+                        const uint32_t d_tmem = tmem_base + (small ? (uint32_t)kBN : 0u);
+                        const bool first = kb == kb0 && (j == 0 || !small);
+                        const uint64_t ad = smem_desc_kmajor(base + ((p.prod_a >> (4 * j)) & 15u) * kSmATile);
+                        const uint64_t wd = smem_desc_kmajor(base + a_bytes + ((p.prod_w >> (4 * j)) & 15u) * kWTile);
 #pragma unroll
-                    for (int k = 0; k < BK / UK; ++k) {
-                        umma_bf16(d_tmem, ad + (uint64_t)(2 * k), wd + (uint64_t)(2 * k), idesc, (uint32_t)!(first && k == 0));
+                        for (int k = 0; k < BK / UK; ++k) {
+                            if (kPair) umma_bf16_pair(d_tmem, ad + (uint64_t)(2 * k), wd + (uint64_t)(2 * k), idesc, (uint32_t)!(first && k == 0));
+                            else umma_bf16(d_tmem, ad + (uint64_t)(2 * k), wd + (uint64_t)(2 * k), idesc, (uint32_t)!(first && k == 0));
+                        }
                     }
+                    if (kPair) umma_commit_pair(smem_u32(&bars.empty[stage]));
+                    else umma_commit(smem_u32(&bars.empty[stage]));
                 }
-                umma_commit(smem_u32(&bars.empty[stage]));
                 if (++stage == p.stages) {
                     stage = 0;
                     phase ^= 1u;
                 }
             }
-            if (ok) umma_commit(smem_u32(&bars.done));
+            if (ok && elect_one()) {
+                if (kPair) umma_commit_pair(smem_u32(&bars.done));
+                else umma_commit(smem_u32(&bars.done));
+            }
         }
     } else {
         if (kSplitA) {
@@ -177,7 +197,8 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     // takes every kRowGroups-th row, kU rows at a time.
     constexpr int kC4 = kBN / 4, kRowGroups = 32 * kSmEpiWarps / kC4, kU = kBN == 256 && !kBf16 ? 4 : 8;
     const int te = (int)threadIdx.x - 64, c4 = te % kC4, rg = te / kC4;
-    const int rows = BM / p.cluster, row_base = rank * rows;
+    const int parts = kPair ? 1 : p.cluster;   // CTAs whose parts of a row are added
+    const int rows = BM / parts, row_base = rank * rows;
     const int n = n0 + 4 * c4;
     Raw4<kBf16> sk[kU], dt[kU];
     // the epilogue's operands come from far: the first rows are asked for while the MMAs run
@@ -223,7 +244,7 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         }
     }
     __syncwarp();
-    if (p.cluster > 1) cluster_sync_all();   // the parts of all CTAs of the cluster are in place
+    if (parts > 1) cluster_sync_all();   // the parts of all CTAs of the cluster are in place
     else __syncthreads();
     if (warp >= 2 && !*abort_flag) {
         const bool n_ok = n < p.N;
@@ -244,13 +265,13 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     if (kEpi == kSmDiag && p.add && r < rows && m < p.M && n_ok)
                         v[i] = *reinterpret_cast<const float4*>(p.add + (size_t)m * p.N + n);
                 }
-                for (int q = 0; q < p.cluster; ++q) {
+                for (int q = 0; q < parts; ++q) {
                     const uint32_t a = map_to_cta(smem_u32(own), (uint32_t)q);
                     float4 t[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
                         if (r1 + i * kRowGroups < rows)
-                            t[i] = p.cluster == 1 ? *reinterpret_cast<const float4*>(own + (size_t)i * kRowGroups * kPitch)
+                            t[i] = parts == 1 ? *reinterpret_cast<const float4*>(own + (size_t)i * kRowGroups * kPitch)
                                                   : ld_cluster_f4(a + (uint32_t)i * (kRowGroups * kPitch * 4u));
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
@@ -298,17 +319,20 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     const float4 u = red[g * kC4 + c4];
                     t.x += u.x, t.y += u.y, t.z += u.z, t.w += u.w;
                 }
-                *reinterpret_cast<float4*>(p.dot_part + (size_t)((tile / p.n_tiles) * p.cluster + rank) * p.N + n) = t;
+                *reinterpret_cast<float4*>(p.dot_part + (size_t)(m_tile * parts + rank) * p.N + n) = t;
             }
         }
     }
     // nobody leaves (or frees tensor memory) while another CTA may still read its part
     tc_fence_before();
     __syncwarp();
-    if (p.cluster > 1) cluster_sync_all();
+    if (kPair || p.cluster > 1) cluster_sync_all();
     else __syncthreads();
     tc_fence_after();
-    if (warp == 1) tmem_dealloc(tmem_base, tmem_cols);
+    if (warp == 1) {
+        if (kPair) tmem_dealloc_pair(tmem_base, tmem_cols);
+        else tmem_dealloc(tmem_base, tmem_cols);
+    }
     if (threadIdx.x == 0 && *abort_flag && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
 }
 
@@ -319,9 +343,12 @@ namespace {
 
 struct SmallShape {
     int bn, cluster, stages;
+    bool pair;
 };
 
-size_t stage_bytes_of(int bn, int planes_a, int planes_w) { return (size_t)planes_a * kSmATile + (size_t)planes_w * bn * BK * 2; }
+size_t stage_bytes_of(int bn, int planes_a, int planes_w, bool pair) {
+    return (size_t)planes_a * kSmATile + (size_t)planes_w * (pair ? bn / 2 : bn) * BK * 2;
+}
 
 // Tile width and cluster size: the pair with the shortest estimated time.  The estimate is a fit, in microseconds, to
 // timings of all pairs on twenty shapes from 16 x 256 x 256 to 4096 x 1024 x 1024, back to back (within 10 % of the
@@ -329,35 +356,37 @@ size_t stage_bytes_of(int bn, int planes_a, int planes_w) { return (size_t)plane
 // the tile (start, first loads, epilogue), its k-blocks at 48 bytes of operands per cycle and SM (L2), 0.95 us where
 // fp32 operands are split on the way, and the exchange between the CTAs of a cluster.
 SmallShape pick_small(int M, int N, int k_blocks, int planes_a, int planes_w, bool split_a, bool w_stacked) {
-    SmallShape best{0, 0, 0};
+    SmallShape best{0, 0, 0, false};
     double best_t = 0.0;
     const int m_tiles = (M + BM - 1) / BM, sms = device_sm_count();
-    for (int bn = 64; bn <= (w_stacked ? 128 : 256); bn *= 2) {
-        const size_t sb = stage_bytes_of(bn, planes_a, planes_w);
+    auto consider = [&](int bn, int c, bool pair) {
+        const size_t sb = stage_bytes_of(bn, planes_a, planes_w, pair);
         const int stages = std::min<int>(kSmMaxStages, (int)((kSmSmemMax - 1024) / sb));
-        if (stages < 2) continue;
-        const int tiles = m_tiles * ((N + bn - 1) / bn);
-        for (int c = 1; c <= 4 && c <= k_blocks; c *= 2) {
-            const int slots = c == 1 ? sms : (c == 2 ? sms - 4 : sms - 16);   // clusters must fit a GPC
-            const int waves = (tiles * c + slots - 1) / slots;
-            const double per_kb = std::max((double)sb / 91000.0, split_a ? 0.95 : 0.0);
-            const double exchange = c == 1 ? 0.0 : bn * c / 256.0;
-            const double t = waves * (4.6 + bn * 0.0115 + exchange + ((k_blocks + c - 1) / c) * per_kb);
-            if (best.bn == 0 || t < best_t) {
-                best_t = t;
-                best = {bn, c, stages};
-            }
+        if (stages < 2) return;
+        const int ctas = (pair ? (m_tiles + 1) / 2 * 2 : m_tiles * c) * ((N + bn - 1) / bn);
+        const int slots = pair || c == 2 ? sms - 4 : (c == 1 ? sms : sms - 16);   // clusters must fit a GPC
+        const int waves = (ctas + slots - 1) / slots;
+        const double per_kb = std::max((double)sb / 91000.0, split_a ? 0.95 : 0.0);
+        const double exchange = c == 1 ? 0.0 : bn * c / 256.0;
+        const double t = waves * (4.6 + bn * 0.0115 + exchange + ((k_blocks + c - 1) / c) * per_kb);
+        if (best.bn == 0 || t < best_t) {
+            best_t = t;
+            best = {bn, c, stages, pair};
         }
-    }
+    };
+    for (int bn = 64; bn <= (w_stacked ? 128 : 256); bn *= 2)
+        for (int c = 1; c <= 4 && c <= k_blocks; c *= 2) consider(bn, c, false);
+    if (!split_a)
+        for (int bn = 128; bn <= 256; bn *= 2) consider(bn, 1, true);
     return best;
 }
 
-template <int kBN, int kEpi, bool kSplitA, bool kBf16>
+template <int kBN, int kEpi, bool kSplitA, bool kBf16, bool kPair>
 int launch_small(const CUtensorMap& ma, const CUtensorMap& mw, const SmallTnArgs& p, int grid, size_t smem, cudaStream_t st) {
-    auto kern = gemm_tc_tn_small_kernel<kBN, kEpi, kSplitA, kBf16>;
+    auto kern = gemm_tc_tn_small_kernel<kBN, kEpi, kSplitA, kBf16, kPair>;
     if (!set_max_dynamic_smem(reinterpret_cast<const void*>(kern), kSmSmemMax)) return SSM_ERR_CUDA;
     count_launch();
-    return launch_dep_cluster(kern, (unsigned)p.cluster, grid, sm_threads(kBN), smem, st, ma, mw, p) ? SSM_OK : SSM_ERR_CUDA;
+    return launch_dep_cluster(kern, kPair ? 2u : (unsigned)p.cluster, grid, sm_threads(kBN), smem, st, ma, mw, p) ? SSM_OK : SSM_ERR_CUDA;
 }
 
 }  // namespace
@@ -397,23 +426,25 @@ int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st) {
     if (s.bn == 0) return SSM_ERR_SHAPE;
     p.cluster = s.cluster;
     p.stages = s.stages;
-    p.stage_bytes = (int)stage_bytes_of(s.bn, p.planes_a, p.planes_w);
+    p.stage_bytes = (int)stage_bytes_of(s.bn, p.planes_a, p.planes_w, s.pair);
     p.n_tiles = (g.N_out + s.bn - 1) / s.bn;
     const size_t smem = std::max((size_t)p.stages * p.stage_bytes, (size_t)BM * (s.bn + 4) * 4) + 1024;
-    const int m_tiles = (g.M + BM - 1) / BM, grid = m_tiles * p.n_tiles * p.cluster;
-    if (g.dot_rows) *g.dot_rows = m_tiles * p.cluster;
+    const int m_tiles = (g.M + BM - 1) / BM, grid = (s.pair ? (m_tiles + 1) / 2 * 2 : m_tiles * p.cluster) * p.n_tiles;
+    if (g.dot_rows) *g.dot_rows = s.pair ? (m_tiles + 1) / 2 * 2 : m_tiles * p.cluster;
     CUtensorMap ma, mw;
     const uint64_t w_rows = (uint64_t)g.N_out * (p.w_stacked ? p.planes_w : 1);
     const uint64_t w_cols = (uint64_t)g.K * (p.w_stacked ? 1 : p.planes_w);
-    if (!make_map(&mw, g.W, w_rows, w_cols, BK, (uint32_t)s.bn)) return SSM_ERR_CUDA;
+    if (!make_map(&mw, g.W, w_rows, w_cols, BK, (uint32_t)(s.pair ? s.bn / 2 : s.bn))) return SSM_ERR_CUDA;
     ma = mw;   // unused when A is split here
     if (!g.a_f32 && !make_map(&ma, g.A, (uint64_t)g.M, (uint64_t)g.K * p.planes_a, BK, BM)) return SSM_ERR_CUDA;
     const bool io_bf16 = g.skip_bf16 && (!g.dot || g.dot_bf16);
 #define SSM_SMALL(EPI, SPLIT, BF)                                                             \
     do {                                                                                      \
-        if (s.bn == 64) return launch_small<64, EPI, SPLIT, BF>(ma, mw, p, grid, smem, st);   \
-        if (s.bn == 128) return launch_small<128, EPI, SPLIT, BF>(ma, mw, p, grid, smem, st); \
-        return launch_small<256, EPI, SPLIT, BF>(ma, mw, p, grid, smem, st);                  \
+        if (s.pair && s.bn == 128) return launch_small<128, EPI, false, BF, true>(ma, mw, p, grid, smem, st); \
+        if (s.pair) return launch_small<256, EPI, false, BF, true>(ma, mw, p, grid, smem, st);                \
+        if (s.bn == 64) return launch_small<64, EPI, SPLIT, BF, false>(ma, mw, p, grid, smem, st);            \
+        if (s.bn == 128) return launch_small<128, EPI, SPLIT, BF, false>(ma, mw, p, grid, smem, st);          \
+        return launch_small<256, EPI, SPLIT, BF, false>(ma, mw, p, grid, smem, st);                           \
     } while (0)
     if (epi == kSmGate) SSM_SMALL(kSmGate, false, true);
     if (epi == kSmStore && g.a_f32) SSM_SMALL(kSmStore, true, true);

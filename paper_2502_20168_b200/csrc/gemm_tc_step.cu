@@ -144,45 +144,47 @@ step_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUt
         constexpr uint32_t bytes0 = P0::planes_w * kWTile + (kF32 ? 0u : a_bytes);
         constexpr uint32_t bytes1 = P1::planes_w * kWTile + (kF32 ? 0u : a_bytes);
         bool ok = true;
-        if (lane == 0) {
-            for (int t = rank; t < p.n_tiles[0] && ok; t += p.cluster)
-                for (int kb = 0; kb < p.k_blocks[0]; ++kb, r.next(p.stages)) {
-                    if (!(ok = mbar_wait(smem_u32(&bars.empty[r.stage]), r.phase ^ 1u, abort_flag))) break;
+        for (int t = rank; t < p.n_tiles[0] && ok; t += p.cluster)
+            for (int kb = 0; kb < p.k_blocks[0]; ++kb, r.next(p.stages)) {
+                if (!(ok = mbar_wait_warp(smem_u32(&bars.empty[r.stage]), r.phase ^ 1u, abort_flag))) break;
+                if (elect_one()) {
                     const uint32_t full = smem_u32(&bars.full[r.stage]);
                     mbar_expect_tx(full, bytes0);
                     load_a(0, kb, r.stage, full);
                     load_w(0, t, kb, r.stage, full);
                 }
-        }
+            }
         __syncwarp();
         cluster_arrive();
         // the weights of the first k-blocks of the second phase do not wait for the states
         Ring r1 = r;
         int pre = 0;
         const bool any = rank < p.n_tiles[1];
-        if (lane == 0 && ok && any)
+        if (ok && any)
             for (; pre < p.stages && pre < p.k_blocks[1]; ++pre, r.next(p.stages)) {
-                if (!(ok = mbar_wait(smem_u32(&bars.empty[r.stage]), r.phase ^ 1u, abort_flag))) break;
-                const uint32_t full = smem_u32(&bars.full[r.stage]);
-                mbar_expect_tx(full, bytes1);
-                load_w(1, rank, pre, r.stage, full);
+                if (!(ok = mbar_wait_warp(smem_u32(&bars.empty[r.stage]), r.phase ^ 1u, abort_flag))) break;
+                if (elect_one()) {
+                    const uint32_t full = smem_u32(&bars.full[r.stage]);
+                    mbar_expect_tx(full, bytes1);
+                    load_w(1, rank, pre, r.stage, full);
+                }
             }
         __syncwarp();
         cluster_wait();
-        if (lane == 0) {
-            if (!kF32) {
-                fence_async_global();
-                for (int kb = 0; kb < pre; ++kb, r1.next(p.stages)) load_a(1, kb, r1.stage, smem_u32(&bars.full[r1.stage]));
-            }
-            for (int t = rank; t < p.n_tiles[1] && ok; t += p.cluster)
-                for (int kb = t == rank ? pre : 0; kb < p.k_blocks[1]; ++kb, r.next(p.stages)) {
-                    if (!(ok = mbar_wait(smem_u32(&bars.empty[r.stage]), r.phase ^ 1u, abort_flag))) break;
+        if (!kF32 && elect_one()) {
+            fence_async_global();
+            for (int kb = 0; kb < pre; ++kb, r1.next(p.stages)) load_a(1, kb, r1.stage, smem_u32(&bars.full[r1.stage]));
+        }
+        for (int t = rank; t < p.n_tiles[1] && ok; t += p.cluster)
+            for (int kb = t == rank ? pre : 0; kb < p.k_blocks[1]; ++kb, r.next(p.stages)) {
+                if (!(ok = mbar_wait_warp(smem_u32(&bars.empty[r.stage]), r.phase ^ 1u, abort_flag))) break;
+                if (elect_one()) {
                     const uint32_t full = smem_u32(&bars.full[r.stage]);
                     mbar_expect_tx(full, bytes1);
                     load_a(1, kb, r.stage, full);
                     load_w(1, t, kb, r.stage, full);
                 }
-        }
+            }
         __syncwarp();
     } else if (warp == 1) {
         Ring r;
@@ -192,35 +194,37 @@ step_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUt
             constexpr uint32_t idesc = instr_desc(BM, kBN, 0, 0);
             for (int t = rank; t < p.n_tiles[ph] && ok; t += p.cluster) {
                 if (used) {   // the epilogue has taken the previous tile out of tensor memory
-                    if (!(ok = mbar_wait(smem_u32(&bars.free), free_phase, abort_flag))) break;
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars.free), free_phase, abort_flag))) break;
                     free_phase ^= 1u;
                     tc_fence_after();
                 }
                 used = true;
                 for (int kb = 0; kb < p.k_blocks[ph]; ++kb, r.next(p.stages)) {
-                    if (!(ok = mbar_wait(smem_u32(&bars.full[r.stage]), r.phase, abort_flag))) break;
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars.full[r.stage]), r.phase, abort_flag))) break;
                     tc_fence_after();
                     const uint32_t base = smem_u32(tiles) + (uint32_t)r.stage * (uint32_t)p.stage_bytes;
-                    for (int j = 0; j < n_prod; ++j) {
-                        const bool small = j < n_prod - 1;
-                        const uint32_t d_tmem = tmem_base + (small ? (uint32_t)kBN : 0u);
-                        const bool first = kb == 0 && (j == 0 || !small);
-                        const uint64_t ad = smem_desc_kmajor(base + ((pa >> (4 * j)) & 15u) * kSmATile);
-                        const uint64_t wd = smem_desc_kmajor(base + a_bytes + ((pw >> (4 * j)) & 15u) * kWTile);
+                    if (elect_one()) {
+                        for (int j = 0; j < n_prod; ++j) {
+                            const bool small = j < n_prod - 1;
+                            const uint32_t d_tmem = tmem_base + (small ? (uint32_t)kBN : 0u);
+                            const bool first = kb == 0 && (j == 0 || !small);
+                            const uint64_t ad = smem_desc_kmajor(base + ((pa >> (4 * j)) & 15u) * kSmATile);
+                            const uint64_t wd = smem_desc_kmajor(base + a_bytes + ((pw >> (4 * j)) & 15u) * kWTile);
 #pragma unroll
-                        for (int k = 0; k < BK / UK; ++k)
-                            umma_bf16(d_tmem, ad + (uint64_t)(2 * k), wd + (uint64_t)(2 * k), idesc, (uint32_t)!(first && k == 0));
+                            for (int k = 0; k < BK / UK; ++k)
+                                umma_bf16(d_tmem, ad + (uint64_t)(2 * k), wd + (uint64_t)(2 * k), idesc, (uint32_t)!(first && k == 0));
+                        }
+                        umma_commit(smem_u32(&bars.empty[r.stage]));
                     }
-                    umma_commit(smem_u32(&bars.empty[r.stage]));
                 }
-                if (ok) umma_commit(smem_u32(&bars.done));
+                if (ok && elect_one()) umma_commit(smem_u32(&bars.done));
             }
         };
-        if (lane == 0) run_phase(0, P0::n, P0::a, P0::w);
+        run_phase(0, P0::n, P0::a, P0::w);
         __syncwarp();
         cluster_arrive();
         cluster_wait();
-        if (lane == 0) run_phase(1, P1::n, P1::a, P1::w);
+        run_phase(1, P1::n, P1::a, P1::w);
         __syncwarp();
     } else {
         constexpr int kC4 = kBN / 4, kRowGroups = kStEpiThreads / kC4, kRows = BM / kRowGroups;
