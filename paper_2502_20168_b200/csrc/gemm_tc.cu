@@ -162,6 +162,50 @@ struct TnParams {
     }
 };
 
+// sums[c] += sum over the 32 rows of a[row][c] * b[row][c], c < 32, for two 32 x 32 bf16 tiles in shared memory (64-byte
+// rows, 64-byte swizzle).  The sums are the diagonal of a^T b: eight 16 x 8 x 16 matrix instructions, of whose results one
+// element in 16 is used.  (On the CUDA cores a lane holds a row, so that the products have to be turned round: 32 products
+// and a butterfly of 31 shuffles, about 190 instructions a tile against 40: du and dD of 16384 x 512 x 512
+// 24.9 -> 20.9 us.)
+__device__ __forceinline__ void add_column_dots(uint32_t a, uint32_t b, int lane, float* sums) {
+    const int g = lane >> 2, t = lane & 3;
+    float d[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) d[j][e] = 0.f;
+    // 8 x 8 blocks, transposed on the way: lanes 8 i .. 8 i + 7 point at the rows of block i of four
+    const int r8 = lane & 7, blk = lane >> 3;
+    auto addr = [&](uint32_t base, int row, int chunk) { return base + (uint32_t)(row * 64 + ((chunk ^ ((row >> 1) & 3)) << 4)); };
+    auto load4 = [](uint32_t p, uint32_t (&f)[4]) {
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3]) : "r"(p) : "memory");
+    };
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            uint32_t fa[4], fb[4];   // fa: (chunk, rows) = (2i, lo), (2i + 1, lo), (2i, hi), (2i + 1, hi); fb: (2i, lo), (2i, hi), ...
+            load4(addr(a, 16 * k + 8 * (blk >> 1) + r8, 2 * i + (blk & 1)), fa);
+            load4(addr(b, 16 * k + 8 * (blk & 1) + r8, 2 * i + (blk >> 1)), fb);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                float(&c)[4] = d[2 * i + j];
+                asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                             : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                             : "r"(fa[0]), "r"(fa[1]), "r"(fa[2]), "r"(fa[3]), "r"(fb[2 * j]), "r"(fb[2 * j + 1]));
+            }
+        }
+    // column 8 j + g of block j is element (g, g) of its half of the results: with the lanes whose t is g / 2
+    if (t == (g >> 1)) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int e = 2 * (j & 1);
+            sums[8 * j + g] += (g & 1) ? d[j][e + 1] : d[j][e];
+        }
+    }
+}
+
 // One epilogue warp's share of a finished accumulator tile: rows m0 + 32 (warp % 4) .. + 31, one half
 // of the tile's output columns (from n_out0), in slabs of 32 columns; a lane holds one row of a slab.
 // Waits for the tile's MMAs; false when aborting.
@@ -201,7 +245,7 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
             tmem_ld32(t_row + (uint32_t)c, r);
             if (kSplitW) tmem_ld32(t_row + (uint32_t)(BN / 2 + c), r2);
             tmem_ld_wait();
-            if (lane == 0) tma_store_wait_read();   // the previous slab has left the staging buffer
+            if (elect_one()) tma_store_wait_read();   // the previous slab has left the staging buffer
             __syncwarp();
             // 16-byte chunk j of row `lane` sits at chunk j ^ (lane & 7): the 128-byte swizzle
 #pragma unroll
@@ -218,7 +262,7 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
             }
             fence_async_smem();
             __syncwarp();
-            if (lane == 0 && row0 < p.M && n_out0 + c < p.ldo) tma_store_2d(tmOut, smem_u32(stg), n_out0 + c, row0);
+            if (row0 < p.M && n_out0 + c < p.ldo && elect_one()) tma_store_2d(tmOut, smem_u32(stg), n_out0 + c, row0);
         }
         return true;
     }
@@ -240,7 +284,7 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
     const bool ahead = skip_ahead && *skip_ahead;   // this tile's first two slabs were requested while the last one was drained
     const bool prefetch_next = kEpi != 2 && skip_ahead && next_m0 >= 0;
     if (skip_ahead) *skip_ahead = prefetch_next;
-    if (lane == 0 && !ahead) {
+    if (!ahead && elect_one()) {
         fence_async_smem();   // (the lanes' reads of the previous tile's last slabs: fenced and joined there)
         fetch_skip(0);
         if (kSlabs > 1) fetch_skip(1);
@@ -267,11 +311,11 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
             // generic proxy: without the proxy fences it can land before a lane's read has been served.
             fence_async_smem();
             __syncwarp();
-            if (lane == 0 && sl + 2 < kSlabs) {
+            if (sl + 2 < kSlabs && elect_one()) {
                 fence_async_smem();
                 fetch_skip(sl + 2);
             }
-            if (lane == 0) tma_store_wait_read();   // the previous slab has left both staging buffers
+            if (elect_one()) tma_store_wait_read();   // the previous slab has left both staging buffers
             __syncwarp();
             uint4 o[4];
 #pragma unroll
@@ -292,7 +336,7 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
             }
             fence_async_smem();
             __syncwarp();
-            if (lane == 0 && row0 < p.M && n_out0 + c < p.ldo) {
+            if (row0 < p.M && n_out0 + c < p.ldo && elect_one()) {
                 tma_store_2d(tmOut, smem_u32(stg), n_out0 + c, row0);
                 tma_store_2d(tmGate, smem_u32(ob), n_out0 + c, row0);
             }
@@ -309,20 +353,10 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
         uint4 sk[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) sk[j] = *reinterpret_cast<const uint4*>(skb + b * 2048 + lane * 64 + ((j ^ swz) << 4));
-        float prod[kDot ? 32 : 1];
-        if (kDot) {   // skip * dot for this lane's row of the slab
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint4 dt = *reinterpret_cast<const uint4*>(skb + 4096 + b * 2048 + lane * 64 + ((j ^ swz) << 4));
-                const __nv_bfloat162* s2 = reinterpret_cast<const __nv_bfloat162*>(&sk[j]);
-                const __nv_bfloat162* d2 = reinterpret_cast<const __nv_bfloat162*>(&dt);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 a = __bfloat1622float2(s2[e]), c2 = __bfloat1622float2(d2[e]);
-                    prod[8 * j + 2 * e] = a.x * c2.x;
-                    prod[8 * j + 2 * e + 1] = a.y * c2.y;
-                }
-            }
+        if (kDot) {
+            const uint32_t dots = smem_u32(skb + b * 2048);
+            float* acc_cols = s.diag + kDotMaxN + (size_t)w * (kDotMaxN / 2) + (n_out0 / BN) * (BN / 2) + sl * 32;
+            add_column_dots(dots, dots + 4096, lane, acc_cols);   // (rows outside M were read as zero)
         }
         tmem_ld_wait();
         // Every lane has asked for its skip row; the buffer takes the slab after next.  That refill is a
@@ -331,7 +365,7 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
         // kernel shared the SMs and the skip rows came from L2).
         fence_async_smem();
         __syncwarp();
-        if (lane == 0) {
+        if (elect_one()) {
             if (sl + 2 < kSlabs) {
                 fence_async_smem();
                 fetch_skip(sl + 2);
@@ -356,31 +390,13 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
             }
         }
         uint8_t* ob = stg_bytes + b * 2048;
-        if (lane == 0) tma_store_wait_read_n<1>();   // the store from this buffer two slabs ago has read it
+        if (elect_one()) tma_store_wait_read_n<1>();   // the store from this buffer two slabs ago has read it
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(ob + lane * 64 + ((j ^ swz) << 4)) = o[j];
         fence_async_smem();
         __syncwarp();
-        if (lane == 0 && row0 < p.M && n_out0 + c < p.ldo) tma_store_2d(tmOut, smem_u32(ob), n_out0 + c, row0);
-        if (kDot) {
-            // Column sums over the warp's 32 rows: at every halving step a lane keeps the half of its values
-            // that its lane bit selects and adds the other lane's; lane l ends with the sum of column l.
-#pragma unroll
-            for (int h = 16; h >= 1; h >>= 1) {
-                const bool upper = (lane & h) != 0;
-#pragma unroll
-                for (int j = 0; j < h; ++j) {
-                    const float send = upper ? prod[j] : prod[j + h];
-                    const float keep = upper ? prod[j + h] : prod[j];
-                    prod[j] = keep + __shfl_xor_sync(0xffffffffu, send, h);
-                }
-            }
-            // this warp's own sums (it always drains the same half of a tile's columns): rows outside M were
-            // read as zero
-            float* acc_col = s.diag + kDotMaxN + (size_t)w * (kDotMaxN / 2) + (n_out0 / BN) * (BN / 2) + sl * 32 + lane;
-            *acc_col += prod[0];
-        }
+        if (row0 < p.M && n_out0 + c < p.ldo && elect_one()) tma_store_2d(tmOut, smem_u32(ob), n_out0 + c, row0);
     }
     return true;
 }
@@ -540,7 +556,7 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             mbar_arrive_cluster(leader_empty0 + 8u * acc);
             if ((acc ^= 1) == 0) acc_phase ^= 1u;
         }
-        if (lane == 0) tma_store_wait_all();
+        if (elect_one()) tma_store_wait_all();
         if (kEpi == 3) {
             // this CTA's column sums: the four warps that drain a column half added in a fixed order, one row
             // of p.dot_part per CTA (the sum over the CTAs follows in another kernel)
@@ -792,7 +808,8 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         const int te = threadIdx.x - 64;            // 0 .. kFsEpiThreads - 1
         const int q = warp & 3, grp = (warp - 2) >> 2;   // drain role: TMEM lane quarter, 32-column group
         const int sp = te % kPairs, sl = te / kPairs;   // scan role: pair of states of the tile, group of its rows
-        const bool group_leader = lane % kPairs == 0;   // the lane that talks to the TMA unit for its row group
+        // the lane that talks to the TMA unit for its row group (always the same one)
+        auto group_leader = [&] { return kPairs == 32 ? elect_one() : lane % kPairs == 0; };
         const int prow = q * 32 + lane;             // drain role: row of the tile
         float4* T4 = reinterpret_cast<float4*>(s.staging);
         const C2 zero = {0ull, 0ull};
@@ -873,7 +890,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 }
                 flag_next = tb + 1 < p.tblocks ? flag_of(chain, tb + 1) : flag_of(chain + npairs, 0);
                 (void)mbar_wait(s.tmem_full(acc), acc_phase, s.abort_flag);
-                if (group_leader) tma_store_wait_read();   // this row group's results of the previous tile have left shared memory
+                if (group_leader()) tma_store_wait_read();   // this row group's results of the previous tile have left shared memory
                 epi_sync();   // flags visible, tile free (nobody reads the previous one any more); also:
                               // the 256 threads leave together or not at all
                 if (*s.abort_flag) {
@@ -1064,7 +1081,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 }
                 fence_async_smem();
                 __syncwarp();
-                if (group_leader && grp_valid) {
+                if (grp_valid && group_leader()) {
                     if (kRagged) tma_store_4d_nocommit(&tmX, smem_u32(warp_out), n_tile * kS, p.T - left + r0, b, 0);   // clipped at T
                     else tma_store_3d_nocommit(&tmX, smem_u32(warp_out), n_tile * kS, m0 + r0, 0);
                     tma_commit_group();
@@ -1095,7 +1112,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 }
             }
         }
-        if (group_leader) tma_store_wait_all();
+        if (group_leader()) tma_store_wait_all();
     }
     tc_fence_before();
     __syncwarp();
@@ -1262,7 +1279,8 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         const int te = threadIdx.x - 64;            // 0 .. kFsEpiThreads - 1
         const int q = warp & 3, grp = (warp - 2) >> 2;   // drain role: TMEM lane quarter, 32-column group
         const int sp = te % kPairs, sl = te / kPairs;   // scan role: pair of states of the tile, group of its rows
-        const bool group_leader = lane % kPairs == 0;   // the lane that talks to the TMA unit for its row group
+        // the lane that talks to the TMA unit for its row group (always the same one)
+        auto group_leader = [&] { return kPairs == 32 ? elect_one() : lane % kPairs == 0; };
         const int prow = q * 32 + lane;             // drain role: row of the tile
         const bool short_seq = !kTPair && !kRagged && p.T < BM;            // then a chain is one tile of 128 / T whole sequences
         const int g0 = sl - sl % p.gps;             // first and last row group of this group's sequence in the tile
@@ -1280,6 +1298,15 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         int acc = 0;
         uint32_t acc_phase = 0;
         bool ok = true;
+        // The flags of this thread's row of a tile, loaded one tile ahead: bit 0 a row's own flag, bit 1 the flag of the row
+        // after it if that row belongs to the same sequence.
+        auto flags_of = [&](int chain, int tb) -> uint32_t {
+            if (!p.done || te >= BM || chain >= p.nchains || seq_of(chain) >= p.n_units) return 0u;
+            const int m = row_of(chain, tb) + te, tix = kTPair ? 2 * tb + (int)rank : tb;   // tix: the tile's place in its sequence
+            const bool next_in_seq = short_seq ? ((te + 1) % p.T != 0 && m + 1 < M) : (tix * BM + te + 1 < p.T);
+            return (m < M && p.done[(size_t)m] != 0 ? 1u : 0u) | (next_in_seq && p.done[(size_t)m + 1] != 0 ? 2u : 0u);
+        };
+        uint32_t flags_next = flags_of(pair, p.tblocks - 1);
         // The chain's multipliers are loaded one chain ahead (a chain is a single tile when the sequences are short).
         auto abar_of = [&](int chain, int k) {
             return chain < p.nchains ? p.Abar[(chain % p.n_tiles) * kS + 2 * sp + k] : make_float2(0.f, 0.f);
@@ -1331,17 +1358,13 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             for (int tb = p.tblocks - 1; tb >= 0; --tb) {
                 const int m0 = row_of(chain, tb);
                 if (p.done && te < BM) {
-                    // a row's own flag, and the flag of the row after it if that row belongs to the same sequence
-                    const int tix = kTPair ? 2 * tb + (int)rank : tb;   // this tile's place in its sequence
-                    const bool next_in_seq = short_seq ? ((te + 1) % p.T != 0 && m0 + te + 1 < M) : (tix * BM + te + 1 < p.T);
-                    const bool f0 = has_seq && m0 + te < M && p.done[(size_t)m0 + te] != 0;
-                    const bool f1 = has_seq && next_in_seq && p.done[(size_t)m0 + te + 1] != 0;
-                    const uint32_t mk0 = __ballot_sync(0xffffffffu, f0), mk1 = __ballot_sync(0xffffffffu, f1);
+                    const uint32_t mk0 = __ballot_sync(0xffffffffu, flags_next & 1u), mk1 = __ballot_sync(0xffffffffu, flags_next & 2u);
                     if (lane == 0) {
                         masks[te >> 5] = mk1;
                         masks[4 + (te >> 5)] = mk0;
                     }
                 }
+                flags_next = tb > 0 ? flags_of(chain, tb - 1) : flags_of(chain + npairs, p.tblocks - 1);
                 (void)mbar_wait(s.tmem_full(acc), acc_phase, s.abort_flag);
                 tc_fence_after();
                 // (1) accumulators -> shared-memory tile: 16-byte chunk j of a 128-byte group sits at j ^ (row & 7).
@@ -1353,7 +1376,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 uint32_t ra[32], ra2[32], rb[32], rb2[32];
                 tmem_ld32(t_row + (uint32_t)(grp * 32), ra);
                 tmem_ld32(t_row + (uint32_t)(Cfg::kCols + grp * 32), ra2);
-                if (group_leader) tma_store_wait_read();   // this row group's results of the previous tile have left shared memory
+                if (group_leader()) tma_store_wait_read();   // this row group's results of the previous tile have left shared memory
                 epi_sync();   // flags visible, tile free (nobody reads the previous one any more); also:
                               // the 256 threads leave together or not at all
                 tmem_ld_wait();
@@ -1431,7 +1454,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 // the warp has its rows: rows m - 1 ... m + R - 2 of x (both planes) into its part of the tile
                 fence_async_smem();
                 __syncwarp();
-                if (group_leader) {
+                if (group_leader()) {
                     mbar_expect_tx(xb, Cfg::kGroupBytes);
                     tma_load_3d(smem_u32(warp_buf), &tmX, xb, n_tile * kS, m0 + r0 - 1, 0);
                     // and the same rows of the tile before this one into L2, where the next load will find them
@@ -1589,7 +1612,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     fold_rows(std::true_type{});
                 fence_async_smem();
                 __syncwarp();
-                if (group_leader && grp_valid) {
+                if (grp_valid && group_leader()) {
                     if (kRagged) tma_store_4d_nocommit(&tmS, smem_u32(warp_buf), n_tile * kS, p.T - left + r0, b, 0);   // clipped at T
                     else tma_store_3d_nocommit(&tmS, smem_u32(warp_buf), n_tile * kS, m0 + r0, 0);
                     tma_commit_group();
@@ -1632,7 +1655,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 p.gA_part[part_row * p.P + pg + 1] = make_float2(sum.y, sum.w);
             }
         }
-        if (group_leader) tma_store_wait_all();
+        if (group_leader()) tma_store_wait_all();
     }
     tc_fence_before();
     __syncwarp();
