@@ -1946,7 +1946,7 @@ static int sm_count() { return device_sm_count(); }
 
 // How many clusters of two CTAs of `kernel` the current device runs at the same time (cached per
 // kernel and device).
-static int resident_pairs(const void* kernel, size_t smem_bytes, int threads = kTnThreads) {
+int resident_pairs(const void* kernel, size_t smem_bytes, int threads) {
     static std::mutex mu;
     static std::map<std::pair<const void*, int>, int> cache;
     int dev = 0;
@@ -2059,7 +2059,7 @@ do {                                                                            
     auto kern = gemm_tc_tn_pair_kernel<EPI, SPLIT>;                                                    \
     constexpr size_t smem = pair_smem_bytes(EPI);                                                      \
     ok = set_smem(kern, smem);                                                                         \
-    const int pairs = ok ? resident_pairs(reinterpret_cast<const void*>(kern), smem) : 0;              \
+    const int pairs = ok ? resident_pairs(reinterpret_cast<const void*>(kern), smem, kTnThreads) : 0;              \
     ok = ok && pairs > 0;                                                                              \
     if (ok) launch_dep(kern, 2 * min(pairs, pair_tiles), kTnThreads, smem, st, ma, mw, mo, ms, mg, p);         \
     if (ok && g.dot_rows) *g.dot_rows = 2 * min(pairs, pair_tiles);                                    \

@@ -2,14 +2,16 @@
 // of both operands, with the layer's epilogue (fp32 store, or out = acc + diag * skip (+ add) and the column sums of
 // skip * dot).
 //
-// Persistent, one CTA per SM on 128 x 128 tiles: a warp brings in every plane of 32 columns of K once (48 KB, four
-// stages), one thread issues the 12 MMAs of a stage, and eight warps run the epilogue of one tile out of one half of
-// tensor memory while the MMAs of the next fill the other.  The one-tile-per-CTA kernel of gemm_tc_small.cu, which
+// Persistent, CTA pairs on 256 x 128 tiles: a CTA holds its 128 rows of A and 64 rows of W and brings in every plane of
+// 32 columns of K once (36 KB, five stages), one thread of the pair issues the 12 MMAs of a stage, and eight warps of
+// each CTA run the epilogue of its half of one tile out of one half of tensor memory while the MMAs of the next fill the
+// other.  The one-tile-per-CTA kernel of gemm_tc_small.cu, which
 // splits an fp32 operand itself and is better for few tiles, alternates on large problems between waiting for memory
 // and multiplying, and splits every row once per column tile: 64000 x 512 x 512 with the skip term and the column sums
-// 329 us there, 152 us here and 52 us for the planes (they serve the weight gradients as well).
-// Bound by shared memory: per 64 columns of K the MMAs read 192 KB and the operands take 96 KB to write, 2250 cycles
-// at 128 B, against 1536 of the tensor core.
+// 329 us there, 149 us here and 52 us for the planes (they serve the weight gradients as well).
+// A 128 x 128 x 16 MMA of one CTA takes 97 cycles, of which 64 are the tensor core's (the operands come from shared
+// memory: 8 KB), a 256 x 128 x 16 MMA of a pair 70 for twice the work.  64000 x 512 x 512 in a layer's passes,
+// one CTA per 128 x 128 tile / pairs: 175 / 136 us, with the skip term and the column sums 189 / 149.
 // hi hi has an accumulator of its own (see gemm_tc_small.cu).
 #include <algorithm>
 
@@ -21,8 +23,8 @@ namespace tc {
 
 constexpr int kPlBN = 128;
 constexpr int kPlBK = 32;      // K extent of an operand stage: 64-byte rows
-constexpr int kPlStages = 4;
-constexpr int kPlATile = BM * kPlBK * 2, kPlWTile = kPlBN * kPlBK * 2;   // one plane
+constexpr int kPlStages = 5;
+constexpr int kPlATile = BM * kPlBK * 2, kPlWTile = kPlBN / 2 * kPlBK * 2;   // one plane, of a CTA
 constexpr int kPlStageBytes = 3 * kPlATile + 3 * kPlWTile;
 constexpr int kPlEpiWarps = 8;
 constexpr int kPlThreads = 64 + 32 * kPlEpiWarps;
@@ -49,13 +51,14 @@ struct PlanesBars {
 };
 
 template <bool kDiag>
-__global__ void __launch_bounds__(kPlThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPlThreads, 1)
 gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ PlanesArgs p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ PlanesBars bars;
     uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     volatile int* abort_flag = &bars.abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = (int)cluster_ctarank();
+    const int pair = (int)blockIdx.x >> 1, npairs = (int)gridDim.x >> 1;
     if (threadIdx.x == 0) {
         for (int i = 0; i < kPlStages; ++i) {
             mbar_init(smem_u32(&bars.full[i]), 1);
@@ -63,7 +66,7 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&bars.done[i]), 1);
-            mbar_init(smem_u32(&bars.free[i]), kPlEpiWarps);
+            mbar_init(smem_u32(&bars.free[i]), 2 * kPlEpiWarps);
         }
         bars.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -72,9 +75,9 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         prefetch_tmap(&tmW);
     }
     __syncwarp();
-    if (warp == 1) tmem_alloc(smem_u32(&bars.tmem), 512);
+    if (warp == 1) tmem_alloc_pair(smem_u32(&bars.tmem), 512);
     tc_fence_before();
-    __syncthreads();
+    cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = bars.tmem;
     grid_dep_wait();
@@ -84,18 +87,18 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         int stage = 0;
         uint32_t phase = 0;
         bool ok = true;
-        for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x) {
-            const int m0 = (tile / p.n_tiles) * BM, n0 = (tile % p.n_tiles) * kPlBN;
+        for (int tile = pair; tile < p.tiles && ok; tile += npairs) {
+            const int m0 = (2 * (tile / p.n_tiles) + rank) * BM, n0 = (tile % p.n_tiles) * kPlBN + rank * (kPlBN / 2);
             for (int kb = 0; kb < p.k_blocks; ++kb) {
                 if (!(ok = mbar_wait_warp(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag))) break;
-                const uint32_t full = smem_u32(&bars.full[stage]);
+                const uint32_t full = map_to_cta(smem_u32(&bars.full[stage]), 0);   // the leader counts both CTAs' loads
                 const uint32_t dst = smem_u32(stages) + (uint32_t)stage * kPlStageBytes;
                 if (elect_one()) {
-                    mbar_expect_tx(full, (uint32_t)(p.planes_a * kPlATile + 3 * kPlWTile));
-                    for (int q = 0; q < p.planes_a; ++q) tma_load_2d(dst + q * kPlATile, &tmA, full, q * p.K + kb * kPlBK, m0);
+                    if (rank == 0) mbar_expect_tx(smem_u32(&bars.full[stage]), 2u * (uint32_t)(p.planes_a * kPlATile + 3 * kPlWTile));
+                    for (int q = 0; q < p.planes_a; ++q) tma_load_2d_pair(dst + q * kPlATile, &tmA, full, q * p.K + kb * kPlBK, m0);
 #pragma unroll
                     for (int q = 0; q < 3; ++q)
-                        tma_load_2d(dst + 3 * kPlATile + q * kPlWTile, &tmW, full, q * p.K + kb * kPlBK, n0);
+                        tma_load_2d_pair(dst + 3 * kPlATile + q * kPlWTile, &tmW, full, q * p.K + kb * kPlBK, n0);
                 }
                 if (++stage == kPlStages) {
                     stage = 0;
@@ -104,41 +107,43 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
             }
         }
     } else if (warp == 1) {
-        constexpr uint32_t idesc = instr_desc(BM, kPlBN, 0, 0);
-        const int n_prod = p.n_prod;
-        const uint32_t pa = p.pa, pw = p.pw;
-        int stage = 0, n = 0;
-        uint32_t phase = 0;
-        bool ok = true;
-        for (int tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x, ++n) {
-            const int buf = n & 1;
-            if (n >= 2) {   // the epilogue has taken tile n - 2 out of this half of tensor memory
-                if (!(ok = mbar_wait_warp(smem_u32(&bars.free[buf]), (uint32_t)((n >> 1) - 1) & 1u, abort_flag))) break;
-                tc_fence_after();
-            }
-            for (int kb = 0; kb < p.k_blocks; ++kb) {
-                if (!(ok = mbar_wait_warp(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
-                tc_fence_after();
-                const uint32_t base = smem_u32(stages) + (uint32_t)stage * kPlStageBytes;
-                if (elect_one()) {
-                    for (int j = 0; j < n_prod; ++j) {
-                        const bool small = j < n_prod - 1;
-                        const uint32_t d_tmem = tmem_base + 256u * (uint32_t)buf + (small ? 128u : 0u);
-                        const uint64_t ad = smem_desc_kmajor64(base + ((pa >> (4 * j)) & 15u) * kPlATile);
-                        const uint64_t wd = smem_desc_kmajor64(base + 3 * kPlATile + ((pw >> (4 * j)) & 15u) * kPlWTile);
+        if (rank == 0) {
+            constexpr uint32_t idesc = instr_desc(2 * BM, kPlBN, 0, 0);
+            const int n_prod = p.n_prod;
+            const uint32_t pa = p.pa, pw = p.pw;
+            int stage = 0, n = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int tile = pair; tile < p.tiles && ok; tile += npairs, ++n) {
+                const int buf = n & 1;
+                if (n >= 2) {   // the epilogue has taken tile n - 2 out of this half of tensor memory
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars.free[buf]), (uint32_t)((n >> 1) - 1) & 1u, abort_flag))) break;
+                    tc_fence_after();
+                }
+                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
+                    tc_fence_after();
+                    const uint32_t base = smem_u32(stages) + (uint32_t)stage * kPlStageBytes;
+                    if (elect_one()) {
+                        for (int j = 0; j < n_prod; ++j) {
+                            const bool small = j < n_prod - 1;
+                            const uint32_t d_tmem = tmem_base + 256u * (uint32_t)buf + (small ? 128u : 0u);
+                            const uint64_t ad = smem_desc_kmajor64(base + ((pa >> (4 * j)) & 15u) * kPlATile);
+                            const uint64_t wd = smem_desc_kmajor64(base + 3 * kPlATile + ((pw >> (4 * j)) & 15u) * kPlWTile);
 #pragma unroll
-                        for (int k = 0; k < kPlBK / UK; ++k)
-                            umma_bf16(d_tmem, ad + (uint64_t)(2 * k), wd + (uint64_t)(2 * k), idesc,
-                                      (uint32_t)!(kb == 0 && k == 0 && (j == 0 || !small)));
+                            for (int k = 0; k < kPlBK / UK; ++k)
+                                umma_bf16_pair(d_tmem, ad + (uint64_t)(2 * k), wd + (uint64_t)(2 * k), idesc,
+                                          (uint32_t)!(kb == 0 && k == 0 && (j == 0 || !small)));
+                        }
+                        umma_commit_pair(smem_u32(&bars.empty[stage]));
                     }
-                    umma_commit(smem_u32(&bars.empty[stage]));
+                    if (++stage == kPlStages) {
+                        stage = 0;
+                        phase ^= 1u;
+                    }
                 }
-                if (++stage == kPlStages) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
+                if (ok && elect_one()) umma_commit_pair(smem_u32(&bars.done[buf]));
             }
-            if (ok && elect_one()) umma_commit(smem_u32(&bars.done[buf]));
         }
     } else {
         // A warp drains 32 rows x 64 columns of a tile in slabs of 32 x 32.  A slab is turned round in the warp's 4 KB of
@@ -147,9 +152,10 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         const int ew = warp - 2, q = warp & 3, half = ew >> 2;
         float4* slab = reinterpret_cast<float4*>(stages + (size_t)kPlStages * kPlStageBytes + (size_t)ew * kPlSlabBytes);
         const int c = lane & 7, rr = lane >> 3;
+        const uint32_t leader_free = map_to_cta(smem_u32(&bars.free[0]), 0);
         int n = 0;
-        for (int tile = blockIdx.x; tile < p.tiles; tile += gridDim.x, ++n) {
-            const int buf = n & 1, m0 = (tile / p.n_tiles) * BM + 32 * q, n0 = (tile % p.n_tiles) * kPlBN + 64 * half;
+        for (int tile = pair; tile < p.tiles; tile += npairs, ++n) {
+            const int buf = n & 1, m_tile = 2 * (tile / p.n_tiles) + rank, m0 = m_tile * BM + 32 * q, n0 = (tile % p.n_tiles) * kPlBN + 64 * half;
             bool ok = true;
 #pragma unroll 1
             for (int sl = 0; sl < 2; ++sl) {
@@ -188,7 +194,7 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                 if (sl == 1) {
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&bars.free[buf]));
+                    if (lane == 0) mbar_arrive_cluster(leader_free + 8u * (uint32_t)buf);
                 }
                 __syncwarp();
                 float4 dg = make_float4(0.f, 0.f, 0.f, 0.f), dsum = dg;
@@ -231,18 +237,20 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                         dsum.z += __shfl_xor_sync(0xffffffffu, dsum.z, o);
                         dsum.w += __shfl_xor_sync(0xffffffffu, dsum.w, o);
                     }
-                    if (rr == 0 && n_ok)
-                        *reinterpret_cast<float4*>(p.dot_part + (size_t)(4 * (tile / p.n_tiles) + q) * p.N + col) = dsum;
+                    if (rr == 0 && n_ok && m_tile * BM < p.M)
+                        *reinterpret_cast<float4*>(p.dot_part + (size_t)(4 * m_tile + q) * p.N + col) = dsum;
                 }
                 __syncwarp();   // the slab is free
             }
             if (!ok) break;
         }
     }
+    // nobody leaves (or frees tensor memory) while the other CTA may still signal or compute
     tc_fence_before();
-    __syncthreads();
+    __syncwarp();
+    cluster_sync_all();
     tc_fence_after();
-    if (warp == 1) tmem_dealloc(tmem_base, 512);
+    if (warp == 1) tmem_dealloc_pair(tmem_base, 512);
     if (threadIdx.x == 0 && *abort_flag && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
 }
 
@@ -262,18 +270,18 @@ int launch_gemm_tc_planes(const GemmTcTN& g, cudaStream_t st) {
     p.planes_a = g.planes_a, p.n_prod = g.n_products, p.pa = g.prod_a, p.pw = g.prod_w;
     p.n_tiles = (g.N_out + kPlBN - 1) / kPlBN;
     const int m_tiles = (g.M + BM - 1) / BM;
-    p.tiles = m_tiles * p.n_tiles;
+    p.tiles = (m_tiles + 1) / 2 * p.n_tiles;
     p.out = g.out, p.diag = g.diag, p.skip = g.skip, p.dot = g.dot, p.add = g.add, p.dot_part = g.dot_part;
     p.out_bf16 = !g.store_f32, p.skip_bf16 = g.skip_bf16, p.dot_bf16 = g.dot_bf16, p.hdr = g.hdr;
     if (g.dot_rows) *g.dot_rows = 4 * m_tiles;
     CUtensorMap ma, mw;
     if (!make_map(&ma, g.A, (uint64_t)g.M, (uint64_t)g.planes_a * g.K, kPlBK, BM, false, CU_TENSOR_MAP_SWIZZLE_64B)) return SSM_ERR_CUDA;
-    if (!make_map(&mw, g.W, (uint64_t)g.N_out, 3 * (uint64_t)g.K, kPlBK, kPlBN, false, CU_TENSOR_MAP_SWIZZLE_64B)) return SSM_ERR_CUDA;
-    const int grid = std::min(p.tiles, device_sm_count());
+    if (!make_map(&mw, g.W, (uint64_t)g.N_out, 3 * (uint64_t)g.K, kPlBK, kPlBN / 2, false, CU_TENSOR_MAP_SWIZZLE_64B)) return SSM_ERR_CUDA;
     count_launch();
     auto run = [&](auto kern) {
-        return set_max_dynamic_smem(reinterpret_cast<const void*>(kern), kPlSmem) &&
-               launch_dep(kern, grid, kPlThreads, kPlSmem, st, ma, mw, p);
+        if (!set_max_dynamic_smem(reinterpret_cast<const void*>(kern), kPlSmem)) return false;
+        const int pairs = std::min(p.tiles, resident_pairs(reinterpret_cast<const void*>(kern), kPlSmem, kPlThreads));
+        return pairs > 0 && launch_dep(kern, 2 * pairs, kPlThreads, kPlSmem, st, ma, mw, p);
     };
     return (g.diag ? run(gemm_tc_planes_kernel<true>) : run(gemm_tc_planes_kernel<false>)) ? SSM_OK : SSM_ERR_CUDA;
 }

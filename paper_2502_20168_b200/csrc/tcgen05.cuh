@@ -194,5 +194,8 @@ inline bool make_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Clusters of two CTAs of `kernel` that the current device runs at the same time (gemm_tc.cu; 0: not launchable).
+int resident_pairs(const void* kernel, size_t smem_bytes, int threads);
+
 }  // namespace tc
 }  // namespace ssm
