@@ -7,8 +7,11 @@
 // twice the size) and took one launch per product.  The last product (hi hi) has an accumulator of its own (see
 // gemm_tc_small.cu).  The tensor core truncates at every addition, so the error of a sum grows with the length of its
 // chain: after kNpSegment k-blocks the epilogue warps take the tile out of tensor memory and add it to their registers
-// while the next segment runs in the other half of tensor memory (64000 rows: dB 1.6e-5 off without).  Bound by operand delivery (96 KB per 1536 tensor-core cycles) on large problems, by the fixed
-// part of a launch on small ones.
+// while the next segment runs in the other half of tensor memory (64000 rows: dB 1.6e-5 off without).
+// kPair: a CTA pair takes a tile of 256 x 128, each CTA 128 columns of A and 64 of B (72 KB a k-block).  A 128 x 128 x 16
+// MMA takes 97 cycles because its operands come out of shared memory at 8 KB per 64 tensor-core cycles, a pair's 256 x
+// 128 x 16 takes 70: both products of 64000 x 512 x 512 350 / 286 us.  Where I leaves half of a pair's last tile empty and there
+// are few tiles (I = 128, 384), one CTA per tile is at least as fast.
 #include <algorithm>
 
 #include "kernels.h"
@@ -44,7 +47,7 @@ struct NtPlanesBars {
     int abort_flag;
 };
 
-template <int kN>
+template <int kN, bool kPair>
 __global__ void __launch_bounds__(kNpThreads, 1)
 gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __grid_constant__ NtPlanesArgs p) {
     extern __shared__ uint8_t smem_raw[];
@@ -54,7 +57,9 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const NtPlanesArgs::Product& pr = p.product[blockIdx.z];
     const CUtensorMap *ta = &maps.a[blockIdx.z], *tb = &maps.b[blockIdx.z];
-    const int i0 = ((int)blockIdx.x / p.j_tiles) * 128, j0 = ((int)blockIdx.x % p.j_tiles) * 128;
+    constexpr int kBTile = kPair ? kNpTile / 2 : kNpTile;   // one plane of this CTA's columns of B
+    const int rank = kPair ? (int)cluster_ctarank() : 0, tile = kPair ? (int)blockIdx.x >> 1 : (int)blockIdx.x;
+    const int i0 = (tile / p.j_tiles) * (kPair ? 256 : 128) + 128 * rank, j0 = (tile % p.j_tiles) * 128;
     const int total = (p.K + BK - 1) / BK;
     const int kb0 = (int)blockIdx.y * p.blocks_per_split, kb1 = min(total, kb0 + p.blocks_per_split);
     const int planes_a = pr.planes_a, planes_b = pr.planes_b;
@@ -65,7 +70,7 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&bars.done[i]), 1);
-            mbar_init(smem_u32(&bars.free[i]), 8);
+            mbar_init(smem_u32(&bars.free[i]), kPair ? 16 : 8);
         }
         bars.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -74,31 +79,40 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __
         prefetch_tmap(tb);
     }
     __syncwarp();
-    if (warp == 1) tmem_alloc(smem_u32(&bars.tmem), 512);
+    if (warp == 1) {
+        if (kPair) tmem_alloc_pair(smem_u32(&bars.tmem), 512);
+        else tmem_alloc(smem_u32(&bars.tmem), 512);
+    }
     tc_fence_before();
-    __syncthreads();
+    if (kPair) cluster_sync_all();   // the other CTA's barriers are set up
+    else __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = bars.tmem;
     grid_dep_wait();
     grid_dep_launch();
 
     if (warp == 0) {
-        const uint32_t bytes = (uint32_t)(planes_a + planes_b) * kNpTile;
+        const uint32_t bytes = (uint32_t)planes_a * kNpTile + (uint32_t)planes_b * kBTile;
         int stage = 0;
         uint32_t phase = 0;
         for (int kb = kb0; kb < kb1; ++kb) {
             if (!mbar_wait_warp(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
-            const uint32_t full = smem_u32(&bars.full[stage]);
+            // (a pair counts both CTAs' loads on the barrier of CTA 0, which issues the MMAs)
+            const uint32_t full = kPair ? map_to_cta(smem_u32(&bars.full[stage]), 0) : smem_u32(&bars.full[stage]);
             uint32_t dst = smem_u32(tiles) + (uint32_t)stage * (uint32_t)p.stage_bytes;
             if (elect_one()) {
-                mbar_expect_tx(full, bytes);
+                if (rank == 0) mbar_expect_tx(smem_u32(&bars.full[stage]), kPair ? 2 * bytes : bytes);
+                auto load = [&](uint32_t to, const CUtensorMap* map, int c0) {
+                    if (kPair) tma_load_2d_pair(to, map, full, c0, kb * BK);
+                    else tma_load_2d(to, map, full, c0, kb * BK);
+                };
                 for (int q = 0; q < planes_a; ++q, dst += kNpTile) {
-                    tma_load_2d(dst, ta, full, q * p.I + i0, kb * BK);
-                    tma_load_2d(dst + kNpTile / 2, ta, full, q * p.I + i0 + 64, kb * BK);
+                    load(dst, ta, q * p.I + i0);
+                    load(dst + kNpTile / 2, ta, q * p.I + i0 + 64);
                 }
-                for (int q = 0; q < planes_b; ++q, dst += kNpTile) {
-                    tma_load_2d(dst, tb, full, q * p.J + j0, kb * BK);
-                    tma_load_2d(dst + kNpTile / 2, tb, full, q * p.J + j0 + 64, kb * BK);
+                for (int q = 0; q < planes_b; ++q, dst += kBTile) {
+                    load(dst, tb, q * p.J + j0 + 64 * rank);
+                    if (!kPair) load(dst + kNpTile / 2, tb, q * p.J + j0 + 64);
                 }
             }
             if (++stage == p.stages) {
@@ -107,8 +121,8 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __
             }
         }
     } else if (warp == 1) {
-        if (kb0 < kb1) {
-            constexpr uint32_t idesc = instr_desc(128, 128, 1, 1);
+        if (kb0 < kb1 && rank == 0) {
+            constexpr uint32_t idesc = instr_desc(kPair ? 256 : 128, 128, 1, 1);
             const int n_prod = pr.n_prod;
             const uint32_t pa = pr.pa, pb = pr.pb;
             int stage = 0;
@@ -130,13 +144,19 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __
                         const uint32_t d_tmem = tmem_base + 256u * (uint32_t)buf + (small ? 128u : 0u);
                         const bool first = seg_first && (j == 0 || !small);
                         const uint64_t ad = smem_desc_mnmajor(base + ((pa >> (4 * j)) & 15u) * kNpTile);
-                        const uint64_t bd = smem_desc_mnmajor(base + ((uint32_t)planes_a + ((pb >> (4 * j)) & 15u)) * kNpTile);
+                        const uint64_t bd = smem_desc_mnmajor(base + (uint32_t)planes_a * kNpTile + ((pb >> (4 * j)) & 15u) * kBTile);
 #pragma unroll
-                        for (int k = 0; k < BK / UK; ++k)   // 16 rows of 128 bytes further: +128 in the address field
-                            umma_bf16(d_tmem, ad + (uint64_t)(128 * k), bd + (uint64_t)(128 * k), idesc, (uint32_t)!(first && k == 0));
+                        for (int k = 0; k < BK / UK; ++k) {   // 16 rows of 128 bytes further: +128 in the address field
+                            if (kPair) umma_bf16_pair(d_tmem, ad + (uint64_t)(128 * k), bd + (uint64_t)(128 * k), idesc, (uint32_t)!(first && k == 0));
+                            else umma_bf16(d_tmem, ad + (uint64_t)(128 * k), bd + (uint64_t)(128 * k), idesc, (uint32_t)!(first && k == 0));
+                        }
                     }
-                    umma_commit(smem_u32(&bars.empty[stage]));
-                    if (kb + 1 == kb1 || (kb + 1 - kb0) % kNpSegment == 0) umma_commit(smem_u32(&bars.done[buf]));
+                    auto commit = [&](uint64_t* bar) {
+                        if (kPair) umma_commit_pair(smem_u32(bar));
+                        else umma_commit(smem_u32(bar));
+                    };
+                    commit(&bars.empty[stage]);
+                    if (kb + 1 == kb1 || (kb + 1 - kb0) % kNpSegment == 0) commit(&bars.done[buf]);
                 }
                 if (++stage == p.stages) {
                     stage = 0;
@@ -169,53 +189,70 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bars.free[buf]));
+            if (lane == 0) {
+                if (kPair) mbar_arrive_cluster(map_to_cta(smem_u32(&bars.free[buf]), 0));
+                else mbar_arrive(smem_u32(&bars.free[buf]));
+            }
         }
-        if (ok)
+        if (ok && row < p.I)
 #pragma unroll
             for (int j = 0; j < 16; ++j)
                 *reinterpret_cast<float4*>(dst + 4 * j) = make_float4(sum[4 * j], sum[4 * j + 1], sum[4 * j + 2], sum[4 * j + 3]);
     }
+    // nobody leaves (or frees tensor memory) while the other CTA may still signal or compute
     tc_fence_before();
-    __syncthreads();
+    __syncwarp();
+    if (kPair) cluster_sync_all();
+    else __syncthreads();
     tc_fence_after();
-    if (warp == 1) tmem_dealloc(tmem_base, 512);
+    if (warp == 1) {
+        if (kPair) tmem_dealloc_pair(tmem_base, 512);
+        else tmem_dealloc(tmem_base, 512);
+    }
     if (threadIdx.x == 0 && *abort_flag && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
 }
 
 }  // namespace tc
 
-// Slices of the rows: as many as leave every SM at most one CTA of the launch.
+// Pairs: where I fills their tiles, and a slice is long enough to pay for the pair's set-up (1024 rows of 256 x 256, one
+// k-block per slice: a pass of that layer takes 64.1 us with single CTAs, 64.9 with pairs; stack of four layers of
+// 1024 rows, 512 x 512, 16 k-blocks per slice: 338.5 and 335.0).
+static bool nt_planes_pairs(int I, int blocks_per_slice) { return blocks_per_slice >= 4 && (I % 256 == 0 || I >= 640); }
+
+// Slices of the rows: as many as leave every SM at most one CTA of the launch (pairs: all but the few SMs that
+// clusters of two cannot use).
 int tc_nt_planes_splits(int K, int I, int J, int n_products) {
-    const int units = n_products * (I / 128) * (J / 128), blocks = (K + tc::BK - 1) / tc::BK;
-    return std::max(1, std::min(std::min(blocks, 64), device_sm_count() / std::max(units, 1)));
+    const int blocks = (K + tc::BK - 1) / tc::BK, most = std::min(blocks, 64);
+    auto slices = [&](int i_tiles, int slots) { return std::max(1, std::min(most, slots / std::max(n_products * i_tiles * (J / 128), 1))); };
+    const int single = slices(I / 128, device_sm_count());
+    return nt_planes_pairs(I, blocks / single) ? slices((I + 255) / 256, (device_sm_count() - 4) / 2) : single;
 }
 
-template <int kN>
+template <int kN, bool kPair>
 static int launch_nt_planes(int K, int I, int J, int splits, int n, const GemmTcNtPlanes* products, WsHeader* hdr, cudaStream_t st) {
     using namespace tc;
-    auto kern = gemm_tc_nt_planes_kernel<kN>;
+    auto kern = gemm_tc_nt_planes_kernel<kN, kPair>;
     if (!set_max_dynamic_smem(reinterpret_cast<const void*>(kern), kNpSmemMax)) return SSM_ERR_CUDA;
     const int blocks = (K + BK - 1) / BK;
     NtPlanesArgs p{};
     NtPlanesMaps<kN> maps{};
     p.K = K, p.I = I, p.J = J, p.j_tiles = J / 128, p.hdr = hdr;
     p.blocks_per_split = (blocks + splits - 1) / splits;
-    int planes = 0;
+    int stage_bytes = 0;
     for (int z = 0; z < n; ++z) {
         const GemmTcNtPlanes& q = products[z];
         if (q.n_products < 2 || q.n_products > 8) return SSM_ERR_SHAPE;
         p.product[z] = {q.planes_a, q.planes_b, q.n_products, q.prod_a, q.prod_b, q.part};
-        planes = std::max(planes, q.planes_a + q.planes_b);
+        stage_bytes = std::max(stage_bytes, q.planes_a * kNpTile + q.planes_b * (kPair ? kNpTile / 2 : kNpTile));
         if (!make_map(&maps.a[z], q.A, (uint64_t)K, (uint64_t)I * q.planes_a, 64, BK)) return SSM_ERR_CUDA;
         if (!make_map(&maps.b[z], q.B, (uint64_t)K, (uint64_t)J * q.planes_b, 64, BK)) return SSM_ERR_CUDA;
     }
-    p.stage_bytes = planes * kNpTile;
+    p.stage_bytes = stage_bytes;
     p.stages = std::min<int>(kNpMaxStages, (int)((kNpSmemMax - 1024) / p.stage_bytes));
     if (p.stages < 2) return SSM_ERR_SHAPE;
     count_launch();
-    const dim3 grid((unsigned)((I / 128) * p.j_tiles), (unsigned)splits, (unsigned)n);
-    return launch_dep(kern, grid, kNpThreads, (size_t)p.stages * p.stage_bytes + 1024, st, maps, p) ? SSM_OK : SSM_ERR_CUDA;
+    const dim3 grid((unsigned)((kPair ? 2 * ((I + 255) / 256) : I / 128) * p.j_tiles), (unsigned)splits, (unsigned)n);
+    return launch_dep_cluster(kern, kPair ? 2u : 1u, grid, kNpThreads, (size_t)p.stages * p.stage_bytes + 1024, st, maps, p) ? SSM_OK : SSM_ERR_CUDA;
 }
 
 int launch_gemm_tc_nt_planes(int K, int I, int J, int splits, int n_products, const GemmTcNtPlanes* products, WsHeader* hdr,
@@ -223,8 +260,9 @@ int launch_gemm_tc_nt_planes(int K, int I, int J, int splits, int n_products, co
     if (I % 128 != 0 || J % 128 != 0) return SSM_ERR_SHAPE;
     for (int first = 0; first < n_products; first += 2 * kLayerBatch) {
         const int n = std::min(2 * kLayerBatch, n_products - first);
-        const int rc = n <= 2 ? launch_nt_planes<2>(K, I, J, splits, n, products + first, hdr, st)
-                              : launch_nt_planes<2 * kLayerBatch>(K, I, J, splits, n, products + first, hdr, st);
+        auto run = [&](auto launch) { return launch(K, I, J, splits, n, products + first, hdr, st); };
+        const int rc = nt_planes_pairs(I, (K + tc::BK - 1) / tc::BK / splits) ? (n <= 2 ? run(launch_nt_planes<2, true>) : run(launch_nt_planes<2 * kLayerBatch, true>))
+                                          : (n <= 2 ? run(launch_nt_planes<2, false>) : run(launch_nt_planes<2 * kLayerBatch, false>));
         if (rc) return rc;
     }
     return SSM_OK;

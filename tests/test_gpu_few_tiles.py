@@ -28,9 +28,10 @@ def test_gate_edges_bf16(rows, H):
     run_gate(I.Workload("few_gate", B=1, T=rows, H=H, P=8, io_dtype="bf16", seed=rows + H))
 
 
-@pytest.mark.parametrize("B,T,H,P", [(1, 65, 256, 128), (3, 4111, 256, 128), (2, 1025, 512, 384)])
+@pytest.mark.parametrize("B,T,H,P", [(1, 65, 256, 128), (3, 4111, 256, 128), (2, 1025, 512, 384), (3, 1100, 384, 128), (3, 1100, 640, 64)])
 def test_weight_gradients_from_planes_fp32(B, T, H, P):
-    # one k-block and a row of the next; slices of several segments with a ragged end; one slice per tile
+    # one k-block and a row of the next; slices of several segments with a ragged end; one slice per tile; single CTAs on
+    # long slices; pairs whose last tile is half empty
     run(I.Workload("nt32", B=B, T=T, H=H, P=P, io_dtype="f32", p_done=0.01, seed=B + T), with_gxT=True)
 
 
