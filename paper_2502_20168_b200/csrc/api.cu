@@ -473,9 +473,8 @@ SSM_API int ssm_glu_fwd(const ssm_shape* shape, const float* W, const void* v, v
     WsHeader* hdr = at<WsHeader>(ws, p.hdr);
     {
         StageTimer tm("glu_pack_gelu", st);
-        launch_glu_pack(s.H, W, p.tc ? at<void>(ws, p.Wt) : nullptr, p.tc ? at<void>(ws, p.Wn) : nullptr,
-                        p.tc ? nullptr : at<float>(ws, p.Wt), hdr, st);
-        launch_glu_gelu(bf16, p.tc, n, s.H, v, at<void>(ws, p.x1), st);
+        launch_glu_pre(bf16, p.tc, n, s.H, v, at<void>(ws, p.x1), W, p.tc ? at<void>(ws, p.Wt) : nullptr, p.tc ? at<void>(ws, p.Wn) : nullptr,
+                       p.tc ? nullptr : at<float>(ws, p.Wt), hdr, st);
     }
     {   // z[m, j] = sum_i x1[m, i] W[i, j]
         StageTimer tm("glu_gemm_z", st);
@@ -529,6 +528,7 @@ SSM_API int ssm_glu_bwd(const ssm_shape* shape, const float* W, const void* v, c
             launch_gemm_tn(g, st);
         }
     }
+    int slices = p.splits;
     {   // dW[i, j] = sum_m x1[m, i] gz[m, j]
         StageTimer tm("glu_gemm_dW", st);
         if (p.tc) {
@@ -538,16 +538,15 @@ SSM_API int ssm_glu_bwd(const ssm_shape* shape, const float* W, const void* v, c
             g1.A = at<void>(ws, p.x1 + (size_t)s.H * 2);
             g1.part = at<float>(ws, p.part) + (size_t)p.splits * HH;
             if (int rc = launch_gemm_tc_nt2(M, s.H, s.H, p.splits, g0, g1, hdr, st)) return rc;
-            launch_glu_reduce(at<float>(ws, p.part), 2 * p.splits, HH, dW, st);
+            slices *= 2;
         } else {
             const GemmNT g{at<void>(ws, p.x1), false, s.H, at<float>(ws, p.gz), s.H, M, p.splits, at<float>(ws, p.part)};
             launch_gemm_nt(&g, 1, nullptr, st);
-            launch_glu_reduce(at<float>(ws, p.part), p.splits, HH, dW, st);
         }
     }
     {
-        StageTimer tm("glu_gv", st);
-        launch_glu_gv(bf16, n, v, gout, at<float>(ws, p.z), at<float>(ws, p.gx1), gv, st);
+        StageTimer tm("glu_gv", st);   // and the sum of dW's slices
+        launch_glu_post(bf16, at<float>(ws, p.part), slices, HH, dW, n, v, gout, at<float>(ws, p.z), at<float>(ws, p.gx1), gv, st);
     }
     SSM_RETURN_IF_CUDA_ERROR();
     return SSM_OK;

@@ -12,51 +12,17 @@ __device__ __forceinline__ float gelu_f(float v) { return 0.5f * v * (1.f + erff
 __device__ __forceinline__ float gelu_grad_f(float v) {
     return 0.5f * (1.f + erff(v * 0.70710678118654752f)) + v * 0.3989422804014327f * expf(-0.5f * v * v);
 }
-__device__ __forceinline__ float sigmoid_f(float z) { return 1.f / (1.f + expf(-z)); }
+// bf16 results take the fast division (2 ulp of fp32), which is a third of the instructions of the exact one.
+template <typename IO>
+__device__ __forceinline__ float sigmoid_f(float z) {
+    const float d = 1.f + expf(-z);
+    return sizeof(IO) == 2 ? __fdividef(1.f, d) : 1.f / d;
+}
 
 constexpr int kThreads = 256;
 inline int blocks_for(size_t n) {
     const size_t b = (n + kThreads - 1) / kThreads;
     return (int)(b < 148 * 32 ? b : 148 * 32);
-}
-
-// Weight operands.  tc: bf16 planes hi, lo = bf16(w - hi) side by side along the reduction index:
-//   Wz [H, 2H]: row j (output column of z = x1 W), reduction index i: W[i, j], i.e. W transposed;
-//   Wn [H, 2H]: row i (output column of g_x1 = gz W^T), reduction index j: W[i, j].
-// Wt_f32 (CUDA-core path): W transposed.  A block turns a 32 x 32 tile round in shared memory, so that both directions
-// move 64 to 128 contiguous bytes per warp (H = 1024: 38 -> 6 us against one thread per element with strided stores).
-// Also clears the status word of the workspace header.
-__global__ void __launch_bounds__(256)
-glu_pack_kernel(int H, const float* W, __nv_bfloat16* Wz, __nv_bfloat16* Wn, float* Wt_f32, WsHeader* hdr) {
-    __shared__ float t[32][33];
-    grid_dep_wait();
-    grid_dep_launch();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
-    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) hdr->status = 0;
-    auto put = [&](__nv_bfloat16* base, int row, int k, float v) {
-        const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-        base[(size_t)row * 2 * H + k] = hi;
-        base[(size_t)row * 2 * H + H + k] = __float2bfloat16_rn(v - __bfloat162float(hi));
-    };
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int i = i0 + w + 8 * q, j = j0 + lane;
-        if (i < H && j < H) {
-            const float v = W[(size_t)i * H + j];
-            t[w + 8 * q][lane] = v;
-            if (Wn) put(Wn, i, j, v);
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int j = j0 + w + 8 * q, i = i0 + lane;
-        if (i < H && j < H) {
-            const float v = t[lane][w + 8 * q];
-            if (Wz) put(Wz, j, i, v);
-            if (Wt_f32) Wt_f32[(size_t)j * H + i] = v;
-        }
-    }
 }
 
 // The elementwise passes work on groups of 8 consecutive elements (H is a multiple of 8): 16- or
@@ -111,14 +77,59 @@ __device__ __forceinline__ void store8_planes(__nv_bfloat16* p, size_t plane, co
     store8<__nv_bfloat16>(p + plane, lo);
 }
 
+// Weight operands.  tc: bf16 planes hi, lo = bf16(w - hi) side by side along the reduction index:
+//   Wz [H, 2H]: row j (output column of z = x1 W), reduction index i: W[i, j], i.e. W transposed;
+//   Wn [H, 2H]: row i (output column of g_x1 = gz W^T), reduction index j: W[i, j].
+// Wt_f32 (CUDA-core path): W transposed.  A block turns a 32 x 32 tile round in shared memory, so that both directions
+// move 64 to 128 contiguous bytes per warp (H = 1024: 38 -> 6 us against one thread per element with strided stores).
+// Also clears the status word of the workspace header.
+__device__ __forceinline__ void pack_weights(int tile, int H, const float* W, __nv_bfloat16* Wz, __nv_bfloat16* Wn, float* Wt_f32, WsHeader* hdr) {
+    __shared__ float t[32][33];
+    const int n = (H + 31) / 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5, i0 = tile / n * 32, j0 = tile % n * 32;
+    if (threadIdx.x == 0 && tile == 0) hdr->status = 0;
+    auto put = [&](__nv_bfloat16* base, int row, int k, float v) {
+        const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+        base[(size_t)row * 2 * H + k] = hi;
+        base[(size_t)row * 2 * H + H + k] = __float2bfloat16_rn(v - __bfloat162float(hi));
+    };
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = i0 + w + 8 * q, j = j0 + lane;
+        if (i < H && j < H) {
+            const float v = W[(size_t)i * H + j];
+            t[w + 8 * q][lane] = v;
+            if (Wn) put(Wn, i, j, v);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int j = j0 + w + 8 * q, i = i0 + lane;
+        if (i < H && j < H) {
+            const float v = t[lane][w + 8 * q];
+            if (Wz) put(Wz, j, i, v);
+            if (Wt_f32) Wt_f32[(size_t)j * H + i] = v;
+        }
+    }
+}
+
+// What the gate's GEMM reads, in one launch (two are a few us longer: both are short and neither fills the machine): the
+// first blocks lay the weights out, the others compute
 // x1 = GELU(v): fp32 [M, H], or bf16 [M, 2H] with the high halves in columns [0, H) and the low
 // halves (bf16(x1 - hi)) in [H, 2H): one operand for the gate's GEMM with both planes along K, two
 // column blocks for the weight-gradient products.  A single bf16 rounding of x1 is not enough there.
 template <typename IO, bool kPlanes>
-__global__ void glu_gelu_kernel(size_t n, int H, const IO* v, void* x1) {
+__global__ void __launch_bounds__(kThreads)
+glu_pre_kernel(int pack_blocks, size_t n, int H, const IO* v, void* x1, const float* W, __nv_bfloat16* Wz, __nv_bfloat16* Wn, float* Wt_f32,
+               WsHeader* hdr) {
     grid_dep_wait();
     grid_dep_launch();
-    for (size_t e = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 8; e < n; e += (size_t)gridDim.x * blockDim.x * 8) {
+    if ((int)blockIdx.x < pack_blocks) {
+        pack_weights((int)blockIdx.x, H, W, Wz, Wn, Wt_f32, hdr);
+        return;
+    }
+    const size_t step = (size_t)(gridDim.x - pack_blocks) * kThreads * 8;
+    for (size_t e = ((size_t)(blockIdx.x - pack_blocks) * kThreads + threadIdx.x) * 8; e < n; e += step) {
         F8 a = load8<IO>(v + e);
 #pragma unroll
         for (int i = 0; i < 8; ++i) a.x[i] = gelu_f(a.x[i]);
@@ -139,7 +150,7 @@ __global__ void glu_out_kernel(size_t n, const IO* v, const float* z, IO* out) {
         const F8 a = load8<IO>(v + e), zz = load8<float>(z + e);
         F8 o;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) o.x[i] = a.x[i] * sigmoid_f(zz.x[i]);
+        for (int i = 0; i < 8; ++i) o.x[i] = a.x[i] * sigmoid_f<IO>(zz.x[i]);
         store8<IO>(out + e, o);
     }
 }
@@ -155,7 +166,7 @@ __global__ void glu_gz_kernel(size_t n, const IO* v, const IO* gout,
         F8 o;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const float s = sigmoid_f(zz.x[i]);
+            const float s = sigmoid_f<IO>(zz.x[i]);
             o.x[i] = g.x[i] * a.x[i] * s * (1.f - s);
         }
         if (kPlanes) store8_planes(reinterpret_cast<__nv_bfloat16*>(gz) + e, plane, o);
@@ -163,47 +174,50 @@ __global__ void glu_gz_kernel(size_t n, const IO* v, const IO* gout,
     }
 }
 
+// The last launch of the backward pass: the first blocks add the slices of dW, the others compute
+// gv = gout * sigmoid(z) + g_x1 * GELU'(v)
 template <typename IO>
-__global__ void glu_gv_kernel(size_t n, const IO* v, const IO* gout,
-                              const float* z, const float* gx1, IO* gv) {
+__global__ void __launch_bounds__(kThreads)
+glu_post_kernel(int reduce_blocks, const float* part, int splits, size_t n_w, float* dW, size_t n, const IO* v, const IO* gout,
+                const float* z, const float* gx1, IO* gv) {
     grid_dep_wait();
     grid_dep_launch();
-    for (size_t e = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 8; e < n; e += (size_t)gridDim.x * blockDim.x * 8) {
+    if ((int)blockIdx.x < reduce_blocks) {
+        const size_t quads = n_w / 4, step = (size_t)reduce_blocks * kThreads;
+        for (size_t e = (size_t)blockIdx.x * kThreads + threadIdx.x; e < quads; e += step) {
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+            for (int s = 0; s < splits; ++s) {
+                const float4 t = ld_stream(reinterpret_cast<const float4*>(part + (size_t)s * n_w) + e);
+                acc.x += t.x, acc.y += t.y, acc.z += t.z, acc.w += t.w;
+            }
+            reinterpret_cast<float4*>(dW)[e] = acc;
+        }
+        return;
+    }
+    const size_t step = (size_t)(gridDim.x - reduce_blocks) * kThreads * 8;
+    for (size_t e = ((size_t)(blockIdx.x - reduce_blocks) * kThreads + threadIdx.x) * 8; e < n; e += step) {
         const F8 a = load8<IO>(v + e), g = load8<IO>(gout + e), zz = load8<float>(z + e), x = load8<float>(gx1 + e);
         F8 o;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) o.x[i] = g.x[i] * sigmoid_f(zz.x[i]) + x.x[i] * gelu_grad_f(a.x[i]);
+        for (int i = 0; i < 8; ++i) o.x[i] = g.x[i] * sigmoid_f<IO>(zz.x[i]) + x.x[i] * gelu_grad_f(a.x[i]);
         store8<IO>(gv + e, o);
-    }
-}
-
-__global__ void glu_reduce_kernel(const float* part, int splits, size_t n, float* out) {
-    grid_dep_wait();
-    grid_dep_launch();
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        float acc = 0.f;
-        for (int s = 0; s < splits; ++s) acc += part[(size_t)s * n + e];
-        out[e] = acc;
     }
 }
 
 }  // namespace
 
-void launch_glu_pack(int H, const float* W, void* Wz, void* Wn, float* Wt_f32, WsHeader* hdr, cudaStream_t st) {
+void launch_glu_pre(bool io_bf16, bool planes, size_t n, int H, const void* v, void* x1, const float* W, void* Wz, void* Wn,
+                    float* Wt_f32, WsHeader* hdr, cudaStream_t st) {
     count_launch();
-    const unsigned n = (unsigned)((H + 31) / 32);
-    launch_dep(glu_pack_kernel, dim3(n, n), 256, 0, st, H, W, (__nv_bfloat16*)Wz, (__nv_bfloat16*)Wn, Wt_f32, hdr);
-}
-
-void launch_glu_gelu(bool io_bf16, bool planes, size_t n, int H, const void* v, void* x1, cudaStream_t st) {
-    count_launch();
-    const int b = blocks_for(n / 8);
+    const int tiles = ((H + 31) / 32) * ((H + 31) / 32), b = tiles + blocks_for(n / 8);
+    auto wz = (__nv_bfloat16*)Wz, wn = (__nv_bfloat16*)Wn;
     if (io_bf16 && planes)
-        launch_dep(glu_gelu_kernel<__nv_bfloat16, true>, b, kThreads, 0, st, n, H, (const __nv_bfloat16*)v, x1);
+        launch_dep(glu_pre_kernel<__nv_bfloat16, true>, b, kThreads, 0, st, tiles, n, H, (const __nv_bfloat16*)v, x1, W, wz, wn, Wt_f32, hdr);
     else if (io_bf16)
-        launch_dep(glu_gelu_kernel<__nv_bfloat16, false>, b, kThreads, 0, st, n, H, (const __nv_bfloat16*)v, x1);
+        launch_dep(glu_pre_kernel<__nv_bfloat16, false>, b, kThreads, 0, st, tiles, n, H, (const __nv_bfloat16*)v, x1, W, wz, wn, Wt_f32, hdr);
     else
-        launch_dep(glu_gelu_kernel<float, false>, b, kThreads, 0, st, n, H, (const float*)v, x1);
+        launch_dep(glu_pre_kernel<float, false>, b, kThreads, 0, st, tiles, n, H, (const float*)v, x1, W, wz, wn, Wt_f32, hdr);
 }
 
 void launch_glu_out(bool io_bf16, size_t n, const void* v, const float* z, void* out, cudaStream_t st) {
@@ -225,19 +239,16 @@ void launch_glu_gz(bool io_bf16, bool planes, size_t n, const void* v, const voi
         launch_dep(glu_gz_kernel<float, false>, b, kThreads, 0, st, n, (const float*)v, (const float*)gout, z, gz, n);
 }
 
-void launch_glu_gv(bool io_bf16, size_t n, const void* v, const void* gout, const float* z, const float* gx1, void* gv,
-                   cudaStream_t st) {
+void launch_glu_post(bool io_bf16, const float* part, int splits, size_t n_w, float* dW, size_t n, const void* v, const void* gout,
+                     const float* z, const float* gx1, void* gv, cudaStream_t st) {
     count_launch();
-    const int b = blocks_for(n / 8);
+    const int rb = blocks_for(n_w / 4), b = rb + blocks_for(n / 8);
     if (io_bf16)
-        launch_dep(glu_gv_kernel<__nv_bfloat16>, b, kThreads, 0, st, n, (const __nv_bfloat16*)v, (const __nv_bfloat16*)gout, z, gx1, (__nv_bfloat16*)gv);
+        launch_dep(glu_post_kernel<__nv_bfloat16>, b, kThreads, 0, st, rb, part, splits, n_w, dW, n, (const __nv_bfloat16*)v,
+                   (const __nv_bfloat16*)gout, z, gx1, (__nv_bfloat16*)gv);
     else
-        launch_dep(glu_gv_kernel<float>, b, kThreads, 0, st, n, (const float*)v, (const float*)gout, z, gx1, (float*)gv);
-}
-
-void launch_glu_reduce(const float* part, int splits, size_t n, float* out, cudaStream_t st) {
-    count_launch();
-    launch_dep(glu_reduce_kernel, blocks_for(n), kThreads, 0, st, part, splits, n, out);
+        launch_dep(glu_post_kernel<float>, b, kThreads, 0, st, rb, part, splits, n_w, dW, n, (const float*)v, (const float*)gout, z, gx1,
+                   (float*)gv);
 }
 
 }  // namespace ssm

@@ -255,16 +255,16 @@ void launch_split_planes(const float* in, size_t M, int K, void* out, cudaStream
 // glu.cu: what surrounds the GEMMs of the half-GLU gate out = v * sigmoid(GELU(v) W).
 // Tensor-core path (may be NULL): Wz, Wn [H, 2H], hi | lo planes of W transposed (z = x1 W) and of W (g_x1 = gz W^T);
 // Wt_f32 (CUDA-core path, may be NULL): W transposed.  Clears the header's status word.
-void launch_glu_pack(int H, const float* W, void* Wz, void* Wn, float* Wt_f32, WsHeader* hdr, cudaStream_t st);
-// x1 = GELU(v); planes: bf16 [M, 2H], high halves in columns [0, H), low halves in [H, 2H); else fp32 [M, H]
-void launch_glu_gelu(bool io_bf16, bool planes, size_t n, int H, const void* v, void* x1, cudaStream_t st);
+// x1 = GELU(v) in the same launch; planes: bf16 [M, 2H], high halves in columns [0, H), low halves in [H, 2H); else fp32 [M, H]
+void launch_glu_pre(bool io_bf16, bool planes, size_t n, int H, const void* v, void* x1, const float* W, void* Wz, void* Wn,
+                    float* Wt_f32, WsHeader* hdr, cudaStream_t st);
 void launch_glu_out(bool io_bf16, size_t n, const void* v, const float* z, void* out, cudaStream_t st);
 // gz = gout * v * s (1 - s), s = sigmoid(z); planes: two bf16 planes (hi, lo) n elements apart, else fp32
 void launch_glu_gz(bool io_bf16, bool planes, size_t n, const void* v, const void* gout, const float* z, void* gz,
                    cudaStream_t st);
-void launch_glu_gv(bool io_bf16, size_t n, const void* v, const void* gout, const float* z, const float* gx1, void* gv,
-                   cudaStream_t st);
-void launch_glu_reduce(const float* part, int splits, size_t n, float* out, cudaStream_t st);
+// dW = the sum of `splits` slices of n_w elements, and gv = gout * sigmoid(z) + g_x1 * GELU'(v)
+void launch_glu_post(bool io_bf16, const float* part, int splits, size_t n_w, float* dW, size_t n, const void* v, const void* gout,
+                     const float* z, const float* gx1, void* gv, cudaStream_t st);
 
 // stack.cu: out = LayerNorm(u + GELU(v)) * w + b per row of H features, and its backward
 // (gz = LN'(g), gv = gz * GELU'(v), dw, db).  v, gz, gv are fp32; u, out and g are fp32 or bf16 as
