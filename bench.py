@@ -45,8 +45,7 @@ STAGE_MODEL = {
     "gemm_gx": (lambda H, P, s: 4.0 * H * P, None),
     "scan_bwd": (None, lambda H, P, s: 24.0 * P),
     "gemm_du": (lambda H, P, s: 4.0 * H * P, None),
-    "gemm_gBbar": (lambda H, P, s: 4.0 * H * P, None),
-    "gemm_gC": (lambda H, P, s: 4.0 * H * P, None),
+    "gemm_gBbar_gC": (lambda H, P, s: 8.0 * H * P, None),      # both weight gradients
 }
 
 
@@ -60,8 +59,7 @@ NCU_TRAFFIC_PER_TIMESTEP = {
     "gemm_gx_scan_bwd": 644.7e6 / 131072,
     "gemm_y": 379.7e6 / 131072,
     "gemm_du": 546.9e6 / 131072,
-    "gemm_gBbar": 406.5e6 / 131072,
-    "gemm_gC": 406.6e6 / 131072,
+    "gemm_gBbar_gC": 813.1e6 / 131072,
     "scan_fwd": None,
     "scan_bwd": None,
     "gemm_Bu": None,

@@ -12,18 +12,20 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,T,H,P", [(1, 1, 128, 64), (127, 1, 128, 64), (1, 129, 640, 64), (9, 57, 384, 320),
-                                     (3, 43, 1152, 128), (60, 65, 384, 64), (31, 125, 768, 256)])
+                                     (3, 43, 1152, 128), (60, 65, 384, 64), (31, 125, 768, 256),
+                                     (31, 125, 512, 256)])   # CTA pairs, the last with one row tile
 def test_bf16_edges(B, T, H, P):
     run(I.Workload("few", B=B, T=T, H=H, P=P, io_dtype="bf16", p_done=0.02, seed=B + H), with_x0=True, with_gxT=True)
 
 
 @pytest.mark.parametrize("B,T,H,P", [(1, 1, 256, 128), (1, 127, 256, 128), (43, 3, 512, 128), (5, 205, 256, 384),
-                                     (2, 64, 1024, 256), (37, 111, 256, 128)])
+                                     (2, 64, 1024, 256), (37, 111, 256, 128),
+                                     (1, 7, 128, 64), (2, 65, 128, 64), (5, 77, 384, 192), (9, 57, 640, 64)])
 def test_fp32_edges(B, T, H, P):
     run(I.Workload("few32", B=B, T=T, H=H, P=P, io_dtype="f32", p_done=0.02, seed=B + H), with_x0=True, with_gxT=True)
 
 
-@pytest.mark.parametrize("rows,H", [(1, 128), (129, 256), (1000, 384)])
+@pytest.mark.parametrize("rows,H", [(1, 128), (129, 256), (1000, 384), (3875, 512), (3875, 1024)])
 def test_gate_edges_bf16(rows, H):
     run_gate(I.Workload("few_gate", B=1, T=rows, H=H, P=8, io_dtype="bf16", seed=rows + H))
 
@@ -35,7 +37,7 @@ def test_weight_gradients_from_planes_fp32(B, T, H, P):
     run(I.Workload("nt32", B=B, T=T, H=H, P=P, io_dtype="f32", p_done=0.01, seed=B + T), with_gxT=True)
 
 
-@pytest.mark.parametrize("B,T,H,P", [(50, 131, 256, 128), (7, 301, 768, 384), (1, 12801, 256, 128)])
+@pytest.mark.parametrize("B,T,H,P", [(50, 131, 256, 128), (7, 301, 768, 384), (1, 12801, 256, 128), (37, 350, 384, 192)])
 def test_many_tiles_fp32(B, T, H, P):
     """The persistent plane kernel: from 100 tiles on, a ragged last row of tiles, more tiles than CTAs.  y, xT, du and dx0
     elementwise as everywhere; the parameter gradients, whose elements cancel to far below their scale in sums over
