@@ -124,6 +124,17 @@ inline bool launch_dep(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     return launch_dep_cluster(kernel, 1, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
+// The same launch without the overlap: the grid is placed when the kernel before it has ended, one block per SM first.
+template <typename... KArgs, typename... Args>
+inline bool launch_after(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...) == cudaSuccess;
+}
+
 class StageTimer {
   public:
     StageTimer(const char* name, cudaStream_t st);

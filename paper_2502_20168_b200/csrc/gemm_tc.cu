@@ -2101,10 +2101,11 @@ static bool make_plane_map4(CUtensorMap* map, const void* planes, int B, int T, 
 }
 
 // Fewest (sequence, state group) chain pairs for which the kernels that scan in the epilogue of a projection
-// are taken: below it too many CTA pairs would idle while a few walk their chains tile by tile.
-#ifndef SSM_FUSED_MIN_PAIRS
-#define SSM_FUSED_MIN_PAIRS 32   // measured: 32 pairs (16 sequences of 256 states) still beat the separate kernels
-#endif
+// are taken: below it too many CTA pairs would idle while a few walk their chains tile by tile.  us per forward and backward
+// pass, separate / fused, at H, P = 512, 256 unless stated: 30 chains 10 x 16384 (384, 192) 968 / 931; 28: 7 x 1000 120 / 103;
+// 24: 6 x 4096 287 / 271, 12 x 1024 (256, 128) 103 / 86; 20: 5 x 2048 168 / 151, 5 x 16384 826 / 854; 18: 9 x 512 (256, 128)
+// 72 / 63; 16: 2 x 4096 the separate kernels.
+static int fused_min_pairs(int T) { return T <= 4096 ? 18 : 24; }
 #ifndef SSM_FUSED_NARROW_BELOW
 #define SSM_FUSED_NARROW_BELOW 0   // 0: chains of 32 states where chains of 64 would occupy at most half of the CTA pairs
 #endif
@@ -2147,9 +2148,9 @@ static FusedMode fused_mode(int B, int T, int H, int P) {
         // round of chains better when there are only a few rounds (48 sequences at P = 256: 96 chains take two
         // rounds on 74 CTA pairs, 192 half-length chains three half-rounds).
         m = {64, tp_ok && tp_steps < steps};
-    } else if (tp_ok && tp_chains >= SSM_FUSED_MIN_PAIRS) {
+    } else if (tp_ok && tp_chains >= fused_min_pairs(T)) {
         m = {64, true};
-    } else if (pairs64 >= SSM_FUSED_MIN_PAIRS) {
+    } else if (pairs64 >= fused_min_pairs(T)) {
         m = {32, false};
     }
     // A ragged length costs the empty rows of each sequence's last tile (empty = rows of its tiles / T).  us per forward and

@@ -583,6 +583,17 @@ bool set_smem(K kernel, size_t bytes) {
     return set_max_dynamic_smem(reinterpret_cast<const void*>(kernel), bytes);
 }
 
+// Long chains, fewer than SMs, want an SM each: blocks launched beside the end of the kernel before are placed two to an SM on
+// the first SMs that come free.  us per forward and backward pass, with the overlap / without, bf16, H, P = 512, 256: 2 x 4096
+// 214 / 204, 3 x 2000 152 / 141, 3 x 16384 753 / 702.  Short chains (8 tiles, 3 x 1000: 92.7 / 97.2) and very few
+// (1 x 2000 at 256, 128, 8 chains: 102.5 / 105.6) are better off with it.
+template <typename K, typename... A>
+void launch_scan(K kern, const Args& k, size_t smem, cudaStream_t st, A&&... args) {
+    const int grid = k.nchains < kCtasPerSm * sm_count() ? k.nchains : kCtasPerSm * sm_count();
+    if (k.nchains >= 16 && k.nchains <= sm_count() && k.ntiles >= 16) launch_after(kern, grid, kThreads, smem, st, std::forward<A>(args)...);
+    else launch_dep(kern, grid, kThreads, smem, st, std::forward<A>(args)...);
+}
+
 }  // namespace
 }  // namespace stream
 
@@ -598,7 +609,6 @@ int launch_scan_fwd_stream(int B, int T, int P, const float2* Abar, const float2
     using namespace stream;
     const Args k = make_args(B, T, P, kFwdRows, true, Abar, Alo, done, hdr);
     const size_t smem = (size_t)k.stages * k.R * k.G * 8 + 128;
-    const int grid = k.nchains < kCtasPerSm * sm_count() ? k.nchains : kCtasPerSm * sm_count();
     const size_t plane_bytes = (size_t)B * T * P * 4;
     CUtensorMap mi, o0, o1;
     if (!make_map3(&mi, Bu, false, B, T, P, k.G, k.R)) return SSM_ERR_CUDA;
@@ -610,7 +620,7 @@ int launch_scan_fwd_stream(int B, int T, int P, const float2* Abar, const float2
     do {                                                                                \
         auto kern = scan_fwd_stream_kernel<GG, XS, PAIR>;                               \
         if (!set_smem(kern, smem)) return SSM_ERR_CUDA;                                 \
-        launch_dep(kern, grid, kThreads, smem, st, k, mi, o0, o1, x0, xT);                      \
+        launch_scan(kern, k, smem, st, k, mi, o0, o1, x0, xT);                          \
     } while (0)
 #define SSM_LAUNCH(XS, PAIR)                                                            \
     do {                                                                                \
@@ -663,11 +673,11 @@ int launch_scan_bwd_stream(int B, int T, int P, const float2* Abar, const float2
         if (tall) {                                                                                \
             auto kern = scan_bwd_stream_kernel<GG, XS, PAIR, kBwdRowsLong>;                        \
             if (!set_smem(kern, smem)) return SSM_ERR_CUDA;                                        \
-            launch_dep(kern, grid, kThreads, smem, st, k, mg, x0m, x1m, o0, o1, x0, gxT, part, gx0);       \
+            launch_scan(kern, k, smem, st, k, mg, x0m, x1m, o0, o1, x0, gxT, part, gx0);            \
         } else {                                                                                   \
             auto kern = scan_bwd_stream_kernel<GG, XS, PAIR, kBwdRows>;                            \
             if (!set_smem(kern, smem)) return SSM_ERR_CUDA;                                        \
-            launch_dep(kern, grid, kThreads, smem, st, k, mg, x0m, x1m, o0, o1, x0, gxT, part, gx0);       \
+            launch_scan(kern, k, smem, st, k, mg, x0m, x1m, o0, o1, x0, gxT, part, gx0);            \
         }                                                                                          \
     } while (0)
 #define SSM_LAUNCH(XS, PAIR)                                                                       \

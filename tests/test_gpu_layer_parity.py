@@ -100,7 +100,8 @@ def test_fused_projection_and_scan_shapes_bf16(B, T, H, P):
 
 
 @pytest.mark.parametrize("B,T,H,P", [(146, 127, 256, 128), (147, 129, 256, 128), (74, 250, 128, 128), (37, 383, 256, 128), (20, 500, 256, 256),
-                                     (9, 1000, 256, 256), (74, 1137, 128, 64), (36, 120, 256, 128), (16, 257, 256, 512)])
+                                     (9, 1000, 256, 256), (74, 1137, 128, 64), (36, 120, 256, 128), (16, 257, 256, 512),
+                                     (9, 512, 256, 128), (18, 128, 256, 128), (5, 640, 256, 256)])   # (few chains)
 def test_fused_projection_and_scan_ragged_lengths_bf16(B, T, H, P):
     # Sequences that end inside a tile (one row short of it, one row into the next, anywhere): the rows after the end
     # belong to the next sequence and must neither be written nor contribute.  Chains of 64 and of 32 states, and both CTAs
