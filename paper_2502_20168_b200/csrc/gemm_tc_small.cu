@@ -7,6 +7,9 @@
 //  * a tile is 128 rows x 64, 128 or 256 columns, and a cluster of 1, 2 or 4 CTAs shares one tile, each taking a
 //    part of the contraction; the parts are added through distributed shared memory in the order of the ranks, so
 //    results repeat bit for bit and no partial sum goes through memory;
+//  * or two CTAs take a tile of 256 rows together (cta_group::2), each with half of the weight tile in its shared
+//    memory: a third less to bring in per k-block where there are enough rows (4096 x 1024 x 1024, two products of
+//    planes: 17.8 -> 16.1 us back to back);
 //  * a k-block brings every plane of both operands into shared memory once and all products of the schedule are
 //    issued from it (the other kernels load a pair of planes per product: 12 tiles instead of 6);
 //  * an fp32 A operand needs no planes in memory: the warps that later run the epilogue read it, split it into its
@@ -350,7 +353,7 @@ size_t stage_bytes_of(int bn, int planes_a, int planes_w, bool pair) {
     return (size_t)planes_a * kSmATile + (size_t)planes_w * (pair ? bn / 2 : bn) * BK * 2;
 }
 
-// Tile width and cluster size: the pair with the shortest estimated time.  The estimate is a fit, in microseconds, to
+// Tile width and cluster size, or a CTA pair: the choice with the shortest estimated time.  The estimate is a fit, in microseconds, to
 // timings of all pairs on twenty shapes from 16 x 256 x 256 to 4096 x 1024 x 1024, back to back (within 10 % of the
 // measured time, and the pair it picks within 8 % of the fastest): a wave of CTAs takes a fixed part that grows with
 // the tile (start, first loads, epilogue), its k-blocks at 48 bytes of operands per cycle and SM (L2), 0.95 us where
