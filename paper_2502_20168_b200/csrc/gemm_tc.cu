@@ -1994,11 +1994,10 @@ bool tc_tn_supported(int M, int N_out, int K, bool split_w) {
 static int pair_tiles_of(int M, int n_tiles) { return ((M + 2 * tc::BM - 1) / (2 * tc::BM)) * n_tiles; }
 
 // Whether a projection has enough 256 x 256 tiles for the kernel on CTA pairs; the others take gemm_tc_small.cu.
-// us back to back, pairs / few tiles, by number of tiles:
+// us back to back, pairs / few tiles, by number of tiles (products of planes: below):
 //   acc + diag * skip:         24 tiles 9.3 / 9.5, 32: 12.2 / 12.4, 48: 9.7 / 11.6, 64: 12.7 / 14.6
 //   the same with column sums: 32: 11.5 / 10.1, 48: 12.0 / 14.2 (the pair kernel keeps the sums of kDotMaxN columns)
 //   hi + lo weights:           32: 6.6 / 5.9 and 10.4 / 11.9, 48: 7.9 / 8.9, 128: 17.4 / 25.0
-//   two products of planes:    64: 19.8 / 17.8, 94: 20.4 / 23.5, 512: 111 / 133;  with the gate 94: 33.0 / 32.8, 512: 118 / 134
 // Six products of planes, whose planes the few-tile kernel loads once, stay there at every size.
 enum { kEpiStore = 0, kEpiDiag = 1, kEpiGate = 2, kEpiDot = 3 };
 static int epi_of(const GemmTcTN& g) { return g.gate_out ? kEpiGate : (g.store_f32 && !g.diag ? kEpiStore : (g.dot ? kEpiDot : kEpiDiag)); }
@@ -2007,7 +2006,12 @@ static bool use_pairs(const GemmTcTN& g) {
     const int out_cols = g.split_w ? tc::BN / 2 : tc::BN, tiles = pair_tiles_of(g.M, (g.N_out + out_cols - 1) / out_cols);
     const int epi = epi_of(g);
     if (epi == kEpiDot && g.N_out > tc::kDotMaxN) return false;
-    return tiles >= (g.n_products > 0 ? 80 : (epi == kEpiDiag ? 32 : 40));
+    // Products of planes, which the few-tile kernel (CTA pairs there too) loads once: us of the gate's forward / backward call,
+    // few tiles / pairs, rows x H: 6400 x 1024 (100 tiles) 64.7 / 69.4 and 104.3 / 105.7, 12800 x 1024 102.6 / 106.0 and
+    // 179.6 / 181.0, 32768 x 1024 232.0 / 235.5 and 451.1 / 454.6; 16384 x 512 (128 tiles) 58.7 / 60.8 and 99.7 / 94.4,
+    // 32768 x 512 105.1 / 100.9 and 185.4 / 179.9, 262144 x 512 736.6 / 697.2 and 1395 / 1300.
+    if (g.n_products > 0) return tiles >= (g.K >= 1024 ? 600 : (epi == kEpiGate ? 160 : 80));
+    return tiles >= (epi == kEpiDiag ? 32 : 40);
 }
 // Whether acc + diag * skip also leaves the column sums of skip * dot: not for many rows of very wide outputs, which the
 // pair kernel takes faster without than the few-tile kernel with them.
