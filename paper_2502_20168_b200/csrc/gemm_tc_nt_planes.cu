@@ -219,11 +219,22 @@ gemm_tc_nt_planes_kernel(const __grid_constant__ NtPlanesMaps<kN> maps, const __
 // 1024 rows, 512 x 512, 16 k-blocks per slice: 338.5 and 335.0).
 static bool nt_planes_pairs(int I, int blocks_per_slice) { return blocks_per_slice >= 4 && (I % 256 == 0 || I >= 640); }
 
-// Slices of the rows: as many as leave every SM at most one CTA of the launch (pairs: all but the few SMs that
-// clusters of two cannot use).
+// Slices of the rows: the shortest estimated time, rounds of CTAs (pairs: on all but the few SMs that clusters of two cannot
+// use) times the k-blocks of a slice and what a CTA costs besides, about six k-blocks.  Up to 4096 rows that is one round;
+// with 16 pair tiles of 64000 rows 4 slices would leave 8 of 72 pairs without work, 9 take two full rounds: a pass
+// of the 64 x 1000 layer (512, 256) 1408 / 1395 us.
 int tc_nt_planes_splits(int K, int I, int J, int n_products) {
     const int blocks = (K + tc::BK - 1) / tc::BK, most = std::min(blocks, 64);
-    auto slices = [&](int i_tiles, int slots) { return std::max(1, std::min(most, slots / std::max(n_products * i_tiles * (J / 128), 1))); };
+    auto slices = [&](int i_tiles, int slots) {
+        const int units = std::max(n_products * i_tiles * (J / 128), 1);
+        int best = 1;
+        long best_t = 0;
+        for (int s = 1; s <= most && (s == 1 || (long)units * s <= 3L * slots); ++s) {
+            const long t = (long)((units * s + slots - 1) / slots) * ((blocks + s - 1) / s + 6);
+            if (s == 1 || t < best_t) best = s, best_t = t;
+        }
+        return best;
+    };
     const int single = slices(I / 128, device_sm_count());
     return nt_planes_pairs(I, blocks / single) ? slices((I + 255) / 256, (device_sm_count() - 4) / 2) : single;
 }
