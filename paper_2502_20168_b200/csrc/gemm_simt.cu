@@ -9,6 +9,7 @@ namespace ssm {
 
 constexpr int TM = 64, TN = 64, TK = 16;
 constexpr int kGemmThreads = 256;
+constexpr long long kMaxGridZ = 65535;
 
 template <typename T>
 __device__ __forceinline__ void load4(const T* p, float (&v)[4]);
@@ -153,7 +154,8 @@ struct NtSimtArgs {
     const void *dot_a, *dot_b;
     bool dot_a_bf16, dot_b_bf16;
     float* dot_part;
-    int dot_groups, dot_blocks;   // row groups; blocks the dot products take
+    int dot_groups;               // row groups
+    long long dot_blocks;         // row groups x 128-column blocks: the blocks behind the products take them in turn
 };
 
 __device__ __forceinline__ void load4_any(const void* p, bool bf16, size_t i, float (&v)[4]) {
@@ -167,36 +169,39 @@ gemm_nt_kernel(const __grid_constant__ NtSimtArgs q) {
     __shared__ __align__(16) float As[TK][TM + 4];
     __shared__ __align__(16) float Bs[TK][TN + 4];
     const int z = (int)blockIdx.z / q.g[0].splits;
-    if (z >= q.n) {   // dot products: block = 32 column quads x 8 row lanes, kDotRows rows
-        const int extra = (int)blockIdx.z - q.n * q.g[0].splits;
-        const int blk = (extra * (int)gridDim.y + (int)blockIdx.y) * (int)gridDim.x + (int)blockIdx.x;
-        grid_dep_launch();
-        if (blk >= q.dot_blocks) return;
-        const int C = q.g[0].I, M = q.g[0].K, grp = blk % q.dot_groups, c = (blk / q.dot_groups * 32 + (threadIdx.x & 31)) * 4;
-        const int rl = threadIdx.x >> 5, r0 = grp * kDotRows, r1 = min(M, r0 + kDotRows);
+    if (z >= q.n) {   // dot products: block = 32 column quads x 8 row lanes, kDotRows rows at a time
+        const int per_z = (int)(gridDim.x * gridDim.y), first_z = q.n * q.g[0].splits;
+        const int C = q.g[0].I, M = q.g[0].K, rl = threadIdx.x >> 5;
         float4(*sm)[32] = reinterpret_cast<float4(*)[32]>(&As[0][0]);   // 8 x 32 float4 = 4 KB
         static_assert(sizeof(As) >= 8 * 32 * sizeof(float4), "the dot products' sums fit the operand tile");
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        if (c < C) {
+        grid_dep_launch();
+        for (long long blk = (long long)((int)blockIdx.z - first_z) * per_z + (int)(blockIdx.y * gridDim.x + blockIdx.x); blk < q.dot_blocks;
+             blk += (long long)((int)gridDim.z - first_z) * per_z) {
+            const int grp = (int)(blk % q.dot_groups), c = (int)(blk / q.dot_groups * 32 + (threadIdx.x & 31)) * 4;
+            const int r0 = grp * kDotRows, r1 = min(M, r0 + kDotRows);
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+            if (c < C) {
 #pragma unroll 4
-            for (int r = r0 + rl; r < r1; r += 8) {
-                float va[4], vb[4];
-                load4_any(q.dot_a, q.dot_a_bf16, (size_t)r * C + c, va);
-                load4_any(q.dot_b, q.dot_b_bf16, (size_t)r * C + c, vb);
+                for (int r = r0 + rl; r < r1; r += 8) {
+                    float va[4], vb[4];
+                    load4_any(q.dot_a, q.dot_a_bf16, (size_t)r * C + c, va);
+                    load4_any(q.dot_b, q.dot_b_bf16, (size_t)r * C + c, vb);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[i] = fmaf(va[i], vb[i], acc[i]);
+                    for (int i = 0; i < 4; ++i) acc[i] = fmaf(va[i], vb[i], acc[i]);
+                }
             }
-        }
-        sm[rl][threadIdx.x & 31] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-        __syncthreads();
-        if (rl == 0 && c < C) {
-            float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+            __syncthreads();   // the sums of the group before have been read
+            sm[rl][threadIdx.x & 31] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+            __syncthreads();
+            if (rl == 0 && c < C) {
+                float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float4 v = sm[i][threadIdx.x];
-                t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+                for (int i = 0; i < 8; ++i) {
+                    const float4 v = sm[i][threadIdx.x];
+                    t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+                }
+                *reinterpret_cast<float4*>(q.dot_part + (size_t)grp * C + c) = t;
             }
-            *reinterpret_cast<float4*>(q.dot_part + (size_t)grp * C + c) = t;
         }
         return;
     }
@@ -265,9 +270,10 @@ void launch_gemm_nt(const GemmNT* g, int n, const SimtDot* dot, cudaStream_t st)
     if (dot) {
         q.dot_a = dot->a, q.dot_b = dot->b, q.dot_a_bf16 = dot->a_bf16, q.dot_b_bf16 = dot->b_bf16, q.dot_part = dot->part;
         q.dot_groups = dot_groups(g->K);
-        q.dot_blocks = q.dot_groups * ((g->I + 127) / 128);
-        const int per_z = (int)(grid.x * grid.y);
-        grid.z += (q.dot_blocks + per_z - 1) / per_z;
+        q.dot_blocks = (long long)q.dot_groups * ((g->I + 127) / 128);
+        // (a grid has at most 65535 blocks along z: from 8.4 million rows of one output tile on a block takes several groups)
+        const long long per_z = (long long)grid.x * grid.y;
+        grid.z += (unsigned)std::min<long long>((q.dot_blocks + per_z - 1) / per_z, kMaxGridZ - grid.z);
     }
     count_launch();
     launch_dep(gemm_nt_kernel, grid, kGemmThreads, 0, st, q);
