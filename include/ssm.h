@@ -180,7 +180,8 @@ int ssm_layer_bwd(const ssm_shape* shape, const ssm_c64* Lambda, const float* De
  *   y[b,h]      = Re sum_p C[h,p] x_next[b,p] + D[h] u[b,h]
  * ssm_step_prepare discretises the parameters and packs the projection operands into ws
  * once (again after every parameter update); ssm_step then runs the step from that
- * workspace and may be called any number of times.  shape->T is ignored (taken as 1);
+ * workspace and may be called any number of times, with the B it was prepared for or another
+ * one that the workspace is large enough for.  shape->T is ignored (taken as 1);
  * u, y are [B,H] in io_dtype; done is [B] or NULL; x_next may alias x_prev.  The state
  * entering the first step is the xT of ssm_layer_fwd over the context, or zero. */
 size_t ssm_step_workspace_bytes(const ssm_shape* shape);

@@ -28,10 +28,12 @@ struct LayerPlan {
 // fp32 layers of tile-sized widths.  us per forward and backward pass, CUDA cores / planes, at H, P = 384, 192: 50 rows
 // 106 / 61, 1024 rows 132 / 74, 40000 rows 2355 / 523; at 128, 64: 8 rows 49 / 53, 64 rows 52 / 53, 1024 rows 58 / 57, 30000
 // rows 274 / 174.  Errors against the oracle are equal or smaller.
-bool planes_supported(const ssm_shape& s) {
+// Single steps take them at every batch size: the operands prepared for one are read at any other (us per step in a graph, fp32
+// weights on the CUDA cores / planes, 8 trajectories: 384, 192 39.4 / 7.1; 128, 64 15.1 / 3.5).
+bool planes_supported(const ssm_shape& s, bool step) {
     const double work = (double)s.B * s.T * s.H * 2 * s.P;
     return s.H % 128 == 0 && s.P % 64 == 0 && s.H <= tc_max_n() && 2 * s.P <= tc_max_n() &&
-           (work >= (1 << 21) || (s.H % 256 == 0 && s.P % 128 == 0));
+           (step || work >= (1 << 21) || (s.H % 256 == 0 && s.P % 128 == 0));
 }
 // Product schedules (plane of the first operand, plane of the second, four bits each, smallest terms first):
 // fp32 x fp32 = lo hi, hi lo, mid mid, mid hi, hi mid, hi hi;  bf16 x fp32 = hi lo, hi mid, hi hi.
@@ -46,14 +48,15 @@ size_t take(size_t& off, size_t bytes) {
     return at;
 }
 
-LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true) {
+// step: the workspace of single-step mode (T = 1), whose path and layout up to the packed operands go by the widths alone.
+LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true, bool step = false) {
     LayerPlan p{};
     size_t off = 0;
     const size_t BT = (size_t)s.B * s.T, PH = (size_t)s.P * s.H;
     const int P2 = 2 * s.P;
     p.tc = allow_tc && s.io_dtype == SSM_BF16 && tc_tn_supported((int)BT, P2, s.H, true) &&
            tc_tn_supported((int)BT, s.H, P2, false) && tc_nt_supported(s.H, P2);
-    p.planes = !p.tc && s.io_dtype == SSM_F32 && planes_supported(s);
+    p.planes = !p.tc && s.io_dtype == SSM_F32 && planes_supported(s, step);
     p.splits = p.tc ? tc_nt_splits((int)BT, s.H, P2) : (p.planes ? tc_nt_planes_splits((int)BT, s.H, P2, 2) : gemm_nt_splits((int)BT, s.H, P2));
     p.hdr = take(off, sizeof(WsHeader));
     p.Abar = take(off, (size_t)s.P * 8);
@@ -384,7 +387,7 @@ static ssm_shape step_shape(const ssm_shape& s) {
 
 SSM_API size_t ssm_step_workspace_bytes(const ssm_shape* shape) {
     if (check_shape(shape) != SSM_OK) return 0;
-    return plan_layer(step_shape(*shape)).total;
+    return plan_layer(step_shape(*shape), true, true).total;
 }
 
 SSM_API int ssm_step_prepare(const ssm_shape* shape, const ssm_c64* Lambda, const float* Delta, const ssm_c64* Bc,
@@ -393,7 +396,7 @@ SSM_API int ssm_step_prepare(const ssm_shape* shape, const ssm_c64* Lambda, cons
     if (!Lambda || !Delta || !Bc || !Cc) return SSM_ERR_NULL;
     if (misaligned(Lambda) || misaligned(Delta) || misaligned(Bc) || misaligned(Cc)) return SSM_ERR_ALIGN;
     const ssm_shape s = step_shape(*shape);
-    const LayerPlan p = plan_layer(s);
+    const LayerPlan p = plan_layer(s, true, true);
     if (int rc = check_ws(ws, ws_bytes, p.total)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     layer_prepare(s, p, Lambda, Delta, Bc, Cc, ws, at<WsHeader>(ws, p.hdr), st);
@@ -408,7 +411,7 @@ SSM_API int ssm_step(const ssm_shape* shape, const float* D, const void* u, cons
     if (misaligned(D) || misaligned(u) || misaligned(x_prev) || misaligned(x_next) || misaligned(y))
         return SSM_ERR_ALIGN;
     const ssm_shape s = step_shape(*shape);
-    const LayerPlan p = plan_layer(s);
+    const LayerPlan p = plan_layer(s, true, true);
     if (int rc = check_ws(ws, ws_bytes, p.total)) return rc;
     // each (trajectory, state) is read as x0 and written as xT by the same thread, so x_next may be x_prev
     const bool few = use_step_small(s.B, s.H, s.P);

@@ -87,6 +87,30 @@ def test_steps_agree_with_the_parallel_form():
     assert_close("final state", harness.to_np(x), full["xT"], 1e-5)
 
 
+@pytest.mark.parametrize("io,H,P", [("f32", 384, 192), ("f32", 128, 64), ("f32", 256, 128), ("f32", 72, 40), ("bf16", 384, 192)])
+def test_workspace_prepared_for_one_batch_size_serves_others(io, H, P):
+    """Operands prepared for 300 trajectories, then steps of 1, 14, 15, 64, 128 and 300 of them."""
+    import torch
+    from paper_2502_20168_b200 import binding as sb, harness
+    w = I.Workload("step_b", B=300, T=1, H=H, P=P, io_dtype=io, p_done=0.1, seed=H)
+    d = I.draw_layer(w, with_x0=True)
+    dev = {k: harness.to_dev(d[k].astype(np.complex64)) for k in ("Lambda", "Bc", "Cc")}
+    dev["Delta"], dev["D"] = (harness.to_dev(d[k].astype(np.float32)) for k in ("Delta", "D"))
+    dtype = torch.bfloat16 if io == "bf16" else torch.float32
+    shape = sb.make_shape(w.B, 1, H, P, io)
+    ws = sb.alloc_workspace(sb.ssm_step_workspace_bytes(shape))
+    sb.ssm_step_prepare(shape, dev["Lambda"], dev["Delta"], dev["Bc"], dev["Cc"], ws)
+    for B in (1, 14, 15, 64, 128, 300):
+        u, done = harness.to_dev(d["u"][:B, 0], dtype), harness.to_dev(d["done"][:B, 0], torch.uint8)
+        x = harness.to_dev(d["x0"][:B].astype(np.complex64))
+        y = torch.empty((B, H), dtype=dtype, device="cuda")
+        sb.ssm_step(sb.make_shape(B, 1, H, P, io), dev["D"], u, done, x, x, y, ws)
+        sb.ssm_check(ws)
+        ref_x, ref_y = O.ssm_step(d["Lambda"], d["Delta"], d["Bc"], d["Cc"], d["D"], d["u"][:B, 0], d["done"][:B, 0], d["x0"][:B])
+        assert_close(f"y of {B}", harness.to_np(y), ref_y, TOL[io])
+        assert_close(f"x of {B}", harness.to_np(x), ref_x, TOL[io])
+
+
 def test_step_argument_errors():
     import torch
     from paper_2502_20168_b200 import binding as sb
