@@ -695,6 +695,9 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     constexpr int kStageB = Cfg::kStageBytes;
     auto epi_sync = [] { epi_sync_n<Cfg::kEpiThreads>(); };
     extern __shared__ uint8_t smem_raw[];
+    // A wait of an epilogue warp gave up: written before their barrier and read after it, so that all of them leave or none
+    // (the load and MMA warps may raise s.abort_flag between two reads).
+    __shared__ int epi_abort;
     __shared__ float4 agg_e[kFsEpiThreads], carry_s[kPairs];   // (re, re, im, im) of two neighbouring states
     __shared__ uint32_t masks[4];
     __shared__ float4 carry_ring[2][kTPair ? kPairs : 1];   // kTPair: the state handed over by the peer CTA, two slots in turn
@@ -713,7 +716,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             mbar_init(s.tmem_empty(i), 2 * kFsEpiThreads);
             mbar_init(smem_u32(&carry_bar[i]), kPairs);
         }
-        *s.abort_flag = 0;
+        *s.abort_flag = epi_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -803,6 +806,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             }
         }
     } else {
+        volatile int* epi_flag = &epi_abort;
         const uint32_t leader_empty0 = map_to_cta(s.tmem_empty(0), 0);
         constexpr int R = kFsRows, nsl = BM / kFsRows;   // rows per thread; groups of rows
         const int te = threadIdx.x - 64;            // 0 .. kFsEpiThreads - 1
@@ -889,11 +893,11 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     if (lane == 0) masks[te >> 5] = mk;
                 }
                 flag_next = tb + 1 < p.tblocks ? flag_of(chain, tb + 1) : flag_of(chain + npairs, 0);
-                (void)mbar_wait(s.tmem_full(acc), acc_phase, s.abort_flag);
+                (void)mbar_wait(s.tmem_full(acc), acc_phase, epi_flag);
                 if (group_leader()) tma_store_wait_read();   // this row group's results of the previous tile have left shared memory
                 epi_sync();   // flags visible, tile free (nobody reads the previous one any more); also:
                               // the 256 threads leave together or not at all
-                if (*s.abort_flag) {
+                if (*epi_flag) {
                     ok = false;
                     break;
                 }
@@ -1003,7 +1007,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                         tile = ((gflags >> (nsl - 1)) & 1u) ? e : cstep2(pr, pi, npi, tile, e);
                     }
                     if (!first) {
-                        (void)mbar_wait_acquire_cluster(smem_u32(&carry_bar[n_recv & 1u]), (n_recv >> 1) & 1u, s.abort_flag);
+                        (void)mbar_wait_acquire_cluster(smem_u32(&carry_bar[n_recv & 1u]), (n_recv >> 1) & 1u, epi_flag);
                         const float4 c = carry_ring[n_recv & 1u][sp];
                         cin.re = pack2(c.x, c.y);
                         cin.im = pack2(c.z, c.w);
@@ -1119,7 +1123,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     cluster_sync_all();
     tc_fence_after();
     if (warp == 1) tmem_dealloc_pair(tmem_base, kTmemCols);
-    if (threadIdx.x == 0 && *s.abort_flag && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
+    if (threadIdx.x == 0 && (*s.abort_flag || *static_cast<volatile int*>(&epi_abort)) && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1166,6 +1170,9 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     constexpr int kStageB = Cfg::kStageBytes;
     auto epi_sync = [] { epi_sync_n<Cfg::kEpiThreads>(); };
     extern __shared__ uint8_t smem_raw[];
+    // A wait of an epilogue warp gave up: written before their barrier and read after it, so that all of them leave or none
+    // (the load and MMA warps may raise s.abort_flag between two reads).
+    __shared__ int epi_abort;
     __shared__ float4 agg_e[kFsEpiThreads], carry_s[kPairs];   // (re, re, im, im) of two neighbouring states
     __shared__ uint32_t masks[8];   // [0, 4): flags of the rows one later (the resets of the reverse scan); [4, 8): of the rows
     __shared__ __align__(8) uint64_t xbar[BM / kFsRows];   // one per row group: its rows of x have arrived
@@ -1186,7 +1193,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             mbar_init(smem_u32(&carry_bar[i]), kPairs);
         }
         for (int i = 0; i < BM / kFsRows; ++i) mbar_init(smem_u32(&xbar[i]), 1);
-        *s.abort_flag = 0;
+        *s.abort_flag = epi_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -1274,6 +1281,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             }
         }
     } else {
+        volatile int* epi_flag = &epi_abort;
         const uint32_t leader_empty0 = map_to_cta(s.tmem_empty(0), 0);
         constexpr int R = kFsRows, nsl = BM / kFsRows;   // rows per thread; groups of rows
         const int te = threadIdx.x - 64;            // 0 .. kFsEpiThreads - 1
@@ -1365,7 +1373,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     }
                 }
                 flags_next = tb > 0 ? flags_of(chain, tb - 1) : flags_of(chain + npairs, p.tblocks - 1);
-                (void)mbar_wait(s.tmem_full(acc), acc_phase, s.abort_flag);
+                (void)mbar_wait(s.tmem_full(acc), acc_phase, epi_flag);
                 tc_fence_after();
                 // (1) accumulators -> shared-memory tile: 16-byte chunk j of a 128-byte group sits at j ^ (row & 7).
                 // A warp drains two groups of 32 columns (hi + lo halves each): the first group's loads are in
@@ -1380,7 +1388,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 epi_sync();   // flags visible, tile free (nobody reads the previous one any more); also:
                               // the 256 threads leave together or not at all
                 tmem_ld_wait();
-                if (*s.abort_flag) {
+                if (*epi_flag) {
                     ok = false;
                     break;
                 }
@@ -1510,7 +1518,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                         tile = (gflags & 1u) ? e : cstep2(pr, pi, npi, tile, e);
                     }
                     if (!first) {
-                        (void)mbar_wait_acquire_cluster(smem_u32(&carry_bar[n_recv & 1u]), (n_recv >> 1) & 1u, s.abort_flag);
+                        (void)mbar_wait_acquire_cluster(smem_u32(&carry_bar[n_recv & 1u]), (n_recv >> 1) & 1u, epi_flag);
                         const float4 c = carry_ring[n_recv & 1u][sp];
                         cin.re = pack2(c.x, c.y);
                         cin.im = pack2(c.z, c.w);
@@ -1552,7 +1560,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     }
                 }
                 // (3) fold again, with x_{t-1} at hand: sums for gAbar, s as hi / lo bf16 halves in place of x
-                if (!mbar_wait(xb, xphase, s.abort_flag)) {
+                if (!mbar_wait(xb, xphase, epi_flag)) {
                     // (the wait gave up: the flag is set, everybody leaves at the next barrier)
                 }
                 xphase ^= 1u;
@@ -1662,7 +1670,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     cluster_sync_all();
     tc_fence_after();
     if (warp == 1) tmem_dealloc_pair(tmem_base, kTmemCols);
-    if (threadIdx.x == 0 && *s.abort_flag && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
+    if (threadIdx.x == 0 && (*s.abort_flag || *static_cast<volatile int*>(&epi_abort)) && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
 }
 
 // ---------------------------------------------------------------------------------------------

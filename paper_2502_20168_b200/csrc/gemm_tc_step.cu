@@ -58,7 +58,8 @@ template <> struct StepProducts<false, 1> {
 struct StepBars {
     uint64_t full[kStMaxStages], empty[kStMaxStages], done, free;
     uint32_t tmem;
-    int abort_flag;
+    int abort_flag;   // a wait of the load or MMA warp gave up
+    int epi_abort;    // a wait of an epilogue warp did: written before their barrier, read after it, so that they agree
 };
 
 struct Ring {   // position in the ring of operand stages
@@ -100,7 +101,7 @@ step_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUt
         }
         mbar_init(smem_u32(&bars.done), 1);
         mbar_init(smem_u32(&bars.free), kStEpiWarps);
-        bars.abort_flag = 0;
+        bars.abort_flag = bars.epi_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         prefetch_tmap(&tmWb);
@@ -233,11 +234,12 @@ step_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUt
         Ring r;
         uint32_t done_phase = 0;
         SplitA<kStEpiThreads> sp;
+        volatile int* epi_abort = &bars.epi_abort;
         auto epi_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kStEpiThreads) : "memory"); };
         auto feed = [&](const float* a, int K, int kbs) {   // fp32: this tile's A operand
             sp.fetch(a, K, p.M, m0, 0, te);
             for (int kb = 0; kb < kbs; ++kb, r.next(p.stages)) {
-                if (!mbar_wait(smem_u32(&bars.empty[r.stage]), r.phase ^ 1u, abort_flag)) break;
+                if (!mbar_wait_warp(smem_u32(&bars.empty[r.stage]), r.phase ^ 1u, epi_abort)) break;
                 sp.store(tiles + (size_t)r.stage * p.stage_bytes, p.M, m0, te);
                 if (kb + 1 < kbs) sp.fetch(a, K, p.M, m0, kb + 1, te);
                 fence_async_smem();
@@ -246,7 +248,7 @@ step_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUt
             }
         };
         auto drain = [&](bool two) {   // accumulators -> staging rows; false when aborting
-            const bool ok = mbar_wait(smem_u32(&bars.done), done_phase, abort_flag);
+            const bool ok = mbar_wait_warp(smem_u32(&bars.done), done_phase, epi_abort);
             done_phase ^= 1u;
             tc_fence_after();
             const int q = warp & 3, grp = (warp - 2) >> 2;
@@ -273,7 +275,7 @@ step_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUt
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&bars.free));
             epi_sync();
-            return !*abort_flag;
+            return !*epi_abort;
         };
         const float* own = reinterpret_cast<const float*>(staging) + 4 * c4;
 
@@ -368,7 +370,7 @@ step_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUt
     __syncthreads();
     tc_fence_after();
     if (warp == 1) tmem_dealloc(tmem_base, kTmem);
-    if (threadIdx.x == 0 && *abort_flag && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
+    if (threadIdx.x == 0 && (*abort_flag || *reinterpret_cast<volatile int*>(&bars.epi_abort)) && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
 }
 
 // ---------------------------------------------------------------------------------------------
