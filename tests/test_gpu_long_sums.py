@@ -1,0 +1,31 @@
+"""Parameter gradients as sums over many rows: how far the order of the fp32 additions lets them drift from the oracle's."""
+import numpy as np
+import pytest
+
+from paper_2502_20168_b200 import inputs as I
+from tests.util import oracle_layer
+
+pytestmark = pytest.mark.gpu
+
+
+def _off(got, ref):
+    return float(np.linalg.norm(got - ref) / np.linalg.norm(ref))
+
+
+def test_gate_weights_fp32_over_12800_rows():
+    # 256 output tiles, which fill the GPU with a single slice: elementwise within the suite's bound, as with few rows
+    from tests.test_gpu_half_glu import _run
+    _run(I.Workload("glu_rows", B=1, T=12800, H=1024, P=8, io_dtype="f32", seed=3))
+
+
+def test_layer_weights_fp32_off_the_tile_widths():
+    """A chain of L additions of terms of random sign carries a relative rounding error of about sqrt(L / 6) 2^-24 (each
+    addition rounds by 2^-24 / sqrt(3) of a partial sum that grows with the root of the terms).  Chains of at most 512 rows:
+    5.5e-7; bound: twice that.  (One chain over all 8000 rows: 2.2e-6.)"""
+    from paper_2502_20168_b200 import harness
+    w = I.Workload("wide_odd", B=8, T=1000, H=1032, P=520, io_dtype="f32", p_done=0.002, seed=7)
+    d = I.draw_layer(w)
+    res = harness.run_layer(d, "f32")
+    ref = oracle_layer(d)
+    assert _off(res["dB"], ref["dB"]) <= 1.1e-6
+    assert _off(res["dC"], ref["dC"]) <= 1.1e-6
