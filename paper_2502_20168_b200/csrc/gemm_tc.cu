@@ -72,6 +72,10 @@ struct Smem {
     __device__ __forceinline__ uint32_t skip_full(int i) const { return skip_full0 + 8u * (uint32_t)i; }
     uint32_t tmem_slot;   // where tcgen05.alloc writes the base address
     volatile int* abort_flag;
+    // Kernels whose epilogue warps meet at barriers: a wait of one of those warps gave up.  Written before their barrier and
+    // read after it, so that all of them leave or none (the load and MMA warps may raise abort_flag between two reads).
+    // It takes the first skip slot, which these kernels do not use, so that one base address serves both flags.
+    __device__ __forceinline__ volatile int* epi_abort() const { return abort_flag + 1; }
     volatile uint32_t* tmem_slot_ptr;
 };
 
@@ -695,9 +699,6 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     constexpr int kStageB = Cfg::kStageBytes;
     auto epi_sync = [] { epi_sync_n<Cfg::kEpiThreads>(); };
     extern __shared__ uint8_t smem_raw[];
-    // A wait of an epilogue warp gave up: written before their barrier and read after it, so that all of them leave or none
-    // (the load and MMA warps may raise s.abort_flag between two reads).
-    __shared__ int epi_abort;
     __shared__ float4 agg_e[kFsEpiThreads], carry_s[kPairs];   // (re, re, im, im) of two neighbouring states
     __shared__ uint32_t masks[4];
     __shared__ float4 carry_ring[2][kTPair ? kPairs : 1];   // kTPair: the state handed over by the peer CTA, two slots in turn
@@ -716,7 +717,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             mbar_init(s.tmem_empty(i), 2 * kFsEpiThreads);
             mbar_init(smem_u32(&carry_bar[i]), kPairs);
         }
-        *s.abort_flag = epi_abort = 0;
+        *s.abort_flag = *s.epi_abort() = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -806,7 +807,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             }
         }
     } else {
-        volatile int* epi_flag = &epi_abort;
+        volatile int* epi_flag = s.epi_abort();
         const uint32_t leader_empty0 = map_to_cta(s.tmem_empty(0), 0);
         constexpr int R = kFsRows, nsl = BM / kFsRows;   // rows per thread; groups of rows
         const int te = threadIdx.x - 64;            // 0 .. kFsEpiThreads - 1
@@ -1123,7 +1124,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     cluster_sync_all();
     tc_fence_after();
     if (warp == 1) tmem_dealloc_pair(tmem_base, kTmemCols);
-    if (threadIdx.x == 0 && (*s.abort_flag || *static_cast<volatile int*>(&epi_abort)) && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
+    if (threadIdx.x == 0 && (*s.abort_flag || *s.epi_abort()) && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1170,9 +1171,6 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     constexpr int kStageB = Cfg::kStageBytes;
     auto epi_sync = [] { epi_sync_n<Cfg::kEpiThreads>(); };
     extern __shared__ uint8_t smem_raw[];
-    // A wait of an epilogue warp gave up: written before their barrier and read after it, so that all of them leave or none
-    // (the load and MMA warps may raise s.abort_flag between two reads).
-    __shared__ int epi_abort;
     __shared__ float4 agg_e[kFsEpiThreads], carry_s[kPairs];   // (re, re, im, im) of two neighbouring states
     __shared__ uint32_t masks[8];   // [0, 4): flags of the rows one later (the resets of the reverse scan); [4, 8): of the rows
     __shared__ __align__(8) uint64_t xbar[BM / kFsRows];   // one per row group: its rows of x have arrived
@@ -1193,7 +1191,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             mbar_init(smem_u32(&carry_bar[i]), kPairs);
         }
         for (int i = 0; i < BM / kFsRows; ++i) mbar_init(smem_u32(&xbar[i]), 1);
-        *s.abort_flag = epi_abort = 0;
+        *s.abort_flag = *s.epi_abort() = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -1281,7 +1279,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             }
         }
     } else {
-        volatile int* epi_flag = &epi_abort;
+        volatile int* epi_flag = s.epi_abort();
         const uint32_t leader_empty0 = map_to_cta(s.tmem_empty(0), 0);
         constexpr int R = kFsRows, nsl = BM / kFsRows;   // rows per thread; groups of rows
         const int te = threadIdx.x - 64;            // 0 .. kFsEpiThreads - 1
@@ -1670,7 +1668,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     cluster_sync_all();
     tc_fence_after();
     if (warp == 1) tmem_dealloc_pair(tmem_base, kTmemCols);
-    if (threadIdx.x == 0 && (*s.abort_flag || *static_cast<volatile int*>(&epi_abort)) && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
+    if (threadIdx.x == 0 && (*s.abort_flag || *s.epi_abort()) && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
 }
 
 // ---------------------------------------------------------------------------------------------
