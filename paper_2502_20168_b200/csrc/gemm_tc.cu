@@ -38,7 +38,10 @@ constexpr int kStages = 4;      // shared-memory stages of the NT kernel (and si
 constexpr int kABytes = BM * BK * 2;
 constexpr int kBBytes = BN * BK * 2;
 constexpr int kStageBytes = kABytes + kBBytes;
-constexpr int kThreads = 192;      // NT kernel: producer, MMA, 4 epilogue warps
+// NT kernels: producer, MMA and epilogue warps; slices of several segments (nt_epilogue) take two warps per TMEM lane quarter
+__host__ __device__ constexpr int nt_epi_warps(bool segs) { return segs ? 8 : 4; }
+__host__ __device__ constexpr int nt_threads(bool segs) { return 64 + 32 * nt_epi_warps(segs); }
+__host__ __device__ constexpr int nt_epi_cols(bool segs) { return BN / 2 * 4 / nt_epi_warps(segs); }   // columns of a warp
 constexpr int kTnEpiWarps = 8;     // TN kernel: two epilogue warps per TMEM lane quarter
 constexpr int kTnThreads = 64 + 32 * kTnEpiWarps;
 constexpr int kTmemCols = 512;  // two accumulator buffers of BN columns
@@ -1688,15 +1691,91 @@ struct NtMaps {
     CUtensorMap a[2], hi[2], lo[2];   // per product
 };
 
+// The tensor core truncates its fp32 accumulator at every addition: a chain of n of them is about n 2^-25 2/3 off its sum.
+// So a slice of more than kNtSegment k-blocks (64 additions) is multiplied in segments of that length, alternately into the
+// two halves of tensor memory, and the epilogue warps add a finished segment to their registers while the next one runs
+// (16384 rows x 1024 x 1024 in one chain: dB 1.9e-5 off, in segments 4.8e-6; 323.9 and 322.3 us for the pass).  Shorter
+// slices take the kernels without that (kSegs = false): with its registers the next kernel finds no room on the SM before
+// this one ends (6400 rows at 256, 128: 55.0 / 57.4 us for the pass).
+constexpr int kNtSegment = 16;
+
+// What an epilogue warp does with a slice: adds its segments, both planes of Bm each, and stores its 32 rows x nt_epi_cols
+// columns (dst: this lane's row).  `leader_empty0`: the tmem_empty barriers of the CTA that issues the MMAs, as a cluster
+// address where kPair.
+template <bool kPair, bool kSegs>
+__device__ __forceinline__ void nt_epilogue(const Smem& s, float* dst, bool row_ok, int nkb, int warp, int lane, uint32_t tmem_base,
+                                            uint32_t leader_empty0) {
+    constexpr int kCols = nt_epi_cols(kSegs);
+    const uint32_t t_row = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(((warp - 2) >> 2) * kCols);
+    if (!kSegs) {
+        if (nkb > 0) {
+            if (!mbar_wait_warp(s.tmem_full(0), 0, s.abort_flag)) return;
+            tc_fence_after();
+        }
+#pragma unroll 1
+        for (int c = 0; c < kCols; c += 32) {
+            uint32_t r[32], r2[32];
+            if (nkb > 0) {
+                tmem_ld32(t_row + (uint32_t)c, r);
+                tmem_ld32(t_row + (uint32_t)(BN / 2 + c), r2);
+                tmem_ld_wait();
+            } else {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) r[i] = r2[i] = 0u;
+            }
+            if (row_ok)
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    reinterpret_cast<float4*>(dst + c)[i] =
+                        make_float4(__uint_as_float(r[4 * i]) + __uint_as_float(r2[4 * i]),
+                                    __uint_as_float(r[4 * i + 1]) + __uint_as_float(r2[4 * i + 1]),
+                                    __uint_as_float(r[4 * i + 2]) + __uint_as_float(r2[4 * i + 2]),
+                                    __uint_as_float(r[4 * i + 3]) + __uint_as_float(r2[4 * i + 3]));
+        }
+        return;
+    }
+    float sum[kCols];
+#pragma unroll
+    for (int i = 0; i < kCols; ++i) sum[i] = 0.f;
+    const int segs = (nkb + kNtSegment - 1) / kNtSegment;
+#pragma unroll 1
+    for (int seg = 0; seg < segs; ++seg) {
+        const int buf = seg & 1;
+        if (!mbar_wait_warp(s.tmem_full(buf), (uint32_t)(seg >> 1) & 1u, s.abort_flag)) return;
+        tc_fence_after();
+#pragma unroll
+        for (int c = 0; c < kCols; c += 16) {   // (16 columns at a time: registers)
+            uint32_t r[16], r2[16];
+            tmem_ld16(t_row + (uint32_t)(buf * BN + c), r);
+            tmem_ld16(t_row + (uint32_t)(buf * BN + BN / 2 + c), r2);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) sum[c + i] += __uint_as_float(r[i]) + __uint_as_float(r2[i]);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+            if (kPair) mbar_arrive_cluster(leader_empty0 + 8u * (uint32_t)buf);
+            else mbar_arrive(s.tmem_empty(buf));
+        }
+    }
+    if (row_ok) {
+#pragma unroll
+        for (int i = 0; i < kCols / 4; ++i)
+            reinterpret_cast<float4*>(dst)[i] = make_float4(sum[4 * i], sum[4 * i + 1], sum[4 * i + 2], sum[4 * i + 3]);
+    }
+}
+
 // The 256 accumulator columns are 128 output columns times the two planes (hi, lo) of Bm, added in the epilogue.
-__global__ void __launch_bounds__(kThreads, 1)
+template <bool kSegs>
+__global__ void __launch_bounds__(nt_threads(kSegs), 1)
 gemm_tc_nt_kernel(const __grid_constant__ NtMaps maps, const __grid_constant__ NtParams p) {
     const int z = (int)blockIdx.z + p.first;
     const CUtensorMap &tmA = maps.a[z], &tmBhi = maps.hi[z], &tmBlo = maps.lo[z];
     extern __shared__ uint8_t smem_raw[];
     const Smem s = carve_smem(smem_raw, kStages, 0, 0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t tmem_base = prologue(s, warp, lane, 128);
+    const uint32_t tmem_base = prologue(s, warp, lane, nt_epi_warps(kSegs));
     grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
     grid_dep_launch();
     const int tile = blockIdx.x, split = blockIdx.y;
@@ -1741,6 +1820,11 @@ gemm_tc_nt_kernel(const __grid_constant__ NtMaps maps, const __grid_constant__ N
             uint32_t phase = 0;
             bool ok = true;
             for (int kb = 0; kb < nkb; ++kb) {
+                const int seg = kSegs ? kb / kNtSegment : 0, buf = seg & 1, in_seg = kSegs ? kb % kNtSegment : kb;
+                if (kSegs && in_seg == 0 && seg >= 2) {   // the epilogue has taken segment seg - 2 out of this half of tensor memory
+                    if (!(ok = mbar_wait_warp(s.tmem_empty(buf), (uint32_t)((seg >> 1) - 1) & 1u, s.abort_flag))) break;
+                    tc_fence_after();
+                }
                 if (!(ok = mbar_wait_warp(s.full(stage), phase, s.abort_flag))) break;
                 tc_fence_after();
                 const uint32_t a_addr = smem_u32(s.tiles + (size_t)stage * kStageBytes);
@@ -1750,53 +1834,21 @@ gemm_tc_nt_kernel(const __grid_constant__ NtMaps maps, const __grid_constant__ N
 #pragma unroll
                     for (int k = 0; k < BK / UK; ++k) {
                         // 16 k-rows of 128 bytes further: +2048 bytes = +128 in the address field
-                        umma_bf16(tmem_base, adesc + (uint64_t)(128 * k), bdesc + (uint64_t)(128 * k), idesc,
-                                  (uint32_t)((kb | k) != 0));
+                        umma_bf16(tmem_base + (uint32_t)(buf * BN), adesc + (uint64_t)(128 * k), bdesc + (uint64_t)(128 * k), idesc,
+                                  (uint32_t)((in_seg | k) != 0));
                     }
                     umma_commit(s.empty(stage));
+                    if (kb + 1 == nkb || (kSegs && in_seg + 1 == kNtSegment)) umma_commit(s.tmem_full(buf));
                 }
                 if (++stage == kStages) {
                     stage = 0;
                     phase ^= 1u;
                 }
             }
-            if (ok && elect_one()) umma_commit(s.tmem_full(0));
         }
     } else {
-        const int q = warp & 3;
-        const int row = i0 + q * 32 + lane;
-        float* dst_row = p.part[z] + ((size_t)split * p.I + row) * p.J + j0;
-        bool ok = true;
-        if (nkb > 0) {
-            ok = mbar_wait(s.tmem_full(0), 0, s.abort_flag);
-            tc_fence_after();
-        }
-        if (ok) {
-            const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
-#pragma unroll 1
-            for (int c = 0; c < kOutCols; c += 32) {
-                float v[32];
-                if (nkb > 0) {
-                    uint32_t r[32];
-                    tmem_ld32(t_row + (uint32_t)c, r);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-                    tmem_ld32(t_row + (uint32_t)(kOutCols + c), r);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] += __uint_as_float(r[i]);
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] = 0.f;
-                }
-                if (row < p.I) {
-                    float4* dst = reinterpret_cast<float4*>(dst_row + c);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                }
-            }
-        }
+        const int row = i0 + (warp & 3) * 32 + lane, col = j0 + ((warp - 2) >> 2) * nt_epi_cols(kSegs);
+        nt_epilogue<false, kSegs>(s, p.part[z] + ((size_t)split * p.I + row) * p.J + col, row < p.I, nkb, warp, lane, tmem_base, 0);
     }
     epilogue_exit(s, warp, tmem_base, p.hdr);
 }
@@ -1814,7 +1866,8 @@ constexpr int kNtPairStages = 6;
 constexpr int kNtPairStageBytes = kABytes + kBBytes / 2;   // 32 KB
 constexpr size_t kNtPairSmemBytes = (size_t)kNtPairStages * kNtPairStageBytes + 1024 + 256;
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+template <bool kSegs>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(nt_threads(kSegs), 1)
 gemm_tc_nt_pair_kernel(const __grid_constant__ NtMaps maps, const __grid_constant__ NtParams p) {
     const int z = (int)blockIdx.z + p.first;
     const CUtensorMap &tmA = maps.a[z], &tmBhi = maps.hi[z], &tmBlo = maps.lo[z];
@@ -1830,13 +1883,16 @@ gemm_tc_nt_pair_kernel(const __grid_constant__ NtMaps maps, const __grid_constan
             mbar_init(rfull(i), 1);
             mbar_init(rempty(i), 1);
         }
-        mbar_init(s.tmem_full(0), 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(s.tmem_full(i), 1);
+            mbar_init(s.tmem_empty(i), 2 * nt_epi_warps(kSegs));
+        }
         *s.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncwarp();
-    if (warp == 1) tmem_alloc_pair(s.tmem_slot, BN);
+    if (warp == 1) tmem_alloc_pair(s.tmem_slot, kSegs ? kTmemCols : BN);
     tc_fence_before();
     cluster_sync_all();
     tc_fence_after();
@@ -1884,6 +1940,11 @@ gemm_tc_nt_pair_kernel(const __grid_constant__ NtMaps maps, const __grid_constan
             uint32_t phase = 0;
             bool ok = true;
             for (int kb = 0; kb < nkb; ++kb) {
+                const int seg = kSegs ? kb / kNtSegment : 0, buf = seg & 1, in_seg = kSegs ? kb % kNtSegment : kb;
+                if (kSegs && in_seg == 0 && seg >= 2) {   // both CTAs' epilogues have taken segment seg - 2 out of this half of tensor memory
+                    if (!(ok = mbar_wait_warp(s.tmem_empty(buf), (uint32_t)((seg >> 1) - 1) & 1u, s.abort_flag))) break;
+                    tc_fence_after();
+                }
                 if (!(ok = mbar_wait_warp(rfull(stage), phase, s.abort_flag))) break;
                 tc_fence_after();
                 const uint32_t a_addr = smem_u32(s.tiles + (size_t)stage * kNtPairStageBytes);
@@ -1892,56 +1953,28 @@ gemm_tc_nt_pair_kernel(const __grid_constant__ NtMaps maps, const __grid_constan
                 if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < BK / UK; ++k)
-                        umma_bf16_pair(tmem_base, adesc + (uint64_t)(128 * k), bdesc + (uint64_t)(128 * k), idesc,
-                                       (uint32_t)((kb | k) != 0));
+                        umma_bf16_pair(tmem_base + (uint32_t)(buf * BN), adesc + (uint64_t)(128 * k), bdesc + (uint64_t)(128 * k), idesc,
+                                       (uint32_t)((in_seg | k) != 0));
                     umma_commit_pair(rempty(stage));
+                    if (kb + 1 == nkb || (kSegs && in_seg + 1 == kNtSegment)) umma_commit_pair(s.tmem_full(buf));
                 }
                 if (++stage == kNtPairStages) {
                     stage = 0;
                     phase ^= 1u;
                 }
             }
-            if (ok && elect_one()) umma_commit_pair(s.tmem_full(0));
         }
     } else {
-        const int q = warp & 3;
-        const int row = i0 + q * 32 + lane;
-        float* dst_row = p.part[z] + ((size_t)split * p.I + row) * p.J + j0;
-        bool ok = true;
-        if (nkb > 0) {
-            ok = mbar_wait(s.tmem_full(0), 0, s.abort_flag);
-            tc_fence_after();
-        }
-        if (ok) {
-            const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
-#pragma unroll 1
-            for (int c = 0; c < kOutCols; c += 32) {
-                float v[32];
-                if (nkb > 0) {
-                    uint32_t r[32], r2[32];
-                    tmem_ld32(t_row + (uint32_t)c, r);
-                    tmem_ld32(t_row + (uint32_t)(kOutCols + c), r2);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]) + __uint_as_float(r2[i]);
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] = 0.f;
-                }
-                if (row < p.I) {
-                    float4* dst = reinterpret_cast<float4*>(dst_row + c);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                }
-            }
-        }
+        const int row = i0 + (warp & 3) * 32 + lane, col = j0 + ((warp - 2) >> 2) * nt_epi_cols(kSegs);
+        nt_epilogue<true, kSegs>(s, p.part[z] + ((size_t)split * p.I + row) * p.J + col, row < p.I, nkb, warp, lane, tmem_base,
+                          map_to_cta(s.tmem_empty(0), 0));
     }
     // nobody leaves (or frees tensor memory) while the other CTA may still signal or compute
     tc_fence_before();
     __syncwarp();
     cluster_sync_all();
     tc_fence_after();
-    if (warp == 1) tmem_dealloc_pair(tmem_base, BN);
+    if (warp == 1) tmem_dealloc_pair(tmem_base, kSegs ? kTmemCols : BN);
     if (threadIdx.x == 0 && *s.abort_flag && p.hdr) p.hdr->status = SSM_ERR_TIMEOUT;
 }
 
@@ -2300,14 +2333,15 @@ int launch_gemm_tc_nt2(int K, int I, int J, int splits, const GemmTcNT& g0, cons
     for (; p.first < 2; p.first += plan.together ? 2 : 1) {
         const unsigned nz = plan.together ? 2 : 1;
         count_launch();
+        auto run = [&](auto kern, unsigned ctas, size_t smem, int threads) {
+            return set_smem(kern, smem) && launch_dep(kern, dim3(ctas * j_tiles, splits, nz), threads, smem, st, maps, p);
+        };
+        const unsigned pairs = 2 * (I / (2 * BM)), singles = I / BM;   // 256 x 256 tiles on CTA pairs, or 128 x 256
         bool ok;
-        if (plan.pairs) {   // 256 x 256 tiles on CTA pairs
-            ok = set_smem(gemm_tc_nt_pair_kernel, kNtPairSmemBytes) &&
-                 launch_dep(gemm_tc_nt_pair_kernel, dim3(2 * (I / (2 * BM)) * j_tiles, splits, nz), kThreads, kNtPairSmemBytes, st, maps, p);
-        } else {
-            ok = set_smem(gemm_tc_nt_kernel, kNtSmemBytes) &&
-                 launch_dep(gemm_tc_nt_kernel, dim3((I / BM) * j_tiles, splits, nz), kThreads, kNtSmemBytes, st, maps, p);
-        }
+        if (p.blocks_per_split > kNtSegment)
+            ok = plan.pairs ? run(gemm_tc_nt_pair_kernel<true>, pairs, kNtPairSmemBytes, nt_threads(true)) : run(gemm_tc_nt_kernel<true>, singles, kNtSmemBytes, nt_threads(true));
+        else
+            ok = plan.pairs ? run(gemm_tc_nt_pair_kernel<false>, pairs, kNtPairSmemBytes, nt_threads(false)) : run(gemm_tc_nt_kernel<false>, singles, kNtSmemBytes, nt_threads(false));
         if (!ok) return SSM_ERR_CUDA;
     }
     return SSM_OK;

@@ -29,3 +29,30 @@ def test_layer_weights_fp32_off_the_tile_widths():
     ref = oracle_layer(d)
     assert _off(res["dB"], ref["dB"]) <= 1.1e-6
     assert _off(res["dC"], ref["dC"]) <= 1.1e-6
+
+
+def test_layer_weights_bf16_wide_outputs():
+    """The tensor core truncates its fp32 accumulator at every addition: a chain of n additions whose partial sums grow with
+    the root of their number is about n 2^-25 2/3 off its sum.  16384 rows in two slices of 128 blocks of 64 rows, four
+    additions a block: 1.0e-5; bound: one and a half times that (the states' 16-bit mantissas add less).  One chain: 2.0e-5."""
+    from paper_2502_20168_b200 import harness
+    w = I.Workload("wide16", B=16, T=1024, H=1024, P=512, io_dtype="bf16", p_done=0.002, seed=7)
+    d = I.draw_layer(w)
+    res = harness.run_layer(d, "bf16")
+    ref = oracle_layer(d)
+    assert _off(res["dB"], ref["dB"]) <= 1.5e-5
+    assert _off(res["dC"], ref["dC"]) <= 1.5e-5
+
+
+@pytest.mark.parametrize("B,T,H,P", [(18, 1024, 256, 128), (18, 1088, 256, 128), (18, 2112, 256, 128), (17, 3203, 256, 128),   # CTA pairs
+                                     (8, 1024, 384, 192), (8, 1088, 384, 192), (8, 2112, 384, 192), (7, 3203, 384, 192)])
+def test_segments_of_a_slice_bf16(B, T, H, P):
+    """Slices of 16 blocks of 64 rows (one segment), 17, 33 and about 50, the last one ragged.  The weights and the states
+    carry 16 bits each (2^-17), and so does what the recurrence makes of them; bound: four such errors."""
+    from paper_2502_20168_b200 import harness
+    w = I.Workload("segs", B=B, T=T, H=H, P=P, io_dtype="bf16", p_done=0.01, seed=B + T)
+    d = I.draw_layer(w)
+    res = harness.run_layer(d, "bf16")
+    ref = oracle_layer(d)
+    for k in ("dB", "dC"):
+        assert _off(res[k], ref[k]) <= 4 * 2.0 ** -17, k
