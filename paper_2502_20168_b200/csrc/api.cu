@@ -21,7 +21,7 @@ struct LayerPlan {
     bool tc;
     bool planes;
     int splits;
-    size_t hdr, Abar, Alo, W0, W1, W2, W3, f32buf, xs, gs, gAbar, gg, scan, part, dot, total;
+    size_t hdr, Abar, Alo, Apow, W0, W1, W2, W3, f32buf, xs, gs, gAbar, gg, scan, part, dot, total;
     size_t u3, gy3, x3, s3;   // plane path: planes of u, gy, x, s for the weight gradients
 };
 
@@ -62,6 +62,7 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true, bool step = false
     p.Abar = take(off, (size_t)s.P * 8);
     p.Alo = take(off, (size_t)s.P * 8);
     if (p.tc) {
+        p.Apow = take(off, (size_t)apow_floats(s.P) * 4);
         p.W0 = take(off, 4 * PH * 2);   // hi/lo stacked Bbar operand  [4P, H] bf16
         p.W1 = take(off, 4 * PH * 2);   // hi/lo stacked conj(C) operand [4P, H] bf16
         p.W2 = take(off, 2 * PH * 2);   // Cp [H, 2P] bf16
@@ -228,7 +229,7 @@ SSM_API int ssm_layer_plan_string(const ssm_shape* shape, char* buf, size_t len)
 static PackJob pack_job(const LayerPlan& p, const ssm_c64* Lambda, const float* Delta, const ssm_c64* Bc, const ssm_c64* Cc,
                         void* ws) {
     return {(const float2*)Lambda, Delta, (const float2*)Bc, (const float2*)Cc, at<float2>(ws, p.Abar), at<float2>(ws, p.Alo),
-            at<void>(ws, p.W0), at<void>(ws, p.W1), at<void>(ws, p.W2), at<void>(ws, p.W3)};
+            at<float>(ws, p.Apow), at<void>(ws, p.W0), at<void>(ws, p.W1), at<void>(ws, p.W2), at<void>(ws, p.W3)};
 }
 static void layer_prepare(const ssm_shape& s, const LayerPlan& p, const ssm_c64* Lambda, const float* Delta,
                           const ssm_c64* Bc, const ssm_c64* Cc, void* ws, WsHeader* hdr, cudaStream_t st) {
@@ -283,7 +284,7 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
     if (p.tc && tc_gemm_scan_fwd_supported(s.B, s.T, s.H, s.P)) {
         {   // projection and scan in one kernel: x = scan(u Bbar^T), Bu stays on chip
             StageTimer tm("gemm_Bu_scan_fwd", st);
-            GemmScanFwd g{u, at<void>(ws, p.W0), s.B, s.T, s.H, s.P, at<float2>(ws, p.Abar), done, (const float2*)x0,
+            GemmScanFwd g{u, at<void>(ws, p.W0), s.B, s.T, s.H, s.P, at<float2>(ws, p.Abar), at<float>(ws, p.Apow), done, (const float2*)x0,
                           at<void>(ws, p.xs), (float2*)xT, hdr};
             if ((rc = launch_gemm_scan_fwd(g, st))) return rc;
         }
@@ -591,7 +592,7 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
         if (tc_gemm_scan_bwd_supported(s.B, s.T, s.H, s.P)) {
             // projection and reverse scan in one kernel: s = reverse scan(gy conj(C)), g_x stays on chip
             StageTimer tm("gemm_gx_scan_bwd", st);
-            GemmScanBwd g{gy, at<void>(ws, p.W1), s.B, s.T, s.H, s.P, at<float2>(ws, p.Abar), done, (const float2*)x0,
+            GemmScanBwd g{gy, at<void>(ws, p.W1), s.B, s.T, s.H, s.P, at<float2>(ws, p.Abar), at<float>(ws, p.Apow), done, (const float2*)x0,
                           (const float2*)gxT, at<void>(ws, p.xs), at<void>(ws, p.gs), nullptr, (float2*)dx0, hdr};
             if ((rc = launch_gemm_scan_bwd_part(g, at<char>(ws, p.scan), &gA_part, &gA_rows, st))) return rc;
         } else {

@@ -236,6 +236,20 @@ pack_params_kernel(int H, int P, const __grid_constant__ PackArgs<kN> o) {
             const float2 ah = make_float2((float)z.ar, (float)z.ai);
             q.Abar[p] = ah;
             q.Alo[p] = make_float2((float)(z.ar - (double)ah.x), (float)(z.ai - (double)ah.y));
+            if (kMode == kPackTc && o.group_log2) {
+                double re = z.ar, im = z.ai;
+#pragma unroll
+                for (int n = 2; n <= 128; n *= 2) {
+                    const double r2 = re * re - im * im;
+                    im = 2.0 * re * im;
+                    re = r2;
+                    if (n == 16 || n == 128) {
+                        float* to = q.Apow + (size_t)(n == 16 ? 0 : 2) * P + 4 * (p >> 1) + (p & 1);
+                        to[0] = (float)re;
+                        to[2] = (float)im;
+                    }
+                }
+            }
         }
     }
     if (threadIdx.x == 32 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && o.hdr) o.hdr->status = 0;

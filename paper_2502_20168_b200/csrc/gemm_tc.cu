@@ -623,6 +623,7 @@ struct FsParams {
     int gps;          // row groups per sequence inside a tile: 8, or T / 16
     int nchains;      // n_tiles * ceil(n_units / 2); kTPair: n_tiles * B
     const float2* Abar;
+    const float4* Apow;   // [2][P / 2]: Abar^16 and Abar^128 of two neighbouring states (re, re, im, im)
     const uint8_t* done;
     const float2* x0;
     float2* xT;
@@ -636,6 +637,7 @@ struct FsParams {
 // hi | lo weight halves), a CTA holds 2 kS weight rows, the fp32 tile it scans is 128 rows x 2 kS columns,
 // and kS / 2 scanning threads (two states each) share a group of 16 rows.
 constexpr int kFsRows = 16;                  // rows per scanning thread; 8 row groups per tile
+static_assert(kFsRows == 16 && BM == 128, "the powers of Abar that pack_params_kernel stores");
 template <int kS>
 struct FsCfg {
     static_assert(kS == 64 || kS == 32, "chains of 64 or 32 states");
@@ -683,6 +685,12 @@ struct C2 {
     f32x2 re, im;   // two complex numbers: (re, re), (im, im)
 };
 // a * x + b for two states at once (nai = -Im a)
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
+// 16 bytes from global to shared memory without a register in between; complete after cp_async_wait.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ C2 cstep2(f32x2 ar, f32x2 ai, f32x2 nai, C2 x, C2 b) {
     C2 r;
     r.re = fma2(ar, x.re, fma2(nai, x.im, b.re));
@@ -703,6 +711,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     auto epi_sync = [] { epi_sync_n<Cfg::kEpiThreads>(); };
     extern __shared__ uint8_t smem_raw[];
     __shared__ float4 agg_e[kFsEpiThreads], carry_s[kPairs];   // (re, re, im, im) of two neighbouring states
+    __shared__ __align__(16) float4 pow_s[2][kTPair ? 2 : 1][kPairs];   // powers of Abar: chains alternate between two slots
     __shared__ uint32_t masks[4];
     __shared__ float4 carry_ring[2][kTPair ? kPairs : 1];   // kTPair: the state handed over by the peer CTA, two slots in turn
     __shared__ __align__(8) uint64_t carry_bar[2];           // kTPair: slot i has arrived (one arrival per sending thread)
@@ -840,6 +849,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             return chain < p.nchains ? p.Abar[(chain % p.n_tiles) * kS + 2 * sp + k] : make_float2(0.f, 0.f);
         };
         float2 a0_next = abar_of(pair, 0), a1_next = abar_of(pair, 1);
+        int chain_par = 0;
         for (int chain = pair; chain < p.nchains && ok; chain += npairs) {
             const int n_tile = chain % p.n_tiles, b = seq_of(chain);
             const bool has_seq = b < p.n_units;
@@ -851,30 +861,14 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             a0_next = abar_of(chain + npairs, 0);
             a1_next = abar_of(chain + npairs, 1);
             const f32x2 ar = pack2(a0.x, a1.x), ai = pack2(a0.y, a1.y), nai = pack2(-a0.y, -a1.y);
-            f32x2 pr, pi, npi;   // Abar^R by squaring in fp32 (a few 1e-7 relative: the results leave as bf16 pairs)
-            f32x2 tr = 0ull, ti = 0ull, nti = 0ull;
-            {
-                float re0 = a0.x, im0 = a0.y, re1 = a1.x, im1 = a1.y;
-#pragma unroll
-                for (int n = 1; n < R; n *= 2) {
-                    const float r0 = fmaf(re0, re0, -im0 * im0), i0 = 2.f * re0 * im0;
-                    const float r1 = fmaf(re1, re1, -im1 * im1), i1 = 2.f * re1 * im1;
-                    re0 = r0, im0 = i0, re1 = r1, im1 = i1;
-                }
-                pr = pack2(re0, re1);
-                pi = pack2(im0, im1);
-                npi = pack2(-im0, -im1);
-                if (kTPair) {   // Abar^128: what a tile without flags does to the state that enters it
-#pragma unroll
-                    for (int n = R; n < BM; n *= 2) {
-                        const float r0 = fmaf(re0, re0, -im0 * im0), i0 = 2.f * re0 * im0;
-                        const float r1 = fmaf(re1, re1, -im1 * im1), i1 = 2.f * re1 * im1;
-                        re0 = r0, im0 = i0, re1 = r1, im1 = i1;
-                    }
-                    tr = pack2(re0, re1);
-                    ti = pack2(im0, im1);
-                    nti = pack2(-im0, -im1);
-                }
+            // Abar^R, what a row group does to the state that enters it, and for kTPair Abar^128, what a tile does: on their way
+            // while the first tile's MMAs run.  (Squared up from the rounded Abar in fp32, every step of a long sequence
+            // carried that rounding: xT of 60 x 3000 steps 4.1e-5 off, with these 9.0e-6.)
+            chain_par ^= 1;
+            if (te < kPairs) {
+                const float4* src = p.Apow + (n_tile * kS) / 2 + te;
+                cp_async16(smem_u32(&pow_s[chain_par][0][te]), src);
+                if (kTPair) cp_async16(smem_u32(&pow_s[chain_par][kTPair ? 1 : 0][te]), src + p.P / 2);
             }
             C2 cin = zero;      // kTPair: the state that enters this CTA's tile
             if (kTPair && rank == 0 && p.x0) {
@@ -898,6 +892,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 }
                 flag_next = tb + 1 < p.tblocks ? flag_of(chain, tb + 1) : flag_of(chain + npairs, 0);
                 (void)mbar_wait(s.tmem_full(acc), acc_phase, epi_flag);
+                cp_async_wait();
                 if (group_leader()) tma_store_wait_read();   // this row group's results of the previous tile have left shared memory
                 epi_sync();   // flags visible, tile free (nobody reads the previous one any more); also:
                               // the 256 threads leave together or not at all
@@ -993,6 +988,8 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     agg_e[te] = make_float4(e0, e1, e2, e3);
                 }
                 epi_sync();   // group results visible; every thread has its rows in registers
+                const float4 pw = pow_s[chain_par][0][sp];
+                const f32x2 pr = pack2(pw.x, pw.y), pi = pack2(pw.z, pw.w), npi = neg2(pi);
                 C2 x = e;
                 if (kTPair) {
                     // The state that enters the tile comes from the peer CTA (the tile before this one), except for
@@ -1001,6 +998,7 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     // peer's state arrives, so the hand-over costs one multiply-add per tile and CTA.
                     const bool first = rank == 0 && tb == 0, last = rank == 1 && tb == p.tblocks - 1;
                     C2 tile = zero;
+                    const float4 tw = pow_s[chain_par][kTPair ? 1 : 0][sp];
                     if (sl == nsl - 1 && !last) {
 #pragma unroll
                         for (int g = 0; g < nsl - 1; ++g) {
@@ -1018,7 +1016,8 @@ gemm_scan_fwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                         ++n_recv;
                     }
                     if (sl == nsl - 1 && !last) {
-                        const C2 out = gflags == 0u ? cstep2(tr, ti, nti, cin, tile) : tile;
+                        const f32x2 tr = pack2(tw.x, tw.y), ti = pack2(tw.z, tw.w);
+                        const C2 out = gflags == 0u ? cstep2(tr, ti, neg2(ti), cin, tile) : tile;
                         float o0, o1, o2, o3;
                         unpack2(out.re, o0, o1);
                         unpack2(out.im, o2, o3);
@@ -1157,6 +1156,7 @@ struct FbParams {
     int gps;          // row groups per sequence inside a tile: 8, or T / 16
     int nchains;      // n_tiles * ceil(n_units / 2); kTPair: n_tiles * B
     const float2* Abar;
+    const float4* Apow;   // [2][P / 2]: Abar^16 and Abar^128 of two neighbouring states (re, re, im, im)
     const uint8_t* done;
     const float2* x0;     // [B, P] or NULL
     const float2* gxT;    // [B, P] or NULL
@@ -1175,6 +1175,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     auto epi_sync = [] { epi_sync_n<Cfg::kEpiThreads>(); };
     extern __shared__ uint8_t smem_raw[];
     __shared__ float4 agg_e[kFsEpiThreads], carry_s[kPairs];   // (re, re, im, im) of two neighbouring states
+    __shared__ __align__(16) float4 pow_s[2][kTPair ? 2 : 1][kPairs];   // powers of Abar: chains alternate between two slots
     __shared__ uint32_t masks[8];   // [0, 4): flags of the rows one later (the resets of the reverse scan); [4, 8): of the rows
     __shared__ __align__(8) uint64_t xbar[BM / kFsRows];   // one per row group: its rows of x have arrived
     __shared__ float4 carry_ring[2][kTPair ? kPairs : 1];   // kTPair: the value handed over by the peer CTA, two slots in turn
@@ -1321,6 +1322,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             return chain < p.nchains ? p.Abar[(chain % p.n_tiles) * kS + 2 * sp + k] : make_float2(0.f, 0.f);
         };
         float2 a0_next = abar_of(pair, 0), a1_next = abar_of(pair, 1);
+        int chain_par = 0;
         for (int chain = pair; chain < p.nchains && ok; chain += npairs) {
             const int n_tile = chain % p.n_tiles, b = seq_of(chain);
             const bool has_seq = b < p.n_units;
@@ -1329,30 +1331,11 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             a0_next = abar_of(chain + npairs, 0);
             a1_next = abar_of(chain + npairs, 1);
             const f32x2 ar = pack2(a0.x, a1.x), ai = pack2(a0.y, a1.y), nai = pack2(-a0.y, -a1.y);
-            f32x2 pr, pi, npi;   // conj(Abar)^R by squaring in fp32
-            f32x2 tr = 0ull, ti = 0ull, nti = 0ull;
-            {
-                float re0 = a0.x, im0 = a0.y, re1 = a1.x, im1 = a1.y;
-#pragma unroll
-                for (int n = 1; n < R; n *= 2) {
-                    const float r0 = fmaf(re0, re0, -im0 * im0), i0 = 2.f * re0 * im0;
-                    const float r1 = fmaf(re1, re1, -im1 * im1), i1 = 2.f * re1 * im1;
-                    re0 = r0, im0 = i0, re1 = r1, im1 = i1;
-                }
-                pr = pack2(re0, re1);
-                pi = pack2(im0, im1);
-                npi = pack2(-im0, -im1);
-                if (kTPair) {   // conj(Abar)^128: what a tile without flags does to the value that enters it
-#pragma unroll
-                    for (int n = R; n < BM; n *= 2) {
-                        const float r0 = fmaf(re0, re0, -im0 * im0), i0 = 2.f * re0 * im0;
-                        const float r1 = fmaf(re1, re1, -im1 * im1), i1 = 2.f * re1 * im1;
-                        re0 = r0, im0 = i0, re1 = r1, im1 = i1;
-                    }
-                    tr = pack2(re0, re1);
-                    ti = pack2(im0, im1);
-                    nti = pack2(-im0, -im1);
-                }
+            chain_par ^= 1;   // Abar^R and, for kTPair, Abar^128: as in the forward kernel
+            if (te < kPairs) {
+                const float4* src = p.Apow + (n_tile * kS) / 2 + te;
+                cp_async16(smem_u32(&pow_s[chain_par][0][te]), src);
+                if (kTPair) cp_async16(smem_u32(&pow_s[chain_par][kTPair ? 1 : 0][te]), src + p.P / 2);
             }
             C2 cin = zero;      // kTPair: s of the row after this CTA's tile (nothing after the sequence's last row)
             C2 g = zero;        // this thread's part of the chain's sums s_t conj(x_{t-1})
@@ -1385,6 +1368,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 uint32_t ra[32], ra2[32], rb[32], rb2[32];
                 tmem_ld32(t_row + (uint32_t)(grp * 32), ra);
                 tmem_ld32(t_row + (uint32_t)(Cfg::kCols + grp * 32), ra2);
+                cp_async_wait();
                 if (group_leader()) tma_store_wait_read();   // this row group's results of the previous tile have left shared memory
                 epi_sync();   // flags visible, tile free (nobody reads the previous one any more); also:
                               // the 256 threads leave together or not at all
@@ -1501,6 +1485,8 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     agg_e[te] = make_float4(e0, e1, e2, e3);
                 }
                 epi_sync();   // group results visible
+                const float4 pw = pow_s[chain_par][0][sp];
+                const f32x2 pr = pack2(pw.x, pw.y), npi = pack2(pw.z, pw.w), pi = neg2(npi);   // (conjugate)
                 C2 x = e;
                 if (kTPair) {
                     // The value that enters the tile (s of the row after it) comes from the peer CTA, which holds the
@@ -1509,6 +1495,7 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     // from zero) is ready before the peer's value arrives.
                     const bool first = rank == 1 && tb == p.tblocks - 1, last = rank == 0 && tb == 0;
                     C2 tile = zero;
+                    const float4 tw = pow_s[chain_par][kTPair ? 1 : 0][sp];
                     if (sl == 0 && !last) {
 #pragma unroll
                         for (int gq = nsl - 1; gq >= 1; --gq) {
@@ -1528,7 +1515,8 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                         cin = zero;
                     }
                     if (sl == 0 && !last) {
-                        const C2 out = gflags == 0u ? cstep2(tr, ti, nti, cin, tile) : tile;
+                        const f32x2 tr = pack2(tw.x, tw.y), nti = pack2(tw.z, tw.w);
+                        const C2 out = gflags == 0u ? cstep2(tr, neg2(nti), nti, cin, tile) : tile;
                         float o0, o1, o2, o3;
                         unpack2(out.re, o0, o1);
                         unpack2(out.im, o2, o3);
@@ -2223,7 +2211,7 @@ static int launch_gemm_scan_fwd_s(const GemmScanFwd& g, cudaStream_t st) {
     const int units = fs_units(g.B, g.T), n_tiles = g.P / kS;
     FsParams p{g.B, g.T, g.P, n_tiles, g.H / BK, kRagged ? fs_tiles(g.T) : (g.T >= BM ? g.T / BM : 1),
                kRagged || g.T >= BM ? g.T : BM, units, kRagged || g.T >= BM ? BM / kFsRows : g.T / kFsRows, n_tiles * ((units + 1) / 2),
-               g.Abar, g.done, g.x0, g.xT, (uint32_t*)g.x_planes, (size_t)M * g.P, g.hdr};
+               g.Abar, (const float4*)g.Apow, g.done, g.x0, g.xT, (uint32_t*)g.x_planes, (size_t)M * g.P, g.hdr};
     if (kTPair) {   // a chain is one sequence; each CTA has every other tile
         p.tblocks = (g.T + 2 * BM - 1) / (2 * BM);
         p.nchains = n_tiles * g.B;
@@ -2268,7 +2256,7 @@ static int launch_gemm_scan_bwd_s(const GemmScanBwd& g, cudaStream_t st) {
     const int units = fs_units(g.B, g.T), n_tiles = g.P / kS;
     FbParams p{g.B, g.T, g.P, n_tiles, g.H / BK, kRagged ? fs_tiles(g.T) : (g.T >= BM ? g.T / BM : 1),
                kRagged || g.T >= BM ? g.T : BM, units, kRagged || g.T >= BM ? BM / kFsRows : g.T / kFsRows, n_tiles * ((units + 1) / 2),
-               g.Abar, g.done, g.x0, g.gxT, g.gA_part, g.gx0, g.hdr};
+               g.Abar, (const float4*)g.Apow, g.done, g.x0, g.gxT, g.gA_part, g.gx0, g.hdr};
     if (kTPair) {
         p.tblocks = (g.T + 2 * BM - 1) / (2 * BM);
         p.nchains = n_tiles * g.B;

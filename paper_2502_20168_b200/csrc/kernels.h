@@ -16,8 +16,12 @@ void launch_discretize_bwd(int H, int P, const float2* Lambda, const float* Delt
 struct PackJob {
     const float2* Lambda; const float* Delta; const float2 *Bc, *Cc;
     float2 *Abar, *Alo;
+    float* Apow;   // tensor-core path with a group: powers of Abar for the kernels that scan in their epilogue
     void *WB, *WC, *Cp, *Bq;
 };
+// Apow: Abar^16 (a row group of those kernels), then Abar^128 (a tile), evaluated in double and rounded once; four floats
+// per two neighbouring states: re, re, im, im.
+constexpr int apow_floats(int P) { return 4 * P; }
 constexpr int kLayerBatch = 16;   // layers of a stack that one launch of the parameter kernels takes
 // Tensor-core path: WB / WC hi/lo stacked [4P, H]; group: 0 = rows in the plain order (2p + c, stacked per 128 rows:
 // GemmTcTN with split_w), or the states per chain (64, 32) of the kernels that scan in their epilogue.
@@ -188,6 +192,7 @@ struct GemmScanFwd {
     const void* Wsplit;     // hi/lo stacked Bbar operand [4P, H] (as for GemmTcTN with split_w)
     int B, T, H, P;
     const float2* Abar;     // [P]
+    const float* Apow;      // powers of Abar (PackJob)
     const uint8_t* done;    // [B*T] or NULL
     const float2* x0;       // [B, P] or NULL
     void* x_planes;         // out: bf16 hi plane [B*T, 2P], then the lo plane
@@ -210,6 +215,7 @@ struct GemmScanBwd {
     const void* Wsplit;     // hi/lo stacked conj(C) operand [4P, H], rows in the pair_cols order
     int B, T, H, P;
     const float2* Abar;     // [P]
+    const float* Apow;      // powers of Abar (PackJob)
     const uint8_t* done;    // [B*T] or NULL
     const float2* x0;       // [B, P] or NULL
     const float2* gxT;      // [B, P] or NULL

@@ -1,4 +1,4 @@
-"""Parameter gradients as sums over many rows: how far the order of the fp32 additions lets them drift from the oracle's."""
+"""Sums and recurrences over many rows: how far the order of the fp32 operations lets their results drift from the oracle's."""
 import numpy as np
 import pytest
 
@@ -56,3 +56,20 @@ def test_segments_of_a_slice_bf16(B, T, H, P):
     ref = oracle_layer(d)
     for k in ("dB", "dC"):
         assert _off(res[k], ref[k]) <= 4 * 2.0 ** -17, k
+
+
+@pytest.mark.parametrize("B,T,H,P", [(16, 1000, 512, 256), (6, 4096, 512, 256), (40, 1500, 256, 128), (150, 2048, 128, 64)])
+def test_states_of_long_sequences_bf16(B, T, H, P):
+    """The final state after T steps of slowly decaying states, on the kernels that scan in their epilogue (both CTAs of a
+    pair on one sequence, or one each).  Bbar carries 16 bits: up to 2^-17 off, 2^-18 on average over a sum.  The
+    multipliers over 16 and 128 steps are rounded once, by up to 2^-25 of their size, which a state that lives through T
+    steps meets T / 16 times.  Bound: 2^-18 + T / 16 2^-25.  (A multiplier that carries the rounding of a single step 16
+    times over is off by T / 2 2^-25 on average: 1.5e-5 after 1000 steps, 6e-5 after 4096.)"""
+    from paper_2502_20168_b200 import harness
+    w = I.Workload("long_x", B=B, T=T, H=H, P=P, io_dtype="bf16", p_done=0.0, seed=7)
+    d = I.draw_layer(w)
+    d["Delta"] = np.full_like(d["Delta"], 1e-3)
+    res = harness.run_layer(d, "bf16")
+    off = _off(res["xT"], oracle_layer(d)["xT"])
+    print(f"T = {T}: xT {off:.2e} off")
+    assert off <= 2.0 ** -18 + T / 16 * 2.0 ** -25
