@@ -371,20 +371,20 @@ layer_finalize_kernel(int H, int P, int gA_rows, int gg_rows, const __grid_const
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int p_blocks = (P + 31) / 32;
     if ((int)blockIdx.x >= p_blocks) {   // 32 columns of one of the sums over row groups (dD, then a stack's dw, db)
-        float(*sD)[33] = reinterpret_cast<float(*)[33]>(sA);
+        double(*sD)[33] = sA[0];
         const int h_blocks = (H + 31) / 32, blk = (int)blockIdx.x - p_blocks, which = blk / h_blocks;
         const int h = (blk - which * h_blocks) * 32 + lane;
         const float* part = q.sum_part[which];
-        float acc = 0.f;
+        double acc = 0.0;
         if (h < H)
-            for (int r = w; r < q.sum_rows[which]; r += 32) acc += part[(size_t)r * H + h];
+            for (int r = w; r < q.sum_rows[which]; r += 32) acc += (double)part[(size_t)r * H + h];
         sD[w][lane] = acc;
         __syncthreads();
         if (w == 0 && h < H) {
-            float t = 0.f;
+            double t = 0.0;
 #pragma unroll
             for (int i = 0; i < 32; ++i) t += sD[i][lane];
-            q.sum_out[which][h] = t;
+            q.sum_out[which][h] = (float)t;
         }
         return;
     }

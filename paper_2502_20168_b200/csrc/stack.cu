@@ -1,5 +1,5 @@
 // Wrapper of the stacked sequence model: out = LayerNorm(u + GELU(v)) * w + b with v = SSM(u),
-// forward and backward.  One CTA per row of H features; arithmetic in fp32.  Only the stack's own
+// forward and backward.  A warp per row of up to 1024 features, a CTA per wider row; arithmetic in fp32.  Only the stack's own
 // input, output and their gradients are in the I/O type; what passes between the layers (v, the
 // layer inputs, the gradients handed down) is fp32, hence the separate element types below.
 #include "kernels.h"
@@ -266,17 +266,22 @@ stack_bwd_row_kernel(int M, int H, const TG* g, const TI* u, const float* v, con
     }
 }
 
-// CTAs of the row kernels: enough to give every warp a row, at most two per SM.
-static int ln_row_blocks(int M) {
-    const int need = (M + kLnWarps - 1) / kLnWarps, most = 2 * device_sm_count();
-    return need < most ? need : most;
+// CTAs of the row kernels: enough to give every warp a row, at most two per SM; in the backward pass as many such rounds
+// as it takes to leave a warp no more than kLnRows rows, since its sums for dw and db are chains of fp32 additions
+// (1048576 x 128 in one round, 443 rows a warp: dw 4.2e-7 off, 1.5e-7 with 16; 591 / 516 us; 64000 x 512 134 / 142).
+constexpr int kLnRows = 16;
+static int ln_row_blocks(int M, bool bwd) {
+    const int need = (M + kLnWarps - 1) / kLnWarps, round = 2 * device_sm_count();
+    if (need <= round) return need;
+    const int least = bwd ? (M + kLnWarps * kLnRows - 1) / (kLnWarps * kLnRows) : 1;
+    return (least + round - 1) / round * round;
 }
 static bool ln_by_rows(int H) { return H <= 1024; }
 
 static inline int ln_groups(int M) { return (M + kLnGradRows - 1) / kLnGradRows; }
 
 // Rows of partial sums of dw and db (each) that launch_stack_bwd leaves, and the floats they and its scratch take.
-static int stack_part_rows(int M, int H) { return ln_by_rows(H) ? ln_row_blocks(M) : ln_groups(M); }
+static int stack_part_rows(int M, int H) { return ln_by_rows(H) ? ln_row_blocks(M, true) : ln_groups(M); }
 size_t stack_tmp_floats(int M, int H) {
     const int g = stack_part_rows(M, H);
     return 2 * ((size_t)g * H + colsum_tmp_floats(g, H));
@@ -285,7 +290,7 @@ size_t stack_tmp_floats(int M, int H) {
 template <typename TI, typename TO>
 static void stack_fwd_launch(int M, int H, const void* u, const float* v, const float* w, const float* b, void* out, float* mu,
                              float* rstd, cudaStream_t st) {
-    const int blocks = ln_row_blocks(M), threads = 32 * kLnWarps;
+    const int blocks = ln_row_blocks(M, false), threads = 32 * kLnWarps;
     const TI* uu = (const TI*)u;
     TO* oo = (TO*)out;
     if (H <= 256) launch_dep(stack_fwd_row_kernel<2, TI, TO>, blocks, threads, 0, st, M, H, uu, v, w, b, oo, mu, rstd);
@@ -309,7 +314,7 @@ static void stack_bwd_launch(int M, int H, const void* g, const void* u, const f
                              const float* rstd, float* gz, float* gv, float* part_w, float* part_b, cudaStream_t st) {
     const TG* gg = (const TG*)g;
     const TI* uu = (const TI*)u;
-    const int blocks = ln_row_blocks(M), threads = 32 * kLnWarps;
+    const int blocks = ln_row_blocks(M, true), threads = 32 * kLnWarps;
     count_launch(ln_by_rows(H) ? 1 : 2);
     if (H <= 256) launch_dep(stack_bwd_row_kernel<2, TG, TI>, blocks, threads, 0, st, M, H, gg, uu, v, w, mu, rstd, gz, gv, part_w, part_b);
     else if (H <= 512) launch_dep(stack_bwd_row_kernel<4, TG, TI>, blocks, threads, 0, st, M, H, gg, uu, v, w, mu, rstd, gz, gv, part_w, part_b);

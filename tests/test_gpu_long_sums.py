@@ -73,3 +73,19 @@ def test_states_of_long_sequences_bf16(B, T, H, P):
     off = _off(res["xT"], oracle_layer(d)["xT"])
     print(f"T = {T}: xT {off:.2e} off")
     assert off <= 2.0 ** -18 + T / 16 * 2.0 ** -25
+
+
+def test_layernorm_bias_gradient_over_a_million_rows():
+    """dln_bias of the last layer is the plain sum of gout over the rows.  Chains of at most 16 rows a warp, 8 warps and groups
+    of 64 such sums, the rest in double: about sqrt(L / 6) 2^-24 for each of these lengths, 1e-7, and the final rounding,
+    3e-8; bound: twice their sum.  (443 rows a warp: 4.3e-7.)"""
+    import torch
+    from paper_2502_20168_b200 import binding as sb, harness
+    w = I.Workload("ln_rows", B=1024, T=1024, H=128, P=8, io_dtype="f32", p_done=0.0, n_layers=2, seed=7)
+    s = harness.StackBuffers(harness.device_drawn(w), "f32")
+    s.forward()
+    s.backward()
+    sb.ssm_check(s.ws)
+    ref = s.gout.double().sum((0, 1))
+    off = torch.linalg.vector_norm(s.grads[-1]["dln_bias"] - ref) / torch.linalg.vector_norm(ref)
+    assert float(off) <= 2.6e-7
