@@ -70,6 +70,19 @@ template <typename T> __device__ __forceinline__ T from_f32(float v);
 template <> __device__ __forceinline__ float from_f32<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
+// 1 / (1 + exp(-z)).  With t = exp(-|z|) <= 1 the divisor lies in [1, 2], where the approximate reciprocal is good to 2 ulp of
+// fp32 (of 1 / (1 + exp(-z)) it makes 0 for z < -87.3).  A result in IO = float gets a Newton step, after which the
+// reciprocal is at most a unit in the last place off; bf16 results come out the same without it (share of outputs that differ
+// from the rounded exact ones 2.3e-4 either way, 2.4e-4 with exact quotients; a projection of 4096 x 1024 with the gate
+// 32.7 us, with exact quotients 33.5).
+template <typename IO>
+__device__ __forceinline__ float sigmoid_f(float z) {
+    const float t = expf(-fabsf(z)), d = 1.f + t;
+    float r = __fdividef(1.f, d);
+    if (sizeof(IO) == 4) r = fmaf(r, fmaf(-d, r, 1.f), r);
+    return z < 0.f ? t * r : r;
+}
+
 // ---- workspace header -------------------------------------------------------------------
 // First 256 bytes of every workspace.  `status` is written by kernels whose bounded waits
 // give up.

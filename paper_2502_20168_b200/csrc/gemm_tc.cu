@@ -337,7 +337,7 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float2 sf = __bfloat1622float2(s2[e]);
-                    o2[e] = __floats2bfloat162_rn(gate_value(sf.x, z[2 * e]), gate_value(sf.y, z[2 * e + 1]));
+                    o2[e] = __floats2bfloat162_rn(sf.x * sigmoid_f<__nv_bfloat16>(z[2 * e]), sf.y * sigmoid_f<__nv_bfloat16>(z[2 * e + 1]));
                 }
                 *reinterpret_cast<uint4*>(ob + lane * 64 + ((j ^ swz) << 4)) = o[j];
             }

@@ -305,7 +305,7 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         const float4 s4 = sk[i0 + i].get(true);
                         *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + e) = v[i];
                         *reinterpret_cast<uint2*>(p.gate_out + e) =
-                            pack4_bf16(make_float4(gate_value(s4.x, v[i].x), gate_value(s4.y, v[i].y), gate_value(s4.z, v[i].z), gate_value(s4.w, v[i].w)));
+                            pack4_bf16(make_float4(s4.x * sigmoid_f<__nv_bfloat16>(v[i].x), s4.y * sigmoid_f<__nv_bfloat16>(v[i].y), s4.z * sigmoid_f<__nv_bfloat16>(v[i].z), s4.w * sigmoid_f<__nv_bfloat16>(v[i].w)));
                     }
                 }
             }

@@ -12,12 +12,6 @@ __device__ __forceinline__ float gelu_f(float v) { return 0.5f * v * (1.f + erff
 __device__ __forceinline__ float gelu_grad_f(float v) {
     return 0.5f * (1.f + erff(v * 0.70710678118654752f)) + v * 0.3989422804014327f * expf(-0.5f * v * v);
 }
-// bf16 results take the fast division (2 ulp of fp32), which is a third of the instructions of the exact one.
-template <typename IO>
-__device__ __forceinline__ float sigmoid_f(float z) {
-    const float d = 1.f + expf(-z);
-    return sizeof(IO) == 2 ? __fdividef(1.f, d) : 1.f / d;
-}
 
 constexpr int kThreads = 256;
 inline int blocks_for(size_t n) {

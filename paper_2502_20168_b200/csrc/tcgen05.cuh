@@ -176,9 +176,6 @@ __host__ __device__ constexpr uint32_t instr_desc(int m, int n, int a_mn, int b_
            ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// v * sigmoid(z) for a bf16 result: the division to 2 ulp (the correctly rounded one is ten times the instructions).
-__device__ __forceinline__ float gate_value(float v, float z) { return __fdividef(v, 1.f + __expf(-z)); }
-
 // Row-major bf16 matrix [rows, cols] (cols contiguous), boxes of box_cols x box_rows, 128-byte swizzle.
 inline bool make_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols,
                      uint32_t box_rows, bool f32 = false, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B,
