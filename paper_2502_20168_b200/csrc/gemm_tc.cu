@@ -1553,6 +1553,11 @@ gemm_scan_bwd_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     // (the wait gave up: the flag is set, everybody leaves at the next barrier)
                 }
                 xphase ^= 1u;
+                if (kRagged && left >= r0 && left < r0 + R) {
+                    // the row after the sequence's last: its s is 0, its x is the sequence's final state, which enters no
+                    // product and may be infinite
+                    xs[(left - r0) * kPairs] = xs[(R + left - r0) * kPairs] = make_uint2(0u, 0u);
+                }
                 const bool seq_start = tb == 0 && sl == g0 && (!kTPair || rank == 0);   // row 0 of this group is the sequence's first row
                 if (short_seq && seq_start) {                // the state before that row: this sequence's x0
                     xinit = zero;

@@ -119,6 +119,26 @@ def test_fused_projection_and_scan_ragged_lengths_bf16(B, T, H, P):
     run(I.small_variant(w, p_done=0.0))
 
 
+@pytest.mark.parametrize("B,T,H,P", [(40, 200, 256, 128), (20, 1000, 128, 64), (30, 120, 256, 128), (12, 600, 256, 256)])
+def test_ragged_lengths_ignore_a_state_after_the_last_row_bf16(B, T, H, P):
+    """Every sequence's state overflows in its last step: no product of dLambda and dDelta has that state in it, but the row
+    after it in memory, which shares its tile and belongs to the next sequence, does."""
+    w = I.Workload("ragged_inf", B=B, T=T, H=H, P=P, io_dtype="bf16", p_done=0.02, seed=B + T)
+    d = I.draw_layer(w)
+    d["Bc"] = (d["Bc"] * 1e4).astype(np.complex64)
+    d["u"] = d["u"].copy()
+    d["u"][:, T - 1] *= np.float32(2.0 ** 124)   # exact in bf16
+    d["gy"] = d["gy"] * np.float32(2.0 ** -100)
+    d["done"][:, 0] = 0
+    from paper_2502_20168_b200 import harness
+    res = harness.run_layer(d, "bf16")
+    ref = oracle_layer(d)
+    assert np.abs(ref["xT"]).max() > 3.5e38   # past the range of fp32
+    for k in ("dLambda", "dDelta", "dB"):
+        assert np.isfinite(res[k]).all(), k
+        assert np.linalg.norm(res[k] - ref[k]) <= TOL["bf16"] * np.linalg.norm(ref[k]), k
+
+
 @pytest.mark.parametrize("io,B,T,H,P", [("f32", 3, 50, 40, 48), ("bf16", 80, 128, 256, 128), ("bf16", 5, 77, 256, 256)])
 def test_conjugate_symmetric_variant_is_the_layer_with_half_the_states_and_doubled_C(io, B, T, H, P):
     """A system whose P states come in conjugate pairs is stored as its first P/2 states and run as
