@@ -218,7 +218,8 @@ pack_params_kernel(int H, int P, const __grid_constant__ PackArgs<kN> o) {
     const float2 *Bc = q.Bc, *Cc = q.Cc;
     __shared__ float2 gamma_s[32];
     __shared__ float2 tB[32][33], tC[32][33];   // tB[state][h], tC[h][state]
-    const int p0 = blockIdx.x * 32, h0 = blockIdx.y * 32;
+    const int p_blocks = (P + 31) / 32, h_tile = (int)blockIdx.x / p_blocks;
+    const int p0 = ((int)blockIdx.x - h_tile * p_blocks) * 32, h0 = h_tile * 32;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const float2 zero = make_float2(0.f, 0.f);
     float2 b[4], c[4];
@@ -232,7 +233,7 @@ pack_params_kernel(int H, int P, const __grid_constant__ PackArgs<kN> o) {
         const int p = p0 + lane;
         const ZohTerms z = zoh_terms(q.Lambda[p], q.Delta[p]);
         gamma_s[lane] = make_float2((float)z.gr, (float)z.gi);
-        if (blockIdx.y == 0) {
+        if (h_tile == 0) {
             const float2 ah = make_float2((float)z.ar, (float)z.ai);
             q.Abar[p] = ah;
             q.Alo[p] = make_float2((float)(z.ar - (double)ah.x), (float)(z.ai - (double)ah.y));
@@ -252,7 +253,7 @@ pack_params_kernel(int H, int P, const __grid_constant__ PackArgs<kN> o) {
             }
         }
     }
-    if (threadIdx.x == 32 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && o.hdr) o.hdr->status = 0;
+    if (threadIdx.x == 32 && blockIdx.x == 0 && blockIdx.z == 0 && o.hdr) o.hdr->status = 0;
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -302,7 +303,8 @@ reduce_weight_grads_kernel(int H, int P, int splits, const __grid_constant__ Tai
     __shared__ float2 gamma_s[32];
     __shared__ float2 t[32][33];   // [feature][state]
     constexpr int kRows = 32 / kReduceWarps;
-    const int p0 = blockIdx.x * 32, h0 = blockIdx.y * 32;
+    const int p_blocks = (P + 31) / 32, h_tile = (int)blockIdx.x / p_blocks;
+    const int p0 = ((int)blockIdx.x - h_tile * p_blocks) * 32, h0 = h_tile * 32;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const bool is_c = (blockIdx.z & 1) != 0, p_ok = p0 + lane < P;
     if (w == kReduceWarps) {
@@ -350,7 +352,7 @@ reduce_weight_grads_kernel(int H, int P, int splits, const __grid_constant__ Tai
             gq.x += __shfl_xor_sync(0xffffffffu, gq.x, m);
             gq.y += __shfl_xor_sync(0xffffffffu, gq.y, m);
         }
-        if (lane == 0) q.gg[(size_t)blockIdx.y * P + p] = gq;
+        if (lane == 0) q.gg[(size_t)h_tile * P + p] = gq;
     }
 }
 
@@ -423,7 +425,8 @@ layer_finalize_kernel(int H, int P, int gA_rows, int gg_rows, const __grid_const
                     q.dLambda[p], q.dDelta[p]);
 }
 
-static dim3 weight_tiles(int H, int P, int z) { return dim3((P + 31) / 32, (H + 31) / 32, z); }
+// One block per 32 x 32 tile, the tiles of 32 features after one another along x (y is limited to 65535 blocks).
+static dim3 weight_tiles(int H, int P, int z) { return dim3((unsigned)((P + 31) / 32) * (unsigned)((H + 31) / 32), 1, z); }
 
 template <int kMode, int kN>
 static void launch_pack_n(int H, int P, int n, const PackJob* jobs, int group, WsHeader* hdr, cudaStream_t st) {

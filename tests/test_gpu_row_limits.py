@@ -1,4 +1,4 @@
-"""Row counts past the limits of a grid's second and third dimension (65535 blocks)."""
+"""Row counts and widths past the limits of a grid's second and third dimension (65535 blocks)."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -36,3 +36,27 @@ def test_more_row_groups_than_a_grid_has_blocks_along_z(io):
         del h
     for k in parts:
         assert float(torch.linalg.vector_norm(whole[k] - parts[k]) / torch.linalg.vector_norm(parts[k])) <= 2.2e-5, k
+
+
+def test_more_features_than_tiles_along_a_grid_dimension():
+    """2097184 features are 65537 tiles of 32.  One step of a layer with 8 states: y and du elementwise against float64, dB and
+    dC against the products they are (one row: no sums)."""
+    import torch
+    from paper_2502_20168_b200 import binding as sb, harness, inputs as I
+    B, T, H, P = 1, 1, 2097184, 8
+    d = I.draw_layer(I.Workload("wide", B=B, T=T, H=H, P=P, io_dtype="f32", p_done=0.0, seed=12))
+    buf = harness.LayerBuffers(d, "f32")
+    buf.forward()
+    buf.backward()
+    sb.ssm_check(buf.ws)
+    c, r = torch.complex128, torch.float64
+    Lam, dt, Bc, Cc = buf.Lambda.to(c), buf.Delta.to(r), buf.Bc.to(c), buf.Cc.to(c)
+    u, gy, D = buf.u.to(r)[0, 0], buf.gy.to(r)[0, 0], buf.D.to(r)
+    gamma = (torch.exp(Lam * dt) - 1) / Lam
+    x = (gamma[:, None] * Bc) @ u.to(c)
+    s = Cc.conj().T @ gy.to(c)
+    assert float((buf.y[0, 0] - ((Cc @ x).real + D * u)).abs().max()) <= 1e-4
+    assert float((buf.du[0, 0] - (((gamma[:, None] * Bc).conj().T @ s).real + D * gy)).abs().max()) <= 1e-4
+    for got, ref in ((buf.dB, gamma.conj()[:, None] * s[:, None] * u), (buf.dC, gy[:, None] * x.conj()[None])):
+        assert float(torch.linalg.vector_norm(got - ref) / torch.linalg.vector_norm(ref)) <= 1e-4
+    assert torch.isfinite(buf.dLambda.real).all() and torch.isfinite(buf.dDelta).all()
