@@ -116,7 +116,7 @@ def _load() -> ctypes.CDLL:
 
 
 _lib = _load()
-_raw_stream = torch._C._cuda_getCurrentRawStream
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # torch builds without CUDA do not have it
 _current_device = torch.cuda.current_device
 
 
@@ -151,7 +151,9 @@ def _ptr(t):
 
 def _stream(stream=None):
     # the raw handle: torch.cuda.current_stream() builds a Stream object on every call
-    return _raw_stream(_current_device()) if stream is None else stream.cuda_stream
+    if stream is None:
+        return _raw_stream(_current_device()) if _raw_stream else torch.cuda.current_stream().cuda_stream
+    return stream.cuda_stream
 
 
 def _nbytes(t) -> int:

@@ -31,6 +31,16 @@ def test_every_declared_symbol_is_exported(sb):
     assert set(names) == set(sb.EXPORTS)
 
 
+def test_binding_imports_where_torch_has_no_cuda_symbols(sb):
+    import subprocess
+    import sys
+    code = ("import torch\n"
+            "if hasattr(torch._C, '_cuda_getCurrentRawStream'): del torch._C._cuda_getCurrentRawStream\n"
+            "from paper_2502_20168_b200 import binding as sb\n"
+            "assert sb.ssm_layer_workspace_bytes(sb.make_shape(2, 8, 16, 8, 'f32')) > 0\n")
+    subprocess.run([sys.executable, "-c", code], cwd=ROOT, check=True, timeout=300)
+
+
 def test_status_strings(sb):
     assert sb.status_string(0) == "ok"
     seen = {sb.status_string(c) for c in range(-7, 1)}
