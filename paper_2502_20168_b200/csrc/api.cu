@@ -177,8 +177,7 @@ SSM_API int ssm_scan_fwd(const ssm_shape* shape, const ssm_c64* Abar, const ssm_
     if (cudaMemsetAsync(ws, 0, sizeof(WsHeader), st) != cudaSuccess) return SSM_ERR_CUDA;
     StageTimer tm("scan_fwd", st);
     int rc = launch_scan_fwd(shape->B, shape->T, shape->P, (const float2*)Abar, nullptr, (const float2*)Bu, done,
-                             (const float2*)x0, x, false, (float2*)xT, at<WsHeader>(ws, 0),
-                             at<char>(ws, sizeof(WsHeader)), st);
+                             (const float2*)x0, x, false, (float2*)xT, at<WsHeader>(ws, 0), st);
     if (rc) return rc;
     SSM_RETURN_IF_CUDA_ERROR();
     return SSM_OK;
@@ -302,8 +301,7 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
         {
             StageTimer tm("scan_fwd", st);
             rc = launch_scan_fwd(s.B, s.T, s.P, at<float2>(ws, p.Abar), at<float2>(ws, p.Alo), at<float2>(ws, p.f32buf), done,
-                                 (const float2*)x0, at<void>(ws, p.xs), true, (float2*)xT, hdr,
-                                 at<char>(ws, p.scan), st);
+                                 (const float2*)x0, at<void>(ws, p.xs), true, (float2*)xT, hdr, st);
             if (rc) return rc;
         }
         {   // y[m,h] = sum_k x[m,k] Cp[h,k] + D[h] u[m,h]
@@ -320,8 +318,7 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
         {
             StageTimer tm("scan_fwd", st);
             rc = launch_scan_fwd(s.B, s.T, s.P, at<float2>(ws, p.Abar), at<float2>(ws, p.Alo), at<float2>(ws, p.xs), done,
-                                 (const float2*)x0, at<void>(ws, p.xs), false, (float2*)xT, hdr,
-                                 at<char>(ws, p.scan), st);
+                                 (const float2*)x0, at<void>(ws, p.xs), false, (float2*)xT, hdr, st);
             if (rc) return rc;
         }
         {   // y = x Cp^T + D u: six products of planes, the skip term in the epilogue
@@ -340,8 +337,7 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
         {
             StageTimer tm("scan_fwd", st);
             rc = launch_scan_fwd(s.B, s.T, s.P, at<float2>(ws, p.Abar), at<float2>(ws, p.Alo), at<float2>(ws, p.xs), done,
-                                 (const float2*)x0, at<void>(ws, p.xs), false, (float2*)xT, hdr,
-                                 at<char>(ws, p.scan), st);
+                                 (const float2*)x0, at<void>(ws, p.xs), false, (float2*)xT, hdr, st);
             if (rc) return rc;
         }
         {

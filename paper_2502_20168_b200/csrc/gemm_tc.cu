@@ -2142,9 +2142,6 @@ static bool make_plane_map4(CUtensorMap* map, const void* planes, int B, int T, 
 // 24: 6 x 4096 287 / 271, 12 x 1024 (256, 128) 103 / 86; 20: 5 x 2048 168 / 151, 5 x 16384 826 / 854; 18: 9 x 512 (256, 128)
 // 72 / 63; 16: 2 x 4096 the separate kernels.
 static int fused_min_pairs(int T) { return T <= 4096 ? 18 : 24; }
-#ifndef SSM_FUSED_NARROW_BELOW
-#define SSM_FUSED_NARROW_BELOW 0   // 0: chains of 32 states where chains of 64 would occupy at most half of the CTA pairs
-#endif
 
 // Sequences whose rows do not fall on tile boundaries: a sequence's last tile is then partly empty.
 static bool fs_ragged(int T) { return !(T % tc::BM == 0 || T == 16 || T == 32 || T == 64); }
@@ -2156,9 +2153,6 @@ static int fs_units(int B, int T) { return T >= tc::BM || fs_ragged(T) ? B : (B 
 // the chains, half the tile), or not at all (group 0); and, for few long sequences, both CTAs of a pair on one
 // sequence (time pairs: CTA 0 has the even tiles, CTA 1 the odd ones, the state passes from one to the other
 // through shared memory), which doubles the chains without halving the tile.
-#ifndef SSM_FUSED_TIME_PAIRS
-#define SSM_FUSED_TIME_PAIRS 1
-#endif
 struct FusedMode {
     int group;
     bool time_pairs;
@@ -2172,8 +2166,8 @@ static FusedMode fused_mode(int B, int T, int H, int P) {
     // where the second half of the CTA pairs would otherwise idle: 16 x 16384 at P = 256 1.88 -> 1.78 ms per step,
     // 16 x 1024 0.242 -> 0.229; with 64 of 74 pairs busy (32 sequences) it costs 30 - 50 % in these kernels.
     // Time pairs double the chains at the full tile: 16 x 16384 1.76 -> 1.48 ms, 16 x 1024 0.228 -> 0.212.
-    const int narrow_below = SSM_FUSED_NARROW_BELOW > 0 ? SSM_FUSED_NARROW_BELOW : tc::sm_count() / 4 + 1;
-    const bool tp_ok = SSM_FUSED_TIME_PAIRS && (T % (2 * tc::BM) == 0 || (ragged && T > tc::BM));
+    const int narrow_below = tc::sm_count() / 4 + 1;
+    const bool tp_ok = (T % (2 * tc::BM) == 0 || (ragged && T > tc::BM));
     // Rounds of chains x tiles per chain: what the kernels' time goes with.
     const int tiles = T >= tc::BM || ragged ? fs_tiles(T) : 1, tp_tiles = (T + 2 * tc::BM - 1) / (2 * tc::BM);
     const int steps = (pairs64 + np - 1) / np * tiles;

@@ -443,8 +443,10 @@ int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st) {
     const bool io_bf16 = g.skip_bf16 && (!g.dot || g.dot_bf16);
 #define SSM_SMALL(EPI, SPLIT, BF)                                                             \
     do {                                                                                      \
-        if (s.pair && s.bn == 128) return launch_small<128, EPI, false, BF, true>(ma, mw, p, grid, smem, st); \
-        if (s.pair) return launch_small<256, EPI, false, BF, true>(ma, mw, p, grid, smem, st);                \
+        if constexpr (!SPLIT) {   /* (an fp32 operand is split by single CTAs) */                             \
+            if (s.pair && s.bn == 128) return launch_small<128, EPI, false, BF, true>(ma, mw, p, grid, smem, st); \
+            if (s.pair) return launch_small<256, EPI, false, BF, true>(ma, mw, p, grid, smem, st);                \
+        }                                                                                                     \
         if (s.bn == 64) return launch_small<64, EPI, SPLIT, BF, false>(ma, mw, p, grid, smem, st);            \
         if (s.bn == 128) return launch_small<128, EPI, SPLIT, BF, false>(ma, mw, p, grid, smem, st);          \
         return launch_small<256, EPI, SPLIT, BF, false>(ma, mw, p, grid, smem, st);                           \
@@ -454,7 +456,7 @@ int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st) {
     if (epi == kSmStore) SSM_SMALL(kSmStore, false, true);
     if (g.a_f32) SSM_SMALL(kSmDiag, true, false);
     if (io_bf16) SSM_SMALL(kSmDiag, false, true);
-    SSM_SMALL(kSmDiag, false, false);
+    return SSM_ERR_SHAPE;   // planes of A with fp32 skip or dot: left to gemm_tc_planes.cu
 #undef SSM_SMALL
 }
 

@@ -382,9 +382,6 @@ struct StepShape {
     int bn, cluster, stages, stage_bytes;
 };
 
-#ifndef SSM_STEP_FORCE
-#define SSM_STEP_FORCE(bn, c) false
-#endif
 // Tile width and cluster size by an estimate in microseconds like that of the few-tile projections.
 StepShape pick_step(int M, int H, int P, bool f32) {
     StepShape best{0, 0, 0, 0};
@@ -396,7 +393,6 @@ StepShape pick_step(int M, int H, int P, bool f32) {
         const int stages = std::min<int>(kStMaxStages, (int)((kStSmemMax - 2048 - (size_t)BM * (bn + 4) * 4) / sb));
         if (stages < 2) continue;
         for (int c = 1; c <= 8; c *= 2) {
-            if (SSM_STEP_FORCE(bn, c)) continue;
             const int slots = c == 1 ? sms : (c == 2 ? sms - 4 : (c == 4 ? sms - 16 : sms - 36));   // clusters must fit a GPC
             const int waves = (m_tiles * c + slots - 1) / slots;
             const int i0 = ((2 * P + bn - 1) / bn + c - 1) / c, i1 = ((H + bn - 1) / bn + c - 1) / c;

@@ -50,8 +50,7 @@ void launch_layer_tail(int H, int P, int splits, int n, const GradTail* tails, i
 size_t scan_scratch_bytes(int B, int T, int P, int rows_per_seq = 1);   // rows_per_seq = 2: room for launch_gemm_scan_bwd_part
 // Alo (may be NULL): low part of Abar, so that Abar + Alo carries the multiplier to ~48 bits.
 int launch_scan_fwd(int B, int T, int P, const float2* Abar, const float2* Alo, const float2* Bu, const uint8_t* done,
-                    const float2* x0, void* x, bool x_bf16, float2* xT, WsHeader* hdr, void* scratch,
-                    cudaStream_t st);
+                    const float2* x0, void* x, bool x_bf16, float2* xT, WsHeader* hdr, cudaStream_t st);
 // x and gBu are stored both as fp32 pairs or both as bf16 pairs (x_bf16 == s_bf16).
 // With gA_part / gA_rows (both or neither) the sum over the sequences is left to the caller: *gA_part points
 // at *gA_rows <= kMaxPartialRows rows of P partial sums inside `scratch`, and gAbar is not written.

@@ -305,8 +305,7 @@ size_t scan_scratch_bytes(int B, int T, int P, int rows_per_seq) {
 }
 
 int launch_scan_fwd(int B, int T, int P, const float2* Abar, const float2* Alo, const float2* Bu, const uint8_t* done,
-                    const float2* x0, void* x, bool x_bf16, float2* xT, WsHeader* hdr, void* scratch,
-                    cudaStream_t st) {
+                    const float2* x0, void* x, bool x_bf16, float2* xT, WsHeader* hdr, cudaStream_t st) {
     if (T == 1) {
         const int n = B * (P / 2);
         count_launch();
