@@ -353,11 +353,14 @@ size_t stage_bytes_of(int bn, int planes_a, int planes_w, bool pair) {
     return (size_t)planes_a * kSmATile + (size_t)planes_w * (pair ? bn / 2 : bn) * BK * 2;
 }
 
-// Tile width and cluster size, or a CTA pair: the choice with the shortest estimated time.  The estimate is a fit, in microseconds, to
-// timings of all pairs on twenty shapes from 16 x 256 x 256 to 4096 x 1024 x 1024, back to back (within 10 % of the
-// measured time, and the pair it picks within 8 % of the fastest): a wave of CTAs takes a fixed part that grows with
-// the tile (start, first loads, epilogue), its k-blocks at 48 bytes of operands per cycle and SM (L2), 0.95 us where
-// fp32 operands are split on the way, and the exchange between the CTAs of a cluster.
+// Tile width and cluster size, or a CTA pair: the choice with the shortest estimated time.  The estimate for single CTAs and
+// clusters is a fit, in microseconds, to timings of all of them on twenty shapes from 16 x 256 x 256 to 4096 x 1024 x 1024,
+// back to back (within 10 % of the measured time, and the one it picks within 8 % of the fastest): a wave of CTAs takes a
+// fixed part that grows with the tile (start, first loads, epilogue), its k-blocks at 48 bytes of operands per cycle and SM
+// (L2), 0.95 us where fp32 operands are split on the way, and the exchange between the CTAs of a cluster.  Pairs go through
+// the same formula with their own operand bytes; it was not fitted to them, only checked on whole passes, with pairs / with
+// single CTAs and clusters: gate of 4096 x 1024 102.4 / 108.2 us, of 4096 x 512 47.9 / 49.7, layer 64 x 100 (256, 128)
+// 55.4 / 57.4, 32 x 128 (512, 256) 63.5 / 63.5, 32 x 128 (1024, 512) 114.6 / 114.2.
 SmallShape pick_small(int M, int N, int k_blocks, int planes_a, int planes_w, bool split_a, bool w_stacked) {
     SmallShape best{0, 0, 0, false};
     double best_t = 0.0;

@@ -382,7 +382,9 @@ struct StepShape {
     int bn, cluster, stages, stage_bytes;
 };
 
-// Tile width and cluster size by an estimate in microseconds like that of the few-tile projections.
+// Tile width and cluster size by an estimate in microseconds built like that of the few-tile projections (fixed cost of a
+// tile, k-blocks at the slower of L2 and tensor core, both phases).  Its constants are taken over from there, not fitted
+// to this kernel.
 StepShape pick_step(int M, int H, int P, bool f32) {
     StepShape best{0, 0, 0, 0};
     double best_t = 0.0;

@@ -83,7 +83,7 @@ def test_layer_plan_names_the_kernels_a_shape_takes(sb):
     assert plan(48, 1024, 512, 256, "bf16") == fused % (64, 1)      # 96 chains: three half-rounds beat two rounds
     assert plan(64, 4096, 512, 256, "bf16") == fused % (64, 0)      # 128 chains: four half-rounds do not
     assert plan(4, 1024, 512, 256, "bf16") == "projections=tensor-cores scans=separate"       # too few chains
-    assert plan(3, 333, 512, 128, "bf16") == "projections=tensor-cores scans=separate"        # T not a multiple of 128
+    assert plan(3, 333, 512, 128, "bf16") == "projections=tensor-cores scans=separate"        # 4 chain pairs: too few
     # argument checks
     import ctypes
     buf = ctypes.create_string_buffer(8)
