@@ -13,6 +13,13 @@
 // memory: 8 KB), a 256 x 128 x 16 MMA of a pair 70 for twice the work.  64000 x 512 x 512 in a layer's passes,
 // one CTA per 128 x 128 tile / pairs: 175 / 136 us, with the skip term and the column sums 189 / 149.
 // hi hi has an accumulator of its own (see gemm_tc_small.cu).
+// The tensor core truncates its accumulator at every addition.  A tile of more than kPlSegment stages of K is multiplied in
+// that many segments of equal length, which take the two halves of tensor memory in turn like tiles of their own: the
+// epilogue warps add a finished segment to their registers while the next one runs.  40000 rows, K = 384, errors of a layer's y and
+// du against float64: 1.8e-7 and 1.2e-7 in one chain, 1.2e-7 and 0.7e-7 in two (CUDA cores: 1.6e-7 and 0.9e-7).  It costs 2 % of
+// 64000 x 512 x 512, 4 to 9 % with the skip term and the column sums, whose epilogue then holds only one half of
+// tensor memory's lead (194 to 198, 205 to 213, 214 to 233 us).  A short last segment: the same time, 1.27e-7 and 0.77e-7 off.
+// Emptying the last segment before the epilogue's operands are requested (registers): du 248 us.
 #include <algorithm>
 
 #include "kernels.h"
@@ -26,6 +33,7 @@ constexpr int kPlBK = 32;      // K extent of an operand stage: 64-byte rows
 constexpr int kPlStages = 5;
 constexpr int kPlATile = BM * kPlBK * 2, kPlWTile = kPlBN / 2 * kPlBK * 2;   // one plane, of a CTA
 constexpr int kPlStageBytes = 3 * kPlATile + 3 * kPlWTile;
+constexpr int kPlSegment = 8;  // stages of a segment at most: 16 additions per accumulator
 constexpr int kPlEpiWarps = 8;
 constexpr int kPlThreads = 64 + 32 * kPlEpiWarps;
 constexpr int kPlSlabBytes = 32 * 32 * 4;
@@ -33,6 +41,7 @@ constexpr size_t kPlSmem = (size_t)kPlStages * kPlStageBytes + kPlEpiWarps * kPl
 
 struct PlanesArgs {
     int M, N, K, n_tiles, tiles, k_blocks;
+    int segs, seg_blocks;      // segments of a tile, stages of a segment (the last one may have fewer)
     int planes_a, n_prod;      // planes of A (3, or 1: a bf16 operand), products of the schedule (see GemmTcTN)
     uint32_t pa, pw;
     void* out;
@@ -50,7 +59,7 @@ struct PlanesBars {
     int abort_flag;
 };
 
-template <bool kDiag>
+template <bool kDiag, bool kSegs>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPlThreads, 1)
 gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ PlanesArgs p) {
     extern __shared__ uint8_t smem_raw[];
@@ -114,13 +123,14 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
             int stage = 0, n = 0;
             uint32_t phase = 0;
             bool ok = true;
-            for (int tile = pair; tile < p.tiles && ok; tile += npairs, ++n) {
-                const int buf = n & 1;
-                if (n >= 2) {   // the epilogue has taken tile n - 2 out of this half of tensor memory
+            for (int tile = pair; tile < p.tiles && ok; tile += npairs)
+            for (int seg = 0; seg < (kSegs ? p.segs : 1) && ok; ++seg, ++n) {   // n: segments so far
+                const int buf = n & 1, kb_first = kSegs ? seg * p.seg_blocks : 0, kb_end = kSegs ? min(p.k_blocks, kb_first + p.seg_blocks) : p.k_blocks;
+                if (n >= 2) {   // the epilogue has taken segment n - 2 out of this half of tensor memory
                     if (!(ok = mbar_wait_warp(smem_u32(&bars.free[buf]), (uint32_t)((n >> 1) - 1) & 1u, abort_flag))) break;
                     tc_fence_after();
                 }
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                for (int kb = kb_first; kb < kb_end; ++kb) {
                     if (!(ok = mbar_wait_warp(smem_u32(&bars.full[stage]), phase, abort_flag))) break;
                     tc_fence_after();
                     const uint32_t base = smem_u32(stages) + (uint32_t)stage * kPlStageBytes;
@@ -133,7 +143,7 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 #pragma unroll
                             for (int k = 0; k < kPlBK / UK; ++k)
                                 umma_bf16_pair(d_tmem, ad + (uint64_t)(2 * k), wd + (uint64_t)(2 * k), idesc,
-                                          (uint32_t)!(kb == 0 && k == 0 && (j == 0 || !small)));
+                                          (uint32_t)!(kb == kb_first && k == 0 && (j == 0 || !small)));
                         }
                         umma_commit_pair(smem_u32(&bars.empty[stage]));
                     }
@@ -155,9 +165,35 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         const uint32_t leader_free = map_to_cta(smem_u32(&bars.free[0]), 0);
         int n = 0;
         for (int tile = pair; tile < p.tiles; tile += npairs, ++n) {
-            const int buf = n & 1, m_tile = 2 * (tile / p.n_tiles) + rank, m0 = m_tile * BM + 32 * q, n0 = (tile % p.n_tiles) * kPlBN + 64 * half;
+            const int m_tile = 2 * (tile / p.n_tiles) + rank, m0 = m_tile * BM + 32 * q, n0 = (tile % p.n_tiles) * kPlBN + 64 * half;
+            const uint32_t t_warp = tmem_base + ((uint32_t)(q * 32) << 16) + 64u * (uint32_t)half;
             bool ok = true;
+            float sum[kSegs ? 64 : 1];   // this lane's row and the warp's 64 columns, all segments but the last
+            if (kSegs) {
+#pragma unroll
+                for (int j = 0; j < (kSegs ? 64 : 1); ++j) sum[j] = 0.f;
 #pragma unroll 1
+                for (int seg = 0; seg + 1 < p.segs; ++seg, ++n) {
+                    const int buf = n & 1;
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars.done[buf]), (uint32_t)(n >> 1) & 1u, abort_flag))) break;
+                    tc_fence_after();
+#pragma unroll
+                    for (int c0 = 0; c0 < (kSegs ? 64 : 0); c0 += 16) {
+                        uint32_t v[16], w[16];
+                        tmem_ld16(t_warp + 256u * (uint32_t)buf + (uint32_t)c0, v);
+                        tmem_ld16(t_warp + 256u * (uint32_t)buf + 128u + (uint32_t)c0, w);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) sum[kSegs ? c0 + j : 0] += __uint_as_float(v[j]) + __uint_as_float(w[j]);
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(leader_free + 8u * (uint32_t)buf);
+                }
+                if (!ok) break;
+            }
+            const int buf = n & 1;
+#pragma unroll(kSegs ? 2 : 1)
             for (int sl = 0; sl < 2; ++sl) {
                 const int col = n0 + 32 * sl + 4 * c;
                 const bool n_ok = col < p.N;
@@ -173,16 +209,19 @@ gemm_tc_planes_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                     }
                 }
                 if (sl == 0) {
-                    if (!(ok = mbar_wait(smem_u32(&bars.done[buf]), (uint32_t)(n >> 1) & 1u, abort_flag))) break;
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars.done[buf]), (uint32_t)(n >> 1) & 1u, abort_flag))) break;
                     tc_fence_after();
                 }
-                const uint32_t t = tmem_base + ((uint32_t)(q * 32) << 16) + 256u * (uint32_t)buf + 64u * (uint32_t)half + 32u * (uint32_t)sl;
+                const uint32_t t = t_warp + 256u * (uint32_t)buf + 32u * (uint32_t)sl;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {   // 16 columns at a time (registers)
                     uint32_t v[16], w[16];
                     tmem_ld16(t + 16u * (uint32_t)h, v);
                     tmem_ld16(t + 128u + 16u * (uint32_t)h, w);
                     tmem_ld_wait();
+                    if (kSegs)
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + sum[kSegs ? 32 * sl + 16 * h + j : 0]);
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
                         slab[lane * 8 + ((4 * h + j) ^ (lane & 7))] =
@@ -268,6 +307,8 @@ int launch_gemm_tc_planes(const GemmTcTN& g, cudaStream_t st) {
     PlanesArgs p{};
     p.M = g.M, p.N = g.N_out, p.K = g.K, p.k_blocks = g.K / kPlBK;
     p.planes_a = g.planes_a, p.n_prod = g.n_products, p.pa = g.prod_a, p.pw = g.prod_w;
+    p.segs = (p.k_blocks + kPlSegment - 1) / kPlSegment;
+    p.seg_blocks = (p.k_blocks + p.segs - 1) / p.segs;
     p.n_tiles = (g.N_out + kPlBN - 1) / kPlBN;
     const int m_tiles = (g.M + BM - 1) / BM;
     p.tiles = (m_tiles + 1) / 2 * p.n_tiles;
@@ -283,7 +324,9 @@ int launch_gemm_tc_planes(const GemmTcTN& g, cudaStream_t st) {
         const int pairs = std::min(p.tiles, resident_pairs(reinterpret_cast<const void*>(kern), kPlSmem, kPlThreads));
         return pairs > 0 && launch_dep(kern, 2 * pairs, kPlThreads, kPlSmem, st, ma, mw, p);
     };
-    return (g.diag ? run(gemm_tc_planes_kernel<true>) : run(gemm_tc_planes_kernel<false>)) ? SSM_OK : SSM_ERR_CUDA;
+    const bool ok = p.segs > 1 ? (g.diag ? run(gemm_tc_planes_kernel<true, true>) : run(gemm_tc_planes_kernel<false, true>))
+                               : (g.diag ? run(gemm_tc_planes_kernel<true, false>) : run(gemm_tc_planes_kernel<false, false>));
+    return ok ? SSM_OK : SSM_ERR_CUDA;
 }
 
 }  // namespace ssm

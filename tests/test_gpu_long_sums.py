@@ -89,3 +89,21 @@ def test_layernorm_bias_gradient_over_a_million_rows():
     ref = s.gout.double().sum((0, 1))
     off = torch.linalg.vector_norm(s.grads[-1]["dln_bias"] - ref) / torch.linalg.vector_norm(ref)
     assert float(off) <= 2.6e-7
+
+
+@pytest.mark.parametrize("B,T,H,P", [(8, 1000, 384, 192), (8, 1000, 512, 256), (7, 1003, 640, 320), (8, 1000, 256, 192)])
+def test_projections_fp32_in_segments(B, T, H, P):
+    """fp32 layers of many tiles without the skip term: y and du are a projection, the recurrence and a projection.  The tensor
+    core truncates at every addition, n 2^-25 2/3 for a chain of n (as above), and the two projections' losses add.  Chains
+    of 16 additions of 16 products; bound: 2 x 16 x 2^-25 2/3 and 2^-24 for the rest.  (Chains of 24 and 32, over all of K: 7.7e-7
+    and 1.0e-6.)  Inner lengths of one segment (256), of one and a half, two and two and a half."""
+    from paper_2502_20168_b200 import harness
+    w = I.Workload("planes_k", B=B, T=T, H=H, P=P, io_dtype="f32", p_done=0.002, seed=7)
+    d = I.draw_layer(w)
+    d["D"] = np.zeros_like(d["D"])
+    res = harness.run_layer(d, "f32")
+    ref = oracle_layer(d)
+    for k in ("y", "du"):
+        off = _off(res[k], ref[k])
+        print(f"({H}, {P}): {k} {off:.2e} off")
+        assert off <= 2 * 16 * 2.0 ** -25 * 2 / 3 + 2.0 ** -24, k
