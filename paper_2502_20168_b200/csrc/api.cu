@@ -26,7 +26,7 @@ struct LayerPlan {
 };
 
 // fp32 layers of tile-sized widths.  us per forward and backward pass, CUDA cores / planes, at H, P = 384, 192: 50 rows
-// 106 / 61, 1024 rows 132 / 74, 40000 rows 2355 / 523; at 128, 64: 8 rows 49 / 53, 64 rows 52 / 53, 1024 rows 58 / 57, 30000
+// 106 / 61, 1024 rows 132 / 74, 40000 rows 2355 / 541; at 128, 64: 8 rows 49 / 53, 64 rows 52 / 53, 1024 rows 58 / 57, 30000
 // rows 274 / 174.  Errors against float64 are smaller with planes: 40000 rows at 384, 192: y 1.6e-7 / 1.2e-7, du 8.8e-8 / 6.9e-8 in
 // the 2-norm, the gradient sums by as much or more.
 // Single steps take them at every batch size: the operands prepared for one are read at any other (us per step in a graph, fp32
