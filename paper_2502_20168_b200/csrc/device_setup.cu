@@ -1,6 +1,7 @@
 // Per-device, per-kernel set-up that launchers would otherwise repeat on every call.
 #include <map>
 #include <mutex>
+#include <set>
 #include <utility>
 
 #include "common.cuh"
@@ -22,6 +23,22 @@ bool set_max_dynamic_smem(const void* kernel, size_t bytes) {
         return false;
     }
     done[{kernel, dev}] = bytes;
+    return true;
+}
+
+// The same for clusters of 16 CTAs, which a kernel has to ask for.
+bool allow_large_clusters(const void* kernel) {
+    static std::mutex mu;
+    static std::set<std::pair<const void*, int>> done;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done.count({kernel, dev})) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    done.insert({kernel, dev});
     return true;
 }
 
