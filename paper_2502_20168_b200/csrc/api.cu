@@ -17,9 +17,11 @@ namespace {
 //  * plane path (fp32 I/O and tile-sized H, P with enough rows): the same projections on tcgen05 as sums
 //    of products of bf16 planes (three planes per fp32 value: exact), fp32 states, scans as on the
 //    CUDA-core path.
+//  * small layers off the tensor cores: each pass in one kernel, a CTA per sequence; fp32 x is all that is kept.
 struct LayerPlan {
     bool tc;
     bool planes;
+    bool small;
     int splits;
     size_t hdr, Abar, Alo, Apow, W0, W1, W2, W3, f32buf, xs, gs, gAbar, gg, scan, part, dot, total;
     size_t u3, gy3, x3, s3;   // plane path: planes of u, gy, x, s for the weight gradients
@@ -58,7 +60,8 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true, bool step = false
     p.tc = allow_tc && s.io_dtype == SSM_BF16 && tc_tn_supported((int)BT, P2, s.H, true) &&
            tc_tn_supported((int)BT, s.H, P2, false) && tc_nt_supported(s.H, P2);
     p.planes = !p.tc && s.io_dtype == SSM_F32 && planes_supported(s, step);
-    p.splits = p.tc ? tc_nt_splits((int)BT, s.H, P2) : (p.planes ? tc_nt_planes_splits((int)BT, s.H, P2, 2) : gemm_nt_splits((int)BT, s.H, P2));
+    p.small = allow_tc && !step && !p.tc && !p.planes && layer_small_cluster(s.B, s.T, s.H, s.P) > 0;
+    p.splits = p.small ? s.B : p.tc ? tc_nt_splits((int)BT, s.H, P2) : (p.planes ? tc_nt_planes_splits((int)BT, s.H, P2, 2) : gemm_nt_splits((int)BT, s.H, P2));
     p.hdr = take(off, sizeof(WsHeader));
     p.Abar = take(off, (size_t)s.P * 8);
     p.Alo = take(off, (size_t)s.P * 8);
@@ -373,6 +376,14 @@ SSM_API int ssm_layer_fwd(const ssm_shape* shape, const ssm_c64* Lambda, const f
     if (int rc = check_ws(ws, ws_bytes, p.total)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     WsHeader* hdr = at<WsHeader>(ws, p.hdr);
+    if (p.small) {
+        StageTimer tm("scan_fwd", st);   // (with everything around the scan)
+        const LayerSmall g{s.B, s.T, s.H, s.P, s.io_dtype == SSM_BF16, (const float2*)Lambda, Delta, (const float2*)Bc, (const float2*)Cc,
+                           D, u, done, (const float2*)x0, nullptr, nullptr, at<float2>(ws, p.xs), y, (float2*)xT, nullptr, hdr};
+        if (int rc = launch_layer_small_fwd(g, st)) return rc;
+        SSM_RETURN_IF_CUDA_ERROR();
+        return SSM_OK;
+    }
     return layer_fwd_impl(s, p, layer_io(s), Lambda, Delta, Bc, Cc, D, u, done, x0, y, xT, ws, hdr, st);
 }
 
@@ -734,6 +745,23 @@ SSM_API int ssm_layer_bwd(const ssm_shape* shape, const ssm_c64* Lambda, const f
     cudaStream_t st = (cudaStream_t)stream;
     WsHeader* hdr = at<WsHeader>(ws, p.hdr);
     LayerTail left{};
+    if (p.small) {
+        {
+            StageTimer tm("scan_bwd", st);   // (with everything around the scan)
+            float* part = at<float>(ws, p.part);
+            left.gA_rows = s.B;
+            left.tail = {(const float2*)Lambda, Delta, (const float2*)Bc, part, part + (size_t)p.splits * 2 * s.P * s.H, (float2*)dB,
+                         (float2*)dC, at<float2>(ws, p.gg), at<float2>(ws, p.scan), (float2*)dLambda, dDelta,
+                         {at<float>(ws, p.dot), nullptr, nullptr}, {s.B, 0, 0}, {dD, nullptr, nullptr}};
+            const LayerSmall g{s.B, s.T, s.H, s.P, s.io_dtype == SSM_BF16, (const float2*)Lambda, Delta, (const float2*)Bc,
+                               (const float2*)Cc, D, u, done, (const float2*)x0, (const float2*)gxT, gy, at<float2>(ws, p.xs), du, nullptr,
+                               (float2*)dx0, hdr};
+            if (int rc = launch_layer_small_bwd(g, left.tail, at<float2>(ws, p.scan), at<float>(ws, p.dot), st)) return rc;
+        }
+        if (s.B > 1) return layer_bwd_tail(s, p, 1, &left, hdr, st);
+        SSM_RETURN_IF_CUDA_ERROR();
+        return SSM_OK;
+    }
     if (int rc = layer_bwd_impl(s, p, layer_io(s), Lambda, Delta, Bc, D, u, done, x0, gy, gxT, nullptr, ws, hdr, du, dLambda,
                                 dDelta, dB, dC, dD, dx0, &left, st))
         return rc;

@@ -3,35 +3,9 @@
 #include <algorithm>
 
 #include "kernels.h"
+#include "zoh.cuh"
 
 namespace ssm {
-
-// exp(z) - 1 for z = a + ib without cancellation near z = 0.
-__device__ __forceinline__ void expm1_complex(double a, double b, double& re, double& im) {
-    double sb, cb;
-    sincos(b, &sb, &cb);
-    double sh = sin(0.5 * b);
-    re = expm1(a) * cb - 2.0 * sh * sh;
-    im = exp(a) * sb;
-}
-
-struct ZohTerms {
-    double ar, ai;  // Abar = exp(Lambda Delta)
-    double gr, gi;  // gamma = (Abar - 1) / Lambda
-};
-
-__device__ __forceinline__ ZohTerms zoh_terms(float2 lam, float dt) {
-    double lr = lam.x, li = lam.y, d = dt;
-    double er, ei;
-    expm1_complex(lr * d, li * d, er, ei);
-    double n = lr * lr + li * li;
-    ZohTerms z;
-    z.ar = er + 1.0;
-    z.ai = ei;
-    z.gr = (er * lr + ei * li) / n;
-    z.gi = (ei * lr - er * li) / n;
-    return z;
-}
 
 // One block per state p: Abar[p], Bbar[p, :] = gamma_p * B[p, :].
 __global__ void discretize_kernel(int H, const float2* Lambda, const float* Delta,
@@ -48,23 +22,6 @@ __global__ void discretize_kernel(int H, const float2* Lambda, const float* Delt
     __syncthreads();
     const float2 g = gamma_s;
     for (int h = threadIdx.x; h < H; h += blockDim.x) Bbar[(size_t)p * H + h] = cmul(g, Bc[(size_t)p * H + h]);
-}
-
-// Adjoint of the discretisation for one state: from gAbar and g_gamma (= sum_h conj(B) gBbar).
-__device__ __forceinline__ void zoh_adjoint(const ZohTerms& z, float2 lam, float dt, double gar, double gai, double ggr,
-                                            double ggi, float2& dLambda, float& dDelta) {
-    const double lr = lam.x, li = lam.y, d = dt;
-    // dgamma/dLambda = (Delta Abar - gamma) / Lambda     (= (Delta Abar Lambda - (Abar-1)) / Lambda^2)
-    const double nr = d * z.ar - z.gr, ni = d * z.ai - z.gi;
-    const double n = lr * lr + li * li;
-    const double qr = (nr * lr + ni * li) / n, qi = (ni * lr - nr * li) / n;
-    // dLambda = conj(Delta Abar) gAbar + conj(dgamma/dLambda) g_gamma
-    const double outr = d * (z.ar * gar + z.ai * gai) + (qr * ggr + qi * ggi);
-    const double outi = d * (z.ar * gai - z.ai * gar) + (qr * ggi - qi * ggr);
-    dLambda = make_float2((float)outr, (float)outi);
-    // dDelta = Re(conj(Lambda Abar) gAbar) + Re(conj(Abar) g_gamma)
-    const double lar = lr * z.ar - li * z.ai, lai = lr * z.ai + li * z.ar;
-    dDelta = (float)((lar * gar + lai * gai) + (z.ar * ggr + z.ai * ggi));
 }
 
 // ssm_discretize_bwd: one block per state p.

@@ -45,6 +45,27 @@ struct GradTail {
 int gamma_part_rows(int H);
 void launch_layer_tail(int H, int P, int splits, int n, const GradTail* tails, int gA_rows, cudaStream_t st);
 
+// layer_small.cu: the passes of a layer of few and narrow sequences, on the CUDA cores, a CTA per sequence.
+struct LayerSmall {
+    int B, T, H, P;
+    bool bf16;                // u, gy, out
+    const float2* Lambda; const float* Delta; const float2 *Bc, *Cc;
+    const float* D;
+    const void* u;
+    const uint8_t* done;      // [B, T] or NULL
+    const float2 *x0, *gxT;   // [B, P] or NULL; gxT: backward
+    const void* gy;           // backward
+    float2* x;                // [B, T, P]: written by the forward pass, read by the backward pass
+    void* out;                // y, or du
+    float2 *xT, *gx0;         // [B, P] or NULL
+    WsHeader* hdr;
+};
+int layer_small_cluster(int B, int T, int H, int P);   // CTAs per sequence; 0: not taken
+int launch_layer_small_fwd(const LayerSmall& g, cudaStream_t st);   // also clears the status word
+// B = 1: all gradients of `tail` are final.  Else part_b and part_c hold B slices, gA_part [B, P] and dD_part [B, H] the rows
+// of partial sums, for launch_layer_tail.
+int launch_layer_small_bwd(const LayerSmall& g, const GradTail& tail, float2* gA_part, float* dD_part, cudaStream_t st);
+
 // scan.cu
 // Scratch the scans need for a [B,T,P] problem: a work counter and the partial sums of gAbar.
 size_t scan_scratch_bytes(int B, int T, int P, int rows_per_seq = 1);   // rows_per_seq = 2: room for launch_gemm_scan_bwd_part
