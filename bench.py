@@ -449,7 +449,8 @@ def scan_stage_summary(r, peaks):
     out = {}
     for key in ("gemm_Bu_scan_fwd", "scan_fwd", "gemm_gx_scan_bwd", "scan_bwd"):
         ms = r["stage_ms_per_step"].get(key)
-        if ms:
+        proj = {"scan_fwd": "gemm_Bu", "scan_bwd": "gemm_gx"}.get(key)
+        if ms and (not proj or proj in r["stage_ms_per_step"]):   # (a scan stage without one has the projection inside)
             gbs = STAGE_MODEL[key][1](r["H"], r["P"], s_io) * n / (ms * 1e-3) / 1e9
             out[key] = {"ms": ms, "algorithmic_GBps": round(gbs, 1), "frac_of_measured_copy": round(gbs / peaks["hbm_gbs"], 4),
                         "frac_of_8TBps": round(gbs / 8000.0, 4)}

@@ -314,6 +314,13 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
             if ((rc = launch_gemm_tc_tn(g, st))) return rc;
         }
     } else if (p.planes) {
+        if (tc_tile_scan_supported(s.B, s.T, s.H, s.P, io.u_bf16)) {
+            StageTimer tm("scan_fwd", st);   // Bu as below, scanned in the projection's epilogue
+            TileScan scan{s.B, s.T, at<float2>(ws, p.Abar), at<float2>(ws, p.Alo), done, (const float2*)x0, nullptr, (float2*)xT};
+            GemmTcTN g{u, at<void>(ws, p.W0), BT, P2, s.H, false, true, at<void>(ws, p.xs), nullptr, nullptr, hdr};
+            g.scan = &scan;
+            if ((rc = plane_projection(g, io.u_bf16, at<void>(ws, p.u3), keep_planes, st))) return rc;
+        } else {
         {   // Bu = u Bbar^T as a sum of plane products (u: three planes of an fp32 input, or the bf16 input itself)
             StageTimer tm("gemm_Bu", st);
             const GemmTcTN g{u, at<void>(ws, p.W0), BT, P2, s.H, false, true, at<void>(ws, p.xs), nullptr, nullptr, hdr};
@@ -324,6 +331,7 @@ static int layer_fwd_run(const ssm_shape& s, const LayerPlan& p, const LayerIo& 
             rc = launch_scan_fwd(s.B, s.T, s.P, at<float2>(ws, p.Abar), at<float2>(ws, p.Alo), at<float2>(ws, p.xs), done,
                                  (const float2*)x0, at<void>(ws, p.xs), false, (float2*)xT, hdr, st);
             if (rc) return rc;
+        }
         }
         {   // y = x Cp^T + D u: six products of planes, the skip term in the epilogue
             StageTimer tm("gemm_y", st);
@@ -635,6 +643,16 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
         }
     } else if (p.planes) {
         const bool gyb = io.gy_bf16, ub = io.u_bf16;
+        if (!gyb && tc_tile_scan_supported(s.B, s.T, s.H, s.P, false)) {
+            StageTimer tm("scan_bwd", st);   // g_x as below, scanned in the projection's epilogue
+            TileScan scan{s.B, s.T, at<float2>(ws, p.Abar), at<float2>(ws, p.Alo), done, (const float2*)x0, (const float2*)gxT, nullptr, (float2*)dx0,
+                          at<float2>(ws, p.xs)};
+            GemmTcTN g{gy, at<void>(ws, p.W1), BT, P2, s.H, false, true, at<void>(ws, p.gs), nullptr, nullptr, hdr};
+            g.scan = &scan;
+            scan.gA_part = scan_partials(at<char>(ws, p.scan));
+            if ((rc = plane_projection(g, false, at<void>(ws, p.gy3), true, st))) return rc;
+            gA_part = reduce_scan_partials(s.B, s.P, at<char>(ws, p.scan), &gA_rows, st);
+        } else {
         {   // g_x = gy conj(C)
             StageTimer tm("gemm_gx", st);
             const GemmTcTN g{gy, at<void>(ws, p.W1), BT, P2, s.H, false, true, at<void>(ws, p.gs), nullptr, nullptr, hdr};
@@ -647,6 +665,7 @@ static int layer_bwd_impl(const ssm_shape& s, const LayerPlan& p, const LayerIo&
                                  at<void>(ws, p.gs), false, at<float2>(ws, p.gAbar), (float2*)dx0, hdr,
                                  at<char>(ws, p.scan), st, &gA_part, &gA_rows);
             if (rc) return rc;
+        }
         }
         {   // du = s Bq^T + D gy (+ the residual branch's gradient), and dD's sums
             StageTimer tm("gemm_du", st);

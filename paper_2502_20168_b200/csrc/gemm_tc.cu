@@ -2034,7 +2034,7 @@ static int pair_tiles_of(int M, int n_tiles) { return ((M + 2 * tc::BM - 1) / (2
 enum { kEpiStore = 0, kEpiDiag = 1, kEpiGate = 2, kEpiDot = 3 };
 static int epi_of(const GemmTcTN& g) { return g.gate_out ? kEpiGate : (g.store_f32 && !g.diag ? kEpiStore : (g.dot ? kEpiDot : kEpiDiag)); }
 static bool use_pairs(const GemmTcTN& g) {
-    if (g.n_products > 3 || g.a_f32 || g.add || (g.diag && g.store_f32)) return false;
+    if (g.n_products > 3 || g.a_f32 || g.scan || g.add || (g.diag && g.store_f32)) return false;
     const int out_cols = g.split_w ? tc::BN / 2 : tc::BN, tiles = pair_tiles_of(g.M, (g.N_out + out_cols - 1) / out_cols);
     const int epi = epi_of(g);
     if (epi == kEpiDot && g.N_out > tc::kDotMaxN) return false;

@@ -19,6 +19,7 @@
 #include <algorithm>
 
 #include "kernels.h"
+#include "scan_math.cuh"
 #include "small_tile.cuh"
 
 namespace ssm {
@@ -51,12 +52,21 @@ struct SmallTnArgs {
     float* dot_part;
     __nv_bfloat16* gate_out;
     bool out_bf16, skip_bf16, dot_bf16;
+    TileScan scan;
+    int tile_rows, seqs;       // rows of a tile: BM, or seqs whole sequences
     WsHeader* hdr;
 };
 
 // Epilogues: fp32 result; out = acc + diag * skip (+ add) with, if asked for, the column sums of skip * dot over the
-// rows of this CTA; fp32 result and out2 = skip * sigmoid(acc) in bf16.
-enum SmallEpi { kSmStore, kSmDiag, kSmGate };
+// rows of this CTA; fp32 result and out2 = skip * sigmoid(acc) in bf16; the scan of the result's rows (columns 2 p, 2 p + 1 are
+// state p), which leaves in its place, forward or backward.
+//
+// The scans: a tile then holds whole sequences, and CTA `rank` finishes all rows of its share of the tile's columns.  A
+// thread has one state and kRows rows; the groups of rows are joined in order through shared memory, as in the streaming
+// kernels.  As kernels of their own the scans of 1024 rows took 4 (forward) and 6 us (backward) of a pass, all latency: forward and
+// backward of 16 x 64 steps at H, P = 256, 128 62.9 -> 55.3 us, a stack of four layers of 512, 256 319 -> 287.
+enum SmallEpi { kSmStore, kSmDiag, kSmGate, kSmScanFwd, kSmScanBwd };
+__host__ __device__ constexpr bool sm_scans(int epi) { return epi >= kSmScanFwd; }
 
 struct SmallBars {
     uint64_t full[kSmMaxStages], empty[kSmMaxStages], done;
@@ -64,7 +74,50 @@ struct SmallBars {
     int abort_flag;
 };
 
-template <int kBN, int kEpi, bool kSplitA, bool kBf16, bool kPair>
+// What a scanning thread reads from afar, asked for while the MMAs run; kRows rows of one state.
+template <int kEpi, int kRows>
+struct ScanThread {
+    int b, t0, len, row0, groups, g;   // sequence, first step, steps, row in the tile; groups of a sequence, the thread's
+    int p;                             // state
+    bool mine;
+    uint32_t flags;
+    float2 a, al, first, before[kEpi == kSmScanBwd ? kRows : 1];
+    __device__ __forceinline__ void fetch(const SmallTnArgs& k, int m_tile, int col0, int te) {
+        constexpr int kStates = 2 * kRows;
+        const TileScan& s = k.scan;
+        groups = (s.T + kRows - 1) / kRows;
+        const int slot = te / kStates, seq = slot / groups;
+        g = slot - seq * groups;
+        b = m_tile * k.seqs + seq;
+        t0 = g * kRows;
+        len = min(kRows, s.T - t0);
+        row0 = seq * s.T + t0;
+        p = col0 / 2 + te % kStates;
+        mine = seq < k.seqs && b < s.B;
+        flags = 0;
+        a = al = first = make_float2(0.f, 0.f);
+        if (!mine) return;
+        a = s.Abar[p], al = s.Alo[p];
+        const size_t m = (size_t)b * s.T + t0, P = (size_t)k.N / 2;
+        if (s.done)
+#pragma unroll
+            for (int i = 0; i < kRows; ++i)
+                if (i < len && s.done[m + i] != 0) flags |= 1u << i;
+        if (kEpi == kSmScanFwd) {
+            if (g == 0 && s.x0) first = s.x0[(size_t)b * P + p];
+        } else {
+            if (g == groups - 1 && s.gxT) first = s.gxT[(size_t)b * P + p];
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) {
+                before[i] = make_float2(0.f, 0.f);
+                if (i < len && t0 + i > 0) before[i] = s.x[(m + i - 1) * P + p];
+                else if (i < len && s.x0) before[i] = s.x0[(size_t)b * P + p];
+            }
+        }
+    }
+};
+
+template <int kBN, int kEpi, bool kSplitA, bool kBf16, bool kPair, int kScanRows = 0>
 __global__ void __launch_bounds__(sm_threads(kBN), 1)
 gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, SmallTnArgs p) {
     extern __shared__ uint8_t smem_raw[];
@@ -78,7 +131,8 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int crank = (int)cluster_ctarank(), rank = kPair ? 0 : crank, tile = (int)blockIdx.x / (kPair ? 2 : p.cluster);
     const int m_tile = kPair ? 2 * (tile / p.n_tiles) + crank : tile / p.n_tiles;
-    const int m0 = m_tile * BM, n0 = (tile % p.n_tiles) * kBN;
+    const int m0 = m_tile * (sm_scans(kEpi) ? p.tile_rows : BM), n0 = (tile % p.n_tiles) * kBN;
+    const int m_end = sm_scans(kEpi) ? min(p.M, m0 + p.tile_rows) : p.M;
     if (threadIdx.x == 0) {
         for (int i = 0; i < p.stages; ++i) {
             mbar_init(smem_u32(&bars.full[i]), kSplitA ? 1 + kSmEpiWarps : 1);
@@ -178,13 +232,13 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         if (kSplitA) {
             const int te = threadIdx.x - 64;
             SplitA<32 * kSmEpiWarps> sp;   // the next k-block's values are on their way while this one is split and stored
-            if (kb0 < kb1) sp.fetch(p.a_f32, p.K, p.M, m0, kb0, te);
+            if (kb0 < kb1) sp.fetch(p.a_f32, p.K, m_end, m0, kb0, te);
             int stage = 0;
             uint32_t phase = 0;
             for (int kb = kb0; kb < kb1; ++kb) {
                 if (!mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
-                sp.store(tiles + (size_t)stage * p.stage_bytes, p.M, m0, te, n0 == 0 ? p.a_planes : nullptr, p.K, kb);
-                if (kb + 1 < kb1) sp.fetch(p.a_f32, p.K, p.M, m0, kb + 1, te);
+                sp.store(tiles + (size_t)stage * p.stage_bytes, m_end, m0, te, n0 == 0 ? p.a_planes : nullptr, p.K, kb);
+                if (kb + 1 < kb1) sp.fetch(p.a_f32, p.K, m_end, m0, kb + 1, te);
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bars.full[stage]));
@@ -209,15 +263,17 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 #pragma unroll
         for (int i = 0; i < kU; ++i) {
             const int r = r0 + i * kRowGroups, m = m0 + row_base + r;
-            if (kEpi != kSmStore && r < rows && m < p.M && n < p.N) {
+            if ((kEpi == kSmDiag || kEpi == kSmGate) && r < rows && m < p.M && n < p.N) {
                 const size_t e = (size_t)m * p.N + n;
                 sk[i].load(p.skip, p.skip_bf16, e);
                 if (kEpi == kSmDiag && p.dot) dt[i].load(p.dot, p.dot_bf16, e);
             }
         }
     };
+    ScanThread<kEpi, kScanRows ? kScanRows : 1> sc;
     if (warp >= 2) {
-        fetch_operands(rg);
+        if (sm_scans(kEpi)) sc.fetch(p, m_tile, n0 + rank * (kBN / parts), te);
+        else fetch_operands(rg);
         if (mbar_wait(smem_u32(&bars.done), 0, abort_flag)) {
             // this CTA's part of the tile -> shared memory (every operand stage has been read: the MMAs are done)
             tc_fence_after();
@@ -249,7 +305,82 @@ gemm_tc_tn_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     __syncwarp();
     if (parts > 1) cluster_sync_all();   // the parts of all CTAs of the cluster are in place
     else __syncthreads();
-    if (warp >= 2 && !*abort_flag) {
+    if (sm_scans(kEpi) && warp >= 2) {
+        constexpr bool kBwd = kEpi == kSmScanBwd;
+        constexpr int kR = kScanRows ? kScanRows : 1, kStates = 2 * kR;
+        __shared__ float4 agg[32 * kSmEpiWarps];
+        auto epi_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(32 * kSmEpiWarps) : "memory"); };
+        const float2 zero = make_float2(0.f, 0.f);
+        const size_t P = (size_t)p.N / 2;
+        float2 v[kR], a = sc.a, al = sc.al, aR, aRl;
+        cpow2_pair<kR>(a, al, aR, aRl);
+        if (kBwd) a = cconj(a), al = cconj(al), aR = cconj(aR), aRl = cconj(aRl);
+        // this thread's rows: the sum of the parts of all CTAs
+        const float* own = reinterpret_cast<const float*>(tiles) + (size_t)sc.row0 * kPitch + rank * (kBN / parts) + 2 * (te % kStates);
+#pragma unroll
+        for (int i = 0; i < kR; ++i) v[i] = zero;
+        if (sc.mine)
+            for (int q = 0; q < parts; ++q) {
+                const uint32_t from = map_to_cta(smem_u32(own), (uint32_t)q);
+                float2 t[kR];
+#pragma unroll
+                for (int i = 0; i < kR; ++i)
+                    if (i < sc.len) t[i] = ld_cluster_f2(from + (uint32_t)i * (kPitch * 4u));
+#pragma unroll
+                for (int i = 0; i < kR; ++i)
+                    if (i < sc.len) v[i] = cadd(v[i], t[i]);
+            }
+        // a group's own contribution; the first one that is folded starts from what enters the sequence
+        float2 e = sc.first;
+        const bool cut = sc.flags != 0u || (kBwd ? sc.g == sc.groups - 1 : sc.g == 0);
+#pragma unroll
+        for (int j = 0; j < kR; ++j) {
+            const int i = kBwd ? kR - 1 - j : j;
+            if (i >= sc.len) continue;
+            if (!kBwd) e = cfma2(a, al, (sc.flags >> i) & 1u ? zero : e, v[i]);
+            else if (i == sc.len - 1) e = cadd(v[i], e);   // (the state's gradient s; what it hands on, conj(Abar) s, is rounded once, below)
+            else e = cfma2(a, al, (sc.flags >> (i + 1)) & 1u ? zero : e, v[i]);
+        }
+        if (kBwd) e = (sc.flags & 1u) ? zero : cfma2(a, al, e, zero);
+        agg[te] = make_float4(e.x, e.y, cut ? 1.f : 0.f, 0.f);
+        epi_sync();
+        float2 c = sc.first, gA = zero;
+        if (sc.mine && !*abort_flag) {
+            const int ahead = kBwd ? sc.groups - 1 - sc.g : sc.g;
+#pragma unroll 4
+            for (int j = ahead; j > 0; --j) {   // the groups before this one, the furthest first
+                const float4 o = agg[te + (kBwd ? j : -j) * kStates];
+                c = o.z != 0.f ? make_float2(o.x, o.y) : cfma2(aR, aRl, c, make_float2(o.x, o.y));
+            }
+            float2* dst = reinterpret_cast<float2*>(p.out) + ((size_t)sc.b * p.scan.T + sc.t0) * P + sc.p;
+#pragma unroll
+            for (int j = 0; j < kR; ++j) {
+                const int i = kBwd ? kR - 1 - j : j;
+                if (i >= sc.len) continue;
+                const bool flag = (sc.flags >> i) & 1u;
+                if (!kBwd) c = cfma2(a, al, flag ? zero : c, v[i]);
+                else if (i == sc.len - 1) c = cadd(v[i], c);
+                else c = cfma2(a, al, (sc.flags >> (i + 1)) & 1u ? zero : c, v[i]);
+                dst[(size_t)i * P] = c;
+                if (kBwd && !flag) gA = cfma(c, cconj(sc.before[kBwd ? i : 0]), gA);
+            }
+            if (kBwd) c = (sc.flags & 1u) ? zero : cfma2(a, al, c, zero);
+            float2* end = kBwd ? p.scan.gx0 : p.scan.xT;
+            if (end && (kBwd ? sc.g == 0 : sc.g == sc.groups - 1)) end[(size_t)sc.b * P + sc.p] = c;
+        }
+        if (kBwd) {   // sum of the groups of a sequence, in order
+            epi_sync();
+            agg[te] = make_float4(gA.x, gA.y, 0.f, 0.f);
+            epi_sync();
+            if (sc.mine && sc.g == 0 && !*abort_flag) {
+                double re = (double)gA.x, im = (double)gA.y;   // (dDelta takes differences of these sums)
+#pragma unroll 4
+                for (int j = 1; j < sc.groups; ++j) re += (double)agg[te + j * kStates].x, im += (double)agg[te + j * kStates].y;
+                p.scan.gA_part[(size_t)sc.b * P + sc.p] = make_float2((float)re, (float)im);
+            }
+        }
+    }
+    if (!sm_scans(kEpi) && warp >= 2 && !*abort_flag) {
         const bool n_ok = n < p.N;
         float4 dg = make_float4(0.f, 0.f, 0.f, 0.f), dsum = dg;
         if (kEpi == kSmDiag && n_ok) dg = *reinterpret_cast<const float4*>(p.diag + n);
@@ -353,6 +484,14 @@ size_t stage_bytes_of(int bn, int planes_a, int planes_w, bool pair) {
     return (size_t)planes_a * kSmATile + (size_t)planes_w * (pair ? bn / 2 : bn) * BK * 2;
 }
 
+// Rows of a scanning thread for a cluster size: kBN / cluster columns of the tile are 2 kRows states.
+constexpr int scan_rows(int cluster) { return 64 / (4 * cluster); }
+// Whole sequences of a tile, so that their groups of rows find a slot of the 256 scanning threads each.
+int scan_seqs(int T, int cluster) {
+    const int r = scan_rows(cluster), slots = 256 / (2 * r), groups = (T + r - 1) / r;
+    return std::min(BM / T, slots / groups);
+}
+
 // Tile width and cluster size, or a CTA pair: the choice with the shortest estimated time.  The estimate for single CTAs and
 // clusters is a fit, in microseconds, to timings of all of them on twenty shapes from 16 x 256 x 256 to 4096 x 1024 x 1024,
 // back to back (within 10 % of the measured time, and the one it picks within 8 % of the fastest): a wave of CTAs takes a
@@ -361,11 +500,15 @@ size_t stage_bytes_of(int bn, int planes_a, int planes_w, bool pair) {
 // the same formula with their own operand bytes; it was not fitted to them, only checked on whole passes, with pairs / with
 // single CTAs and clusters: gate of 4096 x 1024 102.4 / 108.2 us, of 4096 x 512 47.9 / 49.7, layer 64 x 100 (256, 128)
 // 55.4 / 57.4, 32 x 128 (512, 256) 63.5 / 63.5, 32 x 128 (1024, 512) 114.6 / 114.2.
-SmallShape pick_small(int M, int N, int k_blocks, int planes_a, int planes_w, bool split_a, bool w_stacked) {
+SmallShape pick_small(int M, int N, int k_blocks, int planes_a, int planes_w, bool split_a, bool w_stacked,
+                      const TileScan* scan = nullptr, double* us = nullptr) {
     SmallShape best{0, 0, 0, false};
     double best_t = 0.0;
-    const int m_tiles = (M + BM - 1) / BM, sms = device_sm_count();
+    const int sms = device_sm_count();
     auto consider = [&](int bn, int c, bool pair) {
+        const int seqs = scan ? scan_seqs(scan->T, c) : 0;
+        if (scan && seqs == 0) return;
+        const int m_tiles = scan ? (scan->B + seqs - 1) / seqs : (M + BM - 1) / BM;
         const size_t sb = stage_bytes_of(bn, planes_a, planes_w, pair);
         const int stages = std::min<int>(kSmMaxStages, (int)((kSmSmemMax - 1024) / sb));
         if (stages < 2) return;
@@ -380,16 +523,22 @@ SmallShape pick_small(int M, int N, int k_blocks, int planes_a, int planes_w, bo
             best = {bn, c, stages, pair};
         }
     };
+    if (scan) {   // (the scans are built for 64 columns and clusters of 2 and 4)
+        for (int c = 2; c <= 4 && c <= k_blocks; c *= 2) consider(64, c, false);
+        if (us) *us = best_t;
+        return best;
+    }
     for (int bn = 64; bn <= (w_stacked ? 128 : 256); bn *= 2)
         for (int c = 1; c <= 4 && c <= k_blocks; c *= 2) consider(bn, c, false);
     if (!split_a)
         for (int bn = 128; bn <= 256; bn *= 2) consider(bn, 1, true);
+    if (us) *us = best_t;
     return best;
 }
 
-template <int kBN, int kEpi, bool kSplitA, bool kBf16, bool kPair>
+template <int kBN, int kEpi, bool kSplitA, bool kBf16, bool kPair, int kScanRows = 0>
 int launch_small(const CUtensorMap& ma, const CUtensorMap& mw, const SmallTnArgs& p, int grid, size_t smem, cudaStream_t st) {
-    auto kern = gemm_tc_tn_small_kernel<kBN, kEpi, kSplitA, kBf16, kPair>;
+    auto kern = gemm_tc_tn_small_kernel<kBN, kEpi, kSplitA, kBf16, kPair, kScanRows>;
     if (!set_max_dynamic_smem(reinterpret_cast<const void*>(kern), kSmSmemMax)) return SSM_ERR_CUDA;
     count_launch();
     return launch_dep_cluster(kern, kPair ? 2u : (unsigned)p.cluster, grid, sm_threads(kBN), smem, st, ma, mw, p) ? SSM_OK : SSM_ERR_CUDA;
@@ -400,7 +549,7 @@ int launch_small(const CUtensorMap& ma, const CUtensorMap& mw, const SmallTnArgs
 
 int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st) {
     using namespace tc;
-    const int epi = g.gate_out ? kSmGate : (g.store_f32 && !g.diag ? kSmStore : kSmDiag);
+    const int epi = g.scan ? (g.scan->gA_part ? kSmScanBwd : kSmScanFwd) : g.gate_out ? kSmGate : (g.store_f32 && !g.diag ? kSmStore : kSmDiag);
     if (g.K % BK != 0 || g.N_out % 64 != 0 || g.n_products > 8) return SSM_ERR_SHAPE;
     if (epi == kSmDiag && (!g.diag || !g.skip)) return SSM_ERR_SHAPE;
     if (epi == kSmGate && (!g.skip || !g.skip_bf16)) return SSM_ERR_SHAPE;
@@ -428,14 +577,15 @@ int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st) {
     p.dot_part = g.dot_part, p.gate_out = reinterpret_cast<__nv_bfloat16*>(g.gate_out);
     p.out_bf16 = !g.store_f32, p.skip_bf16 = g.skip_bf16, p.dot_bf16 = g.dot_bf16;
     p.hdr = g.hdr;
-    const SmallShape s = pick_small(g.M, g.N_out, p.k_blocks, p.planes_a, p.planes_w, g.a_f32, p.w_stacked != 0);
+    const SmallShape s = pick_small(g.M, g.N_out, p.k_blocks, p.planes_a, p.planes_w, g.a_f32, p.w_stacked != 0, g.scan);
     if (s.bn == 0) return SSM_ERR_SHAPE;
+    if (g.scan) p.scan = *g.scan, p.seqs = scan_seqs(g.scan->T, s.cluster), p.tile_rows = p.seqs * g.scan->T;
     p.cluster = s.cluster;
     p.stages = s.stages;
     p.stage_bytes = (int)stage_bytes_of(s.bn, p.planes_a, p.planes_w, s.pair);
     p.n_tiles = (g.N_out + s.bn - 1) / s.bn;
     const size_t smem = std::max((size_t)p.stages * p.stage_bytes, (size_t)BM * (s.bn + 4) * 4) + 1024;
-    const int m_tiles = (g.M + BM - 1) / BM, grid = (s.pair ? (m_tiles + 1) / 2 * 2 : m_tiles * p.cluster) * p.n_tiles;
+    const int m_tiles = g.scan ? (g.scan->B + p.seqs - 1) / p.seqs : (g.M + BM - 1) / BM, grid = (s.pair ? (m_tiles + 1) / 2 * 2 : m_tiles * p.cluster) * p.n_tiles;
     if (g.dot_rows) *g.dot_rows = s.pair ? (m_tiles + 1) / 2 * 2 : m_tiles * p.cluster;
     CUtensorMap ma, mw;
     const uint64_t w_rows = (uint64_t)g.N_out * (p.w_stacked ? p.planes_w : 1);
@@ -454,6 +604,17 @@ int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st) {
         if (s.bn == 128) return launch_small<128, EPI, SPLIT, BF, false>(ma, mw, p, grid, smem, st);          \
         return launch_small<256, EPI, SPLIT, BF, false>(ma, mw, p, grid, smem, st);                           \
     } while (0)
+    if (epi == kSmScanBwd) {   // (the gradient is fp32 there)
+        if (!g.a_f32) return SSM_ERR_DTYPE;
+        return s.cluster == 4 ? launch_small<64, kSmScanBwd, true, true, false, scan_rows(4)>(ma, mw, p, grid, smem, st)
+                              : launch_small<64, kSmScanBwd, true, true, false, scan_rows(2)>(ma, mw, p, grid, smem, st);
+    }
+    if (epi == kSmScanFwd && g.a_f32)
+        return s.cluster == 4 ? launch_small<64, kSmScanFwd, true, true, false, scan_rows(4)>(ma, mw, p, grid, smem, st)
+                              : launch_small<64, kSmScanFwd, true, true, false, scan_rows(2)>(ma, mw, p, grid, smem, st);
+    if (epi == kSmScanFwd)
+        return s.cluster == 4 ? launch_small<64, kSmScanFwd, false, true, false, scan_rows(4)>(ma, mw, p, grid, smem, st)
+                              : launch_small<64, kSmScanFwd, false, true, false, scan_rows(2)>(ma, mw, p, grid, smem, st);
     if (epi == kSmGate) SSM_SMALL(kSmGate, false, true);
     if (epi == kSmStore && g.a_f32) SSM_SMALL(kSmStore, true, true);
     if (epi == kSmStore) SSM_SMALL(kSmStore, false, true);
@@ -461,6 +622,21 @@ int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st) {
     if (io_bf16) SSM_SMALL(kSmDiag, false, true);
     return SSM_ERR_SHAPE;   // planes of A with fp32 skip or dot: left to gemm_tc_planes.cu
 #undef SSM_SMALL
+}
+
+// The estimate of the projection on whole sequences (64 columns, clusters) may be 3 us above the best without: what a scan of
+// its own costs in the cheaper direction, the forward pass.  us per forward and backward pass in a graph, apart -> together: 8 x 50 (256, 128) 57.3 -> 49.3, 16 x 100
+// 67.5 -> 57.6, 64 x 16 (256, 256) 66.9 -> 59.5, 8 x 128 (512, 256) 82.1 -> 73.9; at 10 x 100 (512, 256), 20 x 70 (256, 128) and
+// 16 x 64 (1024, 512), where the tiles would need another round, they stay apart.
+bool tc_tile_scan_supported(int B, int T, int H, int P, bool a_bf16) {
+    using namespace tc;
+    if (T < 8 || T > BM || H % BK != 0 || (2 * P) % 64 != 0 || tc_planes_many_tiles(B * T, 2 * P)) return false;
+    TileScan scan{};
+    scan.B = B, scan.T = T;
+    double with = 0.0, without = 0.0;
+    const SmallShape s = pick_small(B * T, 2 * P, H / BK, a_bf16 ? 1 : 3, 3, !a_bf16, false, &scan, &with);
+    pick_small(B * T, 2 * P, H / BK, a_bf16 ? 1 : 3, 3, !a_bf16, false, nullptr, &without);
+    return s.bn != 0 && with <= without + 3.0;
 }
 
 // One partial row of column sums per CTA along M.

@@ -81,6 +81,10 @@ int launch_scan_bwd(int B, int T, int P, const float2* Abar, const float2* Alo, 
                     float2* gAbar, float2* gx0, WsHeader* hdr, void* scratch, cudaStream_t st,
                     const float2** gA_part = nullptr, int* gA_rows = nullptr);
 
+// Where a kernel that scans leaves B rows of P partial gAbar sums in `scratch`, and those brought down to *rows <= kMaxPartialRows.
+float2* scan_partials(void* scratch);
+const float2* reduce_scan_partials(int B, int P, void* scratch, int* rows, cudaStream_t st);
+
 // scan_stream.cu: the scans as TMA-fed streaming kernels (a CTA walks whole sequences; all
 // parallelism over time is inside the CTA).  `ticket`: one int of scratch.  The backward pass
 // leaves B rows of P partial gAbar sums in `part`.
@@ -141,6 +145,19 @@ int gemm_nt_splits(int K, int I, int J);
 void launch_gemm_nt(const GemmNT* g, int n, const SimtDot* dot, cudaStream_t st);
 
 // gemm_tc.cu: bf16 projections on tcgen05 tensor cores (operands by TMA, accumulators in TMEM).
+// Scan of a projection's result in its epilogue (gemm_tc_small.cu): forward, out = x with x_t = keep_t Abar x_{t-1} + acc_t, or with
+// gA_part backward, out = s with s_t = acc_t + c_t, c_{t-1} = keep_t conj(Abar) s_t (c_{T-1} = gxT).
+struct TileScan {
+    int B, T;
+    const float2 *Abar, *Alo;
+    const uint8_t* done;      // [B, T] or NULL
+    const float2 *x0, *gxT;   // [B, P] or NULL
+    float2 *xT, *gx0;         // [B, P] or NULL
+    const float2* x;          // backward: [B, T, P]
+    float2* gA_part;          // backward: [B, P], sums of keep_t s_t conj(x_{t-1})
+};
+// Whether such a projection takes no longer than one without and a scan of its own: few tiles, whole sequences in each.
+bool tc_tile_scan_supported(int B, int T, int H, int P, bool a_bf16);
 struct GemmTcTN {
     // out[m, n] = sum_k A[m, k] * W[n, k];  A bf16 [M, K];  W bf16 packed by pack_params_kernel:
     // [N_out, K], or with split_w [2 * N_out, K] where each group of 256 rows holds the high
@@ -171,6 +188,7 @@ struct GemmTcTN {
     void* a_planes_out = nullptr;        // ... and, if asked for, stored [M, 3K] for a later kernel
     bool skip_bf16 = true, dot_bf16 = true;   // types of skip and dot; with diag and store_f32 the result is fp32
     const float* add = nullptr;          // fp32 [M, N_out], added to acc + diag * skip
+    const TileScan* scan = nullptr;
 };
 bool tc_tn_supported(int M, int N_out, int K, bool split_w);
 int launch_gemm_tc_tn_small(const GemmTcTN& g, cudaStream_t st);

@@ -261,11 +261,13 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
                 e = cfma2(a, al, e, v);
             }
         } else {
-            for (int t = t1 - 1; t >= t0; --t) {
-                const float2 st = cadd(f2(vq + t * o.xp), e);
-                if (flags[t]) e = zero, cut = true;
-                else e = cfma2(a, al, st, zero);
+            e = cadd(f2(vq + (t1 - 1) * o.xp), e);   // (the state's gradient s; conj(Abar) s, which it hands on, is rounded once, at the end)
+            cut = cut || flags[t1 - 1];
+            for (int t = t1 - 2; t >= t0; --t) {
+                e = cfma2(a, al, flags[t + 1] ? zero : e, f2(vq + t * o.xp));
+                cut = cut || flags[t];
             }
+            e = flags[t0] ? zero : cfma2(a, al, e, zero);
         }
         agg[tid] = e;
         sums[tid] = cut ? 1.f : 0.f;
@@ -303,17 +305,16 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
         } else {
             const float* xq = x + 2 * q;
             for (int t = t1 - 1; t >= t0; --t) {
-                const float2 st = cadd(f2(vq + t * o.xp), c);
-                *reinterpret_cast<float2*>(vq + t * o.xp) = st;
-                share(t, cfma2(gamma, gammal, st, zero));
-                if (flags[t]) {
-                    c = zero;
-                } else {
+                const float2 v = f2(vq + t * o.xp);
+                c = t == t1 - 1 ? cadd(v, c) : cfma2(a, al, flags[t + 1] ? zero : c, v);
+                *reinterpret_cast<float2*>(vq + t * o.xp) = c;
+                share(t, cfma2(gamma, gammal, c, zero));
+                if (!flags[t]) {
                     const float2 before = t > 0 ? f2(xq + (t - 1) * o.xp) : (p.x0 ? p.x0[(size_t)b * P + p0 + q] : zero);
-                    gA = cfma(st, cconj(before), gA);
-                    c = cfma2(a, al, st, zero);
+                    gA = cfma(c, cconj(before), gA);
                 }
             }
+            c = flags[t0] ? zero : cfma2(a, al, c, zero);
             if (t0 == 0 && p.gx0) p.gx0[(size_t)b * P + p0 + q] = c;
         }
     }

@@ -363,6 +363,13 @@ int launch_scan_bwd(int B, int T, int P, const float2* Abar, const float2* Alo, 
     return SSM_OK;
 }
 
+float2* scan_partials(void* scratch) { return reinterpret_cast<float2*>((char*)scratch + plan_scan(1, 1).off_part); }
+
+const float2* reduce_scan_partials(int B, int P, void* scratch, int* rows, cudaStream_t st) {
+    float* tmp = reinterpret_cast<float*>((char*)scratch + plan_scan(B, P).off_tmp);
+    return reinterpret_cast<const float2*>(launch_reduce_rows((float*)scan_partials(scratch), B, 2 * P, tmp, kMaxPartialRows, rows, st));
+}
+
 int launch_gemm_scan_bwd_part(GemmScanBwd g, void* scratch, const float2** gA_part_out, int* gA_rows, cudaStream_t st) {
     const ScanPlan s = plan_scan(g.B, g.P, 2);
     char* base = (char*)scratch;
