@@ -226,13 +226,13 @@ __device__ __forceinline__ void add_column_dots(uint32_t a, uint32_t b, int lane
 //          With next_m0 >= 0 (the tile this warp drains next) a buffer that has been read is refilled with the next
 //          tile's first slabs, so that they have arrived when that tile starts; *skip_ahead says whether the
 //          tile now starting found its first slabs requested already.
-template <int kEpi, bool kSplitW>
+template <int kEpi, bool kSplitW, int kCols = BN>
 __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, const CUtensorMap* tmOut,
                                               const CUtensorMap* tmSkip, const CUtensorMap* tmGate, int warp, int lane,
                                               int m0, int n_out0, int acc, uint32_t acc_phase, uint32_t tmem_base,
                                               uint32_t& skip_phase, int next_m0 = -1, int next_n_out0 = 0,
                                               bool* skip_ahead = nullptr) {
-    constexpr int kOutCols = kSplitW ? BN / 2 : BN;
+    constexpr int kOutCols = kSplitW ? BN / 2 : kCols;
     const int q = warp & 3;             // TMEM lane quarter this warp may read
     const int half = (warp - 2) >> 2;   // which half of the tile's columns this warp drains
     const int row0 = m0 + q * 32;       // first of this warp's 32 rows
@@ -362,7 +362,7 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
         for (int j = 0; j < 4; ++j) sk[j] = *reinterpret_cast<const uint4*>(skb + b * 2048 + lane * 64 + ((j ^ swz) << 4));
         if (kDot) {
             const uint32_t dots = smem_u32(skb + b * 2048);
-            float* acc_cols = s.diag + kDotMaxN + (size_t)w * (kDotMaxN / 2) + (n_out0 / BN) * (BN / 2) + sl * 32;
+            float* acc_cols = s.diag + kDotMaxN + (size_t)w * (kDotMaxN / 2) + (n_out0 / kCols) * (kCols / 2) + sl * 32;
             add_column_dots(dots, dots + 4096, lane, acc_cols);   // (rows outside M were read as zero)
         }
         tmem_ld_wait();
@@ -426,19 +426,22 @@ constexpr int kPairStageBytes = kABytes + kBBytes / 2;
 #define SSM_PAIR_STAGES_BF16_EPILOGUE 4
 #endif
 __host__ __device__ constexpr int pair_stages(int epi) { return epi == 3 ? 3 : (epi == 1 ? SSM_PAIR_STAGES_BF16_EPILOGUE : kPairStages); }
-constexpr size_t pair_smem_bytes(int epi) {
-    return (size_t)pair_stages(epi) * kPairStageBytes + tn_staging_bytes(epi) + tn_skip_bytes(epi) + tn_diag_bytes(epi) + 1024 +
+__host__ __device__ constexpr int pair_stage_bytes(int cols) { return kABytes + cols / 2 * BK * 2; }
+constexpr size_t pair_smem_bytes(int epi, int cols = BN) {
+    return (size_t)pair_stages(epi) * pair_stage_bytes(cols) + tn_staging_bytes(epi) + tn_skip_bytes(epi) + tn_diag_bytes(epi) + 1024 +
            256;
 }
 
-template <int kEpi, bool kSplitW>
+// kCols: columns of a tile, BN, or BN / 2 for the bf16 epilogues where wider tiles leave pairs without work (narrow_tiles).
+template <int kEpi, bool kSplitW, int kCols = BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTnThreads, 1)
 gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmWh,
                        const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ CUtensorMap tmSkip,
                        const __grid_constant__ CUtensorMap tmGate, TnParams p) {
     extern __shared__ uint8_t smem_raw[];
     constexpr int kSt = pair_stages(kEpi);
-    const Smem s = carve_smem(smem_raw, kSt, tn_staging_bytes(kEpi), tn_diag_bytes(kEpi), kPairStageBytes,
+    constexpr int kStBytes = pair_stage_bytes(kCols);
+    const Smem s = carve_smem(smem_raw, kSt, tn_staging_bytes(kEpi), tn_diag_bytes(kEpi), kStBytes,
                               tn_skip_bytes(kEpi));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
@@ -466,7 +469,7 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     grid_dep_wait();   // the set-up above ran beside the end of the kernel before this one
     grid_dep_launch();
     if (kEpi == 1 || kEpi == 3)   // (zero where the last tile reaches past the output's columns)
-        for (int i = threadIdx.x; i < p.n_tiles * BN; i += kTnThreads) s.diag[i] = i < p.ldo ? p.diag[i] : 0.f;
+        for (int i = threadIdx.x; i < p.n_tiles * kCols; i += kTnThreads) s.diag[i] = i < p.ldo ? p.diag[i] : 0.f;
     if (kEpi == 3)   // the epilogue warps' column sums start at zero
         for (int i = threadIdx.x; i < kTnEpiWarps * (kDotMaxN / 2); i += kTnThreads) s.diag[kDotMaxN + i] = 0.f;
     if (kEpi == 1 || kEpi == 3) __syncthreads();
@@ -474,7 +477,7 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     const int m_pairs = (p.M + 2 * BM - 1) / (2 * BM);
     const int total = m_pairs * p.n_tiles;
-    constexpr int kOutCols = kSplitW ? BN / 2 : BN;
+    constexpr int kOutCols = kSplitW ? BN / 2 : kCols;
 
     if (warp == 0) {
         if (elect_one()) {
@@ -497,13 +500,13 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         prefetch_a(pair);
         for (int tile = pair; tile < total && ok; tile += npairs) {
             const int m0 = (tile / p.n_tiles) * (2 * BM) + (int)rank * BM;
-            const int n0 = (tile % p.n_tiles) * BN + (int)rank * (BN / 2);
+            const int n0 = (tile % p.n_tiles) * kCols + (int)rank * (kCols / 2);
             prefetch_a(tile + npairs);
             for (int kb = 0; kb < p.k_blocks; ++kb) {
                 if (!(ok = mbar_wait_warp(s.empty(stage), phase ^ 1u, s.abort_flag))) break;
                 if (elect_one()) {
-                    if (rank == 0) mbar_expect_tx(s.full(stage), 2 * kPairStageBytes);
-                    const uint32_t a_dst = smem_u32(s.tiles + (size_t)stage * kPairStageBytes);
+                    if (rank == 0) mbar_expect_tx(s.full(stage), 2 * kStBytes);
+                    const uint32_t a_dst = smem_u32(s.tiles + (size_t)stage * kStBytes);
                     tma_load_2d_pair(a_dst, &tmA, leader_full0 + 8u * stage, p.a_col(kb), m0);
                     tma_load_2d_pair(a_dst + kABytes, &tmWh, leader_full0 + 8u * stage, p.w_col(kb), n0);
                 }
@@ -515,7 +518,7 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         }
     } else if (warp == 1) {
         if (rank == 0) {
-            constexpr uint32_t idesc = instr_desc(2 * BM, BN, 0, 0);
+            constexpr uint32_t idesc = instr_desc(2 * BM, kCols, 0, 0);
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
             bool ok = true;
@@ -526,7 +529,7 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                 for (int kb = 0; kb < p.k_blocks; ++kb) {
                     if (!(ok = mbar_wait_warp(s.full(stage), phase, s.abort_flag))) break;
                     tc_fence_after();
-                    const uint32_t a_addr = smem_u32(s.tiles + (size_t)stage * kPairStageBytes);
+                    const uint32_t a_addr = smem_u32(s.tiles + (size_t)stage * kStBytes);
                     const uint64_t adesc = smem_desc_kmajor(a_addr);
                     const uint64_t bdesc = smem_desc_kmajor(a_addr + kABytes);
                     if (elect_one()) {
@@ -556,7 +559,7 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             const int m0 = (tile / p.n_tiles) * (2 * BM) + (int)rank * BM, n_out0 = (tile % p.n_tiles) * kOutCols;
             const int nxt = tile + npairs;
             const int next_m0 = nxt < total ? (nxt / p.n_tiles) * (2 * BM) + (int)rank * BM : -1;
-            if (!(ok = tn_drain_tile<kEpi, kSplitW>(s, p, &tmOut, &tmSkip, &tmGate, warp, lane, m0, n_out0, acc, acc_phase, tmem_base,
+            if (!(ok = tn_drain_tile<kEpi, kSplitW, kCols>(s, p, &tmOut, &tmSkip, &tmGate, warp, lane, m0, n_out0, acc, acc_phase, tmem_base,
                                                     skip_phase, next_m0, nxt < total ? (nxt % p.n_tiles) * kOutCols : 0, &skip_ahead)))
                 break;
             tc_fence_before();
@@ -570,7 +573,7 @@ gemm_tc_tn_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             asm volatile("bar.sync 1, %0;" ::"n"(32 * kTnEpiWarps) : "memory");
             const float* sums = s.diag + kDotMaxN;
             for (int n = threadIdx.x - 64; n < p.ldo; n += 32 * kTnEpiWarps) {
-                const int half = (n % BN) / (BN / 2), idx = (n / BN) * (BN / 2) + n % (BN / 2);
+                const int half = (n % kCols) / (kCols / 2), idx = (n / kCols) * (kCols / 2) + n % (kCols / 2);
                 float t = 0.f;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) t += sums[(size_t)(4 * half + q) * (kDotMaxN / 2) + idx];
@@ -2033,6 +2036,19 @@ static int pair_tiles_of(int M, int n_tiles) { return ((M + 2 * tc::BM - 1) / (2
 // Six products of planes, whose planes the few-tile kernel loads once, stay there at every size.
 enum { kEpiStore = 0, kEpiDiag = 1, kEpiGate = 2, kEpiDot = 3 };
 static int epi_of(const GemmTcTN& g) { return g.gate_out ? kEpiGate : (g.store_f32 && !g.diag ? kEpiStore : (g.dot ? kEpiDot : kEpiDiag)); }
+// Whether the kernel on pairs takes tiles of 128 columns instead of 256 (acc + diag * skip): where the shorter last round, or a
+// last tile of 128 columns that would be half empty, is worth reading A twice as often.  A round of narrow tiles takes
+// 0.7 of a wide one, 0.62 with the column sums, whose epilogue is the longer part.  us incl. 4 of events, wide / narrow, rows x
+// columns: y 4100 x 512 14.8 / 13.1, 9600 x 384 17.1 / 14.7, 30000 x 384 25.0 / 24.8, 12800 x 512 18.9 / 20.6; du 9600 x 384 20.9 / 16.8,
+// 30000 x 384 35.0 / 31.2, 64000 x 384 51.4 / 47.5, 12800 x 512 24.5 / 23.0, 30000 x 512 41.1 / 44.1.  Contractions above 512: never
+// (6400 x 1024 x 1024 25.0 / 27.1 and 31.0 / 33.6).
+static bool narrow_tiles(const GemmTcTN& g) {
+    const int epi = epi_of(g);
+    if ((epi != kEpiDiag && epi != kEpiDot) || g.n_products > 0 || g.K > 512) return false;
+    const int pairs = std::max(1, tc::sm_count() / 2);
+    auto rounds = [&](int cols) { return (pair_tiles_of(g.M, (g.N_out + cols - 1) / cols) + pairs - 1) / pairs; };
+    return rounds(tc::BN / 2) * (epi == kEpiDot ? 0.62 : 0.7) < rounds(tc::BN);
+}
 static bool use_pairs(const GemmTcTN& g) {
     if (g.n_products > 3 || g.a_f32 || g.scan || g.add || (g.diag && g.store_f32)) return false;
     const int out_cols = g.split_w ? tc::BN / 2 : tc::BN, tiles = pair_tiles_of(g.M, (g.N_out + out_cols - 1) / out_cols);
@@ -2043,7 +2059,8 @@ static bool use_pairs(const GemmTcTN& g) {
     // 179.6 / 181.0, 32768 x 1024 232.0 / 235.5 and 451.1 / 454.6; 16384 x 512 (128 tiles) 58.7 / 60.8 and 99.7 / 94.4,
     // 32768 x 512 105.1 / 100.9 and 185.4 / 179.9, 262144 x 512 736.6 / 697.2 and 1395 / 1300.
     if (g.n_products > 0) return tiles >= (g.K >= 1024 ? 600 : (epi == kEpiGate ? 160 : 80));
-    return tiles >= (epi == kEpiDiag ? 32 : 40);
+    // (in narrow tiles that run in one round already from 24: 2000 x 768 14.7 us on the few-tile kernel, 12.7)
+    return tiles >= (epi == kEpiDiag ? (narrow_tiles(g) ? 24 : 32) : 40);
 }
 // Whether acc + diag * skip also leaves the column sums of skip * dot: not for many rows of very wide outputs, which the
 // pair kernel takes faster without than the few-tile kernel with them.
@@ -2054,9 +2071,10 @@ int tc_tn_dot_max_rows(int M) { return std::max(tc_tn_small_max_dot_rows(M), 2 *
 int launch_gemm_tc_tn(const GemmTcTN& g, cudaStream_t st) {
     using namespace tc;
     if (!use_pairs(g)) return launch_gemm_tc_tn_small(g, st);
-    const int out_cols = g.split_w ? BN / 2 : BN;
-    const int n_tiles = (g.N_out + out_cols - 1) / out_cols;
     const int epi = epi_of(g);
+    const bool narrow = narrow_tiles(g);
+    const int out_cols = g.split_w || narrow ? BN / 2 : BN;
+    const int n_tiles = (g.N_out + out_cols - 1) / out_cols;
     if ((epi == 1 || epi == 3) && (g.split_w || !g.diag || !g.skip)) return SSM_ERR_SHAPE;
     if (epi == 3 && (!g.dot_part || !g.dot_rows)) return SSM_ERR_SHAPE;
     if (epi == 2 && (g.split_w || !g.store_f32 || !g.skip)) return SSM_ERR_SHAPE;
@@ -2086,25 +2104,27 @@ int launch_gemm_tc_tn(const GemmTcTN& g, cudaStream_t st) {
     // rows of the packed weight matrix that exist (tiles may reach past them: those rows read as zero)
     const uint64_t w_rows = g.split_w ? (uint64_t)2 * g.N_out : (uint64_t)g.N_out;
     bool ok = true;
-    if (!make_map(&mw, g.W, w_rows, w_cols, BK, BN / 2)) return SSM_ERR_CUDA;
+    if (!make_map(&mw, g.W, w_rows, w_cols, BK, narrow ? BN / 4 : BN / 2)) return SSM_ERR_CUDA;
     count_launch();
     // The kernel is persistent: its grid is the number of CTA pairs the device can hold at once
     // (not every SM has a partner that a cluster may use).
-#define SSM_LAUNCH_PAIR(EPI, SPLIT)                                                                        \
+#define SSM_LAUNCH_PAIR(EPI, SPLIT, COLS)                                                                  \
 do {                                                                                                   \
-    auto kern = gemm_tc_tn_pair_kernel<EPI, SPLIT>;                                                    \
-    constexpr size_t smem = pair_smem_bytes(EPI);                                                      \
+    auto kern = gemm_tc_tn_pair_kernel<EPI, SPLIT, COLS>;                                              \
+    constexpr size_t smem = pair_smem_bytes(EPI, COLS);                                                \
     ok = set_smem(kern, smem);                                                                         \
     const int pairs = ok ? resident_pairs(reinterpret_cast<const void*>(kern), smem, kTnThreads) : 0;              \
     ok = ok && pairs > 0;                                                                              \
     if (ok) launch_dep(kern, 2 * min(pairs, pair_tiles), kTnThreads, smem, st, ma, mw, mo, ms, mg, p);         \
     if (ok && g.dot_rows) *g.dot_rows = 2 * min(pairs, pair_tiles);                                    \
 } while (0)
-    if (epi == 3) SSM_LAUNCH_PAIR(3, false);
-    else if (epi == 2) SSM_LAUNCH_PAIR(2, false);
-    else if (epi == 1) SSM_LAUNCH_PAIR(1, false);
-    else if (g.split_w) SSM_LAUNCH_PAIR(0, true);
-    else SSM_LAUNCH_PAIR(0, false);
+    if (epi == 3 && narrow) SSM_LAUNCH_PAIR(3, false, BN / 2);
+    else if (epi == 3) SSM_LAUNCH_PAIR(3, false, BN);
+    else if (epi == 2) SSM_LAUNCH_PAIR(2, false, BN);
+    else if (epi == 1 && narrow) SSM_LAUNCH_PAIR(1, false, BN / 2);
+    else if (epi == 1) SSM_LAUNCH_PAIR(1, false, BN);
+    else if (g.split_w) SSM_LAUNCH_PAIR(0, true, BN);
+    else SSM_LAUNCH_PAIR(0, false, BN);
 #undef SSM_LAUNCH_PAIR
     return ok ? SSM_OK : SSM_ERR_CUDA;
 }
