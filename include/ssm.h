@@ -153,7 +153,8 @@ size_t ssm_layer_workspace_bytes(const ssm_shape* shape);
  * (host only, nothing is launched; at most len - 1 characters and a terminating 0).  The text is
  * "projections=<tensor-cores|tensor-cores-planes|cuda-cores> scans=<fused|separate>", and for fused scans
  * " chain_states=<64|32> time_pairs=<0|1>": the states a CTA pair scans together, and whether its two CTAs
- * share one sequence (few long sequences) or take two.  Returns SSM_OK, SSM_ERR_NULL (buf NULL or len 0)
+ * share one sequence (few long sequences) or take two.  (Scans that run in the epilogue of an fp32 layer's few-tile
+ * projections, and small layers whose passes are one kernel each, read as separate.)  Returns SSM_OK, SSM_ERR_NULL (buf NULL or len 0)
  * or the shape's error. */
 int ssm_layer_plan_string(const ssm_shape* shape, char* buf, size_t len);
 int ssm_layer_fwd(const ssm_shape* shape, const ssm_c64* Lambda /*[P]*/, const float* Delta /*[P]*/,

@@ -17,7 +17,7 @@ namespace {
 //  * plane path (fp32 I/O and tile-sized H, P with enough rows): the same projections on tcgen05 as sums
 //    of products of bf16 planes (three planes per fp32 value: exact), fp32 states, scans as on the
 //    CUDA-core path.
-//  * small layers off the tensor cores: each pass in one kernel, a CTA per sequence; fp32 x is all that is kept.
+//  * small layers off the tensor cores: each pass in one kernel, a cluster per sequence; fp32 x is all that is kept.
 struct LayerPlan {
     bool tc;
     bool planes;
