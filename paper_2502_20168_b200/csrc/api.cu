@@ -60,8 +60,7 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true, bool step = false
     p.tc = allow_tc && s.io_dtype == SSM_BF16 && tc_tn_supported((int)BT, P2, s.H, true) &&
            tc_tn_supported((int)BT, s.H, P2, false) && tc_nt_supported(s.H, P2);
     p.planes = !p.tc && s.io_dtype == SSM_F32 && planes_supported(s, step);
-    p.small = allow_tc && !step && !p.tc && !p.planes && layer_small_cluster(s.B, s.T, s.H, s.P) > 0;
-    p.splits = p.small ? s.B : p.tc ? tc_nt_splits((int)BT, s.H, P2) : (p.planes ? tc_nt_planes_splits((int)BT, s.H, P2, 2) : gemm_nt_splits((int)BT, s.H, P2));
+    p.splits = p.tc ? tc_nt_splits((int)BT, s.H, P2) : (p.planes ? tc_nt_planes_splits((int)BT, s.H, P2, 2) : gemm_nt_splits((int)BT, s.H, P2));
     p.hdr = take(off, sizeof(WsHeader));
     p.Abar = take(off, (size_t)s.P * 8);
     p.Alo = take(off, (size_t)s.P * 8);
@@ -100,6 +99,23 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true, bool step = false
         p.dot = take(off, std::max(dot_columns_tmp_floats((int)BT, s.H), fused) * 4);
     }
     p.total = off;
+    if (allow_tc && !step && !p.tc && !p.planes && layer_small_cluster(s.B, s.T, s.H, s.P) > 0) {
+        // The passes in one kernel keep x, and with several sequences a slice of both weight gradients for each of them.  They are
+        // taken where that fits what the separate kernels need, so that no batch needs more than a larger one (in a layout of their own
+        // 32 x 10 (184, 128) wanted 13.8 MB, 33 x 10 and the separate kernels 4.0).
+        LayerPlan q{};
+        off = 0;
+        q.small = true;
+        q.splits = s.B;
+        q.hdr = take(off, sizeof(WsHeader));
+        q.xs = take(off, BT * s.P * 8);
+        q.gg = take(off, (size_t)gamma_part_rows(s.H) * s.P * 8);
+        q.scan = take(off, (size_t)s.B * s.P * 8);   // gAbar of every sequence
+        q.dot = take(off, (size_t)s.B * s.H * 4);
+        q.part = take(off, s.B > 1 ? (size_t)2 * q.splits * 2 * PH * 4 : 0);
+        q.total = p.total;
+        if (off <= q.total) return q;
+    }
     return p;
 }
 
