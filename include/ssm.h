@@ -151,10 +151,11 @@ int ssm_check_static(void* stream);
 size_t ssm_layer_workspace_bytes(const ssm_shape* shape);
 /* Which kernels ssm_layer_fwd / ssm_layer_bwd take for a shape on the current device, as text in buf
  * (host only, nothing is launched; at most len - 1 characters and a terminating 0).  The text is
- * "projections=<tensor-cores|tensor-cores-planes|cuda-cores> scans=<fused|separate>", and for fused scans
- * " chain_states=<64|32> time_pairs=<0|1>": the states a CTA pair scans together, and whether its two CTAs
- * share one sequence (few long sequences) or take two.  (Scans that run in the epilogue of an fp32 layer's few-tile
- * projections, and small layers whose passes are one kernel each, read as separate.)  Returns SSM_OK, SSM_ERR_NULL (buf NULL or len 0)
+ * "projections=<tensor-cores|tensor-cores-planes|cuda-cores> scans=<fused|in-epilogue|one-kernel|separate>": scans in one
+ * persistent kernel with the input projection, in the epilogue of an fp32 layer's few-tile projection, a small layer's pass
+ * in one kernel altogether, or kernels of their own.  For fused scans " chain_states=<64|32> time_pairs=<0|1>" follows: the states
+ * a CTA pair scans together, and whether its two CTAs share one sequence (few long sequences) or take two.
+ * Returns SSM_OK, SSM_ERR_NULL (buf NULL or len 0)
  * or the shape's error. */
 int ssm_layer_plan_string(const ssm_shape* shape, char* buf, size_t len);
 int ssm_layer_fwd(const ssm_shape* shape, const ssm_c64* Lambda /*[P]*/, const float* Delta /*[P]*/,

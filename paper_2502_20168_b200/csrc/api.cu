@@ -236,11 +236,12 @@ SSM_API int ssm_layer_plan_string(const ssm_shape* shape, char* buf, size_t len)
     const LayerPlan p = plan_layer(s);
     const int group = p.tc ? tc_gemm_scan_group(s.B, s.T, s.H, s.P) : 0;
     const char* proj = p.tc ? "tensor-cores" : (p.planes ? "tensor-cores-planes" : "cuda-cores");
+    const bool in_epilogue = p.planes && tc_tile_scan_supported(s.B, s.T, s.H, s.P, false);
     if (group)
         snprintf(buf, len, "projections=%s scans=fused chain_states=%d time_pairs=%d", proj, group,
                  tc_gemm_scan_time_pairs(s.B, s.T, s.H, s.P) ? 1 : 0);
     else
-        snprintf(buf, len, "projections=%s scans=separate", proj);
+        snprintf(buf, len, "projections=%s scans=%s", proj, p.small ? "one-kernel" : in_epilogue ? "in-epilogue" : "separate");
     return SSM_OK;
 }
 

@@ -71,8 +71,10 @@ def test_layer_plan_names_the_kernels_a_shape_takes(sb):
     """Host logic only (no GPU: the library then plans for 148 SMs, the B200's count): which projections and
     which form of the scans ssm_layer_fwd / ssm_layer_bwd take for the configurations of the benchmark."""
     plan = lambda *a: sb.ssm_layer_plan_string(sb.make_shape(*a))
-    assert plan(1, 64, 32, 16, "f32") == "projections=cuda-cores scans=separate"              # H, P below a tile
-    assert plan(16, 64, 256, 128, "f32") == "projections=tensor-cores-planes scans=separate"   # fp32 I/O
+    assert plan(1, 64, 32, 16, "f32") == "projections=cuda-cores scans=one-kernel"            # H, P below a tile
+    assert plan(33, 64, 32, 16, "f32") == "projections=cuda-cores scans=separate"             # more sequences than clusters
+    assert plan(16, 64, 256, 128, "f32") == "projections=tensor-cores-planes scans=in-epilogue"   # fp32 I/O
+    assert plan(16, 129, 256, 128, "f32") == "projections=tensor-cores-planes scans=separate"     # one step more than a tile
     fused = "projections=tensor-cores scans=fused chain_states=%d time_pairs=%d"
     assert plan(256, 1024, 512, 256, "bf16") == fused % (64, 0)     # the headline workload
     assert plan(4096, 64, 512, 256, "bf16") == fused % (64, 0)      # whole sequences inside a tile

@@ -294,7 +294,8 @@ def test_backward_results_do_not_depend_on_a_kernel_running_beside_it():
 
 
 @pytest.mark.parametrize("B,T,H,P,io", [(16, 1024, 256, 256, "bf16"), (80, 128, 256, 128, "bf16"), (4, 256, 256, 256, "bf16"),
-                                        (16, 64, 256, 128, "f32"), (2, 40, 32, 16, "f32")])
+                                        (16, 64, 256, 128, "f32"), (2, 40, 32, 16, "f32"),
+                                        (5, 129, 256, 128, "f32"), (40, 40, 32, 16, "f32")])
 def test_plan_string_names_the_stages_that_run(B, T, H, P, io):
     """ssm_layer_plan_string against the stages the library's own timers see for the same shape."""
     import torch
@@ -312,3 +313,6 @@ def test_plan_string_names_the_stages_that_run(B, T, H, P, io):
     fused = "scans=fused" in plan
     assert fused == ("gemm_Bu_scan_fwd" in stages) == ("gemm_gx_scan_bwd" in stages), (plan, stages)
     assert fused != ("scan_fwd" in stages), (plan, stages)
+    # scans with their projection inside, and whole passes in one kernel, are timed as scans
+    assert ("scans=separate" in plan) == ("gemm_Bu" in stages) == ("gemm_gx" in stages), (plan, stages)
+    assert ("scans=one-kernel" in plan) == (not fused and "gemm_y" not in stages), (plan, stages)
