@@ -1,6 +1,6 @@
-"""The kernels that take a small layer's pass at once (layer_small.cu) against the oracle: one state per CTA, groups of rows
-that end short, one step, a sequence on the longest row groups, more threads than rows x columns and fewer, clusters of 8
-and of 4 with the most sequences each takes, and one sequence more (which goes to the separate kernels)."""
+"""The kernels that take a small layer's pass at once (layer_small.cu) against the oracle: one state per CTA, one step, the longest
+sequence, more threads than rows x columns and fewer, clusters of 8 and of 4 with the most sequences each takes, groups of 4
+to 17 rows per scanning thread that end full and short; and the shapes just past its limits, which go to the separate kernels."""
 import pytest
 
 from paper_2502_20168_b200 import inputs as I
@@ -8,10 +8,42 @@ from tests.test_gpu_layer_parity import run
 
 pytestmark = pytest.mark.gpu
 
+ONE_KERNEL = [   # rows of a group in brackets where they are not 4
+    ("f32", 1, 1, 16, 8), ("f32", 1, 7, 8, 8), ("bf16", 1, 64, 32, 16), ("f32", 1, 512, 16, 16), ("f32", 1, 512, 8, 8), ("f32", 2, 33, 72, 40),
+    ("bf16", 3, 4, 192, 120), ("f32", 1, 13, 248, 120), ("f32", 14, 65, 24, 104), ("bf16", 32, 50, 48, 32), ("f32", 2, 8, 248, 256),
+    ("f32", 1, 64, 8, 136),      # [5], the last group 4
+    ("f32", 4, 50, 24, 256),     # [7], the last group 1
+    ("f32", 14, 100, 8, 120),    # [6]
+    ("bf16", 20, 128, 32, 64),   # [8]
+    ("f32", 15, 130, 8, 72),     # [10]
+    ("f32", 32, 256, 8, 48),     # [13], the last group 9
+    ("f32", 32, 64, 8, 208),     # [16]
+    ("bf16", 15, 65, 8, 208),    # [17], the last group 14
+]
+SEPARATE = [
+    ("f32", 33, 50, 48, 32),                                                  # sequences
+    ("f32", 1, 500, 40, 24), ("f32", 1, 512, 16, 56), ("f32", 32, 3, 200, 256),   # shared memory
+    ("f32", 1, 513, 8, 8), ("f32", 1, 8, 264, 8), ("f32", 1, 8, 8, 264),      # steps, features, states
+    ("f32", 15, 18, 136, 48),                                                 # workspace: slices of the weight gradients
+]
 
-@pytest.mark.parametrize("io,B,T,H,P", [("f32", 1, 1, 16, 8), ("f32", 1, 7, 8, 8), ("bf16", 1, 64, 32, 16), ("f32", 1, 500, 40, 24),
-                                        ("f32", 1, 512, 16, 56), ("f32", 2, 33, 72, 40), ("bf16", 3, 4, 192, 120), ("f32", 14, 65, 24, 104),
-                                        ("f32", 15, 18, 136, 48), ("bf16", 32, 50, 48, 32), ("f32", 32, 3, 200, 256), ("f32", 33, 50, 48, 32)])
+
+def _run(io, B, T, H, P, states, kernels):
+    from paper_2502_20168_b200 import binding as sb
+    assert sb.ssm_layer_plan_string(sb.make_shape(B, T, H, P, io)) == f"projections=cuda-cores scans={kernels}"
+    before = sb.ssm_launch_count()
+    run(I.Workload("small", B=B, T=T, H=H, P=P, io_dtype=io, p_done=0.05 if states else 0.0, seed=B + T + H), with_x0=states, with_gxT=states)
+    return sb.ssm_launch_count() - before
+
+
+@pytest.mark.parametrize("io,B,T,H,P", ONE_KERNEL)
 @pytest.mark.parametrize("states", [False, True])
 def test_small_layers(io, B, T, H, P, states):
-    run(I.Workload("small", B=B, T=T, H=H, P=P, io_dtype=io, p_done=0.05 if states else 0.0, seed=B + T + H), with_x0=states, with_gxT=states)
+    launches = _run(io, B, T, H, P, states, "one-kernel")
+    assert launches == 2 if B == 1 else launches <= 4, launches   # (several sequences: and the last kernels of the backward pass)
+
+
+@pytest.mark.parametrize("io,B,T,H,P", SEPARATE)
+@pytest.mark.parametrize("states", [False, True])
+def test_past_the_limits(io, B, T, H, P, states):
+    assert _run(io, B, T, H, P, states, "separate") > 4
