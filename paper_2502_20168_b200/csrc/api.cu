@@ -99,7 +99,7 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true, bool step = false
         p.dot = take(off, std::max(dot_columns_tmp_floats((int)BT, s.H), fused) * 4);
     }
     p.total = off;
-    if (allow_tc && !step && !p.tc && !p.planes && layer_small_cluster(s.B, s.T, s.H, s.P) > 0) {
+    if (allow_tc && !step && !p.tc && !p.planes && layer_small_cluster(s.B, s.T, s.H, s.P, s.io_dtype == SSM_BF16) > 0) {
         // The passes in one kernel keep x, and with several sequences a slice of both weight gradients for each of them.  They are
         // taken where that fits what the separate kernels need, so that no batch needs more than a larger one (in a layout of their own
         // 32 x 10 (184, 128) wanted 13.8 MB, 33 x 10 and the separate kernels 4.0).

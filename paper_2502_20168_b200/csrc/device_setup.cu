@@ -1,7 +1,7 @@
 // Per-device, per-kernel set-up that launchers would otherwise repeat on every call.
 #include <map>
 #include <mutex>
-#include <set>
+#include <tuple>
 #include <utility>
 
 #include "common.cuh"
@@ -26,20 +26,38 @@ bool set_max_dynamic_smem(const void* kernel, size_t bytes) {
     return true;
 }
 
-// The same for clusters of 16 CTAs, which a kernel has to ask for.
-bool allow_large_clusters(const void* kernel) {
+// What the device holds depends on the kernel's registers and shared memory and on how its SMs are grouped: asked once.
+int resident_clusters(const void* kernel, int cluster, size_t smem_bytes, int threads) {
     static std::mutex mu;
-    static std::set<std::pair<const void*, int>> done;
+    static std::map<std::tuple<const void*, int, int>, int> cache;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    std::lock_guard<std::mutex> lock(mu);
-    if (done.count({kernel, dev})) return true;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    if (cudaGetDevice(&dev) != cudaSuccess) {
         (void)cudaGetLastError();
-        return false;
+        return -1;
     }
-    done.insert({kernel, dev});
-    return true;
+    std::lock_guard<std::mutex> lock(mu);
+    const auto key = std::make_tuple(kernel, cluster, dev);
+    const auto it = cache.find(key);
+    if (it != cache.end()) return it->second;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(cluster * device_sm_count()), 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem_bytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if ((cluster > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        n = 0;
+    }
+    cache[key] = n;
+    return n;
 }
 
 // Workspace layouts, operand packing order and kernel choices depend on the SM count, so it is

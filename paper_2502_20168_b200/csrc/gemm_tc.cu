@@ -22,8 +22,6 @@
 // that gives up raises a CTA-wide abort flag, the status word of the workspace header is set, tensor
 // memory is released and the kernel returns.
 #include <algorithm>
-#include <map>
-#include <mutex>
 #include <utility>
 
 #include "kernels.h"
@@ -1979,34 +1977,9 @@ gemm_tc_nt_pair_kernel(const __grid_constant__ NtMaps maps, const __grid_constan
 // ---------------------------------------------------------------------------------------------
 static int sm_count() { return device_sm_count(); }
 
-// How many clusters of two CTAs of `kernel` the current device runs at the same time (cached per
-// kernel and device).
+// How many CTA pairs of `kernel` the current device runs at the same time.
 int resident_pairs(const void* kernel, size_t smem_bytes, int threads) {
-    static std::mutex mu;
-    static std::map<std::pair<const void*, int>, int> cache;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = cache.find({kernel, dev});
-    if (it != cache.end()) return it->second;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * (unsigned)sm_count(), 1, 1);
-    cfg.blockDim = dim3((unsigned)threads, 1, 1);
-    cfg.dynamicSmemBytes = smem_bytes;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
-        (void)cudaGetLastError();
-        n = 0;
-    }
-    cache[{kernel, dev}] = n;
-    return n;
+    return std::max(0, resident_clusters(kernel, 2, smem_bytes, threads));
 }
 
 template <typename K>

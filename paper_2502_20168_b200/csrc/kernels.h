@@ -45,7 +45,7 @@ struct GradTail {
 int gamma_part_rows(int H);
 void launch_layer_tail(int H, int P, int splits, int n, const GradTail* tails, int gA_rows, cudaStream_t st);
 
-// layer_small.cu: the passes of a layer of few and narrow sequences, on the CUDA cores, a CTA per sequence.
+// layer_small.cu: the passes of a layer of few and narrow sequences, on the CUDA cores, a cluster of CTAs per sequence.
 struct LayerSmall {
     int B, T, H, P;
     bool bf16;                // u, gy, out
@@ -60,7 +60,7 @@ struct LayerSmall {
     float2 *xT, *gx0;         // [B, P] or NULL
     WsHeader* hdr;
 };
-int layer_small_cluster(int B, int T, int H, int P);   // CTAs per sequence; 0: not taken
+int layer_small_cluster(int B, int T, int H, int P, bool bf16);   // CTAs per sequence; 0: not taken
 int launch_layer_small_fwd(const LayerSmall& g, cudaStream_t st);   // also clears the status word
 // B = 1: all gradients of `tail` are final.  Else part_b and part_c hold B slices, gA_part [B, P] and dD_part [B, H] the rows
 // of partial sums, for launch_layer_tail.

@@ -429,11 +429,31 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
     }
 }
 
+// us per forward and backward pass in a graph, ten launches -> this (B x T, H, P): 1 x 64, 32, 16 30.9 -> 18.2 (eager 36.5 -> 16.2),
+// 1 x 512, 16, 16 41.2 -> 34.9, 4 x 128, 96, 40 47.3 -> 45.3 (123 K multiply-adds a projection and CTA: the limit is 131 K);
+// clusters of 4: 20 x 128, 32, 64 55.4 -> 45.2, 30 x 20, 176, 72 in bf16 67.7 -> 65.7.  Where the clusters do not run in one round:
+// 16 x 128, 64, 64 (clusters of 8) 53.9 -> 73.2, 36 x 64, 64, 64 (of 4) 55.7 -> 58.6.  One CTA per sequence, 148 x 64, 32, 16: 59.6 -> 76.0.
+int ls_cluster(int B, int T, int H, int P) {
+    if (P > kLsThreads || T > 512 || H > 256 || B > 32) return 0;
+    const int c = B <= 14 ? 8 : 4;
+    return (long long)T * H * 2 * P <= (long long)c << 17 && (size_t)LsSmem(T, H, P, c, true).total * 4 <= kLsSmemMax ? c : 0;
+}
+
+// Whether the device runs that many clusters of both passes at the same time (with the most shared memory; no device: a B200 is planned for).
+template <typename IO>
+bool ls_resident(int cluster, int B) {
+    for (const void* kern : {reinterpret_cast<const void*>(layer_small_kernel<IO, false>), reinterpret_cast<const void*>(layer_small_kernel<IO, true>)}) {
+        const int n = set_max_dynamic_smem(kern, kLsSmemMax) ? resident_clusters(kern, cluster, kLsSmemMax, kLsThreads) : -1;
+        if (n >= 0 && n < B) return false;
+    }
+    return true;
+}
+
 template <typename IO, bool kBwd>
 int launch_ls(LsArgs p, int B, cudaStream_t st) {
     auto kern = layer_small_kernel<IO, kBwd>;
     if (!set_max_dynamic_smem(reinterpret_cast<const void*>(kern), kLsSmemMax)) return SSM_ERR_CUDA;
-    p.cluster = layer_small_cluster(B, p.T, p.H, p.P);
+    p.cluster = ls_cluster(B, p.T, p.H, p.P);
     p.single = B == 1;
     count_launch();
     const size_t smem = (size_t)LsSmem(p.T, p.H, p.P, p.cluster, kBwd).total * 4;
@@ -442,14 +462,9 @@ int launch_ls(LsArgs p, int B, cudaStream_t st) {
 
 }  // namespace
 
-// us per forward and backward pass in a graph, ten launches -> this (B x T, H, P): 1 x 64, 32, 16 30.9 -> 18.2 (eager 36.5 -> 16.2),
-// 1 x 512, 16, 16 41.2 -> 34.9, 4 x 128, 96, 40 47.3 -> 45.3 (123 K multiply-adds a projection and CTA: the limit is 131 K);
-// clusters of 4: 20 x 128, 32, 64 55.4 -> 45.2, 30 x 20, 176, 72 in bf16 67.7 -> 65.7.  Where the clusters do not run in one round:
-// 16 x 128, 64, 64 (clusters of 8) 53.9 -> 73.2, 36 x 64, 64, 64 (of 4) 55.7 -> 58.6.  One CTA per sequence, 148 x 64, 32, 16: 59.6 -> 76.0.
-int layer_small_cluster(int B, int T, int H, int P) {
-    if (P > kLsThreads || T > 512 || H > 256 || B > 32) return 0;
-    const int c = B <= 14 ? 8 : 4;
-    return (long long)T * H * 2 * P <= (long long)c << 17 && (size_t)LsSmem(T, H, P, c, true).total * 4 <= kLsSmemMax ? c : 0;
+int layer_small_cluster(int B, int T, int H, int P, bool bf16) {
+    const int c = ls_cluster(B, T, H, P);
+    return c && (bf16 ? ls_resident<__nv_bfloat16>(c, B) : ls_resident<float>(c, B)) ? c : 0;
 }
 
 int launch_layer_small_fwd(const LayerSmall& g, cudaStream_t st) {

@@ -319,13 +319,17 @@ step_half_kernel(StepHalfArgs p) {
 //   fp32 I/O: H = 512: B = 64: 11.6 / 21.9;  H = 1024: B = 32: 18.3 (three kernels: 21.4), B = 48: 26.1 (21.9).
 bool use_step_small(int B, int H, int P) { return (long long)B * std::max(H, 2 * P) <= 32768; }
 
-// CTAs of a cluster that takes a step's columns in one round, or 0: the halves apart.
+static auto step_cluster_kernel(bool f32) { return f32 ? step_small_kernel<true> : step_small_kernel<false>; }
+// CTAs of a cluster that takes a step's columns in one round, or 0: the halves apart.  The clusters have to run in one round, on a device
+// that holds fewer than a B200 as well.
 static int step_small_cluster(const StepCall& g) {
     const int width = std::max(g.H, 2 * g.P), row_groups = (g.B + kSsRows - 1) / kSsRows;
     int c = 1;
     while (c * kSsWarps * kSsCols < width) c *= 2;
     const int most = c <= 8 ? 112 : (c == 16 && g.f32 ? 64 : 0);   // CTAs
-    return row_groups * c <= most ? c : 0;
+    if (row_groups * c > most) return 0;
+    const size_t smem = kSsRows * kSsWarps * kSsCols * 16 * sizeof(float);   // (of the widest)
+    return resident_clusters(reinterpret_cast<const void*>(step_cluster_kernel(g.f32)), c, smem, 32 * kSsWarps) >= row_groups ? c : 0;
 }
 
 static int launch_step_cluster(const StepCall& g, int cluster, cudaStream_t st) {
@@ -337,11 +341,9 @@ static int launch_step_cluster(const StepCall& g, int cluster, cudaStream_t st) 
     p.x_prev = reinterpret_cast<const float*>(g.x_prev), p.x_next = reinterpret_cast<float*>(g.x_next);
     if (g.f32) p.b_pitch = 3 * H, p.b_plane = H, p.c_pitch = 3 * P2, p.c_plane = P2;
     else p.b_pitch = H, p.b_plane = 128 * H, p.c_pitch = P2;
-    auto kern = g.f32 ? step_small_kernel<true> : step_small_kernel<false>;
-    if (cluster > 8 && !allow_large_clusters(reinterpret_cast<const void*>(kern))) return SSM_ERR_CUDA;
     count_launch();
     const unsigned grid = (unsigned)((g.B + kSsRows - 1) / kSsRows * cluster);
-    return launch_dep_cluster(kern, (unsigned)cluster, grid, 32 * kSsWarps, kSsRows * P2 * sizeof(float), st, p) ? SSM_OK : SSM_ERR_CUDA;
+    return launch_dep_cluster(step_cluster_kernel(g.f32), (unsigned)cluster, grid, 32 * kSsWarps, kSsRows * P2 * sizeof(float), st, p) ? SSM_OK : SSM_ERR_CUDA;
 }
 
 int launch_step_small(const StepCall& g, cudaStream_t st) {
