@@ -6,7 +6,8 @@
 // their weight gradients; the scanned states go to the shared memory of all CTAs of the cluster, each of which
 // projects them onto its part of the features.  The weights are used as the caller stores them: gamma, the factor of
 // the discretisation, multiplies the projected inputs and, conjugated, the gradients of the states, so that its
-// double-precision evaluation (its four functions on different warps) runs while the inputs arrive.
+// double-precision evaluation (its four functions on different warps) runs while the inputs arrive.  What of that could leave the
+// range of fp32 where gamma B does not is computed in its order (an overflowed B u) or scaled exactly (gradients where Delta > 1).
 // fp32 throughout; Abar as an fp32 pair, its power over a group's rows and the adjoint of the discretisation
 // evaluated in double.  A single sequence finishes its parameter gradients itself; several leave them as slices for
 // launch_layer_tail.  Bound by latency: one trip to memory, the exponentials, six barriers.  Measured: see layer_small_cluster.
@@ -138,6 +139,10 @@ __device__ __forceinline__ void product_rows(const float* a, int pa, int M, int 
 
 __device__ __forceinline__ float4 f4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float2 f2(const float* p) { return *reinterpret_cast<const float2*>(p); }
+// The smallest power of two above Delta, or 1 for Delta <= 1.
+__device__ __forceinline__ float step_scale(float delta) {
+    return delta > 1.f ? fminf(2.f * __uint_as_float(__float_as_uint(delta) & 0x7f800000u), 0x1p127f) : 1.f;
+}
 __device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
@@ -175,6 +180,7 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
         copy_pairs(wfeat, o.cp, p.Cc + (size_t)h0 * P, P, hc, P);
     }
     for (int i = tid; i < T; i += kLsThreads) flags[i] = p.done ? p.done[(size_t)b * T + i] != 0 : 0;
+    const float any_step = kBwd && tid < P ? p.Delta[tid] : 0.f;   // (P <= kLsThreads)
     for (int q = p0 + (w >> 2) * 32 + lane; q < p0 + pc; q += 32 * (kLsWarps / 4)) {
         const double lr = p.Lambda[q].x, li = p.Lambda[q].y, d = p.Delta[q];
         double* z = parts + 5 * (q - p0);
@@ -184,7 +190,14 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
         else z[4] = exp(lr * d);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
+    const bool long_step = __syncthreads_or(any_step > 1.f);
+    if (kBwd && long_step)   // |gamma| <= Delta (Re Lambda <= 0), so conj(gamma) s may leave the range of s: B takes a power of two of gamma
+        for (int i = tid; i < P * hc; i += kLsThreads) {
+            const int r = i / hc;
+            float2* w2 = reinterpret_cast<float2*>(wfeat + r * o.cp) + (i - r * hc);
+            const float by = step_scale(p.Delta[r]);
+            *w2 = make_float2(by * w2->x, by * w2->y);
+        }
 
     // ---- own states: B u, or g_x = gy conj(C)
     {
@@ -250,12 +263,26 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
         gammal = make_float2((float)(z.gr - (double)gamma.x), (float)(z.gi - (double)gamma.y));
         aR = make_float2(apow[q].x, apow[q].y), aRl = make_float2(apow[q].z, apow[q].w);
         if (kBwd) a = cconj(a), al = cconj(al), aR = cconj(aR), aRl = cconj(aRl), gamma = cconj(gamma), gammal = cconj(gammal);
+        if (kBwd && long_step) {
+            const float by = 1.f / step_scale(p.Delta[p0 + q]);
+            gamma = make_float2(by * gamma.x, by * gamma.y), gammal = make_float2(by * gammal.x, by * gammal.y);
+        }
         const float2* from = kBwd ? p.gxT : p.x0;
         if (cut && from) first = from[(size_t)b * P + p0 + q];
         float2 e = first;
         if (!kBwd) {
             for (int t = t0; t < t1; ++t) {
-                const float2 v = cfma2(gamma, gammal, f2(vq + t * o.xp), zero);
+                const float2 r = f2(vq + t * o.xp);
+                float2 v = cfma2(gamma, gammal, r, zero);
+                if (!isfinite(r.x + r.y)) {   // B u left the range of fp32, which gamma B u need not have done
+                    v = zero;
+#pragma unroll 1
+                    for (int h = 0; h < H; ++h) {
+                        const float2 bg = cfma2(gamma, gammal, f2(wstate + q * o.wp + 2 * h), zero);
+                        v.x = fmaf(u[t * o.hp + h], bg.x, v.x);
+                        v.y = fmaf(u[t * o.hp + h], bg.y, v.y);
+                    }
+                }
                 *reinterpret_cast<float2*>(vq + t * o.xp) = v;
                 if (flags[t]) e = zero, cut = true;
                 e = cfma2(a, al, e, v);

@@ -1,10 +1,12 @@
 """The kernels that take a small layer's pass at once (layer_small.cu) against the oracle: one state per CTA, one step, the longest
 sequence, more threads than rows x columns and fewer, clusters of 8 and of 4 with the most sequences each takes, groups of 4
 to 17 rows per scanning thread that end full and short; and the shapes just past its limits, which go to the separate kernels."""
+import numpy as np
 import pytest
 
 from paper_2502_20168_b200 import inputs as I
 from tests.test_gpu_layer_parity import run
+from tests.util import oracle_layer
 
 pytestmark = pytest.mark.gpu
 
@@ -47,3 +49,41 @@ def test_small_layers(io, B, T, H, P, states):
 @pytest.mark.parametrize("states", [False, True])
 def test_past_the_limits(io, B, T, H, P, states):
     assert _run(io, B, T, H, P, states, "separate") > 4
+
+
+def _close_in_norm(res, ref, tol=1e-5):   # chains of a few dozen fp32 sums: 1e-6
+    for k in ("y", "xT", "du", "dLambda", "dDelta", "dB", "dC", "dD"):
+        assert np.isfinite(res[k]).all(), k
+        assert np.linalg.norm((res[k] - ref[k]).ravel()) <= tol * np.linalg.norm(np.asarray(ref[k]).ravel()), k
+
+
+@pytest.mark.parametrize("B,T,H,P", [(1, 16, 32, 16), (3, 9, 72, 40)])
+def test_range_of_the_projected_inputs(B, T, H, P):
+    """B u leaves the range of fp32, gamma B u and all that follows do not."""
+    from paper_2502_20168_b200 import harness
+    d = I.draw_layer(I.Workload("range", B=B, T=T, H=H, P=P, io_dtype="f32", p_done=0.05, seed=3))
+    d["Delta"] = np.full(P, 1e-3, np.float32)
+    d["Bc"] = (d["Bc"] * np.float32(1e25)).astype(np.complex64)
+    d["u"] = d["u"] * np.float32(5e14)
+    d["Cc"] = (d["Cc"] * np.float32(1e-25)).astype(np.complex64)
+    d["gy"] = d["gy"] * np.float32(1e-2)
+    assert np.abs(np.einsum("bth,ph->btp", d["u"].astype(np.float64), d["Bc"].astype(np.complex128))).max() > 3.5e38
+    _close_in_norm(harness.run_layer(d, "f32"), oracle_layer(d))
+
+
+@pytest.mark.parametrize("B,T,H,P", [(1, 16, 32, 16), (3, 9, 72, 40)])
+def test_range_of_the_states_gradients(B, T, H, P):
+    """Steps longer than 1: conj(gamma) s leaves the range of fp32, s and conj(gamma B) s do not."""
+    from paper_2502_20168_b200 import harness
+    d = I.draw_layer(I.Workload("range", B=B, T=T, H=H, P=P, io_dtype="f32", seed=3))
+    d["Delta"] = np.linspace(0.5, 9.0, P).astype(np.float32)
+    d["Lambda"] = np.linspace(-0.2, -0.01, P).astype(np.complex64)
+    d["Bc"] = (d["Bc"] * np.float32(1e-20)).astype(np.complex64)
+    d["u"] = d["u"] * np.float32(1e-10)
+    d["gy"] = d["gy"] * np.float32(3e37)
+    d["D"] = d["D"] * np.float32(1e-20)
+    ref = oracle_layer(d)
+    Abar = np.exp(d["Lambda"].astype(np.complex128) * d["Delta"])
+    first = np.abs(ref["dx0"] / Abar.conj())   # s of the first step
+    assert first.max() < 3.4e38 < (first * np.abs((Abar - 1) / d["Lambda"])).max()
+    _close_in_norm(harness.run_layer(d, "f32"), ref)
