@@ -21,7 +21,7 @@ namespace {
 struct LayerPlan {
     bool tc;
     bool planes;
-    bool small;
+    bool small, slices;   // slices: of the weight gradients, by the small layer's kernel
     int splits;
     size_t hdr, Abar, Alo, Apow, W0, W1, W2, W3, f32buf, xs, gs, gAbar, gg, scan, part, dot, total;
     size_t u3, gy3, x3, s3;   // plane path: planes of u, gy, x, s for the weight gradients
@@ -100,21 +100,25 @@ LayerPlan plan_layer(const ssm_shape& s, bool allow_tc = true, bool step = false
     }
     p.total = off;
     if (allow_tc && !step && !p.tc && !p.planes && layer_small_cluster(s.B, s.T, s.H, s.P, s.io_dtype == SSM_BF16) > 0) {
-        // The passes in one kernel keep x, and with several sequences a slice of both weight gradients for each of them.  They are
-        // taken where that fits what the separate kernels need, so that no batch needs more than a larger one (in a layout of their own
-        // 32 x 10 (184, 128) wanted 13.8 MB, 33 x 10 and the separate kernels 4.0).
+        // The passes in one kernel keep x, and with several sequences a slice of both weight gradients for each of them where that
+        // fits what the separate kernels need, so that no batch needs more than a larger one (32 x 10 (184, 128) would want
+        // 13.8 MB, 33 x 10 and the separate kernels 4.0).  Otherwise s, which the separate kernels' products take.
         LayerPlan q{};
-        off = 0;
-        q.small = true;
-        q.splits = s.B;
-        q.hdr = take(off, sizeof(WsHeader));
-        q.xs = take(off, BT * s.P * 8);
-        q.gg = take(off, (size_t)gamma_part_rows(s.H) * s.P * 8);
-        q.scan = take(off, (size_t)s.B * s.P * 8);   // gAbar of every sequence
-        q.dot = take(off, (size_t)s.B * s.H * 4);
-        q.part = take(off, s.B > 1 ? (size_t)2 * q.splits * 2 * PH * 4 : 0);
-        q.total = p.total;
-        if (off <= q.total) return q;
+        for (const bool slices : {true, false}) {
+            off = 0;
+            q.small = true;
+            q.slices = slices;
+            q.splits = slices ? s.B : p.splits;
+            q.hdr = take(off, sizeof(WsHeader));
+            q.xs = take(off, BT * s.P * 8);
+            q.gs = take(off, slices ? 0 : BT * s.P * 8);
+            q.gg = take(off, (size_t)gamma_part_rows(s.H) * s.P * 8);
+            q.scan = take(off, (size_t)s.B * s.P * 8);   // gAbar of every sequence
+            q.dot = take(off, (size_t)s.B * s.H * 4);
+            q.part = take(off, s.B > 1 ? (size_t)2 * q.splits * 2 * PH * 4 : 0);
+            q.total = p.total;
+            if (off <= q.total) return q;
+        }
     }
     return p;
 }
@@ -792,7 +796,16 @@ SSM_API int ssm_layer_bwd(const ssm_shape* shape, const ssm_c64* Lambda, const f
             const LayerSmall g{s.B, s.T, s.H, s.P, s.io_dtype == SSM_BF16, (const float2*)Lambda, Delta, (const float2*)Bc,
                                (const float2*)Cc, D, u, done, (const float2*)x0, (const float2*)gxT, gy, at<float2>(ws, p.xs), du, nullptr,
                                (float2*)dx0, hdr};
-            if (int rc = launch_layer_small_bwd(g, left.tail, at<float2>(ws, p.scan), at<float>(ws, p.dot), st)) return rc;
+            if (int rc = launch_layer_small_bwd(g, left.tail, p.slices ? nullptr : at<float2>(ws, p.gs), at<float2>(ws, p.scan), at<float>(ws, p.dot), st))
+                return rc;
+        }
+        if (!p.slices) {
+            StageTimer tm("gemm_gBbar_gC", st);
+            const int BT = s.B * s.T, P2 = 2 * s.P;
+            const bool b = s.io_dtype == SSM_BF16;
+            const GemmNT g[2] = {{u, b, s.H, at<float>(ws, p.gs), P2, BT, p.splits, const_cast<float*>(left.tail.part_b)},
+                                 {gy, b, s.H, at<float>(ws, p.xs), P2, BT, p.splits, const_cast<float*>(left.tail.part_c)}};
+            launch_gemm_nt(g, 2, nullptr, st);
         }
         if (s.B > 1) return layer_bwd_tail(s, p, 1, &left, hdr, st);
         SSM_RETURN_IF_CUDA_ERROR();

@@ -62,9 +62,9 @@ struct LayerSmall {
 };
 int layer_small_cluster(int B, int T, int H, int P, bool bf16);   // CTAs per sequence; 0: not taken
 int launch_layer_small_fwd(const LayerSmall& g, cudaStream_t st);   // also clears the status word
-// B = 1: all gradients of `tail` are final.  Else part_b and part_c hold B slices, gA_part [B, P] and dD_part [B, H] the rows
-// of partial sums, for launch_layer_tail.
-int launch_layer_small_bwd(const LayerSmall& g, const GradTail& tail, float2* gA_part, float* dD_part, cudaStream_t st);
+// B = 1: all gradients of `tail` are final.  Else gA_part [B, P] and dD_part [B, H] hold the rows of partial sums for
+// launch_layer_tail, and part_b and part_c B slices, or with s (not NULL) the gradients of the states [B, T, P] are there instead.
+int launch_layer_small_bwd(const LayerSmall& g, const GradTail& tail, float2* s, float2* gA_part, float* dD_part, cudaStream_t st);
 
 // scan.cu
 // Scratch the scans need for a [B,T,P] problem: a work counter and the partial sums of gAbar.

@@ -10,7 +10,7 @@
 // range of fp32 where gamma B does not is computed in its order (an overflowed B u) or scaled exactly (gradients where Delta > 1).
 // fp32 throughout; Abar as an fp32 pair, its power over a group's rows and the adjoint of the discretisation
 // evaluated in double.  A single sequence finishes its parameter gradients itself; several leave them as slices for
-// launch_layer_tail.  Bound by latency: one trip to memory, the exponentials, six barriers.  Measured: see layer_small_cluster.
+// launch_layer_tail, or s for the products of the separate kernels where the slices would need more room than those.  Bound by latency: one trip to memory, the exponentials, six barriers.  Measured: see layer_small_cluster.
 #include <type_traits>
 
 #include "kernels.h"
@@ -76,7 +76,8 @@ struct LsArgs {
     float2* x;        // [B, T, P]: kept for the backward pass
     void* out;        // y or du
     float2 *xT, *gx0;
-    float2 *part_b, *part_c;  // [B, H, P]
+    float2 *part_b, *part_c;  // [B, H, P], or with s
+    float2* s;                // [B, T, P]: the weight gradients are left to others
     float2* gA_part;          // [B, P]
     float* dD_part;           // [B, H]; a single sequence: dD itself
     float2 *dLambda, *dB, *dC;   // a single sequence
@@ -336,6 +337,7 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
                 c = t == t1 - 1 ? cadd(v, c) : cfma2(a, al, flags[t + 1] ? zero : c, v);
                 *reinterpret_cast<float2*>(vq + t * o.xp) = c;
                 share(t, cfma2(gamma, gammal, c, zero));
+                if (p.s) p.s[((size_t)b * T + t) * P + p0 + q] = c;
                 if (!flags[t]) {
                     const float2 before = t > 0 ? f2(xq + (t - 1) * o.xp) : (p.x0 ? p.x0[(size_t)b * P + p0 + q] : zero);
                     gA = cfma(c, cconj(before), gA);
@@ -352,7 +354,7 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
         __syncthreads();
         if (mine) agg[tid] = gA;
         const int chunks = (H + 31) / 32;
-        for (int i = w; i < 2 * pc * chunks; i += kLsWarps) {   // a warp: one state, 32 features
+        for (int i = w; i < (p.s ? 0 : 2 * pc * chunks); i += kLsWarps) {   // a warp: one state, 32 features
             const bool is_c = i >= pc * chunks;
             const int j = is_c ? i - pc * chunks : i, st = j / chunks, h = (j - st * chunks) * 32 + lane;
             const float *av = (is_c ? gy : u) + min(h, H - 1), *bv = (is_c ? x : s) + 2 * st;
@@ -501,11 +503,11 @@ int launch_layer_small_fwd(const LayerSmall& g, cudaStream_t st) {
     return g.bf16 ? launch_ls<__nv_bfloat16, false>(p, g.B, st) : launch_ls<float, false>(p, g.B, st);
 }
 
-int launch_layer_small_bwd(const LayerSmall& g, const GradTail& tail, float2* gA_part, float* dD_part, cudaStream_t st) {
+int launch_layer_small_bwd(const LayerSmall& g, const GradTail& tail, float2* s, float2* gA_part, float* dD_part, cudaStream_t st) {
     LsArgs p{};
     p.T = g.T, p.H = g.H, p.P = g.P, p.Lambda = g.Lambda, p.Delta = g.Delta, p.Bc = g.Bc, p.Cc = g.Cc, p.D = g.D, p.u = g.u;
     p.done = g.done, p.x0 = g.x0, p.gxT = g.gxT, p.gy = g.gy, p.x = g.x, p.out = g.out, p.gx0 = g.gx0;
-    p.part_b = (float2*)tail.part_b, p.part_c = (float2*)tail.part_c, p.gA_part = gA_part;
+    p.part_b = (float2*)tail.part_b, p.part_c = (float2*)tail.part_c, p.s = s, p.gA_part = gA_part;
     p.dD_part = g.B == 1 ? tail.sum_out[0] : dD_part;
     p.dLambda = tail.dLambda, p.dDelta = tail.dDelta, p.dB = tail.dB, p.dC = tail.dC;
     return g.bf16 ? launch_ls<__nv_bfloat16, true>(p, g.B, st) : launch_ls<float, true>(p, g.B, st);

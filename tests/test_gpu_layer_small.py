@@ -1,6 +1,7 @@
 """The kernels that take a small layer's pass at once (layer_small.cu) against the oracle: one state per CTA, one step, the longest
 sequence, more threads than rows x columns and fewer, clusters of 8 and of 4 with the most sequences each takes, groups of 4
-to 17 rows per scanning thread that end full and short; and the shapes just past its limits, which go to the separate kernels."""
+to 17 rows per scanning thread that end full and short; weight gradients as slices and as products of their own; and the shapes
+just past its limits, which go to the separate kernels."""
 import numpy as np
 import pytest
 
@@ -12,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 ONE_KERNEL = [   # rows of a group in brackets where they are not 4
     ("f32", 1, 1, 16, 8), ("f32", 1, 7, 8, 8), ("bf16", 1, 64, 32, 16), ("f32", 1, 512, 16, 16), ("f32", 1, 512, 8, 8), ("f32", 2, 33, 72, 40),
-    ("bf16", 3, 4, 192, 120), ("f32", 1, 13, 248, 120), ("f32", 14, 65, 24, 104), ("bf16", 32, 50, 48, 32), ("f32", 2, 8, 248, 256),
+    ("bf16", 3, 4, 192, 120), ("f32", 1, 13, 248, 120), ("f32", 14, 65, 24, 104), ("bf16", 32, 50, 48, 32), ("f32", 14, 1, 8, 8), ("f32", 2, 8, 248, 256),
     ("f32", 1, 64, 8, 136),      # [5], the last group 4
     ("f32", 4, 50, 24, 256),     # [7], the last group 1
     ("f32", 14, 100, 8, 120),    # [6]
@@ -26,7 +27,10 @@ SEPARATE = [
     ("f32", 33, 50, 48, 32),                                                  # sequences
     ("f32", 1, 500, 40, 24), ("f32", 1, 512, 16, 56), ("f32", 32, 3, 200, 256),   # shared memory
     ("f32", 1, 513, 8, 8), ("f32", 1, 8, 264, 8), ("f32", 1, 8, 8, 264),      # steps, features, states
-    ("f32", 15, 18, 136, 48),                                                 # workspace: slices of the weight gradients
+]
+PRODUCTS = [   # slices of the weight gradients would need more workspace than the separate kernels: their products take s
+    ("f32", 15, 18, 136, 48), ("f32", 32, 10, 184, 128), ("f32", 14, 16, 192, 128), ("f32", 4, 2, 208, 256), ("f32", 5, 16, 88, 248),
+    ("bf16", 32, 3, 104, 40), ("f32", 22, 20, 184, 8),
 ]
 
 
@@ -41,8 +45,13 @@ def _run(io, B, T, H, P, states, kernels):
 @pytest.mark.parametrize("io,B,T,H,P", ONE_KERNEL)
 @pytest.mark.parametrize("states", [False, True])
 def test_small_layers(io, B, T, H, P, states):
-    launches = _run(io, B, T, H, P, states, "one-kernel")
-    assert launches == 2 if B == 1 else launches <= 4, launches   # (several sequences: and the last kernels of the backward pass)
+    assert _run(io, B, T, H, P, states, "one-kernel") == (2 if B == 1 else 4)   # (several: and the last two kernels of the backward pass)
+
+
+@pytest.mark.parametrize("io,B,T,H,P", PRODUCTS)
+@pytest.mark.parametrize("states", [False, True])
+def test_small_layers_with_separate_weight_gradients(io, B, T, H, P, states):
+    assert _run(io, B, T, H, P, states, "one-kernel") == 5
 
 
 @pytest.mark.parametrize("io,B,T,H,P", SEPARATE)
