@@ -7,7 +7,7 @@
 // projects them onto its part of the features.  The weights are used as the caller stores them: gamma, the factor of
 // the discretisation, multiplies the projected inputs and, conjugated, the gradients of the states, so that its
 // double-precision evaluation (its four functions on different warps) runs while the inputs arrive.  What of that could leave the
-// range of fp32 where gamma B does not is computed in its order (an overflowed B u) or scaled exactly (gradients where Delta > 1).
+// range of fp32 where gamma B does not is computed in its order (an overflowed B u) or scaled exactly (gradients where |gamma| > 1).
 // fp32 throughout; Abar as an fp32 pair, its power over a group's rows and the adjoint of the discretisation
 // evaluated in double.  A single sequence finishes its parameter gradients itself; several leave them as slices for
 // launch_layer_tail, or s for the products of the separate kernels where the slices would need more room than those.  Bound by latency: one trip to memory, the exponentials, six barriers.  Measured: see layer_small_cluster.
@@ -140,10 +140,7 @@ __device__ __forceinline__ void product_rows(const float* a, int pa, int M, int 
 
 __device__ __forceinline__ float4 f4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float2 f2(const float* p) { return *reinterpret_cast<const float2*>(p); }
-// The smallest power of two above Delta, or 1 for Delta <= 1.
-__device__ __forceinline__ float step_scale(float delta) {
-    return delta > 1.f ? fminf(2.f * __uint_as_float(__float_as_uint(delta) & 0x7f800000u), 0x1p127f) : 1.f;
-}
+__device__ __forceinline__ bool finite(float2 v) { return isfinite(v.x + v.y); }
 __device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
@@ -152,9 +149,6 @@ __global__ void __launch_bounds__(kLsThreads)
 layer_small_kernel(const __grid_constant__ LsArgs p) {
     extern __shared__ float4 ls_raw[];
     float* sm = reinterpret_cast<float*>(ls_raw);
-    cluster_arrive_release();   // (every CTA runs before its shared memory is written)
-    grid_dep_wait();
-    grid_dep_launch();
     const int T = p.T, H = p.H, P = p.P, C = p.cluster, tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     const int rank = (int)tc::cluster_ctarank(), b = (int)blockIdx.x / C;
     const int pc = P / C, hc = H / C, p0 = rank * pc, h0 = rank * hc;
@@ -166,7 +160,13 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
     float2 *agg = reinterpret_cast<float2*>(sm + o.agg), *gq = reinterpret_cast<float2*>(sm + o.gq);
     float* sums = sm + o.sums;
     uint8_t* flags = reinterpret_cast<uint8_t*>(sm + o.flags);
+    float* scale = sm + o.parts + 10 * pc;   // backward: what the states' gradients are divided by, in the room of the other CTAs' parts
     const float2 zero = make_float2(0.f, 0.f);
+    if (kBwd && tid < P) scale[tid] = 1.f;
+    if (kBwd && tid == 0) scale[P] = 1.f;   // (P <= kLsThreads)
+    cluster_arrive_release();   // (every CTA runs before its shared memory is written)
+    grid_dep_wait();
+    grid_dep_launch();
     if (tid == 0 && blockIdx.x == 0 && !kBwd) p.hdr->status = 0;
 
     // ---- inputs and parameters are on their way while the functions of the discretisation are evaluated
@@ -181,7 +181,6 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
         copy_pairs(wfeat, o.cp, p.Cc + (size_t)h0 * P, P, hc, P);
     }
     for (int i = tid; i < T; i += kLsThreads) flags[i] = p.done ? p.done[(size_t)b * T + i] != 0 : 0;
-    const float any_step = kBwd && tid < P ? p.Delta[tid] : 0.f;   // (P <= kLsThreads)
     for (int q = p0 + (w >> 2) * 32 + lane; q < p0 + pc; q += 32 * (kLsWarps / 4)) {
         const double lr = p.Lambda[q].x, li = p.Lambda[q].y, d = p.Delta[q];
         double* z = parts + 5 * (q - p0);
@@ -191,14 +190,7 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
         else z[4] = exp(lr * d);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    const bool long_step = __syncthreads_or(any_step > 1.f);
-    if (kBwd && long_step)   // |gamma| <= Delta (Re Lambda <= 0), so conj(gamma) s may leave the range of s: B takes a power of two of gamma
-        for (int i = tid; i < P * hc; i += kLsThreads) {
-            const int r = i / hc;
-            float2* w2 = reinterpret_cast<float2*>(wfeat + r * o.cp) + (i - r * hc);
-            const float by = step_scale(p.Delta[r]);
-            *w2 = make_float2(by * w2->x, by * w2->y);
-        }
+    __syncthreads();
 
     // ---- own states: B u, or g_x = gy conj(C)
     {
@@ -254,6 +246,7 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
     const int q = tid % pc, g = tid / pc, t0 = g * rows, t1 = min(T, t0 + rows), n_groups = (T + rows - 1) / rows;
     const bool mine = tid < kLsThreads / pc * pc && t0 < T, last = g == n_groups - 1;
     float2 a = zero, al = zero, aR = zero, aRl = zero, gamma = zero, gammal = zero, first = zero;
+    float own_scale = 1.f;
     bool cut = kBwd ? last : g == 0;   // nothing is added to what the first group to be folded ends with
     float* vq = s + 2 * q;
     if (mine) {
@@ -264,29 +257,39 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
         gammal = make_float2((float)(z.gr - (double)gamma.x), (float)(z.gi - (double)gamma.y));
         aR = make_float2(apow[q].x, apow[q].y), aRl = make_float2(apow[q].z, apow[q].w);
         if (kBwd) a = cconj(a), al = cconj(al), aR = cconj(aR), aRl = cconj(aRl), gamma = cconj(gamma), gammal = cconj(gammal);
-        if (kBwd && long_step) {
-            const float by = 1.f / step_scale(p.Delta[p0 + q]);
-            gamma = make_float2(by * gamma.x, by * gamma.y), gammal = make_float2(by * gammal.x, by * gammal.y);
+        if (kBwd && fabsf(gamma.x) + fabsf(gamma.y) > 1.f) {   // conj(gamma) s may leave the range of s: B takes a power of two of gamma
+            const float by = fminf(2.f * __uint_as_float(__float_as_uint(fabsf(gamma.x) + fabsf(gamma.y)) & 0x7f800000u), 0x1p127f), div = 1.f / by;
+            gamma = make_float2(div * gamma.x, div * gamma.y), gammal = make_float2(div * gammal.x, div * gammal.y);
+            own_scale = by;
         }
         const float2* from = kBwd ? p.gxT : p.x0;
         if (cut && from) first = from[(size_t)b * P + p0 + q];
         float2 e = first;
         if (!kBwd) {
+            float2 dropped = zero;
             for (int t = t0; t < t1; ++t) {
-                const float2 r = f2(vq + t * o.xp);
-                float2 v = cfma2(gamma, gammal, r, zero);
-                if (!isfinite(r.x + r.y)) {   // B u left the range of fp32, which gamma B u need not have done
-                    v = zero;
-#pragma unroll 1
-                    for (int h = 0; h < H; ++h) {
-                        const float2 bg = cfma2(gamma, gammal, f2(wstate + q * o.wp + 2 * h), zero);
-                        v.x = fmaf(u[t * o.hp + h], bg.x, v.x);
-                        v.y = fmaf(u[t * o.hp + h], bg.y, v.y);
-                    }
-                }
+                const float2 v = cfma2(gamma, gammal, f2(vq + t * o.xp), zero);
                 *reinterpret_cast<float2*>(vq + t * o.xp) = v;
-                if (flags[t]) e = zero, cut = true;
+                if (flags[t]) dropped = cadd(dropped, e), e = zero, cut = true;
                 e = cfma2(a, al, e, v);
+            }
+            if (!finite(cadd(dropped, e))) {   // B u may have left the range of fp32, which gamma B u need not have done
+                e = first;
+#pragma unroll 1
+                for (int t = t0; t < t1; ++t) {
+                    float2 v = f2(vq + t * o.xp);
+                    if (!finite(v)) {
+                        v = zero;
+#pragma unroll 1
+                        for (int h = 0; h < H; ++h) {
+                            const float2 bg = cfma2(gamma, gammal, f2(wstate + q * o.wp + 2 * h), zero);
+                            v.x = fmaf(u[t * o.hp + h], bg.x, v.x);
+                            v.y = fmaf(u[t * o.hp + h], bg.y, v.y);
+                        }
+                        *reinterpret_cast<float2*>(vq + t * o.xp) = v;
+                    }
+                    e = cfma2(a, al, flags[t] ? zero : e, v);
+                }
             }
         } else {
             e = cadd(f2(vq + (t1 - 1) * o.xp), e);   // (the state's gradient s; conj(Abar) s, which it hands on, is rounded once, at the end)
@@ -345,6 +348,11 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
             }
             c = flags[t0] ? zero : cfma2(a, al, c, zero);
             if (t0 == 0 && p.gx0) p.gx0[(size_t)b * P + p0 + q] = c;
+            if (t0 == 0 && own_scale != 1.f)
+                for (int r = 0; r < C; ++r)
+                    for (const int i : {p0 + q, P})   // (entry P: there are any)
+                        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(tc::map_to_cta(tma::smem_u32(scale + i), (uint32_t)r)), "f"(own_scale)
+                                     : "memory");
         }
     }
     cluster_arrive_release();
@@ -430,6 +438,13 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
     }
     // ---- own features: y = Re(C x) + D u, or du = Re(conj(B) conj(gamma) s) + D gy
     cluster_wait_acquire();
+    if (kBwd && scale[P] != 1.f) {
+        for (int i = tid; i < P * hc; i += kLsThreads) {
+            float2* w2 = reinterpret_cast<float2*>(wfeat + i / hc * o.cp) + i % hc;
+            *w2 = make_float2(scale[i / hc] * w2->x, scale[i / hc] * w2->y);
+        }
+        __syncthreads();
+    }
     {
         const float* skip = kBwd ? gy : u;
         auto out = [&](int t, int h, float v) {
