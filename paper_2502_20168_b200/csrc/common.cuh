@@ -111,7 +111,7 @@ int device_sm_count();
 // Raises a kernel's dynamic shared-memory limit, once per (kernel, device) (device_setup.cu).
 bool set_max_dynamic_smem(const void* kernel, size_t bytes);
 // Clusters of `cluster` CTAs of a kernel (its shared-memory limit raised already) that the current device runs at the same time, cached
-// per (kernel, cluster, device); 0: it cannot launch them; -1: no device answers.  Lets the kernel be launched in clusters of 16.
+// per (kernel, cluster, shared memory, device); 0: it cannot launch them; -1: no device answers.  Lets the kernel be launched in clusters of 16.
 int resident_clusters(const void* kernel, int cluster, size_t smem_bytes, int threads);
 // Launches a kernel of the library: programmatic dependent launch (see grid_dep_wait), optionally in clusters.
 // Between two kernels of a few microseconds the start of the second used to stand idle for about 2 us; its blocks now

@@ -29,14 +29,14 @@ bool set_max_dynamic_smem(const void* kernel, size_t bytes) {
 // What the device holds depends on the kernel's registers and shared memory and on how its SMs are grouped: asked once.
 int resident_clusters(const void* kernel, int cluster, size_t smem_bytes, int threads) {
     static std::mutex mu;
-    static std::map<std::tuple<const void*, int, int>, int> cache;
+    static std::map<std::tuple<const void*, int, size_t, int>, int> cache;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
         (void)cudaGetLastError();
         return -1;
     }
     std::lock_guard<std::mutex> lock(mu);
-    const auto key = std::make_tuple(kernel, cluster, dev);
+    const auto key = std::make_tuple(kernel, cluster, smem_bytes, dev);
     const auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     cudaLaunchConfig_t cfg = {};

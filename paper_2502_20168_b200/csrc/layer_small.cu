@@ -483,14 +483,16 @@ int ls_cluster(int B, int T, int H, int P) {
     return (long long)T * H * 2 * P <= (long long)c << 17 && (size_t)LsSmem(T, H, P, c, true).total * 4 <= kLsSmemMax ? c : 0;
 }
 
-// Whether the device runs that many clusters of both passes at the same time (with the most shared memory; no device: a B200 is planned for).
+// Whether the device runs that many clusters at the same time (of the backward pass, which takes more shared memory and registers;
+// asked for in steps of 40 KB; no device: a B200 is planned for).
 template <typename IO>
-bool ls_resident(int cluster, int B) {
-    for (const void* kern : {reinterpret_cast<const void*>(layer_small_kernel<IO, false>), reinterpret_cast<const void*>(layer_small_kernel<IO, true>)}) {
-        const int n = set_max_dynamic_smem(kern, kLsSmemMax) ? resident_clusters(kern, cluster, kLsSmemMax, kLsThreads) : -1;
-        if (n >= 0 && n < B) return false;
-    }
-    return true;
+bool ls_resident(int cluster, int B, int T, int H, int P) {
+    const void* kern = reinterpret_cast<const void*>(layer_small_kernel<IO, true>);
+    constexpr size_t kStep = 40 * 1024;
+    static_assert(kLsSmemMax % kStep == 0, "steps of shared memory");
+    const size_t smem = ((size_t)LsSmem(T, H, P, cluster, true).total * 4 + kStep - 1) / kStep * kStep;
+    const int n = set_max_dynamic_smem(kern, kLsSmemMax) ? resident_clusters(kern, cluster, smem, kLsThreads) : -1;
+    return n < 0 || n >= B;
 }
 
 template <typename IO, bool kBwd>
@@ -508,7 +510,7 @@ int launch_ls(LsArgs p, int B, cudaStream_t st) {
 
 int layer_small_cluster(int B, int T, int H, int P, bool bf16) {
     const int c = ls_cluster(B, T, H, P);
-    return c && (bf16 ? ls_resident<__nv_bfloat16>(c, B) : ls_resident<float>(c, B)) ? c : 0;
+    return c && (bf16 ? ls_resident<__nv_bfloat16>(c, B, T, H, P) : ls_resident<float>(c, B, T, H, P)) ? c : 0;
 }
 
 int launch_layer_small_fwd(const LayerSmall& g, cudaStream_t st) {

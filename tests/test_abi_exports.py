@@ -72,6 +72,7 @@ def test_layer_plan_names_the_kernels_a_shape_takes(sb):
     which form of the scans ssm_layer_fwd / ssm_layer_bwd take for the configurations of the benchmark."""
     plan = lambda *a: sb.ssm_layer_plan_string(sb.make_shape(*a))
     assert plan(1, 64, 32, 16, "f32") == "projections=cuda-cores scans=one-kernel"            # H, P below a tile
+    assert plan(14, 65, 24, 104, "f32") == plan(32, 64, 8, 208, "bf16") == "projections=cuda-cores scans=one-kernel"   # the most clusters
     assert plan(33, 64, 32, 16, "f32") == "projections=cuda-cores scans=separate"             # more sequences than clusters
     assert plan(16, 64, 256, 128, "f32") == "projections=tensor-cores-planes scans=in-epilogue"   # fp32 I/O
     assert plan(16, 129, 256, 128, "f32") == "projections=tensor-cores-planes scans=separate"     # one step more than a tile
