@@ -113,6 +113,13 @@ bool set_max_dynamic_smem(const void* kernel, size_t bytes);
 // Clusters of `cluster` CTAs of a kernel (its shared-memory limit raised already) that the current device runs at the same time, cached
 // per (kernel, cluster, shared memory, device); 0: it cannot launch them; -1: no device answers.  Lets the kernel be launched in clusters of 16.
 int resident_clusters(const void* kernel, int cluster, size_t smem_bytes, int threads);
+// Whether what is launched on a stream goes into a graph.
+inline bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &status) == cudaSuccess) return status == cudaStreamCaptureStatusActive;
+    (void)cudaGetLastError();
+    return false;
+}
 // Launches a kernel of the library: programmatic dependent launch (see grid_dep_wait), optionally in clusters.
 // Between two kernels of a few microseconds the start of the second used to stand idle for about 2 us; its blocks now
 // set up while the first drains (projection of 4096 x 512 x 512 back to back: 12.3 -> 9.4 us).

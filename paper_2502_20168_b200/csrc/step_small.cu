@@ -8,7 +8,7 @@
 // added over the warp by a halving exchange that leaves one result per lane.  fp32 sums.  The new states go to the
 // shared memory of every CTA of the cluster, from where its warps project them after one cluster barrier; the weights of
 // a warp's first columns there are on their way meanwhile.
-// Bound by latency: a launch, two trips to L2 and the barrier.  Measured per step: see use_step_small.
+// Bound by latency: a launch, two trips to L2 and the barrier.  Measured per step: see halves_shorter.
 #include <algorithm>
 #include <type_traits>
 
@@ -309,25 +309,37 @@ step_half_kernel(StepHalfArgs p) {
     }
 }
 
-// Few trajectories: us per step in a graph / eager, two kernels for the halves -> one kernel in clusters (B, widths up to):
-//   fp32 I/O: 16, 256: 6.2 / 8.8 -> 4.5 / 5.9, 96, 256: 6.8 / 8.8 -> 4.8 / 5.8;  16, 512: 9.7 / 10.1 -> 7.5 / 8.0;  1, 512: 6.7 / 8.9
-//             -> 7.4 / 7.8;  8, 1024 (32 columns a warp): 16.8 / 16.8 -> 40 / 40;
-//   bf16 I/O: 16, 256: 4.5 / 8.9 -> 4.3 / 5.8, 96, 256: 4.9 / 8.7 -> 4.5 / 5.8;  16, 512: 6.2 / 8.9 -> 6.7 / 7.2;
-// where the clusters need a second round, 128, 256 (16 clusters of 8): fp32 7.4 -> 8.7, bf16 6.6 -> 8.1;  64, 512 fp32 (8 of 16): 11.0 -> 14.4.
-// Against the cluster kernel of gemm_tc_step.cu, the two kernels / that one:
+// Against the cluster kernel of gemm_tc_step.cu, us per step, the two halves / that one:
 //   bf16 I/O: B = 64, H = 512: 9.6 / 11.1, B = 96: 12.5 / 11.6;  H = 1024: B = 32: 15.2 / 17.7, B = 48: 19.3 / 17.9;
 //   fp32 I/O: H = 512: B = 64: 11.6 / 21.9;  H = 1024: B = 32: 18.3 (three kernels: 21.4), B = 48: 26.1 (21.9).
 bool use_step_small(int B, int H, int P) { return (long long)B * std::max(H, 2 * P) <= 32768; }
 
 static auto step_cluster_kernel(bool f32) { return f32 ? step_small_kernel<true> : step_small_kernel<false>; }
-// CTAs of a cluster that takes a step's columns in one round, or 0: the halves apart.  The clusters have to run in one round, on a device
-// that holds fewer than a B200 as well.
-static int step_small_cluster(const StepCall& g) {
+// The halves take less time on the device than the one kernel where its clusters are small or hold few rows, and more host time nearly
+// everywhere (two launches: 7.3 us).  us per step in a graph, halves / one kernel (B, H, P):
+//   fp32, clusters of 16: 1, 512, 256 6.9 / 7.7, 4 7.7 / 7.7, 8 9.7 / 7.7;  1, 384, 192 5.5 / 6.5, 4 6.1 / 6.5, 5 6.9 / 6.5;  16, 512, 256 9.9 / 7.7;
+//         4, 384, 64 4.6 / 5.4, 16 5.0 / 5.5, 16, 512, 64 6.0 / 6.0;  of 8: 1, 256, 128 4.7 / 4.6, 16 6.2 / 4.7, 96 6.6 / 4.9;  2, 256, 64 4.0 / 4.2, 8 4.5 / 4.2;
+//         of 4: 8, 128, 64 3.5 / 3.7, 112 3.8 / 3.9, 224 4.7 / 3.9;
+//   bf16, clusters of 8: 1, 256, 128 4.2 / 4.2, 16 4.6 / 4.4;  1, 256, 64 3.6 / 4.0, 8 3.9 / 4.0, 32 4.1 / 4.1;  of 4: 8, 128, 64 3.4 / 3.6, 224 4.6 / 3.8.
+// Eager: 16, 256, 128 7.3 / 5.0, 16, 512, 256 10.5 / 8.3;  1, 512, 256 7.5 / 8.2, 3 8.0 / 8.3;  1, 384, 256 7.3 / 7.6, 2 7.5 / 7.6.  The results are the same bits.
+static bool halves_shorter(const StepCall& g, int cluster, cudaStream_t st) {
+    const int P2 = 2 * g.P;
+    const bool in_graph = g.B <= (cluster == 4 ? 112 : cluster == 8 ? (std::min(g.H, P2) == 128 ? 2 : 0) : (P2 == 128 ? 16 : 4));
+    const bool eager = cluster == 16 && g.B <= 3 && (long long)g.H * P2 >= (g.B == 1 ? 384 : 512) * 512;
+    return in_graph == eager ? eager : (capturing(st) ? in_graph : eager);
+}
+
+// CTAs of a cluster that takes a step's columns in one round, or 0: the halves apart.  The clusters have to run in one round (us in a graph,
+// halves / one kernel: 128, 256, 128, 16 clusters of 8, fp32 7.4 / 8.7, bf16 6.6 / 8.1;  64, 512, 256 in fp32, 8 of 16, 11.0 / 14.4), on a device that
+// holds fewer than a B200 as well.  Wider ones, with several rounds of columns a warp, are slower throughout (8, 1024, 512 in fp32 16.8 / 40), as are
+// clusters of 16 with bf16 I/O (16, 512, 256 6.2 / 6.7).
+static int step_small_cluster(const StepCall& g, cudaStream_t st) {
     const int width = std::max(g.H, 2 * g.P), row_groups = (g.B + kSsRows - 1) / kSsRows;
-    int c = 1;
+    if (std::min(g.H, 2 * g.P) < 128) return 0;   // (every lane has a share of both contractions)
+    int c = 4;
     while (c * kSsWarps * kSsCols < width) c *= 2;
     const int most = c <= 8 ? 112 : (c == 16 && g.f32 ? 64 : 0);   // CTAs
-    if (row_groups * c > most) return 0;
+    if (row_groups * c > most || halves_shorter(g, c, st)) return 0;
     const size_t smem = kSsRows * kSsWarps * kSsCols * 16 * sizeof(float);   // (of the widest)
     return resident_clusters(reinterpret_cast<const void*>(step_cluster_kernel(g.f32)), c, smem, 32 * kSsWarps) >= row_groups ? c : 0;
 }
@@ -347,7 +359,7 @@ static int launch_step_cluster(const StepCall& g, int cluster, cudaStream_t st) 
 }
 
 int launch_step_small(const StepCall& g, cudaStream_t st) {
-    if (const int cluster = step_small_cluster(g)) return launch_step_cluster(g, cluster, st);
+    if (const int cluster = step_small_cluster(g, st)) return launch_step_cluster(g, cluster, st);
     StepHalfArgs p{};
     p.M = g.B;
     p.done = g.done, p.Abar = g.Abar, p.Alo = g.Alo;

@@ -36,6 +36,10 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
 }
 cudaError_t cudaLaunchKernel(const void* f, dim3 g, dim3 b, void** args, size_t s, cudaStream_t st) { return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t st) { return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t st, enum cudaStreamCaptureStatus* s) {
+    *s = getenv("FAKE_CAPTURE") ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
 cudaError_t cudaPeekAtLastError(void) { return cudaSuccess; }
 cudaError_t cudaGetLastError(void) { return cudaSuccess; }
 """
@@ -67,9 +71,9 @@ def fake(tmp_path_factory):
     subprocess.run([shutil.which("gcc") or "gcc", "-shared", "-fPIC", "-w", "-I" + include, "-o", str(d / "fake.so"), str(d / "fake.c")],
                    check=True)
 
-    def calls(cluster, resident, *args):
+    def calls(cluster, resident, *args, **more):
         """[(status, launches)] of each call where clusters above `cluster` CTAs are refused."""
-        env = dict(os.environ, LD_PRELOAD=str(d / "fake.so"), FAKE_CLUSTER=str(cluster), FAKE_RESIDENT=str(resident))
+        env = dict(os.environ, **more, LD_PRELOAD=str(d / "fake.so"), FAKE_CLUSTER=str(cluster), FAKE_RESIDENT=str(resident))
         r = subprocess.run([sys.executable, "-c", PROBE, build.LIB_PATH, *map(str, args)], env=env, capture_output=True, text=True, timeout=300)
         assert r.returncode == 0, r.stderr
         return [tuple(map(int, line.split())) for line in r.stdout.splitlines()]
@@ -83,6 +87,15 @@ def test_steps_without_clusters_take_the_two_halves(fake, B, H, P, io, size):
     groups = (B + 7) // 8
     assert fake(16, groups, "step", B, 1, H, P, io) == [(0, 1)]
     assert fake(16, groups - 1, "step", B, 1, H, P, io) == [(0, 2)]   # not all in one round
+
+
+@pytest.mark.parametrize("B,H,P,io,eager,graph", [(1, 512, 256, 0, 2, 2), (4, 512, 256, 0, 1, 2), (5, 512, 256, 0, 1, 1), (4, 384, 192, 0, 1, 2),
+                                                  (16, 384, 64, 0, 1, 2), (17, 384, 64, 0, 1, 1), (1, 256, 128, 0, 1, 1), (2, 256, 64, 0, 1, 2), (3, 256, 64, 1, 1, 1),
+                                                  (112, 128, 64, 0, 1, 2), (113, 128, 64, 0, 1, 1)])
+def test_steps_in_a_graph_take_the_two_halves_where_those_are_shorter(fake, B, H, P, io, eager, graph):
+    """Launched one by one, two kernels cost their host time; in a graph only what they take on the device."""
+    assert fake(16, 40, "step", B, 1, H, P, io) == [(0, eager)]
+    assert fake(16, 40, "step", B, 1, H, P, io, FAKE_CAPTURE="1") == [(0, graph)]
 
 
 @pytest.mark.parametrize("B,T,H,P,io,size", [(1, 64, 32, 16, 0, 8), (14, 64, 32, 16, 1, 8), (32, 64, 32, 16, 0, 4)])
