@@ -418,7 +418,6 @@ __device__ __forceinline__ bool tn_drain_tile(const Smem& s, const TnParams& p, 
 // on the `empty` / `tmem_full` barriers of both CTAs; both CTAs' epilogue warps arrive on the
 // leader's `tmem_empty` barriers.
 constexpr int kPairStages = 4;
-constexpr int kPairStageBytes = kABytes + kBBytes / 2;
 // (the epilogue with the column sums gives one operand stage up for its second operand tiles and its sums)
 #ifndef SSM_PAIR_STAGES_BF16_EPILOGUE
 #define SSM_PAIR_STAGES_BF16_EPILOGUE 4

@@ -89,7 +89,7 @@ def test_steps_without_clusters_take_the_two_halves(fake, B, H, P, io, size):
     assert fake(16, groups - 1, "step", B, 1, H, P, io) == [(0, 2)]   # not all in one round
 
 
-@pytest.mark.parametrize("B,H,P,io,eager,graph", [(1, 512, 256, 0, 2, 2), (4, 512, 256, 0, 1, 2), (5, 512, 256, 0, 1, 1), (4, 384, 192, 0, 1, 2),
+@pytest.mark.parametrize("B,H,P,io,eager,graph", [(1, 512, 256, 0, 2, 2), (3, 512, 256, 0, 2, 2), (4, 512, 256, 0, 1, 1), (4, 384, 192, 0, 1, 2),
                                                   (16, 384, 64, 0, 1, 2), (17, 384, 64, 0, 1, 1), (1, 256, 128, 0, 1, 1), (2, 256, 64, 0, 1, 2), (3, 256, 64, 1, 1, 1),
                                                   (112, 128, 64, 0, 1, 2), (113, 128, 64, 0, 1, 1)])
 def test_steps_in_a_graph_take_the_two_halves_where_those_are_shorter(fake, B, H, P, io, eager, graph):
