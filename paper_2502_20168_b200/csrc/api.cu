@@ -805,7 +805,7 @@ SSM_API int ssm_layer_bwd(const ssm_shape* shape, const ssm_c64* Lambda, const f
             const bool b = s.io_dtype == SSM_BF16;
             const GemmNT g[2] = {{u, b, s.H, at<float>(ws, p.gs), P2, BT, p.splits, const_cast<float*>(left.tail.part_b)},
                                  {gy, b, s.H, at<float>(ws, p.xs), P2, BT, p.splits, const_cast<float*>(left.tail.part_c)}};
-            launch_gemm_nt(g, 2, nullptr, st);
+            launch_gemm_nt(g, 2, nullptr, st, true);
         }
         if (s.B > 1) return layer_bwd_tail(s, p, 1, &left, hdr, st);
         SSM_RETURN_IF_CUDA_ERROR();

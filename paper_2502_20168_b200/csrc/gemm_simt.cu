@@ -163,6 +163,8 @@ __device__ __forceinline__ void load4_any(const void* p, bool bf16, size_t i, fl
     else load4<float>(reinterpret_cast<const float*>(p) + i, v);
 }
 
+// kChains: rows are summed in chains of 8 before they are added to the rest, as the one-kernel passes of small layers do.
+template <bool kChains>
 __global__ void __launch_bounds__(kGemmThreads)
 gemm_nt_kernel(const __grid_constant__ NtSimtArgs q) {
     grid_dep_wait();
@@ -229,15 +231,26 @@ gemm_nt_kernel(const __grid_constant__ NtSimtArgs q) {
         *reinterpret_cast<float4*>(&Bs[lk][lc]) = make_float4(vb[0], vb[1], vb[2], vb[3]);
         __syncthreads();
         if (k0 + TK < ke) fetch(k0 + TK);
+        constexpr int kChain = kChains ? 8 : TK;
 #pragma unroll
-        for (int k = 0; k < TK; ++k) {
-            const float4 a = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-            const float4 b = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-            const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+        for (int k1 = 0; k1 < TK; k1 += kChain) {
+            float part[4][4] = {};
+            float(&to)[4][4] = kChains ? part : acc;
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int k = k1; k < k1 + kChain; ++k) {
+                const float4 a = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
+                const float4 b = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
+                const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) to[i][j] = fmaf(av[i], bv[j], to[i][j]);
+            }
+            if (kChains)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] += part[i][j];
         }
         __syncthreads();
     }
@@ -263,7 +276,7 @@ int gemm_nt_splits(int K, int I, int J) {
     return std::max(1, std::min(std::max(std::min(want, most), least), 64));
 }
 
-void launch_gemm_nt(const GemmNT* g, int n, const SimtDot* dot, cudaStream_t st) {
+void launch_gemm_nt(const GemmNT* g, int n, const SimtDot* dot, cudaStream_t st, bool short_chains) {
     NtSimtArgs q{};
     for (int i = 0; i < n; ++i) q.g[i] = g[i];
     q.n = n;
@@ -279,7 +292,7 @@ void launch_gemm_nt(const GemmNT* g, int n, const SimtDot* dot, cudaStream_t st)
         grid.z += (unsigned)std::min<long long>((q.dot_blocks + per_z - 1) / per_z, kMaxGridZ - grid.z);
     }
     count_launch();
-    launch_dep(gemm_nt_kernel, grid, kGemmThreads, 0, st, q);
+    launch_dep(short_chains ? gemm_nt_kernel<true> : gemm_nt_kernel<false>, grid, kGemmThreads, 0, st, q);
 }
 
 }  // namespace ssm

@@ -142,7 +142,7 @@ struct SimtDot {
 };
 int gemm_nt_splits(int K, int I, int J);
 // n = 1 or 2 products of one shape in one launch, and dot (may be NULL).
-void launch_gemm_nt(const GemmNT* g, int n, const SimtDot* dot, cudaStream_t st);
+void launch_gemm_nt(const GemmNT* g, int n, const SimtDot* dot, cudaStream_t st, bool short_chains = false);
 
 // gemm_tc.cu: bf16 projections on tcgen05 tensor cores (operands by TMA, accumulators in TMEM).
 // Scan of a projection's result in its epilogue (gemm_tc_small.cu): forward, out = x with x_t = keep_t Abar x_{t-1} + acc_t, or with
