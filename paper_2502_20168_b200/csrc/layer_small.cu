@@ -1,6 +1,6 @@
 // A layer's forward and backward pass in one kernel each, for small layers of widths that the tensor cores do not take.
 //
-// As ten dependent launches a layer of 64 steps, 32 features and 16 states took 33 us, 3 us each, of which the sums are
+// As ten dependent launches a layer of 64 steps, 32 features and 16 states took 31 us (eager 36.5), 3 us each, of which the sums are
 // a fraction.  Here a cluster of CTAs takes one sequence through the whole pass.  Each CTA owns a part of the states: it
 // projects onto them, scans them (groups of rows per state, joined in order, as in the streaming kernels) and forms
 // their weight gradients; the scanned states go to the shared memory of all CTAs of the cluster, each of which
@@ -10,7 +10,10 @@
 // range of fp32 where gamma B does not is computed in its order (an overflowed B u) or scaled exactly (gradients where |gamma| > 1).
 // fp32 throughout; Abar as an fp32 pair, its power over a group's rows and the adjoint of the discretisation
 // evaluated in double.  A single sequence finishes its parameter gradients itself; several leave them as slices for
-// launch_layer_tail, or s for the products of the separate kernels where the slices would need more room than those.  Bound by latency: one trip to memory, the exponentials, six barriers.  Measured: see layer_small_cluster.
+// launch_layer_tail, or s for the products of the separate kernels where the slices would need more room than those.
+// Bound by latency: one trip to memory, the exponentials, six barriers and the fetch of the instructions, which each launch runs once.  Of
+// the cycles between two instructions of a warp at 1 x 64 (32, 16), barriers are 39 % forward and 28 % backward, missing instructions 29 %
+// backward; no unit is above 19 % at 14 sequences.  Measured: see ls_cluster.
 #include <type_traits>
 
 #include "kernels.h"
@@ -473,10 +476,12 @@ layer_small_kernel(const __grid_constant__ LsArgs p) {
     }
 }
 
-// us per forward and backward pass in a graph, ten launches -> this (B x T, H, P): 1 x 64, 32, 16 30.9 -> 18.2 (eager 36.5 -> 16.2),
-// 1 x 512, 16, 16 41.2 -> 34.9, 4 x 128, 96, 40 47.3 -> 45.3 (123 K multiply-adds a projection and CTA: the limit is 131 K);
-// clusters of 4: 20 x 128, 32, 64 55.4 -> 45.2, 30 x 20, 176, 72 in bf16 67.7 -> 65.7.  Where the clusters do not run in one round:
-// 16 x 128, 64, 64 (clusters of 8) 53.9 -> 73.2, 36 x 64, 64, 64 (of 4) 55.7 -> 58.6.  One CTA per sequence, 148 x 64, 32, 16: 59.6 -> 76.0.
+// us per forward and backward pass in a graph (forward alone), ten launches -> this (B x T, H, P): 1 x 64, 32, 16 30.9 -> 15.5 (eager
+// 36.5 -> 15.9), 1 x 1, 16, 8 17.2 -> 11.2 (6.2 -> 4.7), 1 x 512, 16, 16 41.2 -> 34.9, 14 x 64, 72, 104 62.5 -> 47.6 (25.0 -> 13.9), 4 x 128, 96, 40 47.3 -> 45.3
+// (123 K multiply-adds a projection and CTA: the limit is 131 K);  clusters of 4: 32 x 64, 40, 40 44.8 -> 45.7 (15.4 -> 9.7), 20 x 128, 32, 64
+// 55.4 -> 45.2, 32 x 261, 24, 8 107 -> 38.5 (51.4 -> 10.4);  with the weight gradients as products: 32 x 10, 184, 128 73.9 -> 47.7 (32.5 -> 14.9),
+// 14 x 16, 192, 128 71.7 -> 41.1 (31.2 -> 11.6), 4 x 2, 208, 256 92.5 -> 29.8 (43.1 -> 9.9), 15 x 13, 24, 24 in bf16 34.5 -> 24.6 (12.9 -> 6.1).  Of 135 shapes
+// none is slower by more than 2 %, and the forward pass alone never.  Where the clusters do not run in one round: 16 x 128, 64, 64 (clusters of 8) 53.9 -> 73.2, 36 x 64, 64, 64 (of 4) 55.7 -> 58.6.  One CTA per sequence, 148 x 64, 32, 16: 59.6 -> 76.0.
 int ls_cluster(int B, int T, int H, int P) {
     if (P > kLsThreads || T > 512 || H > 256 || B > 32) return 0;
     const int c = B <= 14 ? 8 : 4;

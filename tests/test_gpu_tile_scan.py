@@ -15,6 +15,8 @@ pytestmark = pytest.mark.gpu
                                      (40, 20, 128, 64)])
 @pytest.mark.parametrize("states", [False, True])
 def test_layers_fp32(B, T, H, P, states):
+    from paper_2502_20168_b200 import binding as sb
+    assert sb.ssm_layer_plan_string(sb.make_shape(B, T, H, P, "f32")).endswith("scans=in-epilogue" if T <= 128 else "scans=separate")
     run(I.Workload("tile", B=B, T=T, H=H, P=P, io_dtype="f32", p_done=0.05 if states else 0.0, seed=B + T), with_x0=states, with_gxT=states)
 
 
