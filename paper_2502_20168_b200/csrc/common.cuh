@@ -110,8 +110,8 @@ void count_launch(int n = 1);
 int device_sm_count();
 // Raises a kernel's dynamic shared-memory limit, once per (kernel, device) (device_setup.cu).
 bool set_max_dynamic_smem(const void* kernel, size_t bytes);
-// Clusters of `cluster` CTAs of a kernel (its shared-memory limit raised already) that the current device runs at the same time, cached
-// per (kernel, cluster, shared memory, device); 0: it cannot launch them; -1: no device answers.  Lets the kernel be launched in clusters of 16.
+// Clusters of `cluster` CTAs of a kernel that the current device runs at the same time, cached per (kernel, cluster, shared memory,
+// device); 0: it cannot launch them; -1: no device answers.  Lets the kernel be launched with that much shared memory and in clusters of 16.
 int resident_clusters(const void* kernel, int cluster, size_t smem_bytes, int threads);
 // Whether what is launched on a stream goes into a graph.
 inline bool capturing(cudaStream_t st) {

@@ -56,7 +56,8 @@ int resident_clusters(const void* kernel, int cluster, size_t smem_bytes, int th
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if ((cluster > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+    if ((smem_bytes > 48 * 1024 && !set_max_dynamic_smem(kernel, smem_bytes)) ||
+        (cluster > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
         cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
         (void)cudaGetLastError();
         n = 0;

@@ -496,7 +496,7 @@ bool ls_resident(int cluster, int B, int T, int H, int P) {
     constexpr size_t kStep = 40 * 1024;
     static_assert(kLsSmemMax % kStep == 0, "steps of shared memory");
     const size_t smem = ((size_t)LsSmem(T, H, P, cluster, true).total * 4 + kStep - 1) / kStep * kStep;
-    const int n = set_max_dynamic_smem(kern, kLsSmemMax) ? resident_clusters(kern, cluster, smem, kLsThreads) : -1;
+    const int n = resident_clusters(kern, cluster, smem, kLsThreads);
     return n < 0 || n >= B;
 }
 
